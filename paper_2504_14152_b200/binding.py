@@ -1,7 +1,10 @@
-"""ctypes binding for libfgmp.so.  Names follow include/fgmp.h; no arithmetic happens here."""
+"""Binding for libfgmp.so.  Names follow include/fgmp.h; no arithmetic happens here.  The calls of a decode or prefill
+step go through the CPython entry points of _fgmp_torch.so (csrc/fgmp_torch.cpp), everything else through ctypes."""
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
 
@@ -9,6 +12,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 _LIB_PATH = os.path.join(_HERE, "libfgmp.so")
+_EXT_PATH = os.path.join(_HERE, "_fgmp_torch.so")
 
 SCORE_LP_ERROR, SCORE_HP_TO_LP = 0, 1
 CLIP_NONE, CLIP_SW_BRUTE = 0, 1
@@ -26,6 +30,7 @@ class _Scales(ctypes.Structure):
 
 
 _lib = None
+_ext = None
 
 
 def library_path() -> str:
@@ -93,6 +98,26 @@ def _load():
     L.fgmp_version.restype = ci
     _lib = L
     return L
+
+
+def _load_ext():
+    """Loads the CPython entry points (they link against libfgmp.so beside them)."""
+    global _ext
+    if _ext is None:
+        _load()
+        if not os.path.exists(_EXT_PATH):
+            raise ImportError(f"{_EXT_PATH} is missing: build it with `python -m paper_2504_14152_b200.build`")
+        loader = importlib.machinery.ExtensionFileLoader("_fgmp_torch", _EXT_PATH)
+        spec = importlib.util.spec_from_file_location("_fgmp_torch", _EXT_PATH, loader=loader)
+        mod = importlib.util.module_from_spec(spec)
+        loader.exec_module(mod)
+        _ext = mod
+    return _ext
+
+
+def _failed(r) -> FgmpError:
+    """The (status, call) pair that an entry point returns instead of its result."""
+    return FgmpError(r[0], r[1])
 
 
 def status_string(code: int) -> str:
@@ -193,18 +218,12 @@ def quantize_activations(X: torch.Tensor, fisher: torch.Tensor, *, scale_fp4: fl
                          score_mode: int = SCORE_LP_ERROR, tau: float,
                          out: torch.Tensor | None = None) -> PackedTensor:
     """X bf16 [M, K], fisher fp32 [K] -> packed activations."""
-    L = _load()
     assert X.is_cuda and X.dtype == torch.bfloat16 and fisher.dtype == torch.float32 and X.dim() == 2
+    r = (_ext or _load_ext()).quantize_activations(X, fisher, scale_fp4, ratio, scale_fp8, score_mode, tau, out)
+    if r.__class__ is tuple:
+        raise _failed(r)
     M, K = X.shape
-    nbytes = L.fgmp_acts_bytes(M, K)
-    if nbytes == 0:
-        raise FgmpError(-2, "fgmp_acts_bytes")
-    if out is None:
-        out = _alloc_aligned(nbytes, X.device)
-    _ok(L.fgmp_quantize_activations(X.data_ptr(), X.stride(0), fisher.data_ptr(), M, K, _Scales(scale_fp4, ratio, scale_fp8),
-                                    score_mode, tau, out.data_ptr(), out.numel(), None, 0, _stream()),
-        "fgmp_quantize_activations")
-    return PackedTensor(out, M, K, 0, scale_fp8 > 0)
+    return PackedTensor(r, M, K, 0, scale_fp8 > 0)
 
 
 def calibrate_tau(X: torch.Tensor, fisher: torch.Tensor, *, scale_fp4: float, ratio: int = 3, scale_fp8: float = 0.0,
@@ -277,21 +296,16 @@ def linear(acts: PackedTensor, weights: PackedTensor, *, out_dtype=torch.float32
            out: torch.Tensor | None = None, workspace: torch.Tensor | None = None) -> torch.Tensor:
     """Y [M, N] = acts x weights^T (FP32 accumulation).  Operands packed with an FP8 tensor scale of their
     own go through linear_classes (one accumulation per class of block pair, fp32 output)."""
-    L = _load()
     assert acts.K == weights.K and acts.kind == 0 and weights.kind == 1
     if acts.fp8_free or weights.fp8_free:
         return linear_classes(acts, weights, out=out, workspace=workspace)
-    M, N, K = acts.rows, weights.rows, acts.K
-    if out is None:
-        out = torch.empty(M, N, dtype=out_dtype, device=acts.blob.device)
-    assert out.dtype in (torch.float32, torch.bfloat16)
-    if workspace is None:
-        workspace = alloc_workspace(OP_LINEAR, M, N, K, acts.blob.device)
-    _ok(L.fgmp_linear(acts.blob.data_ptr(), weights.blob.data_ptr(), out.data_ptr(),
-                      1 if out.dtype == torch.bfloat16 else 0, out.stride(0), M, N, K,
-                      workspace.data_ptr(), workspace.numel(), _stream()), "fgmp_linear")
-    linear.last_workspace = workspace
-    return out
+    assert (out_dtype if out is None else out.dtype) in (torch.float32, torch.bfloat16)
+    y, ws = (_ext or _load_ext()).linear(acts.blob, weights.blob, acts.rows, weights.rows, acts.K, out,
+                                         out_dtype is torch.bfloat16, workspace)
+    if ws.__class__ is str:
+        raise _failed((y, ws))
+    linear.last_workspace = ws
+    return y
 
 
 def linear_classes(acts: PackedTensor, weights: PackedTensor, *, out: torch.Tensor | None = None,
@@ -319,25 +333,17 @@ def linear_fused(X: torch.Tensor, fisher: torch.Tensor, weights: PackedTensor, *
     """One decode step in one call: X bf16 [M, K] is quantized (as quantize_activations would) and
     multiplied with the packed weights.  Returns Y, or (Y, PackedTensor) when the packed activations
     are asked for (want_packed / packed_out)."""
-    L = _load()
     assert X.is_cuda and X.dtype == torch.bfloat16 and fisher.dtype == torch.float32 and X.dim() == 2
     assert weights.kind == 1 and X.shape[1] == weights.K
-    M, K = X.shape
-    N = weights.rows
-    if out is None:
-        out = torch.empty(M, N, dtype=out_dtype, device=X.device)
-    if packed_out is None and want_packed:
-        packed_out = _alloc_aligned(L.fgmp_acts_bytes(M, K), X.device)
-    if workspace is None:
-        workspace = alloc_workspace(OP_LINEAR_FUSED, M, N, K, X.device)
-    _ok(L.fgmp_linear_fused(X.data_ptr(), X.stride(0), fisher.data_ptr(), _Scales(scale_fp4, ratio), score_mode, tau,
-                            weights.blob.data_ptr(), out.data_ptr(), 1 if out.dtype == torch.bfloat16 else 0,
-                            out.stride(0), M, N, K, _ptr(packed_out), 0 if packed_out is None else packed_out.numel(),
-                            workspace.data_ptr(), workspace.numel(), _stream()), "fgmp_linear_fused")
-    linear.last_workspace = workspace
-    if packed_out is not None:
-        return out, PackedTensor(packed_out, M, K, 0)
-    return out
+    assert (out_dtype if out is None else out.dtype) in (torch.float32, torch.bfloat16)
+    r = (_ext or _load_ext()).linear_fused(X, fisher, weights.blob, weights.rows, scale_fp4, ratio, score_mode, tau, out,
+                                           out_dtype is torch.bfloat16, packed_out, want_packed, workspace)
+    if len(r) == 2:
+        raise _failed(r)
+    y, packed, linear.last_workspace = r
+    if packed is not None:
+        return y, PackedTensor(packed, X.shape[0], weights.K, 0)
+    return y
 
 
 def linear_quantize(acts: PackedTensor, weights: PackedTensor, fisher_next: torch.Tensor, *, scale_fp4: float,
@@ -345,18 +351,14 @@ def linear_quantize(acts: PackedTensor, weights: PackedTensor, fisher_next: torc
                     workspace: torch.Tensor | None = None) -> PackedTensor:
     """acts x weights^T, quantized for the next layer in the GEMM's epilogue: the packed activations
     [M, N] that quantize_activations(linear(..., bf16), fisher_next, ...) would give."""
-    L = _load()
     assert acts.K == weights.K and acts.kind == 0 and weights.kind == 1
-    M, N, K = acts.rows, weights.rows, acts.K
-    dev = acts.blob.device
-    out = _alloc_aligned(L.fgmp_acts_bytes(M, N), dev)
-    if workspace is None:
-        workspace = alloc_workspace(OP_LINEAR_QUANTIZE, M, N, K, dev)
-    _ok(L.fgmp_linear_quantize(acts.blob.data_ptr(), weights.blob.data_ptr(), M, N, K, fisher_next.data_ptr(),
-                               _Scales(scale_fp4, ratio), score_mode, tau, out.data_ptr(), out.numel(),
-                               workspace.data_ptr(), workspace.numel(), _stream()), "fgmp_linear_quantize")
-    linear.last_workspace = workspace
-    return PackedTensor(out, M, N, 0)
+    M, N = acts.rows, weights.rows
+    blob, ws = (_ext or _load_ext()).linear_quantize(acts.blob, weights.blob, M, N, acts.K, fisher_next, scale_fp4, ratio,
+                                                     score_mode, tau, workspace)
+    if ws.__class__ is str:
+        raise _failed((blob, ws))
+    linear.last_workspace = ws
+    return PackedTensor(blob, M, N, 0)
 
 
 STATIC_SCRATCH_BYTES = 4 * 1024 * 1024
