@@ -35,11 +35,10 @@
  *   mask          : rows * ceil(K/16/32) uint32; bit j of word w of a row = block 32w+j,
  *                   1 = FP8
  *   arec          : (rows <= 16 only) C records of 10752 bytes, one per chunk, holding what the
- *                   decode-sized GEMM streams, for 16 token rows (rows >= M are zero):
+ *                   decode-sized GEMM makes its operands from, for up to 16 token rows:
  *                   2048 B: the E2M1 codes as a 16-row x 128-byte tile, the 16-byte pieces of row m
  *                   XOR-swizzled with m%8 (zero in FP8 blocks) | 256 B: E4M3 microscales [token][block
- *                   column], 0x00 for FP8 blocks | 16 B: two uint32 (one per token octet; their OR is used) whose
- *                   bit j says that block column j of some token is FP8, padding | 256 B padding | 8192 B: every element over the tensor
+ *                   column], 0x00 for FP8 blocks | 256 B not used | 8192 B: every element over the tensor
  *                   scale in fp16 (exact for either format): token octet m/8 in its own 4096 bytes, there
  *                   256 bytes per block column, there 32 bytes per token
  *   codes8        : a dense rows*K byte plane of which only the FP8 blocks are written (the
@@ -50,14 +49,16 @@
  *                   not traffic, and keeps the single-pass quantizer free of a compaction step
  *
  * Weights: header | mask | uptr | records | lists
+ *   mask          : 256 bytes per unit: uint16 per row of the tile, bit j set if the row's block in column j of the
+ *                   chunk is FP8 (fgmp_unpack gives the row-major form)
  *   record        : 18560 bytes per unit, unit (t, c) at index t*C + c:
  *                   16384 B of 8-byte slots as a 128-row x 128-byte tile, the 16-byte pieces of row r
  *                   XOR-swizzled with r%8 (the K-major layout the tensor core reads): the 16 E2M1 codes
  *                   of an NVFP4 block, or E4M3 codes 0..7 of an FP8 block (zero beyond N)
  *                   | 2048 B of E4M3 microscales, 0x00 for FP8 blocks, in the order they go to tensor
  *                   memory: byte of (row r, block column j) = (j/4)*512 + (r%32)*16 + (r/32)*4 + j%4
- *                   | 128 B: uint16 x 17, FP8 blocks of the unit before block column j; entry 16 = all
- *   list          : per unit, its FP8 blocks ordered by (block column, row): one uint32 for each (padded
+ *                   | 128 B: uint16 x 17, FP8 blocks of the unit before row 8 i; entry 16 = all
+ *   list          : per unit, its FP8 blocks ordered by (row, block column): one uint32 for each (padded
  *                   to 16 bytes; low half = byte offset of the block's slot in the tile, high half =
  *                   16 * row + 4 * ((row / 2) % 4)), then E4M3 codes 8..15 of each (8 bytes, padded to 16)
  *   uptr          : uint32 [units + 1]: start of a unit's list in 16-byte steps
@@ -109,7 +110,7 @@ typedef struct {
 /* First 256 bytes of a packed blob (device memory). */
 typedef struct {
     uint32_t magic;          /* 'FGMP' = 0x504d4746                                         */
-    uint32_t version;        /* layout version, 7                                           */
+    uint32_t version;        /* layout version, 8                                           */
     int64_t rows, K;
     float scale_fp4;         /* tensor scale actually used                                  */
     int32_t fp8_log2_ratio;
@@ -247,18 +248,18 @@ fgmp_status fgmp_linear_classes(const void* packed_acts, const void* packed_weig
 /* ---- one decode step in one launch: activation quantizer + GEMM (Section 4.2 into Section 4.1) ----
  * For decode-sized batches (the shapes of fgmp_linear's weight-streaming kernel: 1 <= M <= 16,
  * K % 256 == 0) this is fgmp_quantize_activations(X, ...) followed by fgmp_linear, as one kernel: the
- * thread blocks first share out the quantizer's work (256-element chunks of eight token rows; four lanes
+ * thread blocks first share out the quantizer's work (256-element chunks of four token rows; four lanes
  * per block, the same single-precision steps in the same order, so codes, scales and masks are those of
  * fgmp_quantize_activations bit for bit), while the first weight records are already on their way, and
  * start multiplying once every chunk has been handed in.  Y is what fgmp_linear returns for those packed
  * activations, bit for bit.
  *   packed_acts_out (may be NULL): receives the packed activations (size fgmp_acts_bytes(M, K)) for a
  *     caller that wants them (fgmp_unpack, or a later fgmp_linear with other weights); if NULL only the
- *     fp16 records the GEMM streams are kept, in the workspace.
+ *     records the GEMM streams are kept, in the workspace.
  *   workspace: fgmp_workspace_bytes(FGMP_OP_LINEAR_FUSED, M, N, K), cleared once with
  *     fgmp_workspace_init.  Beside fgmp_linear's words the control area holds the work-item counters of
- *     the quantizer and a "records ready" word; the counters wrap to zero by themselves and the block that
- *     finishes last clears the word, so nothing has to be cleared between calls; after an
+ *     the quantizer and a count of the finished ones; the counters wrap to zero by themselves and the block that
+ *     finishes last clears the count, so nothing has to be cleared between calls; after an
  *     error reported by fgmp_check clear the workspace again.  Calls that share a workspace must not
  *     overlap on the GPU.
  *   The kernel is launched as a programmatic dependent like fgmp_linear's (same condition on

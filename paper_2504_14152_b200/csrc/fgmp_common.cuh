@@ -7,6 +7,7 @@
 #include "fgmp.h"
 
 #define FGMP_MAGIC 0x504d4746u
+#define FGMP_LAYOUT_VERSION 8
 #define FGMP_BS 16
 
 // ---------------------------------------------------------------- blob layout
@@ -15,6 +16,8 @@
 // Weights (kind 1): header | mask | uptr | records | lists.  A unit's record has a fixed size and
 // sits at a fixed place, so that it streams from HBM with one bulk copy whose address needs no
 // look-up; the list of its FP8 blocks follows in the lists section, found through uptr.
+//   mask      256 B per unit: uint16 per row of the tile, bit j set if the row's block in column j is FP8 (zero
+//                       in rows beyond the tensor)
 //   REC_W4    16384 B : one 8-byte slot per block, row r of the tile = 128 bytes whose 16-byte pieces are
 //                       XOR-swizzled with (r & 7) -- the 128B-swizzled K-major tile tcgen05 reads: the 16
 //                       E2M1 codes of an NVFP4 block, or E4M3 codes 0..7 of an FP8 block (which the tensor
@@ -22,12 +25,11 @@
 //   REC_SF     2048 B : E4M3 microscales, 0x00 for FP8 blocks, in the order the scales go to tensor
 //                       memory: four 512-byte tiles (one per MMA step of 64 elements), in a tile 16 bytes
 //                       per r % 32, there 4 bytes per r / 32, there one byte per block of the step
-//   REC_KBSTART 128 B : uint16 x 17 (padded): FP8 blocks of the unit before block column j; entry 16 = all
-// List of a unit with cnt FP8 blocks, ordered by (block column, row) so that blocks meeting the same 16
-// activation elements are neighbours: one uint32 per block (padded to 16 bytes) -- low half: where the
-// block's slot sits in REC_W4, high half: 16 * row + 4 * ((row / 2) % 4), the place of its row in a swizzled
-// [row][16 tokens] fp32 tile -- then E4M3 codes 8..15 of every block (8 bytes each, padded to 16).  uptr[u] (uint32, units + 1 entries) = start of
-// unit u's list in 16-byte steps from off_ovf.
+//   REC_KBSTART 128 B : uint16 x 17 (padded): FP8 blocks of the unit before row 8 i; entry 16 = all
+// List of a unit with cnt FP8 blocks, ordered by (row, block column), so that a thread that owns a row has its blocks
+// one after the other: one uint32 per block (padded to 16 bytes) -- low half: where the block's slot sits in REC_W4,
+// high half: 16 * row + 4 * ((row / 2) % 4) -- then E4M3 codes 8..15 of every block (8 bytes each, padded to 16).
+// uptr[u] (uint32, units + 1 entries) = start of unit u's list in 16-byte steps from off_ovf.
 //
 // Activations (kind 0): header | codes4 | sf | mask | arec | codes8.  codes4 is row-major, sf
 // uses 512-byte tiles over all rows, codes8 is a dense plane of which only FP8 blocks are
@@ -35,8 +37,7 @@
 // token rows (rows >= M are zero):
 //   AREC_A4   2048 B : the E2M1 codes as a 16-row x 128-byte tile, swizzled like REC_W4 (zero in FP8 blocks)
 //   AREC_SF    256 B : E4M3 microscales, [token][block column], 0x00 for FP8 blocks
-//   AREC_HOT    16 B : two uint32, one per token octet (readers use their OR): bit j set if block column j of some token is
-//                      FP8 ("hot" column); then padding
+//   AREC_HOT   256 B : not used
 //   AREC_AT   8192 B : the value over the tensor scale of every element in fp16 (E2M1 x microscale, or E4M3 x
 //                      2^ratio; exact): token octet m / 8 in its own 4096 bytes, there 256 bytes per block
 //                      column, there 32 bytes per token -- what a warp reads for one column is contiguous
@@ -79,7 +80,7 @@ __host__ __device__ inline PackedLayout fgmp_layout(int64_t rows, int64_t K, int
         L.off_arec = o;    if (rows <= 16) o = fgmp_align1k(o + (size_t)L.chunks * AREC_BYTES);
         L.off_codes8 = o;  o = fgmp_align1k(o + (size_t)rows * (size_t)K);
     } else {
-        L.off_mask = o;    o = fgmp_align1k(o + (size_t)rows * (size_t)L.MW * 4);
+        L.off_mask = o;    o = fgmp_align1k(o + (size_t)L.units * 256);
         L.off_uptr = o;    o = fgmp_align1k(o + ((size_t)L.units + 1) * 4);
         L.off_rec = o;     o = fgmp_align1k(o + (size_t)L.units * REC_BYTES);
         // 12 bytes per FP8 block, and up to 24 bytes of padding per unit
@@ -114,43 +115,35 @@ __host__ __device__ inline uint32_t fgmp_list_entry(uint32_t r, uint32_t j)
 }
 
 #ifdef __CUDACC__
-// Where the FP8 blocks of one unit sit in its list.  Called by all 128 threads of a CTA, thread
-// i = row i of the tile, m16 = that row's 16 mask bits of the chunk (0 beyond the last row).
-// On return s_pos[row * 16 + j] = index of block (row, j) among the unit's FP8 blocks in (column, row)
-// order (0xffff if the block is not FP8), s_cnt[j] = FP8 blocks in column j, and the return value is
-// their total.  s_warp is scratch of 64 words.  Ends with a __syncthreads().
-__device__ __forceinline__ uint32_t fgmp_unit_positions(uint32_t m16, uint32_t* s_warp, uint16_t* s_pos, uint32_t* s_cnt)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    uint32_t rank[16];
-#pragma unroll
-    for (int kb = 0; kb < 16; ++kb) {
-        const uint32_t bal = __ballot_sync(0xffffffffu, (m16 >> kb) & 1u);
-        rank[kb] = __popc(bal & ((1u << lane) - 1u));
-        if (lane == 0) s_warp[w * 16 + kb] = __popc(bal);
-    }
-    __syncthreads();
-    uint32_t run = 0;
-#pragma unroll
-    for (int kb = 0; kb < 16; ++kb) {
-        const uint32_t c0 = s_warp[kb], c1 = s_warp[16 + kb], c2 = s_warp[32 + kb], c3 = s_warp[48 + kb];
-        const uint32_t below = (w > 0 ? c0 : 0u) + (w > 1 ? c1 : 0u) + (w > 2 ? c2 : 0u);
-        s_pos[threadIdx.x * 16 + kb] = ((m16 >> kb) & 1u) ? (uint16_t)(run + below + rank[kb]) : (uint16_t)0xffff;
-        if (threadIdx.x == 0) s_cnt[kb] = c0 + c1 + c2 + c3;
-        run += c0 + c1 + c2 + c3;
-    }
-    __syncthreads();
-    return run;
-}
+// Where the FP8 blocks of one unit sit in its list, for 128 threads: thread i brings the 16 mask bits of row i of the
+// tile (0 beyond the last row).
+struct UnitScratch {
+    uint32_t warp[4];
+    uint16_t m16[128], base[128];        // mask bits of a row; FP8 blocks of the unit before it
 
-// the 16 mask bits of (row r, chunk c) of a packed tensor; 0 beyond the last row
-__device__ __forceinline__ uint32_t fgmp_chunk_mask(const uint32_t* mask, const PackedLayout& L, int64_t r, int64_t c)
-{
-    if (r >= L.rows) return 0u;
-    return (mask[r * L.MW + (c >> 1)] >> ((c & 1) * 16)) & 0xffffu;
-}
-
-struct UnitScratch { uint32_t warp[64]; uint32_t cnt[16]; uint16_t pos[128 * 16]; };
+    // fills the tables, returns the unit's number of FP8 blocks; ends with a __syncthreads()
+    __device__ __forceinline__ uint32_t init(uint32_t bits)
+    {
+        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+        const uint32_t own = __popc(bits);
+        uint32_t incl = own;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+        if (lane == 31) warp[w] = incl;
+        __syncthreads();
+        const uint32_t c0 = warp[0], c1 = warp[1], c2 = warp[2], c3 = warp[3];
+        m16[threadIdx.x] = (uint16_t)bits;
+        base[threadIdx.x] = (uint16_t)(incl - own + (w > 0 ? c0 : 0u) + (w > 1 ? c1 : 0u) + (w > 2 ? c2 : 0u));
+        __syncthreads();
+        return c0 + c1 + c2 + c3;
+    }
+    // index of block (row, j) among the unit's FP8 blocks; 0xffff if it is NVFP4
+    __device__ __forceinline__ uint32_t pos(int row, int j) const
+    {
+        const uint32_t m = m16[row];
+        return (m >> j) & 1u ? base[row] + __popc(m & ((1u << j) - 1u)) : 0xffffu;
+    }
+};
 
 // Visits every block of one unit of a packed weight tensor, 128 threads per unit, consecutive
 // threads on consecutive blocks of one row: f(row, kb, row in tile, column in chunk, rec, hi) with
@@ -161,9 +154,7 @@ __device__ __forceinline__ void fgmp_for_each_block(const uint8_t* blob, const P
                                                     UnitScratch& sc, F f)
 {
     const int64_t tile = unit / L.chunks, c = unit % L.chunks;
-    const uint32_t* mask = reinterpret_cast<const uint32_t*>(blob + L.off_mask);
-    const uint32_t m16 = fgmp_chunk_mask(mask, L, tile * 128 + threadIdx.x, c);
-    const uint32_t cnt = fgmp_unit_positions(m16, sc.warp, sc.pos, sc.cnt);
+    const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x]);
     const uint8_t* rec = blob + L.off_rec + (size_t)unit * REC_BYTES;
     const uint8_t* halves = blob + L.off_ovf + (size_t)reinterpret_cast<const uint32_t*>(blob + L.off_uptr)[unit] * 16 + fgmp_list_halves_offset(cnt);
     const int j = threadIdx.x & 15;
@@ -172,7 +163,7 @@ __device__ __forceinline__ void fgmp_for_each_block(const uint8_t* blob, const P
         const int row = (threadIdx.x >> 4) + 8 * i;
         const int64_t r = tile * 128 + row, kb = c * 16 + j;
         if (r >= L.rows || kb >= L.KB) continue;
-        const uint32_t pos = sc.pos[row * 16 + j];
+        const uint32_t pos = sc.pos(row, j);
         f(r, kb, row, j, rec, pos != 0xffffu ? halves + (size_t)pos * 8 : (const uint8_t*)nullptr);
     }
     __syncthreads();

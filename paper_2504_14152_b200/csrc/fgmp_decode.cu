@@ -1,98 +1,119 @@
-// fgmp_linear for decode-sized batches (M <= 16 tokens): a weight-streaming kernel that
-// reads the packed weights exactly once (Section 4.1 of the paper: the four block-pair
-// products, FP32 accumulation), optionally with the activation quantizer of Section 4.2 in
-// its prologue (fgmp_linear_fused).
+// fgmp_linear for decode-sized batches (M <= 16 tokens): a weight-streaming kernel that reads the packed weights
+// exactly once (Section 4.1 of the paper: the four block-pair products, FP32 accumulation), optionally with the
+// activation quantizer of Section 4.2 in front of it (fgmp_linear_fused).
 //
-// At this size the layer is bound by the weight stream.  Converting packed codes to a common number
-// format in the SIMT pipes costs more instructions per byte than the stream leaves time for (an E2M1
-// pair takes a byte extraction, a conversion and a scale multiply), so the bulk of the products must
-// not be converted at all.  Decomposition (exact), with the FP8 blocks as the exceptions:
-//   (1) NVFP4 weight block x NVFP4 activation block: tcgen05.mma kind::mxf4nvf4 straight from the
-//       packed codes, E4M3 block scales in tensor memory, FP32 accumulation there; weights are the
-//       128-row operand, the 16 tokens are N.  A block that must not take part gets a zero scale: the
-//       record stores scale 0 for FP8 weight blocks, the activation record for FP8 activation blocks,
-//       and the scales of every token are zeroed in "hot" block columns (those in which some token of
-//       the batch is FP8), which are left to (3) as a whole.
-//   (2) FP8 weight block x any activation block: mma.sync m16n8k16 on exact fp16 values (an E4M3 code
-//       has 4 significant bits; the activation record holds every activation over its tensor scale in
-//       fp16, exact for either format).  A record lists its FP8 blocks by block column, so sixteen
-//       blocks that meet the same 16 activation elements form the M side; the sums are added to their
-//       rows in a [row][token] tile private to the warp.
-//   (3) NVFP4 weight block x any activation block in a hot column: the column's weights are dequantized
-//       in registers (exact in fp16: 6 significant bits) for mma.sync, 32 rows per warp, sums in registers.
-// Every block pair is in exactly one of the three.  With 10 % FP8 blocks that concentrate in few block
-// columns (outlier channels) (2) and (3) are small; with unstructured activation masks (3) grows towards
-// the whole tensor and the kernel is as fast as its SIMT conversions allow.
+// At this size the layer is bound by the weight stream (a 22 KiB unit of 128 rows x 256 elements every 885 clocks per
+// SM), so the weights must not be converted in the SIMT pipes.  All products run on tcgen05, and what does not fit one
+// operand format is split on the ACTIVATION side, which is small and is prepared once per call.  A tcgen05.mma with
+// M = 128 takes N/2 clocks, but at least 40 when its weights come from shared memory (4 KiB at 128 bytes a clock), so that
+// up to 64 extra columns cost nothing there.
+//   (1) NVFP4 weight blocks x all activations: kind::mxf4nvf4 on the packed codes, E4M3 block scales in tensor memory.
+//       Token m is row m of the activation operand with its NVFP4 blocks.  An FP8 activation block is written as
+//       digits: its E4M3 values are multiples of 2^-9 below 2^9, i.e. 18-bit integers, and six base-8 digits, each of
+//       them an E2M1 value, with block scales 2^(3p - 8), p = 0..5, represent them exactly.  Digit p of token m is row
+//       (p + 1) M + m.  A block that must not take part has scale 0: FP8 weight blocks in the record, the other
+//       format's blocks in the rows of either kind.
+//   (2) FP8 weight blocks x all activations: kind::f8f6f4 on a dense E4M3 tile of the unit that holds its FP8 blocks
+//       and zeros elsewhere, in tensor memory (a thread per row puts it there: from shared memory the tile would cost eight
+//       times 40 clocks, from tensor memory N/2 = 8 to 16 each).  Every activation over its tensor scale has at most 6
+//       significant bits (E2M1 x E4M3 scale; E4M3 x 2^ratio has 4), so it is the exact sum of two E5M2 values: rows m and
+//       M + m.
+//   The epilogue adds the columns of a token: row + 2^ratio_a * digits + 2^ratio_w * (high + low).
+// 12 instructions and about 300 tensor clocks per unit for any mix of formats; the SIMT work that is left is moving the
+// unit's FP8 blocks and its block scales into tensor memory.
 //
-// Work is split stream-K style over (128-row tile, 256-element K chunk) units so that all SMs
-// stream the same number of bytes; a unit is three bulk copies (its fixed-size record, the list of
-// its FP8 blocks, the activation record of its chunk) into a ring of stages.  Tiles shared by several
-// CTAs are reduced in a fixed order by the CTA that arrives last.  Every sum is taken in a fixed
-// order: results are reproducible bit for bit.
+// Work is split stream-K style over (128-row tile, 256-element K chunk) units so that all SMs stream the same number of
+// bytes.  Tiles shared by several CTAs are reduced in a fixed order by the CTA that arrives last: results are
+// reproducible bit for bit.
 //
-// Warp roles (576 threads): warp 0 = producer, warp 1 = MMA issuer and owner of the tensor memory,
-// warps 2-9 = (2): two sets of four warps that take alternate units, four block columns per warp (a warp
-// copies what it needs of a unit into registers and gives the stage back at once), warps 10-13 = (3), 32
-// rows each, warps 14-17 = block scales into tensor memory unit by unit and, at the end of a tile, the
-// epilogue (one lane quadrant each).
+// Where the activation operand (a "step record" per chunk) comes from:
+//   DEC_FUSED_LP, DEC_FUSED_HP  fused calls (by block score): the CTAs share out the quantizer's work, write the records to
+//                the workspace and stream them from there; the first weight copies are in flight meanwhile.
+//   DEC_UNPACK   fgmp_linear: made unit by unit in shared memory from the packed activations' records.
+//
+// Warp roles (480 threads): warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, warps 2-9 = a
+// unit's block scales and FP8 blocks into tensor memory (and before that the quantizer, or the step record of the unit), two
+// sets of four warps that take alternate units and own one dense tile each, warps 10-13 = epilogue (one lane quadrant each),
+// warp 14 = step-record producer.
+//
+// The roles run different code at the same time, a warp or two per scheduler, so a unit costs what its instructions cost to
+// fetch and issue: what a loop needs once per unit is not unrolled or inlined twice, and a unit passes through few hands
+// (producer -> set -> MMA -> producer).  Measured at 70B FC1, one token, time per unit and SM (HBM alone: 0.46 us): SIMT
+// corrections for the FP8 blocks 0.66 us; their products on the tensor core with 109 KiB of code, the dense tile in shared
+// memory and the scales loaded by warps of their own 0.62 to 0.72 us; this form 0.52 us.
 #include "fgmp_common.cuh"
 #include "fgmp_actq.cuh"
 #include "fgmp_host.h"
 #include "fgmp_ptx.cuh"
 #include <cuda_fp16.h>
 #include <mutex>
-#include <type_traits>
 
 namespace {
 
-constexpr int DEC_WARPS = 18, DEC_THREADS = 32 * DEC_WARPS;
-constexpr int W_PROD = 0, W_MMA = 1, W_FP8 = 2, W_HOT = 10, W_EPI = 14;
-constexpr int FP8_WARPS = W_HOT - W_FP8;        // two sets of four: a set takes every second unit
-constexpr int Q_THREADS = 32 * 16;              // warps 2..17 share out the prologue quantizer
-constexpr int TOK = 16;                         // MMA N (token rows, zero padded)
-constexpr uint32_t LIST_CAP = 3968;             // bytes of a unit's FP8 list that fit a stage (about 330 blocks); more is read from global
-constexpr uint32_t STG_LIST = REC_BYTES;                                                         // 18560
-constexpr uint32_t STG_A = STG_LIST + LIST_CAP;                                                  // 22528, 1 KiB aligned
-constexpr uint32_t DEC_STAGE_BYTES = 33792;
-constexpr int DEC_STAGES = 4;
-constexpr int NTILES = FP8_WARPS + 1;           // [row][token] fp32 tiles: one per (2) warp, one shared by the (3) warps
-constexpr uint32_t TILE_FLOATS = 128 * TOK;
-constexpr uint32_t SF_COL0 = 32;                // tensor memory: 2 x 16 accumulator columns, then 32 scale columns per stage
-constexpr uint32_t DEC_TMEM_COLS = 256;
-constexpr size_t DEC_SMEM = (size_t)DEC_STAGES * DEC_STAGE_BYTES + NTILES * TILE_FLOATS * 4 + 1024 /*alignment*/ + 512 /*barriers*/;
-static_assert(STG_A % 1024 == 0 && STG_A + AREC_BYTES <= DEC_STAGE_BYTES, "stage layout");
-static_assert(DEC_SMEM <= 232448, "shared memory of one CTA");
-static_assert(SF_COL0 + 32 * DEC_STAGES <= DEC_TMEM_COLS, "tensor memory columns");
+constexpr int DEC_WARPS = 15, DEC_THREADS = 32 * DEC_WARPS;
+constexpr int W_PROD = 0, W_MMA = 1, W_SET = 2, W_EPI = 10, W_STEP = 14;
+constexpr int SET_THREADS = 128;                // one set of FP8 warps
+constexpr int Q_THREADS = 2 * SET_THREADS;      // both sets share out the quantizer's work items
+constexpr int PIECES = 6;                       // base-8 digits of an FP8 activation block
+constexpr uint32_t STG_MASK = REC_BYTES, STG_LIST = STG_MASK + 256;          // the unit's mask, the list of its FP8 blocks
+constexpr uint32_t LIST_CAP = 3712;             // bytes of the list that fit a stage (about 305 blocks); more is read from global
+constexpr uint32_t STG_STEP = STG_LIST + LIST_CAP;                           // 22528, 1 KiB aligned: step record, then packed activation record (DEC_UNPACK)
+constexpr int DEC_MAX_STAGES = 6;
+// tensor memory columns: accumulators (two buffers of 112 and of 32); of each set: a dense E4M3 tile of 64, scales (32)
+constexpr uint32_t D4_COL = 0, D8_COL = 224, DENSE_COL = 288, SF_COL = 416;
+constexpr uint32_t DEC_TMEM_COLS = 512;
+constexpr size_t SMEM_LIMIT = 232448;
+static_assert(STG_STEP % 1024 == 0, "stage layout");
+static_assert(SF_COL + 32 * 2 <= DEC_TMEM_COLS, "tensor memory columns");
 
-// kind::mxf4nvf4, E2M1 x E2M1, UE4M3 scales, K-major operands, M = 128, N = 16, dense K = 64
-constexpr uint32_t IDESC_NVF4 = (1u << 7) | (1u << 10) | ((uint32_t)(TOK >> 3) << 17) | (0u << 23) | ((uint32_t)(128 >> 4) << 24);
+enum { DEC_FUSED_LP = 0, DEC_FUSED_HP = 1, DEC_UNPACK = 2 };      // the first two are the fgmp_score_mode of the quantizer
+
+// Step record of a chunk for a batch of M tokens: n4 rows x 128 bytes of E2M1 codes | 2 KiB of block scales in tensor-
+// memory order | n8 rows x 128 bytes of E5M2 values of elements 0..127 | the same of elements 128..255.  Both code tiles
+// are K-major with 16-byte pieces XOR-swizzled by the row.  Rows that no token uses are left as they are: they only
+// reach accumulator columns that nobody reads.
+__host__ __device__ inline uint32_t step_n4(int64_t M) { return (uint32_t)(((PIECES + 1) * M + 15) & ~15); }
+__host__ __device__ inline uint32_t step_n8(int64_t M) { return (uint32_t)((2 * M + 15) & ~15); }
+__host__ __device__ inline uint32_t step_bytes(int64_t M) { return step_n4(M) * 128u + 2048u + step_n8(M) * 256u; }
+
+// instruction descriptors without N, M = 128, K-major operands: E2M1 x E2M1 with UE4M3 scales; E4M3 x E5M2
+constexpr uint32_t IDESC_NVF4 = (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);
+constexpr uint32_t IDESC_E4M3_E5M2 = (1u << 4) | (0u << 7) | (1u << 10) | ((uint32_t)(128 >> 4) << 24);
 
 // shared-memory matrix descriptors as (low word | start address >> 4, constant high word)
 constexpr uint32_t SW128_LO = 1u << 16, SW128_HI = (1024u >> 4) | (1u << 14) | (2u << 29);   // 128B swizzle, 8-row groups 1 KiB apart
-__device__ __forceinline__ uint64_t desc64(uint32_t lo, uint32_t hi)
+__device__ __forceinline__ uint64_t desc64(uint32_t lo)
 {
     uint64_t d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(hi));
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "r"(lo), "r"(SW128_HI));
     return d;
+}
+// A (128 rows) from tensor memory: lane = row, four bytes of K per column
+__device__ __forceinline__ void umma_f8f6f4_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], [%1], %2, %3, p;\n\t}"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
 // control words of the workspace (int32, from byte 256): see fgmp_linear_fused
-enum { CW_DONE = 1, CW_CLAIM = 2, CW_QCOUNT = 3, CW_QREADY = 4 };
+enum { CW_DONE = 1, CW_CLAIM = 2, CW_QCOUNT = 3 };
 
 struct DecParams {
     const uint8_t* wblob; const uint8_t* ablob;
     PackedLayout LW, LA;
     float* Y; void* Ybf; int64_t ldy; int y_is_bf16;
     int64_t M, N, K;
-    int64_t total;            // tiles * chunks
-    int64_t chunks;
+    uint32_t chunks;
+    uint32_t span, rest;      // units per CTA: span + 1 for the first `rest` CTAs, span for the others
     int* status; uint32_t* counters; float* partials; int maxseg;
-    // activation quantizer in the prologue (fused launches only)
+    uint32_t stages, stage_bytes;
+    // activation quantizer in front (fused launches only)
     const uint8_t* X; int64_t ldx;        // bf16 [M, ldx]
     const float* fisher;
-    ActQuantScalars q; int q_mode;        // q_mode: fgmp_score_mode
-    uint8_t* arec;                        // where the records of the chunks go (and are streamed from)
-    uint8_t* q_codes4; uint8_t* q_sf; uint8_t* q_mask; uint8_t* q_codes8; fgmp_packed_header* q_header;   // optional packed output
+    ActQuantScalars q;
+    uint8_t* steps;                       // the chunks' step records
+    uint8_t* q_codes4; uint8_t* q_sf; uint8_t* q_mask; uint8_t* q_codes8; uint8_t* q_arec; fgmp_packed_header* q_header;   // optional packed output
     uint32_t* cw;                         // control words
 };
 
@@ -107,17 +128,14 @@ __device__ unsigned long long* g_timeline = nullptr;
 #define FGMP_STAMP_ANY(slot) do { } while (0)
 #endif
 
-__device__ __forceinline__ int64_t cta_of_unit(int64_t i, int64_t G, int64_t total) { return ((i + 1) * G - 1) / total; }
+__device__ __forceinline__ uint32_t span_begin(const DecParams& p, uint32_t cta) { return cta * p.span + min(cta, p.rest); }
+__device__ __forceinline__ uint32_t cta_of_unit(const DecParams& p, uint32_t u)
+{
+    const uint32_t longer = p.rest * (p.span + 1);
+    return u < longer ? u / (p.span + 1) : p.rest + (u - longer) / p.span;
+}
 
 __device__ __forceinline__ void quant_bar() { asm volatile("bar.sync 1, %0;" ::"n"(Q_THREADS) : "memory"); }
-
-// A correction tile holds [128 rows][16 tokens] fp32, a row = 64 bytes = four 16-byte pieces of
-// four tokens; piece index is XOR-ed with (row >> 1) & 3 so that 32 lanes reading one piece of 32
-// consecutive rows (the epilogue) do not collide on banks.  Float index of (row, token):
-__device__ __forceinline__ uint32_t tile_idx(uint32_t row, uint32_t token)
-{
-    return row * 16u + ((((token >> 2) ^ (row >> 1)) & 3u) << 2) + (token & 3u);
-}
 
 // Bounded wait for a word in global memory to take a value that another CTA publishes.
 __device__ __noinline__ bool wait_global_equals(const uint32_t* addr, uint32_t value, volatile int* abort_flag, int* status, int where)
@@ -134,625 +152,512 @@ __device__ __noinline__ bool wait_global_equals(const uint32_t* addr, uint32_t v
             atomicExch(status + 1, where);
             return false;
         }
-        __nanosleep(100);
+        __nanosleep(20);
     }
 }
 
-// One work item of the prologue quantizer: chunk c (256 elements) of the eight token rows of octet o.  Run by
-// the 16 warps 2..17: warp wq takes token 8o + wq/2 and the eight blocks 8(wq%2) .. +7 of the chunk, four lanes
-// per block.  s_hot: one word of shared memory.  Each octet has its own word for the chunk's hot block columns.
-template <int MODE>
-__device__ __forceinline__ void quantize_chunk(const DecParams& p, int64_t c, int o, uint32_t* s_hot)
+__device__ __forceinline__ uint32_t f32x2_to_e5m2x2(float lo, float hi)
 {
-    const uint32_t tq = threadIdx.x - 64u;                 // index among the quantizer's threads
-    const uint32_t wq = tq >> 5, lane = tq & 31u, li = lane & 3u;
-    const uint32_t j = 8u * (wq & 1u) + (lane >> 2);
-    const int64_t kb = 16 * c + j;
-    uint8_t* rec = p.arec + (size_t)c * AREC_BYTES;
-    if (tq == 0) *s_hot = 0u;
-    quant_bar();
-    const uint32_t m = 8u * (uint32_t)o + (wq >> 1);
-    const bool live = (int64_t)m < p.M;
-    uint2 xin = make_uint2(0u, 0u);
-    float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (live) {
-        xin = __ldg(reinterpret_cast<const uint2*>(p.X + ((size_t)m * p.ldx + (size_t)kb * 16 + 4 * li) * 2));
-        f = __ldg(reinterpret_cast<const float4*>(p.fisher + kb * 16 + 4 * li));
+    uint16_t r;
+    asm("cvt.rn.satfinite.e5m2x2.f32 %0, %1, %2;" : "=h"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+__device__ __forceinline__ float2 e5m2x2_to_f32x2(uint32_t two)
+{
+    uint32_t h2;
+    asm("cvt.rn.f16x2.e5m2x2 %0, %1;" : "=r"(h2) : "h"((uint16_t)two));
+    return __half22float2(*reinterpret_cast<__half2*>(&h2));
+}
+
+// The six digits of the E4M3 magnitude `code` (0..126) as E2M1 codes, digit p in bits 4p .. 4p+3.  Base 8, lowest first:
+// the magnitude in units of 2^-9 is an integer of at most 18 bits, a digit d stands for the E2M1 value d / 2.  The top
+// digit is at most 7; 5 and 7 are no E2M1 values (in halves): 5 = 6 - 1 and 7 = 6 + 1 with the 1 as -8 or 8 in the digit
+// below, which is 0 or -4 then (the magnitude has four significant bits).
+__device__ __forceinline__ uint32_t e4m3_digits(uint32_t code)
+{
+    int a = __float2int_rn(e4m3_to_f32(code) * 512.0f);
+    int d[PIECES];
+#pragma unroll
+    for (int p = 0; p < PIECES - 1; ++p) {
+        d[p] = ((a + 4) & 7) - 4;
+        a = (a - d[p]) >> 3;
     }
+    if (a == 5) { a = 6; d[PIECES - 2] -= 8; }
+    if (a == 7) { a = 6; d[PIECES - 2] += 8; }
+    d[PIECES - 1] = a;
+    uint32_t w = 0;
+#pragma unroll
+    for (int p = 0; p < PIECES; p += 2) w |= f32x2_to_e2m1x2(0.5f * (float)d[p], 0.5f * (float)d[p + 1]) << (4 * p);
+    return w;
+}
+
+// Writes what the step record `rec` (global or shared memory) holds of four consecutive elements of token m: quarter li of
+// block column j.  c4: their E2M1 codes and sc: the block's scale (NVFP4 block), or c8: their E4M3 codes (FP8 block);
+// v: the values over the tensor scale; digits: table of e4m3_digits.
+__device__ __forceinline__ void emit_step(uint8_t* rec, uint32_t M, uint32_t n4, uint32_t n8, uint32_t m, uint32_t j, uint32_t li,
+                                          bool is8, uint32_t c4, uint32_t sc, uint32_t c8, const float (&v)[4], const uint32_t* digits)
+{
+    uint8_t* sf = rec + n4 * 128u;
+    uint8_t* b8 = sf + 2048u + (j >> 3) * (n8 * 128u);
+    // E5M2 high and low parts
+    const uint32_t h0 = f32x2_to_e5m2x2(v[0], v[1]), h1 = f32x2_to_e5m2x2(v[2], v[3]);
+    const float2 f0 = e5m2x2_to_f32x2(h0), f1 = e5m2x2_to_f32x2(h1);
+    const uint32_t l0 = f32x2_to_e5m2x2(v[0] - f0.x, v[1] - f0.y), l1 = f32x2_to_e5m2x2(v[2] - f1.x, v[3] - f1.y);
     {
-        uint8_t* a4 = rec + AREC_A4 + fgmp_rec_w4_offset(m, j) + 2u * li;
-        uint8_t* at = rec + fgmp_arec_at_offset(m, j) + 8u * li;
-        if (!live) {                                        // token rows beyond the batch are zero
-            *reinterpret_cast<uint16_t*>(a4) = 0;
-            *reinterpret_cast<uint2*>(at) = make_uint2(0u, 0u);
-            if (li == 0) rec[AREC_SF + m * 16u + j] = 0;
-        } else {
-        const BlockQuarter r = quantize_block_quarter<MODE>(xin, f, p.q);
-        *reinterpret_cast<uint16_t*>(a4) = (uint16_t)r.c4;
-        *reinterpret_cast<uint2*>(at) = r.h;
+        const uint32_t r = m, q = M + m;
+        *reinterpret_cast<uint32_t*>(b8 + r * 128u + (((j & 7u) ^ (r & 7u)) << 4) + 4u * li) = h0 | (h1 << 16);
+        *reinterpret_cast<uint32_t*>(b8 + q * 128u + (((j & 7u) ^ (q & 7u)) << 4) + 4u * li) = l0 | (l1 << 16);
+    }
+    if (!is8) {
+        *reinterpret_cast<uint16_t*>(rec + fgmp_rec_w4_offset(m, j) + 2u * li) = (uint16_t)c4;
+    } else {
+        uint32_t d[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) d[i] = digits[(c8 >> (8 * i)) & 0x7fu] ^ (((c8 >> (8 * i)) & 0x80u) ? 0x888888u : 0u);
+        // digits p and p + 1 of the four elements: bytes 2 x (two elements)
+        const uint32_t e = (d[0] & 0x0f0f0fu) | ((d[1] & 0x0f0f0fu) << 4), o = ((d[0] >> 4) & 0x0f0f0fu) | (d[1] & 0xf0f0f0u);
+        const uint32_t g = (d[2] & 0x0f0f0fu) | ((d[3] & 0x0f0f0fu) << 4), h = ((d[2] >> 4) & 0x0f0f0fu) | (d[3] & 0xf0f0f0u);
+#pragma unroll
+        for (int p = 0; p < PIECES; ++p) {
+            const uint32_t r = (uint32_t)(p + 1) * M + m;
+            const uint32_t c = __byte_perm((p & 1) ? o : e, (p & 1) ? h : g, (p >> 1) | ((4 + (p >> 1)) << 4));
+            *reinterpret_cast<uint16_t*>(rec + fgmp_rec_w4_offset(r, j) + 2u * li) = (uint16_t)c;
+        }
+    }
+    // scales of the token's seven rows, two per lane: row 0 has the NVFP4 scale, digit p has 2^(3p - 8) in E4M3
+#pragma unroll
+    for (uint32_t e = 0; e < 2; ++e) {
+        const uint32_t i = 2u * li + e;
+        if (i <= (uint32_t)PIECES) {
+            const uint32_t digit_sc = i == 1 ? 0x02u : 0x10u + 0x18u * (i - 2u);
+            const uint32_t r = i * M + m;
+            sf[fgmp_rec_sf_offset(r, j)] = (uint8_t)(i == 0 ? (is8 ? 0u : sc) : (is8 ? digit_sc : 0u));
+        }
+    }
+}
+
+// One work item of the quantizer in front of a fused call: chunk c (256 elements) of the token rows 4 quad .. 4 quad + 3.
+// Run by the 256 threads of warps 2..9: 64 threads (two warps) per token, four lanes per block.
+template <int MODE>
+__device__ __forceinline__ void quantize_item(const DecParams& p, uint32_t c, uint32_t quad, const uint32_t* digits)
+{
+    const uint32_t tq = threadIdx.x - 32u * W_SET;         // index among the quantizer's threads
+    const uint32_t lane = tq & 31u, li = tq & 3u, j = (tq >> 2) & 15u;
+    const uint32_t m = 4u * quad + (tq >> 6), M = (uint32_t)p.M;      // the same for a whole warp
+    if (m >= M) return;
+    const int64_t kb = 16 * (int64_t)c + j;
+    const uint2 xin = __ldg(reinterpret_cast<const uint2*>(p.X + ((size_t)m * p.ldx + (size_t)kb * 16 + 4 * li) * 2));
+    const float4 f = __ldg(reinterpret_cast<const float4*>(p.fisher + kb * 16 + 4 * li));
+    const BlockQuarter r = quantize_block_quarter<MODE>(xin, f, p.q);
+    const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&r.h.x)), vb = __half22float2(*reinterpret_cast<const __half2*>(&r.h.y));
+    const float v[4] = {va.x, va.y, vb.x, vb.y};
+    emit_step(p.steps + (size_t)c * step_bytes(M), M, step_n4(M), step_n8(M), m, j, li, r.is8, r.c4, r.sc, r.c8, v, digits);
+    if (p.q_codes4) {
+        uint8_t* rec = p.q_arec + (size_t)c * AREC_BYTES;
+        *reinterpret_cast<uint16_t*>(rec + AREC_A4 + fgmp_rec_w4_offset(m, j) + 2u * li) = (uint16_t)r.c4;
+        *reinterpret_cast<uint2*>(rec + fgmp_arec_at_offset(m, j) + 8u * li) = r.h;
         if (li == 0) rec[AREC_SF + m * 16u + j] = (uint8_t)r.sc;
         const uint32_t bal = __ballot_sync(0xffffffffu, r.is8 && li == 0);
         uint32_t byte = 0;
 #pragma unroll
         for (int b = 0; b < 8; ++b) byte |= ((bal >> (4 * b)) & 1u) << b;
-        if (lane == 0 && byte) atomicOr(s_hot, byte << (8u * (wq & 1u)));
-        if (p.q_codes4) {
-            const int64_t MW = p.LA.MW;
-            *reinterpret_cast<uint16_t*>(p.q_codes4 + ((int64_t)m * p.K) / 2 + kb * 8 + li * 2) = (uint16_t)r.c4;
-            if (li == 0) p.q_sf[fgmp_sf_offset(m, kb, p.K)] = (uint8_t)r.sc;
-            if (r.is8) *reinterpret_cast<uint32_t*>(p.q_codes8 + (int64_t)m * p.K + kb * 16 + 4 * li) = r.c8;
-            if (lane == 0) {
-                uint8_t* mb = p.q_mask + (size_t)m * MW * 4 + (kb >> 3);    // lane 0: first block of the warp's eight
-                mb[0] = (uint8_t)byte;
-                if (kb + 8 == p.LA.KB && (p.LA.KB & 31) != 0) { mb[1] = 0; mb[2] = 0; }   // rest of the row's last mask word
-            }
-        }
+        *reinterpret_cast<uint16_t*>(p.q_codes4 + ((int64_t)m * p.K) / 2 + kb * 8 + li * 2) = (uint16_t)r.c4;
+        if (li == 0) p.q_sf[fgmp_sf_offset(m, kb, p.K)] = (uint8_t)r.sc;
+        if (r.is8) *reinterpret_cast<uint32_t*>(p.q_codes8 + (int64_t)m * p.K + kb * 16 + 4 * li) = r.c8;
+        if (lane == 0) {
+            uint8_t* mb = p.q_mask + (size_t)m * p.LA.MW * 4 + (kb >> 3);    // lane 0: first block of the warp's eight
+            mb[0] = (uint8_t)byte;
+            if (kb + 8 == p.LA.KB && (p.LA.KB & 31) != 0) { mb[1] = 0; mb[2] = 0; }   // rest of the row's last mask word
         }
     }
-    quant_bar();
-    if (tq == 0) reinterpret_cast<uint32_t*>(rec + AREC_HOT)[o] = *s_hot;
 }
 
-// NH = token octets in use: 1 for M <= 8, else 2.  FUSED: the activation quantizer runs in the prologue.
-template <int NH, bool FUSED>
+template <int SRC>
 __global__ void __launch_bounds__(DEC_THREADS, 1)
-decode_kernel(DecParams p)
+decode_kernel(const __grid_constant__ DecParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     // 1 KiB aligned; an offset from the array keeps the pointer known to be shared memory (plain ld.shared / st.shared)
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    constexpr int S = DEC_STAGES;
-    float* tiles = reinterpret_cast<float*>(smem + (size_t)S * DEC_STAGE_BYTES);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tiles + NTILES * TILE_FLOATS);
-    // bars: [0,S) full, [S,2S) empty, [2S,3S) scales in tensor memory, then acc_full[2], acc_empty[2],
-    // corrections of a segment done [2], tiles free [1]
-    StageMeta* smeta = reinterpret_cast<StageMeta*>(bars + 3 * S + 8);
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smeta + S);
+    constexpr bool FUSED = SRC != DEC_UNPACK;
+    constexpr int X = DEC_MAX_STAGES;
+    const uint32_t S = p.stages;
+    const uint32_t M = (uint32_t)p.M, n4 = step_n4(M), n8 = step_n8(M), a_bytes = step_bytes(M);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * p.stage_bytes);
+    StageMeta* smeta = reinterpret_cast<StageMeta*>(bars + 4 * X + 4);
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smeta + X);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    volatile uint32_t* s_misc = reinterpret_cast<volatile uint32_t*>(abort_flag + 1);   // [1..2] claimed item, [3] hot columns of a chunk
+    volatile uint32_t* s_misc = reinterpret_cast<volatile uint32_t*>(abort_flag + 1);   // [1..2] claimed item
+    uint32_t* digits = const_cast<uint32_t*>(s_misc) + 4;                               // 128 entries
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = warp_index(), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) FGMP_STAMP_ANY(0);
-    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * S, sfr0 = empty0 + 8 * S;
-    const uint32_t accf0 = sfr0 + 8 * S, acce0 = accf0 + 16, cdone0 = acce0 + 16, tfree = cdone0 + 16;
-    constexpr uint32_t A_BYTES = NH == 2 ? AREC_BYTES : AREC_AT + 4096u;
+    // barriers of a stage: weights there, step record there, scales and dense tile in tensor memory, unit done (the stage and
+    // what it had in tensor memory are free); accumulators full / empty (two each)
+    const uint32_t wf0 = smem_u32(bars), sf0 = wf0 + 8 * X, rd0 = sf0 + 8 * X, dn0 = rd0 + 8 * X, accf0 = dn0 + 8 * X, acce0 = accf0 + 16;
 
     // this CTA's span of (tile, chunk) units
-    const int64_t G = gridDim.x, C = p.chunks;
-    const int64_t u_begin = ((int64_t)blockIdx.x * p.total) / G, u_end = ((int64_t)(blockIdx.x + 1) * p.total) / G;
-    const uint32_t* uptr = reinterpret_cast<const uint32_t*>(p.wblob + p.LW.off_uptr);
-    const uint8_t* recs = p.wblob + p.LW.off_rec;
+    const uint32_t G = gridDim.x, C = p.chunks;
+    const uint32_t u_begin = span_begin(p, blockIdx.x), u_end = span_begin(p, blockIdx.x + 1), n_units = u_end - u_begin;
     const uint8_t* lists = p.wblob + p.LW.off_ovf;
-    const uint8_t* arec = FUSED ? p.arec : p.ablob + p.LA.off_arec;
+    const bool has_fp8 = __ldg(&reinterpret_cast<const fgmp_packed_header*>(p.wblob)->n_fp8) != 0;
+    const uint32_t quads = (M + 3u) / 4u, n_items = quads * C;      // the quantizer's work items: (chunk, four tokens)
 
-    // One unit's copies into a stage (lane 0 of the producer warp): record and list, then the
-    // activation record of the unit's chunk
-    auto issue_w = [&](int64_t u, int stage, uint32_t step0, uint32_t step1) {
-        const uint32_t bytes = (step1 - step0) * 16u;
-        const uint32_t staged = bytes < LIST_CAP ? bytes : LIST_CAP;
-        smeta[stage].step = step0; smeta[stage].staged = staged;
-        const uint32_t fb = full0 + 8 * stage;
-        const uint32_t dst = smem_u32(smem + (size_t)stage * DEC_STAGE_BYTES);
-        mbar_expect_tx(fb, REC_BYTES + staged + A_BYTES);
-        bulk_load(dst, recs + (size_t)u * REC_BYTES, REC_BYTES, fb);
-        if (staged) bulk_load(dst + STG_LIST, lists + (size_t)step0 * 16, staged, fb);
-    };
-    auto issue_a = [&](int64_t u, int stage) {
-        bulk_load(smem_u32(smem + (size_t)stage * DEC_STAGE_BYTES) + STG_A, arec + (size_t)(u % C) * AREC_BYTES, A_BYTES, full0 + 8 * stage);
-    };
-
-    // ------------------------------------------------------------ set-up.  The packed weights are not written by
-    // whatever runs before this kernel, so the producer's part (barriers, the weight blob's header, the first
-    // stages' weight copies) may overlap the end of that kernel (programmatic dependent launch).
-    int64_t pf_base = u_begin;
-    uint32_t pf = 0;
-    int pre = 0;
-    if (warp == W_PROD) {
-        if (lane == 0) {
-            for (int s = 0; s < S; ++s) {
-                mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1 + 8); mbar_init(sfr0 + 8 * s, 4);
-            }
-            for (int b = 0; b < 2; ++b) {
-                mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 128); mbar_init(cdone0 + 8 * b, FP8_WARPS + 4);
-            }
-            mbar_init(tfree, 4);
-            *abort_flag = 0;
-            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // ------------------------------------------------------------ set-up
+    if (warp == W_PROD && lane == 0) {
+        for (uint32_t s = 0; s < S; ++s) {
+            mbar_init(wf0 + 8 * s, 1); mbar_init(sf0 + 8 * s, FUSED ? 1 : 4); mbar_init(rd0 + 8 * s, 4); mbar_init(dn0 + 8 * s, 1);
         }
-        // nothing is read through the blob's tables before its header has been seen to describe this call
-        const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
-        int okh = 1;
-        if (lane == 0) {
-            const uint2 mv = __ldg(reinterpret_cast<const uint2*>(hw));
-            okh = mv.x == FGMP_MAGIC && mv.y == 7u && __ldg(&hw->rows) == p.N && __ldg(&hw->K) == p.K &&
-                  __ldg(&hw->kind) == 1u && __ldg(&hw->error) == 0 && __ldg(&hw->fp8_scale_free) == 0;
-            if (!okh) { *abort_flag = 1; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, 9); }
-        }
-        okh = __shfl_sync(0xffffffffu, okh, 0);
-        if (okh) {
-            if (pf_base + lane <= p.total) pf = __ldg(uptr + pf_base + lane);
-            pre = (int)min((int64_t)S, u_end - u_begin);
-            for (int s = 0; s < pre; ++s) {
-                const uint32_t step0 = __shfl_sync(0xffffffffu, pf, s), step1 = __shfl_sync(0xffffffffu, pf, s + 1);
-                if (lane == 0) issue_w(u_begin + s, s, step0, step1);
-            }
-        }
+        for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 4); }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // The first of the quantizer's work items is asked for right away.  (This kernel may have started before the one
+    // before it in the stream has finished; that one lets it start only after its own last claim.)
+    if (FUSED && threadIdx.x == 32 * W_SET) s_misc[1] = atomicInc(p.cw + CW_CLAIM, n_items + G - 1u);
     if (warp == W_MMA) tmem_alloc(smem_u32(tmem_slot), DEC_TMEM_COLS);
-    if (warp >= W_FP8 && warp < W_EPI) {               // the tiles start at zero
-        float4* z = reinterpret_cast<float4*>(tiles);
-        for (int i = (warp - W_FP8) * 32 + lane; i < (int)(NTILES * TILE_FLOATS / 4); i += (W_EPI - W_FP8) * 32) z[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
+    if (warp >= W_EPI && warp < W_STEP) digits[threadIdx.x - 32 * W_EPI] = e4m3_digits(min(threadIdx.x - 32u * W_EPI, 126u));
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
     if (threadIdx.x == 0) FGMP_STAMP_ANY(1);
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    // Launched as a programmatic dependent of the preceding kernel in the stream, this kernel may have
-    // started before that one finished: everything above touches neither its output nor the workspace.
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (threadIdx.x == 0) FGMP_STAMP_ANY(2);
-    if (FUSED) {
-        // the first of the quantizer's work items is asked for right away
-        if (threadIdx.x == 64 && !*abort_flag) s_misc[1] = atomicInc(p.cw + CW_CLAIM, 2u * (uint32_t)C + (uint32_t)G - 1u);
-        __syncthreads();
-    }
-    const bool dead = *abort_flag != 0;                // the weight blob does not belong to this call: nothing else is read
 
-    if (FUSED && !dead && warp >= W_FP8) {
-        // The quantizer's work items (chunks) are handed out through a counter, so that every item is taken by
-        // a CTA that is running: no CTA ever waits for one that has not started.  The counter and the count of
-        // finished items wrap to zero with the call's last access.
-        const uint32_t n_items = 2u * (uint32_t)C;          // (chunk, token octet)
-        for (uint32_t it = 0;; ++it) {
-            const uint32_t item = s_misc[1 + (it & 1u)];
-            if (item >= n_items) break;
-            // the next item is asked for while this one is worked on
-            if (threadIdx.x == 64) s_misc[1 + ((it + 1u) & 1u)] = atomicInc(p.cw + CW_CLAIM, n_items + (uint32_t)G - 1u);
-            if (item == 0 && threadIdx.x == 64 && p.q_header) {
-                fgmp_packed_header* h = p.q_header;
-                h->magic = FGMP_MAGIC; h->version = 7; h->rows = p.M; h->K = p.K; h->scale_fp4 = p.q.s4;
-                h->fp8_log2_ratio = p.q.ratio; h->n_fp8 = (p.q.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
-                h->error = 0; h->scale_fp8 = p.q.s8; h->fp8_scale_free = 0;
-            }
-            if (p.q_mode == 0) quantize_chunk<0>(p, (int64_t)(item >> 1), (int)(item & 1u), const_cast<uint32_t*>(s_misc + 3));
-            else               quantize_chunk<1>(p, (int64_t)(item >> 1), (int)(item & 1u), const_cast<uint32_t*>(s_misc + 3));
-            // The item's stores become visible with the counter: the barrier orders them before the one thread's
-            // release, and the last arrival's acquire sees every earlier release of the counter.
-            quant_bar();
-            if (threadIdx.x == 64) {
-                uint32_t old;
-                asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(p.cw + CW_QCOUNT), "r"(n_items - 1u) : "memory");
-                if (old == n_items - 1u)
-                    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.cw + CW_QREADY), "r"(1u) : "memory");
-            }
-        }
-    }
-
-    if (threadIdx.x == 64) FGMP_STAMP_ANY(3);          // this CTA's share of the quantizer is done
-    if (dead) {
-    } else if (warp == W_PROD) {
-        // ------------------------------------------------------------ producer (whole warp; lane 0 issues)
-        int ok = 1;
-        if (lane == 0) {
-            if (FUSED) {
-                // every chunk's record is in place once the last work item of the quantizer has been handed in
-                ok = wait_global_equals(p.cw + CW_QREADY, 1u, abort_flag, p.status, 8) ? 1 : 0;
-                asm volatile("fence.proxy.async;" ::: "memory");   // records were written with ordinary stores, the bulk copy reads them
-            } else {
-                const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
-                const uint2 mv = __ldg(reinterpret_cast<const uint2*>(ha));
-                if (!(mv.x == FGMP_MAGIC && mv.y == 7u && __ldg(&ha->rows) == p.M && __ldg(&ha->K) == p.K && __ldg(&ha->kind) == 0u && __ldg(&ha->fp8_scale_free) == 0)) {
-                    *abort_flag = 1; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, 10);
-                    ok = 0;
+    if (warp == W_PROD) {
+        // ------------------------------------------------------------ weights producer (whole warp; lane 0 issues)
+        // The packed weights are not written by whatever runs before this kernel, so their first copies overlap the end
+        // of that kernel (programmatic dependent launch).  Nothing is read through the blob's tables before its header has
+        // been seen to describe this call.
+        const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
+        const uint2 mv = __ldg(reinterpret_cast<const uint2*>(hw));
+        const int64_t rows = __ldg(&hw->rows), k = __ldg(&hw->K);
+        const uint32_t kind = __ldg(&hw->kind);
+        const int err = __ldg(&hw->error), free8 = __ldg(&hw->fp8_scale_free);
+        int ok = mv.x == FGMP_MAGIC && mv.y == FGMP_LAYOUT_VERSION && rows == p.N && k == p.K && kind == 1u && err == 0 && free8 == 0;
+        int bad = ok ? 0 : 9;
+        const uint32_t arec_bytes = FUSED ? 0u : (M <= 8 ? AREC_AT + 4096u : AREC_BYTES);
+        const uint32_t* uptr = reinterpret_cast<const uint32_t*>(p.wblob + p.LW.off_uptr);
+        uint32_t pf_base = u_begin, pf = 0, stage = 0, phase = 1;
+        const uint32_t pre = min(S, n_units);
+        for (uint32_t i = 0; i <= n_units; ++i) {
+            if (i == pre || !ok) {
+                asm volatile("griddepcontrol.wait;" ::: "memory");
+                if (threadIdx.x == 0) FGMP_STAMP_ANY(2);
+                if (!FUSED) {
+                    const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
+                    if (ok && !(ha->magic == FGMP_MAGIC && ha->version == FGMP_LAYOUT_VERSION && ha->rows == p.M && ha->K == p.K && ha->kind == 0u && ha->fp8_scale_free == 0)) { ok = 0; bad = 10; }
+                    if (ok && lane < pre)              // the packed activation records of the stages under way
+                        bulk_load(smem_u32(smem + lane * p.stage_bytes) + STG_STEP + a_bytes, p.ablob + p.LA.off_arec + (size_t)((u_begin + lane) % C) * AREC_BYTES, arec_bytes, wf0 + 8 * lane);
                 }
+                if (bad && lane == 0) { *abort_flag = 1; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, bad); }
             }
-            if (ok) for (int s = 0; s < pre; ++s) issue_a(u_begin + s, s);
-            FGMP_STAMP_ANY(4);                         // all activation records are in place
-        }
-        ok = __shfl_sync(0xffffffffu, ok, 0);
-        int stage = pre % S; uint32_t phase = (uint32_t)(pre / S) & 1u;
-        for (int64_t u = u_begin + pre; u < u_end && ok; ++u) {
-            if (u + 1 - pf_base > 31) {                // next 32 list starts
+            if (!ok || i == n_units) break;
+            const uint32_t u = u_begin + i;
+            if (i == 0 || u + 1 - pf_base > 31) {      // next 32 list starts
                 pf_base = u;
-                pf = (pf_base + lane <= p.total) ? __ldg(uptr + pf_base + lane) : 0u;
+                pf = pf_base + lane <= u_end ? __ldg(uptr + pf_base + lane) : 0u;
             }
-            const uint32_t step0 = __shfl_sync(0xffffffffu, pf, (int)(u - pf_base));
-            const uint32_t step1 = __shfl_sync(0xffffffffu, pf, (int)(u + 1 - pf_base));
+            const uint32_t step0 = __shfl_sync(0xffffffffu, pf, (int)(u - pf_base)), step1 = __shfl_sync(0xffffffffu, pf, (int)(u + 1 - pf_base));
             if (lane == 0) {
-                ok = mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 1) ? 1 : 0;  /*lane*/
-                if (ok) { issue_w(u, stage, step0, step1); issue_a(u, stage); }
+                ok = mbar_wait(dn0 + 8 * stage, phase, abort_flag, p.status, 1) ? 1 : 0;
+                if (ok) {
+                    // one unit's copies: record, mask and list of the weights; the packed activation record goes with them
+                    const uint32_t staged = min((step1 - step0) * 16u, LIST_CAP);
+                    smeta[stage].step = step0; smeta[stage].staged = staged;
+                    const uint32_t fb = wf0 + 8 * stage, dst = smem_u32(smem + stage * p.stage_bytes);
+                    mbar_expect_tx(fb, REC_BYTES + 256u + staged + arec_bytes);
+                    bulk_load(dst, p.wblob + p.LW.off_rec + (size_t)u * REC_BYTES, REC_BYTES, fb);
+                    bulk_load(dst + STG_MASK, p.wblob + p.LW.off_mask + (size_t)u * 256, 256u, fb);
+                    if (staged) bulk_load(dst + STG_LIST, lists + (size_t)step0 * 16, staged, fb);
+                    if (!FUSED && i >= pre) bulk_load(dst + STG_STEP + a_bytes, p.ablob + p.LA.off_arec + (size_t)(u % C) * AREC_BYTES, arec_bytes, fb);
+                }
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (++stage == S) { stage = 0; phase ^= 1; }
         }
+    } else {
+        // Everything before this touches neither the preceding kernel's output nor (but for the claim) the workspace.
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (!FUSED) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+
+    if (FUSED && warp >= W_SET && warp < W_EPI) {
+        // ------------------------------------------------------------ quantizer
+        // Work items are handed out through a counter, so that every item is taken by a CTA that is running: no CTA
+        // ever waits for one that has not started.  The counter wraps to zero with the call's last claim.
+        for (uint32_t it = 0;; ++it) {
+            const uint32_t item = s_misc[1 + (it & 1u)];
+            if (item >= n_items) break;
+            // the next item is asked for while this one is worked on
+            if (threadIdx.x == 32 * W_SET) s_misc[1 + ((it + 1u) & 1u)] = atomicInc(p.cw + CW_CLAIM, n_items + G - 1u);
+            if (item == 0 && threadIdx.x == 32 * W_SET && p.q_header) {
+                fgmp_packed_header* h = p.q_header;
+                h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = p.M; h->K = p.K; h->scale_fp4 = p.q.s4;
+                h->fp8_log2_ratio = p.q.ratio; h->n_fp8 = (p.q.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
+                h->error = 0; h->scale_fp8 = p.q.s8; h->fp8_scale_free = 0;
+            }
+            quantize_item<SRC>(p, item / quads, item % quads, digits);
+            // The item's stores become visible with the count of finished items: the barrier orders them before the one
+            // thread's release.
+            quant_bar();
+            if (threadIdx.x == 32 * W_SET)
+                asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.cw + CW_QCOUNT), "r"(1u) : "memory");
+        }
+        if (threadIdx.x == 32 * W_SET) {
+            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // this CTA has made its last claim
+            FGMP_STAMP_ANY(3);
+        }
+    }
+
+    if (warp == W_STEP) {
+        // ------------------------------------------------------------ step-record producer
+        if (FUSED && lane == 0) {
+            // every chunk's record is in place once the last work item of the quantizer has been handed in
+            bool ok = wait_global_equals(p.cw + CW_QCOUNT, n_items, abort_flag, p.status, 8);
+            asm volatile("fence.proxy.async;" ::: "memory");   // records were written with ordinary stores, the bulk copy reads them
+            FGMP_STAMP_ANY(4);
+            uint32_t stage = 0, phase = 1, c = u_begin % C;
+            for (uint32_t i = 0; i < n_units && ok; ++i) {
+                if (!(ok = mbar_wait(dn0 + 8 * stage, phase, abort_flag, p.status, 13))) break;
+                mbar_expect_tx(sf0 + 8 * stage, a_bytes);
+                bulk_load(smem_u32(smem + stage * p.stage_bytes) + STG_STEP, p.steps + (size_t)c * a_bytes, a_bytes, sf0 + 8 * stage);
+                if (++stage == S) { stage = 0; phase ^= 1; }
+                if (++c == C) c = 0;
+            }
+        }
+        __syncwarp();
     } else if (warp == W_MMA) {
         // ------------------------------------------------------------ MMA issuer
-        // The whole warp walks the loop; lane 0 alone issues the tcgen05 instructions, so that every
-        // commit tracks every MMA before it.
-        const uint32_t smem0 = smem_u32(smem);
-        int stage = 0; uint32_t phase = 0; bool ok = true;
-        int seg = 0;
-        for (int64_t u = u_begin; u < u_end && ok; ++seg) {
-            const int64_t tile = u / C;
-            const int64_t seg_end = min(u_end, (tile + 1) * C);
-            const int acc = seg & 1; const uint32_t acc_phase = (uint32_t)((seg >> 1) & 1);
-            if (!(ok = mbar_wait_warp(acce0 + 8 * acc, acc_phase ^ 1, abort_flag, p.status, 2))) break;
+        // The whole warp walks the loop; one elected lane issues the tcgen05 instructions, so that every commit tracks
+        // every MMA before it.  The set that hands over a unit has seen the weights and the step record complete.
+        const uint32_t idesc4 = IDESC_NVF4 | ((n4 >> 3) << 17), idesc8 = IDESC_E4M3_E5M2 | ((n8 >> 3) << 17);
+        const uint32_t step_lo = (p.stage_bytes >> 4), b8_lo = (n4 * 128u + 2048u) >> 4, b8_half = n8 * 8u;
+        const uint32_t w_first = (smem_u32(smem) >> 4) | SW128_LO;
+        uint32_t stage = 0, phase = 0, w4 = w_first, left = C - u_begin % C, accum = 0, acc = 0, acc_phase = 1;
+        for (uint32_t i = 0; i < n_units; ++i) {
+            if (accum == 0) {                          // a tile begins
+                if (!mbar_wait_uniform(acce0 + 8 * acc, acc_phase, abort_flag, p.status, 2)) break;
+            }
+            if (!mbar_wait_uniform(rd0 + 8 * stage, phase, abort_flag, p.status, 8)) break;
+            if (i == 0 && lane == 0) FGMP_STAMP_ANY(5);
+            if (i == n_units - 1 && lane == 0) FGMP_STAMP_ANY(6);
             tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)(acc * TOK);
-            uint32_t accum = 0;
-            for (; u < seg_end && ok; ++u) {
-                if (!(ok = mbar_wait_warp(full0 + 8 * stage, phase, abort_flag, p.status, 3))) break;
-                if (!(ok = mbar_wait_warp(sfr0 + 8 * stage, phase, abort_flag, p.status, 8))) break;   // the scales are in tensor memory
-                if (u == u_begin && lane == 0) FGMP_STAMP_ANY(5);
-                if (u == u_end - 1 && lane == 0) FGMP_STAMP_ANY(6);
-                tc_fence_after();
-                const uint32_t sb = smem0 + (uint32_t)stage * DEC_STAGE_BYTES;
-                const uint32_t sf_t = tmem_base + SF_COL0 + (uint32_t)stage * 32;   // [0,16) weights, [16,32) tokens
-                const uint32_t w4_lo = ((sb + REC_W4) >> 4) | SW128_LO, a4_lo = ((sb + STG_A + AREC_A4) >> 4) | SW128_LO;
-                if (lane == 0) {
+            const uint32_t set = i & 1u, a4 = w4 + (STG_STEP >> 4), a8 = a4 + b8_lo;
+            const uint32_t d4 = tmem_base + D4_COL + acc * 112, d8 = tmem_base + D8_COL + acc * 32;
+            const uint32_t sf_t = tmem_base + SF_COL + set * 32, w8 = tmem_base + DENSE_COL + set * 64;
+            if (elect_one()) {
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        umma_nvf4(d_tmem, desc64(w4_lo + 2 * j, SW128_HI), desc64(a4_lo + 2 * j, SW128_HI), IDESC_NVF4,
-                                  sf_t + 4 * j, sf_t + 16 + 4 * j, accum);
-                        accum = 1;
-                    }
-                    umma_commit(empty0 + 8 * stage);
+                for (int j = 0; j < 4; ++j)
+                    umma_nvf4(d4, desc64(w4 + 2 * j), desc64(a4 + 2 * j), idesc4, sf_t + 4 * j, sf_t + 16 + 4 * j, j ? 1u : accum);
+                if (has_fp8) {
+#pragma unroll
+                    for (uint32_t k = 0; k < 8; ++k)
+                        umma_f8f6f4_ta(d8, w8 + 8 * k, desc64(a8 + (k >> 2) * b8_half + 2 * (k & 3u)), idesc8, k ? 1u : accum);
                 }
-                accum = 1;
-                __syncwarp();
-                if (++stage == S) { stage = 0; phase ^= 1; }
+                umma_commit(dn0 + 8 * stage);
             }
-            if (ok && lane == 0) umma_commit(accf0 + 8 * acc);
             __syncwarp();
+            accum = 1; w4 += step_lo;
+            if (++stage == S) { stage = 0; phase ^= 1; w4 = w_first; }
+            if (--left == 0 || i + 1 == n_units) {     // the tile (or this CTA's part of it) ends
+                if (elect_one()) umma_commit(accf0 + 8 * acc);
+                __syncwarp();
+                left = C; accum = 0;
+                acc ^= 1u;
+                if (acc == 0) acc_phase ^= 1u;
+            }
         }
-    } else if (warp < W_HOT) {
-        // ------------------------------------------------------------ (2): FP8 weight blocks of block columns bq, bq+4, bq+8, bq+12
-        // of every second unit.  The E4M3 codes go into the MMA as they are; the factor 2^ratio between the
-        // FP8 and NVFP4 tensor scales is applied once to the tile sums in the epilogue.
-        const int bq = (warp - W_FP8) & 3, par = (warp - W_FP8) >> 2;
-        const uint32_t g = lane >> 2, t = lane & 3;
-        float* mytile = tiles + (warp - W_FP8) * TILE_FLOATS;
-        const uint32_t tcol = (2 * t) & 3u, tpiece = t >> 1;
-        // tile[row][tokens] += sums of one group.  Within one column every block has its own row, so the
-        // read-modify-writes of a group touch distinct addresses: all loads first, then all stores.
-        // (tlA, tlB: the rows' places in the tile as the list gives them, 0xffff = no block)
-        const uint32_t tx = tpiece << 2;
-        auto group_add = [&](const float (&c)[4], const float (&d)[4], uint32_t tlA, uint32_t tlB) {
-            const uint32_t iA = (tlA ^ tx) + tcol, iB = (tlB ^ tx) + tcol;      // tokens 2t, 2t+1; tokens 8+2t, 9+2t are 8 floats on
-            float2 vA0 = make_float2(0.f, 0.f), vA1 = vA0, vB0 = vA0, vB1 = vA0;
-            if (tlA != 0xffffu) {
-                vA0 = *reinterpret_cast<const float2*>(mytile + iA);
-                if (NH == 2) vA1 = *reinterpret_cast<const float2*>(mytile + (iA ^ 8u));
-            }
-            if (tlB != 0xffffu) {
-                vB0 = *reinterpret_cast<const float2*>(mytile + iB);
-                if (NH == 2) vB1 = *reinterpret_cast<const float2*>(mytile + (iB ^ 8u));
-            }
-            if (tlA != 0xffffu) {
-                *reinterpret_cast<float2*>(mytile + iA) = make_float2(vA0.x + c[0], vA0.y + c[1]);
-                if (NH == 2) *reinterpret_cast<float2*>(mytile + (iA ^ 8u)) = make_float2(vA1.x + d[0], vA1.y + d[1]);
-            }
-            if (tlB != 0xffffu) {
-                *reinterpret_cast<float2*>(mytile + iB) = make_float2(vB0.x + c[2], vB0.y + c[3]);
-                if (NH == 2) *reinterpret_cast<float2*>(mytile + (iB ^ 8u)) = make_float2(vB1.x + d[2], vB1.y + d[3]);
-            }
-            __syncwarp();                  // a later group may add to the same rows
-        };
-        // blocks iA = e + g and iB = e + g + 8 of a group as the M side of the mma.sync (tokens 0-7 and 8-15 as N);
-        // c/d[0..1]: block iA, tokens 2t, 2t+1 / 8+2t, 9+2t; [2..3]: block iB
-        auto group_mma = [&](uint32_t rawA, uint32_t rawB, const uint2& bt0, const uint2& bt1, float (&c)[4], float (&d)[4]) {
-            uint32_t a0, a1, a2, a3;
-            asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(a0) : "h"((uint16_t)rawA));
-            asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(a2) : "h"((uint16_t)(rawA >> 16)));
-            asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(a1) : "h"((uint16_t)rawB));
-            asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(a3) : "h"((uint16_t)(rawB >> 16)));
-            c[0] = c[1] = c[2] = c[3] = 0.f; d[0] = d[1] = d[2] = d[3] = 0.f;
-            mma_f16_16816(c, a0, a1, a2, a3, bt0.x, bt0.y);
-            if (NH == 2) mma_f16_16816(d, a0, a1, a2, a3, bt1.x, bt1.y);
-        };
-
-        bool ok = true;
-        int seg = 0;
-        const int n_units = (int)(u_end - u_begin);
-        for (int sbeg = 0; sbeg < n_units && ok; ++seg) {
-            const int64_t tile = (u_begin + sbeg) / C;
-            const int send = (int)min((int64_t)n_units, (tile + 1) * C - u_begin);
-            // the epilogue has taken (and cleared) the previous segment's sums
-            if (seg > 0 && !(ok = mbar_wait_warp(tfree, (uint32_t)(seg - 1) & 1u, abort_flag, p.status, 7))) break;
-            for (int i = sbeg + ((par ^ sbeg) & 1); i < send; i += 2) {
-                const int stage = i % S; const uint32_t phase = (uint32_t)(i / S) & 1u;
-                if (!(ok = mbar_wait_warp(full0 + 8 * stage, phase, abort_flag, p.status, 5))) break;
-                const uint8_t* sb = smem + (size_t)stage * DEC_STAGE_BYTES;
-                const uint8_t* sa = sb + STG_A;
-                const uint32_t staged = smeta[stage].staged;
-                const uint8_t* list_g = lists + (size_t)smeta[stage].step * 16;
-                const uint16_t* kbs = reinterpret_cast<const uint16_t*>(sb + REC_KBSTART);
-                const uint32_t ntot = kbs[16];
-                const uint32_t hoff = fgmp_list_halves_offset(ntot);
-                const bool all = hoff + ntot * 8 <= staged;        // the whole list is in the stage (the usual case)
-                uint32_t st[4], en[4], rowA[8], rowB[8], rawA[8], rawB[8];     // [4 gr + cc]: group gr (blocks 16 gr ..) of column cc
-                uint2 bt0[4], bt1[4];
-                bool plain = all;                                  // ... and no column has more than two groups of 16
-#pragma unroll
-                for (int cc = 0; cc < 4; ++cc) {
-                    const uint32_t j = (uint32_t)bq + 4u * cc;
-                    st[cc] = kbs[j]; en[cc] = kbs[j + 1];
-                    plain = plain && (en[cc] - st[cc] <= 32u);
-                    bt0[cc] = *reinterpret_cast<const uint2*>(sa + fgmp_arec_at_offset(g, j) + 8 * t);
-                    bt1[cc] = make_uint2(0u, 0u);
-                    if (NH == 2) bt1[cc] = *reinterpret_cast<const uint2*>(sa + fgmp_arec_at_offset(g + 8, j) + 8 * t);
-                }
-                if (plain) {
-                    // Everything the four columns need, into registers.  Lane t has elements 4t .. 4t+3 of a block:
-                    // from its slot in the record (t < 2) or from the list (t >= 2).
-#pragma unroll
-                    for (int gr = 0; gr < 2; ++gr)
-#pragma unroll
-                        for (int cc = 0; cc < 4; ++cc) {
-                            const uint32_t iA = st[cc] + 16u * gr + g, iB = iA + 8;
-                            const bool hasA = iA < en[cc], hasB = iB < en[cc];
-                            const uint32_t mA = hasA ? *reinterpret_cast<const uint32_t*>(sb + STG_LIST + 4 * iA) : 0xffffffffu;
-                            const uint32_t mB = hasB ? *reinterpret_cast<const uint32_t*>(sb + STG_LIST + 4 * iB) : 0xffffffffu;
-                            const uint32_t oA = t < 2 ? REC_W4 + (mA & 0xffffu) + 4 * t : STG_LIST + hoff + iA * 8 + 4 * (t - 2);
-                            const uint32_t oB = t < 2 ? REC_W4 + (mB & 0xffffu) + 4 * t : STG_LIST + hoff + iB * 8 + 4 * (t - 2);
-                            rawA[4 * gr + cc] = hasA ? *reinterpret_cast<const uint32_t*>(sb + oA) : 0u;
-                            rawB[4 * gr + cc] = hasB ? *reinterpret_cast<const uint32_t*>(sb + oB) : 0u;
-                            rowA[4 * gr + cc] = mA >> 16;
-                            rowB[4 * gr + cc] = mB >> 16;
-                        }
-                } else {
-                    // a list that does not fit the stage, or a column with more than 32 FP8 blocks (rare): group by
-                    // group straight from the stage or from global memory, before the stage is given back
-                    auto fetch = [&](uint32_t i_, uint32_t& row, uint32_t& raw) {
-                        const uint32_t m_ = (all || 4 * i_ + 4 <= staged) ? *reinterpret_cast<const uint32_t*>(sb + STG_LIST + 4 * i_)
-                                                                          : __ldg(reinterpret_cast<const uint32_t*>(list_g + 4 * i_));
-                        row = m_ >> 16;
-                        if (t < 2) {
-                            raw = *reinterpret_cast<const uint32_t*>(sb + REC_W4 + (m_ & 0xffffu) + 4 * t);
-                        } else {
-                            const uint32_t o = hoff + i_ * 8 + 4 * (t - 2);
-                            raw = (all || o + 4 <= staged) ? *reinterpret_cast<const uint32_t*>(sb + STG_LIST + o)
-                                                           : __ldg(reinterpret_cast<const uint32_t*>(list_g + o));
-                        }
-                    };
+    } else if (warp >= W_SET && warp < W_EPI) {
+        // ------------------------------------------------------------ sets: units set, set + 2, ...: scales and FP8 blocks
+        // Thread = row of the tile = lane of tensor memory (quadrant warp % 4).
+        const uint32_t set = (uint32_t)(warp - W_SET) >> 2, row = 32u * (warp & 3) + lane;
+        const uint32_t quadrant = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t dense = quadrant + DENSE_COL + set * 64, sf_t = quadrant + SF_COL + set * 32;
+        float unscale = 0.f;                           // 2^-ratio: back to the E4M3 value of an FP8 element
+        if (!FUSED) unscale = __int_as_float((127 - reinterpret_cast<const fgmp_packed_header*>(p.ablob)->fp8_log2_ratio) << 23);
+        uint32_t stage = set, phase = 0, done = set, dphase = 0;      // done: stage of the set's last unit
+        for (uint32_t i = set; i < n_units; i += 2) {
+            const uint8_t* sb = smem + stage * p.stage_bytes;
+            if (!mbar_wait_warp(wf0 + 8 * stage, phase, abort_flag, p.status, 5)) break;
+            if (!FUSED) {
+                // the unit's step record from the packed activation record (where a block with scale 0 is FP8, or all zero)
+                uint8_t* rec = smem + stage * p.stage_bytes + STG_STEP;
+                const uint8_t* ar = rec + a_bytes;
+                const uint32_t ts = (threadIdx.x - 32u * W_SET) & (SET_THREADS - 1u), li = ts & 3u, j = (ts >> 2) & 15u;
 #pragma unroll 1
-                    for (int cc = 0; cc < 4; ++cc) {
-                        const uint32_t j = (uint32_t)bq + 4u * cc;
-                        const uint32_t st_ = kbs[j], en_ = kbs[j + 1];
-                        const uint2 b0 = *reinterpret_cast<const uint2*>(sa + fgmp_arec_at_offset(g, j) + 8 * t);
-                        uint2 b1 = make_uint2(0u, 0u);
-                        if (NH == 2) b1 = *reinterpret_cast<const uint2*>(sa + fgmp_arec_at_offset(g + 8, j) + 8 * t);
-                        for (uint32_t e = st_; e < en_; e += 16) {
-                            uint32_t rA = 0xffffu, rB = 0xffffu, wA = 0u, wB = 0u;
-                            if (e + g < en_) fetch(e + g, rA, wA);
-                            if (e + g + 8 < en_) fetch(e + g + 8, rB, wB);
-                            float c[4], d[4];
-                            group_mma(wA, wB, b0, b1, c, d);
-                            group_add(c, d, rA, rB);
-                        }
-                    }
+                for (uint32_t m = ts >> 6; m < M; m += 2) {
+                    const uint2 h = *reinterpret_cast<const uint2*>(ar + fgmp_arec_at_offset(m, j) + 8u * li);
+                    const uint32_t c4 = *reinterpret_cast<const uint16_t*>(ar + AREC_A4 + fgmp_rec_w4_offset(m, j) + 2u * li);
+                    const uint32_t sc = ar[AREC_SF + m * 16u + j];
+                    const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&h.x)), vb = __half22float2(*reinterpret_cast<const __half2*>(&h.y));
+                    const float v[4] = {va.x, va.y, vb.x, vb.y};
+                    const uint32_t c8 = f32x2_to_e4m3x2(v[0] * unscale, v[1] * unscale) | (f32x2_to_e4m3x2(v[2] * unscale, v[3] * unscale) << 16);
+                    emit_step(rec, M, n4, n8, m, j, li, sc == 0, c4, sc, c8, v, digits);
                 }
-                // the stage is no longer needed
+                fence_proxy_async();                   // the tensor core reads what ordinary stores wrote
                 __syncwarp();
-                if (lane == 0) mbar_arrive(empty0 + 8 * stage);
-                if (plain) {
-#pragma unroll
-                    for (int gr = 0; gr < 2; ++gr)
-#pragma unroll
-                        for (int cc = 0; cc < 4; ++cc) {
-                            if (gr == 1 && en[cc] - st[cc] <= 16u) continue;      // (the same for every lane)
-                            float c[4], d[4];
-                            group_mma(rawA[4 * gr + cc], rawB[4 * gr + cc], bt0[cc], bt1[cc], c, d);
-                            group_add(c, d, rowA[4 * gr + cc], rowB[4 * gr + cc]);
-                        }
-                }
+                if (lane == 0) mbar_arrive(sf0 + 8 * stage);
             }
-            if (!ok) break;
-            __syncwarp();
-            if (lane == 0) mbar_arrive(cdone0 + 8 * (seg & 1));
-            sbeg = send;
-        }
-    } else if (warp < W_EPI) {
-        // ------------------------------------------------------------ (3): hot block columns, rows 32jr .. 32jr+31
-        // Lane (g, t) has elements 4t .. 4t+3 of the column's block in rows 32jr + 16mt + {g, g + 8}: two code
-        // bytes and the block's microscale (zero for an FP8 weight block, which (2) covers).
-        const uint32_t jr = (uint32_t)(warp - W_HOT);
-        const uint32_t g = lane >> 2, t = lane & 3;
-        float* tile3 = tiles + FP8_WARPS * TILE_FLOATS;
-        int stage = 0; uint32_t phase = 0; bool ok = true;
-        int seg = 0;
-        for (int64_t u = u_begin; u < u_end && ok; ++seg) {
-            const int64_t tile = u / C;
-            const int64_t seg_end = min(u_end, (tile + 1) * C);
-            float acc[2][NH][4];
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                for (int nh = 0; nh < NH; ++nh) acc[mt][nh][0] = acc[mt][nh][1] = acc[mt][nh][2] = acc[mt][nh][3] = 0.f;
-            for (; u < seg_end; ++u) {
-                if (!(ok = mbar_wait_warp(full0 + 8 * stage, phase, abort_flag, p.status, 6))) break;
-                const uint8_t* sb = smem + (size_t)stage * DEC_STAGE_BYTES;
-                const uint8_t* sa = sb + STG_A;
-                const uint2 hw2 = *reinterpret_cast<const uint2*>(sa + AREC_HOT);      // one word per token octet
-                const uint32_t hot = hw2.x | hw2.y;
-                uint32_t todo = hot & 0xffffu;
-                while (todo) {
-                    const uint32_t j = (uint32_t)__ffs(todo) - 1u;
-                    todo &= todo - 1;
-                    uint2 b[NH];
-#pragma unroll
-                    for (int nh = 0; nh < NH; ++nh) b[nh] = *reinterpret_cast<const uint2*>(sa + fgmp_arec_at_offset(g + 8 * nh, j) + 8 * t);
-#pragma unroll
-                    for (int mt = 0; mt < 2; ++mt) {
-                        uint32_t x[2][2];
-#pragma unroll
-                        for (int rh = 0; rh < 2; ++rh) {
-                            const uint32_t r = 32 * jr + 16 * (uint32_t)mt + 8 * (uint32_t)rh + g;
-                            const uint32_t codes = *reinterpret_cast<const uint16_t*>(sb + REC_W4 + fgmp_rec_w4_offset(r, j) + 2 * t);
-                            const uint32_t sfb = sb[REC_SF + fgmp_rec_sf_offset(r, j)];
-                            uint32_t q0, q1, sc2;
-                            // (one byte at a time: unpacking a word into byte registers of which only some are used
-                            // gave wrong values on this toolchain)
-                            asm("{\n\t.reg .b8 b;\n\tcvt.u8.u32 b, %1;\n\tcvt.rn.f16x2.e2m1x2 %0, b;\n\t}" : "=r"(q0) : "r"(codes & 0xffu));
-                            asm("{\n\t.reg .b8 b;\n\tcvt.u8.u32 b, %1;\n\tcvt.rn.f16x2.e2m1x2 %0, b;\n\t}" : "=r"(q1) : "r"(codes >> 8));
-                            asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(sc2) : "h"((uint16_t)(sfb | (sfb << 8))));
-                            asm("mul.f16x2 %0, %1, %2;" : "=r"(x[rh][0]) : "r"(q0), "r"(sc2));
-                            asm("mul.f16x2 %0, %1, %2;" : "=r"(x[rh][1]) : "r"(q1), "r"(sc2));
-                        }
-#pragma unroll
-                        for (int nh = 0; nh < NH; ++nh) mma_f16_16816(acc[mt][nh], x[0][0], x[1][0], x[0][1], x[1][1], b[nh].x, b[nh].y);
-                    }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(empty0 + 8 * stage);
-                if (++stage == S) { stage = 0; phase ^= 1; }
+            // the tensor core has read what the set's last unit had in tensor memory
+            if (i >= 2) {
+                if (!mbar_wait_warp(dn0 + 8 * done, dphase, abort_flag, p.status, 7)) break;
+                tc_fence_after();
+                done += 2;
+                if (done >= S) { done -= S; dphase ^= 1; }
             }
-            if (!ok) break;
-            // the epilogue has taken the previous segment's sums; now this segment's go in:
-            // acc[mt][nh] = rows 32jr + 16mt + {g, g + 8} x tokens 8nh + {2t, 2t+1}
-            if (seg > 0 && !(ok = mbar_wait_warp(tfree, (uint32_t)(seg - 1) & 1u, abort_flag, p.status, 7))) break;
-#pragma unroll
-            for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-                for (int nh = 0; nh < NH; ++nh) {
-                    const uint32_t r = 32 * jr + 16 * (uint32_t)mt + g, m = 8 * (uint32_t)nh + 2 * t;
-                    tile3[tile_idx(r, m)] = acc[mt][nh][0];
-                    tile3[tile_idx(r, m + 1)] = acc[mt][nh][1];
-                    tile3[tile_idx(r + 8, m)] = acc[mt][nh][2];
-                    tile3[tile_idx(r + 8, m + 1)] = acc[mt][nh][3];
-                }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(cdone0 + 8 * (seg & 1));
-        }
-    } else {
-        // ------------------------------------------------------------ epilogue: tensor-memory lane quadrant warp % 4
-        const int q = warp & 3;
-        const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
-        const float s4a = FUSED ? p.q.s4 : __ldg(&reinterpret_cast<const fgmp_packed_header*>(p.ablob)->scale_fp4);
-        const float alpha = __fmul_rn(s4a, __ldg(&hw->scale_fp4));
-        const float r8 = __int_as_float((127 + __ldg(&hw->fp8_log2_ratio)) << 23);     // FP8 tensor scale / NVFP4 tensor scale of the weights
-        const int row = 32 * q + lane;
-        bool ok = true;
-        int seg = 0;
-        int stage = 0; uint32_t phase = 0;
-        for (int64_t u = u_begin; u < u_end && ok; ++seg) {
-            const int64_t tile = u / C;
-            const int64_t seg_begin = u, seg_end = min(u_end, (tile + 1) * C);
-            // Block scales of the segment's units into tensor memory, lane quadrant warp % 4: lane i holds, for MMA
-            // step j, the four scale bytes of rows i, 32+i, 64+i, 96+i in columns 4j..4j+3 -- 16 bytes of scale tile j
-            // of the record; the token scales follow in columns 16..31 (16 tokens: lanes 0..15, first column of
-            // every step), zeroed in the chunk's hot block columns.
-            for (; u < seg_end; ++u) {
-                if (!(ok = mbar_wait_warp(full0 + 8 * stage, phase, abort_flag, p.status, 4))) break;
-                const uint8_t* sb = smem + (size_t)stage * DEC_STAGE_BYTES;
-                const uint8_t* sa = sb + STG_A;
-                const uint2 hw2 = *reinterpret_cast<const uint2*>(sa + AREC_HOT);      // one word per token octet
-                const uint32_t hot = hw2.x | hw2.y;
+            // Block scales: lane i holds, for MMA step j, the four scale bytes of operand rows i, 32+i, 64+i, 96+i in columns
+            // 4j..4j+3: 16 bytes of scale tile j of the weight record; of the step record in columns 16..31.
+            auto scales = [&](const uint8_t* src, uint32_t dst) {
                 uint32_t r[16];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const uint4 x = *reinterpret_cast<const uint4*>(sb + REC_SF + 512 * j + lane * 16);
+                    const uint4 x = *reinterpret_cast<const uint4*>(src + 512 * j);
                     r[4 * j] = x.x; r[4 * j + 1] = x.y; r[4 * j + 2] = x.z; r[4 * j + 3] = x.w;
                 }
-                const uint32_t sf_t = tmem_base + ((uint32_t)(q * 32) << 16) + SF_COL0 + (uint32_t)stage * 32;
-                tmem_st16(sf_t, r);
-                const uint4 ts = *reinterpret_cast<const uint4*>(sa + AREC_SF + (lane & 15) * 16);
-                const uint32_t tsw[4] = {ts.x, ts.y, ts.z, ts.w};
+                tmem_st16(dst, r);
+            };
+            scales(sb + REC_SF + lane * 16, sf_t);
+            if (has_fp8) {
+                // The row's FP8 blocks lie one after the other in the list.
+                const uint16_t* before = reinterpret_cast<const uint16_t*>(sb + REC_KBSTART);
+                const uint32_t cnt = before[16], hoff = fgmp_list_halves_offset(cnt), m16 = reinterpret_cast<const uint16_t*>(sb + STG_MASK)[row];
+                uint32_t at = __popc(m16);             // sum over the rows 8 (row / 8) .. row
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    // bits 4j .. 4j+3 of the cold columns spread to the four bytes of the step's scale word
-                    const uint32_t keep = ((((~hot >> (4 * j)) & 0xfu) * 0x00204081u) & 0x01010101u) * 0xffu;
-                    r[4 * j] = lane < 16 ? (tsw[j] & keep) : 0u;
-                    r[4 * j + 1] = 0u; r[4 * j + 2] = 0u; r[4 * j + 3] = 0u;
+                for (int o = 1; o < 8; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, at, o, 8); if ((lane & 7) >= o) at += y; }
+                at = hoff + 8u * (before[row >> 3] + at - __popc(m16));
+                const bool all = hoff + 8u * cnt <= smeta[stage].staged;       // the usual case: the whole list is in the stage
+                const uint32_t slot = smem_u32(sb) + REC_W4 + row * 128u;
+                uint32_t hs = smem_u32(sb) + STG_LIST + at;
+#pragma unroll 1
+                for (uint32_t c = 0; c < 2; ++c) {     // eight block columns at a time
+                    uint32_t r[32];
+#pragma unroll
+                    for (uint32_t k = 0; k < 8; ++k) {
+                        const uint32_t is8 = (m16 >> (8 * c + k)) & 1u;
+                        const uint2 lo = lds64_if(slot + (((4 * c + (k >> 1)) ^ (row & 7u)) << 4) + (k & 1u) * 8u, is8);
+                        const uint2 hi = lds64_if(hs, is8 && all);
+                        hs += 8u * is8;
+                        r[4 * k] = lo.x; r[4 * k + 1] = lo.y; r[4 * k + 2] = hi.x; r[4 * k + 3] = hi.y;
+                    }
+                    if (!all) {
+                        const uint8_t* list_g = lists + (size_t)smeta[stage].step * 16;
+#pragma unroll
+                        for (uint32_t k = 0; k < 8; ++k)
+                            if ((m16 >> (8 * c + k)) & 1u) {
+                                const uint2 hi = __ldg(reinterpret_cast<const uint2*>(list_g + at));
+                                at += 8u;
+                                r[4 * k + 2] = hi.x; r[4 * k + 3] = hi.y;
+                            }
+                        __syncwarp();
+                    }
+                    tmem_st32(dense + 32 * c, r);
                 }
-                tmem_st16(sf_t + 16, r);
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(sfr0 + 8 * stage);
-                if (++stage == S) { stage = 0; phase ^= 1; }
             }
-            if (!ok) break;
-            const int accb = seg & 1; const uint32_t acc_phase = (uint32_t)((seg >> 1) & 1);
-            if (!(ok = mbar_wait_warp(accf0 + 8 * accb, acc_phase, abort_flag, p.status, 11))) break;
+            if (!mbar_wait_warp(sf0 + 8 * stage, phase, abort_flag, p.status, 16)) break;
+            scales(sb + STG_STEP + n4 * 128u + lane * 16, sf_t + 16);
+            tmem_wait_st();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(rd0 + 8 * stage);
+            stage += 2;
+            if (stage >= S) { stage -= S; phase ^= 1; }
+        }
+    }
+    else if (warp >= W_EPI && warp < W_STEP) {
+        // ------------------------------------------------------------ epilogue: tensor-memory lane quadrant warp % 4
+        const int q = warp & 3;
+        const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
+        const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
+        const float alpha = __fmul_rn(FUSED ? p.q.s4 : ha->scale_fp4, __ldg(&hw->scale_fp4));
+        // FP8 tensor scale / NVFP4 tensor scale of either operand
+        const float rw = __int_as_float((127 + __ldg(&hw->fp8_log2_ratio)) << 23);
+        const float ra = FUSED ? p.q.r8 : __int_as_float((127 + ha->fp8_log2_ratio) << 23);
+        const uint32_t row = 32 * q + lane;
+        uint32_t accb = 0, acc_phase = 0, tile = u_begin / C;
+        for (uint32_t u = u_begin; u < u_end; ++tile) {
+            const uint32_t t_begin = tile * C, t_end = t_begin + C;
+            const bool whole = u == t_begin && t_end <= u_end;
+            uint32_t nseg = 1, slot = 0;
+            if (!whole) {                              // (before the wait: the divisions take a while)
+                const uint32_t c_first = cta_of_unit(p, t_begin);
+                nseg = cta_of_unit(p, t_end - 1) - c_first + 1;
+                slot = blockIdx.x - c_first;
+            }
+            u = min(t_end, u_end);
+            if (!mbar_wait_warp(accf0 + 8 * accb, acc_phase, abort_flag, p.status, 11)) break;
             tc_fence_after();
+            if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(10);
             // a tile shared with other CTAs: how many of them have handed in their sums already (the answer is
             // needed only after this CTA's own sums are complete, so the load costs nothing)
-            const bool whole = (seg_begin == tile * C) && (seg_end == (tile + 1) * C);
-            int nseg = 1, slot = 0;
+            uint32_t* counter = p.counters + tile * 8 + q;
             uint32_t seen = 0;
-            if (!whole) {
-                const int64_t c_first = cta_of_unit(tile * C, G, p.total);
-                const int64_t c_last = cta_of_unit((tile + 1) * C - 1, G, p.total);
-                nseg = (int)(c_last - c_first + 1);
-                slot = (int)(blockIdx.x - c_first);
-                if (lane == 0) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(p.counters + tile * 8 + q) : "memory");
+            if (!whole && lane == 0) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
+            // columns m (NVFP4 blocks), (p + 1) M + m (digits); FP8 weights: m (high), M + m (low)
+            const uint32_t d4 = tmem_base + ((uint32_t)(q * 32) << 16) + D4_COL + accb * 112;
+            const uint32_t d8 = tmem_base + ((uint32_t)(q * 32) << 16) + D8_COL + accb * 32;
+            float v[16], t[16];
+            uint32_t r0[16], r1[16], r2[16];
+            // (three loads in flight at a time)
+            tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1); tmem_ld16_async(d8 + M, r2);
+            tmem_wait_ld(r0, r1, r2);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                v[j] = __uint_as_float(r0[j]); t[j] = 0.f;
+                if (has_fp8) v[j] += (__uint_as_float(r1[j]) + __uint_as_float(r2[j])) * rw;     // (else those columns hold nothing)
             }
-            uint32_t rr[16];
-            tmem_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(accb * TOK), rr);
+#pragma unroll 1
+            for (uint32_t pc = 1; pc < PIECES; pc += 3) {
+                tmem_ld16_async(d4 + pc * M, r0); tmem_ld16_async(d4 + (pc + 1) * M, r1); tmem_ld16_async(d4 + (pc + 2) * M, r2);
+                tmem_wait_ld(r0, r1, r2);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) t[j] += (__uint_as_float(r0[j]) + __uint_as_float(r1[j])) + __uint_as_float(r2[j]);
+            }
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] += t[j] * ra;
             tc_fence_before();
-            mbar_arrive(acce0 + 8 * accb);
-            float v[16];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(rr[j]);
-            // corrections (2) and (3) of the segment: this row of every tile, in tile order; the rows of (2)
-            // are cleared for the next segment on the way
-            if (!(ok = mbar_wait_warp(cdone0 + 8 * accb, acc_phase, abort_flag, p.status, 12))) break;
-            float c2[16];                              // (2): sums of the FP8 weight codes, still without 2^ratio
-#pragma unroll
-            for (int j = 0; j < 16; ++j) c2[j] = 0.f;
-#pragma unroll
-            for (int w = 0; w < NTILES; ++w) {
-                float4* src = reinterpret_cast<float4*>(tiles + w * TILE_FLOATS + row * TOK);
-                float4 x[4];
-#pragma unroll
-                for (int j = 0; j < 2 * NH; ++j) x[j] = src[(j ^ (row >> 1)) & 3];       // tokens 4j .. 4j+3
-#pragma unroll
-                for (int j = 0; j < 2 * NH; ++j) {
-                    if (w < FP8_WARPS) { c2[4 * j] += x[j].x; c2[4 * j + 1] += x[j].y; c2[4 * j + 2] += x[j].z; c2[4 * j + 3] += x[j].w; }
-                    else               { v[4 * j] += x[j].x; v[4 * j + 1] += x[j].y; v[4 * j + 2] += x[j].z; v[4 * j + 3] += x[j].w; }
-                    if (w < FP8_WARPS) src[(j ^ (row >> 1)) & 3] = make_float4(0.f, 0.f, 0.f, 0.f);   // the tile of (3) is overwritten
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] += c2[j] * r8;
             __syncwarp();
-            if (lane == 0) mbar_arrive(tfree);
+            if (lane == 0) mbar_arrive(acce0 + 8 * accb);
+            accb ^= 1u;
+            if (accb == 0) acc_phase ^= 1u;
+            if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(11);
 
-            const int64_t n = tile * 128 + row;
+            const int64_t n = (int64_t)tile * 128 + row;
             bool write_out = whole;
             if (!whole) {
                 // partial tile: publish, and let the warp that arrives last add everything up.  When all the
                 // others were seen to have arrived, this warp is the last without asking and skips the counter.
-                float* dst = p.partials + (((size_t)tile * p.maxseg + slot) * 128 + row) * 16;
+                float* base = p.partials + ((size_t)tile * p.maxseg * 128 + row) * 16;
+                float* dst = base + (size_t)slot * 2048;
                 // (32 bytes per store: whole sectors)
 #pragma unroll
-                for (int j = 0; j < 8 * NH; j += 8)
-                    asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                                 ::"l"(dst + j), "r"(__float_as_uint(v[j])), "r"(__float_as_uint(v[j + 1])), "r"(__float_as_uint(v[j + 2])),
-                                   "r"(__float_as_uint(v[j + 3])), "r"(__float_as_uint(v[j + 4])), "r"(__float_as_uint(v[j + 5])),
-                                   "r"(__float_as_uint(v[j + 6])), "r"(__float_as_uint(v[j + 7])) : "memory");
+                for (int j = 0; j < 16; j += 8)
+                    if (j < (int)M)
+                        asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                     ::"l"(dst + j), "r"(__float_as_uint(v[j])), "r"(__float_as_uint(v[j + 1])), "r"(__float_as_uint(v[j + 2])),
+                                       "r"(__float_as_uint(v[j + 3])), "r"(__float_as_uint(v[j + 4])), "r"(__float_as_uint(v[j + 5])),
+                                       "r"(__float_as_uint(v[j + 6])), "r"(__float_as_uint(v[j + 7])) : "memory");
                 // The counter wraps to zero with the last arrival (or is put back by the warp that skipped
                 // it), so the workspace is ready for the next call without being cleared.
                 uint32_t old = __shfl_sync(0xffffffffu, seen, 0);
-                if (old != (uint32_t)(nseg - 1)) {
+                if (old != nseg - 1) {
                     // the warp's stores are ordered before lane 0's release of the counter; its acquire sees the others'
                     __syncwarp();
                     if (lane == 0)
-                        asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(p.counters + tile * 8 + q), "r"((uint32_t)(nseg - 1)) : "memory");
+                        asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(counter), "r"(nseg - 1) : "memory");
                     old = __shfl_sync(0xffffffffu, old, 0);
                 } else if (lane == 0) {
-                    p.counters[tile * 8 + q] = 0u;
+                    *counter = 0u;
                 }
-                if (old == (uint32_t)(nseg - 1)) {
+                if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(12);
+                if (old == nseg - 1) {
 #pragma unroll
                     for (int j = 0; j < 16; ++j) v[j] = 0.f;
-                    for (int sgi = 0; sgi < nseg; ++sgi) {       // one sum in slot order
-                        const float* src = p.partials + (((size_t)tile * p.maxseg + sgi) * 128 + row) * 16;
+#pragma unroll 1
+                    for (uint32_t sgi = 0; sgi < nseg; ++sgi) {       // one sum in slot order
+                        const float* src = base + (size_t)sgi * 2048;
 #pragma unroll
-                        for (int j = 0; j < 8 * NH; j += 8) {
+                        for (int j = 0; j < 16; j += 8) {
+                            if (j >= (int)M) break;
                             uint32_t y8[8];
                             asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                                          : "=r"(y8[0]), "=r"(y8[1]), "=r"(y8[2]), "=r"(y8[3]), "=r"(y8[4]), "=r"(y8[5]), "=r"(y8[6]), "=r"(y8[7])
@@ -767,8 +672,8 @@ decode_kernel(DecParams p)
             if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(whole ? 7 : 8);    // last segment: sums complete / handed in
             if (write_out && n < p.N) {
 #pragma unroll
-                for (int j = 0; j < 8 * NH; ++j) {
-                    if (j < p.M) {
+                for (int j = 0; j < 16; ++j) {
+                    if (j < (int)M) {
                         if (p.y_is_bf16) reinterpret_cast<__nv_bfloat16*>(p.Ybf)[(int64_t)j * p.ldy + n] = __float2bfloat16_rn(v[j] * alpha);
                         else p.Y[(int64_t)j * p.ldy + n] = v[j] * alpha;
                     }
@@ -784,9 +689,9 @@ decode_kernel(DecParams p)
         while (globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
         __syncthreads();
     } else if (FUSED && threadIdx.x == 0) {
-        // the CTA that finishes last takes the "records ready" word back, so that the control area is as the next call needs it
-        if (atomicInc(p.cw + CW_DONE, (uint32_t)G - 1u) == (uint32_t)G - 1u)
-            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.cw + CW_QREADY), "r"(0u) : "memory");
+        // the CTA that finishes last takes the count of finished items back, so that the control area is as the next call needs it
+        if (atomicInc(p.cw + CW_DONE, G - 1u) == G - 1u)
+            asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.cw + CW_QCOUNT), "r"(0u) : "memory");
     }
     if (warp == W_MMA) {
         tc_fence_after();
@@ -794,7 +699,7 @@ decode_kernel(DecParams p)
     }
 }
 
-struct DecPlan { int64_t tiles, chunks, total; int grid; int maxseg; };
+struct DecPlan { int64_t tiles, chunks, total; int grid; int maxseg; int64_t span, rest; };
 
 DecPlan decode_plan(int64_t N, int64_t K)
 {
@@ -803,8 +708,8 @@ DecPlan decode_plan(int64_t N, int64_t K)
     const int sms = fgmp_sm_count();
     d.grid = (int)(d.total < sms ? d.total : sms);
     // a tile of `chunks` units meets at most this many CTA spans of >= floor(total/grid) units
-    const int64_t span = d.total / d.grid;
-    d.maxseg = (int)((d.chunks + span - 1) / span + 1);
+    d.span = d.total / d.grid; d.rest = d.total % d.grid;
+    d.maxseg = (int)((d.chunks + d.span - 1) / d.span + 1);
     return d;
 }
 
@@ -817,10 +722,9 @@ fgmp_status set_attrs_once()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
     std::lock_guard<std::mutex> lk(g_dec_mu);
     if (!g_attr_set[dev]) {
-        if (cudaFuncSetAttribute(decode_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(decode_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(decode_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(decode_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DEC_SMEM) != cudaSuccess)
+        if (cudaFuncSetAttribute(decode_kernel<DEC_FUSED_LP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess ||
+            cudaFuncSetAttribute(decode_kernel<DEC_FUSED_HP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess ||
+            cudaFuncSetAttribute(decode_kernel<DEC_UNPACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess)
             return FGMP_ERR_CUDA;
         g_attr_set[dev] = true;
     }
@@ -829,8 +733,8 @@ fgmp_status set_attrs_once()
 
 // Workspace of the decode path, all inside the control area that must be zero before the first call and
 // that every call leaves zero: status at 0, control words at 256, stream-K
-// counters from 1024 (32 bytes per tile); partial sums behind the control area, then (fused calls
-// without a packed output) the activation records.
+// counters from 1024 (32 bytes per tile); partial sums behind the control area, then (fused calls) the
+// step records.
 DecParams base_params(const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
                       void* workspace, const DecPlan& d)
 {
@@ -839,7 +743,7 @@ DecParams base_params(const void* packed_weights, void* Y, int y_is_bf16, int64_
     p.wblob = (const uint8_t*)packed_weights;
     p.LW = fgmp_layout(N, K, 1, 0); p.LA = fgmp_layout(M, K, 0, 0);
     p.Y = (float*)Y; p.Ybf = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16;
-    p.M = M; p.N = N; p.K = K; p.total = d.total; p.chunks = d.chunks;
+    p.M = M; p.N = N; p.K = K; p.chunks = (uint32_t)d.chunks; p.span = (uint32_t)d.span; p.rest = (uint32_t)d.rest;
     p.status = reinterpret_cast<int*>(ws);
     p.cw = reinterpret_cast<uint32_t*>(ws + 256);
     p.counters = reinterpret_cast<uint32_t*>(ws + 1024);
@@ -848,17 +752,22 @@ DecParams base_params(const void* packed_weights, void* Y, int y_is_bf16, int64_
     return p;
 }
 
-template <bool FUSED>
-fgmp_status launch_decode(const DecParams& p, const DecPlan& d, bool programmatic, cudaStream_t s)
+template <int SRC>
+fgmp_status launch_decode(DecParams p, const DecPlan& d, bool programmatic, cudaStream_t s)
 {
+    const uint32_t arec = SRC == DEC_UNPACK ? (p.M <= 8 ? AREC_AT + 4096u : AREC_BYTES) : 0u;
+    p.stage_bytes = (STG_STEP + step_bytes(p.M) + arec + 1023u) & ~1023u;
+    const size_t fixed = 1024 /*alignment*/ + 1024 /*barriers, digit table*/;
+    const uint32_t fit = (uint32_t)((SMEM_LIMIT - fixed) / p.stage_bytes);         // 3 (DEC_UNPACK, 16 tokens) to 7
+    p.stages = fit < (uint32_t)DEC_MAX_STAGES ? fit : (uint32_t)DEC_MAX_STAGES;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)d.grid); cfg.blockDim = dim3(DEC_THREADS); cfg.dynamicSmemBytes = DEC_SMEM; cfg.stream = s;
+    cfg.gridDim = dim3((unsigned)d.grid); cfg.blockDim = dim3(DEC_THREADS); cfg.stream = s;
+    cfg.dynamicSmemBytes = fixed + (size_t)p.stages * p.stage_bytes;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = programmatic ? 1 : 0;
-    if (p.M <= 8) { FGMP_LAUNCH(FGMP_K_DECODE, s, cudaLaunchKernelEx(&cfg, decode_kernel<1, FUSED>, p)); }
-    else          { FGMP_LAUNCH(FGMP_K_DECODE, s, cudaLaunchKernelEx(&cfg, decode_kernel<2, FUSED>, p)); }
+    FGMP_LAUNCH(FGMP_K_DECODE, s, cudaLaunchKernelEx(&cfg, decode_kernel<SRC>, p));
     return fgmp_launch_status();
 }
 
@@ -880,7 +789,7 @@ size_t fgmp_ws_decode(int64_t M, int64_t N, int64_t K)
 size_t fgmp_ws_linear_fused(int64_t M, int64_t N, int64_t K)
 {
     if (!fgmp_decode_supported(M, N, K)) return fgmp_ws_linear(M, N, K);
-    return fgmp_align1k(fgmp_ws_decode(M, N, K)) + (size_t)(K / 256) * AREC_BYTES;
+    return fgmp_align1k(fgmp_ws_decode(M, N, K)) + (size_t)(K / 256) * step_bytes(M);
 }
 
 // clear_first: zero the control area on the stream before the kernel (for scratch whose state the
@@ -895,7 +804,7 @@ fgmp_status fgmp_linear_decode(const void* packed_acts, const void* packed_weigh
     fgmp_status st = set_attrs_once();
     if (st != FGMP_OK) return st;
     if (clear_first && cudaMemsetAsync(workspace, 0, 1024 + (size_t)d.tiles * 32, s) != cudaSuccess) return FGMP_ERR_CUDA;
-    return launch_decode<false>(p, d, !clear_first, s);
+    return launch_decode<DEC_UNPACK>(p, d, !clear_first, s);
 }
 
 extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const float* fisher_chan,
@@ -933,16 +842,15 @@ extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const 
     p.q.s8 = ldexpf(sc.scale_fp4, sc.fp8_log2_ratio);
     p.q.inv8 = 1.0f / p.q.s8;
     p.q.tau = tau; p.q.ratio = sc.fp8_log2_ratio; p.q.r8 = ldexpf(1.0f, sc.fp8_log2_ratio);
-    p.q_mode = (int)sm;
     if (packed_acts_out) {
         uint8_t* blob = (uint8_t*)packed_acts_out;
         p.q_codes4 = blob + p.LA.off_codes4; p.q_sf = blob + p.LA.off_sf; p.q_mask = blob + p.LA.off_mask;
         p.q_codes8 = blob + p.LA.off_codes8; p.q_header = reinterpret_cast<fgmp_packed_header*>(blob);
-        p.arec = blob + p.LA.off_arec;
-    } else {
-        p.arec = (uint8_t*)workspace + fgmp_align1k(fgmp_ws_decode(M, N, K));
+        p.q_arec = blob + p.LA.off_arec;
     }
-    return launch_decode<true>(p, d, true, (cudaStream_t)cuda_stream);
+    p.steps = (uint8_t*)workspace + fgmp_align1k(fgmp_ws_decode(M, N, K));
+    return sm == FGMP_SCORE_LP_ERROR ? launch_decode<DEC_FUSED_LP>(p, d, true, (cudaStream_t)cuda_stream)
+                                     : launch_decode<DEC_FUSED_HP>(p, d, true, (cudaStream_t)cuda_stream);
 }
 
 #ifdef FGMP_TIMELINE

@@ -65,7 +65,7 @@ __device__ __forceinline__ void nvfp4x16_scaled(const uint2& c, uint32_t scale_c
 // NVFP4 / only the FP8 blocks, each over its own tensor scale (the per-class passes of fgmp_linear_classes)
 __device__ __forceinline__ bool header_matches(const fgmp_packed_header* h, int64_t rows, int64_t K, uint32_t kind, int* status, int where, int cls = 0)
 {
-    const bool ok = h->magic == FGMP_MAGIC && h->version == 7u && h->rows == rows && h->K == K && h->kind == kind && h->error == 0 &&
+    const bool ok = h->magic == FGMP_MAGIC && h->version == FGMP_LAYOUT_VERSION && h->rows == rows && h->K == K && h->kind == kind && h->error == 0 &&
                     (cls != 0 || h->fp8_scale_free == 0);
     if (!ok && threadIdx.x == 0) { atomicCAS(status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(status + 1, where); }
     return ok;
@@ -108,9 +108,7 @@ __global__ void __launch_bounds__(128) expand_w_kernel(const uint8_t* __restrict
     const PackedLayout L = fgmp_layout(rows, K, 1, 0);
     const float r8 = cls ? 1.0f : __int_as_float((127 + h->fp8_log2_ratio) << 23);
     const int64_t unit = blockIdx.x, tile = unit / L.chunks, c = unit % L.chunks;
-    const uint32_t* mask = reinterpret_cast<const uint32_t*>(blob + L.off_mask);
-    const uint32_t m16 = fgmp_chunk_mask(mask, L, tile * 128 + threadIdx.x, c);
-    const uint32_t cnt = fgmp_unit_positions(m16, sc.warp, sc.pos, sc.cnt);
+    const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x]);
     const uint8_t* rec = blob + L.off_rec + (size_t)unit * REC_BYTES;
     const uint8_t* halves = blob + L.off_ovf + (size_t)reinterpret_cast<const uint32_t*>(blob + L.off_uptr)[unit] * 16 + fgmp_list_halves_offset(cnt);
     const int j = threadIdx.x & 15;
@@ -123,7 +121,7 @@ __global__ void __launch_bounds__(128) expand_w_kernel(const uint8_t* __restrict
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int row = (threadIdx.x >> 4) + 8 * (i0 + i);
-            pos[i] = sc.pos[row * 16 + j];
+            pos[i] = sc.pos(row, j);
             slot[i] = __ldg(reinterpret_cast<const uint2*>(rec + REC_W4 + fgmp_rec_w4_offset(row, j)));
             sfb[i] = __ldg(rec + REC_SF + fgmp_rec_sf_offset(row, j));
             hi[i] = make_uint2(0u, 0u);
@@ -344,7 +342,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 
     if (p.q.codes4 && blockIdx.x == 0 && threadIdx.x == 0) {
         fgmp_packed_header* h = p.q.header;
-        h->magic = FGMP_MAGIC; h->version = 7; h->rows = p.M; h->K = p.N; h->scale_fp4 = p.q.s4;
+        h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = p.M; h->K = p.N; h->scale_fp4 = p.q.s4;
         h->fp8_log2_ratio = p.q.ratio; h->n_fp8 = (p.q.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
         h->error = 0; h->scale_fp8 = p.q.s8; h->fp8_scale_free = p.q.free8;
     }

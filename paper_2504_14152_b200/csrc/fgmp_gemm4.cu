@@ -62,8 +62,8 @@ __device__ __forceinline__ bool g4_applicable(const Gemm4Params& p)
 {
     const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
     const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
-    return ha->magic == FGMP_MAGIC && ha->version == 7u && ha->rows == p.M && ha->K == p.K && ha->kind == 0u && ha->n_fp8 == 0 &&
-           hw->magic == FGMP_MAGIC && hw->version == 7u && hw->rows == p.N && hw->K == p.K && hw->kind == 1u && hw->error == 0 &&
+    return ha->magic == FGMP_MAGIC && ha->version == FGMP_LAYOUT_VERSION && ha->rows == p.M && ha->K == p.K && ha->kind == 0u && ha->n_fp8 == 0 &&
+           hw->magic == FGMP_MAGIC && hw->version == FGMP_LAYOUT_VERSION && hw->rows == p.N && hw->K == p.K && hw->kind == 1u && hw->error == 0 &&
            hw->n_fp8 == 0;
 }
 

@@ -40,21 +40,9 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
     if (!SCORE_ONLY) {
         if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
             fgmp_packed_header* h = p.header;
-            h->magic = FGMP_MAGIC; h->version = 7; h->rows = p.M; h->K = p.K; h->scale_fp4 = p.s4;
+            h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = p.M; h->K = p.K; h->scale_fp4 = p.s4;
             h->fp8_log2_ratio = p.ratio; h->n_fp8 = (p.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
             h->error = 0; h->scale_fp8 = p.s8; h->fp8_scale_free = p.free8;
-        }
-        // token rows M..15 of the decode records are zero (the grid covers 16 rows in that mode)
-        if (p.arec && m0 >= p.M) {
-            if (active) {
-                uint8_t* rec = p.arec + (size_t)(kb >> 4) * AREC_BYTES;
-                const uint32_t j = (uint32_t)kb & 15u, m = (uint32_t)m0;
-                *reinterpret_cast<uint2*>(rec + AREC_A4 + fgmp_rec_w4_offset(m, j)) = make_uint2(0u, 0u);
-                rec[AREC_SF + m * 16 + j] = 0;
-                uint4* at = reinterpret_cast<uint4*>(rec + fgmp_arec_at_offset(m, j));
-                at[0] = make_uint4(0, 0, 0, 0); at[1] = make_uint4(0, 0, 0, 0);
-            }
-            return;
         }
     }
 
@@ -126,11 +114,9 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
                     uint4* at = reinterpret_cast<uint4*>(rec + fgmp_arec_at_offset((uint32_t)m, j));
                     at[0] = make_uint4(o[0], o[1], o[2], o[3]);
                     at[1] = make_uint4(o[4], o[5], o[6], o[7]);
-                    // what the tensor core reads: codes and microscale (both zero for an FP8 block), and the
-                    // chunk's set of block columns that hold an FP8 block of some token
+                    // codes and microscale, both zero for an FP8 block
                     *reinterpret_cast<uint2*>(rec + AREC_A4 + fgmp_rec_w4_offset((uint32_t)m, j)) = make_uint2(c4[0], c4[1]);
                     rec[AREC_SF + (uint32_t)m * 16 + j] = (uint8_t)sc;
-                    if (is8) atomicOr(reinterpret_cast<unsigned int*>(rec + AREC_HOT), 1u << j);
                 }
                 *reinterpret_cast<uint2*>(p.codes4 + (m * p.K) / 2 + kb * 8) = make_uint2(c4[0], c4[1]);
                 p.sf[fgmp_sf_offset(m, kb, p.K)] = (uint8_t)sc;
@@ -177,9 +163,10 @@ __global__ void __launch_bounds__(128) unpack_w_kernel(const uint8_t* blob, int6
 {
     __shared__ UnitScratch sc;
     const PackedLayout L = fgmp_layout(rows, K, 1, 0);
-    if (mask) {
-        const uint32_t* pmask = reinterpret_cast<const uint32_t*>(blob + L.off_mask);
-        for (int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x; i < rows * L.MW; i += (int64_t)gridDim.x * 128) mask[i] = pmask[i];
+    if (mask) {                                         // canonical order: a row's bits of all chunks, two chunks per word
+        const int64_t tile = blockIdx.x / L.chunks, c = blockIdx.x % L.chunks, r = tile * 128 + threadIdx.x;
+        const uint16_t* m16 = reinterpret_cast<const uint16_t*>(blob + L.off_mask) + (size_t)blockIdx.x * 128 + threadIdx.x;
+        if (r < rows && (c & 1) == 0) mask[r * L.MW + (c >> 1)] = m16[0] | (c + 1 < L.chunks ? (uint32_t)m16[128] << 16 : 0u);
     }
     fgmp_for_each_block(blob, L, blockIdx.x, sc, [&](int64_t r, int64_t kb, int row, int j, const uint8_t* rec, const uint8_t* hi) {
         const uint2 slot = *reinterpret_cast<const uint2*>(rec + REC_W4 + fgmp_rec_w4_offset(row, j));
@@ -258,15 +245,8 @@ extern "C" fgmp_status fgmp_quantize_activations(const void* X_bf16, int64_t ldx
     p.codes4 = blob + L.off_codes4; p.sf = blob + L.off_sf;
     p.mask = reinterpret_cast<uint32_t*>(blob + L.off_mask); p.codes8 = blob + L.off_codes8;
     p.header = reinterpret_cast<fgmp_packed_header*>(blob);
-    int64_t grid_rows = M;
-    if (M <= 16 && !p.free8) {         // decode-sized batch: also emit the records of the decode GEMM, 16 token rows (tied scales only)
-        p.arec = blob + L.off_arec;
-        p.rows_per_cta = 1;
-        grid_rows = 16;
-        // the sets of hot block columns are OR-ed together by the kernel's threads
-        if (cudaMemset2DAsync(blob + L.off_arec + AREC_HOT, AREC_BYTES, 0, 16, (size_t)L.chunks, s) != cudaSuccess) return FGMP_ERR_CUDA;
-    }
-    dim3 grid((unsigned)((p.KB + QA_THREADS - 1) / QA_THREADS), (unsigned)((grid_rows + p.rows_per_cta - 1) / p.rows_per_cta));
+    if (M <= 16 && !p.free8) p.arec = blob + L.off_arec;     // decode-sized batch: also emit the records of the decode GEMM (tied scales only)
+    dim3 grid((unsigned)((p.KB + QA_THREADS - 1) / QA_THREADS), (unsigned)((M + p.rows_per_cta - 1) / p.rows_per_cta));
     if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, quant_act_kernel<0, false><<<grid, QA_THREADS, 0, s>>>(p));
     else                           FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, quant_act_kernel<1, false><<<grid, QA_THREADS, 0, s>>>(p));
     return fgmp_launch_status();

@@ -223,8 +223,9 @@ __global__ void w_eqcount_kernel(const float* scores, int64_t N, int64_t KB, int
     }
 }
 
+// (mask16: the bits in the order of the packed tensor, a uint16 per row of a unit)
 __global__ void w_mask_kernel(const float* scores, int64_t N, int64_t KB, int64_t MW, const SelectState* st,
-                              const uint32_t* eqprefix, uint32_t* mask, uint32_t* wcnt)
+                              const uint32_t* eqprefix, uint16_t* mask16, int64_t chunks)
 {
     const float tau = st->tau;
     const bool use_eq = st->use_eq != 0;
@@ -243,7 +244,9 @@ __global__ void w_mask_kernel(const float* scores, int64_t N, int64_t KB, int64_
             take = rank < need_eq;
         }
         uint32_t word = __ballot_sync(0xffffffffu, take);
-        if (lane == 0) { mask[w] = word; wcnt[w] = __popc(word); }
+        // lanes 0 and 1: the word's two chunks
+        const int64_t c = 2 * (w % MW) + lane;
+        if (lane < 2 && c < chunks) mask16[((n >> 7) * chunks + c) * 128 + (n & 127)] = (uint16_t)(word >> (16 * lane));
     }
 }
 
@@ -281,13 +284,16 @@ __global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* in, uint32_t
 
 // per unit (128-row tile x 16-block K chunk): size of its list of FP8 blocks in 16-byte steps, and the
 // running total of FP8 blocks.  One CTA of 128 threads per unit, a thread per row.
-__global__ void __launch_bounds__(128) w_unit_count_kernel(const uint32_t* mask, PackedLayout L, uint32_t* list_steps,
+// Mask bits of rows beyond the tensor are cleared here.
+__global__ void __launch_bounds__(128) w_unit_count_kernel(uint16_t* mask16, PackedLayout L, uint32_t* list_steps,
                                                            SelectState* st)
 {
     __shared__ uint32_t s_cnt[4];
     const int64_t unit = blockIdx.x;
-    const uint32_t m16 = fgmp_chunk_mask(mask, L, (unit / L.chunks) * 128 + threadIdx.x, unit % L.chunks);
-    uint32_t c = __popc(m16);
+    uint16_t* own = mask16 + unit * 128 + threadIdx.x;
+    uint32_t c = 0;
+    if ((unit / L.chunks) * 128 + threadIdx.x < L.rows) c = __popc((uint32_t)*own);
+    else *own = 0;
     for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
     if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = c;
     __syncthreads();
@@ -299,7 +305,7 @@ __global__ void __launch_bounds__(128) w_unit_count_kernel(const uint32_t* mask,
 }
 
 // Writes the record of one unit (codes and microscales of its NVFP4 blocks, the first halves of its FP8
-// blocks, the per-column running counts) and the list of its FP8 blocks (rows, second halves).  One CTA
+// blocks, the running counts of FP8 blocks by row) and the list of its FP8 blocks (rows, second halves).  One CTA
 // of 128 threads per unit.
 __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw8, int ratio, float s8_given, const SelectState* st,
                                                      const uint8_t* sc_in, uint8_t* blob, PackedLayout L, int64_t room_steps)
@@ -311,18 +317,13 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
     const float s4 = st->s4;
     const float s8 = s8_given > 0.f ? s8_given : __fmul_rn(s4, __int_as_float((127 + ratio) << 23));
     const float inv8 = __fdiv_rn(1.0f, s8);
-    const uint32_t* mask = reinterpret_cast<const uint32_t*>(blob + L.off_mask);
-    const uint32_t m16 = fgmp_chunk_mask(mask, L, tile * 128 + threadIdx.x, c);
-    const uint32_t cnt = fgmp_unit_positions(m16, sc.warp, sc.pos, sc.cnt);
+    const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x]);
     uint8_t* rec = blob + L.off_rec + (size_t)unit * REC_BYTES;
     uint8_t* list = blob + L.off_ovf + (size_t)uptr[unit] * 16;
     uint32_t* entries = reinterpret_cast<uint32_t*>(list);
     uint8_t* halves = list + fgmp_list_halves_offset(cnt);
-    if (threadIdx.x < 64) {                                    // running sums of the per-column counts, then padding
-        uint32_t before = 0;
-        for (int i = 0; i < 16 && i < (int)threadIdx.x; ++i) before += sc.cnt[i];
-        reinterpret_cast<uint16_t*>(rec + REC_KBSTART)[threadIdx.x] = threadIdx.x <= 16 ? (uint16_t)before : (uint16_t)0;
-    }
+    if (threadIdx.x < 64)                                      // FP8 blocks before every eighth row, then padding
+        reinterpret_cast<uint16_t*>(rec + REC_KBSTART)[threadIdx.x] = threadIdx.x < 16 ? sc.base[8 * threadIdx.x] : threadIdx.x == 16 ? (uint16_t)cnt : (uint16_t)0;
     if (fits) {                                                // padding behind the entries and behind the last half
         for (uint32_t i = cnt + threadIdx.x; i < fgmp_list_halves_offset(cnt) / 4; i += 128) entries[i] = 0;
         if (threadIdx.x == 0 && (cnt & 1u)) *reinterpret_cast<uint2*>(halves + (size_t)cnt * 8) = make_uint2(0u, 0u);
@@ -337,7 +338,7 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
         if (n < L.rows && kb < L.KB) {
             float v[16], f[16];
             load_block(W, ldw8, nullptr, 0, n, kb, v, f);
-            const uint32_t pos = sc.pos[row * 16 + j];
+            const uint32_t pos = sc.pos(row, j);
             if (pos != 0xffffu) {
                 uint32_t c8[4];
                 float dq8[16];
@@ -374,7 +375,7 @@ __global__ void w_header_kernel(fgmp_packed_header* h, const SelectState* st, co
                                 float* tau_eff_out)
 {
     if (threadIdx.x == 0) {
-        h->magic = FGMP_MAGIC; h->version = 7; h->rows = N; h->K = K; h->scale_fp4 = st->s4;
+        h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = N; h->K = K; h->scale_fp4 = st->s4;
         h->fp8_log2_ratio = ratio; h->n_fp8 = (int64_t)st->n_fp8; h->kind = 1; h->capacity = room_steps;
         float teff = fraction_mode ? st->tau : tau_given;
         h->tau_eff = teff;
@@ -487,7 +488,7 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
             else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<1, false><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
         }
     }
-    uint32_t* mask = reinterpret_cast<uint32_t*>(blob + L.off_mask);
+    uint16_t* mask16 = reinterpret_cast<uint16_t*>(blob + L.off_mask);
     uint32_t* uptr = reinterpret_cast<uint32_t*>(blob + L.off_uptr);
     const int64_t NCT = L.units;
     const int gw = grid_for(NW * 32, 256, 8);
@@ -499,8 +500,8 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
         // k == 0: nothing is FP8 (tau_eff = +inf); threshold mode: the given tau
         FGMP_LAUNCH(FGMP_K_W_AUX, s, set_tau_kernel<<<1, 32, 0, s>>>(st, fraction_mode ? INFINITY : tau));
     }
-    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_mask_kernel<<<gw, 256, 0, s>>>(scores, N, KB, MW, st, tmp_b, mask, tmp_a));
-    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_unit_count_kernel<<<(unsigned)NCT, 128, 0, s>>>(mask, L, tmp_a, st));
+    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_mask_kernel<<<gw, 256, 0, s>>>(scores, N, KB, MW, st, tmp_b, mask16, L.chunks));
+    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_unit_count_kernel<<<(unsigned)NCT, 128, 0, s>>>(mask16, L, tmp_a, st));
     FGMP_LAUNCH(FGMP_K_SCAN, s, scan_kernel<<<1, 1024, 0, s>>>(tmp_a, uptr, NCT, nullptr, 1));
     FGMP_LAUNCH(FGMP_K_W_EMIT, s, w_emit_kernel<<<(unsigned)NCT, 128, 0, s>>>(W, ldw / 8, ratio, s8_given, st, sc_tmp, blob, L, room_steps));
     FGMP_LAUNCH(FGMP_K_W_AUX, s, w_header_kernel<<<1, 32, 0, s>>>(reinterpret_cast<fgmp_packed_header*>(blob), st, uptr, NCT, N, K, ratio, s8_given,
