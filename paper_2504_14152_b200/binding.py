@@ -15,6 +15,7 @@ _LIB_PATH = os.path.join(_HERE, "libfgmp.so")
 _EXT_PATH = os.path.join(_HERE, "_fgmp_torch.so")
 
 SCORE_LP_ERROR, SCORE_HP_TO_LP = 0, 1
+_INF = float("inf")
 CLIP_NONE, CLIP_SW_BRUTE = 0, 1
 OP_QUANTIZE_WEIGHTS, OP_QUANTIZE_ACTIVATIONS, OP_LINEAR, OP_CALIBRATE_TAU, OP_GLOBAL_TAU, OP_LINEAR_QUANTIZE, OP_LINEAR_FUSED, OP_LINEAR_CLASSES = 0, 1, 2, 3, 4, 5, 6, 7
 
@@ -179,6 +180,7 @@ class PackedTensor:
     K: int
     kind: int               # 0 activations, 1 weights
     fp8_free: bool = False  # packed with an FP8 tensor scale of its own (scale_fp8 > 0): multiplied by linear_classes
+    nvfp4: bool | None = None   # no FP8 block in it (True), some or not excluded by the header (False), not known here (None)
 
     def header(self) -> dict:
         h = self.blob[:128].cpu().numpy().tobytes()
@@ -211,7 +213,7 @@ def quantize_weights(W: torch.Tensor, fisher: torch.Tensor, *, scale_fp4: float 
                                 _Scales(scale_fp4, ratio, scale_fp8), score_mode, clip_mode, float(fp8_fraction), tau,
                                 out.data_ptr(), out.numel(), None, workspace.data_ptr(), workspace.numel(),
                                 _stream()), "fgmp_quantize_weights")
-    return PackedTensor(out, N, K, 1, scale_fp8 > 0)
+    return PackedTensor(out, N, K, 1, scale_fp8 > 0, None if fp8_fraction < 0 else int(fp8_fraction * B + 0.5) == 0)
 
 
 def quantize_activations(X: torch.Tensor, fisher: torch.Tensor, *, scale_fp4: float, ratio: int = 3, scale_fp8: float = 0.0,
@@ -223,7 +225,7 @@ def quantize_activations(X: torch.Tensor, fisher: torch.Tensor, *, scale_fp4: fl
     if r.__class__ is tuple:
         raise _failed(r)
     M, K = X.shape
-    return PackedTensor(r, M, K, 0, scale_fp8 > 0)
+    return PackedTensor(r, M, K, 0, scale_fp8 > 0, tau == _INF)
 
 
 def calibrate_tau(X: torch.Tensor, fisher: torch.Tensor, *, scale_fp4: float, ratio: int = 3, scale_fp8: float = 0.0,
@@ -300,8 +302,10 @@ def linear(acts: PackedTensor, weights: PackedTensor, *, out_dtype=torch.float32
     if acts.fp8_free or weights.fp8_free:
         return linear_classes(acts, weights, out=out, workspace=workspace)
     assert (out_dtype if out is None else out.dtype) in (torch.float32, torch.bfloat16)
+    a4, w4 = acts.nvfp4, weights.nvfp4
+    known = 0 if a4 is False or w4 is False else 1 if a4 and w4 else -1
     y, ws = (_ext or _load_ext()).linear(acts.blob, weights.blob, acts.rows, weights.rows, acts.K, out,
-                                         out_dtype is torch.bfloat16, workspace)
+                                         out_dtype is torch.bfloat16, workspace, known)
     if ws.__class__ is str:
         raise _failed((y, ws))
     linear.last_workspace = ws
@@ -342,7 +346,7 @@ def linear_fused(X: torch.Tensor, fisher: torch.Tensor, weights: PackedTensor, *
         raise _failed(r)
     y, packed, linear.last_workspace = r
     if packed is not None:
-        return y, PackedTensor(packed, X.shape[0], weights.K, 0)
+        return y, PackedTensor(packed, X.shape[0], weights.K, 0, False, tau == _INF)
     return y
 
 
@@ -358,7 +362,7 @@ def linear_quantize(acts: PackedTensor, weights: PackedTensor, fisher_next: torc
     if ws.__class__ is str:
         raise _failed((blob, ws))
     linear.last_workspace = ws
-    return PackedTensor(blob, M, N, 0)
+    return PackedTensor(blob, M, N, 0, False, tau == _INF)
 
 
 STATIC_SCRATCH_BYTES = 4 * 1024 * 1024

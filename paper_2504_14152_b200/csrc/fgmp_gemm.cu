@@ -16,7 +16,9 @@
 #include "fgmp_common.cuh"
 #include "fgmp_host.h"
 #include "fgmp_ptx.cuh"
+#include "fgmp_quantnext.cuh"
 #include <mutex>
+#include <stdlib.h>
 
 namespace {
 
@@ -176,18 +178,6 @@ __device__ __forceinline__ void pair_tile_coords(int64_t t, int64_t tiles_m, int
     tn = r / rows;
 }
 
-// The activation quantizer of the NEXT layer, run on the accumulators in the epilogue (Section 4.2:
-// the post-processing unit quantizes each output block to FP4 or FP8 from the FP32 partial sums).
-// codes4 == nullptr: off.  The output row of length N is the next layer's K.
-struct QuantNext {
-    const float* fisher;                 // [N] per-channel sensitivity of the next layer's input
-    float s4, k6, s8, inv8, tau;
-    int mode, ratio, free8;
-    uint8_t* codes4; uint8_t* sf; uint32_t* mask; uint8_t* codes8;
-    fgmp_packed_header* header;
-    int64_t MW;                          // mask words per output row
-};
-
 struct GemmParams {
     void* Y; int64_t ldy; int y_is_bf16;
     int64_t M, N, K;
@@ -197,53 +187,6 @@ struct GemmParams {
     int cls_a, cls_w;       // 0, or the class of each operand's plane (1 = NVFP4 blocks, 2 = FP8 blocks): picks the tensor scales
     int accumulate;         // add to Y (fp32) instead of storing
 };
-
-// One row of 32 accumulator columns = two blocks of the next layer's activations: round to bf16 (what an
-// unfused fgmp_linear would have stored), then the quantizer's steps in its order.  Returns the two mask bits.
-__device__ __forceinline__ uint32_t quantize_chunk32(const GemmParams& p, int64_t row, int64_t col0, const uint32_t (&r)[32], float alpha)
-{
-    const QuantNext& q = p.q;
-    uint32_t bits = 0;
-    if (row >= p.M) return 0u;
-#pragma unroll
-    for (int hb = 0; hb < 2; ++hb) {
-        const int64_t col = col0 + 16 * hb;
-        if (col + 16 > p.N) break;
-        const int64_t kb = col >> 4;
-        float v[16], f[16], dq4[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) v[i] = __bfloat162float(__float2bfloat16_rn(__uint_as_float(r[16 * hb + i]) * alpha));
-        const float4* fp = reinterpret_cast<const float4*>(q.fisher + col);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float4 t = __ldg(fp + i);
-            f[4 * i] = t.x; f[4 * i + 1] = t.y; f[4 * i + 2] = t.z; f[4 * i + 3] = t.w;
-        }
-        uint32_t sc = block_dynamic_scale(v, q.k6);
-        uint32_t c4[2], c8[4];
-        block_nvfp4(v, sc, q.s4, c4, dq4);
-        float score;
-        if (q.mode == 0) {
-            score = weighted_sq_sum(v, dq4, f);
-        } else {
-            float dq8[16];
-            block_fp8(v, q.inv8, q.s8, c8, dq8);
-            score = weighted_sq_sum(dq4, dq8, f);
-        }
-        if (score > q.tau) {
-            if (q.mode == 0) {
-                float dq8[16];
-                block_fp8(v, q.inv8, q.s8, c8, dq8);
-            }
-            *reinterpret_cast<uint4*>(q.codes8 + row * p.N + kb * 16) = make_uint4(c8[0], c8[1], c8[2], c8[3]);
-            c4[0] = 0; c4[1] = 0; sc = 0;
-            bits |= 1u << hb;
-        }
-        *reinterpret_cast<uint2*>(q.codes4 + (row * p.N) / 2 + kb * 8) = make_uint2(c4[0], c4[1]);
-        q.sf[fgmp_sf_offset(row, kb, p.N)] = (uint8_t)sc;
-    }
-    return bits;
-}
 
 // one row of 32 accumulator columns -> Y (scaled by the product of the tensor scales)
 __device__ __forceinline__ void store_chunk32(const GemmParams& p, int64_t row, int64_t col0, const uint32_t (&r)[32], float alpha)
@@ -412,7 +355,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
             for (int c = 0; c < P_BN / 32; ++c) {
                 uint32_t r[32];
                 tmem_ld32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * P_BN + c * 32), r);
-                if (p.q.codes4) mbits |= quantize_chunk32(p, row, n0 + c * 32, r, alpha) << (2 * c);
+                if (p.q.codes4) mbits |= quantize_chunk32(p.q, p.M, p.N, row, n0 + c * 32, r, alpha) << (2 * c);
                 else store_chunk32(p, row, n0 + c * 32, r, alpha);
             }
             if (p.q.codes4 && row < p.M) {
@@ -482,7 +425,8 @@ size_t fgmp_ws_linear_quantize(int64_t M, int64_t N, int64_t K)
 size_t fgmp_ws_linear(int64_t M, int64_t N, int64_t K)
 {
     if (fgmp_decode_supported(M, N, K)) return fgmp_ws_decode(M, N, K);
-    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + fgmp_align1k((size_t)N * K * 2);
+    const size_t planes = (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + fgmp_align1k((size_t)N * K * 2), mixed = fgmp_ws_mixed(M, N, K);
+    return planes > mixed ? planes : mixed;
 }
 
 // CTA pairs that can be resident at once on this device (a pair needs two SMs of one cluster domain)
@@ -509,8 +453,20 @@ static fgmp_status resident_pairs(int* pairs)
 
 // expand both operands and run the pair GEMM (M > 16 or a shape the weight-streaming kernel does not take)
 static fgmp_status launch_prefill(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                                  int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, cudaStream_t s)
+                                  int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, int nvfp4, cudaStream_t s)
 {
+    static const int mx_limit = getenv("FGMP_MX") ? atoi(getenv("FGMP_MX")) : 1 << 30;
+    if (M <= mx_limit) {
+        // Operands without any FP8 block go through the NVFP4 tensor-core kind straight from the packed form.  Whether that
+        // is the case is written in the two headers: unless the caller knows (nvfp4 0 or 1), both GEMMs are launched and look
+        // themselves.  (With the next layer's quantizer in the epilogue there is one path.)
+        const bool plain = !qn.codes4;
+        fgmp_status st = FGMP_OK;
+        if (nvfp4 != 1 || !plain)
+            st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, qn, plain && nvfp4 != 0, s);
+        if (st != FGMP_OK || !plain || nvfp4 == 0) return st;
+        return fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, reinterpret_cast<int*>(workspace), s);
+    }
     uint8_t* ws = (uint8_t*)workspace;
     int* status = reinterpret_cast<int*>(ws);
     uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;       // the control area stays as the decode-sized calls need it
@@ -552,9 +508,11 @@ static fgmp_status launch_prefill(const void* packed_acts, const void* packed_we
     return fgmp_launch_status();
 }
 
-extern "C" fgmp_status fgmp_linear(const void* packed_acts, const void* packed_weights,
-                                   void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
-                                   void* workspace, size_t ws_bytes, void* cuda_stream)
+// fgmp_linear for a caller that knows what is in the operands' headers: nvfp4 = 1 no FP8 block in either, 0 some in one of
+// them, -1 not known
+extern "C" fgmp_status fgmp_linear_known(const void* packed_acts, const void* packed_weights,
+                                         void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
+                                         void* workspace, size_t ws_bytes, int nvfp4, void* cuda_stream)
 {
     if (!packed_acts || !packed_weights || !Y || !workspace) return FGMP_ERR_INVALID_ARG;
     if (M < 1 || N < 1 || K < 64 || (K % 64) != 0 || ldy < N) return FGMP_ERR_SHAPE;
@@ -567,7 +525,14 @@ extern "C" fgmp_status fgmp_linear(const void* packed_acts, const void* packed_w
     if (fgmp_decode_supported(M, N, K))
         return fgmp_linear_decode(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, false, s);
     QuantNext off{};
-    return launch_prefill(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, off, s);
+    return launch_prefill(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, off, nvfp4, s);
+}
+
+extern "C" fgmp_status fgmp_linear(const void* packed_acts, const void* packed_weights,
+                                   void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
+                                   void* workspace, size_t ws_bytes, void* cuda_stream)
+{
+    return fgmp_linear_known(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, -1, cuda_stream);
 }
 
 size_t fgmp_ws_linear_classes(int64_t M, int64_t N, int64_t K)
@@ -671,7 +636,7 @@ extern "C" fgmp_status fgmp_linear_quantize(const void* packed_acts, const void*
     q.mask = reinterpret_cast<uint32_t*>(blob + L.off_mask); q.codes8 = blob + L.off_codes8;
     q.header = reinterpret_cast<fgmp_packed_header*>(blob);
     q.MW = L.MW;
-    return launch_prefill(packed_acts, packed_weights, nullptr, 0, N, M, N, K, workspace, q, (cudaStream_t)cuda_stream);
+    return launch_prefill(packed_acts, packed_weights, nullptr, 0, N, M, N, K, workspace, q, -1, (cudaStream_t)cuda_stream);
 }
 
 extern "C" fgmp_status fgmp_workspace_init(void* workspace, size_t ws_bytes, void* cuda_stream)

@@ -75,6 +75,8 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
         if (blockIdx.x == 0 && threadIdx.x == 0) p.status[2] = 0;
         return;
     }
+    // (the headers were complete before this kernel could start; everything else waits for the kernel before it)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (blockIdx.x == 0 && threadIdx.x == 0) p.status[2] = 1;
 
     extern __shared__ uint8_t smem_raw[];
@@ -343,6 +345,13 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     const int64_t tiles = ((M + 127) / 128) * ((p.LW.tiles + 1) / 2);
     const int sms = fgmp_sm_count();
     const int grid = (int)(tiles < sms ? tiles : sms);
-    FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, gemm_nvfp4_kernel<<<grid, G4_THREADS, G4_SMEM, s>>>(tmA, p));
+    // a programmatic dependent: where it does not apply it is gone when the kernel before it ends
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(G4_THREADS); cfg.dynamicSmemBytes = G4_SMEM; cfg.stream = s;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel, tmA, p));
     return fgmp_launch_status();
 }

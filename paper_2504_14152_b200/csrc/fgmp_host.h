@@ -27,6 +27,12 @@ fgmp_status fgmp_linear_decode(const void* packed_acts, const void* packed_weigh
 fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                                    int64_t M, int64_t N, int64_t K, int* status, cudaStream_t s);
 
+// GEMM on the packed weights (fgmp_mixed.cu)
+struct QuantNext;
+size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K);
+fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
+                              int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, cudaStream_t s);
+
 // ---- the FP8 tensor scale of a call (fgmp_scales): given on its own, or scale_fp4 * 2^ratio ----
 #include <math.h>
 inline bool fgmp_scales_valid(const fgmp_scales& sc)
@@ -40,7 +46,7 @@ inline float fgmp_fp8_scale(const fgmp_scales& sc) { return sc.scale_fp8 > 0.f ?
 enum FgmpKernelId {
     FGMP_K_ACT_QUANT = 0, FGMP_K_ACT_AUX, FGMP_K_UNPACK, FGMP_K_EXPAND_A, FGMP_K_EXPAND_W, FGMP_K_GEMM_BF16,
     FGMP_K_W_AMAX, FGMP_K_W_SCORE, FGMP_K_SELECT, FGMP_K_W_MASK, FGMP_K_SCAN, FGMP_K_W_EMIT, FGMP_K_W_AUX,
-    FGMP_K_ACT_SCORES, FGMP_K_DECODE, FGMP_K_GEMM_NVFP4, FGMP_K_COUNT
+    FGMP_K_ACT_SCORES, FGMP_K_DECODE, FGMP_K_GEMM_NVFP4, FGMP_K_GEMM_MIXED, FGMP_K_GEMM_REDUCE, FGMP_K_COUNT
 };
 // Brackets one kernel launch: counts it and, when event timing of this kernel id is on,
 // records a CUDA event before and after it on the launch stream.

@@ -8,6 +8,10 @@
 #include <c10/cuda/CUDAStream.h>
 #include "fgmp.h"
 
+extern "C" fgmp_status fgmp_linear_known(const void* packed_acts, const void* packed_weights,
+                                         void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
+                                         void* workspace, size_t ws_bytes, int nvfp4, void* cuda_stream);
+
 namespace {
 
 // The calls that can return a status raise it through here: the Python side turns the pair into its exception type.
@@ -79,11 +83,11 @@ PyObject* py_quantize_activations(PyObject*, PyObject* const* a, Py_ssize_t n)
     END_HANDLE_TH_ERRORS
 }
 
-// linear(acts, weights, M, N, K, out | None, bf16, workspace | None) -> (Y, workspace)
+// linear(acts, weights, M, N, K, out | None, bf16, workspace | None, nvfp4) -> (Y, workspace)
 PyObject* py_linear(PyObject*, PyObject* const* a, Py_ssize_t n)
 {
     HANDLE_TH_ERRORS
-    TORCH_CHECK_TYPE(n == 8, "linear takes 8 arguments");
+    TORCH_CHECK_TYPE(n == 9, "linear takes 9 arguments");
     const at::Tensor &acts = tensor_of(a[0]), &w = tensor_of(a[1]);
     const int64_t M = as_int(a[2]), N = as_int(a[3]), K = as_int(a[4]);
     void* s = current_stream();
@@ -91,8 +95,8 @@ PyObject* py_linear(PyObject*, PyObject* const* a, Py_ssize_t n)
     fgmp_status st = FGMP_OK;
     at::Tensor ws = workspace_for(a[7], FGMP_OP_LINEAR, M, N, K, acts.device(), s, &st);
     if (st != FGMP_OK) return fail(st, "fgmp_workspace_init");
-    st = fgmp_linear(acts.data_ptr(), w.data_ptr(), out.data_ptr(), out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0), M, N, K,
-                     ws.data_ptr(), (size_t)ws.numel(), s);
+    st = fgmp_linear_known(acts.data_ptr(), w.data_ptr(), out.data_ptr(), out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0), M, N, K,
+                     ws.data_ptr(), (size_t)ws.numel(), (int)as_int(a[8]), s);
     if (st != FGMP_OK) return fail(st, "fgmp_linear");
     PyObject* r = PyTuple_New(2);
     PyTuple_SET_ITEM(r, 0, THPVariable_Wrap(std::move(out)));
