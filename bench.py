@@ -302,7 +302,7 @@ def timed_runs(fn, graph, steps, replays, world):
 def kernel_pass(fg, wk, steps, world):
     """The same steps launched eagerly with CUDA events around every launch of the library's kernels (recorded
     by the library on the launch stream): launch counts and per-kernel durations."""
-    timed = ("expand_acts", "expand_weights", "gemm_bf16_tcgen05", "gemm_nvfp4_tcgen05", "decode_gemm", "quant_act")
+    timed = ("expand_acts", "expand_weights", "gemm_f16_tcgen05", "gemm_mixed_tcgen05", "gemm_reduce", "gemm_nvfp4_tcgen05", "decode_gemm", "quant_act")
     timed = tuple(k for k in timed if k in fg.kernel_names())
     fg.profile_begin(timed)
     for i in range(steps):
@@ -511,9 +511,6 @@ def run_ours(args, world, rank, local):
 # DRAM bytes (read + write) per launch from the committed ncu captures (profiles/*.md).  An entry is
 # removed when its kernel changes after the capture.
 NCU_TRAFFIC = {
-    ("llama2-7b-fc1-decode", "decode_gemm"): {"bytes": 29184000, "file": "profiles/decode_kernel_llama2-7b-fc1-decode.md"},
-    ("llama2-13b-fc1-prefill", "gemm_nvfp4_tcgen05"): {"bytes": 109814016, "file": "profiles/gemm_nvfp4_kernel_llama2-13b-fc1-prefill.md"},
-    ("llama2-7b-fc2-prefill", "gemm_bf16_tcgen05"): {"bytes": 536672512, "file": "profiles/gemm_bf16_pair_kernel_llama2-7b-fc2-prefill.md"},
 }
 
 

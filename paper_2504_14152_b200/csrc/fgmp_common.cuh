@@ -215,6 +215,10 @@ __device__ __forceinline__ float e4m3_to_f32(uint32_t code) { return e4m3x2_to_f
 __device__ __forceinline__ float bf16lo_to_f32(uint32_t pair) { return __uint_as_float(pair << 16); }
 __device__ __forceinline__ float bf16hi_to_f32(uint32_t pair) { return __uint_as_float(pair & 0xffff0000u); }
 
+// Weights go into an fp16 GEMM over 2^t: an FP8 block needs no factor then if t is the ratio of its tensor scale to the NVFP4
+// one, and fp16 holds every NVFP4 value (up to 2688) over 2^t as long as t >= -4.
+__device__ __forceinline__ int fgmp_weight_exponent(const fgmp_packed_header* h) { return max(h->fp8_log2_ratio, -4); }
+
 // ---------------------------------------------------------------- block math
 // One block of 16 values in registers.  Every step below is a single IEEE fp32 operation
 // (no contraction): this sequence is what makes codes and scores reproducible bit for bit.

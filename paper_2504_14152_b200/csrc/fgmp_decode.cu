@@ -320,7 +320,7 @@ decode_kernel(const __grid_constant__ DecParams p)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    const uint32_t tmem_base = TMEM_ALL;
     if (threadIdx.x == 0) FGMP_STAMP_ANY(1);
 
     if (warp == W_PROD) {

@@ -1,11 +1,10 @@
 // fgmp_linear: the mixed-precision GEMM (Section 4.1 of the paper).
 //
-// General path ("common container"): every block of both operands, whatever its format, is
-// an exact bf16 number once its microscale is folded in (E2M1 x E4M3 scale has at most 6
-// significant bits, E4M3 has 4).  A streaming pass expands the packed operands into bf16
-// planes, and a persistent tcgen05 kernel multiplies them with FP32 accumulation in TMEM;
-// the two FP32 tensor scales are applied in the epilogue.  All four block-pair products of
-// the paper's datapath (FP4xFP4, FP4xFP8, FP8xFP4, FP8xFP8) are therefore exact products.
+// Large batches ("common container"): every block of both operands, whatever its format, is an exact fp16 number once its
+// microscale is folded in (E2M1 x E4M3 scale has at most 6 significant bits, E4M3 has 4).  A streaming pass expands the packed
+// operands into fp16 planes, and a persistent tcgen05 kernel multiplies them with FP32 accumulation in TMEM; the two FP32
+// tensor scales are applied in the epilogue.  All four block-pair products of the paper's datapath (FP4xFP4, FP4xFP8, FP8xFP4,
+// FP8xFP8) are therefore exact products.  Smaller batches: fgmp_mixed.cu.
 //
 // Kernel structure (one CTA per SM, 192 threads):
 //   warp 0    : TMA producer   (global -> 128B-swizzled shared tiles, mbarrier complete_tx)
@@ -17,48 +16,35 @@
 #include "fgmp_host.h"
 #include "fgmp_ptx.cuh"
 #include "fgmp_quantnext.cuh"
+#include "fgmp_deq.cuh"
 #include <mutex>
-#include <stdlib.h>
 
 namespace {
 
-// ------------------------------------------------------------------ expand to bf16 planes
-// plane[r, k] = e2m1 * e4m3scale (NVFP4 block) or e4m3 * 2^ratio (FP8 block); exact in bf16.
-__device__ __forceinline__ void e4m3x16_scaled(const uint4& c, float r8, float (&v)[16])
-{
-    const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        float2 a = e4m3x2_to_f32x2(w[i] & 0xffff), bb = e4m3x2_to_f32x2(w[i] >> 16);
-        v[4 * i] = a.x * r8; v[4 * i + 1] = a.y * r8; v[4 * i + 2] = bb.x * r8; v[4 * i + 3] = bb.y * r8;
-    }
-}
-
+// ------------------------------------------------------------------ expand to fp16 planes
 __device__ __forceinline__ void store_256(void* dst, const uint32_t (&o)[8])
 {
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
                  ::"l"(dst), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
 }
-
-// 16 values that are exact in bf16 (the low 16 bits of every float are zero) -> 32 bytes
-__device__ __forceinline__ void store_bf16x16(uint4* dst, const float (&v)[16])
+// a block's 16 values as 8 pairs: E2M1 codes times the microscale times a power of two, or E4M3 codes times a power of two
+__device__ __forceinline__ void deq_nvfp4(const uint2& c, uint32_t scale_code, uint32_t factor, uint32_t (&o)[8])
 {
-    uint32_t o[8];
+    const uint32_t d = hmul2(e4m3x2_to_f16x2(scale_code | (scale_code << 8)), factor);
+    e2m1x8_to_f16(c.x, o); e2m1x8_to_f16(c.y, o + 4);
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-        o[i] = (__float_as_uint(v[2 * i]) >> 16) | (__float_as_uint(v[2 * i + 1]) & 0xffff0000u);
-    store_256(dst, o);        // one 32-byte store (the planes are 32-byte aligned and a block is 32 bytes): whole sectors per lane
+    for (int i = 0; i < 8; ++i) o[i] = hmul2(o[i], d);
 }
-
-__device__ __forceinline__ void nvfp4x16_scaled(const uint2& c, uint32_t scale_code, float (&v)[16])
+__device__ __forceinline__ void deq_fp8(const uint4& c, uint32_t factor, uint32_t (&o)[8])
 {
-    const float d = e4m3_to_f32(scale_code);
-    const uint32_t w[2] = {c.x, c.y};
+    const uint32_t w[4] = {c.x, c.y, c.z, c.w};
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        float2 q = e2m1x2_to_f32x2((w[i >> 2] >> ((i & 3) * 8)) & 0xff);
-        v[2 * i] = q.x * d; v[2 * i + 1] = q.y * d;
-    }
+    for (int i = 0; i < 4; ++i) { o[2 * i] = hmul2(e4m3x2_to_f16x2(w[i] & 0xffffu), factor); o[2 * i + 1] = hmul2(e4m3x2_to_f16x2(w[i] >> 16), factor); }
+}
+__device__ __forceinline__ uint32_t pow2_f16x2(int e)
+{
+    const __half2 h = __float2half2_rn(__int_as_float((127 + e) << 23));
+    return *reinterpret_cast<const uint32_t*>(&h);
 }
 
 // A packed tensor is read only if its header describes the tensor the call was given; otherwise the
@@ -73,80 +59,128 @@ __device__ __forceinline__ bool header_matches(const fgmp_packed_header* h, int6
     return ok;
 }
 
-// packed activations -> bf16 plane; one thread per block
-__global__ void __launch_bounds__(256) expand_kernel(const uint8_t* blob, int64_t rows, int64_t K, uint4* plane, int* status, int cls)
+// Whether the all-NVFP4 GEMM takes the call (decided alike by every kernel of it from the two headers)
+__device__ __forceinline__ bool no_fp8_block(const uint8_t* ablob, const uint8_t* wblob)
 {
-    if (status[2]) return;                              // the all-NVFP4 GEMM has produced the result already
-    const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(blob);
-    if (!header_matches(h, rows, K, 0u, status, 11, cls)) return;
-    const PackedLayout L = fgmp_layout(rows, K, 0, 0);
-    const uint32_t* pmask = reinterpret_cast<const uint32_t*>(blob + L.off_mask);
-    const float r8 = cls ? 1.0f : __int_as_float((127 + h->fp8_log2_ratio) << 23);
-    const int64_t nblk = rows * L.KB;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblk; b += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r = b / L.KB, kb = b % L.KB;
-        uint32_t word = pmask[r * L.MW + (kb >> 5)];
-        bool is8 = (word >> (kb & 31)) & 1;
-        float v[16];
-        if (is8) e4m3x16_scaled(*reinterpret_cast<const uint4*>(blob + L.off_codes8 + (size_t)(r * K + kb * 16)), r8, v);
-        else nvfp4x16_scaled(*reinterpret_cast<const uint2*>(blob + L.off_codes4 + (r * K) / 2 + kb * 8),
-                             blob[L.off_sf + fgmp_sf_offset(r, kb, K)], v);
-        if (cls && (is8 != (cls == 2))) {               // a block of the other class
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = 0.f;
-        }
-        store_bf16x16(plane + (r * K) / 8 + kb * 2, v);
-    }
+    return reinterpret_cast<const fgmp_packed_header*>(ablob)->n_fp8 == 0 && reinterpret_cast<const fgmp_packed_header*>(wblob)->n_fp8 == 0;
 }
 
-// packed weights -> bf16 plane; one CTA of 128 threads per unit record, consecutive threads on
-// consecutive blocks of one row, four blocks per thread in flight at a time
-__global__ void __launch_bounds__(128) expand_w_kernel(const uint8_t* __restrict__ blob, int64_t rows, int64_t K, uint4* __restrict__ plane, int* status, int cls)
+// Packed operands -> fp16 planes over their NVFP4 tensor scales (the weights over a further 2^t, see fgmp_weight_exponent), both
+// in one launch: the first blocks take a unit of the weights each (consecutive threads on consecutive blocks of a row, eight
+// blocks per thread in flight), the others 512 blocks of the activations.  Bound by the stores (32 bytes per
+// block and lane): 4096 x 11008 weights and 4096 x 4096 activations together XX us, YY TB/s; as two kernels that went through
+// fp32 49 us.
+struct ExpandParams {
+    const uint8_t* ablob; const uint8_t* wblob;
+    int64_t M, N, K;
+    uint8_t* planeA; uint8_t* planeW;
+    int* status;
+    int cls_a, cls_w, leave_nvfp4;
+    uint32_t w_blocks;                   // thread blocks for the weights
+};
+__global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ ExpandParams p)
 {
     __shared__ UnitScratch sc;
-    if (status[2]) return;                              // the all-NVFP4 GEMM has produced the result already
-    const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(blob);
-    if (!header_matches(h, rows, K, 1u, status, 12, cls)) return;
-    const PackedLayout L = fgmp_layout(rows, K, 1, 0);
-    const float r8 = cls ? 1.0f : __int_as_float((127 + h->fp8_log2_ratio) << 23);
-    const int64_t unit = blockIdx.x, tile = unit / L.chunks, c = unit % L.chunks;
-    const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x]);
-    const uint8_t* rec = blob + L.off_rec + (size_t)unit * REC_BYTES;
-    const uint8_t* halves = blob + L.off_ovf + (size_t)reinterpret_cast<const uint32_t*>(blob + L.off_uptr)[unit] * 16 + fgmp_list_halves_offset(cnt);
-    const int j = threadIdx.x & 15;
-    const int64_t kb = c * 16 + j;
-    if (kb >= L.KB) return;
-#pragma unroll 1
-    for (int i0 = 0; i0 < 16; i0 += 4) {
-        uint2 slot[4], hi[4];
-        uint32_t sfb[4], pos[4];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (p.leave_nvfp4 && no_fp8_block(p.ablob, p.wblob)) return;
+    if (blockIdx.x >= p.w_blocks) {
+        const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
+        if (!header_matches(h, p.M, p.K, 0u, p.status, 11, p.cls_a)) return;
+        const PackedLayout L = fgmp_layout(p.M, p.K, 0, 0);
+        const uint32_t* pmask = reinterpret_cast<const uint32_t*>(p.ablob + L.off_mask);
+        const uint32_t f8 = pow2_f16x2(p.cls_a ? 0 : h->fp8_log2_ratio), one = pow2_f16x2(0), KB = (uint32_t)L.KB;
+        // four blocks per thread, the loads of all of them before the first is converted
+        const uint64_t b0 = (uint64_t)(blockIdx.x - p.w_blocks) * 512 + threadIdx.x, nblk = (uint64_t)p.M * KB;
+        uint32_t word[4], sf[4];
+        uint2 c4[4];
+        uint4 c8[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int row = (threadIdx.x >> 4) + 8 * (i0 + i);
-            pos[i] = sc.pos(row, j);
+            const uint64_t b = b0 + 128 * i;
+            word[i] = 0; sf[i] = 0; c4[i] = make_uint2(0u, 0u);
+            if (b < nblk) {
+                const uint32_t r = (uint32_t)(b / KB), kb = (uint32_t)(b - (uint64_t)r * KB);
+                word[i] = (__ldg(pmask + (size_t)r * L.MW + (kb >> 5)) >> (kb & 31)) & 1u;
+                sf[i] = __ldg(p.ablob + L.off_sf + fgmp_sf_offset(r, kb, p.K));
+                c4[i] = __ldg(reinterpret_cast<const uint2*>(p.ablob + L.off_codes4 + (size_t)b * 8));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            c8[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (word[i]) c8[i] = __ldg(reinterpret_cast<const uint4*>(p.ablob + L.off_codes8 + (size_t)(b0 + 128 * i) * 16));
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint64_t b = b0 + 128 * i;
+            if (b >= nblk) break;
+            uint32_t o[8];
+            if (word[i]) deq_fp8(c8[i], f8, o);
+            else deq_nvfp4(c4[i], sf[i], one, o);
+            if (p.cls_a && ((word[i] != 0) != (p.cls_a == 2))) {       // a block of the other class
+#pragma unroll
+                for (int e = 0; e < 8; ++e) o[e] = 0;
+            }
+            store_256(p.planeA + (size_t)b * 32, o);
+        }
+        return;
+    }
+    const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
+    if (!header_matches(h, p.N, p.K, 1u, p.status, 12, p.cls_w)) return;
+    const PackedLayout L = fgmp_layout(p.N, p.K, 1, 0);
+    const int t = p.cls_w ? 0 : fgmp_weight_exponent(h);
+    const uint32_t f4 = pow2_f16x2(-t), f8 = pow2_f16x2(p.cls_w ? 0 : h->fp8_log2_ratio - t);
+    const uint32_t unit = blockIdx.x, tile = unit / (uint32_t)L.chunks, c = unit % (uint32_t)L.chunks;
+    const uint8_t* rec = p.wblob + L.off_rec + (size_t)unit * REC_BYTES;
+    const uint32_t j = threadIdx.x & 15, row0 = threadIdx.x >> 4;
+    const int64_t kb = (int64_t)c * 16 + j;
+    // eight blocks of the thread in flight; the first ones while the positions in the list are worked out
+    uint2 slot[8];
+    uint32_t sfb[8];
+    auto fetch = [&](uint32_t i0) {
+#pragma unroll
+        for (uint32_t i = 0; i < 8; ++i) {
+            const uint32_t row = row0 + 8 * (i0 + i);
             slot[i] = __ldg(reinterpret_cast<const uint2*>(rec + REC_W4 + fgmp_rec_w4_offset(row, j)));
             sfb[i] = __ldg(rec + REC_SF + fgmp_rec_sf_offset(row, j));
+        }
+    };
+    const uint32_t first = reinterpret_cast<const uint32_t*>(p.wblob + L.off_uptr)[unit];
+    const uint32_t bits = reinterpret_cast<const uint16_t*>(p.wblob + L.off_mask)[(size_t)unit * 128 + threadIdx.x];
+    fetch(0);
+    const uint32_t cnt = sc.init(bits);
+    const uint8_t* halves = p.wblob + L.off_ovf + (size_t)first * 16 + fgmp_list_halves_offset(cnt);
+    if (kb >= L.KB) return;
+#pragma unroll
+    for (uint32_t i0 = 0; i0 < 16; i0 += 8) {
+        uint2 hi[8];
+        uint32_t is8 = 0;
+#pragma unroll
+        for (uint32_t i = 0; i < 8; ++i) {
+            const uint32_t pos = sc.pos(row0 + 8 * (i0 + i), j);
             hi[i] = make_uint2(0u, 0u);
-            if (pos[i] != 0xffffu) hi[i] = __ldg(reinterpret_cast<const uint2*>(halves + (size_t)pos[i] * 8));
+            if (pos != 0xffffu) { hi[i] = __ldg(reinterpret_cast<const uint2*>(halves + (size_t)pos * 8)); is8 |= 1u << i; }
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int row = (threadIdx.x >> 4) + 8 * (i0 + i);
-            const int64_t r = tile * 128 + row;
+        for (uint32_t i = 0; i < 8; ++i) {
+            const int64_t r = (int64_t)tile * 128 + row0 + 8 * (i0 + i);
             if (r >= L.rows) continue;
-            float v[16];
-            if (pos[i] != 0xffffu) e4m3x16_scaled(make_uint4(slot[i].x, slot[i].y, hi[i].x, hi[i].y), r8, v);
-            else nvfp4x16_scaled(slot[i], sfb[i], v);
-            if (cls && ((pos[i] != 0xffffu) != (cls == 2))) {
+            const bool b8 = (is8 >> i) & 1u;
+            uint32_t o[8];
+            if (b8) deq_fp8(make_uint4(slot[i].x, slot[i].y, hi[i].x, hi[i].y), f8, o);
+            else deq_nvfp4(slot[i], sfb[i], f4, o);
+            if (p.cls_w && (b8 != (p.cls_w == 2))) {
 #pragma unroll
-                for (int e = 0; e < 16; ++e) v[e] = 0.f;
+                for (int e = 0; e < 8; ++e) o[e] = 0;
             }
-            store_bf16x16(plane + (r * K) / 8 + kb * 2, v);
+            store_256(p.planeW + (size_t)(r * p.K + kb * 16) * 2, o);
         }
+        if (i0 == 0) fetch(8);
     }
 }
 
-// ------------------------------------------------------------------ bf16 tcgen05 GEMM on CTA pairs
+// ------------------------------------------------------------------ fp16 tcgen05 GEMM on CTA pairs
 // Two CTAs of a cluster share one 256 x 256 output tile: each loads its 128 rows of A and its half
 // (128 rows) of B, the pair's leader issues tcgen05.mma cta_group::2 (M = 256), which reads both
 // halves of B from the two shared memories, and each CTA's TMEM holds the accumulators of its own
@@ -154,7 +188,7 @@ __global__ void __launch_bounds__(128) expand_w_kernel(const uint8_t* __restrict
 // CTA with a 128 x 256 tile needs 48 KiB for half of that), which is what the L2 -> shared-memory path can
 // sustain.  No TMA multicast.  Persistent: warp 0 = TMA producer, warp 1 = MMA issuer (leader CTA
 // only) and TMEM owner, warps 2-5 = epilogue; two accumulator buffers of 256 TMEM columns.
-constexpr int BK = 64;                              // BK bf16 = one 128-byte swizzle row
+constexpr int BK = 64;                              // BK fp16 = one 128-byte swizzle row
 constexpr int UMMA_K = 16;
 constexpr int GEMM_THREADS = 192;
 constexpr int P_BM = 256, P_BN = 256;               // per pair
@@ -162,8 +196,8 @@ constexpr int P_STAGES = 6;
 constexpr uint32_t P_A_BYTES = 128 * BK * 2, P_B_BYTES = 128 * BK * 2, P_STAGE_BYTES = P_A_BYTES + P_B_BYTES;
 constexpr uint32_t TMEM_COLS = 2 * P_BN;            // two accumulator buffers
 constexpr size_t PAIR_SMEM = (size_t)P_STAGES * P_STAGE_BYTES + 1024 /*alignment slack*/ + 256 /*barriers*/;
-// instruction descriptor, kind::f16: D=f32, A=B=bf16, both K-major, N=256, M=256
-constexpr uint32_t IDESC_BF16_PAIR = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(P_BN >> 3) << 17) | ((uint32_t)(P_BM >> 4) << 24);
+// instruction descriptor, kind::f16: D=f32, A=B=f16, both K-major, N=256, M=256
+constexpr uint32_t IDESC_F16_PAIR = (1u << 4) | ((uint32_t)(P_BN >> 3) << 17) | ((uint32_t)(P_BM >> 4) << 24);
 
 // Tile order: bands of P_RASTER_M tile rows, all tile columns of a band before the next band, tile rows
 // fastest inside a band.  The pairs that run together then share few A and B panels, which the
@@ -186,6 +220,7 @@ struct GemmParams {
     QuantNext q;
     int cls_a, cls_w;       // 0, or the class of each operand's plane (1 = NVFP4 blocks, 2 = FP8 blocks): picks the tensor scales
     int accumulate;         // add to Y (fp32) instead of storing
+    int leave_nvfp4;        // operands without any FP8 block are left to the all-NVFP4 GEMM
 };
 
 // one row of 32 accumulator columns -> Y (scaled by the product of the tensor scales)
@@ -255,9 +290,12 @@ __device__ __forceinline__ void store_chunk32(const GemmParams& p, int64_t row, 
 }
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
-gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmParams p)
+gemm_f16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, GemmParams p)
 {
-    if (p.status[2]) return;                            // the all-NVFP4 GEMM has produced the result already (every thread of every CTA sees the same word)
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    if (p.leave_nvfp4 && p.ha->n_fp8 == 0 && p.hw->n_fp8 == 0) return;      // (the same for every thread of every CTA)
+    if (blockIdx.x == 0 && threadIdx.x == 0) p.status[2] = 0;               // word 2: the all-NVFP4 GEMM has produced Y
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // offset from the array: stays known as shared memory
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)P_STAGES * P_STAGE_BYTES);
@@ -330,7 +368,7 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
 #pragma unroll
                     for (int k = 0; k < BK / UMMA_K; ++k)
                         umma_f16_pair(d_tmem, adesc + (uint64_t)(k * UMMA_K * 2 / 16), bdesc + (uint64_t)(k * UMMA_K * 2 / 16),
-                                      IDESC_BF16_PAIR, (kb | k) ? 1u : 0u);
+                                      IDESC_F16_PAIR, (kb | k) ? 1u : 0u);
                     umma_commit_pair(empty0 + 8 * stage, 3);          // the stage is free in both CTAs
                     if (++stage == P_STAGES) { stage = 0; phase ^= 1; }
                 }
@@ -339,7 +377,8 @@ gemm_bf16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_cons
         }
     } else {
         const int q = warp & 3;                        // TMEM lane quadrant this warp may read
-        const float alpha = __fmul_rn(p.cls_a == 2 ? p.ha->scale_fp8 : p.ha->scale_fp4, p.cls_w == 2 ? p.hw->scale_fp8 : p.hw->scale_fp4);
+        float alpha = __fmul_rn(p.cls_a == 2 ? p.ha->scale_fp8 : p.ha->scale_fp4, p.cls_w == 2 ? p.hw->scale_fp8 : p.hw->scale_fp4);
+        if (!p.cls_w) alpha = __fmul_rn(alpha, __int_as_float((127 + fgmp_weight_exponent(p.hw)) << 23));
         bool ok = true;
         int64_t it = 0;
         for (int64_t t = pair; t < num_tiles && ok; t += num_pairs, ++it) {
@@ -401,8 +440,8 @@ EncodeTiledFn get_encode_fn()
     return fn;
 }
 
-// 2-D bf16 row-major [rows, K] tensor, box = [box_rows, 64 elements], 128-byte swizzle
-bool make_tmap_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int box_rows)
+// 2-D fp16 row-major [rows, K] tensor, box = [box_rows, 64 elements], 128-byte swizzle
+bool make_tmap_f16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int box_rows)
 {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
@@ -410,7 +449,7 @@ bool make_tmap_bf16(CUtensorMap* map, const void* base, int64_t rows, int64_t K,
     cuuint64_t strides[1] = {(cuuint64_t)K * 2};
     cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
+    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
@@ -439,12 +478,12 @@ static fgmp_status resident_pairs(int* pairs)
     if (dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
     std::lock_guard<std::mutex> lk(mu);
     if (!pairs_of_device[dev]) {
-        if (cudaFuncSetAttribute(gemm_bf16_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_SMEM) != cudaSuccess)
+        if (cudaFuncSetAttribute(gemm_f16_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PAIR_SMEM) != cudaSuccess)
             return FGMP_ERR_CUDA;
         cudaLaunchConfig_t qc = {};
         qc.gridDim = dim3((unsigned)(fgmp_sm_count() & ~1)); qc.blockDim = dim3(GEMM_THREADS); qc.dynamicSmemBytes = PAIR_SMEM;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, gemm_bf16_pair_kernel, &qc) != cudaSuccess || n < 1) return FGMP_ERR_CUDA;
+        if (cudaOccupancyMaxActiveClusters(&n, gemm_f16_pair_kernel, &qc) != cudaSuccess || n < 1) return FGMP_ERR_CUDA;
         pairs_of_device[dev] = n;
     }
     *pairs = pairs_of_device[dev];
@@ -452,60 +491,83 @@ static fgmp_status resident_pairs(int* pairs)
 }
 
 // expand both operands and run the pair GEMM (M > 16 or a shape the weight-streaming kernel does not take)
+fgmp_status fgmp_expand(const void* packed_acts, const void* packed_weights, int64_t M, int64_t N, int64_t K, uint8_t* planeA, uint8_t* planeW,
+                        int* status, int cls_a, int cls_w, bool leave_nvfp4, cudaStream_t s)
+{
+    ExpandParams p;
+    p.ablob = (const uint8_t*)packed_acts; p.wblob = (const uint8_t*)packed_weights;
+    p.M = M; p.N = N; p.K = K; p.planeA = planeA; p.planeW = planeW; p.status = status;
+    p.cls_a = cls_a; p.cls_w = cls_w; p.leave_nvfp4 = leave_nvfp4 ? 1 : 0;
+    p.w_blocks = planeW ? (uint32_t)fgmp_layout(N, K, 1, 0).units : 0u;
+    const int64_t nblk = planeA ? M * (K / 16) : 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.gridDim = dim3(p.w_blocks + (unsigned)((nblk + 511) / 512)); cfg.blockDim = dim3(128);
+    FGMP_LAUNCH(planeW ? FGMP_K_EXPAND_W : FGMP_K_EXPAND_A, s, cudaLaunchKernelEx(&cfg, expand_kernel, p));
+    return fgmp_launch_status();
+}
+
+// the pair GEMM over the planes
+static fgmp_status launch_pair_gemm(const GemmParams& p, const uint8_t* planeA, const uint8_t* planeW, cudaStream_t s)
+{
+    int pairs_avail = 0;
+    const fgmp_status st = resident_pairs(&pairs_avail);
+    if (st != FGMP_OK) return st;
+    CUtensorMap tmA, tmB;
+    if (!make_tmap_f16(&tmA, planeA, p.M, p.K, 128) || !make_tmap_f16(&tmB, planeW, p.N, p.K, 128)) return FGMP_ERR_CUDA;
+    const int64_t tiles = ((p.M + P_BM - 1) / P_BM) * ((p.N + P_BN - 1) / P_BN);
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.gridDim = dim3(2u * (unsigned)(tiles < pairs_avail ? tiles : pairs_avail)); cfg.blockDim = dim3(GEMM_THREADS); cfg.dynamicSmemBytes = PAIR_SMEM;
+    FGMP_LAUNCH(FGMP_K_GEMM_F16, s, cudaLaunchKernelEx(&cfg, gemm_f16_pair_kernel, tmA, tmB, p));
+    return fgmp_launch_status();
+}
+
+// Modelled time in us of expansion and pair GEMM, beside fgmp_mixed_us: launches and tails, 0.65 us per million elements of
+// either operand, then waves of 256 x 256 tiles over the pairs at 0.34 us per 64 elements of K.
+static double planes_us(int64_t M, int64_t N, int64_t K)
+{
+    const int64_t tiles = ((M + P_BM - 1) / P_BM) * ((N + P_BN - 1) / P_BN), pairs = fgmp_sm_count() / 2;
+    return 10.0 + 0.65e-6 * (double)(M + N) * (double)K + (double)((tiles + pairs - 1) / pairs) * (double)(K / 64) * 0.34;
+}
+
+// M > 16 or a shape the weight-streaming kernel does not take.  nvfp4: 1 no FP8 block in either operand, 0 some in one of
+// them, -1 not known.
 static fgmp_status launch_prefill(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                                   int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, int nvfp4, cudaStream_t s)
 {
-    static const int mx_limit = getenv("FGMP_MX") ? atoi(getenv("FGMP_MX")) : 1 << 30;
-    if (M <= mx_limit) {
-        // Operands without any FP8 block go through the NVFP4 tensor-core kind straight from the packed form.  Whether that
-        // is the case is written in the two headers: unless the caller knows (nvfp4 0 or 1), both GEMMs are launched and look
-        // themselves.  (With the next layer's quantizer in the epilogue there is one path.)
-        const bool plain = !qn.codes4;
-        fgmp_status st = FGMP_OK;
-        if (nvfp4 != 1 || !plain)
-            st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, qn, plain && nvfp4 != 0, s);
-        if (st != FGMP_OK || !plain || nvfp4 == 0) return st;
-        return fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, reinterpret_cast<int*>(workspace), s);
-    }
     uint8_t* ws = (uint8_t*)workspace;
     int* status = reinterpret_cast<int*>(ws);
-    uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;       // the control area stays as the decode-sized calls need it
-    uint8_t* planeW = planeA + fgmp_align1k((size_t)M * K * 2);
-
-    int pairs_avail = 0;
-    fgmp_status stp = resident_pairs(&pairs_avail);
-    if (stp != FGMP_OK) return stp;
-    CUtensorMap tmA, tmB;
-    if (!make_tmap_bf16(&tmA, planeA, M, K, 128) || !make_tmap_bf16(&tmB, planeW, N, K, 128)) return FGMP_ERR_CUDA;
-
-    if (cudaMemsetAsync(status, 0, 256, s) != cudaSuccess) return FGMP_ERR_CUDA;
-    // Operands without any FP8 block go through the NVFP4 tensor-core kind straight from the packed form; whether
-    // that is the case is written in the two headers, so the kernel looks itself and leaves word 2 of the status
-    // area at 1 if it has done the work.  (The variant with the next layer's quantizer in the epilogue has the
-    // general path only.)
-    if (!qn.codes4) {
-        const fgmp_status st4 = fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, s);
-        if (st4 != FGMP_OK) return st4;
+    // Operands without any FP8 block go through the NVFP4 tensor-core kind straight from the packed form.  Whether that is
+    // the case is written in the two headers: unless the caller knows, the kernels of both ways are launched and look
+    // themselves.  (With the next layer's quantizer in the epilogue there is the general way only.)
+    const bool plain = !qn.codes4, leave = plain && nvfp4 < 0;
+    if (plain && nvfp4 == 1) return fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, true, s);
+    fgmp_status st;
+    // At small and middling batches the weights are dequantized inside the GEMM, once per token tile; with many token tiles a
+    // plane that is expanded once is read faster than that (777 x 11008 x 4096: 86 against 105 us; 2048 x 4096 x 4096: 81
+    // against 60).
+    if (fgmp_mixed_us(M, N, K) <= planes_us(M, N, K)) {
+        st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, qn, leave, s);
+    } else {
+        uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;   // the control area stays as the decode-sized calls need it
+        uint8_t* planeW = planeA + fgmp_align1k((size_t)M * K * 2);
+        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, planeA, planeW, status, 0, 0, leave, s)) != FGMP_OK) return st;
+        GemmParams p{};
+        p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K;
+        p.ha = reinterpret_cast<const fgmp_packed_header*>(packed_acts);
+        p.hw = reinterpret_cast<const fgmp_packed_header*>(packed_weights);
+        p.status = status; p.q = qn; p.leave_nvfp4 = leave ? 1 : 0;
+        st = launch_pair_gemm(p, planeA, planeW, s);
     }
-    const int sms = fgmp_sm_count();
-    {
-        const int64_t nb = M * (K / 16);
-        const int g = (int)((nb + 255) / 256 < (int64_t)sms * 8 ? (nb + 255) / 256 : (int64_t)sms * 8);
-        FGMP_LAUNCH(FGMP_K_EXPAND_A, s, expand_kernel<<<g, 256, 0, s>>>((const uint8_t*)packed_acts, M, K, reinterpret_cast<uint4*>(planeA), status, 0));
-        const PackedLayout LW = fgmp_layout(N, K, 1, 0);
-        FGMP_LAUNCH(FGMP_K_EXPAND_W, s, expand_w_kernel<<<(unsigned)LW.units, 128, 0, s>>>((const uint8_t*)packed_weights, N, K, reinterpret_cast<uint4*>(planeW), status, 0));
-    }
-    GemmParams p;
-    p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K;
-    p.ha = reinterpret_cast<const fgmp_packed_header*>(packed_acts);
-    p.hw = reinterpret_cast<const fgmp_packed_header*>(packed_weights);
-    p.status = status;
-    p.q = qn;
-    p.cls_a = 0; p.cls_w = 0; p.accumulate = 0;
-    const int64_t tiles = ((M + P_BM - 1) / P_BM) * ((N + P_BN - 1) / P_BN);
-    const int pairs = (int)(tiles < pairs_avail ? tiles : pairs_avail);
-    FGMP_LAUNCH(FGMP_K_GEMM_BF16, s, gemm_bf16_pair_kernel<<<2 * pairs, GEMM_THREADS, PAIR_SMEM, s>>>(tmA, tmB, p));
-    return fgmp_launch_status();
+    if (st != FGMP_OK || !leave) return st;
+    return fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, false, s);
 }
 
 // fgmp_linear for a caller that knows what is in the operands' headers: nvfp4 = 1 no FP8 block in either, 0 some in one of
@@ -559,40 +621,24 @@ extern "C" fgmp_status fgmp_linear_classes(const void* packed_acts, const void* 
     int* status = reinterpret_cast<int*>(ws);
     uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;
     uint8_t* planeW = planeA + fgmp_align1k((size_t)M * K * 2);
-    int pairs_avail = 0;
-    if ((st = resident_pairs(&pairs_avail)) != FGMP_OK) return st;
-    CUtensorMap tmA, tmB;
-    if (!make_tmap_bf16(&tmA, planeA, M, K, 128) || !make_tmap_bf16(&tmB, planeW, N, K, 128)) return FGMP_ERR_CUDA;
     if (cudaMemsetAsync(status, 0, 256, s) != cudaSuccess) return FGMP_ERR_CUDA;
-    const int sms = fgmp_sm_count();
-    const int64_t nb = M * (K / 16);
-    const int ga = (int)((nb + 255) / 256 < (int64_t)sms * 8 ? (nb + 255) / 256 : (int64_t)sms * 8);
-    const PackedLayout LW = fgmp_layout(N, K, 1, 0);
-    GemmParams p;
+    GemmParams p{};
     p.Y = Y; p.ldy = ldy; p.y_is_bf16 = 0; p.M = M; p.N = N; p.K = K;
     p.ha = reinterpret_cast<const fgmp_packed_header*>(packed_acts);
     p.hw = reinterpret_cast<const fgmp_packed_header*>(packed_weights);
     p.status = status;
-    p.q = QuantNext{};
-    const int64_t tiles = ((M + P_BM - 1) / P_BM) * ((N + P_BN - 1) / P_BN);
-    const int pairs = (int)(tiles < pairs_avail ? tiles : pairs_avail);
     // (activation class, weight class) in an order that re-expands one operand per pass
     const int order[4][2] = {{1, 1}, {1, 2}, {2, 2}, {2, 1}};
     int have_a = 0, have_w = 0;
     for (int i = 0; i < 4; ++i) {
         const int ca = order[i][0], cw = order[i][1];
-        if (ca != have_a) {
-            FGMP_LAUNCH(FGMP_K_EXPAND_A, s, expand_kernel<<<ga, 256, 0, s>>>((const uint8_t*)packed_acts, M, K, reinterpret_cast<uint4*>(planeA), status, ca));
-            have_a = ca;
-        }
-        if (cw != have_w) {
-            FGMP_LAUNCH(FGMP_K_EXPAND_W, s, expand_w_kernel<<<(unsigned)LW.units, 128, 0, s>>>((const uint8_t*)packed_weights, N, K, reinterpret_cast<uint4*>(planeW), status, cw));
-            have_w = cw;
-        }
+        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, ca != have_a ? planeA : nullptr, cw != have_w ? planeW : nullptr, status, ca, cw, false, s)) != FGMP_OK)
+            return st;
+        have_a = ca; have_w = cw;
         p.cls_a = ca; p.cls_w = cw; p.accumulate = i > 0;
-        FGMP_LAUNCH(FGMP_K_GEMM_BF16, s, gemm_bf16_pair_kernel<<<2 * pairs, GEMM_THREADS, PAIR_SMEM, s>>>(tmA, tmB, p));
+        if ((st = launch_pair_gemm(p, planeA, planeW, s)) != FGMP_OK) return st;
     }
-    return fgmp_launch_status();
+    return FGMP_OK;
 }
 
 extern "C" fgmp_status fgmp_linear_quantize(const void* packed_acts, const void* packed_weights,

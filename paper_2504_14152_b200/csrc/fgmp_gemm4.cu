@@ -55,6 +55,7 @@ struct Gemm4Params {
     PackedLayout LA, LW;
     void* Y; int64_t ldy; int y_is_bf16;
     int64_t M, N, K;
+    int sole;                             // nothing else takes the call if this kernel does not
     int* status;                          // [0..1] device-side status, [2] 1 = this kernel has produced Y
 };
 
@@ -70,13 +71,12 @@ __device__ __forceinline__ bool g4_applicable(const Gemm4Params& p)
 __global__ void __launch_bounds__(G4_THREADS, 1)
 gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
 {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     // operands with FP8 blocks (or headers that do not match the call) are left to the general path
     if (!g4_applicable(p)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) p.status[2] = 0;
+        if (p.sole && blockIdx.x == 0 && threadIdx.x == 0) { p.status[2] = 0; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, 13); }
         return;
     }
-    // (the headers were complete before this kernel could start; everything else waits for the kernel before it)
-    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (blockIdx.x == 0 && threadIdx.x == 0) p.status[2] = 1;
 
     extern __shared__ uint8_t smem_raw[];
@@ -310,7 +310,7 @@ bool g4_attr_set[64] = {};
 // Launches the all-NVFP4 GEMM; it decides on the device (from the two headers) whether it applies and says so in
 // status[2], which the general path's kernels read.
 fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                                   int64_t M, int64_t N, int64_t K, int* status, cudaStream_t s)
+                                   int64_t M, int64_t N, int64_t K, int* status, bool sole, cudaStream_t s)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
@@ -332,7 +332,7 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     Gemm4Params p;
     p.ablob = (const uint8_t*)packed_acts; p.wblob = (const uint8_t*)packed_weights;
     p.LA = fgmp_layout(M, K, 0, 0); p.LW = fgmp_layout(N, K, 1, 0);
-    p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K; p.status = status;
+    p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K; p.status = status; p.sole = sole ? 1 : 0;
     // the activations' code plane: bytes [M, K/2] row-major, boxes of 128 rows x 128 bytes, swizzled on the way in
     CUtensorMap tmA;
     cuuint64_t dims[2] = {(cuuint64_t)(K / 2), (cuuint64_t)M};

@@ -79,7 +79,7 @@ long long g_prof_count[FGMP_K_COUNT];
 std::vector<ProfRec> g_prof_recs;
 std::vector<cudaEvent_t> g_event_pool;
 const char* const g_kernel_names[FGMP_K_COUNT] = {
-    "quant_act", "act_aux", "unpack", "expand_acts", "expand_weights", "gemm_bf16_tcgen05",
+    "quant_act", "act_aux", "unpack", "expand_acts", "expand_weights", "gemm_f16_tcgen05",
     "w_amax", "w_score_clip", "select", "w_mask", "scan", "w_emit", "w_aux", "act_scores", "decode_gemm", "gemm_nvfp4_tcgen05", "gemm_mixed_tcgen05", "gemm_reduce"};
 cudaEvent_t get_event()
 {

@@ -23,12 +23,18 @@ size_t fgmp_ws_decode(int64_t M, int64_t N, int64_t K);
 fgmp_status fgmp_linear_decode(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                                int64_t M, int64_t N, int64_t K, void* workspace, bool clear_first, cudaStream_t s);
 
-// all-NVFP4 prefill GEMM (fgmp_gemm4.cu): decides on the device whether it applies, answer in status[2]
+// all-NVFP4 prefill GEMM (fgmp_gemm4.cu): looks on the device whether it applies, and says so in status[2]; sole: nothing else
+// takes the call if it does not
 fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                                   int64_t M, int64_t N, int64_t K, int* status, cudaStream_t s);
+                                   int64_t M, int64_t N, int64_t K, int* status, bool sole, cudaStream_t s);
 
-// GEMM on the packed weights (fgmp_mixed.cu)
+// packed operands -> fp16 planes (planeW may be null: the activations only); cls_*: see fgmp_linear_classes
+fgmp_status fgmp_expand(const void* packed_acts, const void* packed_weights, int64_t M, int64_t N, int64_t K, uint8_t* planeA, uint8_t* planeW,
+                        int* status, int cls_a, int cls_w, bool leave_nvfp4, cudaStream_t s);
+
+// GEMM on the packed weights (fgmp_mixed.cu), and its modelled time
 struct QuantNext;
+double fgmp_mixed_us(int64_t M, int64_t N, int64_t K);
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K);
 fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                               int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, cudaStream_t s);
@@ -44,7 +50,7 @@ inline float fgmp_fp8_scale(const fgmp_scales& sc) { return sc.scale_fp8 > 0.f ?
 
 // ---- launch accounting (see fgmp_profile_begin in fgmp.h) ----
 enum FgmpKernelId {
-    FGMP_K_ACT_QUANT = 0, FGMP_K_ACT_AUX, FGMP_K_UNPACK, FGMP_K_EXPAND_A, FGMP_K_EXPAND_W, FGMP_K_GEMM_BF16,
+    FGMP_K_ACT_QUANT = 0, FGMP_K_ACT_AUX, FGMP_K_UNPACK, FGMP_K_EXPAND_A, FGMP_K_EXPAND_W, FGMP_K_GEMM_F16,
     FGMP_K_W_AMAX, FGMP_K_W_SCORE, FGMP_K_SELECT, FGMP_K_W_MASK, FGMP_K_SCAN, FGMP_K_W_EMIT, FGMP_K_W_AUX,
     FGMP_K_ACT_SCORES, FGMP_K_DECODE, FGMP_K_GEMM_NVFP4, FGMP_K_GEMM_MIXED, FGMP_K_GEMM_REDUCE, FGMP_K_COUNT
 };

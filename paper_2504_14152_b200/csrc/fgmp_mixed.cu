@@ -12,10 +12,11 @@
 //     the MMAs (16 of N/2 clocks for N tokens) bound from 128 tokens on, the dequantization below;
 //   - the operand from tensor memory leaves shared memory to the token tiles (from shared memory the 64 KiB of a
 //     dequantized unit would be written and read there, 1024 clocks by themselves);
-//   - L2 -> shared-memory traffic: one weight tile against a token tile of N needs N * 512 + 20 K bytes per 8 N clocks, 70
-//     bytes per clock at N = 208; two weight tiles (TS = 2) that share the token tile need 42.
+//   - a unit takes 1.08 us + 4.2 ns per token (MMAs alone 4.3 ns per token at 1.85 GHz): the dequantizing warps, whose step is a
+//     chain of shared-memory loads, conversions, a tensor-memory store and three barriers, and the MMA issuer share four
+//     schedulers.  CTA pairs that share a token tile (half the L2 traffic) were measured and are no faster.
 //
-// Work is (group of TS weight tiles, token tile, 256-element K chunk) units in that order, split over the CTAs either in
+// Work is (weight tile, token tile, 256-element K chunk) units in that order, split over the CTAs either in
 // equal contiguous spans (stream-K: the partial sums of tiles shared by several CTAs are stored column by column and added
 // up in CTA order by a kernel of their own, which has the whole chip's loads in flight: 43 MB at 203 tokens and 13824 weight
 // rows, 20 us if the CTA that arrives last does it) or in whole tiles, whichever the model in mixed_plan says is faster.
@@ -30,13 +31,13 @@
 #include "fgmp_host.h"
 #include "fgmp_ptx.cuh"
 #include "fgmp_quantnext.cuh"
+#include "fgmp_deq.cuh"
 
 namespace {
 
 constexpr int W_PROD = 0, W_MMA = 1, W_TOK = 2, W_EPI = 3, W_DEQ = 7;
-// dequantization groups: as many as the registers of a thread allow (quantizing in the epilogue takes more of them)
-constexpr int mx_groups(bool quant) { return quant ? 3 : 4; }
-constexpr int mx_threads(bool quant) { return 32 * (W_DEQ + 4 * mx_groups(quant)); }
+constexpr int MX_GROUPS = 3;                    // dequantization groups (four are no faster, two 10 % slower)
+constexpr int MX_THREADS = 32 * (W_DEQ + 4 * MX_GROUPS);
 constexpr uint32_t STG_MASK = REC_BYTES, STG_HALF = STG_MASK + 256;      // a weight stage: record, mask, second halves of the FP8 blocks
 constexpr uint32_t HALF_CAP = 5248;             // 656 FP8 blocks (32 %); with more the halves are read from global memory
 constexpr uint32_t WSTAGE = STG_HALF + HALF_CAP;                         // 24064
@@ -44,15 +45,14 @@ constexpr int MAX_WSTAGES = 4, MAX_BSTAGES = 12, MAX_SLOTS = 8;
 constexpr uint32_t MX_TMEM_COLS = 512;
 constexpr size_t MX_SMEM_LIMIT = 232448;
 constexpr uint32_t SW128_LO = 1u << 16, SW128_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
-constexpr uint32_t IDESC_F16 = (1u << 4) | ((uint32_t)(128 >> 4) << 24);          // f32 += f16 x f16, M = 128, K-major; N added at run time
+constexpr uint32_t IDESC_F16 = 1u << 4;         // f32 += f16 x f16, K-major; M and N added
 
 struct MixedPlan {
-    int ts;                              // weight tiles per unit
-    uint32_t n_tok, tok_tiles, groups;   // tokens per tile (multiple of 16), token tiles, groups of ts weight tiles
-    uint32_t chunks, tiles;              // tiles = groups * tok_tiles
+    uint32_t n_tok, tok_tiles;           // tokens per tile (multiple of 16), token tiles
+    uint32_t chunks, tiles;              // tiles = wtiles * tok_tiles
     uint32_t grid, span, rest, quantum;  // a CTA's span in quanta of `quantum` units (1, or chunks: whole tiles)
-    uint32_t wstages, bstages, slots, max_parts;
-    double cost;                         // modelled clocks
+    uint32_t wstages, bstages, slots, naccs, max_parts;
+    double us;                           // modelled time
 };
 
 struct MixedParams {
@@ -79,67 +79,11 @@ __device__ __forceinline__ void umma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ uint32_t hmul2(uint32_t a, uint32_t b)
-{
-    uint32_t r;
-    asm("mul.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
-    return r;
-}
-__device__ __forceinline__ uint32_t e4m3x2_to_f16x2(uint32_t two)
-{
-    uint32_t r;
-    asm("cvt.rn.f16x2.e4m3x2 %0, %1;" : "=r"(r) : "h"((uint16_t)two));
-    return r;
-}
-// eight E2M1 codes -> four pairs (all four bytes unpacked at once: byte by byte it takes 1.7 times as long)
-__device__ __forceinline__ void e2m1x8_to_f16(uint32_t w, uint32_t* r)
-{
-    asm("{\n\t.reg .b8 a, b, c, d;\n\tmov.b32 {a, b, c, d}, %4;\n\tcvt.rn.f16x2.e2m1x2 %0, a;\n\tcvt.rn.f16x2.e2m1x2 %1, b;\n\t"
-        "cvt.rn.f16x2.e2m1x2 %2, c;\n\tcvt.rn.f16x2.e2m1x2 %3, d;\n\t}" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(w));
-}
-
 __device__ __forceinline__ uint32_t unit_begin(const MixedPlan& pl, uint32_t cta) { return (cta * pl.span + min(cta, pl.rest)) * pl.quantum; }
 __device__ __forceinline__ uint32_t cta_of(const MixedPlan& pl, uint32_t u)
 {
     const uint32_t i = u / pl.quantum, longer = pl.rest * (pl.span + 1);
     return i < longer ? i / (pl.span + 1) : pl.rest + (i - longer) / pl.span;
-}
-
-// packed activations -> fp16 plane [M, K] of values over the tensor scale; one thread per block
-__global__ void __launch_bounds__(256) expand_f16_kernel(const uint8_t* blob, const uint8_t* wblob, int64_t rows, int64_t K, uint8_t* plane, int* status, int leave_nvfp4)
-{
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(blob);
-    if (!(h->magic == FGMP_MAGIC && h->version == FGMP_LAYOUT_VERSION && h->rows == rows && h->K == K && h->kind == 0u && h->fp8_scale_free == 0)) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) { atomicCAS(status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(status + 1, 11); }
-        return;
-    }
-    // operands without any FP8 block are multiplied as they are packed
-    if (leave_nvfp4 && h->n_fp8 == 0 && reinterpret_cast<const fgmp_packed_header*>(wblob)->n_fp8 == 0) return;
-    const PackedLayout L = fgmp_layout(rows, K, 0, 0);
-    const uint32_t* pmask = reinterpret_cast<const uint32_t*>(blob + L.off_mask);
-    const __half2 r8 = __float2half2_rn(__int_as_float((127 + h->fp8_log2_ratio) << 23));
-    const uint32_t f8 = *reinterpret_cast<const uint32_t*>(&r8);
-    const int64_t nblk = rows * L.KB;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nblk; b += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = b / L.KB, kb = b - r * L.KB;
-        uint32_t o[8];
-        if ((pmask[r * L.MW + (kb >> 5)] >> (kb & 31)) & 1u) {
-            const uint4 c = *reinterpret_cast<const uint4*>(blob + L.off_codes8 + (size_t)(r * K + kb * 16));
-            const uint32_t w[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { o[2 * i] = hmul2(e4m3x2_to_f16x2(w[i] & 0xffffu), f8); o[2 * i + 1] = hmul2(e4m3x2_to_f16x2(w[i] >> 16), f8); }
-        } else {
-            const uint2 c = *reinterpret_cast<const uint2*>(blob + L.off_codes4 + (r * K) / 2 + kb * 8);
-            const uint32_t sc = blob[L.off_sf + fgmp_sf_offset(r, kb, K)], d = e4m3x2_to_f16x2(sc | (sc << 8));
-            e2m1x8_to_f16(c.x, o); e2m1x8_to_f16(c.y, o + 4);
-#pragma unroll
-            for (int i = 0; i < 8; ++i) o[i] = hmul2(o[i], d);
-        }
-        asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                     ::"l"(plane + (size_t)(r * K + kb * 16) * 2), "r"(o[0]), "r"(o[1]), "r"(o[2]), "r"(o[3]), "r"(o[4]), "r"(o[5]), "r"(o[6]), "r"(o[7]) : "memory");
-    }
 }
 
 // 32 consecutive values of a row of the result = two blocks of the next layer's activations
@@ -185,7 +129,7 @@ __device__ __forceinline__ void mixed_emit(const MixedParams& p, const uint32_t 
 }
 
 // Epilogue warps: tensor-memory lane quadrant warp % 4, lane = weight row, column = token
-template <int TS, bool QUANT>
+template <bool QUANT>
 __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tmem_base, int warp, int lane, uint32_t u_begin, uint32_t u_end,
                                                uint32_t accf0, uint32_t acce0, volatile int* abort_flag, int t_w, float* extra)
 {
@@ -194,45 +138,36 @@ __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tm
     const float alpha = __fmul_rn(__fmul_rn(p.ha->scale_fp4, __ldg(&reinterpret_cast<const fgmp_packed_header*>(p.wblob)->scale_fp4)),
                                   __int_as_float((127 + t_w) << 23));
     uint32_t* turn = reinterpret_cast<uint32_t*>(extra) + q * 32 * 33;
-    uint32_t acc_phase = 0;
-    bool ok = true;
-    for (uint32_t u = u_begin; u < u_end && ok;) {
+    uint32_t acc = 0, acc_phase = 0;
+    for (uint32_t u = u_begin; u < u_end;) {
         const uint32_t tile = u / C, t_begin = tile * C, t_end = t_begin + C, seg_end = min(t_end, u_end);
         const bool whole = u == t_begin && seg_end == t_end;
-        const uint32_t g = tile / pl.tok_tiles;
-        const int64_t m0 = (int64_t)(tile % pl.tok_tiles) * NT;
-        const uint32_t which = u == u_begin ? 0u : 1u;       // a CTA's first segment, or its last
+        const uint32_t wt = tile / pl.tok_tiles, which = u == u_begin ? 0u : 1u;       // a span's first segment, or its last
+        const int64_t m0 = (int64_t)(tile % pl.tok_tiles) * NT, n = (int64_t)wt * 128 + row;
         u = seg_end;
+        if (!mbar_wait_warp(accf0 + 8 * acc, acc_phase, abort_flag, p.status, 8)) break;
+        tc_fence_after();
+        const uint32_t d = tmem_base + ((q * 32u) << 16) + acc * NT;
+        float* mine = p.parts + ((size_t)(blockIdx.x * 2 + which)) * NP * 128 + row;
 #pragma unroll 1
-        for (int t = 0; t < TS; ++t) {
-            const uint32_t wt = g * TS + t;
-            const int64_t n = (int64_t)wt * 128 + row;
-            if (!(ok = mbar_wait_warp(accf0 + 8 * t, acc_phase, abort_flag, p.status, 8))) break;
-            tc_fence_after();
-            const uint32_t d = tmem_base + ((q * 32u) << 16) + t * NT;
-            const bool there = wt < (uint32_t)p.LW.tiles;
-            float* mine = p.parts + ((size_t)(blockIdx.x * 2 + which) * TS + t) * NP * 128 + row;
-            if (there)
-#pragma unroll 1
-                for (uint32_t cc = 0; cc < NT; cc += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(d + cc, v);
-                    if (whole) mixed_emit<QUANT>(p, v, n, m0, cc, alpha, lane, turn);
-                    else
+        for (uint32_t cc = 0; cc < NT; cc += 32) {
+                uint32_t v[32];
+                tmem_ld32(d + cc, v);
+                if (whole) mixed_emit<QUANT>(p, v, n, m0, cc, alpha, lane, turn);
+                else
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) __stcg(mine + (cc + j) * 128, __uint_as_float(v[j]));
-                }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acce0 + 8 * t);
-        }
-        acc_phase ^= 1u;
+                    for (int j = 0; j < 32; ++j) __stcg(mine + (cc + j) * 128, __uint_as_float(v[j]));
+            }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(acce0 + 8 * acc);
+        if (++acc == pl.naccs) { acc = 0; acc_phase ^= 1u; }
     }
 }
 
-// TS = weight tiles per unit.  QUANT: the next layer's activation quantizer in the epilogue instead of Y.
-template <int TS, bool QUANT>
-__global__ void __launch_bounds__(mx_threads(QUANT), 1)
+// QUANT: the next layer's activation quantizer in the epilogue instead of Y.
+template <bool QUANT>
+__global__ void __launch_bounds__(MX_THREADS, 1)
 mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ MixedParams p)
 {
     extern __shared__ uint8_t smem_raw[];
@@ -240,30 +175,35 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     const MixedPlan& pl = p.pl;
     const uint32_t BS = pl.bstages, WS = pl.wstages, R = pl.slots, NT = pl.n_tok, C = pl.chunks;
     // (no more groups than slots: a group that was further ahead could take an older phase of a slot's barrier for the one it waits for)
-    const uint32_t NG = min((uint32_t)mx_groups(QUANT), R);
-    const uint32_t b_bytes = NT * 128u;                  // token stage: NT rows x 64 elements, swizzled (a multiple of 2 KiB)
+    const uint32_t NG = min((uint32_t)MX_GROUPS, R);
+    const uint32_t b_bytes = NT * 128u;                 // token stage: NT rows x 64 elements, swizzled (a multiple of 2 KiB)
     uint8_t* wst0 = smem + BS * b_bytes;
-    uint8_t* extra = wst0 + WS * TS * WSTAGE;            // QUANT: 4 x 32 x 33 floats
+    uint8_t* extra = wst0 + WS * WSTAGE;                 // QUANT: 4 x 32 x 33 floats
     uint64_t* bars = reinterpret_cast<uint64_t*>(extra + (QUANT ? 4 * 32 * 33 * 4 + 128 : 0));
-    uint32_t* wmeta = reinterpret_cast<uint32_t*>(bars + 2 * MAX_WSTAGES + 2 * MAX_BSTAGES + 2 * MAX_SLOTS + 4);   // [stage][tile]: list start, steps
-    uint32_t* tmem_slot = wmeta + MAX_WSTAGES * TS * 2;
+    uint32_t* wmeta = reinterpret_cast<uint32_t*>(bars + 2 * MAX_WSTAGES + 2 * MAX_BSTAGES + MAX_SLOTS + 4);   // per stage: list start, bytes of it there
+    uint32_t* tmem_slot = wmeta + MAX_WSTAGES * 2;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
-    // barriers: weight stage full / empty, token stage full / empty, dequantized step in tensor memory full / empty,
-    // accumulators full / empty (one per weight tile)
-    const uint32_t wf0 = smem_u32(bars), we0 = wf0 + 8 * MAX_WSTAGES, bf0 = we0 + 8 * MAX_WSTAGES, be0 = bf0 + 8 * MAX_BSTAGES;
-    const uint32_t sf0 = be0 + 8 * MAX_BSTAGES, se0 = sf0 + 8 * MAX_SLOTS, accf0 = se0 + 8 * MAX_SLOTS, acce0 = accf0 + 16;
-    const uint32_t slot_col = TS * NT;                   // tensor memory: TS accumulators of NT columns, then slots of 32
+    // The MMA issuer is a single thread whose every wait (75 clocks) and commit (40) comes on top of 40 clocks per MMA, so it has
+    // one of each per step of 64 elements: step i is ready (barrier i % R) when the dequantized weights are in tensor
+    // memory and the warps that put them there have seen the token tile of the step; when it is done (barrier i % L, L the
+    // longer of the two rings), both its slot and its token stage are free.
+    // barriers: weight stage full / empty, token stage full; step ready, step done; accumulators full / empty
+    const uint32_t wf0 = smem_u32(bars), we0 = wf0 + 8 * MAX_WSTAGES, bf0 = we0 + 8 * MAX_WSTAGES, dn0 = bf0 + 8 * MAX_BSTAGES;
+    const uint32_t sf0 = dn0 + 8 * MAX_BSTAGES, accf0 = sf0 + 8 * MAX_SLOTS, acce0 = accf0 + 16;
+    const uint32_t L = max(R, BS);
+    const uint32_t slot_col = pl.naccs * NT;             // tensor memory: accumulators of NT columns, then slots of 32
 
     const uint32_t u_begin = unit_begin(pl, blockIdx.x), u_end = unit_begin(pl, blockIdx.x + 1);
-    const uint32_t wtiles = (uint32_t)p.LW.tiles, last_steps = (uint32_t)(p.K / 64) - 4u * (C - 1u);
+    const uint32_t last_steps = (uint32_t)(p.K / 64) - 4u * (C - 1u);
 
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < WS; ++s) { mbar_init(wf0 + 8 * s, 1); mbar_init(we0 + 8 * s, 4 * NG); }
-        for (uint32_t s = 0; s < BS; ++s) { mbar_init(bf0 + 8 * s, 1); mbar_init(be0 + 8 * s, 1); }
-        for (uint32_t s = 0; s < R; ++s) { mbar_init(sf0 + 8 * s, 4); mbar_init(se0 + 8 * s, 1); }
-        for (int t = 0; t < TS; ++t) { mbar_init(accf0 + 8 * t, 1); mbar_init(acce0 + 8 * t, 4); }
+        for (uint32_t s = 0; s < BS; ++s) mbar_init(bf0 + 8 * s, 1);
+        for (uint32_t s = 0; s < L; ++s) mbar_init(dn0 + 8 * s, 1);
+        for (uint32_t s = 0; s < R; ++s) mbar_init(sf0 + 8 * s, 4);
+        for (uint32_t t = 0; t < pl.naccs; ++t) { mbar_init(accf0 + 8 * t, 1); mbar_init(acce0 + 8 * t, 4); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -271,14 +211,14 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+    const uint32_t tmem_base = TMEM_ALL;
     const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
     const int ratio_w = __ldg(&hw->fp8_log2_ratio);
     // The weights go in over 2^t: an FP8 block needs no factor then if t is the ratio of its tensor scale to the NVFP4 one,
     // and fp16 holds every NVFP4 value (up to 2688) over 2^t as long as t >= -4.
     const int t_w = max(ratio_w, -4);
-
     const bool has_fp8 = __ldg(&hw->n_fp8) != 0, may_skip = p.leave_nvfp4 && !has_fp8;
+
     if (warp == W_PROD) {
         // ------------------------------------------------------------ weights producer (whole warp; lane 0 issues)
         // The packed weights are not written by whatever runs before this kernel: their first copies overlap its end.
@@ -294,35 +234,26 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
             if (p.ha->n_fp8 == 0) ok = 0;
         }
         for (uint32_t u = u_begin; u < u_end && ok; ++u, ++issued) {
-            const uint32_t c = u % C, g = u / C / pl.tok_tiles;
-            // lane t of the first TS: the list of weight tile t's unit
-            const uint32_t tile = g * TS + lane, rec = tile * C + c;
-            uint32_t st0 = 0, st1 = 0;
-            if (lane < TS && tile < wtiles) { st0 = __ldg(uptr + rec); st1 = __ldg(uptr + rec + 1); }
+            const uint32_t c = u % C, tile = u / C / pl.tok_tiles, rec = tile * C + c;
             if (issued == WS && !waited) {
                 // the status word may be looked at once the preceding kernel is done
                 asm volatile("griddepcontrol.wait;" ::: "memory");
                 waited = true;
             }
-            if (lane == 0) ok = mbar_wait(we0 + 8 * stage, phase, abort_flag, p.status, 1) ? 1 : 0;
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) break;
-            const uint32_t steps = st1 - st0, h = 2u * steps / 3u, staged = min(h * 16u, HALF_CAP);     // the list's words, then h steps of halves
-            const bool there = lane < TS && tile < wtiles;
-            const uint32_t mine = there ? REC_BYTES + 256u + staged : 0u;
-            uint32_t all = mine;
-            if (TS == 2) all += __shfl_down_sync(0xffffffffu, mine, 1);
-            if (there) { wmeta[(stage * TS + lane) * 2] = st0 + (steps - h); wmeta[(stage * TS + lane) * 2 + 1] = staged; }
-            __syncwarp();
-            if (lane == 0) mbar_expect_tx(wf0 + 8 * stage, all);
-            __syncwarp();
-            if (there) {
-                const uint32_t dst = smem_u32(wst0 + (stage * TS + lane) * WSTAGE), fb = wf0 + 8 * stage;
-                bulk_load(dst, p.wblob + p.LW.off_rec + (size_t)rec * REC_BYTES, REC_BYTES, fb);
-                bulk_load(dst + STG_MASK, p.wblob + p.LW.off_mask + (size_t)rec * 256, 256u, fb);
-                if (staged) bulk_load(dst + STG_HALF, p.wblob + p.LW.off_ovf + (size_t)(st0 + (steps - h)) * 16, staged, fb);
+            if (lane == 0) {
+                const uint32_t st0 = __ldg(uptr + rec), st1 = __ldg(uptr + rec + 1);
+                ok = mbar_wait(we0 + 8 * stage, phase, abort_flag, p.status, 1) ? 1 : 0;
+                if (ok) {
+                    const uint32_t steps = st1 - st0, h = 2u * steps / 3u, staged = min(h * 16u, HALF_CAP);     // the list's words, then h steps of halves
+                    const uint32_t dst = smem_u32(wst0 + stage * WSTAGE), fb = wf0 + 8 * stage;
+                    wmeta[stage * 2] = st0 + (steps - h); wmeta[stage * 2 + 1] = staged;
+                    mbar_expect_tx(fb, REC_BYTES + 256u + staged);
+                    bulk_load(dst, p.wblob + p.LW.off_rec + (size_t)rec * REC_BYTES, REC_BYTES, fb);
+                    bulk_load(dst + STG_MASK, p.wblob + p.LW.off_mask + (size_t)rec * 256, 256u, fb);
+                    if (staged) bulk_load(dst + STG_HALF, p.wblob + p.LW.off_ovf + (size_t)(st0 + (steps - h)) * 16, staged, fb);
+                }
             }
-            __syncwarp();
+            ok = __shfl_sync(0xffffffffu, ok, 0);
             if (++stage == WS) { stage = 0; phase ^= 1; }
         }
         if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -344,150 +275,158 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     } else if (warp == W_TOK) {
         // ------------------------------------------------------------ token-tile producer
         if (lane == 0) {
-            uint32_t stage = 0, phase = 1;
+            uint32_t stage = 0, ds = 0, dph = 0, i = 0;  // ds: barrier of step i - BS
             bool ok = true;
             for (uint32_t u = u_begin; u < u_end && ok; ++u) {
                 const uint32_t c = u % C, m0 = (u / C) % pl.tok_tiles * NT, steps = c == C - 1 ? last_steps : 4u;
-                for (uint32_t s = 0; s < steps; ++s) {
-                    if (!(ok = mbar_wait(be0 + 8 * stage, phase, abort_flag, p.status, 2))) break;
+                for (uint32_t s = 0; s < steps; ++s, ++i) {
+                    if (i >= BS) {
+                        if (!(ok = mbar_wait(dn0 + 8 * ds, dph, abort_flag, p.status, 2))) break;
+                        if (++ds == L) { ds = 0; dph ^= 1; }
+                    }
                     mbar_expect_tx(bf0 + 8 * stage, b_bytes);
                     tma_load_2d(smem_u32(smem + stage * b_bytes), &tmB, (int32_t)(c * 256 + s * 64), (int32_t)m0, bf0 + 8 * stage);
-                    if (++stage == BS) { stage = 0; phase ^= 1; }
+                    if (++stage == BS) stage = 0;
                 }
             }
         }
         __syncwarp();
     } else if (warp == W_MMA) {
         // ------------------------------------------------------------ MMA issuer (one elected lane)
-        const uint32_t idesc = IDESC_F16 | ((NT >> 3) << 17), b_first = (smem_u32(smem) >> 4) | SW128_LO, b_step = b_bytes >> 4;
-        uint32_t bst = 0, bph = 0, slot = 0, sph = 0, c = u_begin % C, acc_phase = 1, b_lo = b_first;
-        bool first = true, ok = true;
-        for (uint32_t u = u_begin; u < u_end && ok; ++u) {
-            const uint32_t steps = c == C - 1 ? last_steps : 4u;
-            const bool last_unit = c == C - 1 || u + 1 == u_end;
-            for (uint32_t s = 0; s < steps && ok; ++s) {
-                if (!(ok = mbar_wait_uniform(bf0 + 8 * bst, bph, abort_flag, p.status, 3))) break;
-#pragma unroll
-                for (int t = 0; t < TS; ++t) {
-                    if (first && !(ok = mbar_wait_uniform(acce0 + 8 * t, acc_phase, abort_flag, p.status, 4))) break;
-                    if (!(ok = mbar_wait_uniform(sf0 + 8 * slot, sph, abort_flag, p.status, 5))) break;
+        {
+            const uint32_t idesc = IDESC_F16 | ((NT >> 3) << 17) | ((128u >> 4) << 24), b_first = (smem_u32(smem) >> 4) | SW128_LO, b_step = b_bytes >> 4;
+            uint32_t bst = 0, slot = 0, sph = 0, ds = 0, c = u_begin % C, acc = 0, acc_phase = 1, accum = 0, b_lo = b_first;
+            bool ok = true, ready = false;
+            for (uint32_t u = u_begin; u < u_end && ok; ++u) {
+                const uint32_t steps = c == C - 1 ? last_steps : 4u, d = tmem_base + acc * NT;
+                const bool last_unit = c == C - 1 || u + 1 == u_end;
+                if (accum == 0 && !mbar_wait_uniform(acce0 + 8 * acc, acc_phase, abort_flag, p.status, 4)) break;
+                for (uint32_t s = 0; s < steps; ++s) {
+                    if (!ready && !(ok = mbar_wait_uniform(sf0 + 8 * slot, sph, abort_flag, p.status, 5))) break;
                     tc_fence_after();
-                    const uint32_t d = tmem_base + t * NT, a = tmem_base + slot_col + slot * 32;
+                    const uint32_t a = tmem_base + slot_col + slot * 32;
+                    if (++slot == R) { slot = 0; sph ^= 1; }
+                    const bool peek = mbar_test_wait(sf0 + 8 * slot, sph);      // the next step's; the answer comes while this one's MMAs are issued
                     if (elect_one()) {
 #pragma unroll
-                        for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d, a + 8 * k, mx_desc(b_lo + 2 * k), idesc, k ? 1u : (first ? 0u : 1u));
-                        umma_commit(se0 + 8 * slot);
-                        if (last_unit && s + 1 == steps) umma_commit(accf0 + 8 * t);
-                        if (t == TS - 1) umma_commit(be0 + 8 * bst);
+                        for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d, a + 8 * k, mx_desc(b_lo + 2 * k), idesc, k ? 1u : accum);
+                        umma_commit(dn0 + 8 * ds);
                     }
-                    __syncwarp();
-                    if (++slot == R) { slot = 0; sph ^= 1; }
+                    accum = 1;
+                    b_lo += b_step;
+                    if (++bst == BS) { bst = 0; b_lo = b_first; }
+                    if (++ds == L) ds = 0;
+                    ready = __all_sync(0xffffffffu, peek);
                 }
-                first = false;
-                b_lo += b_step;
-                if (++bst == BS) { bst = 0; bph ^= 1; b_lo = b_first; }
+                if (last_unit) {
+                    if (elect_one()) umma_commit(accf0 + 8 * acc);
+                    __syncwarp();
+                    accum = 0;
+                    if (++acc == pl.naccs) { acc = 0; acc_phase ^= 1; }
+                }
+                if (++c == C) c = 0;
             }
-            if (last_unit) { first = true; acc_phase ^= 1; }
-            if (++c == C) c = 0;
         }
+        __syncwarp();
     } else if (warp >= W_DEQ + 4 * (int)NG) {
     } else if (warp >= W_DEQ) {
         // ------------------------------------------------------------ dequantization: thread = row of the weight tile
-        // The groups take the steps in turn: step a of a unit is elements 64 (a / TS) .. of weight tile a % TS.
+        // The groups take the steps of 64 elements in turn.
         const uint32_t group = (uint32_t)(warp - W_DEQ) >> 2, row = 32u * (warp & 3) + lane, r7 = row & 7u;
         const uint32_t quadrant = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + slot_col;
         const __half2 inv2 = __float2half2_rn(__int_as_float((127 - t_w) << 23)), f82 = __float2half2_rn(__int_as_float((127 + ratio_w - t_w) << 23));
         const uint32_t inv = *reinterpret_cast<const uint32_t*>(&inv2), f8 = *reinterpret_cast<const uint32_t*>(&f82);
         const bool scaled8 = ratio_w != t_w;             // (for every thread alike)
-        uint32_t stage = 0, phase = 0, c = u_begin % C, slot = group % R, sph = group / R & 1u ? 0u : 1u, next = group;    // next: steps until the group's turn
+        uint32_t stage = 0, phase = 0, c = u_begin % C, slot = group, next = group;    // next: steps until the group's turn
+        uint32_t bst = group, bph = 0, ds = 0, dph = 0, i = group;        // i: the step; ds: barrier of step i - R
+        while (bst >= BS) { bst -= BS; bph ^= 1; }
         bool ok = true;
         for (uint32_t u = u_begin; u < u_end && ok; ++u) {
-            const uint32_t steps = (c == C - 1 ? last_steps : 4u) * TS;
+            const uint32_t steps = c == C - 1 ? last_steps : 4u;
             if (!(ok = mbar_wait_warp(wf0 + 8 * stage, phase, abort_flag, p.status, 6))) break;
-            const bool pair = TS == 2 && (u / C / pl.tok_tiles) * TS + 1 < wtiles;     // an odd number of weight tiles: the last group has one
-            uint32_t m16s[TS], ats[TS], alls = 0;
-#pragma unroll
-            for (int t = 0; t < TS; ++t) {
+            const uint8_t* sp = wst0 + stage * WSTAGE;
+            uint32_t mt = 0, at = 0;
+            bool all = true;
+            if (has_fp8) {
                 // the row's FP8 blocks lie one after the other in the list
-                m16s[t] = 0; ats[t] = 0;
-                if (has_fp8 && (t == 0 || pair)) {
-                    const uint8_t* sb = wst0 + (stage * TS + t) * WSTAGE;
-                    const uint16_t* before = reinterpret_cast<const uint16_t*>(sb + REC_KBSTART);
-                    m16s[t] = reinterpret_cast<const uint16_t*>(sb + STG_MASK)[row];
-                    uint32_t at = __popc(m16s[t]);
+                const uint16_t* before = reinterpret_cast<const uint16_t*>(sp + REC_KBSTART);
+                mt = reinterpret_cast<const uint16_t*>(sp + STG_MASK)[row];
+                at = __popc(mt);
 #pragma unroll
-                    for (int o = 1; o < 8; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, at, o, 8); if ((lane & 7) >= o) at += y; }
-                    ats[t] = 8u * (before[row >> 3] + at - __popc(m16s[t]));
-                    if (8u * before[16] <= wmeta[(stage * TS + t) * 2 + 1]) alls |= 1u << t;
-                }
+                for (int o = 1; o < 8; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, at, o, 8); if ((lane & 7) >= o) at += y; }
+                at = 8u * (before[row >> 3] + at - __popc(mt));
+                all = 8u * before[16] <= wmeta[stage * 2 + 1];
             }
 #pragma unroll 1
             for (; next < steps; next += NG) {
-                const uint32_t t = next % TS, s = next / TS;
+                const uint32_t s = next;
                 uint32_t r[32];
-                if (t == 0 || pair) {
-                    const uint32_t sb = smem_u32(wst0 + (stage * TS + t) * WSTAGE), codes = sb + row * 128u, sfw = sb + REC_SF + (row & 31u) * 16u + (row >> 5) * 4u;
-                    const uint32_t mt = TS == 2 && t ? m16s[TS - 1] : m16s[0], m16 = mt >> (4 * s);
-                    const bool all = (alls >> t) & 1u;
-                    uint32_t hg = (TS == 2 && t ? ats[TS - 1] : ats[0]) + 8u * __popc(mt & ((1u << (4 * s)) - 1u)), hs = sb + STG_HALF + hg;
-                    uint4 q0, q1;
-                    uint32_t sc;
-                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q0.x), "=r"(q0.y), "=r"(q0.z), "=r"(q0.w) : "r"(codes + (((2 * s) ^ r7) << 4)));
-                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q1.x), "=r"(q1.y), "=r"(q1.z), "=r"(q1.w) : "r"(codes + (((2 * s + 1) ^ r7) << 4)));
-                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(sc) : "r"(sfw + 512u * s));
-                    const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-                    uint2 hi[4];
+                const uint32_t sb = smem_u32(sp), codes = sb + row * 128u, sfw = sb + REC_SF + (row & 31u) * 16u + (row >> 5) * 4u;
+                const uint32_t m16 = mt >> (4 * s);
+                uint32_t hg = at + 8u * __popc(mt & ((1u << (4 * s)) - 1u)), hs = sb + STG_HALF + hg;
+                uint4 q0, q1;
+                uint32_t sc;
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q0.x), "=r"(q0.y), "=r"(q0.z), "=r"(q0.w) : "r"(codes + (((2 * s) ^ r7) << 4)));
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q1.x), "=r"(q1.y), "=r"(q1.z), "=r"(q1.w) : "r"(codes + (((2 * s + 1) ^ r7) << 4)));
+                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(sc) : "r"(sfw + 512u * s));
+                const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+                uint2 hi[4];
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k) {
+                    const uint32_t is8 = (m16 >> k) & 1u;
+                    hi[k] = lds64_if(hs, is8 && all);
+                    hs += 8u * is8;
+                }
+                if (!all) {
+                    const uint8_t* half_g = p.wblob + p.LW.off_ovf + (size_t)wmeta[stage * 2] * 16;
+#pragma unroll
+                    for (uint32_t k = 0; k < 4; ++k)
+                        if ((m16 >> k) & 1u) { hi[k] = __ldg(reinterpret_cast<const uint2*>(half_g + hg)); hg += 8u; }
+                    __syncwarp();
+                }
+                const uint32_t d01 = hmul2(e4m3x2_to_f16x2(sc & 0xffffu), inv), d23 = hmul2(e4m3x2_to_f16x2(sc >> 16), inv);
+                const uint32_t d[4] = {__byte_perm(d01, 0, 0x1010), __byte_perm(d01, 0, 0x3232), __byte_perm(d23, 0, 0x1010), __byte_perm(d23, 0, 0x3232)};
+#pragma unroll
+                for (uint32_t k = 0; k < 4; ++k) {
+                    e2m1x8_to_f16(w[2 * k], r + 8 * k); e2m1x8_to_f16(w[2 * k + 1], r + 8 * k + 4);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) r[8 * k + e] = hmul2(r[8 * k + e], d[k]);
+                }
+                if (has_fp8) {
+                    // E4M3 codes 0..7 in the slot, 8..15 in the list; selected, not branched to: with 10 % FP8 blocks some
+                    // row of a warp has one in nearly every column
 #pragma unroll
                     for (uint32_t k = 0; k < 4; ++k) {
-                        const uint32_t is8 = (m16 >> k) & 1u;
-                        hi[k] = lds64_if(hs, is8 && all);
-                        hs += 8u * is8;
-                    }
-                    if (!all) {
-                        const uint8_t* half_g = p.wblob + p.LW.off_ovf + (size_t)wmeta[(stage * TS + t) * 2] * 16;
+                        const bool is8 = (m16 >> k) & 1u;
+                        const uint32_t v[4] = {w[2 * k], w[2 * k + 1], hi[k].x, hi[k].y};
 #pragma unroll
-                        for (uint32_t k = 0; k < 4; ++k)
-                            if ((m16 >> k) & 1u) { hi[k] = __ldg(reinterpret_cast<const uint2*>(half_g + hg)); hg += 8u; }
-                        __syncwarp();
-                    }
-                    const uint32_t d01 = hmul2(e4m3x2_to_f16x2(sc & 0xffffu), inv), d23 = hmul2(e4m3x2_to_f16x2(sc >> 16), inv);
-                    const uint32_t d[4] = {__byte_perm(d01, 0, 0x1010), __byte_perm(d01, 0, 0x3232), __byte_perm(d23, 0, 0x1010), __byte_perm(d23, 0, 0x3232)};
-#pragma unroll
-                    for (uint32_t k = 0; k < 4; ++k) {
-                        e2m1x8_to_f16(w[2 * k], r + 8 * k); e2m1x8_to_f16(w[2 * k + 1], r + 8 * k + 4);
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) r[8 * k + e] = hmul2(r[8 * k + e], d[k]);
-                    }
-                    if (has_fp8) {
-                        // E4M3 codes 0..7 in the slot, 8..15 in the list; selected, not branched to: with 10 % FP8 blocks some
-                        // row of a warp has one in nearly every column
-#pragma unroll
-                        for (uint32_t k = 0; k < 4; ++k) {
-                            const bool is8 = (m16 >> k) & 1u;
-                            const uint32_t v[4] = {w[2 * k], w[2 * k + 1], hi[k].x, hi[k].y};
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                uint32_t a = e4m3x2_to_f16x2(v[e] & 0xffffu), b = e4m3x2_to_f16x2(v[e] >> 16);
-                                if (scaled8) { a = hmul2(a, f8); b = hmul2(b, f8); }
-                                r[8 * k + 2 * e] = is8 ? a : r[8 * k + 2 * e];
-                                r[8 * k + 2 * e + 1] = is8 ? b : r[8 * k + 2 * e + 1];
-                            }
+                        for (int e = 0; e < 4; ++e) {
+                            uint32_t a = e4m3x2_to_f16x2(v[e] & 0xffffu), b = e4m3x2_to_f16x2(v[e] >> 16);
+                            if (scaled8) { a = hmul2(a, f8); b = hmul2(b, f8); }
+                            r[8 * k + 2 * e] = is8 ? a : r[8 * k + 2 * e];
+                            r[8 * k + 2 * e + 1] = is8 ? b : r[8 * k + 2 * e + 1];
                         }
                     }
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; ++e) r[e] = 0;
                 }
                 __syncwarp();
-                if (!(ok = mbar_wait_warp(se0 + 8 * slot, sph, abort_flag, p.status, 7))) break;
-                tc_fence_after();
+                if (i >= R) {
+                    if (i < R + NG) ds = (i - R) % L;              // the group's first wait
+                    if (!(ok = mbar_wait_warp(dn0 + 8 * ds, dph, abort_flag, p.status, 7))) break;
+                    tc_fence_after();
+                    ds += NG;
+                    if (ds >= L) { ds -= L; dph ^= 1; }
+                }
                 tmem_st32(quadrant + slot * 32, r);
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(sf0 + 8 * slot);
+                if (lane == 0 && mbar_wait(bf0 + 8 * bst, bph, abort_flag, p.status, 3)) mbar_arrive(sf0 + 8 * slot);
+                __syncwarp();
+                i += NG;
                 slot += NG;
-                while (slot >= R) { slot -= R; sph ^= 1; }
+                if (slot >= R) slot -= R;
+                bst += NG;
+                while (bst >= BS) { bst -= BS; bph ^= 1; }
             }
             next -= steps;
             __syncwarp();
@@ -496,7 +435,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
             if (++c == C) c = 0;
         }
     } else {
-        mixed_epilogue<TS, QUANT>(p, tmem_base, warp, lane, u_begin, u_end, accf0, acce0, abort_flag, t_w, reinterpret_cast<float*>(extra));
+        mixed_epilogue<QUANT>(p, tmem_base, warp, lane, u_begin, u_end, accf0, acce0, abort_flag, t_w, reinterpret_cast<float*>(extra));
     }
 
     __syncthreads();
@@ -518,11 +457,11 @@ template <bool QUANT>
 __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const __grid_constant__ MixedParams p)
 {
     const MixedPlan& pl = p.pl;
-    const uint32_t C = pl.chunks, TS = (uint32_t)pl.ts, NP = (pl.n_tok + 31u) & ~31u;
-    const uint32_t tile = blockIdx.x / TS, t = blockIdx.x % TS, t_begin = tile * C, wt = tile / pl.tok_tiles * TS + t;
+    const uint32_t C = pl.chunks, NP = (pl.n_tok + 31u) & ~31u;
+    const uint32_t tile = blockIdx.x, t_begin = tile * C, wt = tile / pl.tok_tiles;
     const uint32_t c_first = cta_of(pl, t_begin), nseg = cta_of(pl, t_begin + C - 1) - c_first + 1;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (nseg == 1 || wt >= (uint32_t)p.LW.tiles) return;         // written by the CTA that has it
+    if (nseg == 1) return;                               // written by the CTA that has it
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (p.status[0] != 0) return;
     const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
@@ -531,7 +470,7 @@ __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const _
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t m0 = (int64_t)(tile % pl.tok_tiles) * pl.n_tok, m_end = min(p.M, m0 + pl.n_tok);
     auto part = [&](uint32_t i) {
-        return p.parts + ((size_t)((c_first + i) * 2 + (unit_begin(pl, c_first + i) >= t_begin ? 0u : 1u)) * TS + t) * NP * 128;
+        return p.parts + ((size_t)((c_first + i) * 2 + (unit_begin(pl, c_first + i) >= t_begin ? 0u : 1u))) * NP * 128;
     };
     if (QUANT) {
         const uint32_t col = blockIdx.y * 32 + lane;
@@ -584,55 +523,49 @@ __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const _
 }
 
 // ------------------------------------------------------------------ host side
-constexpr uint32_t MX_FIXED = 1024 /*alignment*/ + 1024 /*barriers, stage table*/;
+constexpr uint32_t MX_FIXED = 1024 /*alignment*/ + 1024 /*barriers, stage table*/, MX_TURN = 4 * 32 * 33 * 4 + 128;
 
-// Modelled clocks of a unit: dequantization (about 1100 per weight tile), MMAs (16 of N/2 clocks per weight tile), copies
-// from L2 (42 bytes per clock and SM).
-double unit_cost(int ts, uint32_t n_tok)
-{
-    const double deq = 1100.0 * ts, mma = 8.0 * n_tok * ts, l2 = (20000.0 * ts + 512.0 * n_tok) / 42.0;
-    return deq > mma ? (deq > l2 ? deq : l2) : (mma > l2 ? mma : l2);
-}
+// Modelled time of a unit in us (measured: 1.55 at 112 tokens, 1.75 at 160, 1.95 at 208, 2.15 at 256)
+double unit_us(uint32_t n_tok) { return 1.08 + 0.0042 * n_tok; }
 
-// How the work is cut: weight tiles per unit, tokens per tile, and whether CTAs take whole tiles or equal spans of units.
-// The choice is the least modelled time; measured against it on the B200 the model is within 15 % from 17 to 1000 tokens.
+// How the work is cut: tokens per tile, and whether CTAs take whole tiles or equal spans of units: the least modelled time
+// (within 10 % of the measured one from 17 to 2048 tokens).
 MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
 {
     const uint32_t wtiles = (uint32_t)((N + 127) / 128), chunks = (uint32_t)((K / 64 + 3) / 4), sms = (uint32_t)fgmp_sm_count();
+    const uint32_t t_min = (uint32_t)((M + 255) / 256);
     MixedPlan best{};
-    best.cost = 1e300;
-    for (int ts = 1; ts <= 2; ++ts) {
-        const uint32_t n_max = ts == 1 ? 256 : 208;      // 512 columns: ts accumulators and at least three steps of 32
-        const uint32_t t_min = (uint32_t)((M + n_max - 1) / n_max);
-        for (uint32_t T = t_min; T < t_min + 4 && (int64_t)(T - 1) * 16 < M; ++T) {
-            MixedPlan pl{};
-            pl.ts = ts; pl.chunks = chunks;
-            pl.n_tok = (uint32_t)(((M + T - 1) / T + 15) & ~(int64_t)15);
-            pl.tok_tiles = (uint32_t)((M + pl.n_tok - 1) / pl.n_tok);
-            pl.groups = (wtiles + ts - 1) / ts;
-            pl.tiles = pl.groups * pl.tok_tiles;
-            const double unit = unit_cost(ts, pl.n_tok), drain = 12.0 * pl.n_tok * ts;
-            const uint64_t total = (uint64_t)pl.tiles * chunks;
-            for (int split = 0; split < 2; ++split) {
-                pl.quantum = split ? 1 : chunks;
-                const uint64_t quanta = total / pl.quantum;
-                if (split && chunks == 1) continue;
-                pl.grid = (uint32_t)(quanta < sms ? quanta : sms);
-                pl.span = (uint32_t)(quanta / pl.grid); pl.rest = (uint32_t)(quanta % pl.grid);
-                const double most = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum;
-                pl.cost = most * unit + (split ? 4000.0 + 2.0 * drain : most / chunks * drain);
-                if (pl.cost < best.cost) best = pl;
-            }
+    best.us = 1e300;
+    for (uint32_t T = t_min; T < 2 * t_min + 2 && (int64_t)(T - 1) * 16 < M; ++T) {
+        MixedPlan pl{};
+        pl.chunks = chunks;
+        pl.n_tok = (uint32_t)((M + T - 1) / T + 15) / 16 * 16;
+        pl.tok_tiles = (uint32_t)((M + pl.n_tok - 1) / pl.n_tok);
+        pl.tiles = wtiles * pl.tok_tiles;
+        pl.naccs = 2 * pl.n_tok + 96 <= MX_TMEM_COLS ? 2 : 1;
+        // reading an accumulator out hides behind the next tile's products if there are two
+        const double unit = unit_us(pl.n_tok), drain = 0.012 * pl.n_tok;
+        const uint64_t total = (uint64_t)pl.tiles * chunks;
+        for (int split = 0; split < (chunks > 1 ? 2 : 1); ++split) {
+            pl.quantum = split ? 1 : chunks;
+            const uint64_t quanta = total / pl.quantum;
+            pl.grid = (uint32_t)(quanta < sms ? quanta : sms);
+            pl.span = (uint32_t)(quanta / pl.grid); pl.rest = (uint32_t)(quanta % pl.grid);
+            const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / chunks;
+            pl.us = units * unit + (pl.naccs == 2 || tiles < 1.0 ? 1.0 : tiles) * drain + (split ? 0.0 : 3.0 * tiles);
+            // the second kernel, and what it moves: a partial tile per span or two, written and read
+            if (split) pl.us += 2.0 + 2.6 * pl.grid * pl.n_tok * 512.0 / 8e6;
+            if (pl.us < best.us) best = pl;
         }
     }
     best.max_parts = best.quantum == 1 ? best.grid * 2 : 0;
-    const uint32_t tmem_slots = (MX_TMEM_COLS - best.ts * best.n_tok) / 32;
+    const uint32_t tmem_slots = (MX_TMEM_COLS - best.naccs * best.n_tok) / 32;
     best.slots = tmem_slots < (uint32_t)MAX_SLOTS ? tmem_slots : (uint32_t)MAX_SLOTS;
-    // shared memory: two weight stages, the rest token stages; with many of those, a third weight stage
-    const uint32_t room = (uint32_t)MX_SMEM_LIMIT - MX_FIXED - (4 * 32 * 33 * 4 + 128), wst = best.ts * WSTAGE, bst = best.n_tok * 128u;
+    // shared memory: two to four weight stages (a chunk each), the rest token stages
+    const uint32_t room = (uint32_t)MX_SMEM_LIMIT - MX_FIXED - MX_TURN, bst = best.n_tok * 128u;
     best.wstages = 2;
-    while (best.wstages < (uint32_t)MAX_WSTAGES && (room - (best.wstages + 1) * wst) / bst >= 5 && room > (best.wstages + 1) * wst) ++best.wstages;
-    best.bstages = (room - best.wstages * wst) / bst;
+    while (best.wstages < (uint32_t)MAX_WSTAGES && room - (best.wstages + 1) * WSTAGE >= 5 * bst) ++best.wstages;
+    best.bstages = (room - best.wstages * WSTAGE) / bst;
     if (best.bstages > (uint32_t)MAX_BSTAGES) best.bstages = MAX_BSTAGES;
     return best;
 }
@@ -646,10 +579,12 @@ bool mx_attr_set[64] = {};
 
 }  // namespace
 
+double fgmp_mixed_us(int64_t M, int64_t N, int64_t K) { return mixed_plan(M, N, K).us; }
+
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K)
 {
     const MixedPlan pl = mixed_plan(M, N, K);
-    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + (size_t)pl.max_parts * pl.ts * ((pl.n_tok + 31u) & ~31u) * 512;
+    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + (size_t)pl.max_parts * ((pl.n_tok + 31u) & ~31u) * 512;
 }
 
 // expands the activations and multiplies; leave_nvfp4: unless neither operand has an FP8 block
@@ -668,10 +603,8 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
             mx_encode = reinterpret_cast<EncodeTiledFn>(fn);
         }
         if (!mx_attr_set[dev]) {
-            if (cudaFuncSetAttribute(mixed_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess ||
-                cudaFuncSetAttribute(mixed_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess ||
-                cudaFuncSetAttribute(mixed_kernel<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess ||
-                cudaFuncSetAttribute(mixed_kernel<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess)
+            if (cudaFuncSetAttribute(mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess ||
+                cudaFuncSetAttribute(mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess)
                 return FGMP_ERR_CUDA;
             mx_attr_set[dev] = true;
         }
@@ -701,21 +634,15 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
-    const int64_t nb = M * (K / 16), sms = fgmp_sm_count();
-    cfg.gridDim = dim3((unsigned)((nb + 255) / 256 < sms * 8 ? (nb + 255) / 256 : sms * 8)); cfg.blockDim = dim3(256);
-    FGMP_LAUNCH(FGMP_K_EXPAND_A, s, cudaLaunchKernelEx(&cfg, expand_f16_kernel, (const uint8_t*)packed_acts, (const uint8_t*)packed_weights, M, K, plane, p.status, p.leave_nvfp4));
+    const fgmp_status st = fgmp_expand(packed_acts, packed_weights, M, N, K, plane, nullptr, p.status, 0, 0, leave_nvfp4, s);
+    if (st != FGMP_OK) return st;
     const bool quant = qn.codes4 != nullptr;
-    cfg.gridDim = dim3(p.pl.grid); cfg.blockDim = dim3((unsigned)mx_threads(quant));
-    cfg.dynamicSmemBytes = (size_t)p.pl.bstages * p.pl.n_tok * 128 + (size_t)p.pl.wstages * p.pl.ts * WSTAGE + MX_FIXED + 4 * 32 * 33 * 4 + 128;
-    if (p.pl.ts == 1) {
-        if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<1, true>, tmB, p)); }
-        else       { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<1, false>, tmB, p)); }
-    } else {
-        if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<2, true>, tmB, p)); }
-        else       { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<2, false>, tmB, p)); }
-    }
+    cfg.gridDim = dim3(p.pl.grid); cfg.blockDim = dim3(MX_THREADS);
+    cfg.dynamicSmemBytes = (size_t)p.pl.bstages * p.pl.n_tok * 128 + (size_t)p.pl.wstages * WSTAGE + MX_FIXED + (quant ? MX_TURN : 0);
+    if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<true>, tmB, p)); }
+    else       { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<false>, tmB, p)); }
     if (p.pl.quantum == 1) {
-        cfg.gridDim = dim3(p.pl.tiles * (unsigned)p.pl.ts, (p.pl.n_tok + 31) / 32); cfg.dynamicSmemBytes = 0;
+        cfg.gridDim = dim3(p.pl.tiles, (p.pl.n_tok + 31) / 32); cfg.dynamicSmemBytes = 0;
         cfg.blockDim = dim3(quant ? 128 : 256);
         if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_REDUCE, s, cudaLaunchKernelEx(&cfg, mixed_reduce_kernel<true>, p)); }
         else       { FGMP_LAUNCH(FGMP_K_GEMM_REDUCE, s, cudaLaunchKernelEx(&cfg, mixed_reduce_kernel<false>, p)); }

@@ -29,7 +29,15 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-// the same, but the thread may stay suspended in hardware for up to `ns` before the answer comes
+// a look at the barrier that never suspends the thread
+__device__ __forceinline__ bool mbar_test_wait(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return ok != 0;
+}
+// mbar_try_wait, but the thread may stay suspended in hardware for up to `ns` before the answer comes
 __device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t ns)
 {
     uint32_t ok;
@@ -70,11 +78,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (mbar_try_wait(bar, parity)) return true;
     return mbar_wait_slow(bar, parity, abort_flag, status, where, limit_ns);
 }
-// The same for a converged warp: one lane waits, the others are parked at the warp barrier; afterwards
-// every lane looks at the barrier once itself (it has completed: the look orders the lane's later reads).
+// The same for a warp: one lane waits, the others are parked at the warp barrier; afterwards every lane looks at the
+// barrier once itself (it has completed: the look orders the lane's later reads).  The first look is put to the vote: lanes
+// that are not converged here may see different things, and the decision has to be one for all of them.
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int where)
 {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     int ok = 1;
     if ((threadIdx.x & 31) == 0) ok = mbar_wait_slow(bar, parity, abort_flag, status, where, MBAR_WAIT_LIMIT_NS) ? 1 : 0;
     ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -123,6 +132,9 @@ __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t ncols)
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(ncols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+// Where an allocation of all 512 columns starts.  As a constant it keeps the operands of tcgen05.mma in uniform registers (read
+// back from shared memory it is moved there in front of every instruction).
+constexpr uint32_t TMEM_ALL = 0;
 __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
 {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
@@ -286,10 +298,11 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t smem_addr, uint32_t ran
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
 }
-// arrive on an mbarrier given by its shared::cluster address (possibly in the other CTA)
+// arrive on an mbarrier given by its shared::cluster address (possibly in the other CTA).  (With .release.cluster spelled out
+// a warp spends about 1000 clocks here.)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
 {
-    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // TMA tile load of a CTA pair: data into this CTA's shared memory, bytes counted on the mbarrier at
 // the shared::cluster address `bar` (the pair's leader)
