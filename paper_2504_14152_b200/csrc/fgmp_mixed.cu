@@ -564,7 +564,7 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
     // shared memory: two to four weight stages (a chunk each), the rest token stages
     const uint32_t room = (uint32_t)MX_SMEM_LIMIT - MX_FIXED - MX_TURN, bst = best.n_tok * 128u;
     best.wstages = 2;
-    while (best.wstages < (uint32_t)MAX_WSTAGES && room - (best.wstages + 1) * WSTAGE >= 5 * bst) ++best.wstages;
+    while (best.wstages < (uint32_t)MAX_WSTAGES && room - (best.wstages + 1) * WSTAGE >= 10 * bst) ++best.wstages;
     best.bstages = (room - best.wstages * WSTAGE) / bst;
     if (best.bstages > (uint32_t)MAX_BSTAGES) best.bstages = MAX_BSTAGES;
     return best;

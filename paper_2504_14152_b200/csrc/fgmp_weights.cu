@@ -7,55 +7,82 @@
 
 namespace {
 
+constexpr int SEL_BINS = 2048;           // bins of a digit of the radix select
+
 // Device-resident state of one packing call (lives at the start of the workspace).
 struct SelectState {
-    uint32_t hist[256];
+    uint32_t hist[SEL_BINS];
+    uint32_t arrived;        // thread blocks that have finished the current kernel (the last one does what follows it)
     uint32_t amax_bits;      // max |w| as fp32 bits
     float s4;                // NVFP4 tensor scale in use
     uint32_t prefix;         // radix-select prefix (high bits of the k-th largest score)
-    uint32_t pad0;
     unsigned long long krem; // how many blocks are still to be taken inside the prefix group
     float tau;               // threshold: FP8 iff score > tau, or == tau within the first need_eq
-    uint32_t use_eq;
+    uint32_t use_eq;         // 0: none of the blocks equal to tau is taken, 1: the first need_eq of them, 2: all
     unsigned long long need_eq;
     unsigned long long n_fp8;
     float next_below;        // calibration: largest score strictly below tau
     uint32_t pad1;
 };
 
-constexpr size_t STATE_BYTES = 2048;
+constexpr size_t STATE_BYTES = 16384;
+static_assert(sizeof(SelectState) <= STATE_BYTES, "state section of the workspace");
 
-__global__ void state_init_kernel(SelectState* st, float s4_given, unsigned long long k)
+__global__ void state_init_kernel(SelectState* st, float s4_given, unsigned long long k, float tau)
 {
-    int t = threadIdx.x;
-    if (t < 256) st->hist[t] = 0;
-    if (t == 0) {
-        st->amax_bits = 0; st->s4 = s4_given; st->prefix = 0; st->krem = k; st->tau = 0.f;
+    for (int t = threadIdx.x; t < SEL_BINS; t += blockDim.x) st->hist[t] = 0;
+    if (threadIdx.x == 0) {
+        st->arrived = 0;
+        st->amax_bits = 0; st->s4 = s4_given; st->prefix = 0; st->krem = k; st->tau = tau;
         st->use_eq = 0; st->need_eq = 0; st->n_fp8 = 0; st->next_below = 0.f;
     }
 }
 
-__global__ void w_amax_kernel(const uint4* W, int64_t ldw8, int64_t N, int64_t K8, SelectState* st)
+// The last thread block of a grid to come here goes on with what used to be a kernel of its own (it sees what every other
+// block has written before); the counter is ready for the next kernel.  Called by all threads of the block.
+__device__ __forceinline__ bool last_block(uint32_t* arrived)
+{
+    __shared__ uint32_t s_old;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_old = atomicInc(arrived, gridDim.x * gridDim.y - 1);
+    __syncthreads();
+    __threadfence();
+    return s_old == gridDim.x * gridDim.y - 1;
+}
+
+// max |w| and the tensor scale.  A block takes four rows of W at a time: four 16-byte loads per thread in flight.
+__global__ void __launch_bounds__(256) w_amax_kernel(const uint4* W, int64_t ldw8, int64_t N, uint32_t K8, SelectState* st)
 {
     uint32_t m = 0;
-    const int64_t total = N * K8;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t n = i / K8, c = i % K8;
-        uint4 x = __ldg(W + n * ldw8 + c);
+    auto take = [&](const uint4& x) {
         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             m = max(m, (w[j] << 16) & 0x7fffffffu);
             m = max(m, w[j] & 0x7fff0000u);
         }
+    };
+    for (int64_t n = 4 * (int64_t)blockIdx.x; n < N; n += 4 * (int64_t)gridDim.x) {
+        const uint4* row = W + n * ldw8;
+        for (uint32_t c = threadIdx.x; c < K8; c += 256) {
+            uint4 x[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) x[i] = n + i < N ? __ldg(row + i * ldw8 + c) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) take(x[i]);
+        }
     }
     for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&st->amax_bits, m);
-}
-
-__global__ void w_scale_kernel(SelectState* st)
-{
-    if (threadIdx.x == 0) st->s4 = __fdiv_rn(__uint_as_float(st->amax_bits), 2688.0f);
+    __shared__ uint32_t s_max[8];
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {                              // one atomic per block: they all go to one word
+        for (int i = 1; i < 8; ++i) m = max(m, s_max[i]);
+        atomicMax(&st->amax_bits, m);
+    }
+    if (last_block(&st->arrived) && threadIdx.x == 0)
+        st->s4 = __fdiv_rn(__uint_as_float(*reinterpret_cast<volatile uint32_t*>(&st->amax_bits)), 2688.0f);
 }
 
 __device__ __forceinline__ void load_block(const uint4* W, int64_t ldw8, const float* F, int64_t ldf,
@@ -73,19 +100,55 @@ __device__ __forceinline__ void load_block(const uint4* W, int64_t ldw8, const f
     }
 }
 
-// per block: microscale (dynamic max or Eq. 11 brute force) and the score under it
+// two values rounded to E2M1 and back
+__device__ __forceinline__ float2 round_e2m1x2(float lo, float hi)
+{
+    uint32_t h2;
+    asm("{\n\t.reg .b8 t;\n\tcvt.rn.satfinite.e2m1x2.f32 t, %1, %2;\n\tcvt.rn.f16x2.e2m1x2 %0, t;\n\t}" : "=r"(h2) : "f"(hi), "f"(lo));
+    return __half22float2(*reinterpret_cast<__half2*>(&h2));
+}
+
+// Weighted squared error of a block under microscale d (inv = 1/d), the terms added in element order.  BOUND: clipped = the
+// largest term of an element whose magnitude is not below 6 d, i.e. that is clipped: it only grows with a smaller scale.
+template <bool BOUND>
+__device__ __forceinline__ float clip_error(const float (&v)[16], const float (&f)[16], float2 dd, float& clipped)
+{
+    const float d = dd.x, inv = dd.y, d6 = __fmul_rn(6.0f, d);
+    float j = 0.f, top = 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) {
+        const float2 q = round_e2m1x2(__fmul_rn(v[i], inv), __fmul_rn(v[i + 1], inv));
+        const float e0 = __fsub_rn(__fmul_rn(q.x, d), v[i]), t0 = __fmul_rn(__fmul_rn(f[i], e0), e0);
+        const float e1 = __fsub_rn(__fmul_rn(q.y, d), v[i + 1]), t1 = __fmul_rn(__fmul_rn(f[i + 1], e1), e1);
+        j = __fadd_rn(__fadd_rn(j, t0), t1);
+        if (BOUND) {
+            top = fmaxf(top, fabsf(v[i]) >= d6 ? t0 : 0.f);
+            top = fmaxf(top, fabsf(v[i + 1]) >= d6 ? t1 : 0.f);
+        }
+    }
+    if (BOUND) clipped = top;
+    return j;
+}
+
+// Per block: microscale (dynamic max or Eq. 11 search) and the score under it.
+//
+// The search asks for the scale with the least error among all 126, ties to the dynamic-max scale and then to the smaller
+// code.  It need not look at all of them: going down from the dynamic-max code, an element that is clipped has an error that
+// only grows (every rounding step is monotone), and a sum of non-negative terms is never below one of them, so once such a
+// term alone exceeds the least error found no smaller scale can win.  Going up there are few codes left, because the tensor
+// scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left (25 for the longest of a warp): 4096 x 4096 takes 185 us, 680
+// before.
 template <int MODE, bool CLIP>
 __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ldw8, const float* F, int64_t ldf,
                                                       int64_t N, int64_t KB, int ratio, float s8_given, const SelectState* st,
                                                       uint8_t* sc_out, float* scores)
 {
-    __shared__ float s_d[128], s_inv[128];
+    __shared__ float2 s_d[127];                          // scale and its inverse, by code
     const float s4 = st->s4;
     if (CLIP) {
         if (threadIdx.x < 127) {
-            float d = __fmul_rn(e4m3_to_f32(threadIdx.x), s4);
-            s_d[threadIdx.x] = d;
-            s_inv[threadIdx.x] = (d == 0.f) ? 0.f : __fdiv_rn(1.0f, d);
+            const float d = __fmul_rn(e4m3_to_f32(threadIdx.x), s4);
+            s_d[threadIdx.x] = make_float2(d, (d == 0.f) ? 0.f : __fdiv_rn(1.0f, d));
         }
         __syncthreads();
     }
@@ -98,32 +161,20 @@ __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ld
         load_block(W, ldw8, F, ldf, b / KB, b % KB, v, f);
         uint32_t sc = block_dynamic_scale(v, k6);
         if (CLIP) {
-            // incumbent = dynamic max; ascending scan, strict improvement only
-            float best;
-            {
-                float d = s_d[sc], inv = s_inv[sc];
-                best = 0.f;
-#pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                    float2 q = e2m1x2_to_f32x2(f32x2_to_e2m1x2(__fmul_rn(v[i], inv), __fmul_rn(v[i + 1], inv)));
-                    float e0 = __fsub_rn(__fmul_rn(q.x, d), v[i]);
-                    best = __fadd_rn(best, __fmul_rn(__fmul_rn(f[i], e0), e0));
-                    float e1 = __fsub_rn(__fmul_rn(q.y, d), v[i + 1]);
-                    best = __fadd_rn(best, __fmul_rn(__fmul_rn(f[i + 1], e1), e1));
-                }
+            const int dyn = (int)sc;
+            float clipped, best = clip_error<true>(v, f, s_d[dyn], clipped);
+            bool more = !(clipped > best);
+#pragma unroll 1
+            for (int c = dyn - 1; more && c >= 1; --c) {
+                const float j = clip_error<true>(v, f, s_d[c], clipped);
+                // going down, a tie is a smaller code: it wins unless the dynamic-max code holds the lead
+                if (j < best || (j == best && (int)sc != dyn)) { best = j; sc = (uint32_t)c; }
+                more = !(clipped > best);
             }
-            for (uint32_t c = 1; c <= 0x7e; ++c) {
-                float d = s_d[c], inv = s_inv[c];
-                float j = 0.f;
-#pragma unroll
-                for (int i = 0; i < 16; i += 2) {
-                    float2 q = e2m1x2_to_f32x2(f32x2_to_e2m1x2(__fmul_rn(v[i], inv), __fmul_rn(v[i + 1], inv)));
-                    float e0 = __fsub_rn(__fmul_rn(q.x, d), v[i]);
-                    j = __fadd_rn(j, __fmul_rn(__fmul_rn(f[i], e0), e0));
-                    float e1 = __fsub_rn(__fmul_rn(q.y, d), v[i + 1]);
-                    j = __fadd_rn(j, __fmul_rn(__fmul_rn(f[i + 1], e1), e1));
-                }
-                if (j < best) { best = j; sc = c; }
+#pragma unroll 1
+            for (int c = dyn + 1; c <= 0x7e; ++c) {
+                const float j = clip_error<false>(v, f, s_d[c], clipped);
+                if (j < best) { best = j; sc = (uint32_t)c; }
             }
         }
         uint32_t c4[2];
@@ -144,74 +195,93 @@ __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ld
 }
 
 // ------------------------------------------------------------ radix select (k-th largest)
-// Scores are >= 0, so their fp32 bit patterns order like unsigned integers.
-__global__ void select_hist_kernel(const float* scores, int64_t B, int pass, SelectState* st)
+// Scores are >= 0, so their fp32 bit patterns order like unsigned integers.  Three digits (11, 11, 10 bits) with a pass over
+// the scores each; the last thread block of a pass picks the digit, so that a pass is one launch.  (Four digits of eight bits
+// and a launch for each pick took 200 us for a packing and a calibration, of which the shared counters' conflicts most: the
+// upper eight bits of the scores take a few values only.)
+__global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_t B, int pass, SelectState* st)
 {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
+    __shared__ uint32_t h[SEL_BINS];
+    __shared__ unsigned long long s_sum[512];
+    const int bits = pass == 2 ? 10 : 11, shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
+    for (int i = threadIdx.x; i < SEL_BINS; i += 512) h[i] = 0;
     __syncthreads();
-    const int shift = 24 - 8 * pass;
-    const uint32_t prefix = st->prefix;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < B; b += (int64_t)gridDim.x * blockDim.x) {
-        uint32_t u = __float_as_uint(scores[b]);
-        if (pass == 0 || (u >> (shift + 8)) == prefix) atomicAdd(&h[(u >> shift) & 255], 1u);
+    const uint32_t prefix = st->prefix, low = (1u << bits) - 1u;
+    const int64_t stride = (int64_t)gridDim.x * 512;
+    for (int64_t b = (int64_t)blockIdx.x * 512 + threadIdx.x; b < B; b += 4 * stride) {
+        uint32_t u[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) u[i] = b + i * stride < B ? __float_as_uint(__ldg(scores + b + i * stride)) : 0u;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            if (b + i * stride < B && (pass == 0 || (u[i] >> (shift + bits)) == prefix)) atomicAdd(&h[(u[i] >> shift) & low], 1u);
     }
     __syncthreads();
-    if (h[threadIdx.x]) atomicAdd(&st->hist[threadIdx.x], h[threadIdx.x]);
-}
-
-__global__ void select_pick_kernel(SelectState* st, int pass)
-{
-    if (threadIdx.x == 0) {
-        unsigned long long krem = st->krem, cum = 0;
-        int bin = 255;
-        for (; bin > 0; --bin) {
-            if (cum + st->hist[bin] >= krem) break;
-            cum += st->hist[bin];
-        }
-        st->prefix = (st->prefix << 8) | (uint32_t)bin;
-        st->krem = krem - cum;
-        if (pass == 3) {
-            st->tau = __uint_as_float(st->prefix);
-            st->need_eq = st->krem;          // of the blocks equal to tau, take this many
-            st->use_eq = 1;
+    for (int i = threadIdx.x; i < SEL_BINS; i += 512)
+        if (h[i]) atomicAdd(&st->hist[i], h[i]);
+    if (!last_block(&st->arrived)) return;
+    // thread t has bins 4t .. 4t+3; from the top: the bin in which the count of larger ones and its own reaches krem
+    uint32_t own[4];
+    unsigned long long sum = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) { own[i] = *reinterpret_cast<volatile uint32_t*>(&st->hist[4 * threadIdx.x + i]); sum += own[i]; }
+    s_sum[threadIdx.x] = sum;
+    __syncthreads();
+    for (int o = 1; o < 512; o <<= 1) {                  // sums over the threads t, t + 1, ...
+        const unsigned long long y = threadIdx.x + o < 512 ? s_sum[threadIdx.x + o] : 0ull;
+        __syncthreads();
+        s_sum[threadIdx.x] += y;
+        __syncthreads();
+    }
+    const unsigned long long krem = st->krem;
+    unsigned long long above = s_sum[threadIdx.x] - sum;
+    if (above < krem && krem <= s_sum[threadIdx.x]) {
+        int i = 3;
+        while (i > 0 && above + own[i] < krem) above += own[i--];
+        st->prefix = (prefix << bits) | (uint32_t)(4 * threadIdx.x + i);
+        st->krem = krem - above;
+        if (pass == 2) {
+            st->tau = __uint_as_float((prefix << bits) | (uint32_t)(4 * threadIdx.x + i));
+            st->need_eq = krem - above;                  // of the blocks equal to tau, take this many
+            st->use_eq = krem - above == own[i] ? 2u : 1u;
         }
     }
-    __syncthreads();
-    if (threadIdx.x < 256) st->hist[threadIdx.x] = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) st->hist[4 * threadIdx.x + i] = 0;
 }
 
-// largest score strictly below tau (calibration: the (k+1)-th largest when there are no ties)
-__global__ void next_below_kernel(const float* scores, int64_t B, SelectState* st)
+// Threshold of a calibration: midway between the k-th largest score and the largest below it (all_or_none: see the callers)
+__global__ void __launch_bounds__(512) calib_finish_kernel(const float* scores, int64_t B, SelectState* st, float* tau_out, int all_or_none)
 {
+    if (all_or_none) {
+        // k = 0: nothing exceeds +inf; k = all
+        if (blockIdx.x == 0 && threadIdx.x == 0) *tau_out = all_or_none == 1 ? __int_as_float(0x7f800000) : -1.0f;
+        return;
+    }
     const float tau = st->tau;
     uint32_t m = 0;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < B; b += (int64_t)gridDim.x * blockDim.x) {
-        float s = scores[b];
-        if (s < tau) m = max(m, __float_as_uint(s));
+    const int64_t stride = (int64_t)gridDim.x * 512;
+    for (int64_t b = (int64_t)blockIdx.x * 512 + threadIdx.x; b < B; b += 4 * stride) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float s = b + i * stride < B ? __ldg(scores + b + i * stride) : 0.f;
+            if (s < tau) m = max(m, __float_as_uint(s));
+        }
     }
     for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<uint32_t*>(&st->next_below), m);
-}
-
-__global__ void calib_finish_kernel(const SelectState* st, float* tau_out, int all_or_none)
-{
-    if (threadIdx.x == 0) {
-        if (all_or_none == 1) *tau_out = __int_as_float(0x7f800000);   // k = 0: nothing exceeds +inf
-        else if (all_or_none == 2) *tau_out = -1.0f;                   // k = all
-        else {
-            // midway between the k-th largest score and the next one below it; if fp32 cannot
-            // separate them, the lower neighbour itself (score > tau still selects the top k)
-            float t = __fmul_rn(0.5f, __fadd_rn(st->tau, st->next_below));
-            *tau_out = (t < st->tau && t >= st->next_below) ? t : st->next_below;
-        }
+    if (last_block(&st->arrived) && threadIdx.x == 0) {
+        // if fp32 cannot separate the two, the lower neighbour itself (score > tau still selects the top k)
+        const float below = *reinterpret_cast<volatile float*>(&st->next_below), t = __fmul_rn(0.5f, __fadd_rn(tau, below));
+        *tau_out = (t < tau && t >= below) ? t : below;
     }
 }
 
 // ------------------------------------------------------------ mask, prefix sums, emission
-// per mask word: how many of its blocks have score == tau
+// per mask word: how many of its blocks have score == tau (needed only if some of them are taken and some are not)
 __global__ void w_eqcount_kernel(const float* scores, int64_t N, int64_t KB, int64_t MW, const SelectState* st, uint32_t* cnt)
 {
+    if (st->use_eq != 1) return;
     const float tau = st->tau;
     const int lane = threadIdx.x & 31;
     const int64_t nw = N * MW;
@@ -223,37 +293,11 @@ __global__ void w_eqcount_kernel(const float* scores, int64_t N, int64_t KB, int
     }
 }
 
-// (mask16: the bits in the order of the packed tensor, a uint16 per row of a unit)
-__global__ void w_mask_kernel(const float* scores, int64_t N, int64_t KB, int64_t MW, const SelectState* st,
-                              const uint32_t* eqprefix, uint16_t* mask16, int64_t chunks)
+// exclusive prefix sum of n uint32 by one CTA of 1024 threads
+// (of the counts that w_eqcount_kernel has left, where it has)
+__global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* in, uint32_t* out, int64_t n, const SelectState* st)
 {
-    const float tau = st->tau;
-    const bool use_eq = st->use_eq != 0;
-    const unsigned long long need_eq = st->need_eq;
-    const int lane = threadIdx.x & 31;
-    const int64_t nw = N * MW;
-    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw; w += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        int64_t n = w / MW, kb = (w % MW) * 32 + lane;
-        float s = kb < KB ? scores[n * KB + kb] : -1.f;
-        bool gt = kb < KB && s > tau;
-        bool eq = use_eq && kb < KB && s == tau;
-        uint32_t eqbal = __ballot_sync(0xffffffffu, eq);
-        bool take = gt;
-        if (eq) {
-            unsigned long long rank = (unsigned long long)eqprefix[w] + __popc(eqbal & ((1u << lane) - 1u));
-            take = rank < need_eq;
-        }
-        uint32_t word = __ballot_sync(0xffffffffu, take);
-        // lanes 0 and 1: the word's two chunks
-        const int64_t c = 2 * (w % MW) + lane;
-        if (lane < 2 && c < chunks) mask16[((n >> 7) * chunks + c) * 128 + (n & 127)] = (uint16_t)(word >> (16 * lane));
-    }
-}
-
-// exclusive prefix sum of n uint32 by one CTA of 1024 threads; total -> *total_out (may be NULL)
-__global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* in, uint32_t* out, int64_t n, unsigned long long* total_out,
-                                                    int append_total)
-{
+    if (st->use_eq != 1) return;
     __shared__ uint32_t warp_sums[32];
     __shared__ unsigned long long carry_s;
     if (threadIdx.x == 0) carry_s = 0;
@@ -278,29 +322,87 @@ __global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* in, uint32_t
         if (threadIdx.x == 1023) carry_s = carry + warp_sums[31] + incl;
         __syncthreads();
     }
-    if (threadIdx.x == 0 && total_out) *total_out = carry_s;
-    if (threadIdx.x == 0 && append_total) out[n] = (uint32_t)carry_s;
 }
 
-// per unit (128-row tile x 16-block K chunk): size of its list of FP8 blocks in 16-byte steps, and the
-// running total of FP8 blocks.  One CTA of 128 threads per unit, a thread per row.
-// Mask bits of rows beyond the tensor are cleared here.
-__global__ void __launch_bounds__(128) w_unit_count_kernel(uint16_t* mask16, PackedLayout L, uint32_t* list_steps,
-                                                           SelectState* st)
+// The mask of one unit (128-row tile x 16-block K chunk), a thread per row, and the size of its list of FP8 blocks in 16-byte
+// steps.  The last thread block then has what concerns the whole tensor: where the lists start, and the header.  With too
+// little room the starts are pulled back inside the blob, so that a reader that follows them stays within the allocation.
+struct MaskParams {
+    const float* scores; const uint32_t* eqprefix; uint16_t* mask16; uint32_t* list_steps; uint32_t* uptr;
+    fgmp_packed_header* header; SelectState* st;
+    PackedLayout L;
+    int64_t room_steps;
+    int ratio; float s8_given;
+};
+__global__ void __launch_bounds__(128) w_mask_kernel(const __grid_constant__ MaskParams p)
 {
     __shared__ uint32_t s_cnt[4];
-    const int64_t unit = blockIdx.x;
-    uint16_t* own = mask16 + unit * 128 + threadIdx.x;
-    uint32_t c = 0;
-    if ((unit / L.chunks) * 128 + threadIdx.x < L.rows) c = __popc((uint32_t)*own);
-    else *own = 0;
-    for (int o = 16; o; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-    if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = c;
+    const PackedLayout& L = p.L;
+    const int64_t unit = blockIdx.x, n = unit / L.chunks * 128 + threadIdx.x, c = unit % L.chunks;
+    const float tau = p.st->tau;
+    const uint32_t use_eq = p.st->use_eq;
+    const int blocks = (int)min((int64_t)16, L.KB - c * 16);
+    uint32_t gt = 0, eq = 0;
+    if (n < L.rows) {
+        const float4* src = reinterpret_cast<const float4*>(p.scores + n * L.KB + c * 16);      // (KB is a multiple of four)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (4 * i < blocks) {
+                const float4 x = __ldg(src + i);
+                const float v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) { gt |= (v[e] > tau ? 1u : 0u) << (4 * i + e); eq |= (v[e] == tau ? 1u : 0u) << (4 * i + e); }
+            }
+        }
+        if (use_eq == 2) gt |= eq;
+        else if (use_eq == 1 && eq) {
+            // of the blocks equal to tau the first need_eq in row-major order: those before this mask word, and in its first half
+            unsigned long long rank = p.eqprefix[n * L.MW + (c >> 1)];
+            if (c & 1)
+                for (int i = 0; i < 16; ++i) rank += p.scores[n * L.KB + (c - 1) * 16 + i] == tau ? 1u : 0u;
+            for (uint32_t todo = eq; todo; todo &= todo - 1u, ++rank)
+                if (rank < p.st->need_eq) gt |= todo & (0u - todo);
+        }
+    }
+    p.mask16[unit * 128 + threadIdx.x] = (uint16_t)gt;
+    uint32_t cnt = __popc(gt);
+    for (int o = 16; o; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    if ((threadIdx.x & 31) == 0) s_cnt[threadIdx.x >> 5] = cnt;
     __syncthreads();
     if (threadIdx.x == 0) {
-        const uint32_t cnt = s_cnt[0] + s_cnt[1] + s_cnt[2] + s_cnt[3];
-        list_steps[unit] = fgmp_list_steps(cnt);
-        atomicAdd(&st->n_fp8, (unsigned long long)cnt);
+        cnt = s_cnt[0] + s_cnt[1] + s_cnt[2] + s_cnt[3];
+        p.list_steps[unit] = fgmp_list_steps(cnt);
+        atomicAdd(&p.st->n_fp8, (unsigned long long)cnt);
+    }
+    if (!last_block(&p.st->arrived)) return;
+    // exclusive sums over the units, 128 at a time
+    __shared__ uint32_t s_warp[4];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned long long carry = 0;
+    const uint32_t room = (uint32_t)min(p.room_steps, (int64_t)0xffffffffll);
+    for (int64_t base = 0; base < L.units; base += 128) {
+        const int64_t i = base + threadIdx.x;
+        const uint32_t x = i < L.units ? __ldcg(p.list_steps + i) : 0u;
+        uint32_t incl = x;
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+        if (lane == 31) s_warp[w] = incl;
+        __syncthreads();
+        uint32_t before = 0;
+        for (int k = 0; k < w; ++k) before += s_warp[k];
+        const unsigned long long at = carry + before + incl - x;
+        if (i < L.units) p.uptr[i] = (uint32_t)min(at, (unsigned long long)room);
+        carry += s_warp[0] + s_warp[1] + s_warp[2] + s_warp[3];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        p.uptr[L.units] = (uint32_t)min(carry, (unsigned long long)room);
+        fgmp_packed_header* h = p.header;
+        const float s4 = p.st->s4;
+        h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = L.rows; h->K = L.K; h->scale_fp4 = s4;
+        h->fp8_log2_ratio = p.ratio; h->n_fp8 = (int64_t)*reinterpret_cast<volatile unsigned long long*>(&p.st->n_fp8); h->kind = 1; h->capacity = p.room_steps;
+        h->error = (int64_t)carry > p.room_steps ? (int32_t)FGMP_ERR_CAPACITY : 0;
+        h->scale_fp8 = p.s8_given > 0.f ? p.s8_given : __fmul_rn(s4, __int_as_float((127 + p.ratio) << 23));
+        h->fp8_scale_free = p.s8_given > 0.f ? 1 : 0;
     }
 }
 
@@ -308,12 +410,12 @@ __global__ void __launch_bounds__(128) w_unit_count_kernel(uint16_t* mask16, Pac
 // blocks, the running counts of FP8 blocks by row) and the list of its FP8 blocks (rows, second halves).  One CTA
 // of 128 threads per unit.
 __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw8, int ratio, float s8_given, const SelectState* st,
-                                                     const uint8_t* sc_in, uint8_t* blob, PackedLayout L, int64_t room_steps)
+                                                     const uint8_t* sc_in, uint8_t* blob, PackedLayout L)
 {
     __shared__ UnitScratch sc;
     const int64_t unit = blockIdx.x, tile = unit / L.chunks, c = unit % L.chunks;
     const uint32_t* uptr = reinterpret_cast<const uint32_t*>(blob + L.off_uptr);
-    const bool fits = (int64_t)uptr[unit + 1] <= room_steps;   // else the blob is too small: header.error says so
+    const bool fits = reinterpret_cast<const fgmp_packed_header*>(blob)->error == 0;   // else the blob is too small for the lists
     const float s4 = st->s4;
     const float s8 = s8_given > 0.f ? s8_given : __fmul_rn(s4, __int_as_float((127 + ratio) << 23));
     const float inv8 = __fdiv_rn(1.0f, s8);
@@ -361,34 +463,12 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
     }
 }
 
-// With too little room the starts of the overflow entries are pulled back inside the blob, so that a
-// reader that follows them stays within the allocation (the entries themselves were not written).
-__global__ void w_clamp_uptr_kernel(const fgmp_packed_header* h, uint32_t* uptr, int64_t n, int64_t room_steps)
+// The last kernel of a packing writes what nobody reads early (see fgmp_linear on programmatic dependents).
+__global__ void w_finish_kernel(fgmp_packed_header* h, const SelectState* st, int fraction_mode, float tau_given, float* tau_eff_out)
 {
-    if (h->error == 0) return;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        if ((int64_t)uptr[i] > room_steps) uptr[i] = (uint32_t)room_steps;
-}
-
-__global__ void w_header_kernel(fgmp_packed_header* h, const SelectState* st, const uint32_t* uptr, int64_t units,
-                                int64_t N, int64_t K, int ratio, float s8_given, int64_t room_steps, int fraction_mode, float tau_given,
-                                float* tau_eff_out)
-{
-    if (threadIdx.x == 0) {
-        h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = N; h->K = K; h->scale_fp4 = st->s4;
-        h->fp8_log2_ratio = ratio; h->n_fp8 = (int64_t)st->n_fp8; h->kind = 1; h->capacity = room_steps;
-        float teff = fraction_mode ? st->tau : tau_given;
-        h->tau_eff = teff;
-        h->error = ((int64_t)uptr[units] > room_steps) ? (int32_t)FGMP_ERR_CAPACITY : 0;
-        h->scale_fp8 = s8_given > 0.f ? s8_given : __fmul_rn(st->s4, __int_as_float((127 + ratio) << 23));
-        h->fp8_scale_free = s8_given > 0.f ? 1 : 0;
-        if (tau_eff_out) *tau_eff_out = teff;
-    }
-}
-
-__global__ void set_tau_kernel(SelectState* st, float tau)
-{
-    if (threadIdx.x == 0) { st->tau = tau; st->use_eq = 0; st->need_eq = 0; }
+    const float teff = fraction_mode ? st->tau : tau_given;
+    h->tau_eff = teff;
+    if (tau_eff_out) *tau_eff_out = teff;
 }
 
 int grid_for(int64_t work_items, int threads, int max_ctas_per_sm)
@@ -400,14 +480,24 @@ int grid_for(int64_t work_items, int threads, int max_ctas_per_sm)
     return (int)g;
 }
 
-// runs the 4-pass radix select for the k-th largest of scores[0..B)
+// three-pass radix select for the k-th largest of scores[0..B)
 void run_select(const float* scores, int64_t B, SelectState* st, cudaStream_t s)
 {
-    int g = grid_for(B, 256, 8);
-    for (int pass = 0; pass < 4; ++pass) {
-        FGMP_LAUNCH(FGMP_K_SELECT, s, select_hist_kernel<<<g, 256, 0, s>>>(scores, B, pass, st));
-        FGMP_LAUNCH(FGMP_K_SELECT, s, select_pick_kernel<<<1, 256, 0, s>>>(st, pass));
+    const int g = grid_for(B, 512 * 4, 1);      // (a block ends with an atomic per bin in use: few blocks)
+    for (int pass = 0; pass < 3; ++pass) FGMP_LAUNCH(FGMP_K_SELECT, s, select_kernel<<<g, 512, 0, s>>>(scores, B, pass, st));
+}
+
+// the threshold from the scores (k of B blocks above it)
+fgmp_status run_calibration(const float* scores, int64_t B, int64_t k, SelectState* st, float* tau_out, cudaStream_t s)
+{
+    if (k == 0 || k == B) {
+        FGMP_LAUNCH(FGMP_K_SELECT, s, calib_finish_kernel<<<1, 512, 0, s>>>(scores, B, st, tau_out, k == 0 ? 1 : 2));
+    } else {
+        FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 1024, 0, s>>>(st, 1.0f, (unsigned long long)k, 0.f));
+        run_select(scores, B, st, s);
+        FGMP_LAUNCH(FGMP_K_SELECT, s, calib_finish_kernel<<<grid_for(B, 512 * 4, 2), 512, 0, s>>>(scores, B, st, tau_out, 0));
     }
+    return fgmp_launch_status();
 }
 
 // words in each of the two scratch arrays: one per mask word, or one per (tile, chunk) + 1
@@ -473,11 +563,10 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
     const int ratio = sc.fp8_log2_ratio;
     const float s8_given = sc.scale_fp8;
 
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 256, 0, s>>>(st, sc.scale_fp4, (unsigned long long)k));
-    if (sc.scale_fp4 == 0.f) {
-        FGMP_LAUNCH(FGMP_K_W_AMAX, s, w_amax_kernel<<<grid_for(N * (K / 8), 256, 8), 256, 0, s>>>(W, ldw / 8, N, K / 8, st));
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, w_scale_kernel<<<1, 32, 0, s>>>(st));
-    }
+    // (k == 0: nothing is FP8, tau_eff = +inf; threshold mode: the given tau)
+    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 1024, 0, s>>>(st, sc.scale_fp4, (unsigned long long)k, fraction_mode ? INFINITY : tau));
+    if (sc.scale_fp4 == 0.f)
+        FGMP_LAUNCH(FGMP_K_W_AMAX, s, w_amax_kernel<<<grid_for(N, 4, 8), 256, 0, s>>>(W, ldw / 8, N, (uint32_t)(K / 8), st));
     {
         int g = grid_for(B, 256, 4);
         if (sm == FGMP_SCORE_LP_ERROR) {
@@ -488,25 +577,19 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
             else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<1, false><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
         }
     }
-    uint16_t* mask16 = reinterpret_cast<uint16_t*>(blob + L.off_mask);
-    uint32_t* uptr = reinterpret_cast<uint32_t*>(blob + L.off_uptr);
-    const int64_t NCT = L.units;
     const int gw = grid_for(NW * 32, 256, 8);
     if (fraction_mode && k > 0) {
         run_select(scores, B, st, s);
         FGMP_LAUNCH(FGMP_K_W_MASK, s, w_eqcount_kernel<<<gw, 256, 0, s>>>(scores, N, KB, MW, st, tmp_a));
-        FGMP_LAUNCH(FGMP_K_SCAN, s, scan_kernel<<<1, 1024, 0, s>>>(tmp_a, tmp_b, NW, nullptr, 0));
-    } else {
-        // k == 0: nothing is FP8 (tau_eff = +inf); threshold mode: the given tau
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, set_tau_kernel<<<1, 32, 0, s>>>(st, fraction_mode ? INFINITY : tau));
+        FGMP_LAUNCH(FGMP_K_SCAN, s, scan_kernel<<<1, 1024, 0, s>>>(tmp_a, tmp_b, NW, st));
     }
-    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_mask_kernel<<<gw, 256, 0, s>>>(scores, N, KB, MW, st, tmp_b, mask16, L.chunks));
-    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_unit_count_kernel<<<(unsigned)NCT, 128, 0, s>>>(mask16, L, tmp_a, st));
-    FGMP_LAUNCH(FGMP_K_SCAN, s, scan_kernel<<<1, 1024, 0, s>>>(tmp_a, uptr, NCT, nullptr, 1));
-    FGMP_LAUNCH(FGMP_K_W_EMIT, s, w_emit_kernel<<<(unsigned)NCT, 128, 0, s>>>(W, ldw / 8, ratio, s8_given, st, sc_tmp, blob, L, room_steps));
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, w_header_kernel<<<1, 32, 0, s>>>(reinterpret_cast<fgmp_packed_header*>(blob), st, uptr, NCT, N, K, ratio, s8_given,
-                                     room_steps, fraction_mode ? 1 : 0, tau, tau_eff_out));
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, w_clamp_uptr_kernel<<<grid_for(NCT + 1, 256, 1), 256, 0, s>>>(reinterpret_cast<const fgmp_packed_header*>(blob), uptr, NCT + 1, room_steps));
+    MaskParams mp;
+    mp.scores = scores; mp.eqprefix = tmp_b; mp.mask16 = reinterpret_cast<uint16_t*>(blob + L.off_mask); mp.list_steps = tmp_a;
+    mp.uptr = reinterpret_cast<uint32_t*>(blob + L.off_uptr); mp.header = reinterpret_cast<fgmp_packed_header*>(blob); mp.st = st;
+    mp.L = L; mp.room_steps = room_steps; mp.ratio = ratio; mp.s8_given = s8_given;
+    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_mask_kernel<<<(unsigned)L.units, 128, 0, s>>>(mp));
+    FGMP_LAUNCH(FGMP_K_W_EMIT, s, w_emit_kernel<<<(unsigned)L.units, 128, 0, s>>>(W, ldw / 8, ratio, s8_given, st, sc_tmp, blob, L));
+    FGMP_LAUNCH(FGMP_K_W_AUX, s, w_finish_kernel<<<1, 1, 0, s>>>(reinterpret_cast<fgmp_packed_header*>(blob), st, fraction_mode ? 1 : 0, tau, tau_eff_out));
     return fgmp_launch_status();
 }
 
@@ -529,15 +612,7 @@ extern "C" fgmp_status fgmp_calibrate_tau(const void* X_bf16, int64_t ldx, const
     if (stt != FGMP_OK) return stt;
     int64_t k = (int64_t)floor(fp8_fraction * (double)B + 0.5);
     if (k > B) k = B;
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 256, 0, s>>>(st, sc.scale_fp4, (unsigned long long)k));
-    if (k == 0 || k == B) {
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, calib_finish_kernel<<<1, 32, 0, s>>>(st, tau_out, k == 0 ? 1 : 2));
-    } else {
-        run_select(scores, B, st, s);
-        FGMP_LAUNCH(FGMP_K_SELECT, s, next_below_kernel<<<grid_for(B, 256, 8), 256, 0, s>>>(scores, B, st));
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, calib_finish_kernel<<<1, 32, 0, s>>>(st, tau_out, 0));
-    }
-    return fgmp_launch_status();
+    return run_calibration(scores, B, k, st, tau_out, s);
 }
 
 extern "C" fgmp_status fgmp_weight_scores(const void* W_bf16, int64_t ldw, const float* fisher_elem, int64_t ldf,
@@ -563,11 +638,9 @@ extern "C" fgmp_status fgmp_weight_scores(const void* W_bf16, int64_t ldw, const
     const uint4* W = reinterpret_cast<const uint4*>(W_bf16);
     const int ratio = sc.fp8_log2_ratio;
     const float s8_given = sc.scale_fp8;
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 256, 0, s>>>(st, sc.scale_fp4, 0ull));
-    if (sc.scale_fp4 == 0.f) {
-        FGMP_LAUNCH(FGMP_K_W_AMAX, s, w_amax_kernel<<<grid_for(N * (K / 8), 256, 8), 256, 0, s>>>(W, ldw / 8, N, K / 8, st));
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, w_scale_kernel<<<1, 32, 0, s>>>(st));
-    }
+    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 1024, 0, s>>>(st, sc.scale_fp4, 0ull, 0.f));
+    if (sc.scale_fp4 == 0.f)
+        FGMP_LAUNCH(FGMP_K_W_AMAX, s, w_amax_kernel<<<grid_for(N, 4, 8), 256, 0, s>>>(W, ldw / 8, N, (uint32_t)(K / 8), st));
     const int g = grid_for(B, 256, 4);
     if (sm == FGMP_SCORE_LP_ERROR) {
         if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<0, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
@@ -610,13 +683,5 @@ extern "C" fgmp_status fgmp_global_tau(const float* const* score_arrays, const i
     }
     int64_t k = (int64_t)floor(fp8_fraction * (double)B + 0.5);
     if (k > B) k = B;
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 256, 0, s>>>(st, 1.0f, (unsigned long long)k));
-    if (k == 0 || k == B) {
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, calib_finish_kernel<<<1, 32, 0, s>>>(st, tau_out, k == 0 ? 1 : 2));
-    } else {
-        run_select(scores, B, st, s);
-        FGMP_LAUNCH(FGMP_K_SELECT, s, next_below_kernel<<<grid_for(B, 256, 8), 256, 0, s>>>(scores, B, st));
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, calib_finish_kernel<<<1, 32, 0, s>>>(st, tau_out, 0));
-    }
-    return fgmp_launch_status();
+    return run_calibration(scores, B, k, st, tau_out, s);
 }
