@@ -228,31 +228,53 @@ struct BlockQ {
     float score;
 };
 
+// largest magnitude of 16 values, two at a time (a NaN counts for nothing)
+__device__ __forceinline__ float block_amax(const float (&v)[16])
+{
+    float a = 0.f;
+#pragma unroll
+    for (int i = 0; i < 16; i += 2) asm("max.abs.f32 %0, %0, %1, %2;" : "+f"(a) : "f"(v[i]), "f"(v[i + 1]));
+    return a;
+}
+
 // dynamic-max microscale code: E4M3(amax * k6), k6 = 1 / (6 * s4)
 __device__ __forceinline__ uint32_t block_dynamic_scale(const float (&v)[16], float k6)
 {
-    float amax = 0.f;
+    return f32x2_to_e4m3x2(__fmul_rn(block_amax(v), k6), 0.f) & 0x7f;
+}
+
+// four pairs of values -> eight E2M1 codes in a word, and the codes' values
+__device__ __forceinline__ uint32_t round_e2m1x8(const float (&y)[8], float2 (&q)[4])
+{
+    uint32_t w, h[4];
+    asm("{\n\t.reg .b8 a, b, c, d;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 a, %6, %5;\n\tcvt.rn.satfinite.e2m1x2.f32 b, %8, %7;\n\t"
+        "cvt.rn.satfinite.e2m1x2.f32 c, %10, %9;\n\tcvt.rn.satfinite.e2m1x2.f32 d, %12, %11;\n\t"
+        "cvt.rn.f16x2.e2m1x2 %1, a;\n\tcvt.rn.f16x2.e2m1x2 %2, b;\n\tcvt.rn.f16x2.e2m1x2 %3, c;\n\tcvt.rn.f16x2.e2m1x2 %4, d;\n\t"
+        "mov.b32 %0, {a, b, c, d};\n\t}"
+        : "=r"(w), "=r"(h[0]), "=r"(h[1]), "=r"(h[2]), "=r"(h[3])
+        : "f"(y[0]), "f"(y[1]), "f"(y[2]), "f"(y[3]), "f"(y[4]), "f"(y[5]), "f"(y[6]), "f"(y[7]));
 #pragma unroll
-    for (int i = 0; i < 16; ++i) amax = fmaxf(amax, fabsf(v[i]));
-    return f32x2_to_e4m3x2(__fmul_rn(amax, k6), 0.f) & 0x7f;
+    for (int i = 0; i < 4; ++i) q[i] = __half22float2(*reinterpret_cast<__half2*>(&h[i]));
+    return w;
 }
 
 // NVFP4 rounding under microscale code `sc`; dq receives the dequantized values
 __device__ __forceinline__ void block_nvfp4(const float (&v)[16], uint32_t sc, float s4,
                                             uint32_t (&c4)[2], float (&dq)[16])
 {
-    float d = __fmul_rn(e4m3_to_f32(sc), s4);
-    float inv = (d == 0.f) ? 0.f : __fdiv_rn(1.0f, d);
-    c4[0] = 0; c4[1] = 0;
+    const float d = __fmul_rn(e4m3_to_f32(sc), s4);
+    const float inv = (d == 0.f) ? 0.f : __fdiv_rn(1.0f, d);
 #pragma unroll
-    for (int i = 0; i < 16; i += 2) {
-        float y0 = __fmul_rn(v[i], inv), y1 = __fmul_rn(v[i + 1], inv);
-        // inv == 0 (zero scale): keep only the signs, as -0.0 * 0 = -0.0 does
-        uint32_t b = f32x2_to_e2m1x2(y0, y1);
-        float2 q = e2m1x2_to_f32x2(b);
-        dq[i] = __fmul_rn(q.x, d);
-        dq[i + 1] = __fmul_rn(q.y, d);
-        c4[i >> 3] |= b << ((i & 7) * 4);
+    for (int w = 0; w < 2; ++w) {
+        // (inv == 0, a zero scale: only the signs stay, as -0.0 * 0 = -0.0)
+        float y[8];
+        float2 q[4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) y[i] = __fmul_rn(v[8 * w + i], inv);
+        c4[w] = round_e2m1x8(y, q);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { dq[8 * w + 2 * i] = __fmul_rn(q[i].x, d); dq[8 * w + 2 * i + 1] = __fmul_rn(q[i].y, d); }
     }
 }
 
@@ -261,12 +283,12 @@ __device__ __forceinline__ void block_fp8(const float (&v)[16], float inv8, floa
                                           uint32_t (&c8)[4], float (&dq)[16])
 {
 #pragma unroll
-    for (int i = 0; i < 16; i += 2) {
-        uint32_t two = f32x2_to_e4m3x2(__fmul_rn(v[i], inv8), __fmul_rn(v[i + 1], inv8));
-        float2 q = e4m3x2_to_f32x2(two);
-        dq[i] = __fmul_rn(q.x, s8);
-        dq[i + 1] = __fmul_rn(q.y, s8);
-        if ((i & 3) == 0) c8[i >> 2] = two; else c8[i >> 2] |= two << 16;
+    for (int i = 0; i < 16; i += 4) {
+        const uint32_t lo = f32x2_to_e4m3x2(__fmul_rn(v[i], inv8), __fmul_rn(v[i + 1], inv8));
+        const uint32_t hi = f32x2_to_e4m3x2(__fmul_rn(v[i + 2], inv8), __fmul_rn(v[i + 3], inv8));
+        const float2 a = e4m3x2_to_f32x2(lo), b = e4m3x2_to_f32x2(hi);
+        dq[i] = __fmul_rn(a.x, s8); dq[i + 1] = __fmul_rn(a.y, s8); dq[i + 2] = __fmul_rn(b.x, s8); dq[i + 3] = __fmul_rn(b.y, s8);
+        c8[i >> 2] = lo | (hi << 16);
     }
 }
 

@@ -1,16 +1,19 @@
 // Online activation quantizer (Section 4.2 of the paper), block scores, and the
 // packed -> canonical unpacker.
 //
-// Thread mapping: one thread owns one 16-element block column (kb) and walks down the rows
-// of its CTA, so the 16 per-channel Fisher weights stay in registers.  A warp covers 32
-// consecutive blocks of one row = one mask word, produced with a ballot.
+// Thread mapping: a warp owns 32 consecutive block columns (one mask word, produced with a ballot) and walks down a few rows, a
+// thread per column, so the 16 per-channel Fisher weights stay in registers; the next row is loaded while one is worked on.
+//
+// Bound by instruction issue from a few hundred rows on (rounding to both formats and back, the score in element order), by the launch
+// below that.  2048 x 5120 takes 10.8 us (2.7 TB/s) and 8192 x 8192 43 us; with blocks of 256 columns
+// and one load at a time it was 16.5 and 45 us.  Asking for more resident warps (64 registers) is slower, 13.8 us for the former.
 #include "fgmp_common.cuh"
 #include "fgmp_host.h"
 #include <cuda_bf16.h>
 
 namespace {
 
-constexpr int QA_THREADS = 256;
+constexpr int QA_THREADS = 128;
 
 struct ActParams {
     const uint4* X; int64_t ldx8;        // row stride in 16-byte units
@@ -24,7 +27,8 @@ struct ActParams {
     float r8;                            // 2^ratio
     int ratio;
     int free8;                           // the FP8 tensor scale was given on its own
-    int rows_per_cta;
+    int rows_per_warp;
+    uint32_t groups;                     // row groups: warps = groups * MW
 };
 
 template <int MODE, bool SCORE_ONLY>
@@ -33,18 +37,18 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
     // A kernel launched behind this one as a programmatic dependent (the decode-sized GEMM) may
     // start setting itself up now; it waits for this grid to complete before it reads the result.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int64_t kb = (int64_t)blockIdx.x * QA_THREADS + threadIdx.x;
-    const bool active = kb < p.KB;
-    const int64_t m0 = (int64_t)blockIdx.y * p.rows_per_cta;
-    const int64_t m1 = min(m0 + (int64_t)p.rows_per_cta, p.M);
-    if (!SCORE_ONLY) {
-        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
-            fgmp_packed_header* h = p.header;
-            h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = p.M; h->K = p.K; h->scale_fp4 = p.s4;
-            h->fp8_log2_ratio = p.ratio; h->n_fp8 = (p.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
-            h->error = 0; h->scale_fp8 = p.s8; h->fp8_scale_free = p.free8;
-        }
+    if (!SCORE_ONLY && blockIdx.x == 0 && threadIdx.x == 0) {
+        fgmp_packed_header* h = p.header;
+        h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = p.M; h->K = p.K; h->scale_fp4 = p.s4;
+        h->fp8_log2_ratio = p.ratio; h->n_fp8 = (p.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
+        h->error = 0; h->scale_fp8 = p.s8; h->fp8_scale_free = p.free8;
     }
+    const uint32_t warp = blockIdx.x * (QA_THREADS / 32) + (threadIdx.x >> 5), MW = (uint32_t)p.MW, group = warp / MW, word = warp - group * MW;
+    if (group >= p.groups) return;
+    const int64_t kb = (int64_t)word * 32 + (threadIdx.x & 31);
+    const bool active = kb < p.KB;
+    const int64_t m0 = (int64_t)group * p.rows_per_warp;
+    const int64_t m1 = min(m0 + (int64_t)p.rows_per_warp, p.M);
 
     float f[16];
     if (active) {
@@ -59,11 +63,16 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
         for (int i = 0; i < 16; ++i) f[i] = 0.f;
     }
 
+    uint4 na = make_uint4(0u, 0u, 0u, 0u), nb = na;
+    const uint4* xp = p.X + m0 * p.ldx8 + kb * 2;
+    if (active) { na = __ldcs(xp); nb = __ldcs(xp + 1); }
+#pragma unroll 1
     for (int64_t m = m0; m < m1; ++m) {
         bool is8 = false;
+        const uint4 xa = na, xb = nb;
+        xp += p.ldx8;
+        if (active && m + 1 < m1) { na = __ldcs(xp); nb = __ldcs(xp + 1); }
         if (active) {
-            const uint4* xp = p.X + m * p.ldx8 + kb * 2;
-            uint4 xa = __ldcs(xp), xb = __ldcs(xp + 1);
             float v[16], dq4[16];
             unpack_bf16x16(xa, xb, v);
             uint32_t sc = block_dynamic_scale(v, p.k6);
@@ -123,11 +132,8 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
             }
         }
         if (!SCORE_ONLY) {
-            uint32_t word = __ballot_sync(0xffffffffu, is8);
-            int64_t w = kb >> 5;
-            if ((threadIdx.x & 31) == 0 && w < p.MW) {
-                p.mask[m * p.MW + w] = word;
-            }
+            const uint32_t bits = __ballot_sync(0xffffffffu, is8);
+            if ((threadIdx.x & 31) == 0) p.mask[m * p.MW + word] = bits;
         }
     }
 }
@@ -218,8 +224,11 @@ ActParams make_act_params(const void* X, int64_t ldx, const float* fisher, int64
     p.tau = tau;
     p.ratio = sc.fp8_log2_ratio;
     p.r8 = ldexpf(1.0f, sc.fp8_log2_ratio);
-    // enough CTAs to fill the machine when M is small, few row-loop iterations otherwise
-    p.rows_per_cta = (M >= 2048) ? 8 : (M >= 256 ? 4 : 1);
+    // rows per warp: one while there are fewer warps than the machine holds (28 per SM), up to eight so that the Fisher weights
+    // are loaded rarely (8192 x 8192: 43 us with up to eight, 46 with four, 53 with two, 70 with one)
+    const int64_t words = M * p.MW, fit = words / ((int64_t)fgmp_sm_count() * 28);
+    p.rows_per_warp = (int)(fit < 1 ? 1 : fit > 8 ? 8 : fit);
+    p.groups = (uint32_t)((M + p.rows_per_warp - 1) / p.rows_per_warp);
     return p;
 }
 
@@ -246,7 +255,7 @@ extern "C" fgmp_status fgmp_quantize_activations(const void* X_bf16, int64_t ldx
     p.mask = reinterpret_cast<uint32_t*>(blob + L.off_mask); p.codes8 = blob + L.off_codes8;
     p.header = reinterpret_cast<fgmp_packed_header*>(blob);
     if (M <= 16 && !p.free8) p.arec = blob + L.off_arec;     // decode-sized batch: also emit the records of the decode GEMM (tied scales only)
-    dim3 grid((unsigned)((p.KB + QA_THREADS - 1) / QA_THREADS), (unsigned)((M + p.rows_per_cta - 1) / p.rows_per_cta));
+    const dim3 grid((unsigned)(((int64_t)p.groups * p.MW + QA_THREADS / 32 - 1) / (QA_THREADS / 32)));
     if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, quant_act_kernel<0, false><<<grid, QA_THREADS, 0, s>>>(p));
     else                           FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, quant_act_kernel<1, false><<<grid, QA_THREADS, 0, s>>>(p));
     return fgmp_launch_status();
@@ -263,7 +272,7 @@ extern "C" fgmp_status fgmp_activation_scores(const void* X_bf16, int64_t ldx, c
     cudaStream_t s = (cudaStream_t)cuda_stream;
     ActParams p = make_act_params(X_bf16, ldx, fisher_chan, M, K, sc, 0.f);
     p.scores = scores;
-    dim3 grid((unsigned)((p.KB + QA_THREADS - 1) / QA_THREADS), (unsigned)((M + p.rows_per_cta - 1) / p.rows_per_cta));
+    const dim3 grid((unsigned)(((int64_t)p.groups * p.MW + QA_THREADS / 32 - 1) / (QA_THREADS / 32)));
     if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, quant_act_kernel<0, true><<<grid, QA_THREADS, 0, s>>>(p));
     else                           FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, quant_act_kernel<1, true><<<grid, QA_THREADS, 0, s>>>(p));
     return fgmp_launch_status();
