@@ -1,0 +1,129 @@
+"""GPU parity at the edges of each kernel's and each dispatch rule's range: tile remainders, the smallest and largest sizes
+of a path, block mixes that take a kernel's side routes.  Same oracle and bars as test_gpu_parity.py."""
+import numpy as np
+import pytest
+import torch
+
+import fgmp_inputs as gi
+import oracle
+from test_gpu_parity import GEMM_TOL, compare_packed, fg, quantize_both, tau_for_fraction   # noqa: F401  (fg is a fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def check_linear(fg, qa, qw, pa, pw, rel=1e-5):
+    """fp32 and bf16 output, the latter with a row pitch that rules wide stores out, against the oracle."""
+    Y, S = oracle.linear(qa, qw)
+    y = fg.linear(pa, pw)
+    fg.check(fg.linear.last_workspace)
+    err = np.abs(y.cpu().numpy().astype(np.float64) - Y)
+    assert (err <= rel * S + 1e-30).all(), f"max err/S = {(err / np.maximum(S, 1e-300)).max():.3e}"
+    wide = torch.zeros(qa.rows, qw.rows + 3, dtype=torch.bfloat16, device="cuda")
+    fg.linear(pa, pw, out=wide[:, :qw.rows])
+    fg.check(fg.linear.last_workspace)
+    yb = wide.float().cpu().numpy().astype(np.float64)
+    assert (np.abs(yb[:, :qw.rows] - Y) <= GEMM_TOL * S + np.abs(Y) * 2.0 ** -8 + 1e-30).all()
+    assert not yb[:, qw.rows:].any(), "stored outside the output"
+
+
+# one CTA per tile; pairs with a last tile that has one row in the second CTA, none, and a single weight tile
+@pytest.mark.parametrize("M,N,K", [(17, 130, 64), (129, 257, 320), (385, 9857, 128), (260, 12673, 64), (257, 256, 1088)])
+def test_nvfp4_gemm_tiles(fg, M, N, K):
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("n4", M, N, K, seed=61), 0.0, 0.0, clip=False)
+    check_linear(fg, qa, qw, pa, pw)
+
+
+# token tiles of 16 to 256, one chunk and many, part of a last chunk, part of a weight tile; FP8 shares below and above what a
+# stage holds; split and whole tiles
+@pytest.mark.parametrize("M,N,K", [(17, 129, 64), (33, 300, 576), (100, 257, 1088), (256, 640, 2112), (273, 5000, 320)])
+@pytest.mark.parametrize("frac_a,frac_w", [(0.1, 0.1), (0.0, 0.35), (1.0, 1.0), (0.3, 0.0)])
+def test_gemm_on_packed_weights_edges(fg, M, N, K, frac_a, frac_w):
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("mx", M, N, K, seed=62), frac_a, frac_w, clip=False)
+    check_linear(fg, qa, qw, pa, pw)
+    assert torch.equal(fg.linear(pa, pw), fg.linear(pa, pw)), "the sum over the parts of a tile has a fixed order"
+
+
+@pytest.mark.parametrize("M,N,K,mode", [(17, 192, 64, 0), (49, 320, 1088, 1), (130, 1088, 2112, 0)])
+def test_quantizer_behind_split_tiles(fg, M, N, K, mode):
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("mq", M, N, K, seed=63), 0.1, 0.1, clip=False)
+    y = fg.linear(pa, pw, out_dtype=torch.bfloat16)
+    f = torch.rand(N, generator=torch.Generator().manual_seed(1)) + 0.5
+    s4 = gi.tensor_scale(y.float().cpu())
+    tau = tau_for_fraction(oracle.quantize_activations(gi.bf16_bits(y.cpu()), f.numpy(), s4, tau=np.inf, mode=mode).scores, 0.2)
+    q = oracle.quantize_activations(gi.bf16_bits(y.cpu()), f.numpy(), s4, tau=tau, mode=mode)
+    compare_packed(fg, fg.linear_quantize(pa, pw, f.cuda(), scale_fp4=s4, score_mode=mode, tau=tau), q, tau, "hidden")
+
+
+# large batch: both operands expanded to fp16 planes, ragged in every direction
+@pytest.mark.parametrize("frac_a,frac_w", [(0.1, 0.1), (0.0, 1.0)])
+def test_gemm_on_expanded_planes_ragged(fg, frac_a, frac_w):
+    M, N, K = 2049, 4113, 4160
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("pl", M, N, K, seed=64), frac_a, frac_w, clip=False)
+    y = fg.linear(pa, pw).cpu().numpy().astype(np.float64)
+    fg.check(fg.linear.last_workspace)
+    rng = np.random.default_rng(0)
+    ms, nn = np.r_[rng.integers(0, M, 4000), [M - 1, M - 1, 0]], np.r_[rng.integers(0, N, 4000), [N - 1, 0, N - 1]]
+    Y, S = oracle.linear_sampled(qa, qw, ms, nn)
+    assert (np.abs(y[ms, nn] - Y) <= 1e-5 * S + 1e-30).all() and np.isfinite(y).all()
+
+
+# both formats over the whole range of the ratio of their tensor scales: the common scale of the fp16 values shifts with it
+@pytest.mark.parametrize("ratio", [-7, 0, 7])
+@pytest.mark.parametrize("M", [7, 40])
+def test_ratio_of_the_tensor_scales(fg, M, ratio):
+    wl = gi.llama("r", M, 300, 576, seed=65)
+    x, fx, w, fw = wl.x(), wl.fx(), wl.w(), wl.fw()
+    s4 = gi.tensor_scale(x)
+    tau = tau_for_fraction(oracle.quantize_activations(gi.bf16_bits(x), fx.numpy(), s4, ratio=ratio).scores, 0.3)
+    qa = oracle.quantize_activations(gi.bf16_bits(x), fx.numpy(), s4, ratio=ratio, tau=tau)
+    qw = oracle.quantize_weights(gi.bf16_bits(w), fw.numpy(), ratio=ratio, clip=False, fp8_fraction=0.3)
+    pa = fg.quantize_activations(x.cuda(), fx.cuda(), scale_fp4=s4, ratio=ratio, tau=tau)
+    pw = fg.quantize_weights(w.cuda(), fw.cuda(), ratio=ratio, clip_mode=0, fp8_fraction=0.3)
+    compare_packed(fg, pa, qa, tau, "activations")
+    compare_packed(fg, pw, qw, None, "weights")
+    check_linear(fg, qa, qw, pa, pw)
+
+
+# rows per warp from one to eight, block columns that do not fill a mask word
+@pytest.mark.parametrize("M,K", [(1, 64), (3, 448), (900, 8256), (2500, 8256)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_quantizer_row_groups(fg, M, K, mode):
+    wl = gi.llama("q", M, 16, K, seed=66)
+    x, fx = wl.x(), wl.fx()
+    x[::7, :48] = 0
+    s4 = gi.tensor_scale(x)
+    tau = tau_for_fraction(oracle.quantize_activations(gi.bf16_bits(x), fx.numpy(), s4, mode=mode).scores, 0.1)
+    q = oracle.quantize_activations(gi.bf16_bits(x), fx.numpy(), s4, tau=tau, mode=mode)
+    compare_packed(fg, fg.quantize_activations(x.cuda(), fx.cuda(), scale_fp4=s4, score_mode=mode, tau=tau), q, tau, f"{M}x{K}")
+
+
+# the search for the clipping scale, where it may leave scales out: heavy tails, blocks of one value, of zeros and of signed zeros, a
+# tensor scale under which every scale clips and one under which none does
+@pytest.mark.parametrize("N,K,scale", [(1, 64, 0.0), (5, 192, 0.0), (131, 448, 0.0), (33, 1088, 1e-7), (33, 1088, 0.5)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_clip_search_equals_the_exhaustive_one(fg, N, K, scale, mode):
+    g = torch.Generator().manual_seed(N * K + mode)
+    w = (torch.randn(N, K, generator=g) * torch.exp(2.0 * torch.randn(N, K, generator=g)) * 0.02)
+    w[:, :16] = 0
+    w[N // 2, 16:32] = 0.01
+    w[0, 32:48] *= -0.0
+    w = w.to(torch.bfloat16)
+    fw = torch.exp(1.5 * torch.randn(N, K, generator=g))
+    fw[:, 48:56] = 0
+    q = oracle.quantize_weights(gi.bf16_bits(w), fw.numpy(), scale_fp4=scale, clip=True, mode=mode, fp8_fraction=0.1)
+    p = fg.quantize_weights(w.cuda(), fw.cuda(), scale_fp4=scale, clip_mode=1, score_mode=mode, fp8_fraction=0.1)
+    compare_packed(fg, p, q, None, f"{N}x{K}")
+
+
+# equal scores at the threshold: none, some and all of them taken, from one block to many
+@pytest.mark.parametrize("rows,same", [(1, 1), (5, 3), (300, 299), (300, 150)])
+def test_selection_among_equal_scores(fg, rows, same):
+    K = 192
+    w = gi.weights(rows, K, 67)
+    w[:same] = w[0]
+    fw = torch.ones(rows, K)
+    for frac in (1 / (rows * 12), 0.25, 0.6, same / rows):
+        q = oracle.quantize_weights(gi.bf16_bits(w), fw.numpy(), clip=False, fp8_fraction=frac)
+        p = fg.quantize_weights(w.cuda(), fw.cuda(), clip_mode=0, fp8_fraction=frac)
+        compare_packed(fg, p, q, None, f"frac={frac}")
+        assert p.header()["n_fp8"] == q.mask_bits().sum()
