@@ -8,13 +8,17 @@
 // its 128-row operand from.  What bounds what:
 //   - expanding the weights to a plane first costs 2.7 bytes written and read for every packed byte, which is the whole
 //     call at small batches (4096 x 4096, 48 tokens: 59 us with the plane);
-//   - a 128 x 256 unit of weights takes about 1000 clocks of the SIMT pipes (1024 conversions at one per clock), so that
-//     the MMAs (16 of N/2 clocks for N tokens) bound from 128 tokens on, the dequantization below;
+//   - a 128 x 256 unit of weights takes about 1000 clocks of the SIMT pipes (1024 conversions at one per clock), its MMAs 16 of
+//     N/2 clocks for N tokens;
 //   - the operand from tensor memory leaves shared memory to the token tiles (from shared memory the 64 KiB of a
 //     dequantized unit would be written and read there, 1024 clocks by themselves);
-//   - a unit takes 1.08 us + 4.2 ns per token (MMAs alone 4.3 ns per token at 1.85 GHz): the dequantizing warps, whose step is a
-//     chain of shared-memory loads, conversions, a tensor-memory store and three barriers, and the MMA issuer share four
-//     schedulers.  CTA pairs that share a token tile (half the L2 traffic) were measured and are no faster.
+//   - a unit takes 1.08 us + 4.2 ns per token, more than its MMAs (4.3 ns per token) or its dequantization: with either of them or
+//     the token copies left out it is 7 to 20 % faster, with all of them left out 27 %.  What remains is the way of a slot through
+//     three groups of warps (copy, dequantize, multiply, release), some 2000 clocks, and at full rate the token tiles would
+//     take 64 bytes per clock and SM from L2.  Four groups, CTA pairs that share a token tile, more weight stages, spinning
+//     instead of suspended waits and a loop of one elected thread in the issuer were measured and are no faster.
+//   - so a unit is worth as many tokens as fit: up to 416 (two MMAs side by side on one dequantized operand) where a CTA's share lies within
+//     a tile (400 x 11008 x 4096: 48 us, 54 with two tiles of 208; 1200 x 4096 x 4096: 52 and 57).
 //
 // Work is (weight tile, token tile, 256-element K chunk) units in that order, split over the CTAs either in
 // equal contiguous spans (stream-K: the partial sums of tiles shared by several CTAs are stored column by column and added
@@ -43,12 +47,14 @@ constexpr uint32_t HALF_CAP = 5248;             // 656 FP8 blocks (32 %); with m
 constexpr uint32_t WSTAGE = STG_HALF + HALF_CAP;                         // 24064
 constexpr int MAX_WSTAGES = 4, MAX_BSTAGES = 12, MAX_SLOTS = 8;
 constexpr uint32_t MX_TMEM_COLS = 512;
+constexpr uint32_t MX_MAX_TOK = 416;            // tokens of a tile: columns of its accumulator, beside three slots of 32
 constexpr size_t MX_SMEM_LIMIT = 232448;
 constexpr uint32_t SW128_LO = 1u << 16, SW128_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 constexpr uint32_t IDESC_F16 = 1u << 4;         // f32 += f16 x f16, K-major; M and N added
 
 struct MixedPlan {
     uint32_t n_tok, tok_tiles;           // tokens per tile (multiple of 16), token tiles
+    uint32_t n_half;                     // tokens of one MMA: n_tok, or the first half (rounded up to 16) of a tile of more than 256
     uint32_t chunks, tiles;              // tiles = wtiles * tok_tiles
     uint32_t grid, span, rest, quantum;  // a CTA's span in quanta of `quantum` units (1, or chunks: whole tiles)
     uint32_t wstages, bstages, slots, naccs, max_parts;
@@ -176,7 +182,8 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     const uint32_t BS = pl.bstages, WS = pl.wstages, R = pl.slots, NT = pl.n_tok, C = pl.chunks;
     // (no more groups than slots: a group that was further ahead could take an older phase of a slot's barrier for the one it waits for)
     const uint32_t NG = min((uint32_t)MX_GROUPS, R);
-    const uint32_t b_bytes = NT * 128u;                 // token stage: NT rows x 64 elements, swizzled (a multiple of 2 KiB)
+    const uint32_t NH = pl.n_half;
+    const uint32_t b_bytes = (NT > NH ? 2u : 1u) * NH * 128u;   // token stage: rows of 64 elements, swizzled (a multiple of 2 KiB)
     uint8_t* wst0 = smem + BS * b_bytes;
     uint8_t* extra = wst0 + WS * WSTAGE;                 // QUANT: 4 x 32 x 33 floats
     uint64_t* bars = reinterpret_cast<uint64_t*>(extra + (QUANT ? 4 * 32 * 33 * 4 + 128 : 0));
@@ -286,6 +293,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
                     }
                     mbar_expect_tx(bf0 + 8 * stage, b_bytes);
                     tma_load_2d(smem_u32(smem + stage * b_bytes), &tmB, (int32_t)(c * 256 + s * 64), (int32_t)m0, bf0 + 8 * stage);
+                    if (NT > NH) tma_load_2d(smem_u32(smem + stage * b_bytes) + NH * 128u, &tmB, (int32_t)(c * 256 + s * 64), (int32_t)(m0 + NH), bf0 + 8 * stage);
                     if (++stage == BS) stage = 0;
                 }
             }
@@ -294,7 +302,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     } else if (warp == W_MMA) {
         // ------------------------------------------------------------ MMA issuer (one elected lane)
         {
-            const uint32_t idesc = IDESC_F16 | ((NT >> 3) << 17) | ((128u >> 4) << 24), b_first = (smem_u32(smem) >> 4) | SW128_LO, b_step = b_bytes >> 4;
+            const uint32_t idesc = IDESC_F16 | ((NH >> 3) << 17) | ((128u >> 4) << 24), idesc2 = IDESC_F16 | (((NT - NH) >> 3) << 17) | ((128u >> 4) << 24), b_first = (smem_u32(smem) >> 4) | SW128_LO, b_step = b_bytes >> 4;
             uint32_t bst = 0, slot = 0, sph = 0, ds = 0, c = u_begin % C, acc = 0, acc_phase = 1, accum = 0, b_lo = b_first;
             bool ok = true, ready = false;
             for (uint32_t u = u_begin; u < u_end && ok; ++u) {
@@ -310,6 +318,10 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
                     if (elect_one()) {
 #pragma unroll
                         for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d, a + 8 * k, mx_desc(b_lo + 2 * k), idesc, k ? 1u : accum);
+                        if (NT > NH) {
+#pragma unroll
+                            for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d + NH, a + 8 * k, mx_desc(b_lo + NH * 8u + 2 * k), idesc2, k ? 1u : accum);
+                        }
                         umma_commit(dn0 + 8 * ds);
                     }
                     accum = 1;
@@ -533,13 +545,14 @@ double unit_us(uint32_t n_tok) { return 1.08 + 0.0042 * n_tok; }
 MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
 {
     const uint32_t wtiles = (uint32_t)((N + 127) / 128), chunks = (uint32_t)((K / 64 + 3) / 4), sms = (uint32_t)fgmp_sm_count();
-    const uint32_t t_min = (uint32_t)((M + 255) / 256);
+    const uint32_t t_min = (uint32_t)((M + MX_MAX_TOK - 1) / MX_MAX_TOK), t_max = 2 * (uint32_t)((M + 255) / 256) + 2;
     MixedPlan best{};
     best.us = 1e300;
-    for (uint32_t T = t_min; T < 2 * t_min + 2 && (int64_t)(T - 1) * 16 < M; ++T) {
+    for (uint32_t T = t_min; T < t_max && (int64_t)(T - 1) * 16 < M; ++T) {
         MixedPlan pl{};
         pl.chunks = chunks;
         pl.n_tok = (uint32_t)((M + T - 1) / T + 15) / 16 * 16;
+        pl.n_half = pl.n_tok <= 256 ? pl.n_tok : (pl.n_tok + 31) / 32 * 16;
         pl.tok_tiles = (uint32_t)((M + pl.n_tok - 1) / pl.n_tok);
         pl.tiles = wtiles * pl.tok_tiles;
         pl.naccs = 2 * pl.n_tok + 96 <= MX_TMEM_COLS ? 2 : 1;
@@ -552,7 +565,10 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
             pl.grid = (uint32_t)(quanta < sms ? quanta : sms);
             pl.span = (uint32_t)(quanta / pl.grid); pl.rest = (uint32_t)(quanta % pl.grid);
             const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / chunks;
-            pl.us = units * unit + (pl.naccs == 2 || tiles < 1.0 ? 1.0 : tiles) * drain + (split ? 0.0 : 3.0 * tiles);
+            // (beyond 256 tokens only spans within one tile pay: where a CTA goes on to another one its three slots and three
+            // token stages run empty as well)
+            const double drains = pl.naccs == 2 || tiles < 1.0 ? 1.0 : pl.n_tok <= 256 ? tiles : 2.0 * (tiles + 1.0);
+            pl.us = units * unit + drains * drain + (split ? 0.0 : 3.0 * tiles);
             // the second kernel, and what it moves: a partial tile per span or two, written and read
             if (split) pl.us += 2.0 + 2.6 * pl.grid * pl.n_tok * 512.0 / 8e6;
             if (pl.us < best.us) best = pl;
@@ -562,7 +578,7 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
     const uint32_t tmem_slots = (MX_TMEM_COLS - best.naccs * best.n_tok) / 32;
     best.slots = tmem_slots < (uint32_t)MAX_SLOTS ? tmem_slots : (uint32_t)MAX_SLOTS;
     // shared memory: two to four weight stages (a chunk each), the rest token stages
-    const uint32_t room = (uint32_t)MX_SMEM_LIMIT - MX_FIXED - MX_TURN, bst = best.n_tok * 128u;
+    const uint32_t room = (uint32_t)MX_SMEM_LIMIT - MX_FIXED - MX_TURN, bst = (best.n_tok > best.n_half ? 2u : 1u) * best.n_half * 128u;
     best.wstages = 2;
     while (best.wstages < (uint32_t)MAX_WSTAGES && room - (best.wstages + 1) * WSTAGE >= 10 * bst) ++best.wstages;
     best.bstages = (room - best.wstages * WSTAGE) / bst;
@@ -620,11 +636,11 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     uint8_t* plane = ws + FGMP_WS_CONTROL_BYTES;
     p.parts = reinterpret_cast<float*>(plane + fgmp_align1k((size_t)M * K * 2));
     p.q = qn;
-    // the activations' fp16 plane [M, K]: boxes of n_tok rows x 64 elements, swizzled; rows beyond M are zero
+    // the activations' fp16 plane [M, K]: boxes of n_half rows x 64 elements, swizzled; rows beyond M are zero
     CUtensorMap tmB;
     cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
     cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {64, p.pl.n_tok};
+    cuuint32_t box[2] = {64, p.pl.n_half};
     cuuint32_t estr[2] = {1, 1};
     if (mx_encode(&tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plane, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return FGMP_ERR_CUDA;
@@ -638,7 +654,7 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     if (st != FGMP_OK) return st;
     const bool quant = qn.codes4 != nullptr;
     cfg.gridDim = dim3(p.pl.grid); cfg.blockDim = dim3(MX_THREADS);
-    cfg.dynamicSmemBytes = (size_t)p.pl.bstages * p.pl.n_tok * 128 + (size_t)p.pl.wstages * WSTAGE + MX_FIXED + (quant ? MX_TURN : 0);
+    cfg.dynamicSmemBytes = (size_t)p.pl.bstages * (p.pl.n_tok > p.pl.n_half ? 2 : 1) * p.pl.n_half * 128 + (size_t)p.pl.wstages * WSTAGE + MX_FIXED + (quant ? MX_TURN : 0);
     if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<true>, tmB, p)); }
     else       { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<false>, tmB, p)); }
     if (p.pl.quantum == 1) {

@@ -54,6 +54,24 @@ def test_quantizer_behind_split_tiles(fg, M, N, K, mode):
     compare_packed(fg, fg.linear_quantize(pa, pw, f.cuda(), scale_fp4=s4, score_mode=mode, tau=tau), q, tau, "hidden")
 
 
+# a tile of more than 256 tokens (two products on one dequantized operand), the last row of its second half, a ragged weight tile
+@pytest.mark.parametrize("M,N", [(289, 8200), (416, 8256)])
+def test_gemm_on_packed_weights_wide_tiles(fg, M, N):
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("wd", M, N, 5184, seed=68), 0.1, 0.1, clip=False)
+    y16 = fg.linear(pa, pw, out_dtype=torch.bfloat16)
+    y = fg.linear(pa, pw).cpu().numpy().astype(np.float64)
+    fg.check(fg.linear.last_workspace)
+    rng = np.random.default_rng(0)
+    ms, nn = np.r_[rng.integers(0, M, 4000), [M - 1, M - 1, 0]], np.r_[rng.integers(0, N, 4000), [N - 1, 0, N - 1]]
+    Y, S = oracle.linear_sampled(qa, qw, ms, nn)
+    assert (np.abs(y[ms, nn] - Y) <= 1e-5 * S + 1e-30).all() and np.isfinite(y).all()
+    if N % 64 == 0:
+        f = torch.ones(N)
+        s4 = gi.tensor_scale(y16.float().cpu())
+        q = oracle.quantize_activations(gi.bf16_bits(y16.cpu()), f.numpy(), s4, tau=s4 * s4)
+        compare_packed(fg, fg.linear_quantize(pa, pw, f.cuda(), scale_fp4=s4, tau=s4 * s4), q, s4 * s4, "hidden")
+
+
 # large batch: both operands expanded to fp16 planes, ragged in every direction
 @pytest.mark.parametrize("frac_a,frac_w", [(0.1, 0.1), (0.0, 1.0)])
 def test_gemm_on_expanded_planes_ragged(fg, frac_a, frac_w):
