@@ -5,7 +5,7 @@
 // thread per column, so the 16 per-channel Fisher weights stay in registers; the next row is loaded while one is worked on.
 //
 // Bound by instruction issue from a few hundred rows on (rounding to both formats and back, the score in element order), by the launch
-// below that.  2048 x 5120 takes 10.8 us (2.7 TB/s) and 8192 x 8192 43 us; with blocks of 256 columns
+// below that.  2048 x 5120 takes 10.4 us (2.8 TB/s) and 8192 x 8192 41.5 us; with blocks of 256 columns
 // and one load at a time it was 16.5 and 45 us.  Asking for more resident warps (64 registers) is slower, 13.8 us for the former.
 #include "fgmp_common.cuh"
 #include "fgmp_host.h"

@@ -114,16 +114,17 @@ template <bool BOUND>
 __device__ __forceinline__ float clip_error(const float (&v)[16], const float (&f)[16], float2 dd, float& clipped)
 {
     const float d = dd.x, inv = dd.y, d6 = __fmul_rn(6.0f, d);
+    const uint64_t d2 = f32x2_pack(d, d), inv2 = f32x2_pack(inv, inv);
     float j = 0.f, top = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
-        const float2 q = round_e2m1x2(__fmul_rn(v[i], inv), __fmul_rn(v[i + 1], inv));
-        const float e0 = __fsub_rn(__fmul_rn(q.x, d), v[i]), t0 = __fmul_rn(__fmul_rn(f[i], e0), e0);
-        const float e1 = __fsub_rn(__fmul_rn(q.y, d), v[i + 1]), t1 = __fmul_rn(__fmul_rn(f[i + 1], e1), e1);
-        j = __fadd_rn(__fadd_rn(j, t0), t1);
+        const float2 y = f32x2_unpack(f32x2_mul(f32x2_pack(v[i], v[i + 1]), inv2)), q = round_e2m1x2(y.x, y.y);
+        const uint64_t e = f32x2_sub(f32x2_mul(f32x2_pack(q.x, q.y), d2), f32x2_pack(v[i], v[i + 1]));
+        const float2 t = f32x2_unpack(f32x2_mul(f32x2_mul(f32x2_pack(f[i], f[i + 1]), e), e));
+        j = __fadd_rn(__fadd_rn(j, t.x), t.y);
         if (BOUND) {
-            top = fmaxf(top, fabsf(v[i]) >= d6 ? t0 : 0.f);
-            top = fmaxf(top, fabsf(v[i + 1]) >= d6 ? t1 : 0.f);
+            top = fmaxf(top, fabsf(v[i]) >= d6 ? t.x : 0.f);
+            top = fmaxf(top, fabsf(v[i + 1]) >= d6 ? t.y : 0.f);
         }
     }
     if (BOUND) clipped = top;
@@ -136,8 +137,8 @@ __device__ __forceinline__ float clip_error(const float (&v)[16], const float (&
 // code.  It need not look at all of them: going down from the dynamic-max code, an element that is clipped has an error that
 // only grows (every rounding step is monotone), and a sum of non-negative terms is never below one of them, so once such a
 // term alone exceeds the least error found no smaller scale can win.  Going up there are few codes left, because the tensor
-// scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left (25 for the longest of a warp): 4096 x 4096 takes 185 us, 680
-// before.
+// scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left (25 for the longest of a warp): 4096 x 4096 takes 152 us,
+// 172 without packed fp32 instructions, 680 with all 126.
 template <int MODE, bool CLIP>
 __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ldw8, const float* F, int64_t ldf,
                                                       int64_t N, int64_t KB, int ratio, float s8_given, const SelectState* st,
