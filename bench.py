@@ -468,7 +468,7 @@ def run_ours(args, world, rank, local):
         "config": {"workload": args.workload, "M": M, "N": N, "K": K, "fp8_fraction_weights": p,
                    "fp8_fraction_activations": p, "score_mode": "lp_error(Eq.6)", "clip": "sw_brute(Eq.11)",
                    "l2": f"rotating {wk.n_copies} packed weight copies ({wk.n_copies * wk.wbytes / 1e6:.0f} MB > 126 MB L2)"
-                   if kind == "decode" else "operands + bf16 planes exceed L2",
+                   if kind == "decode" else "operands + fp16 planes exceed L2",
                    "step": ("fgmp_linear_fused: activation quantizer + GEMM in one launch" if kind == "decode"
                             else "quantize_activations + linear (online path)") + "; weight packing is offline",
                    "launch": graph_note,

@@ -184,23 +184,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// shared-memory descriptor of a 32-row x 16-byte block-scale tile without swizzle
-// (rows 16 bytes apart, 8-row groups 128 bytes apart)
-__device__ __forceinline__ uint64_t smem_desc_sf(uint32_t saddr)
-{
-    uint64_t d = (uint64_t)((saddr & 0x3ffff) >> 4);
-    d |= (uint64_t)(128 >> 4) << 16;        // leading byte offset (single 16-byte column: unused)
-    d |= (uint64_t)(128 >> 4) << 32;        // stride byte offset between 8-row groups
-    d |= (uint64_t)1 << 46;                 // descriptor version for sm_100
-    return d;                               // layout type 0: no swizzle
-}
-
-// shared -> TMEM copy of one 32x16-byte scale tile, replicated to the four lane quadrants
-__device__ __forceinline__ void tmem_cp_sf(uint32_t taddr, uint64_t sdesc)
-{
-    asm volatile("tcgen05.cp.cta_group::1.32x128b.warpx4 [%0], %1;" ::"r"(taddr), "l"(sdesc) : "memory");
-}
-
 // D[tmem] (+)= A[smem] * B[smem], E2M1 operands with one UE4M3 scale per 16 elements
 __device__ __forceinline__ void umma_nvf4(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                           uint32_t sfa_tmem, uint32_t sfb_tmem, uint32_t accumulate)
@@ -210,18 +193,7 @@ __device__ __forceinline__ void umma_nvf4(uint32_t d_tmem, uint64_t adesc, uint6
                  ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate), "r"(sfa_tmem), "r"(sfb_tmem) : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-
-// the same without the wait: tmem_wait_ld names the registers, so that nothing reads them before it
+// Sixteen columns, without the wait: tmem_wait_ld names the registers, so that nothing reads them before it
 __device__ __forceinline__ void tmem_ld16_async(uint32_t taddr, uint32_t (&r)[16])
 {
     asm volatile(
@@ -270,14 +242,6 @@ __device__ __forceinline__ uint2 lds64_if(uint32_t saddr, bool want)
     return v;
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ void mma_f16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                              uint32_t b0, uint32_t b1)
-{
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
 
 // ---------------------------------------------------------------- CTA pairs (cluster of two, tcgen05 cta_group::2)
 __device__ __forceinline__ uint32_t cluster_ctarank()
