@@ -57,6 +57,7 @@ struct MixedPlan {
     uint32_t n_half;                     // tokens of one MMA: n_tok, or the first half (rounded up to 16) of a tile of more than 256
     uint32_t chunks, tiles;              // tiles = wtiles * tok_tiles
     uint32_t grid, span, rest, quantum;  // a CTA's span in quanta of `quantum` units (1, or chunks: whole tiles)
+    uint32_t split;                      // 1: some tile is shared by several CTAs, whose parts are added up behind this kernel
     uint32_t wstages, bstages, slots, naccs, max_parts;
     double us;                           // modelled time
 };
@@ -472,9 +473,11 @@ __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const _
     const uint32_t C = pl.chunks, NP = (pl.n_tok + 31u) & ~31u;
     const uint32_t tile = blockIdx.x, t_begin = tile * C, wt = tile / pl.tok_tiles;
     const uint32_t c_first = cta_of(pl, t_begin), nseg = cta_of(pl, t_begin + C - 1) - c_first + 1;
+    // Every block waits, those without anything to add up too: this grid lets its dependents start early, and what they wait for
+    // is its end, which must not come before the end of the kernel that wrote the other tiles and reads the workspace.
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    if (nseg == 1) return;                               // written by the CTA that has it
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (nseg == 1) return;                               // written by the CTA that has it
     if (p.status[0] != 0) return;
     const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
     if (p.leave_nvfp4 && hw->n_fp8 == 0 && p.ha->n_fp8 == 0) return;
@@ -564,6 +567,9 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
             const uint64_t quanta = total / pl.quantum;
             pl.grid = (uint32_t)(quanta < sms ? quanta : sms);
             pl.span = (uint32_t)(quanta / pl.grid); pl.rest = (uint32_t)(quanta % pl.grid);
+            // equal spans that are whole tiles after all are the other way of cutting, which needs no second kernel
+            pl.split = split;
+            if (split && pl.rest == 0 && pl.span % chunks == 0) continue;
             const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / chunks;
             // (beyond 256 tokens only spans within one tile pay: where a CTA goes on to another one its three slots and three
             // token stages run empty as well)
@@ -574,7 +580,7 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
             if (pl.us < best.us) best = pl;
         }
     }
-    best.max_parts = best.quantum == 1 ? best.grid * 2 : 0;
+    best.max_parts = best.split ? best.grid * 2 : 0;
     const uint32_t tmem_slots = (MX_TMEM_COLS - best.naccs * best.n_tok) / 32;
     best.slots = tmem_slots < (uint32_t)MAX_SLOTS ? tmem_slots : (uint32_t)MAX_SLOTS;
     // shared memory: two to four weight stages (a chunk each), the rest token stages
@@ -657,7 +663,7 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     cfg.dynamicSmemBytes = (size_t)p.pl.bstages * (p.pl.n_tok > p.pl.n_half ? 2 : 1) * p.pl.n_half * 128 + (size_t)p.pl.wstages * WSTAGE + MX_FIXED + (quant ? MX_TURN : 0);
     if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<true>, tmB, p)); }
     else       { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<false>, tmB, p)); }
-    if (p.pl.quantum == 1) {
+    if (p.pl.split) {
         cfg.gridDim = dim3(p.pl.tiles, (p.pl.n_tok + 31) / 32); cfg.dynamicSmemBytes = 0;
         cfg.blockDim = dim3(quant ? 128 : 256);
         if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_REDUCE, s, cudaLaunchKernelEx(&cfg, mixed_reduce_kernel<true>, p)); }

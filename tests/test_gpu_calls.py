@@ -1,0 +1,70 @@
+"""GPU tests of calls behind one another: on one stream without a synchronisation between them, on one workspace, on buffers that
+are used again, with what an earlier call has left there.  Inputs are drawn on the GPU; what a call returns by itself is the
+reference of what it returns among others."""
+import pytest
+import torch
+
+from test_gpu_parity import fg   # noqa: F401  (a fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+def draw_acts(fg, M, K, seed, fp8=0.1, **kw):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    x = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16)
+    f = torch.rand(K, generator=g, device="cuda") + 0.5
+    s4 = float(x.abs().max()) / 2688.0
+    tau = float(fg.calibrate_tau(x, f, scale_fp4=s4, fp8_fraction=fp8))
+    return fg.quantize_activations(x, f, scale_fp4=s4, tau=tau, **kw)
+
+
+def draw_weights(fg, N, K, seed, fp8=0.1):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    w = (torch.randn(N, K, generator=g, device="cuda") * 0.02).to(torch.bfloat16)
+    return fg.quantize_weights(w, torch.rand(N, K, generator=g, device="cuda") + 0.5, clip_mode=0, fp8_fraction=fp8)
+
+
+def launches(fg, call):
+    fg.profile_begin()
+    call()
+    return {name: n for name, (n, _) in fg.profile_end().items()}
+
+
+# Tiles that one CTA has each: one chunk of K, and spans that are whole tiles (a weight tile per SM).  There is nothing to add up
+# behind the GEMM, and what follows it in the stream waits for the GEMM itself.
+@pytest.mark.parametrize("M,N,K", [(64, 256, 256), (32, 0, 3584)])
+def test_calls_in_a_row_where_no_tile_is_shared(fg, M, N, K):
+    N = N or 128 * torch.cuda.get_device_properties(0).multi_processor_count
+    w, acts = draw_weights(fg, N, K, 1), [draw_acts(fg, M, K, 2 + i) for i in range(4)]
+    ws = fg.alloc_workspace(fg.OP_LINEAR, M, N, K, torch.device("cuda"))
+    count = launches(fg, lambda: fg.linear(acts[0], w, workspace=ws))
+    assert count.get("gemm_mixed_tcgen05") == 1 and "gemm_reduce" not in count, count
+    alone = []
+    for a in acts:
+        alone.append(fg.linear(a, w, workspace=ws))
+        torch.cuda.synchronize()
+    for _ in range(10):
+        ys = [fg.linear(a, w, workspace=ws) for a in acts]
+        for y, y0 in zip(ys, alone):
+            assert torch.equal(y, y0)
+    fg.check(ws)
+
+
+@pytest.mark.parametrize("N,K", [(512, 256), (1024, 1024)])
+def test_linear_right_behind_the_quantizing_one(fg, N, K):
+    M = 64
+    w, w2, acts = draw_weights(fg, N, K, 1), draw_weights(fg, 320, N, 2), [draw_acts(fg, M, K, 3 + i) for i in range(4)]
+    f = torch.ones(N, device="cuda")
+    ws = fg.alloc_workspace(fg.OP_LINEAR_QUANTIZE, M, max(N, 320), max(N, K), torch.device("cuda"))
+    hidden = lambda a: fg.linear_quantize(a, w, f, scale_fp4=1e-3, tau=1e-4, workspace=ws)   # noqa: E731
+    alone = []
+    for a in acts:
+        h = hidden(a)
+        torch.cuda.synchronize()
+        alone.append(fg.linear(h, w2, workspace=ws))
+        torch.cuda.synchronize()
+    for _ in range(10):
+        ys = [fg.linear(hidden(a), w2, workspace=ws) for a in acts]
+        for y, y0 in zip(ys, alone):
+            assert torch.equal(y, y0)
+    fg.check(ws)
