@@ -478,6 +478,10 @@ decode_kernel(const __grid_constant__ DecParams p)
         uint32_t stage = set, phase = 0, done = set, dphase = 0;      // done: stage of the set's last unit
         for (uint32_t i = set; i < n_units; i += 2) {
             const uint8_t* sb = smem + stage * p.stage_bytes;
+            // Barriers are waited for by parity, so the stage's unit before this one must be known to be in.  With three stages it is the other
+            // set's, and this set has seen unit i - 4 done at best (with more stages that is enough): its end comes first.
+            // (The copies of unit i begin behind that end, so the wait takes no time of its own.)
+            if (S == 3 && i >= 3 && !mbar_wait_warp(dn0 + 8 * stage, phase ^ 1u, abort_flag, p.status, 5)) break;
             if (!mbar_wait_warp(wf0 + 8 * stage, phase, abort_flag, p.status, 5)) break;
             if (!FUSED) {
                 // the unit's step record from the packed activation record (where a block with scale 0 is FP8, or all zero)

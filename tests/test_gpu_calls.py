@@ -68,3 +68,22 @@ def test_linear_right_behind_the_quantizing_one(fg, N, K):
         for y, y0 in zip(ys, alone):
             assert torch.equal(y, y0)
     fg.check(ws)
+
+
+# A CTA has more units than the decode kernel has stages, which is three with 14 to 16 packed tokens, four or more in a fused call:
+# the same sums either way, over and over, with the weights' copies out of L2 and out of HBM.
+@pytest.mark.parametrize("M", [9, 13, 14, 16])
+def test_decode_of_packed_tokens_equals_the_fused_step(fg, M):
+    N, K = 8192, 4096
+    g = torch.Generator(device="cuda").manual_seed(M)
+    x, f = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16), torch.rand(K, generator=g, device="cuda") + 0.5
+    s4 = float(x.abs().max()) / 2688.0
+    tau = float(fg.calibrate_tau(x, f, scale_fp4=s4, fp8_fraction=0.1))
+    acts = fg.quantize_activations(x, f, scale_fp4=s4, tau=tau)
+    for fp8 in (0.1, 0.3):
+        ws = [draw_weights(fg, N, K, 20 + i, fp8) for i in range(6)]
+        want = [fg.linear_fused(x, f, w, scale_fp4=s4, tau=tau) for w in ws]
+        torch.cuda.synchronize()
+        for _ in range(30):
+            for w, y in zip(ws, want):
+                assert torch.equal(fg.linear(acts, w), y)
