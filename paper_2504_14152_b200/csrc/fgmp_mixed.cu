@@ -589,6 +589,9 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
     while (best.wstages < (uint32_t)MAX_WSTAGES && room - (best.wstages + 1) * WSTAGE >= 10 * bst) ++best.wstages;
     best.bstages = (room - best.wstages * WSTAGE) / bst;
     if (best.bstages > (uint32_t)MAX_BSTAGES) best.bstages = MAX_BSTAGES;
+    // No more slots than token stages: a group that fills the slot of step i then knows step i - bstages done, so that the parity of its token
+    // stage's barrier can only mean step i (with more slots it could be taken in by a stage whose step before was still on its way).
+    if (best.slots > best.bstages) best.slots = best.bstages;
     return best;
 }
 

@@ -87,3 +87,16 @@ def test_decode_of_packed_tokens_equals_the_fused_step(fg, M):
         for _ in range(30):
             for w, y in zip(ws, want):
                 assert torch.equal(fg.linear(acts, w), y)
+
+
+# Token tiles of 224 to 384: fewer stages for the tokens than slots for the weights.  Against the GEMM over expanded planes; both sum
+# exact products in fp32 (K = 4096 terms in another order: about 1e-7 of the norm, a stale or early tile is of the order of one).
+@pytest.mark.parametrize("M", [224, 256, 277, 310, 340, 384])
+def test_gemm_on_packed_weights_with_few_token_stages(fg, M):
+    N, K = 11008, 4096
+    w, acts = draw_weights(fg, N, K, 30), draw_acts(fg, M, K, 31)
+    y0, ref = fg.linear(acts, w), fg.linear_classes(acts, w)
+    d = (y0 - ref).double()
+    assert d.norm() <= 1e-6 * ref.double().norm() and d.abs().max() <= 1e-5 * ref.double().pow(2).mean().sqrt()
+    for _ in range(30):
+        assert torch.equal(fg.linear(acts, w), y0)
