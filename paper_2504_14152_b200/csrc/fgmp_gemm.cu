@@ -47,16 +47,13 @@ __device__ __forceinline__ uint32_t pow2_f16x2(int e)
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// A packed tensor is read only if its header describes the tensor the call was given; otherwise the
-// status word of the workspace says so and the kernel leaves.
+// A packed tensor is read only if its header describes the tensor the call was given.
 // cls: 0 = every block on the NVFP4 tensor scale (needs the power-of-two tie of the two scales), 1 / 2 = only the
 // NVFP4 / only the FP8 blocks, each over its own tensor scale (the per-class passes of fgmp_linear_classes)
-__device__ __forceinline__ bool header_matches(const fgmp_packed_header* h, int64_t rows, int64_t K, uint32_t kind, int* status, int where, int cls = 0)
+__device__ __forceinline__ bool header_matches(const fgmp_packed_header* h, int64_t rows, int64_t K, uint32_t kind, int cls)
 {
-    const bool ok = h->magic == FGMP_MAGIC && h->version == FGMP_LAYOUT_VERSION && h->rows == rows && h->K == K && h->kind == kind && h->error == 0 &&
-                    (cls != 0 || h->fp8_scale_free == 0);
-    if (!ok && threadIdx.x == 0) { atomicCAS(status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(status + 1, where); }
-    return ok;
+    return h->magic == FGMP_MAGIC && h->version == FGMP_LAYOUT_VERSION && h->rows == rows && h->K == K && h->kind == kind && h->error == 0 &&
+           (cls != 0 || h->fp8_scale_free == 0);
 }
 
 // Whether the all-NVFP4 GEMM takes the call (decided alike by every kernel of it from the two headers)
@@ -83,10 +80,18 @@ __global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ Exp
     __shared__ UnitScratch sc;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
+    const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
+    // One thread says what the two headers are worth, whoever takes the call: a header that describes no tensor may also say that
+    // there is no FP8 block in it.
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const bool ok_a = header_matches(ha, p.M, p.K, 0u, p.cls_a), ok_w = header_matches(hw, p.N, p.K, 1u, p.cls_w);
+        if (!ok_a || !ok_w) { atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, ok_a ? 12 : 11); }
+    }
     if (p.leave_nvfp4 && no_fp8_block(p.ablob, p.wblob)) return;
     if (blockIdx.x >= p.w_blocks) {
-        const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
-        if (!header_matches(h, p.M, p.K, 0u, p.status, 11, p.cls_a)) return;
+        const fgmp_packed_header* h = ha;
+        if (!header_matches(h, p.M, p.K, 0u, p.cls_a)) return;
         const PackedLayout L = fgmp_layout(p.M, p.K, 0, 0);
         const uint32_t* pmask = reinterpret_cast<const uint32_t*>(p.ablob + L.off_mask);
         const uint32_t f8 = pow2_f16x2(p.cls_a ? 0 : h->fp8_log2_ratio), one = pow2_f16x2(0), KB = (uint32_t)L.KB;
@@ -126,8 +131,8 @@ __global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ Exp
         }
         return;
     }
-    const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
-    if (!header_matches(h, p.N, p.K, 1u, p.status, 12, p.cls_w)) return;
+    const fgmp_packed_header* h = hw;
+    if (!header_matches(h, p.N, p.K, 1u, p.cls_w)) return;
     const PackedLayout L = fgmp_layout(p.N, p.K, 1, 0);
     const int t = p.cls_w ? 0 : fgmp_weight_exponent(h);
     const uint32_t f4 = pow2_f16x2(-t), f8 = pow2_f16x2(p.cls_w ? 0 : h->fp8_log2_ratio - t);

@@ -100,3 +100,27 @@ def test_gemm_on_packed_weights_with_few_token_stages(fg, M):
     assert d.norm() <= 1e-6 * ref.double().norm() and d.abs().max() <= 1e-5 * ref.double().pow(2).mean().sqrt()
     for _ in range(30):
         assert torch.equal(fg.linear(acts, w), y0)
+
+
+# A blob that is not the tensor of the call is reported, also where its header says that it has no FP8 block: on the GEMM over
+# expanded planes and on the one over packed weights, for either operand, and for a blob without any header.
+@pytest.mark.parametrize("M,N,K,kernel", [(2048, 4096, 4096, "gemm_f16_tcgen05"), (64, 512, 576, "gemm_mixed_tcgen05")])
+@pytest.mark.parametrize("which", ["acts", "weights"])
+@pytest.mark.parametrize("what", ["other shape", "zeros"])
+def test_foreign_blob_without_fp8_blocks_is_reported(fg, M, N, K, kernel, which, what):
+    acts, w = draw_acts(fg, M, K, 40, fp8=0.0), draw_weights(fg, N, K, 41, fp8=0.0)
+    bad = acts if which == "acts" else w
+    blob = fg.binding._alloc_aligned(bad.blob.numel(), bad.blob.device).zero_()
+    if what == "other shape":
+        part = draw_acts(fg, M // 2, K, 42, fp8=0.0) if which == "acts" else draw_weights(fg, N // 2, K, 42, fp8=0.0)
+        blob[:part.blob.numel()] = part.blob
+    bad = fg.PackedTensor(blob, bad.rows, K, bad.kind)
+    good = fg.PackedTensor(*((w.blob, N, K, 1) if which == "acts" else (acts.blob, M, K, 0)))
+    pair = (bad, good) if which == "acts" else (good, bad)
+    count = launches(fg, lambda: fg.linear(*pair))
+    assert count.get(kernel) == 1, count
+    with pytest.raises(fg.FgmpError) as e:
+        fg.check(fg.linear.last_workspace)
+    assert e.value.code == -1
+    assert torch.isfinite(fg.linear(acts, w)).all()
+    fg.check(fg.linear.last_workspace)
