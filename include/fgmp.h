@@ -316,7 +316,8 @@ fgmp_status fgmp_linear_static(const void* packed_acts, const void* packed_weigh
 
 /* Synchronizes the stream and returns the device-side status recorded in a workspace used
  * by fgmp_linear (FGMP_OK, FGMP_ERR_TIMEOUT, or FGMP_ERR_INVALID_ARG for a packed tensor whose
- * header does not match the call). */
+ * header does not match the call).  A call of prefill size (M > 16 or K % 256 != 0) starts the status anew, so that
+ * it speaks of that call; decode-sized calls leave an earlier error in place. */
 fgmp_status fgmp_check(const void* workspace, void* cuda_stream);
 
 /* ---- parity support: packed -> canonical arrays (device) ----

@@ -73,6 +73,7 @@ struct ExpandParams {
     uint8_t* planeA; uint8_t* planeW;
     int* status;
     int cls_a, cls_w, leave_nvfp4;
+    int first;                           // the first kernel of a call: the status starts anew, whatever was in it
     uint32_t w_blocks;                   // thread blocks for the weights
 };
 __global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ ExpandParams p)
@@ -86,7 +87,8 @@ __global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ Exp
     // there is no FP8 block in it.
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         const bool ok_a = header_matches(ha, p.M, p.K, 0u, p.cls_a), ok_w = header_matches(hw, p.N, p.K, 1u, p.cls_w);
-        if (!ok_a || !ok_w) { atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, ok_a ? 12 : 11); }
+        if (p.first) { p.status[0] = ok_a && ok_w ? 0 : (int)FGMP_ERR_INVALID_ARG; p.status[1] = ok_a ? (ok_w ? 0 : 12) : 11; }
+        else if (!ok_a || !ok_w) { atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, ok_a ? 12 : 11); }
     }
     if (p.leave_nvfp4 && no_fp8_block(p.ablob, p.wblob)) return;
     if (blockIdx.x >= p.w_blocks) {
@@ -497,12 +499,12 @@ static fgmp_status resident_pairs(int* pairs)
 
 // expand both operands and run the pair GEMM (M > 16 or a shape the weight-streaming kernel does not take)
 fgmp_status fgmp_expand(const void* packed_acts, const void* packed_weights, int64_t M, int64_t N, int64_t K, uint8_t* planeA, uint8_t* planeW,
-                        int* status, int cls_a, int cls_w, bool leave_nvfp4, cudaStream_t s)
+                        int* status, int cls_a, int cls_w, bool leave_nvfp4, bool first, cudaStream_t s)
 {
     ExpandParams p;
     p.ablob = (const uint8_t*)packed_acts; p.wblob = (const uint8_t*)packed_weights;
     p.M = M; p.N = N; p.K = K; p.planeA = planeA; p.planeW = planeW; p.status = status;
-    p.cls_a = cls_a; p.cls_w = cls_w; p.leave_nvfp4 = leave_nvfp4 ? 1 : 0;
+    p.cls_a = cls_a; p.cls_w = cls_w; p.leave_nvfp4 = leave_nvfp4 ? 1 : 0; p.first = first ? 1 : 0;
     p.w_blocks = planeW ? (uint32_t)fgmp_layout(N, K, 1, 0).units : 0u;
     const int64_t nblk = planeA ? M * (K / 16) : 0;
     cudaLaunchAttribute attr[1];
@@ -563,7 +565,7 @@ static fgmp_status launch_prefill(const void* packed_acts, const void* packed_we
     } else {
         uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;   // the control area stays as the decode-sized calls need it
         uint8_t* planeW = planeA + fgmp_align1k((size_t)M * K * 2);
-        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, planeA, planeW, status, 0, 0, leave, s)) != FGMP_OK) return st;
+        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, planeA, planeW, status, 0, 0, leave, true, s)) != FGMP_OK) return st;
         GemmParams p{};
         p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K;
         p.ha = reinterpret_cast<const fgmp_packed_header*>(packed_acts);
@@ -637,7 +639,7 @@ extern "C" fgmp_status fgmp_linear_classes(const void* packed_acts, const void* 
     int have_a = 0, have_w = 0;
     for (int i = 0; i < 4; ++i) {
         const int ca = order[i][0], cw = order[i][1];
-        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, ca != have_a ? planeA : nullptr, cw != have_w ? planeW : nullptr, status, ca, cw, false, s)) != FGMP_OK)
+        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, ca != have_a ? planeA : nullptr, cw != have_w ? planeW : nullptr, status, ca, cw, false, false, s)) != FGMP_OK)
             return st;
         have_a = ca; have_w = cw;
         p.cls_a = ca; p.cls_w = cw; p.accumulate = i > 0;

@@ -143,10 +143,13 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     // operands with FP8 blocks (or headers that do not match the call) are left to the general path
     if (!g4_applicable(p)) {
-        if (p.sole && blockIdx.x == 0 && threadIdx.x == 0) { p.status[2] = 0; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, 13); }
+        if (p.sole && blockIdx.x == 0 && threadIdx.x == 0) { p.status[0] = (int)FGMP_ERR_INVALID_ARG; p.status[1] = 13; p.status[2] = 0; }
         return;
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) p.status[2] = 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (p.sole) { p.status[0] = 0; p.status[1] = 0; }                   // the status of the call starts here
+        p.status[2] = 1;
+    }
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);

@@ -28,9 +28,10 @@ fgmp_status fgmp_linear_decode(const void* packed_acts, const void* packed_weigh
 fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                                    int64_t M, int64_t N, int64_t K, int* status, bool sole, cudaStream_t s);
 
-// packed operands -> fp16 planes (planeW may be null: the activations only); cls_*: see fgmp_linear_classes
+// packed operands -> fp16 planes (planeW may be null: the activations only); cls_*: see fgmp_linear_classes; first: the call's status
+// starts with this kernel
 fgmp_status fgmp_expand(const void* packed_acts, const void* packed_weights, int64_t M, int64_t N, int64_t K, uint8_t* planeA, uint8_t* planeW,
-                        int* status, int cls_a, int cls_w, bool leave_nvfp4, cudaStream_t s);
+                        int* status, int cls_a, int cls_w, bool leave_nvfp4, bool first, cudaStream_t s);
 
 // GEMM on the packed weights (fgmp_mixed.cu), and its modelled time
 struct QuantNext;

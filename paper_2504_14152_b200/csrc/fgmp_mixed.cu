@@ -659,7 +659,7 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
-    const fgmp_status st = fgmp_expand(packed_acts, packed_weights, M, N, K, plane, nullptr, p.status, 0, 0, leave_nvfp4, s);
+    const fgmp_status st = fgmp_expand(packed_acts, packed_weights, M, N, K, plane, nullptr, p.status, 0, 0, leave_nvfp4, true, s);
     if (st != FGMP_OK) return st;
     const bool quant = qn.codes4 != nullptr;
     cfg.gridDim = dim3(p.pl.grid); cfg.blockDim = dim3(MX_THREADS);

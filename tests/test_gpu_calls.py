@@ -124,3 +124,21 @@ def test_foreign_blob_without_fp8_blocks_is_reported(fg, M, N, K, kernel, which,
     assert e.value.code == -1
     assert torch.isfinite(fg.linear(acts, w)).all()
     fg.check(fg.linear.last_workspace)
+
+
+# What an earlier call left in the status words -- an error, or anything where nothing had been there -- says nothing about this call.
+@pytest.mark.parametrize("M,N,K,fp8", [(2048, 4096, 4096, 0.1), (100, 1000, 1088, 0.1), (100, 1000, 1088, 0.0)])
+def test_prefill_call_starts_its_status_anew(fg, M, N, K, fp8):
+    acts, w = draw_acts(fg, M, K, 50, fp8), draw_weights(fg, N, K, 51, fp8)
+    ws = fg.alloc_workspace(fg.OP_LINEAR, M, N, K, torch.device("cuda"))
+    y0 = fg.linear(acts, w, workspace=ws)
+    fg.check(ws)
+    blob = fg.binding._alloc_aligned(w.blob.numel(), w.blob.device).zero_()
+    fg.linear(acts, fg.PackedTensor(blob, N, K, 1), workspace=ws)
+    with pytest.raises(fg.FgmpError):
+        fg.check(ws)
+    assert torch.equal(fg.linear(acts, w, workspace=ws), y0)
+    fg.check(ws)
+    ws[:256] = 0x5a
+    assert torch.equal(fg.linear(acts, w, workspace=ws), y0)
+    fg.check(ws)
