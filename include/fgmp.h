@@ -232,6 +232,14 @@ fgmp_status fgmp_linear(const void* packed_acts, const void* packed_weights,
                         void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
                         void* workspace, size_t ws_bytes, void* cuda_stream);
 
+/* fgmp_linear for a caller that expects something of the operands: nvfp4 = 1 no FP8 block in either, 0 some in one of them, -1
+ * nothing.  Which products are made does not depend on it (what is in the blobs is read from their headers when the kernels run), the
+ * order of their fp32 sums may; at prefill sizes the way that fits the expectation comes first, and the launches of the other
+ * follow it, look and leave. */
+fgmp_status fgmp_linear_expect(const void* packed_acts, const void* packed_weights,
+                               void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
+                               void* workspace, size_t ws_bytes, int nvfp4, void* cuda_stream);
+
 /* ---- the same GEMM with one accumulation per class of block pair (Section 4.1: the four dot-product
  * units; Section 5.1: FP8 blocks under a per-tensor scale of their own) ----
  * For operands whose FP8 tensor scale is not tied to the NVFP4 one by a power of two (fgmp_scales.scale_fp8 > 0

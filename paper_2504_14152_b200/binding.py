@@ -180,7 +180,7 @@ class PackedTensor:
     K: int
     kind: int               # 0 activations, 1 weights
     fp8_free: bool = False  # packed with an FP8 tensor scale of its own (scale_fp8 > 0): multiplied by linear_classes
-    nvfp4: bool | None = None   # no FP8 block in it (True), some or not excluded by the header (False), not known here (None)
+    nvfp4: bool | None = None   # expected to hold no FP8 block (True) or some (False); decides the order of launches, not the result
 
     def header(self) -> dict:
         h = self.blob[:128].cpu().numpy().tobytes()
@@ -303,9 +303,9 @@ def linear(acts: PackedTensor, weights: PackedTensor, *, out_dtype=torch.float32
         return linear_classes(acts, weights, out=out, workspace=workspace)
     assert (out_dtype if out is None else out.dtype) in (torch.float32, torch.bfloat16)
     a4, w4 = acts.nvfp4, weights.nvfp4
-    known = 0 if a4 is False or w4 is False else 1 if a4 and w4 else -1
+    expect = 0 if a4 is False or w4 is False else 1 if a4 and w4 else -1
     y, ws = (_ext or _load_ext()).linear(acts.blob, weights.blob, acts.rows, weights.rows, acts.K, out,
-                                         out_dtype is torch.bfloat16, workspace, known)
+                                         out_dtype is torch.bfloat16, workspace, expect)
     if ws.__class__ is str:
         raise _failed((y, ws))
     linear.last_workspace = ws

@@ -63,7 +63,7 @@ __device__ __forceinline__ bool no_fp8_block(const uint8_t* ablob, const uint8_t
 }
 
 // Packed operands -> fp16 planes over their NVFP4 tensor scales (the weights over a further 2^t, see fgmp_weight_exponent), both
-// in one launch: the first blocks take a unit of the weights each (consecutive threads on consecutive blocks of a row, eight
+// in one launch: the first blocks of work are a unit of the weights each (consecutive threads on consecutive blocks of a row, eight
 // blocks per thread in flight), the others 512 blocks of the activations.  Bound by the stores (32 bytes per
 // block and lane): 4096 x 11008 weights and 4096 x 4096 activations together 32 us, 5.1 TB/s; as two kernels that went through
 // fp32 49 us.
@@ -74,31 +74,18 @@ struct ExpandParams {
     int* status;
     int cls_a, cls_w, leave_nvfp4;
     int first;                           // the first kernel of a call: the status starts anew, whatever was in it
-    uint32_t w_blocks;                   // thread blocks for the weights
+    uint32_t w_blocks, blocks;           // blocks of work for the weights, and for both
 };
-__global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ ExpandParams p)
+__device__ __forceinline__ void expand_block(const ExpandParams& p, UnitScratch& sc, uint32_t block)
 {
-    __shared__ UnitScratch sc;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
-    const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
-    // One thread says what the two headers are worth, whoever takes the call: a header that describes no tensor may also say that
-    // there is no FP8 block in it.
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        const bool ok_a = header_matches(ha, p.M, p.K, 0u, p.cls_a), ok_w = header_matches(hw, p.N, p.K, 1u, p.cls_w);
-        if (p.first) { p.status[0] = ok_a && ok_w ? 0 : (int)FGMP_ERR_INVALID_ARG; p.status[1] = ok_a ? (ok_w ? 0 : 12) : 11; }
-        else if (!ok_a || !ok_w) { atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, ok_a ? 12 : 11); }
-    }
-    if (p.leave_nvfp4 && no_fp8_block(p.ablob, p.wblob)) return;
-    if (blockIdx.x >= p.w_blocks) {
-        const fgmp_packed_header* h = ha;
+    if (block >= p.w_blocks) {
+        const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
         if (!header_matches(h, p.M, p.K, 0u, p.cls_a)) return;
         const PackedLayout L = fgmp_layout(p.M, p.K, 0, 0);
         const uint32_t* pmask = reinterpret_cast<const uint32_t*>(p.ablob + L.off_mask);
         const uint32_t f8 = pow2_f16x2(p.cls_a ? 0 : h->fp8_log2_ratio), one = pow2_f16x2(0), KB = (uint32_t)L.KB;
         // four blocks per thread, the loads of all of them before the first is converted
-        const uint64_t b0 = (uint64_t)(blockIdx.x - p.w_blocks) * 512 + threadIdx.x, nblk = (uint64_t)p.M * KB;
+        const uint64_t b0 = (uint64_t)(block - p.w_blocks) * 512 + threadIdx.x, nblk = (uint64_t)p.M * KB;
         uint32_t word[4], sf[4];
         uint2 c4[4];
         uint4 c8[4];
@@ -133,12 +120,12 @@ __global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ Exp
         }
         return;
     }
-    const fgmp_packed_header* h = hw;
+    const fgmp_packed_header* h = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
     if (!header_matches(h, p.N, p.K, 1u, p.cls_w)) return;
     const PackedLayout L = fgmp_layout(p.N, p.K, 1, 0);
     const int t = p.cls_w ? 0 : fgmp_weight_exponent(h);
     const uint32_t f4 = pow2_f16x2(-t), f8 = pow2_f16x2(p.cls_w ? 0 : h->fp8_log2_ratio - t);
-    const uint32_t unit = blockIdx.x, tile = unit / (uint32_t)L.chunks, c = unit % (uint32_t)L.chunks;
+    const uint32_t unit = block, tile = unit / (uint32_t)L.chunks, c = unit % (uint32_t)L.chunks;
     const uint8_t* rec = p.wblob + L.off_rec + (size_t)unit * REC_BYTES;
     const uint32_t j = threadIdx.x & 15, row0 = threadIdx.x >> 4;
     const int64_t kb = (int64_t)c * 16 + j;
@@ -184,6 +171,35 @@ __global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ Exp
             store_256(p.planeW + (size_t)(r * p.K + kb * 16) * 2, o);
         }
         if (i0 == 0) fetch(8);
+    }
+}
+
+// FEW: fewer thread blocks than blocks of work, for launches that hardly ever have anything to do (what leaving costs is the number of
+// thread blocks); the loop by itself makes the expansion of 4096 x 4096 twice 5 us slower.
+template <bool FEW>
+__global__ void __launch_bounds__(128) expand_kernel(const __grid_constant__ ExpandParams p)
+{
+    __shared__ UnitScratch sc;
+    // Behind the all-NVFP4 GEMM, where there is hardly ever anything to do, the pair GEMM may come up at once: it reads nothing before
+    // this grid has ended.  (The GEMM on packed weights reads those early: it comes up when what ran before this kernel is done.)
+    if (p.leave_nvfp4 && !p.first) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
+    const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
+    // One thread says what the two headers are worth, whoever takes the call: a header that describes no tensor may also say that
+    // there is no FP8 block in it.
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        const bool ok_a = header_matches(ha, p.M, p.K, 0u, p.cls_a), ok_w = header_matches(hw, p.N, p.K, 1u, p.cls_w);
+        if (p.first) { p.status[0] = ok_a && ok_w ? 0 : (int)FGMP_ERR_INVALID_ARG; p.status[1] = ok_a ? (ok_w ? 0 : 12) : 11; }
+        else if (!ok_a || !ok_w) { atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, ok_a ? 12 : 11); }
+    }
+    if (p.leave_nvfp4 && no_fp8_block(p.ablob, p.wblob)) return;
+    if (FEW) {
+#pragma unroll 1
+        for (uint32_t block = blockIdx.x; block < p.blocks; block += gridDim.x) expand_block(p, sc, block);
+    } else {
+        expand_block(p, sc, blockIdx.x);
     }
 }
 
@@ -512,8 +528,12 @@ fgmp_status fgmp_expand(const void* packed_acts, const void* packed_weights, int
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
-    cfg.gridDim = dim3(p.w_blocks + (unsigned)((nblk + 511) / 512)); cfg.blockDim = dim3(128);
-    FGMP_LAUNCH(planeW ? FGMP_K_EXPAND_W : FGMP_K_EXPAND_A, s, cudaLaunchKernelEx(&cfg, expand_kernel, p));
+    p.blocks = p.w_blocks + (uint32_t)((nblk + 511) / 512);
+    const uint32_t few = (uint32_t)fgmp_sm_count() * 4u;
+    const bool behind = leave_nvfp4 && !first && p.blocks > few;          // the all-NVFP4 GEMM has been launched before
+    cfg.gridDim = dim3(behind ? few : p.blocks); cfg.blockDim = dim3(128);
+    if (behind) { FGMP_LAUNCH(planeW ? FGMP_K_EXPAND_W : FGMP_K_EXPAND_A, s, cudaLaunchKernelEx(&cfg, expand_kernel<true>, p)); }
+    else        { FGMP_LAUNCH(planeW ? FGMP_K_EXPAND_W : FGMP_K_EXPAND_A, s, cudaLaunchKernelEx(&cfg, expand_kernel<false>, p)); }
     return fgmp_launch_status();
 }
 
@@ -544,28 +564,30 @@ static double planes_us(int64_t M, int64_t N, int64_t K)
     return 10.0 + 0.65e-6 * (double)(M + N) * (double)K + (double)((tiles + pairs - 1) / pairs) * (double)(K / 64) * 0.34;
 }
 
-// M > 16 or a shape the weight-streaming kernel does not take.  nvfp4: 1 no FP8 block in either operand, 0 some in one of
-// them, -1 not known.
+// M > 16 or a shape the weight-streaming kernel does not take.  nvfp4: what the caller expects of the operands, see fgmp_linear_expect.
 static fgmp_status launch_prefill(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                                   int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, int nvfp4, cudaStream_t s)
 {
     uint8_t* ws = (uint8_t*)workspace;
     int* status = reinterpret_cast<int*>(ws);
     // Operands without any FP8 block go through the NVFP4 tensor-core kind straight from the packed form.  Whether that is
-    // the case is written in the two headers: unless the caller knows, the kernels of both ways are launched and look
-    // themselves.  (With the next layer's quantizer in the epilogue there is the general way only.)
-    const bool plain = !qn.codes4, leave = plain && nvfp4 < 0;
-    if (plain && nvfp4 == 1) return fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, true, s);
+    // the case is written in the two headers when the kernels run (a blob may have been packed anew since its owner last knew, or the
+    // launches recorded in a graph): the kernels of both ways are launched and look themselves.  What the caller expects decides which
+    // come first, and an operand with FP8 blocks, which the general way takes in any case, saves the launch of the other.  (With the
+    // next layer's quantizer in the epilogue there is the general way only.)
+    const bool leave = !qn.codes4 && nvfp4 != 0, nvfp4_first = leave && nvfp4 == 1;
     fgmp_status st;
+    if (nvfp4_first && (st = fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, true, s)) != FGMP_OK) return st;
     // At small and middling batches the weights are dequantized inside the GEMM, once per token tile; with many token tiles a
     // plane that is expanded once is read faster than that (777 x 11008 x 4096: 86 against 105 us; 2048 x 4096 x 4096: 81
     // against 60).
-    if (fgmp_mixed_us(M, N, K) <= planes_us(M, N, K)) {
-        st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, qn, leave, s);
+    // (Behind the all-NVFP4 GEMM: the way of two launches, not three.)
+    if (!nvfp4_first && fgmp_mixed_us(M, N, K) <= planes_us(M, N, K)) {
+        st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, qn, leave, !nvfp4_first, s);
     } else {
         uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;   // the control area stays as the decode-sized calls need it
         uint8_t* planeW = planeA + fgmp_align1k((size_t)M * K * 2);
-        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, planeA, planeW, status, 0, 0, leave, true, s)) != FGMP_OK) return st;
+        if ((st = fgmp_expand(packed_acts, packed_weights, M, N, K, planeA, planeW, status, 0, 0, leave, !nvfp4_first, s)) != FGMP_OK) return st;
         GemmParams p{};
         p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K;
         p.ha = reinterpret_cast<const fgmp_packed_header*>(packed_acts);
@@ -573,15 +595,13 @@ static fgmp_status launch_prefill(const void* packed_acts, const void* packed_we
         p.status = status; p.q = qn; p.leave_nvfp4 = leave ? 1 : 0;
         st = launch_pair_gemm(p, planeA, planeW, s);
     }
-    if (st != FGMP_OK || !leave) return st;
+    if (st != FGMP_OK || !leave || nvfp4_first) return st;
     return fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, false, s);
 }
 
-// fgmp_linear for a caller that knows what is in the operands' headers: nvfp4 = 1 no FP8 block in either, 0 some in one of
-// them, -1 not known
-extern "C" fgmp_status fgmp_linear_known(const void* packed_acts, const void* packed_weights,
-                                         void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
-                                         void* workspace, size_t ws_bytes, int nvfp4, void* cuda_stream)
+extern "C" fgmp_status fgmp_linear_expect(const void* packed_acts, const void* packed_weights,
+                                          void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
+                                          void* workspace, size_t ws_bytes, int nvfp4, void* cuda_stream)
 {
     if (!packed_acts || !packed_weights || !Y || !workspace) return FGMP_ERR_INVALID_ARG;
     if (M < 1 || N < 1 || K < 64 || (K % 64) != 0 || ldy < N) return FGMP_ERR_SHAPE;
@@ -601,7 +621,7 @@ extern "C" fgmp_status fgmp_linear(const void* packed_acts, const void* packed_w
                                    void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
                                    void* workspace, size_t ws_bytes, void* cuda_stream)
 {
-    return fgmp_linear_known(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, -1, cuda_stream);
+    return fgmp_linear_expect(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, -1, cuda_stream);
 }
 
 size_t fgmp_ws_linear_classes(int64_t M, int64_t N, int64_t K)

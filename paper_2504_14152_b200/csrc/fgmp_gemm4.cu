@@ -66,7 +66,7 @@ struct Gemm4Params {
     PackedLayout LA, LW;
     void* Y; int64_t ldy; int y_is_bf16;
     int64_t M, N, K;
-    int sole;                             // nothing else takes the call if this kernel does not
+    int first;                            // the first kernel of the call: the status starts here
     int* status;                          // [0..1] device-side status, [2] 1 = this kernel has produced Y
 };
 
@@ -141,15 +141,14 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
 {
     using C = G4<PAIR>;
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // operands with FP8 blocks (or headers that do not match the call) are left to the general path
-    if (!g4_applicable(p)) {
-        if (p.sole && blockIdx.x == 0 && threadIdx.x == 0) { p.status[0] = (int)FGMP_ERR_INVALID_ARG; p.status[1] = 13; p.status[2] = 0; }
-        return;
-    }
+    const bool applies = g4_applicable(p);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        if (p.sole) { p.status[0] = 0; p.status[1] = 0; }                   // the status of the call starts here
-        p.status[2] = 1;
+        if (p.first) { p.status[0] = 0; p.status[1] = 0; }
+        if (applies) p.status[2] = 1;
     }
+    if (!applies) return;
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -345,10 +344,10 @@ int g4_pairs[64] = {};                 // CTA pairs that run at once
 
 }  // namespace
 
-// Launches the all-NVFP4 GEMM; it decides on the device (from the two headers) whether it applies and says so in
-// status[2], which the general path's kernels read.
+// Launches the all-NVFP4 GEMM; it decides on the device (from the two headers) whether it applies, as the general path's kernels
+// do, and says so in status[2].
 fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                                   int64_t M, int64_t N, int64_t K, int* status, bool sole, cudaStream_t s)
+                                   int64_t M, int64_t N, int64_t K, int* status, bool first, cudaStream_t s)
 {
     int dev = 0, pairs = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
@@ -379,7 +378,7 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     Gemm4Params p;
     p.ablob = (const uint8_t*)packed_acts; p.wblob = (const uint8_t*)packed_weights;
     p.LA = fgmp_layout(M, K, 0, 0); p.LW = fgmp_layout(N, K, 1, 0);
-    p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K; p.status = status; p.sole = sole ? 1 : 0;
+    p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K; p.status = status; p.first = first ? 1 : 0;
     // the activations' code plane: bytes [M, K/2] row-major, boxes of 128 rows x 128 bytes, swizzled on the way in
     CUtensorMap tmA;
     cuuint64_t dims[2] = {(cuuint64_t)(K / 2), (cuuint64_t)M};

@@ -23,10 +23,10 @@ size_t fgmp_ws_decode(int64_t M, int64_t N, int64_t K);
 fgmp_status fgmp_linear_decode(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                                int64_t M, int64_t N, int64_t K, void* workspace, bool clear_first, cudaStream_t s);
 
-// all-NVFP4 prefill GEMM (fgmp_gemm4.cu): looks on the device whether it applies, and says so in status[2]; sole: nothing else
-// takes the call if it does not
+// all-NVFP4 prefill GEMM (fgmp_gemm4.cu): looks on the device whether it applies, and says so in status[2]; first: the call's
+// status starts with this kernel
 fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                                   int64_t M, int64_t N, int64_t K, int* status, bool sole, cudaStream_t s);
+                                   int64_t M, int64_t N, int64_t K, int* status, bool first, cudaStream_t s);
 
 // packed operands -> fp16 planes (planeW may be null: the activations only); cls_*: see fgmp_linear_classes; first: the call's status
 // starts with this kernel
@@ -38,7 +38,7 @@ struct QuantNext;
 double fgmp_mixed_us(int64_t M, int64_t N, int64_t K);
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K);
 fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                              int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, cudaStream_t s);
+                              int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, bool first, cudaStream_t s);
 
 // ---- the FP8 tensor scale of a call (fgmp_scales): given on its own, or scale_fp4 * 2^ratio ----
 #include <math.h>

@@ -67,7 +67,7 @@ struct MixedParams {
     const fgmp_packed_header* ha;
     void* Y; int64_t ldy; int y_is_bf16;
     int64_t M, N, K;
-    int leave_nvfp4;                     // operands without any FP8 block are left to the all-NVFP4 GEMM, launched behind this kernel
+    int leave_nvfp4;                     // operands without any FP8 block are left to the all-NVFP4 GEMM, launched before or behind this kernel
     MixedPlan pl;
     int* status; float* parts;
     QuantNext q;
@@ -614,7 +614,7 @@ size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K)
 
 // expands the activations and multiplies; leave_nvfp4: unless neither operand has an FP8 block
 fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                              int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, cudaStream_t s)
+                              int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, bool first, cudaStream_t s)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
@@ -659,7 +659,7 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
-    const fgmp_status st = fgmp_expand(packed_acts, packed_weights, M, N, K, plane, nullptr, p.status, 0, 0, leave_nvfp4, true, s);
+    const fgmp_status st = fgmp_expand(packed_acts, packed_weights, M, N, K, plane, nullptr, p.status, 0, 0, leave_nvfp4, first, s);
     if (st != FGMP_OK) return st;
     const bool quant = qn.codes4 != nullptr;
     cfg.gridDim = dim3(p.pl.grid); cfg.blockDim = dim3(MX_THREADS);

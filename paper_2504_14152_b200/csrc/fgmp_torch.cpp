@@ -8,10 +8,6 @@
 #include <c10/cuda/CUDAStream.h>
 #include "fgmp.h"
 
-extern "C" fgmp_status fgmp_linear_known(const void* packed_acts, const void* packed_weights,
-                                         void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t N, int64_t K,
-                                         void* workspace, size_t ws_bytes, int nvfp4, void* cuda_stream);
-
 namespace {
 
 // The calls that can return a status raise it through here: the Python side turns the pair into its exception type.
@@ -95,7 +91,7 @@ PyObject* py_linear(PyObject*, PyObject* const* a, Py_ssize_t n)
     fgmp_status st = FGMP_OK;
     at::Tensor ws = workspace_for(a[7], FGMP_OP_LINEAR, M, N, K, acts.device(), s, &st);
     if (st != FGMP_OK) return fail(st, "fgmp_workspace_init");
-    st = fgmp_linear_known(acts.data_ptr(), w.data_ptr(), out.data_ptr(), out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0), M, N, K,
+    st = fgmp_linear_expect(acts.data_ptr(), w.data_ptr(), out.data_ptr(), out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0), M, N, K,
                      ws.data_ptr(), (size_t)ws.numel(), (int)as_int(a[8]), s);
     if (st != FGMP_OK) return fail(st, "fgmp_linear");
     PyObject* r = PyTuple_New(2);

@@ -142,3 +142,28 @@ def test_prefill_call_starts_its_status_anew(fg, M, N, K, fp8):
     ws[:256] = 0x5a
     assert torch.equal(fg.linear(acts, w, workspace=ws), y0)
     fg.check(ws)
+
+
+# A buffer that is packed anew, seen through the object of its first packing: what is in the buffer counts, not what was in it.  Also for a
+# recorded call that is replayed after the buffer has changed.  (Exact products in fp32 sums whose order may differ: see above.)
+@pytest.mark.parametrize("M,N,K", [(2048, 4096, 4096), (100, 1000, 1088)])
+def test_packed_buffer_that_is_filled_anew(fg, M, N, K):
+    w = draw_weights(fg, N, K, 60, fp8=0.0)
+    acts = draw_acts(fg, M, K, 61, fp8=0.0)
+    mixed = draw_acts(fg, M, K, 62, fp8=0.1)
+    want0, want1 = fg.linear(acts, w), fg.linear(mixed, w)
+    same = lambda y, y0: (y - y0).double().norm() <= 1e-6 * y0.double().norm()   # noqa: E731
+    ws = fg.alloc_workspace(fg.OP_LINEAR, M, N, K, torch.device("cuda"))
+    out, graph = torch.empty_like(want0), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        fg.linear(acts, w, out=out, workspace=ws)
+    graph.replay()
+    assert torch.equal(out, want0)
+    draw_acts(fg, M, K, 62, fp8=0.1, out=acts.blob)
+    assert same(fg.linear(acts, w, workspace=ws), want1)
+    out.zero_()
+    graph.replay()
+    assert same(out, want1)
+    fg.check(ws)
+    first = draw_acts(fg, M, K, 61, fp8=0.0, out=mixed.blob)      # and the other way round
+    assert torch.equal(fg.linear(first, w), want0) and same(fg.linear(mixed, w), want0)
