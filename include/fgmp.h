@@ -287,9 +287,8 @@ fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const float* fish
  * accumulator is scaled, rounded to bf16 and quantized in registers by the GEMM's epilogue.
  * packed_out is a packed activation tensor of M rows and N columns (N is the next layer's K; size from
  * fgmp_acts_bytes(M, N)); fisher_chan_next [N], sc_next, sm and tau_next are the arguments
- * fgmp_quantize_activations would get.  N % 64 == 0.  Decode-sized batches (the shapes that take the
- * weight-streaming kernel, whose threads hold output rows rather than token rows) run as the two
- * launches, with the bf16 outputs (at most 16 x N) passing through the workspace.
+ * fgmp_quantize_activations would get.  N % 64 == 0.  Batches of up to 16 tokens run as the two
+ * calls, with the bf16 outputs (at most 16 x N) passing through the workspace.
  * workspace: fgmp_workspace_bytes(FGMP_OP_LINEAR_QUANTIZE, M, N, K), cleared once like fgmp_linear's. */
 fgmp_status fgmp_linear_quantize(const void* packed_acts, const void* packed_weights,
                                  int64_t M, int64_t N, int64_t K,

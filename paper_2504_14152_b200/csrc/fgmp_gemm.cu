@@ -481,7 +481,7 @@ bool make_tmap_f16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, 
 
 size_t fgmp_ws_linear_quantize(int64_t M, int64_t N, int64_t K)
 {
-    return fgmp_ws_linear(M, N, K) + (fgmp_decode_supported(M, N, K) ? fgmp_align1k((size_t)M * N * 2) : 0);
+    return fgmp_ws_linear(M, N, K) + (M <= 16 ? fgmp_align1k((size_t)M * N * 2) : 0);
 }
 
 size_t fgmp_ws_linear(int64_t M, int64_t N, int64_t K)
@@ -683,17 +683,18 @@ extern "C" fgmp_status fgmp_linear_quantize(const void* packed_acts, const void*
     if (((uintptr_t)packed_acts & 1023) || ((uintptr_t)packed_weights & 1023) || ((uintptr_t)workspace & 1023) ||
         ((uintptr_t)packed_out & 1023) || ((uintptr_t)fisher_chan_next & 15)) return FGMP_ERR_SHAPE;
     if (ws_bytes < fgmp_ws_linear_quantize(M, N, K)) return FGMP_ERR_WORKSPACE;
-    if (fgmp_decode_supported(M, N, K)) {
-        // decode-sized batch: the weight-streaming kernel holds an output row per thread, not a token row, so the
-        // two steps stay two launches; the bf16 outputs (at most 16 x N) pass through the end of the workspace
+    const PackedLayout L = fgmp_layout(M, N, 0, 0);
+    if (packed_bytes < L.total) return FGMP_ERR_WORKSPACE;
+    if (M <= 16) {
+        // At most 16 tokens: the two steps stay two calls, the bf16 outputs (at most 16 x N) passing through the end of the workspace.  The
+        // weight-streaming kernel holds an output row per thread, not a token row, and a packed tensor of so few rows also has
+        // the records that kernel reads in the next layer, which the quantizer of a GEMM's epilogue does not write.
         uint8_t* ybf = (uint8_t*)workspace + fgmp_ws_linear(M, N, K);
         fgmp_status st2 = fgmp_linear(packed_acts, packed_weights, ybf, 1, N, M, N, K, workspace, fgmp_ws_linear(M, N, K), cuda_stream);
         if (st2 != FGMP_OK) return st2;
         return fgmp_quantize_activations(ybf, N, fisher_chan_next, M, N, sc_next, sm, tau_next, packed_out, packed_bytes,
                                          nullptr, 0, cuda_stream);
     }
-    const PackedLayout L = fgmp_layout(M, N, 0, 0);
-    if (packed_bytes < L.total) return FGMP_ERR_WORKSPACE;
     fgmp_status st;
     if ((st = fgmp_require_sm100()) != FGMP_OK) return st;
     uint8_t* blob = (uint8_t*)packed_out;

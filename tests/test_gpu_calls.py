@@ -167,3 +167,21 @@ def test_packed_buffer_that_is_filled_anew(fg, M, N, K):
     fg.check(ws)
     first = draw_acts(fg, M, K, 61, fp8=0.0, out=mixed.blob)      # and the other way round
     assert torch.equal(fg.linear(first, w), want0) and same(fg.linear(mixed, w), want0)
+
+
+# At most 16 tokens and a K that the weight-streaming kernel does not take, behind it a layer whose K it takes: the packed tensor between the
+# two has everything that a packed tensor of its shape has.
+@pytest.mark.parametrize("M,N,K", [(1, 256, 64), (8, 512, 320), (16, 1024, 576), (16, 512, 512)])
+def test_packed_tokens_between_two_layers(fg, M, N, K):
+    w, w2, acts = draw_weights(fg, N, K, 70), draw_weights(fg, 320, N, 71), draw_acts(fg, M, K, 72)
+    f, kw = torch.rand(N, generator=torch.Generator(device="cuda").manual_seed(73), device="cuda"), dict(scale_fp4=1e-3, tau=1e-4)
+    stale = fg.binding._alloc_aligned(fg.acts_bytes(M, N), "cuda").fill_(0xff)
+    del stale                                             # (what the call's own buffer may hold)
+    hidden = fg.linear_quantize(acts, w, f, **kw)
+    fg.check(fg.linear.last_workspace)
+    want = fg.quantize_activations(fg.linear(acts, w, out_dtype=torch.bfloat16), f, **kw)
+    for a, b in zip(fg.unpack(hidden), fg.unpack(want)):
+        assert torch.equal(a, b)
+    y, y0 = fg.linear(hidden, w2), fg.linear(want, w2)
+    fg.check(fg.linear.last_workspace)
+    assert torch.isfinite(y0).all() and torch.equal(y, y0)
