@@ -428,7 +428,7 @@ gemm_f16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(cluster_map(acce0 + 8 * acc, 0));
+            if (lane == 0) mbar_arrive_cluster_tmem(cluster_map(acce0 + 8 * acc, 0));
         }
     }
 

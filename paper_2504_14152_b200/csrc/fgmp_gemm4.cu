@@ -137,7 +137,7 @@ __device__ __forceinline__ bool g4_applicable(const Gemm4Params& p)
 
 template <bool PAIR>
 __global__ void __launch_bounds__(G4_THREADS, 1)
-gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
+gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, Gemm4Params p)
 {
     using C = G4<PAIR>;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -154,15 +154,17 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     constexpr int S = C::STAGES;
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * C::STAGE_BYTES);
-    // bars: [0,S) full, [S,2S) empty, [2S,3S) stage loaded and its scales in tensor memory (leader), then acc_full, acc_empty (leader)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 3 * S + 2);
+    // bars: [0,S) full, [S,2S) empty, [2S,3S) scales in tensor memory, [3S,4S) scales loaded, then acc_full, acc_empty.  Of a pair, the
+    // leader's "full" counts the codes of both CTAs, since its thread multiplies both; the scales are each CTA's own matter until they are in
+    // tensor memory, and "scales loaded" counts them.  A single CTA has its scales counted by "full".
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4 * S + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
     const int warp = warp_index(), lane = threadIdx.x & 31;
     const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
-    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * S, sfr0 = empty0 + 8 * S, accf = sfr0 + 8 * S, acce = accf + 8;
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * S, sfr0 = empty0 + 8 * S, sfl0 = PAIR ? sfr0 + 8 * S : full0, accf = sfr0 + 16 * S, acce = accf + 8;
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < S; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); mbar_init(sfr0 + 8 * s, PAIR ? 8 : 4); }
+        for (int s = 0; s < S; ++s) { mbar_init(full0 + 8 * s, 1); mbar_init(empty0 + 8 * s, 1); mbar_init(sfr0 + 8 * s, PAIR ? 8 : 4); if (PAIR) mbar_init(sfl0 + 8 * s, 1); }
         mbar_init(accf, 1); mbar_init(acce, PAIR ? 16 : 8);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -173,6 +175,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
     if (PAIR) cluster_sync();                           // the other CTA's barriers exist before anything signals them
     tc_fence_after();
     constexpr uint32_t tmem_base = TMEM_ALL;
+    static_assert(REC_W4 == 0 && REC_BYTES % 128 == 0, "records as rows of 128 bytes");
 
     const int64_t tiles_m = (p.M + C::TM - 1) / C::TM, wtiles = p.LW.tiles, tiles_n = (wtiles + 1) / 2;
     const int64_t num_tiles = tiles_m * tiles_n;
@@ -190,26 +193,33 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
                 const int64_t tm = t % tiles_m, tn = t / tiles_m;             // token tiles fastest: CTAs that run together share weights
                 const int64_t m0 = tm * C::TM + 128 * rank;
                 const bool two = 2 * tn + 1 < wtiles, rows = m0 < p.M;
-                const uint32_t wbytes = PAIR ? (two || rank == 0 ? 16384u : 0u) + (two ? 4096u : 2048u) : (two ? 2u : 1u) * (16384u + 2048u);
                 const uint8_t* r0 = recs + (size_t)(2 * tn * chunks) * REC_BYTES;
                 const uint8_t* r1 = r0 + (size_t)chunks * REC_BYTES;
                 const uint8_t* sfa = asf + (size_t)(m0 >> 7) * (size_t)ksteps_total * 512;
+                // what the two CTAs of a pair load: the leader's rows are always there
+                const uint32_t pair_codes = 16384u * (1u + (m0 + 128 < p.M ? 1u : 0u) + (two ? 2u : 1u));
+                const int32_t w_row = (int32_t)((2 * tn + rank) * chunks * (REC_BYTES / 128));      // a record is 145 rows of 128 bytes
                 for (int64_t c = 0; c < chunks; ++c, r0 += REC_BYTES, r1 += REC_BYTES, sfa += 2048) {
                     if (!(ok = mbar_wait(empty0 + 8 * stage, phase ^ 1, abort_flag, p.status, 1))) break;
                     const uint32_t ks = (uint32_t)min((int64_t)4, ksteps_total - 4 * c);
-                    const uint32_t fb = full0 + 8 * stage;
+                    const uint32_t fb = full0 + 8 * stage, sb = sfl0 + 8 * stage;
                     const uint32_t dst = smem_u32(smem + (size_t)stage * C::STAGE_BYTES);
-                    mbar_expect_tx(fb, (rows ? 16384u + ks * 512u : 0u) + wbytes);
-                    if (rows) {
-                        tma_load_2d(dst + C::A4, &tmA, (int32_t)(c * 128), (int32_t)m0, fb);
-                        bulk_load(dst + C::SFA, sfa, ks * 512u, fb);
+                    const uint32_t scales = (rows ? ks * 512u : 0u) + (two ? 4096u : 2048u);
+                    if (PAIR) {
+                        if (rank == 0) mbar_expect_tx(fb, pair_codes);
+                        mbar_expect_tx(sb, scales);
+                        const uint32_t leader = cluster_map(fb, 0);
+                        if (rows) tma_load_2d_pair(dst + C::A4, &tmA, (int32_t)(c * 128), (int32_t)m0, leader);
+                        if (rank == 0 || two) tma_load_2d_pair(dst + C::B0, &tmW, 0, w_row + (int32_t)c * (int32_t)(REC_BYTES / 128), leader);
+                    } else {
+                        mbar_expect_tx(fb, (rows ? 16384u : 0u) + (two ? 2u : 1u) * 16384u + scales);
+                        if (rows) tma_load_2d(dst + C::A4, &tmA, (int32_t)(c * 128), (int32_t)m0, fb);
+                        bulk_load(dst + C::B0, r0 + REC_W4, 16384, fb);
+                        if (two) bulk_load(dst + C::B1, r1 + REC_W4, 16384, fb);
                     }
-                    if (!PAIR || rank == 0) bulk_load(dst + C::B0, r0 + REC_W4, 16384, fb);
-                    bulk_load(dst + C::SFB, r0 + REC_SF, 2048, fb);
-                    if (two) {
-                        if (!PAIR || rank == 1) bulk_load(dst + (PAIR ? C::B0 : C::B1), r1 + REC_W4, 16384, fb);
-                        bulk_load(dst + C::SFB + 2048, r1 + REC_SF, 2048, fb);
-                    }
+                    if (rows) bulk_load(dst + C::SFA, sfa, ks * 512u, sb);
+                    bulk_load(dst + C::SFB, r0 + REC_SF, 2048, sb);
+                    if (two) bulk_load(dst + C::SFB + 2048, r1 + REC_SF, 2048, sb);
                     if (++stage == S) { stage = 0; phase ^= 1; }
                 }
             }
@@ -227,8 +237,9 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
                 tc_fence_after();
                 uint32_t accum = 0;
                 for (int64_t c = 0; c < chunks; ++c) {
-                    // (the scale warps arrive behind the stage's loads: theirs is the only signal to wait for)
+                    // (of a single CTA, the scale warps arrive behind the stage's loads: theirs is the only signal to wait for)
                     if (!(ok = mbar_wait(sfr0 + 8 * stage, phase, abort_flag, p.status, 3))) break;
+                    if (PAIR && !(ok = mbar_wait(full0 + 8 * stage, phase, abort_flag, p.status, 8))) break;
                     tc_fence_after();
                     const uint32_t ks = (uint32_t)min((int64_t)4, ksteps_total - 4 * c);
                     const uint32_t sb = smem0 + (uint32_t)stage * C::STAGE_BYTES;
@@ -255,7 +266,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
             const int64_t tm = t % tiles_m, tn = t / tiles_m;
             const bool two = 2 * tn + 1 < wtiles, rows = tm * C::TM + 128 * rank < p.M;
             for (int64_t c = 0; c < chunks; ++c) {
-                if (!(ok = mbar_wait_warp(full0 + 8 * stage, phase, abort_flag, p.status, 4))) break;
+                if (!(ok = mbar_wait_warp(sfl0 + 8 * stage, phase, abort_flag, p.status, 4))) break;
                 const uint32_t ks = rows ? (uint32_t)min((int64_t)4, ksteps_total - 4 * c) : 0u;
                 const uint8_t* sb = smem + (size_t)stage * C::STAGE_BYTES;
                 const uint32_t sf_t = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + G4_SF_COL0 + (uint32_t)stage * 48;
@@ -283,7 +294,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) { if (PAIR) mbar_arrive_cluster(ready0 + 8 * stage); else mbar_arrive(ready0 + 8 * stage); }
+                if (lane == 0) { if (PAIR) mbar_arrive_cluster_tmem(ready0 + 8 * stage); else mbar_arrive(ready0 + 8 * stage); }
                 if (++stage == S) { stage = 0; phase ^= 1; }
             }
         }
@@ -315,7 +326,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, Gemm4Params p)
             tmem_ld32(src + 96, r[0]);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) { if (PAIR) mbar_arrive_cluster(drained); else mbar_arrive(drained); }
+            if (lane == 0) { if (PAIR) mbar_arrive_cluster_tmem(drained); else mbar_arrive(drained); }
 #pragma unroll
             for (int c = 1; c < 4; ++c) g4_store(p, at + c * 32, r[c % 3], alpha, left - c * 32, wide);
         }
@@ -388,6 +399,13 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     if (g4_encode(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(p.ablob + p.LA.off_codes4), dims, strides, box, estr,
                   CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return FGMP_ERR_CUDA;
+    // pairs: the weights' records as rows of 128 bytes, boxes of a tile's 128 rows (swizzled already), whose loads may be counted in the leader
+    CUtensorMap tmW;
+    cuuint64_t dims_w[2] = {128, (cuuint64_t)(p.LW.units * (REC_BYTES / 128))};
+    cuuint64_t strides_w[1] = {128};
+    if (g4_encode(&tmW, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(p.wblob + p.LW.off_rec), dims_w, strides_w, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return FGMP_ERR_CUDA;
     const int64_t cols = (p.LW.tiles + 1) / 2, tiles = ((M + 127) / 128) * cols, tiles2 = ((M + 255) / 256) * cols;
     const int sms = fgmp_sm_count();
     // pairs where the tiles take more than one round of the machine (2048 x 13824 x 5120: 63 us, 70 on single CTAs; 777 x 11008 x 4096: 28.2,
@@ -405,7 +423,7 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(G4_THREADS); cfg.stream = s;
     cfg.dynamicSmemBytes = pair ? G4<true>::SMEM : G4<false>::SMEM;
     cfg.attrs = attr; cfg.numAttrs = pair ? 2 : 1;
-    if (pair) FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<true>, tmA, p));
-    else FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<false>, tmA, p));
+    if (pair) FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<true>, tmA, tmW, p));
+    else FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<false>, tmA, tmW, p));
     return fgmp_launch_status();
 }

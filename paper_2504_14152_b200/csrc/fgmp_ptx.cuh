@@ -262,11 +262,13 @@ __device__ __forceinline__ uint32_t cluster_map(uint32_t smem_addr, uint32_t ran
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr), "r"(rank));
     return r;
 }
-// arrive on an mbarrier given by its shared::cluster address (possibly in the other CTA).  (With .release.cluster spelled out
-// a warp spends about 1000 clocks here.)
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr)
+// Arrive on an mbarrier given by its shared::cluster address (possibly in the other CTA) with no order of its own: for handing over
+// tensor memory, between tcgen05.fence::before_thread_sync here and ::after_thread_sync there, which order the tcgen05 operations of both
+// sides.  It hands over nothing else -- in particular no shared memory.  (A warp spends about 1000 clocks on a release at
+// cluster scope: one for every stage makes the NVFP4 GEMM of 2048 x 13824 x 5120 take 160 us a call instead of 90.)
+__device__ __forceinline__ void mbar_arrive_cluster_tmem(uint32_t cluster_addr)
 {
-    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // TMA tile load of a CTA pair: data into this CTA's shared memory, bytes counted on the mbarrier at
 // the shared::cluster address `bar` (the pair's leader)

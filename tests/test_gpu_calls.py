@@ -185,3 +185,16 @@ def test_packed_tokens_between_two_layers(fg, M, N, K):
     y, y0 = fg.linear(hidden, w2), fg.linear(want, w2)
     fg.check(fg.linear.last_workspace)
     assert torch.isfinite(y0).all() and torch.equal(y, y0)
+
+
+# All-NVFP4 operands on CTA pairs: the codes of both CTAs counted in the leader, a last pair of tiles with one weight tile, a last tile with no
+# rows for the second CTA.  Against the GEMM over expanded planes, and the same every time.
+@pytest.mark.parametrize("M,N,K", [(777, 11008, 4096), (1100, 9857, 320), (640, 16512, 2112)])
+def test_nvfp4_gemm_on_pairs(fg, M, N, K):
+    w, acts = draw_weights(fg, N, K, 80, fp8=0.0), draw_acts(fg, M, K, 81, fp8=0.0)
+    y0, ref = fg.linear(acts, w), fg.linear_classes(acts, w)
+    fg.check(fg.linear.last_workspace)
+    d = (y0 - ref).double()
+    assert d.norm() <= 1e-6 * ref.double().norm() and d.abs().max() <= 1e-5 * ref.double().pow(2).mean().sqrt()
+    for _ in range(30):
+        assert torch.equal(fg.linear(acts, w), y0)
