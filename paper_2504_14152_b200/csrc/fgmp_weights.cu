@@ -100,6 +100,9 @@ __device__ __forceinline__ void load_block(const uint4* W, int64_t ldw8, const f
     }
 }
 
+// A tensor of zeros has the tensor scale zero: all its codes are zero then, instead of what 0 times infinity rounds to.
+__device__ __forceinline__ float inverse_scale(float s) { return s == 0.f ? 0.f : __fdiv_rn(1.0f, s); }
+
 // two values rounded to E2M1 and back
 __device__ __forceinline__ float2 round_e2m1x2(float lo, float hi)
 {
@@ -144,18 +147,20 @@ __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ld
                                                       int64_t N, int64_t KB, int ratio, float s8_given, const SelectState* st,
                                                       uint8_t* sc_out, float* scores)
 {
-    __shared__ float2 s_d[127];                          // scale and its inverse, by code
+    // scale and its inverse, by code; 127, NaN, is what a block gets whose largest magnitude over a tensor scale of infinity or NaN has
+    // no code (weights that are not finite): no scale is better than it
+    __shared__ float2 s_d[128];
     const float s4 = st->s4;
     if (CLIP) {
-        if (threadIdx.x < 127) {
+        if (threadIdx.x < 128) {
             const float d = __fmul_rn(e4m3_to_f32(threadIdx.x), s4);
             s_d[threadIdx.x] = make_float2(d, (d == 0.f) ? 0.f : __fdiv_rn(1.0f, d));
         }
         __syncthreads();
     }
-    const float k6 = __fdiv_rn(1.0f, __fmul_rn(6.0f, s4));
+    const float k6 = inverse_scale(__fmul_rn(6.0f, s4));
     const float s8 = s8_given > 0.f ? s8_given : __fmul_rn(s4, __int_as_float((127 + ratio) << 23));
-    const float inv8 = __fdiv_rn(1.0f, s8);
+    const float inv8 = inverse_scale(s8);
     const int64_t B = N * KB;
     for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < B; b += (int64_t)gridDim.x * blockDim.x) {
         float v[16], f[16];
@@ -419,7 +424,7 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
     const bool fits = reinterpret_cast<const fgmp_packed_header*>(blob)->error == 0;   // else the blob is too small for the lists
     const float s4 = st->s4;
     const float s8 = s8_given > 0.f ? s8_given : __fmul_rn(s4, __int_as_float((127 + ratio) << 23));
-    const float inv8 = __fdiv_rn(1.0f, s8);
+    const float inv8 = inverse_scale(s8);
     const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x]);
     uint8_t* rec = blob + L.off_rec + (size_t)unit * REC_BYTES;
     uint8_t* list = blob + L.off_ovf + (size_t)uptr[unit] * 16;

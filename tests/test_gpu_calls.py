@@ -1,10 +1,13 @@
 """GPU tests of calls behind one another: on one stream without a synchronisation between them, on one workspace, on buffers that
 are used again, with what an earlier call has left there.  Inputs are drawn on the GPU; what a call returns by itself is the
 reference of what it returns among others."""
+import numpy as np
 import pytest
 import torch
 
-from test_gpu_parity import fg   # noqa: F401  (a fixture)
+import fgmp_inputs as gi
+import oracle
+from test_gpu_parity import compare_packed, fg   # noqa: F401  (fg is a fixture)
 
 pytestmark = pytest.mark.gpu
 
@@ -198,3 +201,18 @@ def test_nvfp4_gemm_on_pairs(fg, M, N, K):
     assert d.norm() <= 1e-6 * ref.double().norm() and d.abs().max() <= 1e-5 * ref.double().pow(2).mean().sqrt()
     for _ in range(30):
         assert torch.equal(fg.linear(acts, w), y0)
+
+
+# A weight tensor of zeros: the derived tensor scale is zero, and so is every code.
+@pytest.mark.parametrize("clip", [0, 1])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_weights_of_zeros(fg, clip, mode):
+    N, K = 130, 320
+    w, f = torch.zeros(N, K, dtype=torch.bfloat16), torch.ones(N, K)
+    w[1, 3:9] = -0.0
+    for frac in (0.0, 0.1):
+        p = fg.quantize_weights(w.cuda(), f.cuda(), clip_mode=clip, score_mode=mode, fp8_fraction=frac)
+        if frac == 0.0:                       # (the sign of an E4M3 zero over a scale of zero is nobody's business)
+            compare_packed(fg, p, oracle.quantize_weights(gi.bf16_bits(w), f.numpy(), clip=bool(clip), mode=mode, fp8_fraction=frac), None, "zeros")
+        for M in (8, 40):
+            assert not fg.linear(draw_acts(fg, M, K, 90), p).any()
