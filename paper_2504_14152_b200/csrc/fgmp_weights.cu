@@ -139,7 +139,8 @@ __device__ __forceinline__ float clip_error(const float (&v)[16], const float (&
 // The search asks for the scale with the least error among all 126, ties to the dynamic-max scale and then to the smaller
 // code.  It need not look at all of them: going down from the dynamic-max code, an element that is clipped has an error that
 // only grows (every rounding step is monotone), and a sum of non-negative terms is never below one of them, so once such a
-// term alone exceeds the least error found no smaller scale can win.  Going up there are few codes left, because the tensor
+// term alone exceeds the least error found no smaller scale can win.  (Where a sensitivity is negative or NaN the terms are not what
+// this rests on, and all scales are looked at.)  Going up there are few codes left, because the tensor
 // scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left (25 for the longest of a warp): 4096 x 4096 takes 152 us,
 // 172 without packed fp32 instructions, 680 with all 126.
 template <int MODE, bool CLIP>
@@ -168,14 +169,17 @@ __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ld
         uint32_t sc = block_dynamic_scale(v, k6);
         if (CLIP) {
             const int dyn = (int)sc;
+            bool ordered = true;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) ordered &= f[i] >= 0.f;
             float clipped, best = clip_error<true>(v, f, s_d[dyn], clipped);
-            bool more = !(clipped > best);
+            bool more = !(ordered && clipped > best);
 #pragma unroll 1
             for (int c = dyn - 1; more && c >= 1; --c) {
                 const float j = clip_error<true>(v, f, s_d[c], clipped);
                 // going down, a tie is a smaller code: it wins unless the dynamic-max code holds the lead
                 if (j < best || (j == best && (int)sc != dyn)) { best = j; sc = (uint32_t)c; }
-                more = !(clipped > best);
+                more = !(ordered && clipped > best);
             }
 #pragma unroll 1
             for (int c = dyn + 1; c <= 0x7e; ++c) {

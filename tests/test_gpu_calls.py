@@ -216,3 +216,15 @@ def test_weights_of_zeros(fg, clip, mode):
             compare_packed(fg, p, oracle.quantize_weights(gi.bf16_bits(w), f.numpy(), clip=bool(clip), mode=mode, fp8_fraction=frac), None, "zeros")
         for M in (8, 40):
             assert not fg.linear(draw_acts(fg, M, K, 90), p).any()
+
+
+# Sensitivities that are not a mean of squares (some negative, some NaN): the search for the clipping scale still is the exhaustive one.
+def test_clip_search_with_any_sensitivity(fg):
+    N, K = 200, 448
+    g = torch.Generator().manual_seed(100)
+    w = (torch.randn(N, K, generator=g) * torch.exp(torch.randn(N, K, generator=g)) * 0.02).to(torch.bfloat16)
+    f = torch.randn(N, K, generator=g)
+    f[:50] = f[:50].abs()
+    f[60, 5::32] = float("nan")
+    q = oracle.quantize_weights(gi.bf16_bits(w), f.numpy(), clip=True, fp8_fraction=0.0)
+    compare_packed(fg, fg.quantize_weights(w.cuda(), f.cuda(), clip_mode=1, fp8_fraction=0.0), q, None, "any sign")
