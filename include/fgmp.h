@@ -220,7 +220,9 @@ fgmp_status fgmp_workspace_init(void* workspace, size_t ws_bytes, void* cuda_str
  * Y[m, n] = sum over blocks of dot16(A[m, kb], W[n, kb]) with each block pair multiplied in
  * its own formats (FP4xFP4, FP4xFP8, FP8xFP4, FP8xFP8), microscales and tensor scales
  * applied, accumulated in FP32.  Y is fp32 (y_is_bf16 = 0) or bf16 [M, ldy].  The workspace
- * must have been cleared once with fgmp_workspace_init.  For 1 <= M <= 16, K % 256 == 0 and
+ * must have been cleared once with fgmp_workspace_init; one that is sized for a batch of prefill size serves every smaller
+ * one of the same layer (with less room than fgmp_workspace_bytes asks for, the work may be cut another way, and the sums
+ * taken in another order).  For 1 <= M <= 16, K % 256 == 0 and
  * N <= 258048 the weight-streaming kernel runs, launched as a programmatic dependent of the kernel
  * before it in the stream (its set-up and its first reads of packed_weights overlap that kernel's
  * end; it reads the packed activations and the workspace only after that kernel has completed).  So

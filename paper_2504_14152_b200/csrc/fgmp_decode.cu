@@ -824,7 +824,7 @@ extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const 
     if (M < 1 || N < 1 || K < 64 || (K % 64) != 0 || ldy < N || ldx < K || (ldx % 8) != 0) return FGMP_ERR_SHAPE;
     if (((uintptr_t)X_bf16 & 15) || ((uintptr_t)fisher_chan & 15) || ((uintptr_t)packed_weights & 1023) ||
         ((uintptr_t)workspace & 1023) || ((uintptr_t)Y & 15) || ((uintptr_t)packed_acts_out & 1023)) return FGMP_ERR_SHAPE;
-    if (ws_bytes < fgmp_ws_linear_fused(M, N, K)) return FGMP_ERR_WORKSPACE;
+    if (ws_bytes < (fgmp_decode_supported(M, N, K) ? fgmp_ws_linear_fused(M, N, K) : fgmp_ws_linear_least(M, N, K))) return FGMP_ERR_WORKSPACE;
     if (packed_acts_out && packed_bytes < fgmp_layout(M, K, 0, 0).total) return FGMP_ERR_WORKSPACE;
     if (!fgmp_decode_supported(M, N, K)) {
         // larger batches: the two calls (the quantizer is then a small part of the step)

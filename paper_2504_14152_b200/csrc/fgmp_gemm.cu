@@ -484,11 +484,19 @@ size_t fgmp_ws_linear_quantize(int64_t M, int64_t N, int64_t K)
     return fgmp_ws_linear(M, N, K) + (M <= 16 ? fgmp_align1k((size_t)M * N * 2) : 0);
 }
 
-size_t fgmp_ws_linear(int64_t M, int64_t N, int64_t K)
+// The two planes are enough for every call, and grow with M: a workspace sized for one batch serves the smaller ones.  The parts of shared
+// tiles may take more at middling M (4096 x 4096: 70 MB at 800 tokens, 40 at 817); where they do not fit, the work is cut another way.
+size_t fgmp_ws_linear_least(int64_t M, int64_t N, int64_t K)
 {
     if (fgmp_decode_supported(M, N, K)) return fgmp_ws_decode(M, N, K);
-    const size_t planes = (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + fgmp_align1k((size_t)N * K * 2), mixed = fgmp_ws_mixed(M, N, K);
-    return planes > mixed ? planes : mixed;
+    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + fgmp_align1k((size_t)N * K * 2);
+}
+size_t fgmp_ws_linear(int64_t M, int64_t N, int64_t K)
+{
+    const size_t least = fgmp_ws_linear_least(M, N, K);
+    if (fgmp_decode_supported(M, N, K)) return least;
+    const size_t mixed = fgmp_ws_mixed(M, N, K);
+    return least > mixed ? least : mixed;
 }
 
 // CTA pairs that can be resident at once on this device (a pair needs two SMs of one cluster domain)
@@ -566,7 +574,7 @@ static double planes_us(int64_t M, int64_t N, int64_t K)
 
 // M > 16 or a shape the weight-streaming kernel does not take.  nvfp4: what the caller expects of the operands, see fgmp_linear_expect.
 static fgmp_status launch_prefill(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                                  int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, int nvfp4, cudaStream_t s)
+                                  int64_t M, int64_t N, int64_t K, void* workspace, size_t ws_bytes, const QuantNext& qn, int nvfp4, cudaStream_t s)
 {
     uint8_t* ws = (uint8_t*)workspace;
     int* status = reinterpret_cast<int*>(ws);
@@ -582,8 +590,8 @@ static fgmp_status launch_prefill(const void* packed_acts, const void* packed_we
     // plane that is expanded once is read faster than that (777 x 11008 x 4096: 86 against 105 us; 2048 x 4096 x 4096: 81
     // against 60).
     // (Behind the all-NVFP4 GEMM: the way of two launches, not three.)
-    if (!nvfp4_first && fgmp_mixed_us(M, N, K) <= planes_us(M, N, K)) {
-        st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, qn, leave, !nvfp4_first, s);
+    if (!nvfp4_first && fgmp_mixed_us(M, N, K, ws_bytes) <= planes_us(M, N, K)) {
+        st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, qn, leave, !nvfp4_first, s);
     } else {
         uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;   // the control area stays as the decode-sized calls need it
         uint8_t* planeW = planeA + fgmp_align1k((size_t)M * K * 2);
@@ -607,14 +615,14 @@ extern "C" fgmp_status fgmp_linear_expect(const void* packed_acts, const void* p
     if (M < 1 || N < 1 || K < 64 || (K % 64) != 0 || ldy < N) return FGMP_ERR_SHAPE;
     if (((uintptr_t)packed_acts & 1023) || ((uintptr_t)packed_weights & 1023) || ((uintptr_t)workspace & 1023) ||
         ((uintptr_t)Y & 15)) return FGMP_ERR_SHAPE;
-    if (ws_bytes < fgmp_ws_linear(M, N, K)) return FGMP_ERR_WORKSPACE;
+    if (ws_bytes < fgmp_ws_linear_least(M, N, K)) return FGMP_ERR_WORKSPACE;
     fgmp_status st;
     if ((st = fgmp_require_sm100()) != FGMP_OK) return st;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     if (fgmp_decode_supported(M, N, K))
         return fgmp_linear_decode(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, false, s);
     QuantNext off{};
-    return launch_prefill(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, off, nvfp4, s);
+    return launch_prefill(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, off, nvfp4, s);
 }
 
 extern "C" fgmp_status fgmp_linear(const void* packed_acts, const void* packed_weights,
@@ -682,15 +690,17 @@ extern "C" fgmp_status fgmp_linear_quantize(const void* packed_acts, const void*
     if (M < 1 || N < 64 || (N % 64) != 0 || K < 64 || (K % 64) != 0) return FGMP_ERR_SHAPE;
     if (((uintptr_t)packed_acts & 1023) || ((uintptr_t)packed_weights & 1023) || ((uintptr_t)workspace & 1023) ||
         ((uintptr_t)packed_out & 1023) || ((uintptr_t)fisher_chan_next & 15)) return FGMP_ERR_SHAPE;
-    if (ws_bytes < fgmp_ws_linear_quantize(M, N, K)) return FGMP_ERR_WORKSPACE;
+    const size_t tail = M <= 16 ? fgmp_align1k((size_t)M * N * 2) : 0;
+    if (ws_bytes < fgmp_ws_linear_least(M, N, K) + tail) return FGMP_ERR_WORKSPACE;
     const PackedLayout L = fgmp_layout(M, N, 0, 0);
     if (packed_bytes < L.total) return FGMP_ERR_WORKSPACE;
     if (M <= 16) {
         // At most 16 tokens: the two steps stay two calls, the bf16 outputs (at most 16 x N) passing through the end of the workspace.  The
         // weight-streaming kernel holds an output row per thread, not a token row, and a packed tensor of so few rows also has
         // the records that kernel reads in the next layer, which the quantizer of a GEMM's epilogue does not write.
-        uint8_t* ybf = (uint8_t*)workspace + fgmp_ws_linear(M, N, K);
-        fgmp_status st2 = fgmp_linear(packed_acts, packed_weights, ybf, 1, N, M, N, K, workspace, fgmp_ws_linear(M, N, K), cuda_stream);
+        const size_t front = (ws_bytes - tail) & ~(size_t)1023;
+        uint8_t* ybf = (uint8_t*)workspace + front;
+        fgmp_status st2 = fgmp_linear(packed_acts, packed_weights, ybf, 1, N, M, N, K, workspace, front, cuda_stream);
         if (st2 != FGMP_OK) return st2;
         return fgmp_quantize_activations(ybf, N, fisher_chan_next, M, N, sc_next, sm, tau_next, packed_out, packed_bytes,
                                          nullptr, 0, cuda_stream);
@@ -710,7 +720,7 @@ extern "C" fgmp_status fgmp_linear_quantize(const void* packed_acts, const void*
     q.mask = reinterpret_cast<uint32_t*>(blob + L.off_mask); q.codes8 = blob + L.off_codes8;
     q.header = reinterpret_cast<fgmp_packed_header*>(blob);
     q.MW = L.MW;
-    return launch_prefill(packed_acts, packed_weights, nullptr, 0, N, M, N, K, workspace, q, -1, (cudaStream_t)cuda_stream);
+    return launch_prefill(packed_acts, packed_weights, nullptr, 0, N, M, N, K, workspace, ws_bytes, q, -1, (cudaStream_t)cuda_stream);
 }
 
 extern "C" fgmp_status fgmp_workspace_init(void* workspace, size_t ws_bytes, void* cuda_stream)

@@ -13,6 +13,7 @@ int fgmp_sm_count();
 size_t fgmp_ws_quantize_weights(int64_t N, int64_t K);
 size_t fgmp_ws_calibrate(int64_t M, int64_t K);
 size_t fgmp_ws_linear(int64_t M, int64_t N, int64_t K);
+size_t fgmp_ws_linear_least(int64_t M, int64_t N, int64_t K);          // what a call must be given, see fgmp_linear
 size_t fgmp_ws_linear_quantize(int64_t M, int64_t N, int64_t K);
 size_t fgmp_ws_linear_fused(int64_t M, int64_t N, int64_t K);
 size_t fgmp_ws_linear_classes(int64_t M, int64_t N, int64_t K);
@@ -33,12 +34,12 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
 fgmp_status fgmp_expand(const void* packed_acts, const void* packed_weights, int64_t M, int64_t N, int64_t K, uint8_t* planeA, uint8_t* planeW,
                         int* status, int cls_a, int cls_w, bool leave_nvfp4, bool first, cudaStream_t s);
 
-// GEMM on the packed weights (fgmp_mixed.cu), and its modelled time
+// GEMM on the packed weights (fgmp_mixed.cu), and its modelled time in a workspace of that size
 struct QuantNext;
-double fgmp_mixed_us(int64_t M, int64_t N, int64_t K);
+double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes);
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K);
 fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                              int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, bool first, cudaStream_t s);
+                              int64_t M, int64_t N, int64_t K, void* workspace, size_t ws_bytes, const QuantNext& qn, bool leave_nvfp4, bool first, cudaStream_t s);
 
 // ---- the FP8 tensor scale of a call (fgmp_scales): given on its own, or scale_fp4 * 2^ratio ----
 #include <math.h>

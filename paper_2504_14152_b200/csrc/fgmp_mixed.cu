@@ -58,7 +58,7 @@ struct MixedPlan {
     uint32_t chunks, tiles;              // tiles = wtiles * tok_tiles
     uint32_t grid, span, rest, quantum;  // a CTA's span in quanta of `quantum` units (1, or chunks: whole tiles)
     uint32_t split;                      // 1: some tile is shared by several CTAs, whose parts are added up behind this kernel
-    uint32_t wstages, bstages, slots, naccs, max_parts;
+    uint32_t wstages, bstages, slots, naccs;
     double us;                           // modelled time
 };
 
@@ -543,9 +543,12 @@ constexpr uint32_t MX_FIXED = 1024 /*alignment*/ + 1024 /*barriers, stage table*
 // Modelled time of a unit in us (measured: 1.55 at 112 tokens, 1.75 at 160, 1.95 at 208, 2.15 at 256)
 double unit_us(uint32_t n_tok) { return 1.08 + 0.0042 * n_tok; }
 
+// bytes for the parts of shared tiles: at most two tiles of a span are shared
+size_t parts_bytes(const MixedPlan& pl) { return pl.split ? (size_t)pl.grid * 2 * ((pl.n_tok + 31u) & ~31u) * 512 : 0; }
+
 // How the work is cut: tokens per tile, and whether CTAs take whole tiles or equal spans of units: the least modelled time
-// (within 10 % of the measured one from 17 to 2048 tokens).
-MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
+// (within 10 % of the measured one from 17 to 2048 tokens) among the ways whose parts of tiles fit in `room` bytes.
+MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts)
 {
     const uint32_t wtiles = (uint32_t)((N + 127) / 128), chunks = (uint32_t)((K / 64 + 3) / 4), sms = (uint32_t)fgmp_sm_count();
     const uint32_t t_min = (uint32_t)((M + MX_MAX_TOK - 1) / MX_MAX_TOK), t_max = 2 * (uint32_t)((M + 255) / 256) + 2;
@@ -570,6 +573,7 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
             // equal spans that are whole tiles after all are the other way of cutting, which needs no second kernel
             pl.split = split;
             if (split && pl.rest == 0 && pl.span % chunks == 0) continue;
+            if (parts_bytes(pl) > room_for_parts) continue;
             const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / chunks;
             // (beyond 256 tokens only spans within one tile pay: where a CTA goes on to another one its three slots and three
             // token stages run empty as well)
@@ -580,7 +584,6 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K)
             if (pl.us < best.us) best = pl;
         }
     }
-    best.max_parts = best.split ? best.grid * 2 : 0;
     const uint32_t tmem_slots = (MX_TMEM_COLS - best.naccs * best.n_tok) / 32;
     best.slots = tmem_slots < (uint32_t)MAX_SLOTS ? tmem_slots : (uint32_t)MAX_SLOTS;
     // shared memory: two to four weight stages (a chunk each), the rest token stages
@@ -604,17 +607,23 @@ bool mx_attr_set[64] = {};
 
 }  // namespace
 
-double fgmp_mixed_us(int64_t M, int64_t N, int64_t K) { return mixed_plan(M, N, K).us; }
+// room for parts in a workspace of ws_bytes, behind the activations' plane
+static size_t room_in(size_t ws_bytes, int64_t M, int64_t K)
+{
+    const size_t before = (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2);
+    return ws_bytes > before ? ws_bytes - before : 0;
+}
+
+double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes) { return mixed_plan(M, N, K, room_in(ws_bytes, M, K)).us; }
 
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K)
 {
-    const MixedPlan pl = mixed_plan(M, N, K);
-    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + (size_t)pl.max_parts * ((pl.n_tok + 31u) & ~31u) * 512;
+    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + parts_bytes(mixed_plan(M, N, K, SIZE_MAX));
 }
 
 // expands the activations and multiplies; leave_nvfp4: unless neither operand has an FP8 block
 fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
-                              int64_t M, int64_t N, int64_t K, void* workspace, const QuantNext& qn, bool leave_nvfp4, bool first, cudaStream_t s)
+                              int64_t M, int64_t N, int64_t K, void* workspace, size_t ws_bytes, const QuantNext& qn, bool leave_nvfp4, bool first, cudaStream_t s)
 {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
@@ -640,7 +649,7 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     p.ha = reinterpret_cast<const fgmp_packed_header*>(packed_acts);
     p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K;
     p.leave_nvfp4 = leave_nvfp4 ? 1 : 0;
-    p.pl = mixed_plan(M, N, K);
+    p.pl = mixed_plan(M, N, K, room_in(ws_bytes, M, K));
     p.status = reinterpret_cast<int*>(ws);
     uint8_t* plane = ws + FGMP_WS_CONTROL_BYTES;
     p.parts = reinterpret_cast<float*>(plane + fgmp_align1k((size_t)M * K * 2));

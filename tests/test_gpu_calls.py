@@ -228,3 +228,36 @@ def test_clip_search_with_any_sensitivity(fg):
     f[60, 5::32] = float("nan")
     q = oracle.quantize_weights(gi.bf16_bits(w), f.numpy(), clip=True, fp8_fraction=0.0)
     compare_packed(fg, fg.quantize_weights(w.cuda(), f.cuda(), clip_mode=1, fp8_fraction=0.0), q, None, "any sign")
+
+
+# A workspace sized for the largest batch serves the smaller ones, among them those whose own size would be larger (the parts of shared
+# tiles take most at middling batches); one byte less than two planes of fp16 is refused.
+@pytest.mark.parametrize("N,K,largest", [(2048, 2048, 1024), (4096, 4096, 817), (1024, 320, 1000)])
+def test_workspace_of_the_largest_batch_serves_the_smaller_ones(fg, N, K, largest):
+    dev = torch.device("cuda")
+    w = draw_weights(fg, N, K, 110)
+    f = torch.ones(N, device=dev)
+    sizes = [M for M in {17, 18, 33, 100, 129, 257, 300, 417, 513, 600, 720, 769, 800, 817, 1000, 1024} if M <= largest]
+    assert any(fg.workspace_bytes(fg.OP_LINEAR, M, N, K) > fg.workspace_bytes(fg.OP_LINEAR, largest, N, K) for M in sizes)
+    ws = fg.alloc_workspace(fg.OP_LINEAR, largest, N, K, dev)
+    guard = fg.binding._alloc_aligned(ws.numel() + 4096, dev)
+    guard[ws.numel():] = 0xa5
+    ws = fg.workspace_init(guard[:ws.numel()])
+    for M in sorted(sizes):
+        acts = draw_acts(fg, M, K, 111)
+        y, y0 = fg.linear(acts, w, workspace=ws), fg.linear(acts, w)
+        assert (y - y0).double().norm() <= 1e-6 * y0.double().norm(), M
+        h = fg.linear_quantize(acts, w, f, scale_fp4=1e-3, tau=1e-4, workspace=ws)
+        want = fg.quantize_activations(fg.linear(acts, w, out_dtype=torch.bfloat16, workspace=ws), f, scale_fp4=1e-3, tau=1e-4)
+        for a, b in zip(fg.unpack(h), fg.unpack(want)):
+            assert torch.equal(a, b), M
+        fg.check(ws)
+    assert (guard[ws.numel():] == 0xa5).all()
+    M = sorted(sizes)[-2]
+    align = lambda n: (n + 1023) // 1024 * 1024   # noqa: E731
+    least = 65536 + align(M * K * 2) + align(N * K * 2)
+    acts = draw_acts(fg, M, K, 111)
+    fg.linear(acts, w, workspace=ws[:least])
+    with pytest.raises(fg.FgmpError) as e:
+        fg.linear(acts, w, workspace=ws[:least - 1])
+    assert e.value.code == -3
