@@ -45,17 +45,23 @@ inline int64_t as_int(PyObject* o)
     if (v == -1 && PyErr_Occurred()) throw python_error();
     return v;
 }
+inline at::Tensor optional_tensor(PyObject* o) { return is_none(o) ? at::Tensor() : tensor_of(o); }
+// The interpreter lock is given up for what may wait: allocations, and launches on a full queue.
+struct WithoutLock {
+    PyThreadState* state = PyEval_SaveThread();
+    ~WithoutLock() { PyEval_RestoreThread(state); }
+};
 // workspace given by the caller, or a cleared one of this call's own
-inline at::Tensor workspace_for(PyObject* given, int op, int64_t M, int64_t N, int64_t K, c10::Device dev, void* stream, fgmp_status* st)
+inline at::Tensor workspace_for(const at::Tensor& given, int op, int64_t M, int64_t N, int64_t K, c10::Device dev, void* stream, fgmp_status* st)
 {
-    if (!is_none(given)) return tensor_of(given);
+    if (given.defined()) return given;
     at::Tensor ws = empty_aligned((int64_t)fgmp_workspace_bytes(op, M, N, K), dev);
     *st = fgmp_workspace_init(ws.data_ptr(), (size_t)ws.numel(), stream);
     return ws;
 }
-inline at::Tensor output_for(PyObject* given, bool bf16, int64_t M, int64_t N, c10::Device dev)
+inline at::Tensor output_for(const at::Tensor& given, bool bf16, int64_t M, int64_t N, c10::Device dev)
 {
-    if (!is_none(given)) return tensor_of(given);
+    if (given.defined()) return given;
     return empty_cuda({M, N}, bf16 ? at::kBFloat16 : at::kFloat, dev);
 }
 
@@ -71,9 +77,14 @@ PyObject* py_quantize_activations(PyObject*, PyObject* const* a, Py_ssize_t n)
     const fgmp_scales sc{(float)as_double(a[2]), (int)as_int(a[3]), (float)as_double(a[4])};
     const int mode = (int)as_int(a[5]);
     const float tau = (float)as_double(a[6]);
-    at::Tensor out = is_none(a[7]) ? empty_aligned((int64_t)nbytes, X.device()) : tensor_of(a[7]);
-    const fgmp_status st = fgmp_quantize_activations(X.data_ptr(), X.stride(0), (const float*)f.data_ptr(), M, K, sc, (fgmp_score_mode)mode, tau,
-                                                     out.data_ptr(), (size_t)out.numel(), nullptr, 0, current_stream());
+    at::Tensor out = optional_tensor(a[7]);
+    fgmp_status st = FGMP_OK;
+    {
+        WithoutLock no_lock;
+        if (!out.defined()) out = empty_aligned((int64_t)nbytes, X.device());
+        st = fgmp_quantize_activations(X.data_ptr(), X.stride(0), (const float*)f.data_ptr(), M, K, sc, (fgmp_score_mode)mode, tau,
+                                       out.data_ptr(), (size_t)out.numel(), nullptr, 0, current_stream());
+    }
     if (st != FGMP_OK) return fail(st, "fgmp_quantize_activations");
     return THPVariable_Wrap(std::move(out));
     END_HANDLE_TH_ERRORS
@@ -86,14 +97,23 @@ PyObject* py_linear(PyObject*, PyObject* const* a, Py_ssize_t n)
     TORCH_CHECK_TYPE(n == 9, "linear takes 9 arguments");
     const at::Tensor &acts = tensor_of(a[0]), &w = tensor_of(a[1]);
     const int64_t M = as_int(a[2]), N = as_int(a[3]), K = as_int(a[4]);
-    void* s = current_stream();
-    at::Tensor out = output_for(a[5], PyObject_IsTrue(a[6]) == 1, M, N, acts.device());
+    const bool bf16 = PyObject_IsTrue(a[6]) == 1;
+    const int nvfp4 = (int)as_int(a[8]);
+    at::Tensor out = optional_tensor(a[5]), ws = optional_tensor(a[7]);
     fgmp_status st = FGMP_OK;
-    at::Tensor ws = workspace_for(a[7], FGMP_OP_LINEAR, M, N, K, acts.device(), s, &st);
-    if (st != FGMP_OK) return fail(st, "fgmp_workspace_init");
-    st = fgmp_linear_expect(acts.data_ptr(), w.data_ptr(), out.data_ptr(), out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0), M, N, K,
-                     ws.data_ptr(), (size_t)ws.numel(), (int)as_int(a[8]), s);
-    if (st != FGMP_OK) return fail(st, "fgmp_linear");
+    const char* call = "fgmp_workspace_init";
+    {
+        WithoutLock no_lock;
+        void* s = current_stream();
+        out = output_for(out, bf16, M, N, acts.device());
+        ws = workspace_for(ws, FGMP_OP_LINEAR, M, N, K, acts.device(), s, &st);
+        if (st == FGMP_OK) {
+            call = "fgmp_linear";
+            st = fgmp_linear_expect(acts.data_ptr(), w.data_ptr(), out.data_ptr(), out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0),
+                                    M, N, K, ws.data_ptr(), (size_t)ws.numel(), nvfp4, s);
+        }
+    }
+    if (st != FGMP_OK) return fail(st, call);
     PyObject* r = PyTuple_New(2);
     PyTuple_SET_ITEM(r, 0, THPVariable_Wrap(std::move(out)));
     PyTuple_SET_ITEM(r, 1, THPVariable_Wrap(std::move(ws)));
@@ -112,18 +132,25 @@ PyObject* py_linear_fused(PyObject*, PyObject* const* a, Py_ssize_t n)
     const fgmp_scales sc{(float)as_double(a[4]), (int)as_int(a[5]), 0.f};
     const int mode = (int)as_int(a[6]);
     const float tau = (float)as_double(a[7]);
-    void* s = current_stream();
-    at::Tensor out = output_for(a[8], PyObject_IsTrue(a[9]) == 1, M, N, X.device());
-    at::Tensor packed;
-    if (!is_none(a[10])) packed = tensor_of(a[10]);
-    else if (PyObject_IsTrue(a[11]) == 1) packed = empty_aligned((int64_t)fgmp_acts_bytes(M, K), X.device());
+    const bool bf16 = PyObject_IsTrue(a[9]) == 1, want_packed = PyObject_IsTrue(a[11]) == 1;
+    at::Tensor out = optional_tensor(a[8]), packed = optional_tensor(a[10]), ws = optional_tensor(a[12]);
     fgmp_status st = FGMP_OK;
-    at::Tensor ws = workspace_for(a[12], FGMP_OP_LINEAR_FUSED, M, N, K, X.device(), s, &st);
-    if (st != FGMP_OK) return fail(st, "fgmp_workspace_init");
-    st = fgmp_linear_fused(X.data_ptr(), X.stride(0), (const float*)f.data_ptr(), sc, (fgmp_score_mode)mode, tau, w.data_ptr(), out.data_ptr(),
-                           out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0), M, N, K, packed.defined() ? packed.data_ptr() : nullptr,
-                           packed.defined() ? (size_t)packed.numel() : 0, ws.data_ptr(), (size_t)ws.numel(), s);
-    if (st != FGMP_OK) return fail(st, "fgmp_linear_fused");
+    const char* call = "fgmp_workspace_init";
+    {
+        WithoutLock no_lock;
+        void* s = current_stream();
+        out = output_for(out, bf16, M, N, X.device());
+        if (!packed.defined() && want_packed) packed = empty_aligned((int64_t)fgmp_acts_bytes(M, K), X.device());
+        ws = workspace_for(ws, FGMP_OP_LINEAR_FUSED, M, N, K, X.device(), s, &st);
+        if (st == FGMP_OK) {
+            call = "fgmp_linear_fused";
+            st = fgmp_linear_fused(X.data_ptr(), X.stride(0), (const float*)f.data_ptr(), sc, (fgmp_score_mode)mode, tau, w.data_ptr(),
+                                   out.data_ptr(), out.scalar_type() == at::kBFloat16 ? 1 : 0, out.stride(0), M, N, K,
+                                   packed.defined() ? packed.data_ptr() : nullptr, packed.defined() ? (size_t)packed.numel() : 0,
+                                   ws.data_ptr(), (size_t)ws.numel(), s);
+        }
+    }
+    if (st != FGMP_OK) return fail(st, call);
     PyObject* r = PyTuple_New(3);
     PyTuple_SET_ITEM(r, 0, THPVariable_Wrap(std::move(out)));
     if (packed.defined()) PyTuple_SET_ITEM(r, 1, THPVariable_Wrap(std::move(packed)));
@@ -143,14 +170,21 @@ PyObject* py_linear_quantize(PyObject*, PyObject* const* a, Py_ssize_t n)
     const fgmp_scales sc{(float)as_double(a[6]), (int)as_int(a[7]), 0.f};
     const int mode = (int)as_int(a[8]);
     const float tau = (float)as_double(a[9]);
-    void* s = current_stream();
-    at::Tensor out = empty_aligned((int64_t)fgmp_acts_bytes(M, N), acts.device());
+    at::Tensor out, ws = optional_tensor(a[10]);
     fgmp_status st = FGMP_OK;
-    at::Tensor ws = workspace_for(a[10], FGMP_OP_LINEAR_QUANTIZE, M, N, K, acts.device(), s, &st);
-    if (st != FGMP_OK) return fail(st, "fgmp_workspace_init");
-    st = fgmp_linear_quantize(acts.data_ptr(), w.data_ptr(), M, N, K, (const float*)f.data_ptr(), sc, (fgmp_score_mode)mode, tau,
-                              out.data_ptr(), (size_t)out.numel(), ws.data_ptr(), (size_t)ws.numel(), s);
-    if (st != FGMP_OK) return fail(st, "fgmp_linear_quantize");
+    const char* call = "fgmp_workspace_init";
+    {
+        WithoutLock no_lock;
+        void* s = current_stream();
+        out = empty_aligned((int64_t)fgmp_acts_bytes(M, N), acts.device());
+        ws = workspace_for(ws, FGMP_OP_LINEAR_QUANTIZE, M, N, K, acts.device(), s, &st);
+        if (st == FGMP_OK) {
+            call = "fgmp_linear_quantize";
+            st = fgmp_linear_quantize(acts.data_ptr(), w.data_ptr(), M, N, K, (const float*)f.data_ptr(), sc, (fgmp_score_mode)mode, tau,
+                                      out.data_ptr(), (size_t)out.numel(), ws.data_ptr(), (size_t)ws.numel(), s);
+        }
+    }
+    if (st != FGMP_OK) return fail(st, call);
     PyObject* r = PyTuple_New(2);
     PyTuple_SET_ITEM(r, 0, THPVariable_Wrap(std::move(out)));
     PyTuple_SET_ITEM(r, 1, THPVariable_Wrap(std::move(ws)));

@@ -1,7 +1,9 @@
 """GPU tests of calls behind one another: on one stream without a synchronisation between them, on one workspace, on buffers that
 are used again, with what an earlier call has left there.  Inputs are drawn on the GPU; what a call returns by itself is the
 reference of what it returns among others."""
-import numpy as np
+import threading
+import time
+
 import pytest
 import torch
 
@@ -261,3 +263,36 @@ def test_workspace_of_the_largest_batch_serves_the_smaller_ones(fg, N, K, larges
     with pytest.raises(fg.FgmpError) as e:
         fg.linear(acts, w, workspace=ws[:least - 1])
     assert e.value.code == -3
+
+
+# A thread whose launches wait for room in the queue (the stream is busy for about half a second) does not keep the interpreter from the others.
+@pytest.mark.parametrize("M", [4, 64])
+def test_other_threads_run_while_a_call_waits_for_the_queue(fg, M):
+    N, K = 256, 256
+    w, acts = draw_weights(fg, N, K, 120), draw_acts(fg, M, K, 121)
+    ws, out = fg.alloc_workspace(fg.OP_LINEAR, M, N, K, torch.device("cuda")), torch.empty(M, N, device="cuda")
+    fg.linear(acts, w, out=out, workspace=ws)
+    torch.cuda.synchronize()
+    stop, gap = threading.Event(), [0.0]
+
+    def tick():
+        last = time.perf_counter()
+        while not stop.is_set():
+            time.sleep(0.001)
+            now = time.perf_counter()
+            gap[0] = max(gap[0], now - last)
+            last = now
+
+    other = threading.Thread(target=tick)
+    other.start()
+    t0 = time.perf_counter()
+    torch.cuda._sleep(1_000_000_000)
+    for _ in range(3000):
+        fg.linear(acts, w, out=out, workspace=ws)
+    busy = time.perf_counter() - t0
+    stop.set()
+    other.join()
+    torch.cuda.synchronize()
+    fg.check(ws)
+    assert busy > 0.2, "the queue took all calls: nothing was waited for"
+    assert gap[0] < 0.1, f"the other thread stood still for {gap[0]:.3f} s"
