@@ -290,7 +290,7 @@ extern "C" fgmp_status fgmp_unpack(const void* packed, int64_t rows, int64_t K, 
     fgmp_packed_header h;
     if (cudaMemcpyAsync(&h, packed, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess) return FGMP_ERR_CUDA;
-    if (h.magic != FGMP_MAGIC || h.rows != rows || h.K != K || h.error != 0) return FGMP_ERR_INVALID_ARG;
+    if (h.magic != FGMP_MAGIC || h.version != FGMP_LAYOUT_VERSION || h.rows != rows || h.K != K || h.error != 0) return FGMP_ERR_INVALID_ARG;
     if (h.kind == 1) {
         const PackedLayout L = fgmp_layout(rows, K, 1, 0);
         FGMP_LAUNCH(FGMP_K_UNPACK, s, unpack_w_kernel<<<(unsigned)L.units, 128, 0, s>>>((const uint8_t*)packed, rows, K, codes4, codes8, scales, mask));

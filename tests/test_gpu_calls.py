@@ -296,3 +296,14 @@ def test_other_threads_run_while_a_call_waits_for_the_queue(fg, M):
     fg.check(ws)
     assert busy > 0.2, "the queue took all calls: nothing was waited for"
     assert gap[0] < 0.1, f"the other thread stood still for {gap[0]:.3f} s"
+
+
+# A blob of another layout version (kept in a file, say) is refused by the unpacker as by the GEMMs: its sections lie elsewhere.
+@pytest.mark.parametrize("kind", [0, 1])
+def test_blob_of_another_layout_is_not_unpacked(fg, kind):
+    p = draw_weights(fg, 130, 320, 130) if kind else draw_acts(fg, 130, 320, 130)
+    fg.unpack(p)
+    p.blob[4:8].view(torch.int32).sub_(1)
+    with pytest.raises(fg.FgmpError) as e:
+        fg.unpack(p)
+    assert e.value.code == -1
