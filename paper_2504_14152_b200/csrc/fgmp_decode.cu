@@ -57,7 +57,11 @@ constexpr int Q_THREADS = 2 * SET_THREADS;      // both sets share out the quant
 constexpr int PIECES = 6;                       // base-8 digits of an FP8 activation block
 constexpr uint32_t STG_MASK = REC_BYTES, STG_LIST = STG_MASK + 256;          // the unit's mask, the list of its FP8 blocks
 constexpr uint32_t LIST_CAP = 3712;             // bytes of the list that fit a stage (about 305 blocks); more is read from global
-constexpr uint32_t STG_STEP = STG_LIST + LIST_CAP;                           // 22528, 1 KiB aligned: step record, then packed activation record (DEC_UNPACK)
+constexpr uint32_t STG_STEP = STG_LIST + LIST_CAP;                           // 22528, 1 KiB aligned: step record
+// DEC_UNPACK: the packed activation records of the stages lie behind the last stage.  From 14 tokens on four of them fit only without the 256
+// bytes that nothing uses, in two copies.
+constexpr uint32_t AREC_GAP = AREC_AT - AREC_HOT;
+__host__ __device__ inline uint32_t arec_gap(int64_t M) { return M >= 14 ? AREC_GAP : 0u; }
 constexpr int DEC_MAX_STAGES = 6;
 // tensor memory columns: accumulators (two buffers of 112 and of 32); of each set: a dense E4M3 tile of 64, scales (32)
 constexpr uint32_t D4_COL = 0, D8_COL = 224, DENSE_COL = 288, SF_COL = 416;
@@ -107,7 +111,7 @@ struct DecParams {
     uint32_t chunks;
     uint32_t span, rest;      // units per CTA: span + 1 for the first `rest` CTAs, span for the others
     int* status; uint32_t* counters; float* partials; int maxseg;
-    uint32_t stages, stage_bytes;
+    uint32_t stages, stage_bytes, arec_bytes;    // arec_bytes: of a packed activation record in shared memory (DEC_UNPACK)
     // activation quantizer in front (fused launches only)
     const uint8_t* X; int64_t ldx;        // bf16 [M, ldx]
     const float* fisher;
@@ -191,7 +195,26 @@ __device__ __forceinline__ uint32_t e4m3_digits(uint32_t code)
     return w;
 }
 
-// Writes what the step record `rec` (global or shared memory) holds of four consecutive elements of token m: quarter li of
+// Four elements of an FP8 block, E4M3 codes c8 -> their digits: c[p] = the elements' E2M1 codes of digit p (16 bits)
+__device__ __forceinline__ void fp8_digits4(uint32_t c8, const uint32_t* digits, uint32_t (&c)[PIECES])
+{
+    uint32_t d[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = digits[(c8 >> (8 * i)) & 0x7fu] ^ (((c8 >> (8 * i)) & 0x80u) ? 0x888888u : 0u);
+    // digits p and p + 1 of the four elements: bytes 2 x (two elements)
+    const uint32_t e = (d[0] & 0x0f0f0fu) | ((d[1] & 0x0f0f0fu) << 4), o = ((d[0] >> 4) & 0x0f0f0fu) | (d[1] & 0xf0f0f0u);
+    const uint32_t g = (d[2] & 0x0f0f0fu) | ((d[3] & 0x0f0f0fu) << 4), h = ((d[2] >> 4) & 0x0f0f0fu) | (d[3] & 0xf0f0f0u);
+#pragma unroll
+    for (int p = 0; p < PIECES; ++p) c[p] = __byte_perm((p & 1) ? o : e, (p & 1) ? h : g, (p >> 1) | ((4 + (p >> 1)) << 4)) & 0xffffu;
+}
+// block scale of row i (of seven) of a token: row 0 has the NVFP4 scale, digit p has 2^(3p - 8) in E4M3
+__device__ __forceinline__ uint32_t step_scale(uint32_t i, bool is8, uint32_t sc)
+{
+    const uint32_t digit_sc = i == 1 ? 0x02u : 0x10u + 0x18u * (i - 2u);
+    return i == 0 ? (is8 ? 0u : sc) : (is8 ? digit_sc : 0u);
+}
+
+// Writes what the step record `rec` holds of four consecutive elements of token m: quarter li of
 // block column j.  c4: their E2M1 codes and sc: the block's scale (NVFP4 block), or c8: their E4M3 codes (FP8 block);
 // v: the values over the tensor scale; digits: table of e4m3_digits.
 __device__ __forceinline__ void emit_step(uint8_t* rec, uint32_t M, uint32_t n4, uint32_t n8, uint32_t m, uint32_t j, uint32_t li,
@@ -211,29 +234,83 @@ __device__ __forceinline__ void emit_step(uint8_t* rec, uint32_t M, uint32_t n4,
     if (!is8) {
         *reinterpret_cast<uint16_t*>(rec + fgmp_rec_w4_offset(m, j) + 2u * li) = (uint16_t)c4;
     } else {
-        uint32_t d[4];
+        uint32_t c[PIECES];
+        fp8_digits4(c8, digits, c);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) d[i] = digits[(c8 >> (8 * i)) & 0x7fu] ^ (((c8 >> (8 * i)) & 0x80u) ? 0x888888u : 0u);
-        // digits p and p + 1 of the four elements: bytes 2 x (two elements)
-        const uint32_t e = (d[0] & 0x0f0f0fu) | ((d[1] & 0x0f0f0fu) << 4), o = ((d[0] >> 4) & 0x0f0f0fu) | (d[1] & 0xf0f0f0u);
-        const uint32_t g = (d[2] & 0x0f0f0fu) | ((d[3] & 0x0f0f0fu) << 4), h = ((d[2] >> 4) & 0x0f0f0fu) | (d[3] & 0xf0f0f0u);
-#pragma unroll
-        for (int p = 0; p < PIECES; ++p) {
-            const uint32_t r = (uint32_t)(p + 1) * M + m;
-            const uint32_t c = __byte_perm((p & 1) ? o : e, (p & 1) ? h : g, (p >> 1) | ((4 + (p >> 1)) << 4));
-            *reinterpret_cast<uint16_t*>(rec + fgmp_rec_w4_offset(r, j) + 2u * li) = (uint16_t)c;
-        }
+        for (int p = 0; p < PIECES; ++p)
+            *reinterpret_cast<uint16_t*>(rec + fgmp_rec_w4_offset((uint32_t)(p + 1) * M + m, j) + 2u * li) = (uint16_t)c[p];
     }
-    // scales of the token's seven rows, two per lane: row 0 has the NVFP4 scale, digit p has 2^(3p - 8) in E4M3
+    // scales of the token's seven rows, two per lane
 #pragma unroll
     for (uint32_t e = 0; e < 2; ++e) {
         const uint32_t i = 2u * li + e;
-        if (i <= (uint32_t)PIECES) {
-            const uint32_t digit_sc = i == 1 ? 0x02u : 0x10u + 0x18u * (i - 2u);
-            const uint32_t r = i * M + m;
-            sf[fgmp_rec_sf_offset(r, j)] = (uint8_t)(i == 0 ? (is8 ? 0u : sc) : (is8 ? digit_sc : 0u));
+        if (i <= (uint32_t)PIECES) sf[fgmp_rec_sf_offset(i * M + m, j)] = (uint8_t)step_scale(i, is8, sc);
+    }
+}
+
+__device__ __forceinline__ uint32_t f16x2_to_e5m2x2(uint32_t h)
+{
+    uint16_t r;
+    asm("cvt.rn.satfinite.e5m2x2.f16x2 %0, %1;" : "=h"(r) : "r"(h));
+    return r;
+}
+__device__ __forceinline__ uint32_t f16x2_to_e4m3x2(uint32_t h)
+{
+    uint16_t r;
+    asm("cvt.rn.satfinite.e4m3x2.f16x2 %0, %1;" : "=h"(r) : "r"(h));
+    return r;
+}
+// The same for a whole block (token m, block column j) of the packed activation record `ar`, both in shared memory; unscale: 2^-ratio
+// twice in fp16; wanted8: whether the weights have FP8 blocks, which the E5M2 values are for.  Every step is exact: the values have at most
+// six significant bits, a part of them three.
+__device__ __forceinline__ void unpack_block(uint8_t* rec, const uint8_t* ar, uint32_t M, uint32_t n4, uint32_t n8, uint32_t m, uint32_t j, uint32_t unscale,
+                                             bool wanted8, const uint32_t* digits)
+{
+    const uint4* at = reinterpret_cast<const uint4*>(ar + fgmp_arec_at_offset(m, j) - arec_gap(M));
+    const uint4 a = at[0], b = at[1];
+    const uint32_t sc = ar[AREC_SF + m * 16u + j], w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    const bool is8 = sc == 0;                            // (or a block of zeros)
+    uint8_t* sf = rec + n4 * 128u;
+    if (wanted8) {
+        uint8_t* b8 = sf + 2048u + (j >> 3) * (n8 * 128u);
+        const uint32_t q = M + m;
+        uint32_t hi[4], lo[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            uint32_t h[2], l[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                uint32_t back, rest;
+                h[e] = f16x2_to_e5m2x2(w[2 * k + e]);
+                asm("cvt.rn.f16x2.e5m2x2 %0, %1;" : "=r"(back) : "h"((uint16_t)h[e]));
+                asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(rest) : "r"(w[2 * k + e]), "r"(back));
+                l[e] = f16x2_to_e5m2x2(rest);
+            }
+            hi[k] = h[0] | (h[1] << 16); lo[k] = l[0] | (l[1] << 16);
+        }
+        *reinterpret_cast<uint4*>(b8 + m * 128u + (((j & 7u) ^ (m & 7u)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+        *reinterpret_cast<uint4*>(b8 + q * 128u + (((j & 7u) ^ (q & 7u)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    }
+    if (!is8) {
+        *reinterpret_cast<uint2*>(rec + fgmp_rec_w4_offset(m, j)) = *reinterpret_cast<const uint2*>(ar + AREC_A4 + fgmp_rec_w4_offset(m, j));
+    } else {
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            uint32_t c[2][PIECES];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                uint32_t x0, x1;
+                asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(x0) : "r"(w[4 * half + 2 * e]), "r"(unscale));
+                asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(x1) : "r"(w[4 * half + 2 * e + 1]), "r"(unscale));
+                fp8_digits4(f16x2_to_e4m3x2(x0) | (f16x2_to_e4m3x2(x1) << 16), digits, c[e]);
+            }
+#pragma unroll
+            for (int p = 0; p < PIECES; ++p)
+                *reinterpret_cast<uint32_t*>(rec + fgmp_rec_w4_offset((uint32_t)(p + 1) * M + m, j) + 4u * half) = c[0][p] | (c[1][p] << 16);
         }
     }
+#pragma unroll
+    for (uint32_t i = 0; i <= (uint32_t)PIECES; ++i) sf[fgmp_rec_sf_offset(i * M + m, j)] = (uint8_t)step_scale(i, is8, sc);
 }
 
 // One work item of the quantizer in front of a fused call: chunk c (256 elements) of the token rows 4 quad .. 4 quad + 3.
@@ -283,7 +360,8 @@ decode_kernel(const __grid_constant__ DecParams p)
     constexpr int X = DEC_MAX_STAGES;
     const uint32_t S = p.stages;
     const uint32_t M = (uint32_t)p.M, n4 = step_n4(M), n8 = step_n8(M), a_bytes = step_bytes(M);
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + S * p.stage_bytes);
+    uint8_t* arecs = smem + S * p.stage_bytes;           // DEC_UNPACK: S packed activation records
+    uint64_t* bars = reinterpret_cast<uint64_t*>(arecs + S * p.arec_bytes);
     StageMeta* smeta = reinterpret_cast<StageMeta*>(bars + 4 * X + 4);
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smeta + X);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -335,7 +413,13 @@ decode_kernel(const __grid_constant__ DecParams p)
         const int err = __ldg(&hw->error), free8 = __ldg(&hw->fp8_scale_free);
         int ok = mv.x == FGMP_MAGIC && mv.y == FGMP_LAYOUT_VERSION && rows == p.N && k == p.K && kind == 1u && err == 0 && free8 == 0;
         int bad = ok ? 0 : 9;
-        const uint32_t arec_bytes = FUSED ? 0u : (M <= 8 ? AREC_AT + 4096u : AREC_BYTES);
+        auto load_arec = [&](uint32_t s, uint32_t unit) {    // the unit's packed activation record into stage s
+            const uint8_t* src = p.ablob + p.LA.off_arec + (size_t)(unit % C) * AREC_BYTES;
+            const uint32_t dst = smem_u32(arecs + s * p.arec_bytes);
+            if (M < 14) { bulk_load(dst, src, p.arec_bytes, wf0 + 8 * s); return; }
+            bulk_load(dst, src, AREC_HOT, wf0 + 8 * s);
+            bulk_load(dst + AREC_HOT, src + AREC_AT, p.arec_bytes - AREC_HOT, wf0 + 8 * s);
+        };
         const uint32_t* uptr = reinterpret_cast<const uint32_t*>(p.wblob + p.LW.off_uptr);
         uint32_t pf_base = u_begin, pf = 0, stage = 0, phase = 1;
         const uint32_t pre = min(S, n_units);
@@ -346,8 +430,7 @@ decode_kernel(const __grid_constant__ DecParams p)
                 if (!FUSED) {
                     const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
                     if (ok && !(ha->magic == FGMP_MAGIC && ha->version == FGMP_LAYOUT_VERSION && ha->rows == p.M && ha->K == p.K && ha->kind == 0u && ha->fp8_scale_free == 0)) { ok = 0; bad = 10; }
-                    if (ok && lane < pre)              // the packed activation records of the stages under way
-                        bulk_load(smem_u32(smem + lane * p.stage_bytes) + STG_STEP + a_bytes, p.ablob + p.LA.off_arec + (size_t)((u_begin + lane) % C) * AREC_BYTES, arec_bytes, wf0 + 8 * lane);
+                    if (ok && lane < pre) load_arec(lane, u_begin + lane);         // of the stages under way
                 }
                 if (bad && lane == 0) { *abort_flag = 1; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, bad); }
             }
@@ -365,11 +448,11 @@ decode_kernel(const __grid_constant__ DecParams p)
                     const uint32_t staged = min((step1 - step0) * 16u, LIST_CAP);
                     smeta[stage].step = step0; smeta[stage].staged = staged;
                     const uint32_t fb = wf0 + 8 * stage, dst = smem_u32(smem + stage * p.stage_bytes);
-                    mbar_expect_tx(fb, REC_BYTES + 256u + staged + arec_bytes);
+                    mbar_expect_tx(fb, REC_BYTES + 256u + staged + (FUSED ? 0u : p.arec_bytes));
                     bulk_load(dst, p.wblob + p.LW.off_rec + (size_t)u * REC_BYTES, REC_BYTES, fb);
                     bulk_load(dst + STG_MASK, p.wblob + p.LW.off_mask + (size_t)u * 256, 256u, fb);
                     if (staged) bulk_load(dst + STG_LIST, lists + (size_t)step0 * 16, staged, fb);
-                    if (!FUSED && i >= pre) bulk_load(dst + STG_STEP + a_bytes, p.ablob + p.LA.off_arec + (size_t)(u % C) * AREC_BYTES, arec_bytes, fb);
+                    if (!FUSED && i >= pre) load_arec(stage, u);
                 }
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -473,30 +556,38 @@ decode_kernel(const __grid_constant__ DecParams p)
         const uint32_t set = (uint32_t)(warp - W_SET) >> 2, row = 32u * (warp & 3) + lane;
         const uint32_t quadrant = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
         const uint32_t dense = quadrant + DENSE_COL + set * 64, sf_t = quadrant + SF_COL + set * 32;
-        float unscale = 0.f;                           // 2^-ratio: back to the E4M3 value of an FP8 element
-        if (!FUSED) unscale = __int_as_float((127 - reinterpret_cast<const fgmp_packed_header*>(p.ablob)->fp8_log2_ratio) << 23);
+        uint32_t unscale = 0;                          // 2^-ratio, twice in fp16: back to the E4M3 value of an FP8 element
+        if (!FUSED) unscale = (uint32_t)(15 - reinterpret_cast<const fgmp_packed_header*>(p.ablob)->fp8_log2_ratio) * 0x04000400u;
         uint32_t stage = set, phase = 0, done = set, dphase = 0;      // done: stage of the set's last unit
         for (uint32_t i = set; i < n_units; i += 2) {
             const uint8_t* sb = smem + stage * p.stage_bytes;
-            // Barriers are waited for by parity, so the stage's unit before this one must be known to be in.  With three stages it is the other
-            // set's, and this set has seen unit i - 4 done at best (with more stages that is enough): its end comes first.
-            // (The copies of unit i begin behind that end, so the wait takes no time of its own.)
-            if (S == 3 && i >= 3 && !mbar_wait_warp(dn0 + 8 * stage, phase ^ 1u, abort_flag, p.status, 5)) break;
+            // (Barriers are waited for by parity, so the stage's unit before this one, the other set's where the number of stages is odd, must be
+            // known to be in.  This set has seen unit i - 4 done, which says so from four stages on.)
             if (!mbar_wait_warp(wf0 + 8 * stage, phase, abort_flag, p.status, 5)) break;
             if (!FUSED) {
-                // the unit's step record from the packed activation record (where a block with scale 0 is FP8, or all zero)
+                // the unit's step record from the packed activation record
                 uint8_t* rec = smem + stage * p.stage_bytes + STG_STEP;
-                const uint8_t* ar = rec + a_bytes;
-                const uint32_t ts = (threadIdx.x - 32u * W_SET) & (SET_THREADS - 1u), li = ts & 3u, j = (ts >> 2) & 15u;
+                const uint8_t* ar = arecs + stage * p.arec_bytes;
+                // Up to four tokens a quarter of a block per thread, above that a whole block, tokens fastest, so that a quarter of a warp reads
+                // 256 and writes 128 contiguous bytes at a time.  (28672 x 8192: 1 token 36.9 us by quarters, 40.5 by blocks; 8 tokens
+                // 49.9 by quarters, 42.7 by blocks.)
+                const uint32_t ts = (threadIdx.x - 32u * W_SET) & (SET_THREADS - 1u);
+                if (M <= 4) {
+                    const uint32_t li = ts & 3u, j = (ts >> 2) & 15u;
 #pragma unroll 1
-                for (uint32_t m = ts >> 6; m < M; m += 2) {
-                    const uint2 h = *reinterpret_cast<const uint2*>(ar + fgmp_arec_at_offset(m, j) + 8u * li);
-                    const uint32_t c4 = *reinterpret_cast<const uint16_t*>(ar + AREC_A4 + fgmp_rec_w4_offset(m, j) + 2u * li);
-                    const uint32_t sc = ar[AREC_SF + m * 16u + j];
-                    const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&h.x)), vb = __half22float2(*reinterpret_cast<const __half2*>(&h.y));
-                    const float v[4] = {va.x, va.y, vb.x, vb.y};
-                    const uint32_t c8 = f32x2_to_e4m3x2(v[0] * unscale, v[1] * unscale) | (f32x2_to_e4m3x2(v[2] * unscale, v[3] * unscale) << 16);
-                    emit_step(rec, M, n4, n8, m, j, li, sc == 0, c4, sc, c8, v, digits);
+                    for (uint32_t m = ts >> 6; m < M; m += 2) {
+                        const uint2 h = *reinterpret_cast<const uint2*>(ar + fgmp_arec_at_offset(m, j) + 8u * li);
+                        const uint32_t c4 = *reinterpret_cast<const uint16_t*>(ar + AREC_A4 + fgmp_rec_w4_offset(m, j) + 2u * li), sc = ar[AREC_SF + m * 16u + j];
+                        const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&h.x)), vb = __half22float2(*reinterpret_cast<const __half2*>(&h.y));
+                        const float v[4] = {va.x, va.y, vb.x, vb.y};
+                        uint32_t x0, x1;
+                        asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(x0) : "r"(h.x), "r"(unscale));
+                        asm("mul.rn.f16x2 %0, %1, %2;" : "=r"(x1) : "r"(h.y), "r"(unscale));
+                        emit_step(rec, M, n4, n8, m, j, li, sc == 0, c4, sc, f16x2_to_e4m3x2(x0) | (f16x2_to_e4m3x2(x1) << 16), v, digits);
+                    }
+                } else {
+#pragma unroll 1
+                    for (uint32_t m = ts & 7u; m < M; m += 8) unpack_block(rec, ar, M, n4, n8, m, ts >> 3, unscale, has_fp8, digits);
                 }
                 fence_proxy_async();                   // the tensor core reads what ordinary stores wrote
                 __syncwarp();
@@ -759,14 +850,16 @@ DecParams base_params(const void* packed_weights, void* Y, int y_is_bf16, int64_
 template <int SRC>
 fgmp_status launch_decode(DecParams p, const DecPlan& d, bool programmatic, cudaStream_t s)
 {
-    const uint32_t arec = SRC == DEC_UNPACK ? (p.M <= 8 ? AREC_AT + 4096u : AREC_BYTES) : 0u;
-    p.stage_bytes = (STG_STEP + step_bytes(p.M) + arec + 1023u) & ~1023u;
-    const size_t fixed = 1024 /*alignment*/ + 1024 /*barriers, digit table*/;
-    const uint32_t fit = (uint32_t)((SMEM_LIMIT - fixed) / p.stage_bytes);         // 3 (DEC_UNPACK, 16 tokens) to 7
+    p.arec_bytes = SRC == DEC_UNPACK ? (p.M <= 8 ? AREC_BYTES - 4096u : AREC_BYTES) - arec_gap(p.M) : 0u;
+    p.stage_bytes = (STG_STEP + step_bytes(p.M) + 1023u) & ~1023u;
+    constexpr size_t fixed = 1024 /*alignment*/ + 1024 /*barriers, digit table*/;
+    const uint32_t fit = (uint32_t)((SMEM_LIMIT - fixed) / (p.stage_bytes + p.arec_bytes));      // 4 (16 tokens) to 7
+    // step records of 16 tokens (see step_bytes); the kernel's sets count on four stages at least
+    static_assert(4 * (STG_STEP + 112 * 128 + 2048 + 32 * 256 + AREC_BYTES - AREC_GAP) + fixed <= SMEM_LIMIT && STG_STEP % 1024 == 0, "four stages");
     p.stages = fit < (uint32_t)DEC_MAX_STAGES ? fit : (uint32_t)DEC_MAX_STAGES;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)d.grid); cfg.blockDim = dim3(DEC_THREADS); cfg.stream = s;
-    cfg.dynamicSmemBytes = fixed + (size_t)p.stages * p.stage_bytes;
+    cfg.dynamicSmemBytes = fixed + (size_t)p.stages * (p.stage_bytes + p.arec_bytes);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;

@@ -75,9 +75,9 @@ def test_linear_right_behind_the_quantizing_one(fg, N, K):
     fg.check(ws)
 
 
-# A CTA has more units than the decode kernel has stages, which is three with 14 to 16 packed tokens, four or more in a fused call:
+# A CTA has more units than the decode kernel has stages (four to six), whose number is odd for some batches:
 # the same sums either way, over and over, with the weights' copies out of L2 and out of HBM.
-@pytest.mark.parametrize("M", [9, 13, 14, 16])
+@pytest.mark.parametrize("M", [1, 3, 4, 5, 8, 9, 13, 14, 16])
 def test_decode_of_packed_tokens_equals_the_fused_step(fg, M):
     N, K = 8192, 4096
     g = torch.Generator(device="cuda").manual_seed(M)
@@ -85,7 +85,7 @@ def test_decode_of_packed_tokens_equals_the_fused_step(fg, M):
     s4 = float(x.abs().max()) / 2688.0
     tau = float(fg.calibrate_tau(x, f, scale_fp4=s4, fp8_fraction=0.1))
     acts = fg.quantize_activations(x, f, scale_fp4=s4, tau=tau)
-    for fp8 in (0.1, 0.3):
+    for fp8 in (0.0, 0.1, 0.3):
         ws = [draw_weights(fg, N, K, 20 + i, fp8) for i in range(6)]
         want = [fg.linear_fused(x, f, w, scale_fp4=s4, tau=tau) for w in ws]
         torch.cuda.synchronize()
