@@ -11,6 +11,13 @@ from test_gpu_parity import GEMM_TOL, compare_packed, fg, quantize_both, tau_for
 pytestmark = pytest.mark.gpu
 
 
+def launches(fg, call):
+    """{kernel: launches} of a call"""
+    fg.profile_begin()
+    call()
+    return {name: n for name, (n, _) in fg.profile_end().items()}
+
+
 def check_linear(fg, qa, qw, pa, pw, rel=1e-5):
     """fp32 and bf16 output, the latter with a row pitch that rules wide stores out, against the oracle."""
     Y, S = oracle.linear(qa, qw)
@@ -31,6 +38,7 @@ def check_linear(fg, qa, qw, pa, pw, rel=1e-5):
 def test_nvfp4_gemm_tiles(fg, M, N, K):
     qa, qw, pa, pw = quantize_both(fg, gi.llama("n4", M, N, K, seed=61), 0.0, 0.0, clip=False)
     check_linear(fg, qa, qw, pa, pw)
+    assert fg.linear.last_workspace[8:12].view(torch.int32).item() == 1, "the all-NVFP4 GEMM has made the result"
 
 
 # token tiles of 16 to 256, one chunk and many, part of a last chunk, part of a weight tile; FP8 shares below and above what a
@@ -59,6 +67,8 @@ def test_quantizer_behind_split_tiles(fg, M, N, K, mode):
 def test_gemm_on_packed_weights_wide_tiles(fg, M, N):
     qa, qw, pa, pw = quantize_both(fg, gi.llama("wd", M, N, 5184, seed=68), 0.1, 0.1, clip=False)
     y16 = fg.linear(pa, pw, out_dtype=torch.bfloat16)
+    count = launches(fg, lambda: fg.linear(pa, pw))
+    assert count.get("gemm_mixed_tcgen05") == 1 and "gemm_f16_tcgen05" not in count, count
     y = fg.linear(pa, pw).cpu().numpy().astype(np.float64)
     fg.check(fg.linear.last_workspace)
     rng = np.random.default_rng(0)
@@ -75,8 +85,10 @@ def test_gemm_on_packed_weights_wide_tiles(fg, M, N):
 # large batch: both operands expanded to fp16 planes, ragged in every direction
 @pytest.mark.parametrize("frac_a,frac_w", [(0.1, 0.1), (0.0, 1.0)])
 def test_gemm_on_expanded_planes_ragged(fg, frac_a, frac_w):
-    M, N, K = 2049, 4113, 4160
+    M, N, K = 4001, 4113, 2112                   # (on 148 SMs modelled at 66 us, 90 on the packed weights)
     qa, qw, pa, pw = quantize_both(fg, gi.llama("pl", M, N, K, seed=64), frac_a, frac_w, clip=False)
+    count = launches(fg, lambda: fg.linear(pa, pw))
+    assert count.get("gemm_f16_tcgen05") == 1 and "gemm_mixed_tcgen05" not in count, count
     y = fg.linear(pa, pw).cpu().numpy().astype(np.float64)
     fg.check(fg.linear.last_workspace)
     rng = np.random.default_rng(0)
