@@ -223,11 +223,6 @@ __device__ __forceinline__ int fgmp_weight_exponent(const fgmp_packed_header* h)
 // One block of 16 values in registers.  Every step below is a single IEEE fp32 operation
 // (no contraction): this sequence is what makes codes and scores reproducible bit for bit.
 
-struct BlockQ {
-    uint32_t c4[2];     // 16 E2M1 codes, element i in nibble i
-    float score;
-};
-
 // Two fp32 operations per instruction, each rounded as it would be alone.  The quantizers are bound by instruction issue: the search for
 // the clipping scale of 4096 x 4096 weights takes 152 us with these, 172 without.
 __device__ __forceinline__ uint64_t f32x2_pack(float a, float b) { uint64_t r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b)); return r; }
