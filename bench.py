@@ -511,6 +511,7 @@ def run_ours(args, world, rank, local):
 # DRAM bytes (read + write) per launch from the committed ncu captures (profiles/*.md).  An entry is
 # removed when its kernel changes after the capture.
 NCU_TRAFFIC = {
+    ("llama2-7b-fc1-decode", "decode_gemm"): {"bytes": 29722368, "file": "profiles/decode_kernel_llama2-7b-fc1-decode.md"},
 }
 
 

@@ -546,8 +546,9 @@ double unit_us(uint32_t n_tok) { return 1.08 + 0.0042 * n_tok; }
 // bytes for the parts of shared tiles: at most two tiles of a span are shared
 size_t parts_bytes(const MixedPlan& pl) { return pl.split ? (size_t)pl.grid * 2 * ((pl.n_tok + 31u) & ~31u) * 512 : 0; }
 
-// How the work is cut: tokens per tile, and whether CTAs take whole tiles or equal spans of units: the least modelled time
-// (within 10 % of the measured one from 17 to 2048 tokens) among the ways whose parts of tiles fit in `room` bytes.
+// How the work is cut: tokens per tile, and whether CTAs take whole tiles or equal spans of units: the least modelled time among the
+// ways whose parts of tiles fit in `room_for_parts` bytes.  (A fit without the expansion's launch: whole calls take 7 to 9 us more at 48 tokens,
+// and are within 10 % of it from 203 tokens on at 11008 x 4096 and 13824 x 5120.)
 MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts)
 {
     const uint32_t wtiles = (uint32_t)((N + 127) / 128), chunks = (uint32_t)((K / 64 + 3) / 4), sms = (uint32_t)fgmp_sm_count();
