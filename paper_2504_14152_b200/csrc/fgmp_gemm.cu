@@ -445,39 +445,9 @@ gemm_f16_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     }
 }
 
-// ------------------------------------------------------------------ host side
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-EncodeTiledFn get_encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-    }
-    return fn;
-}
-
-// 2-D fp16 row-major [rows, K] tensor, box = [box_rows, 64 elements], 128-byte swizzle
-bool make_tmap_f16(CUtensorMap* map, const void* base, int64_t rows, int64_t K, int box_rows)
-{
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {(cuuint32_t)BK, (cuuint32_t)box_rows};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 }  // namespace
+
+// ------------------------------------------------------------------ host side
 
 size_t fgmp_ws_linear_quantize(int64_t M, int64_t N, int64_t K)
 {
@@ -552,7 +522,8 @@ static fgmp_status launch_pair_gemm(const GemmParams& p, const uint8_t* planeA, 
     const fgmp_status st = resident_pairs(&pairs_avail);
     if (st != FGMP_OK) return st;
     CUtensorMap tmA, tmB;
-    if (!make_tmap_f16(&tmA, planeA, p.M, p.K, 128) || !make_tmap_f16(&tmB, planeW, p.N, p.K, 128)) return FGMP_ERR_CUDA;
+    if (!fgmp_map_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, planeA, p.M, p.K, p.K * 2, 128, BK) ||
+        !fgmp_map_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, planeW, p.N, p.K, p.K * 2, 128, BK)) return FGMP_ERR_CUDA;
     const int64_t tiles = ((p.M + P_BM - 1) / P_BM) * ((p.N + P_BN - 1) / P_BN);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

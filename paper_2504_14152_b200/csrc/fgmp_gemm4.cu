@@ -18,7 +18,9 @@
 // Single CTAs are bound by the copies from L2 (18 TB/s over the machine without the products), pairs by the length of a stage's cycle
 // (tensor pipe 51 % of the active cycles, L2 39 % of its peak).  2048 x 13824 x 5120, fp32 output: 88.6 us when one
 // tile's stores ended before the next tile's products began and one of 32 lanes issued the products, 78.8 us with the accumulator
-// drained into registers first and an elected thread, 71.5 us on pairs (bf16 output: 79.9, 70.4, 63.0).
+// drained into registers first and an elected thread, 71.5 us on pairs (bf16 output: 79.9, 70.4, 63.0).  With Y leaving as TMA tiles a
+// tile takes 14200 clocks instead of 16400, of which 10240 are products; the clock falls under that load, and the call takes 96.0 us instead
+// of 98.3 (777 x 11008 x 4096, bf16: 37.5 and 38.8).
 #include <cuda.h>
 #include <mutex>
 #include "fgmp_common.cuh"
@@ -33,7 +35,8 @@ constexpr int G4_THREADS = 448;
 template <bool PAIR> struct G4 {
     static constexpr int STAGES = PAIR ? 5 : 4;
     static constexpr uint32_t A4 = 0, B0 = 16384, B1 = 32768, SFB = PAIR ? 32768 : 49152, SFA = SFB + 4096, STAGE_BYTES = SFA + 2048;
-    static constexpr size_t SMEM = (size_t)STAGES * STAGE_BYTES + 1024 /*alignment*/ + 512 /*barriers*/;
+    static constexpr uint32_t OUT = STAGES * STAGE_BYTES, OUT_BYTES = PAIR ? 8 * TILE_STORE_BYTES : 0;     // tiles of Y on their way out
+    static constexpr size_t SMEM = (size_t)OUT + OUT_BYTES + 1024 /*alignment*/ + 512 /*barriers*/;
     static constexpr int64_t TM = PAIR ? 256 : 128;                       // tokens of an output tile
     static_assert(SMEM <= 232448, "shared memory of one CTA");
     static_assert(256 + 48 * STAGES <= 512, "tensor memory columns");
@@ -66,6 +69,7 @@ struct Gemm4Params {
     PackedLayout LA, LW;
     void* Y; int64_t ldy; int y_is_bf16;
     int64_t M, N, K;
+    int64_t tile_cols;                    // columns of Y that leave as TMA tiles, see fgmp_tile_cols
     int first;                            // the first kernel of the call: the status starts here
     int* status;                          // [0..1] device-side status, [2] 1 = this kernel has produced Y
 };
@@ -137,7 +141,7 @@ __device__ __forceinline__ bool g4_applicable(const Gemm4Params& p)
 
 template <bool PAIR>
 __global__ void __launch_bounds__(G4_THREADS, 1)
-gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, Gemm4Params p)
+gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmY, Gemm4Params p)
 {
     using C = G4<PAIR>;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -153,7 +157,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     constexpr int S = C::STAGES;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * C::STAGE_BYTES);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OUT + C::OUT_BYTES);
     // bars: [0,S) full, [S,2S) empty, [2S,3S) scales in tensor memory, [3S,4S) scales loaded, then acc_full, acc_empty.  Of a pair, the
     // leader's "full" counts the codes of both CTAs, since its thread multiplies both; the scales are each CTA's own matter until they are in
     // tensor memory, and "scales loaded" counts them.  A single CTA has its scales counted by "full".
@@ -306,8 +310,9 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
         const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
         const float alpha = __fmul_rn(ha->scale_fp4, hw->scale_fp4);
-        // Y and its row pitch 32-byte aligned: a lane writes whole sectors
+        // Y and its row pitch 32-byte aligned: a lane that stores its row writes whole sectors
         const bool wide = ((uintptr_t)p.Y & 31) == 0 && ((p.ldy * (p.y_is_bf16 ? 2 : 4)) % 32) == 0;
+        const uint32_t buf = smem_u32(smem + C::OUT) + (uint32_t)(warp - 6) * TILE_STORE_BYTES;
         const uint32_t drained = PAIR ? cluster_map(acce, 0) : acce, src = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(half * 128);
         bool ok = true;
         int64_t it = 0;
@@ -315,21 +320,37 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
             const int64_t tm = t % tiles_m, tn = t / tiles_m;
             if (!(ok = mbar_wait_warp(accf, (uint32_t)(it & 1), abort_flag, p.status, 5))) break;
             tc_fence_after();
-            const int64_t row = tm * C::TM + 128 * rank + q * 32 + lane, n0 = tn * 256 + half * 128;
-            const int64_t left = row < p.M ? p.N - n0 : 0;                // columns that this thread has to store
-            const int64_t at = row * p.ldy + n0;
+            const int64_t row0 = tm * C::TM + 128 * rank + q * 32, n0 = tn * 256 + half * 128;
             uint32_t r[3][32];
 #pragma unroll
             for (int c = 0; c < 3; ++c) tmem_ld32(src + (uint32_t)(c * 32), r[c]);
-            g4_store(p, at, r[0], alpha, left, wide);
+            // 32 columns out; in bf16 a tile of Y has 64
+            auto out = [&](const uint32_t (&v)[32], int c) {
+                const int64_t n = n0 + 32 * c;
+                if (!PAIR || n - 32 * (p.y_is_bf16 ? c & 1 : 0) >= p.tile_cols) {
+                    g4_store(p, (row0 + lane) * p.ldy + n, v, alpha, row0 + lane < p.M ? p.N - n : 0, wide);
+                    return;
+                }
+                if (p.y_is_bf16) {
+                    if ((c & 1) == 0) tile_wait(lane);
+                    tile_put_bf16(buf, lane, c & 1, v, alpha);
+                    if ((c & 1) && row0 < p.M) tile_store(&tmY, buf, lane, (int32_t)(n - 32), (int32_t)row0);
+                } else {
+                    tile_wait(lane);
+                    tile_put_f32(buf, lane, v, alpha);
+                    if (row0 < p.M) tile_store(&tmY, buf, lane, (int32_t)n, (int32_t)row0);
+                }
+            };
+            out(r[0], 0);
             __syncwarp();
             tmem_ld32(src + 96, r[0]);
             tc_fence_before();
             __syncwarp();
             if (lane == 0) { if (PAIR) mbar_arrive_cluster_tmem(drained); else mbar_arrive(drained); }
 #pragma unroll
-            for (int c = 1; c < 4; ++c) g4_store(p, at + c * 32, r[c % 3], alpha, left - c * 32, wide);
+            for (int c = 1; c < 4; ++c) out(r[c % 3], c);
         }
+        if (PAIR) tile_drain(lane);
     }
 
     __syncthreads();
@@ -345,12 +366,7 @@ gemm_nvfp4_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
     }
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
 std::mutex g4_mu;
-EncodeTiledFn g4_encode = nullptr;
 int g4_pairs[64] = {};                 // CTA pairs that run at once
 
 }  // namespace
@@ -364,13 +380,6 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
     {
         std::lock_guard<std::mutex> lk(g4_mu);
-        if (!g4_encode) {
-            void* fn = nullptr;
-            cudaDriverEntryPointQueryResult q;
-            if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess ||
-                q != cudaDriverEntryPointSuccess) return FGMP_ERR_CUDA;
-            g4_encode = reinterpret_cast<EncodeTiledFn>(fn);
-        }
         if (!g4_pairs[dev]) {
             cudaLaunchConfig_t qc = {};
             cudaLaunchAttribute qa[1];
@@ -390,28 +399,21 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     p.ablob = (const uint8_t*)packed_acts; p.wblob = (const uint8_t*)packed_weights;
     p.LA = fgmp_layout(M, K, 0, 0); p.LW = fgmp_layout(N, K, 1, 0);
     p.Y = Y; p.ldy = ldy; p.y_is_bf16 = y_is_bf16; p.M = M; p.N = N; p.K = K; p.status = status; p.first = first ? 1 : 0;
-    // the activations' code plane: bytes [M, K/2] row-major, boxes of 128 rows x 128 bytes, swizzled on the way in
-    CUtensorMap tmA;
-    cuuint64_t dims[2] = {(cuuint64_t)(K / 2), (cuuint64_t)M};
-    cuuint64_t strides[1] = {(cuuint64_t)(K / 2)};
-    cuuint32_t box[2] = {128, 128};
-    cuuint32_t estr[2] = {1, 1};
-    if (g4_encode(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(p.ablob + p.LA.off_codes4), dims, strides, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return FGMP_ERR_CUDA;
-    // pairs: the weights' records as rows of 128 bytes, boxes of a tile's 128 rows (swizzled already), whose loads may be counted in the leader
-    CUtensorMap tmW;
-    cuuint64_t dims_w[2] = {128, (cuuint64_t)(p.LW.units * (REC_BYTES / 128))};
-    cuuint64_t strides_w[1] = {128};
-    if (g4_encode(&tmW, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(p.wblob + p.LW.off_rec), dims_w, strides_w, box, estr,
-                  CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return FGMP_ERR_CUDA;
+    // the activations' code plane: bytes [M, K/2] row-major, boxes of 128 rows x 128 bytes, swizzled on the way in; pairs: the weights'
+    // records as rows of 128 bytes, boxes of a tile's 128 rows (swizzled already), whose loads may be counted in the leader
+    CUtensorMap tmA, tmW;
+    if (!fgmp_map_2d(&tmA, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.ablob + p.LA.off_codes4, M, K / 2, K / 2, 128, 128) ||
+        !fgmp_map_2d(&tmW, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.wblob + p.LW.off_rec, p.LW.units * (REC_BYTES / 128), 128, 128, 128, 128, false))
+        return FGMP_ERR_CUDA;
     const int64_t cols = (p.LW.tiles + 1) / 2, tiles = ((M + 127) / 128) * cols, tiles2 = ((M + 255) / 256) * cols;
     const int sms = fgmp_sm_count();
     // pairs where the tiles take more than one round of the machine (2048 x 13824 x 5120: 63 us, 70 on single CTAs; 777 x 11008 x 4096: 28.2,
     // 30.4) and the larger tiles do not take a round more; within one round the smaller tile's shorter start wins (384 x 5120 x 5120: 13.8 us,
     // 14.5 on pairs)
     const bool pair = tiles > sms && (tiles2 + pairs - 1) / pairs <= (tiles + sms - 1) / sms;
+    CUtensorMap tmY = tmA;
+    p.tile_cols = pair ? fgmp_tile_cols(N, ldy, y_is_bf16) : 0;
+    if (p.tile_cols && !fgmp_map_y(&tmY, Y, y_is_bf16, ldy, M, p.tile_cols)) return FGMP_ERR_CUDA;
     const int grid = pair ? 2 * (int)(tiles2 < pairs ? tiles2 : pairs) : (int)(tiles < sms ? tiles : sms);
     // a programmatic dependent: where it does not apply it is gone when the kernel before it ends
     cudaLaunchAttribute attr[2];
@@ -423,7 +425,7 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
     cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3(G4_THREADS); cfg.stream = s;
     cfg.dynamicSmemBytes = pair ? G4<true>::SMEM : G4<false>::SMEM;
     cfg.attrs = attr; cfg.numAttrs = pair ? 2 : 1;
-    if (pair) FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<true>, tmA, tmW, p));
-    else FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<false>, tmA, tmW, p));
+    if (pair) FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<true>, tmA, tmW, tmY, p));
+    else FGMP_LAUNCH(FGMP_K_GEMM_NVFP4, s, cudaLaunchKernelEx(&cfg, gemm_nvfp4_kernel<false>, tmA, tmW, tmY, p));
     return fgmp_launch_status();
 }

@@ -1,6 +1,7 @@
 // Host utilities: device capability check, status strings, size queries.
 #include "fgmp_common.cuh"
 #include "fgmp_host.h"
+#include <atomic>
 #include <vector>
 #include <mutex>
 
@@ -33,6 +34,28 @@ int fgmp_sm_count()
 {
     DevInfo* i = cur_dev();
     return i ? i->sms : 148;
+}
+
+bool fgmp_map_2d(CUtensorMap* map, CUtensorMapDataType type, const void* base, int64_t rows, int64_t cols, int64_t row_bytes, uint32_t box_rows,
+                 uint32_t box_cols, bool swizzled)
+{
+    typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                      const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static std::atomic<EncodeTiledFn> found{nullptr};
+    EncodeTiledFn encode = found.load(std::memory_order_acquire);
+    if (!encode) {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess)
+            return false;
+        encode = reinterpret_cast<EncodeTiledFn>(fn);
+        found.store(encode, std::memory_order_release);
+    }
+    const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows}, strides[1] = {(cuuint64_t)row_bytes};
+    const cuuint32_t box[2] = {box_cols, box_rows}, estr[2] = {1, 1};
+    return encode(map, type, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 fgmp_status fgmp_launch_status()

@@ -1,5 +1,6 @@
 // Host-side helpers shared by the translation units of libfgmp.
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include "fgmp.h"
 
@@ -9,6 +10,22 @@ fgmp_status fgmp_require_sm100();
 fgmp_status fgmp_launch_status();
 // number of SMs of the current device (cached)
 int fgmp_sm_count();
+// 2-D tensor map: rows of `cols` elements, row_bytes apart (base and row_bytes multiples of 16 bytes), in boxes of box_rows x box_cols whose
+// rows are at most 128 bytes, swizzled by 128 bytes or as they lie; reads beyond the tensor give zeros
+bool fgmp_map_2d(CUtensorMap* map, CUtensorMapDataType type, const void* base, int64_t rows, int64_t cols, int64_t row_bytes, uint32_t box_rows,
+                 uint32_t box_cols, bool swizzled = true);
+// Y in tiles of 32 rows x 128 bytes (tile_store in fgmp_ptx.cuh): how many of its columns leave so.  None where its rows are not 16-byte aligned; not
+// a last part of a tile that does not end on such a boundary (the last 16 bytes would be written as a whole).
+inline int64_t fgmp_tile_cols(int64_t N, int64_t ldy, int y_is_bf16)
+{
+    const int64_t size = y_is_bf16 ? 2 : 4;
+    return ldy * size % 16 ? 0 : N * size % 16 ? N - N % (128 / size) : N;
+}
+inline bool fgmp_map_y(CUtensorMap* map, void* Y, int y_is_bf16, int64_t ldy, int64_t M, int64_t tile_cols)
+{
+    return fgmp_map_2d(map, y_is_bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, Y, M, tile_cols, ldy * (y_is_bf16 ? 2 : 4), 32,
+                       y_is_bf16 ? 64 : 32);
+}
 // workspace sizes of the individual operations
 size_t fgmp_ws_quantize_weights(int64_t N, int64_t K);
 size_t fgmp_ws_calibrate(int64_t M, int64_t K);

@@ -599,11 +599,7 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts)
     return best;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 std::mutex mx_mu;
-EncodeTiledFn mx_encode = nullptr;
 bool mx_attr_set[64] = {};
 
 }  // namespace
@@ -630,13 +626,6 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
     {
         std::lock_guard<std::mutex> lk(mx_mu);
-        if (!mx_encode) {
-            void* fn = nullptr;
-            cudaDriverEntryPointQueryResult q;
-            if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &q) != cudaSuccess ||
-                q != cudaDriverEntryPointSuccess) return FGMP_ERR_CUDA;
-            mx_encode = reinterpret_cast<EncodeTiledFn>(fn);
-        }
         if (!mx_attr_set[dev]) {
             if (cudaFuncSetAttribute(mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess ||
                 cudaFuncSetAttribute(mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess)
@@ -657,12 +646,7 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     p.q = qn;
     // the activations' fp16 plane [M, K]: boxes of n_half rows x 64 elements, swizzled; rows beyond M are zero
     CUtensorMap tmB;
-    cuuint64_t dims[2] = {(cuuint64_t)K, (cuuint64_t)M};
-    cuuint64_t strides[1] = {(cuuint64_t)K * 2};
-    cuuint32_t box[2] = {64, p.pl.n_half};
-    cuuint32_t estr[2] = {1, 1};
-    if (mx_encode(&tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 2, plane, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) return FGMP_ERR_CUDA;
+    if (!fgmp_map_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, plane, M, K, K * 2, p.pl.n_half, 64)) return FGMP_ERR_CUDA;
 
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -6,6 +6,7 @@ import torch
 
 import fgmp_inputs as gi
 import oracle
+from test_gpu_calls import draw_acts, draw_weights
 from test_gpu_parity import GEMM_TOL, compare_packed, fg, quantize_both, tau_for_fraction   # noqa: F401  (fg is a fixture)
 
 pytestmark = pytest.mark.gpu
@@ -157,3 +158,21 @@ def test_selection_among_equal_scores(fg, rows, same):
         p = fg.quantize_weights(w.cuda(), fw.cuda(), clip_mode=0, fp8_fraction=frac)
         compare_packed(fg, p, q, None, f"frac={frac}")
         assert p.header()["n_fp8"] == q.mask_bits().sum()
+
+
+# Y leaves as tiles of 32 rows x 128 bytes where its rows are 16-byte aligned, by rows elsewhere and where it ends off such a boundary: ragged tiles in both
+# directions, a pitch wider than the result, whose other columns and the rows behind it stay as they were
+@pytest.mark.parametrize("M,N,K", [(385, 9864, 128), (1289, 4105, 64), (2305, 4096, 320)])
+@pytest.mark.parametrize("dtype,quantum", [(torch.bfloat16, 8), (torch.float32, 4)])
+def test_output_tiles(fg, M, N, K, dtype, quantum):
+    acts, w = draw_acts(fg, M, K, 71, 0.0), draw_weights(fg, N, K, 72, 0.0)
+    aligned = (N + quantum - 1) // quantum * quantum + quantum
+    wide, odd = (torch.full((M + 3, ld), -7.0, dtype=dtype, device="cuda") for ld in (aligned, aligned + 1))
+    count = launches(fg, lambda: fg.linear(acts, w, out=wide[:M, :N]))
+    assert count.get("gemm_nvfp4_tcgen05") == 1, count
+    fg.linear(acts, w, out=odd[:M, :N])
+    fg.check(fg.linear.last_workspace)
+    assert fg.linear.last_workspace[8:12].view(torch.int32).item() == 1, "the all-NVFP4 GEMM has made the result"
+    assert torch.equal(wide[:M, :N], odd[:M, :N]) and bool((wide[:M, :N] != -7.0).any(dim=0).all())
+    for y in (wide, odd):
+        assert bool((y[M:] == -7.0).all()) and bool((y[:, N:] == -7.0).all()), "stored outside the output"
