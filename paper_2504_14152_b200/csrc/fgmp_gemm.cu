@@ -85,7 +85,9 @@ __device__ __forceinline__ void expand_block(const ExpandParams& p, UnitScratch&
         const uint32_t* pmask = reinterpret_cast<const uint32_t*>(p.ablob + L.off_mask);
         const uint32_t f8 = pow2_f16x2(p.cls_a ? 0 : h->fp8_log2_ratio), one = pow2_f16x2(0), KB = (uint32_t)L.KB;
         // four blocks per thread, the loads of all of them before the first is converted
-        const uint64_t b0 = (uint64_t)(block - p.w_blocks) * 512 + threadIdx.x, nblk = (uint64_t)p.M * KB;
+        const uint64_t base = (uint64_t)(block - p.w_blocks) * 512, b0 = base + threadIdx.x, nblk = (uint64_t)p.M * KB;
+        // (one division of 64 bits, the same for all; the threads divide 32 bits)
+        const uint32_t base_row = (uint32_t)(base / KB), base_kb = (uint32_t)(base - (uint64_t)base_row * KB);
         uint32_t word[4], sf[4];
         uint2 c4[4];
         uint4 c8[4];
@@ -94,7 +96,7 @@ __device__ __forceinline__ void expand_block(const ExpandParams& p, UnitScratch&
             const uint64_t b = b0 + 128 * i;
             word[i] = 0; sf[i] = 0; c4[i] = make_uint2(0u, 0u);
             if (b < nblk) {
-                const uint32_t r = (uint32_t)(b / KB), kb = (uint32_t)(b - (uint64_t)r * KB);
+                const uint32_t o = base_kb + threadIdx.x + 128 * i, down = o / KB, r = base_row + down, kb = o - down * KB;
                 word[i] = (__ldg(pmask + (size_t)r * L.MW + (kb >> 5)) >> (kb & 31)) & 1u;
                 sf[i] = __ldg(p.ablob + L.off_sf + fgmp_sf_offset(r, kb, p.K));
                 c4[i] = __ldg(reinterpret_cast<const uint2*>(p.ablob + L.off_codes4 + (size_t)b * 8));
@@ -535,12 +537,12 @@ static fgmp_status launch_pair_gemm(const GemmParams& p, const uint8_t* planeA, 
     return fgmp_launch_status();
 }
 
-// Modelled time in us of expansion and pair GEMM, beside fgmp_mixed_us (measured calls are 0 to 20 % shorter): launches and tails, 0.65 us per million elements of
-// either operand, then waves of 256 x 256 tiles over the pairs at 0.34 us per 64 elements of K.
+// Modelled time in us of expansion and pair GEMM, beside fgmp_mixed_us: launches and tails, 0.5 us per million elements of either operand, then waves of
+// 256 x 256 tiles over the pairs at 0.32 us per 64 elements of K (13 shapes from 128 to 2048 tokens: within 10 %).
 static double planes_us(int64_t M, int64_t N, int64_t K)
 {
     const int64_t tiles = ((M + P_BM - 1) / P_BM) * ((N + P_BN - 1) / P_BN), pairs = fgmp_sm_count() / 2;
-    return 10.0 + 0.65e-6 * (double)(M + N) * (double)K + (double)((tiles + pairs - 1) / pairs) * (double)(K / 64) * 0.34;
+    return 8.0 + 0.5e-6 * (double)(M + N) * (double)K + (double)((tiles + pairs - 1) / pairs) * (double)(K / 64) * 0.32;
 }
 
 // M > 16 or a shape the weight-streaming kernel does not take.  nvfp4: what the caller expects of the operands, see fgmp_linear_expect.

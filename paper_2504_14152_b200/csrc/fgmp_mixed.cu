@@ -8,25 +8,27 @@
 // its 128-row operand from.  What bounds what:
 //   - expanding the weights to a plane first costs 2.7 bytes written and read for every packed byte, which is the whole
 //     call at small batches (4096 x 4096, 48 tokens: 59 us with the plane);
-//   - a 128 x 256 unit of weights takes about 1000 clocks of the SIMT pipes (1024 conversions at one per clock), its MMAs 16 of
-//     N/2 clocks for N tokens;
+//   - a 128 x 256 unit of weights takes 1024 clocks of the SIMT pipes at least (256 conversions and 128 multiplies per scheduler, two clocks each),
+//     its MMAs 16 of N/2 clocks for N tokens;
 //   - the operand from tensor memory leaves shared memory to the token tiles (from shared memory the 64 KiB of a
 //     dequantized unit would be written and read there, 1024 clocks by themselves);
-//   - a unit takes 1.08 us + 4.2 ns per token, more than its MMAs (4.3 ns per token) or its dequantization: with either of them or
-//     the token copies left out it is 7 to 20 % faster, with all of them left out 27 %.  What remains is the way of a slot through
-//     three groups of warps (copy, dequantize, multiply, release), some 2000 clocks, and at full rate the token tiles would
-//     take 64 bytes per clock and SM from L2.  Four groups, CTA pairs that share a token tile, more weight stages, spinning
-//     instead of suspended waits and a loop of one elected thread in the issuer were measured and are no faster.
-//   - so a unit is worth as many tokens as fit: up to 416 (two MMAs side by side on one dequantized operand) where a CTA's share lies within
-//     a tile (400 x 11008 x 4096: 48 us, 54 with two tiles of 208; 1200 x 4096 x 4096: 52 and 57).
+//   - the issuer and the dequantizing warps share their schedulers, so that a unit costs what its instructions cost to issue: 1380 per scheduler
+//     before, 1200 now.  Hence steps of 128 elements (half as many waits and commits), one wait and one commit for a step's weights and tokens
+//     together, the FP8 blocks' conversions and loads under one predicate with the microscale or the FP8 factor chosen per block, and groups that
+//     pass over units none of whose steps is theirs.  64 x 28672 x 8192 a call: 91 -> 65 us (1.05 us a unit);
+//   - beyond 160 tokens the token tiles: 12 TB/s come out of L2 then, 45 bytes a clock and SM (64 would be needed at full MMA rate), and a second
+//     accumulator no longer fits beside the slots.  So 160 tokens are the most for the time a unit takes (777 x 11008 x 4096: five tiles of 160 as
+//     whole tiles 60 us, four of 208 in spans 77).
+// Four groups, CTA pairs that share a token tile, spinning instead of suspended waits and a loop of one elected thread in the issuer were measured
+// and are no faster.
 //
 // Work is (weight tile, token tile, 256-element K chunk) units in that order, split over the CTAs either in
-// equal contiguous spans (stream-K: the partial sums of tiles shared by several CTAs are stored column by column and added
+// equal contiguous spans (stream-K: the partial sums of tiles shared by several CTAs are stored, eight columns of a row at a time, and added
 // up in CTA order by a kernel of their own, which has the whole chip's loads in flight: 43 MB at 203 tokens and 13824 weight
 // rows, 20 us if the CTA that arrives last does it) or in whole tiles, whichever the model in mixed_plan says is faster.
 //
 // Warp roles: warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, warp 2 = token-tile producer,
-// warps 3-6 = epilogue, then the dequantization, NG groups of four warps that take the steps of 64 elements in turn.  Every
+// warps 3-6 = epilogue, then the dequantization, NG groups of four warps that take the steps in turn.  Every
 // wait is bounded.
 #include <cuda.h>
 #include <cuda_fp16.h>
@@ -45,7 +47,7 @@ constexpr int MX_THREADS = 32 * (W_DEQ + 4 * MX_GROUPS);
 constexpr uint32_t STG_MASK = REC_BYTES, STG_HALF = STG_MASK + 256;      // a weight stage: record, mask, second halves of the FP8 blocks
 constexpr uint32_t HALF_CAP = 5248;             // 656 FP8 blocks (32 %); with more the halves are read from global memory
 constexpr uint32_t WSTAGE = STG_HALF + HALF_CAP;                         // 24064
-constexpr int MAX_WSTAGES = 4, MAX_BSTAGES = 12, MAX_SLOTS = 8;
+constexpr int MAX_WSTAGES = 4, MAX_STEPS = 12, MAX_SLOTS = 8;
 constexpr uint32_t MX_TMEM_COLS = 512;
 constexpr uint32_t MX_MAX_TOK = 416;            // tokens of a tile: columns of its accumulator, beside three slots of 32
 constexpr size_t MX_SMEM_LIMIT = 232448;
@@ -58,7 +60,9 @@ struct MixedPlan {
     uint32_t chunks, tiles;              // tiles = wtiles * tok_tiles
     uint32_t grid, span, rest, quantum;  // a CTA's span in quanta of `quantum` units (1, or chunks: whole tiles)
     uint32_t split;                      // 1: some tile is shared by several CTAs, whose parts are added up behind this kernel
-    uint32_t wstages, bstages, slots, naccs;
+    uint32_t ks;                         // steps of 64 elements of K that are handed to the MMA issuer at once (1 or 2)
+    uint32_t wstages, slots, naccs;
+    uint32_t ring;                       // token stages, of ks steps each
     double us;                           // modelled time
 };
 
@@ -135,6 +139,21 @@ __device__ __forceinline__ void mixed_emit(const MixedParams& p, const uint32_t 
     }
 }
 
+__device__ __forceinline__ void store_parts8(float* dst, const uint32_t* v)
+{
+    asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+
+__device__ __forceinline__ void add_parts8(const float* src, float* s)
+{
+    uint32_t x[8];
+    asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]) : "l"(src) : "memory");
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s[j] += __uint_as_float(x[j]);
+}
+
 // Epilogue warps: tensor-memory lane quadrant warp % 4, lane = weight row, column = token
 template <bool QUANT>
 __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tmem_base, int warp, int lane, uint32_t u_begin, uint32_t u_end,
@@ -155,7 +174,7 @@ __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tm
         if (!mbar_wait_warp(accf0 + 8 * acc, acc_phase, abort_flag, p.status, 8)) break;
         tc_fence_after();
         const uint32_t d = tmem_base + ((q * 32u) << 16) + acc * NT;
-        float* mine = p.parts + ((size_t)(blockIdx.x * 2 + which)) * NP * 128 + row;
+        float* mine = p.parts + ((size_t)(blockIdx.x * 2 + which)) * NP * 128 + row * 8;        // eight columns of all rows, then the next eight
 #pragma unroll 1
         for (uint32_t cc = 0; cc < NT; cc += 32) {
                 uint32_t v[32];
@@ -163,7 +182,7 @@ __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tm
                 if (whole) mixed_emit<QUANT>(p, v, n, m0, cc, alpha, lane, turn);
                 else
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) __stcg(mine + (cc + j) * 128, __uint_as_float(v[j]));
+                    for (int j = 0; j < 32; j += 8) store_parts8(mine + (cc + j) * 128, v + j);
             }
         tc_fence_before();
         __syncwarp();
@@ -172,45 +191,43 @@ __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tm
     }
 }
 
-// QUANT: the next layer's activation quantizer in the epilogue instead of Y.
-template <bool QUANT>
+// QUANT: the next layer's activation quantizer in the epilogue instead of Y.  KS: MixedPlan::ks.
+template <bool QUANT, uint32_t KS>
 __global__ void __launch_bounds__(MX_THREADS, 1)
 mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ MixedParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
     const MixedPlan& pl = p.pl;
-    const uint32_t BS = pl.bstages, WS = pl.wstages, R = pl.slots, NT = pl.n_tok, C = pl.chunks;
+    const uint32_t L = pl.ring, WS = pl.wstages, R = pl.slots, NT = pl.n_tok, C = pl.chunks;
     // (no more groups than slots: a group that was further ahead could take an older phase of a slot's barrier for the one it waits for)
     const uint32_t NG = min((uint32_t)MX_GROUPS, R);
     const uint32_t NH = pl.n_half;
-    const uint32_t b_bytes = (NT > NH ? 2u : 1u) * NH * 128u;   // token stage: rows of 64 elements, swizzled (a multiple of 2 KiB)
-    uint8_t* wst0 = smem + BS * b_bytes;
+    const uint32_t b_bytes = (NT > NH ? 2u : 1u) * NH * 128u;   // tokens of a step of 64 elements: rows, swizzled (a multiple of 2 KiB)
+    uint8_t* wst0 = smem + L * KS * b_bytes;
     uint8_t* extra = wst0 + WS * WSTAGE;                 // QUANT: 4 x 32 x 33 floats
     uint64_t* bars = reinterpret_cast<uint64_t*>(extra + (QUANT ? 4 * 32 * 33 * 4 + 128 : 0));
-    uint32_t* wmeta = reinterpret_cast<uint32_t*>(bars + 2 * MAX_WSTAGES + 2 * MAX_BSTAGES + MAX_SLOTS + 4);   // per stage: list start, bytes of it there
+    uint32_t* wmeta = reinterpret_cast<uint32_t*>(bars + 2 * MAX_WSTAGES + 2 * MAX_STEPS + 4);   // per stage: list start, bytes of it there
     uint32_t* tmem_slot = wmeta + MAX_WSTAGES * 2;
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = warp_index(), lane = threadIdx.x & 31;
-    // The MMA issuer is a single thread whose every wait (75 clocks) and commit (40) comes on top of 40 clocks per MMA, so it has
-    // one of each per step of 64 elements: step i is ready (barrier i % R) when the dequantized weights are in tensor
-    // memory and the warps that put them there have seen the token tile of the step; when it is done (barrier i % L, L the
-    // longer of the two rings), both its slot and its token stage are free.
-    // barriers: weight stage full / empty, token stage full; step ready, step done; accumulators full / empty
-    const uint32_t wf0 = smem_u32(bars), we0 = wf0 + 8 * MAX_WSTAGES, bf0 = we0 + 8 * MAX_WSTAGES, dn0 = bf0 + 8 * MAX_BSTAGES;
-    const uint32_t sf0 = dn0 + 8 * MAX_BSTAGES, accf0 = sf0 + 8 * MAX_SLOTS, acce0 = accf0 + 16;
-    const uint32_t L = max(R, BS);
-    const uint32_t slot_col = pl.naccs * NT;             // tensor memory: accumulators of NT columns, then slots of 32
+    // Steps of KS times 64 elements go round a ring of L token stages and one of R <= L slots of dequantized weights in tensor memory.  The MMA
+    // issuer has one wait and one commit for a step: it is ready when its token tiles and its weights are there, and done when both its stage and its
+    // slot are free.
+    // barriers: weight stage full / empty, step ready / done, accumulators full / empty
+    const uint32_t wf0 = smem_u32(bars), we0 = wf0 + 8 * MAX_WSTAGES, rd0 = we0 + 8 * MAX_WSTAGES, dn0 = rd0 + 8 * MAX_STEPS;
+    const uint32_t accf0 = dn0 + 8 * MAX_STEPS, acce0 = accf0 + 16;
+    const uint32_t slot_col = pl.naccs * NT;             // tensor memory: accumulators of NT columns, then slots of 32 KS
 
     const uint32_t u_begin = unit_begin(pl, blockIdx.x), u_end = unit_begin(pl, blockIdx.x + 1);
-    const uint32_t last_steps = (uint32_t)(p.K / 64) - 4u * (C - 1u);
+    // steps (of KS times 64 elements) of a chunk, and of the last one: what of its last step lies beyond K is zeros
+    constexpr uint32_t STEPS = 4 / KS;
+    const uint32_t last_steps = ((uint32_t)(p.K / 64) - 4u * (C - 1u) + KS - 1u) / KS;
 
     if (threadIdx.x == 0) {
         for (uint32_t s = 0; s < WS; ++s) { mbar_init(wf0 + 8 * s, 1); mbar_init(we0 + 8 * s, 4 * NG); }
-        for (uint32_t s = 0; s < BS; ++s) mbar_init(bf0 + 8 * s, 1);
-        for (uint32_t s = 0; s < L; ++s) mbar_init(dn0 + 8 * s, 1);
-        for (uint32_t s = 0; s < R; ++s) mbar_init(sf0 + 8 * s, 4);
+        for (uint32_t s = 0; s < L; ++s) { mbar_init(rd0 + 8 * s, 5); mbar_init(dn0 + 8 * s, 1); }      // (four warps, and the copies)
         for (uint32_t t = 0; t < pl.naccs; ++t) { mbar_init(accf0 + 8 * t, 1); mbar_init(acce0 + 8 * t, 4); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -225,7 +242,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     // The weights go in over 2^t: an FP8 block needs no factor then if t is the ratio of its tensor scale to the NVFP4 one,
     // and fp16 holds every NVFP4 value (up to 2688) over 2^t as long as t >= -4.
     const int t_w = max(ratio_w, -4);
-    const bool has_fp8 = __ldg(&hw->n_fp8) != 0, may_skip = p.leave_nvfp4 && !has_fp8;
+    const bool may_skip = p.leave_nvfp4 && __ldg(&hw->n_fp8) == 0;
 
     if (warp == W_PROD) {
         // ------------------------------------------------------------ weights producer (whole warp; lane 0 issues)
@@ -241,8 +258,8 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
             asm volatile("griddepcontrol.wait;" ::: "memory");
             if (p.ha->n_fp8 == 0) ok = 0;
         }
+        uint32_t c = u_begin % C, tile = u_begin / C, rec = tile / pl.tok_tiles * C + c;
         for (uint32_t u = u_begin; u < u_end && ok; ++u, ++issued) {
-            const uint32_t c = u % C, tile = u / C / pl.tok_tiles, rec = tile * C + c;
             if (issued == WS && !waited) {
                 // the status word may be looked at once the preceding kernel is done
                 asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -263,13 +280,17 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (++stage == WS) { stage = 0; phase ^= 1; }
+            ++rec;
+            if (++c == C) { c = 0; rec = ++tile / pl.tok_tiles * C; }
         }
         if (!waited) asm volatile("griddepcontrol.wait;" ::: "memory");
         if (bad && lane == 0) { *abort_flag = 1; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, 12); }
-    } else {
+    } else if (may_skip || (warp < W_DEQ && warp != W_MMA)) {
+        if (warp == W_TOK && lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");
         asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
+    // (The weights are dequantized before the kernel in front is done, as far as there are slots: only the tokens are its.)
     if (QUANT && blockIdx.x == 0 && threadIdx.x == 32 * W_EPI) {
         fgmp_packed_header* h = p.q.header;
         h->magic = FGMP_MAGIC; h->version = FGMP_LAYOUT_VERSION; h->rows = p.M; h->K = p.N; h->scale_fp4 = p.q.s4;
@@ -283,164 +304,151 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     } else if (warp == W_TOK) {
         // ------------------------------------------------------------ token-tile producer
         if (lane == 0) {
-            uint32_t stage = 0, ds = 0, dph = 0, i = 0;  // ds: barrier of step i - BS
+            uint32_t stage = 0, phase = 1, c = u_begin % C, tok = u_begin / C % pl.tok_tiles;
             bool ok = true;
             for (uint32_t u = u_begin; u < u_end && ok; ++u) {
-                const uint32_t c = u % C, m0 = (u / C) % pl.tok_tiles * NT, steps = c == C - 1 ? last_steps : 4u;
-                for (uint32_t s = 0; s < steps; ++s, ++i) {
-                    if (i >= BS) {
-                        if (!(ok = mbar_wait(dn0 + 8 * ds, dph, abort_flag, p.status, 2))) break;
-                        if (++ds == L) { ds = 0; dph ^= 1; }
+                const uint32_t m0 = tok * NT, steps = c == C - 1 ? last_steps : STEPS;
+                for (uint32_t s = 0; s < steps; ++s) {
+                    if (!(ok = mbar_wait(dn0 + 8 * stage, phase, abort_flag, p.status, 2))) break;
+                    const uint32_t bar = rd0 + 8 * stage, dst = smem_u32(smem) + stage * (KS * b_bytes);
+                    mbar_expect_tx(bar, KS * b_bytes);
+#pragma unroll
+                    for (uint32_t h = 0; h < KS; ++h) {
+                        const int32_t k = (int32_t)(c * 256 + (s * KS + h) * 64);        // (beyond K: zeros)
+                        tma_load_2d(dst + h * b_bytes, &tmB, k, (int32_t)m0, bar);
+                        if (NT > NH) tma_load_2d(dst + h * b_bytes + NH * 128u, &tmB, k, (int32_t)(m0 + NH), bar);
                     }
-                    mbar_expect_tx(bf0 + 8 * stage, b_bytes);
-                    tma_load_2d(smem_u32(smem + stage * b_bytes), &tmB, (int32_t)(c * 256 + s * 64), (int32_t)m0, bf0 + 8 * stage);
-                    if (NT > NH) tma_load_2d(smem_u32(smem + stage * b_bytes) + NH * 128u, &tmB, (int32_t)(c * 256 + s * 64), (int32_t)(m0 + NH), bf0 + 8 * stage);
-                    if (++stage == BS) stage = 0;
+                    if (++stage == L) { stage = 0; phase ^= 1; }
                 }
+                if (++c == C) { c = 0; if (++tok == pl.tok_tiles) tok = 0; }
             }
         }
         __syncwarp();
     } else if (warp == W_MMA) {
-        // ------------------------------------------------------------ MMA issuer (one elected lane)
-        {
-            const uint32_t idesc = IDESC_F16 | ((NH >> 3) << 17) | ((128u >> 4) << 24), idesc2 = IDESC_F16 | (((NT - NH) >> 3) << 17) | ((128u >> 4) << 24), b_first = (smem_u32(smem) >> 4) | SW128_LO, b_step = b_bytes >> 4;
-            uint32_t bst = 0, slot = 0, sph = 0, ds = 0, c = u_begin % C, acc = 0, acc_phase = 1, accum = 0, b_lo = b_first;
-            bool ok = true, ready = false;
-            for (uint32_t u = u_begin; u < u_end && ok; ++u) {
-                const uint32_t steps = c == C - 1 ? last_steps : 4u, d = tmem_base + acc * NT;
-                const bool last_unit = c == C - 1 || u + 1 == u_end;
-                if (accum == 0 && !mbar_wait_uniform(acce0 + 8 * acc, acc_phase, abort_flag, p.status, 4)) break;
-                for (uint32_t s = 0; s < steps; ++s) {
-                    if (!ready && !(ok = mbar_wait_uniform(sf0 + 8 * slot, sph, abort_flag, p.status, 5))) break;
-                    tc_fence_after();
-                    const uint32_t a = tmem_base + slot_col + slot * 32;
-                    if (++slot == R) { slot = 0; sph ^= 1; }
-                    const bool peek = mbar_test_wait(sf0 + 8 * slot, sph);      // the next step's; the answer comes while this one's MMAs are issued
-                    if (elect_one()) {
+        // ------------------------------------------------------------ MMA issuer (the whole warp walks the loop, an elected lane issues)
+        const uint32_t idesc = IDESC_F16 | ((NH >> 3) << 17) | ((128u >> 4) << 24), idesc2 = IDESC_F16 | (((NT - NH) >> 3) << 17) | ((128u >> 4) << 24);
+        const uint32_t b_first = (smem_u32(smem) >> 4) | SW128_LO, b_step = b_bytes >> 4, a_first = tmem_base + slot_col;
+        uint32_t stage = 0, phase = 0, slot = 0, acc = 0, acc_phase = 1, b_lo = b_first, a = a_first;
+        bool ok = true, ready = false;
+        for (uint32_t u = u_begin; u < u_end && ok;) {
+            // the steps of one tile
+            const uint32_t t_end = (u / C + 1) * C, seg_end = min(t_end, u_end), d = tmem_base + acc * NT;
+            uint32_t left = (seg_end - u) * STEPS - (seg_end == t_end ? STEPS - last_steps : 0u), accum = 0;
+            u = seg_end;
+            if (!mbar_wait_uniform(acce0 + 8 * acc, acc_phase, abort_flag, p.status, 4)) break;
+            for (; left; --left) {
+                if (!ready && !(ok = mbar_wait_uniform(rd0 + 8 * stage, phase, abort_flag, p.status, 5))) break;
+                tc_fence_after();
+                const uint32_t done = dn0 + 8 * stage, b = b_lo;
+                b_lo += KS * b_step;
+                if (++stage == L) { stage = 0; phase ^= 1; b_lo = b_first; }
+                const bool peek = mbar_test_wait(rd0 + 8 * stage, phase);     // the next step's; the answer comes while this one's MMAs are issued
+                if (elect_one()) {
 #pragma unroll
-                        for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d, a + 8 * k, mx_desc(b_lo + 2 * k), idesc, k ? 1u : accum);
+                    for (uint32_t h = 0; h < KS; ++h) {
+#pragma unroll
+                        for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d, a + 32 * h + 8 * k, mx_desc(b + h * b_step + 2 * k), idesc, h + k ? 1u : accum);
                         if (NT > NH) {
 #pragma unroll
-                            for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d + NH, a + 8 * k, mx_desc(b_lo + NH * 8u + 2 * k), idesc2, k ? 1u : accum);
+                            for (uint32_t k = 0; k < 4; ++k) umma_f16_ta(d + NH, a + 32 * h + 8 * k, mx_desc(b + h * b_step + NH * 8u + 2 * k), idesc2, h + k ? 1u : accum);
                         }
-                        umma_commit(dn0 + 8 * ds);
                     }
-                    accum = 1;
-                    b_lo += b_step;
-                    if (++bst == BS) { bst = 0; b_lo = b_first; }
-                    if (++ds == L) ds = 0;
-                    ready = __all_sync(0xffffffffu, peek);
+                    umma_commit(done);
+                    if (left == 1) umma_commit(accf0 + 8 * acc);
                 }
-                if (last_unit) {
-                    if (elect_one()) umma_commit(accf0 + 8 * acc);
-                    __syncwarp();
-                    accum = 0;
-                    if (++acc == pl.naccs) { acc = 0; acc_phase ^= 1; }
-                }
-                if (++c == C) c = 0;
+                accum = 1; a += 32 * KS;
+                if (++slot == R) { slot = 0; a = a_first; }
+                ready = __all_sync(0xffffffffu, peek);
             }
+            if (++acc == pl.naccs) { acc = 0; acc_phase ^= 1; }
         }
         __syncwarp();
     } else if (warp >= W_DEQ + 4 * (int)NG) {
     } else if (warp >= W_DEQ) {
         // ------------------------------------------------------------ dequantization: thread = row of the weight tile
-        // The groups take the steps of 64 elements in turn.
+        // The groups take the steps in turn.
         const uint32_t group = (uint32_t)(warp - W_DEQ) >> 2, row = 32u * (warp & 3) + lane, r7 = row & 7u;
         const uint32_t quadrant = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + slot_col;
         const __half2 inv2 = __float2half2_rn(__int_as_float((127 - t_w) << 23)), f82 = __float2half2_rn(__int_as_float((127 + ratio_w - t_w) << 23));
         const uint32_t inv = *reinterpret_cast<const uint32_t*>(&inv2), f8 = *reinterpret_cast<const uint32_t*>(&f82);
-        const bool scaled8 = ratio_w != t_w;             // (for every thread alike)
+        // masks of the rows of an octet that lie before this one, two to a word
+        const auto pair_before = [&](uint32_t i) { return r7 > 2 * i + 1 ? 0xffffffffu : r7 > 2 * i ? 0xffffu : 0u; };
+        const uint32_t rows01 = pair_before(0), rows23 = pair_before(1), rows45 = pair_before(2), rows67 = pair_before(3);
         uint32_t stage = 0, phase = 0, c = u_begin % C, slot = group, next = group;    // next: steps until the group's turn
-        uint32_t bst = group, bph = 0, ds = 0, dph = 0, i = group;        // i: the step; ds: barrier of step i - R
-        while (bst >= BS) { bst -= BS; bph ^= 1; }
+        uint32_t st = group, ds = L - R + group, dph = 1;     // ring positions of the group's step and of the one R before it, whose slot it takes
         bool ok = true;
         for (uint32_t u = u_begin; u < u_end && ok; ++u) {
-            const uint32_t steps = c == C - 1 ? last_steps : 4u;
+            const uint32_t steps = c == C - 1 ? last_steps : STEPS;
+            if (next >= steps) {                         // none of the unit's steps is the group's
+                next -= steps;
+                // (one lane waits all the same: an arrival must not be taken for one of the stage's unit before)
+                if (lane == 0 && (ok = mbar_wait(wf0 + 8 * stage, phase, abort_flag, p.status, 6))) mbar_arrive(we0 + 8 * stage);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                if (++stage == WS) { stage = 0; phase ^= 1; }
+                if (++c == C) c = 0;
+                continue;
+            }
             if (!(ok = mbar_wait_warp(wf0 + 8 * stage, phase, abort_flag, p.status, 6))) break;
             const uint8_t* sp = wst0 + stage * WSTAGE;
-            uint32_t mt = 0, at = 0;
-            bool all = true;
-            if (has_fp8) {
-                // the row's FP8 blocks lie one after the other in the list
-                const uint16_t* before = reinterpret_cast<const uint16_t*>(sp + REC_KBSTART);
-                mt = reinterpret_cast<const uint16_t*>(sp + STG_MASK)[row];
-                at = __popc(mt);
-#pragma unroll
-                for (int o = 1; o < 8; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, at, o, 8); if ((lane & 7) >= o) at += y; }
-                at = 8u * (before[row >> 3] + at - __popc(mt));
-                all = 8u * before[16] <= wmeta[stage * 2 + 1];
-            }
+            // The row's FP8 blocks lie one after the other in the list, behind those of the rows before: of every eight rows that is written in
+            // the record, the rest are counted in the masks of the row's own eight.
+            const uint16_t* before = reinterpret_cast<const uint16_t*>(sp + REC_KBSTART);
+            const uint4 m8 = reinterpret_cast<const uint4*>(sp + STG_MASK)[row >> 3];
+            const uint32_t mt = reinterpret_cast<const uint16_t*>(sp + STG_MASK)[row], sb = smem_u32(sp);
+            const uint32_t half0 = sb + STG_HALF + 8u * (before[row >> 3] + __popc(m8.x & rows01) + __popc(m8.y & rows23) + __popc(m8.z & rows45) + __popc(m8.w & rows67));
+            const bool all = 8u * before[16] <= wmeta[stage * 2 + 1];
+            const uint32_t row16 = sb + row * 128u + (r7 << 4), sfw = sb + REC_SF + (row & 31u) * 16u + (row >> 5) * 4u;      // (sb: a multiple of 128)
 #pragma unroll 1
-            for (; next < steps; next += NG) {
-                const uint32_t s = next;
-                uint32_t r[32];
-                const uint32_t sb = smem_u32(sp), codes = sb + row * 128u, sfw = sb + REC_SF + (row & 31u) * 16u + (row >> 5) * 4u;
-                const uint32_t m16 = mt >> (4 * s);
-                uint32_t hg = at + 8u * __popc(mt & ((1u << (4 * s)) - 1u)), hs = sb + STG_HALF + hg;
-                uint4 q0, q1;
-                uint32_t sc;
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q0.x), "=r"(q0.y), "=r"(q0.z), "=r"(q0.w) : "r"(codes + (((2 * s) ^ r7) << 4)));
-                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q1.x), "=r"(q1.y), "=r"(q1.z), "=r"(q1.w) : "r"(codes + (((2 * s + 1) ^ r7) << 4)));
-                asm volatile("ld.shared.b32 %0, [%1];" : "=r"(sc) : "r"(sfw + 512u * s));
-                const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-                uint2 hi[4];
+            for (; next < steps && ok; next += NG) {
+#pragma unroll 1
+                for (uint32_t h = 0; h < KS; ++h) {
+                    const uint32_t s = KS * next + h, at16 = row16 ^ (s << 5), m4 = mt >> (4 * s);
+                    uint32_t r[32], d[4], sc, hs = half0 + 8u * __popc(mt & ((1u << (4 * s)) - 1u));
+                    uint4 q0, q1;
+                    uint2 hi[4];
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q0.x), "=r"(q0.y), "=r"(q0.z), "=r"(q0.w) : "r"(at16));
+                    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(q1.x), "=r"(q1.y), "=r"(q1.z), "=r"(q1.w) : "r"(at16 ^ 16u));
+                    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(sc) : "r"(sfw + 512u * s));
+                    const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+                    const uint32_t d01 = hmul2(e4m3x2_to_f16x2(sc & 0xffffu), inv), d23 = hmul2(e4m3x2_to_f16x2(sc >> 16), inv);
+                    d[0] = __byte_perm(d01, 0, 0x1010); d[1] = __byte_perm(d01, 0, 0x3232); d[2] = __byte_perm(d23, 0, 0x1010); d[3] = __byte_perm(d23, 0, 0x3232);
+                    // E4M3 codes 0..7 of an FP8 block in the slot, 8..15 in the list, and its factor instead of the microscale; under a
+                    // predicate, not branched to: with 10 % FP8 blocks some row of a warp has one in nearly every column
+                    if (all) {
 #pragma unroll
-                for (uint32_t k = 0; k < 4; ++k) {
-                    const uint32_t is8 = (m16 >> k) & 1u;
-                    hi[k] = lds64_if(hs, is8 && all);
-                    hs += 8u * is8;
-                }
-                if (!all) {
-                    const uint8_t* half_g = p.wblob + p.LW.off_ovf + (size_t)wmeta[stage * 2] * 16;
+                        for (uint32_t k = 0; k < 4; ++k) fp8_half(m4, 1u << k, hs, hi[k], d[k], f8);
+                    } else {
+                        const uint8_t* half_g = p.wblob + p.LW.off_ovf + (size_t)wmeta[stage * 2] * 16 + (hs - (smem_u32(sp) + STG_HALF));
 #pragma unroll
-                    for (uint32_t k = 0; k < 4; ++k)
-                        if ((m16 >> k) & 1u) { hi[k] = __ldg(reinterpret_cast<const uint2*>(half_g + hg)); hg += 8u; }
-                    __syncwarp();
-                }
-                const uint32_t d01 = hmul2(e4m3x2_to_f16x2(sc & 0xffffu), inv), d23 = hmul2(e4m3x2_to_f16x2(sc >> 16), inv);
-                const uint32_t d[4] = {__byte_perm(d01, 0, 0x1010), __byte_perm(d01, 0, 0x3232), __byte_perm(d23, 0, 0x1010), __byte_perm(d23, 0, 0x3232)};
-#pragma unroll
-                for (uint32_t k = 0; k < 4; ++k) {
-                    e2m1x8_to_f16(w[2 * k], r + 8 * k); e2m1x8_to_f16(w[2 * k + 1], r + 8 * k + 4);
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) r[8 * k + e] = hmul2(r[8 * k + e], d[k]);
-                }
-                if (has_fp8) {
-                    // E4M3 codes 0..7 in the slot, 8..15 in the list; selected, not branched to: with 10 % FP8 blocks some
-                    // row of a warp has one in nearly every column
+                        for (uint32_t k = 0; k < 4; ++k)
+                            if ((m4 >> k) & 1u) { hi[k] = __ldg(reinterpret_cast<const uint2*>(half_g)); half_g += 8; d[k] = f8; }
+                        __syncwarp();
+                    }
 #pragma unroll
                     for (uint32_t k = 0; k < 4; ++k) {
-                        const bool is8 = (m16 >> k) & 1u;
-                        const uint32_t v[4] = {w[2 * k], w[2 * k + 1], hi[k].x, hi[k].y};
+                        e2m1x8_to_f16(w[2 * k], r + 8 * k); e2m1x8_to_f16(w[2 * k + 1], r + 8 * k + 4);
+                        e4m3x16_to_f16_if(m4, 1u << k, w[2 * k], w[2 * k + 1], hi[k].x, hi[k].y, r + 8 * k);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            uint32_t a = e4m3x2_to_f16x2(v[e] & 0xffffu), b = e4m3x2_to_f16x2(v[e] >> 16);
-                            if (scaled8) { a = hmul2(a, f8); b = hmul2(b, f8); }
-                            r[8 * k + 2 * e] = is8 ? a : r[8 * k + 2 * e];
-                            r[8 * k + 2 * e + 1] = is8 ? b : r[8 * k + 2 * e + 1];
-                        }
+                        for (int e = 0; e < 8; ++e) r[8 * k + e] = hmul2(r[8 * k + e], d[k]);
                     }
+                    __syncwarp();
+                    if (h == 0) {
+                        if (!(ok = mbar_wait_warp(dn0 + 8 * ds, dph, abort_flag, p.status, 7))) break;
+                        tc_fence_after();
+                    }
+                    tmem_st32(quadrant + slot * (32 * KS) + 32 * h, r);
                 }
-                __syncwarp();
-                if (i >= R) {
-                    if (i < R + NG) ds = (i - R) % L;              // the group's first wait
-                    if (!(ok = mbar_wait_warp(dn0 + 8 * ds, dph, abort_flag, p.status, 7))) break;
-                    tc_fence_after();
-                    ds += NG;
-                    if (ds >= L) { ds -= L; dph ^= 1; }
-                }
-                tmem_st32(quadrant + slot * 32, r);
+                if (!ok) break;
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0 && mbar_wait(bf0 + 8 * bst, bph, abort_flag, p.status, 3)) mbar_arrive(sf0 + 8 * slot);
-                __syncwarp();
-                i += NG;
-                slot += NG;
+                if (lane == 0) mbar_arrive(rd0 + 8 * st);
+                slot += NG; st += NG; ds += NG;
                 if (slot >= R) slot -= R;
-                bst += NG;
-                while (bst >= BS) { bst -= BS; bph ^= 1; }
+                if (st >= L) st -= L;
+                if (ds >= L) { ds -= L; dph ^= 1; }
             }
+            if (!ok) break;
             next -= steps;
             __syncwarp();
             if (lane == 0) mbar_arrive(we0 + 8 * stage);
@@ -464,8 +472,8 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     }
 }
 
-// Adds up the partial sums of the tiles that several CTAs share, in CTA order.  A block has 32 token columns of one weight
-// tile, a warp four of them, a lane four consecutive weight rows (QUANT: a warp has 32 rows, a lane a column).
+// Adds up the partial sums of the tiles that several CTAs share, in CTA order.  A block has 32 token columns of a weight tile.  Y: a thread adds
+// eight columns of two weight rows.  QUANT: a lane adds 32 columns of a row, turned round in shared memory to 32 rows of a column.
 template <bool QUANT>
 __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const __grid_constant__ MixedParams p)
 {
@@ -482,56 +490,56 @@ __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const _
     const fgmp_packed_header* hw = reinterpret_cast<const fgmp_packed_header*>(p.wblob);
     if (p.leave_nvfp4 && hw->n_fp8 == 0 && p.ha->n_fp8 == 0) return;
     const float alpha = __fmul_rn(__fmul_rn(p.ha->scale_fp4, hw->scale_fp4), __int_as_float((127 + max(hw->fp8_log2_ratio, -4)) << 23));
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;       // (a warp of QUANT: 32 weight rows)
     const int64_t m0 = (int64_t)(tile % pl.tok_tiles) * pl.n_tok, m_end = min(p.M, m0 + pl.n_tok);
     auto part = [&](uint32_t i) {
         return p.parts + ((size_t)((c_first + i) * 2 + (unit_begin(pl, c_first + i) >= t_begin ? 0u : 1u))) * NP * 128;
     };
     if (QUANT) {
-        const uint32_t col = blockIdx.y * 32 + lane;
-        const int64_t n = (int64_t)wt * 128 + 32 * warp;
+        __shared__ uint32_t turn_all[4 * 32 * 33];
+        uint32_t* turn = turn_all + warp * 32 * 33;
         float s[32];
 #pragma unroll
         for (int j = 0; j < 32; ++j) s[j] = 0.f;
-#pragma unroll 1
+#pragma unroll 2
         for (uint32_t i = 0; i < nseg; ++i) {
-            const float4* src = reinterpret_cast<const float4*>(part(i) + (size_t)col * 128 + 32 * warp);
+            const float* src = part(i) + (size_t)blockIdx.y * 4096 + (32 * warp + lane) * 8;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { const float4 x = __ldcg(src + j); s[4 * j] += x.x; s[4 * j + 1] += x.y; s[4 * j + 2] += x.z; s[4 * j + 3] += x.w; }
+            for (int j = 0; j < 4; ++j) add_parts8(src + j * 1024, s + 8 * j);
         }
+#pragma unroll
+        for (int j = 0; j < 32; ++j) turn[j * 33 + lane] = __float_as_uint(s[j]);
+        __syncwarp();
         uint32_t r[32];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(s[j]);
-        if (m0 + col < m_end && n < p.N) quantize_row32(p, m0 + col, n, r, alpha);
+        for (int j = 0; j < 32; ++j) r[j] = turn[lane * 33 + j];
+        const int64_t m = m0 + blockIdx.y * 32 + lane, n = (int64_t)wt * 128 + 32 * warp;
+        if (m < m_end && n < p.N) quantize_row32(p, m, n, r, alpha);
     } else {
-        const int64_t n = (int64_t)wt * 128 + 4 * lane;
-        float4 s[4];
+        const uint32_t row = (threadIdx.x & 63u) * 2, col = blockIdx.y * 32 + (threadIdx.x >> 6) * 8;
+        const int64_t n = (int64_t)wt * 128 + row, m = m0 + col;
+        float s[16];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) s[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int j = 0; j < 16; ++j) s[j] = 0.f;
 #pragma unroll 4
         for (uint32_t i = 0; i < nseg; ++i) {
-            const float4* src = reinterpret_cast<const float4*>(part(i) + (size_t)(blockIdx.y * 32 + warp * 4) * 128) + lane;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) { const float4 x = __ldcg(src + j * 32); s[j].x += x.x; s[j].y += x.y; s[j].z += x.z; s[j].w += x.w; }
+            const float* src = part(i) + (size_t)col * 128 + row * 8;
+            add_parts8(src, s); add_parts8(src + 8, s + 8);
         }
-        const bool wide = n + 4 <= p.N && (p.ldy & 3) == 0;      // (Y is 16-byte aligned)
+        if (n >= p.N) return;
+        const bool two = n + 1 < p.N, wide = two && (p.ldy & 1) == 0;      // (Y is 16-byte aligned)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int64_t m = m0 + blockIdx.y * 32 + warp * 4 + j;
-            if (m >= m_end) break;
-            const float v[4] = {s[j].x * alpha, s[j].y * alpha, s[j].z * alpha, s[j].w * alpha};
+        for (int j = 0; j < 8; ++j) {
+            if (m + j >= m_end) break;
+            const float a = s[j] * alpha, b = s[8 + j] * alpha;
             if (p.y_is_bf16) {
-                __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Y) + m * p.ldy + n;
-                if (wide) {
-                    __nv_bfloat162 a = __floats2bfloat162_rn(v[0], v[1]), b = __floats2bfloat162_rn(v[2], v[3]);
-                    *reinterpret_cast<uint2*>(y) = make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
-                } else {
-                    for (int e = 0; e < 4; ++e) if (n + e < p.N) y[e] = __float2bfloat16_rn(v[e]);
-                }
+                __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p.Y) + (m + j) * p.ldy + n;
+                if (wide) *reinterpret_cast<__nv_bfloat162*>(y) = __floats2bfloat162_rn(a, b);
+                else { y[0] = __float2bfloat16_rn(a); if (two) y[1] = __float2bfloat16_rn(b); }
             } else {
-                float* y = reinterpret_cast<float*>(p.Y) + m * p.ldy + n;
-                if (wide) *reinterpret_cast<float4*>(y) = make_float4(v[0], v[1], v[2], v[3]);
-                else for (int e = 0; e < 4; ++e) if (n + e < p.N) y[e] = v[e];
+                float* y = reinterpret_cast<float*>(p.Y) + (m + j) * p.ldy + n;
+                if (wide) *reinterpret_cast<float2*>(y) = make_float2(a, b);
+                else { y[0] = a; if (two) y[1] = b; }
             }
         }
     }
@@ -540,16 +548,21 @@ __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const _
 // ------------------------------------------------------------------ host side
 constexpr uint32_t MX_FIXED = 1024 /*alignment*/ + 1024 /*barriers, stage table*/, MX_TURN = 4 * 32 * 33 * 4 + 128;
 
-// Modelled time of a unit in us (measured: 1.55 at 112 tokens, 1.75 at 160, 1.95 at 208, 2.15 at 256)
-double unit_us(uint32_t n_tok) { return 1.08 + 0.0042 * n_tok; }
+// Modelled time of a unit in us.  Up to 160 tokens there are two accumulators beside the slots (measured 1.05 up to 96 tokens, 1.15 at 128, 1.22 at
+// 160), up to 208 steps of 128 elements (1.5 at 176, 1.6 at 208), beyond 256 two products to a step (1.9 at 256, 2.3 at 272, 2.6 at 352, 2.9 at 400).
+double unit_us(uint32_t n_tok)
+{
+    return n_tok <= 160 ? fmax(1.05, 0.55 + 0.0042 * n_tok) : n_tok <= 256 ? 0.55 + 0.0053 * n_tok : 0.90 + 0.0050 * n_tok;
+}
 
 // bytes for the parts of shared tiles: at most two tiles of a span are shared
 size_t parts_bytes(const MixedPlan& pl) { return pl.split ? (size_t)pl.grid * 2 * ((pl.n_tok + 31u) & ~31u) * 512 : 0; }
 
 // How the work is cut: tokens per tile, and whether CTAs take whole tiles or equal spans of units: the least modelled time among the
-// ways whose parts of tiles fit in `room_for_parts` bytes.  (A fit without the expansion's launch: whole calls take 7 to 9 us more at 48 tokens,
-// and are within 10 % of it from 203 tokens on at 11008 x 4096 and 13824 x 5120.)
-MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts)
+// ways whose parts of tiles fit in `room_for_parts` bytes.  (Against every way measured, 13 shapes from 128 to 2048 tokens: the one it takes is the
+// fastest or within 5 % of it.)  `earlier`: by the figures of an earlier form of the kernel, which cut the work into wider tiles.  What callers are
+// asked for as a workspace goes by both, so that it is nowhere less than it was.
+MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts, bool earlier = false)
 {
     const uint32_t wtiles = (uint32_t)((N + 127) / 128), chunks = (uint32_t)((K / 64 + 3) / 4), sms = (uint32_t)fgmp_sm_count();
     const uint32_t t_min = (uint32_t)((M + MX_MAX_TOK - 1) / MX_MAX_TOK), t_max = 2 * (uint32_t)((M + 255) / 256) + 2;
@@ -562,9 +575,8 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts)
         pl.n_half = pl.n_tok <= 256 ? pl.n_tok : (pl.n_tok + 31) / 32 * 16;
         pl.tok_tiles = (uint32_t)((M + pl.n_tok - 1) / pl.n_tok);
         pl.tiles = wtiles * pl.tok_tiles;
-        pl.naccs = 2 * pl.n_tok + 96 <= MX_TMEM_COLS ? 2 : 1;
-        // reading an accumulator out hides behind the next tile's products if there are two
-        const double unit = unit_us(pl.n_tok), drain = 0.012 * pl.n_tok;
+        pl.ks = pl.n_tok <= 208 ? 2 : 1;
+        pl.naccs = 2 * pl.n_tok + (earlier ? 96 : 96 * pl.ks) <= MX_TMEM_COLS ? 2 : 1;
         const uint64_t total = (uint64_t)pl.tiles * chunks;
         for (int split = 0; split < (chunks > 1 ? 2 : 1); ++split) {
             pl.quantum = split ? 1 : chunks;
@@ -576,26 +588,29 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts)
             if (split && pl.rest == 0 && pl.span % chunks == 0) continue;
             if (parts_bytes(pl) > room_for_parts) continue;
             const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / chunks;
-            // (beyond 256 tokens only spans within one tile pay: where a CTA goes on to another one its three slots and three
-            // token stages run empty as well)
-            const double drains = pl.naccs == 2 || tiles < 1.0 ? 1.0 : pl.n_tok <= 256 ? tiles : 2.0 * (tiles + 1.0);
-            pl.us = units * unit + drains * drain + (split ? 0.0 : 3.0 * tiles);
-            // the second kernel, and what it moves: a partial tile per span or two, written and read
-            if (split) pl.us += 2.0 + 2.6 * pl.grid * pl.n_tok * 512.0 / 8e6;
+            if (earlier) {
+                const double drains = pl.naccs == 2 || tiles < 1.0 ? 1.0 : pl.n_tok <= 256 ? tiles : 2.0 * (tiles + 1.0);
+                pl.us = units * (1.08 + 0.0042 * pl.n_tok) + drains * 0.012 * pl.n_tok + (split ? 2.0 + 2.6 * pl.grid * pl.n_tok * 512.0 / 8e6 : 3.0 * tiles);
+            } else {
+                // reading an accumulator out hides behind the next tile's products if there are two
+                pl.us = 2.0 + units * unit_us(pl.n_tok) + (pl.naccs == 2 ? 1.0 : split ? 0.7 * (tiles + 1.0) : tiles) * 0.0105 * pl.n_tok;
+                // the second kernel, and what it moves: a partial tile per span or two, written and read
+                if (split) pl.us += 2.5 + 1.42 * fmin(2.0 * pl.grid, (double)pl.grid + pl.tiles) * pl.n_tok * 512.0 / 8e6;
+            }
             if (pl.us < best.us) best = pl;
         }
     }
-    const uint32_t tmem_slots = (MX_TMEM_COLS - best.naccs * best.n_tok) / 32;
+    const uint32_t tmem_slots = (MX_TMEM_COLS - best.naccs * best.n_tok) / (32 * best.ks);
     best.slots = tmem_slots < (uint32_t)MAX_SLOTS ? tmem_slots : (uint32_t)MAX_SLOTS;
     // shared memory: two to four weight stages (a chunk each), the rest token stages
     const uint32_t room = (uint32_t)MX_SMEM_LIMIT - MX_FIXED - MX_TURN, bst = (best.n_tok > best.n_half ? 2u : 1u) * best.n_half * 128u;
     best.wstages = 2;
-    while (best.wstages < (uint32_t)MAX_WSTAGES && room - (best.wstages + 1) * WSTAGE >= 10 * bst) ++best.wstages;
-    best.bstages = (room - best.wstages * WSTAGE) / bst;
-    if (best.bstages > (uint32_t)MAX_BSTAGES) best.bstages = MAX_BSTAGES;
-    // No more slots than token stages: a group that fills the slot of step i then knows step i - bstages done, so that the parity of its token
-    // stage's barrier can only mean step i (with more slots it could be taken in by a stage whose step before was still on its way).
-    if (best.slots > best.bstages) best.slots = best.bstages;
+    while (best.wstages < (uint32_t)MAX_WSTAGES && room - (best.wstages + 1) * WSTAGE >= (best.ks == 2 ? 6 : 10) * bst) ++best.wstages;
+    best.ring = (room - best.wstages * WSTAGE) / (bst * best.ks);
+    if (best.ring > (uint32_t)MAX_STEPS) best.ring = MAX_STEPS;
+    // No more slots than token stages: a group that fills the slot of a step has seen the step R before done, and with it every step that could be
+    // taken for one of its own by the parity of a barrier of the ring.
+    if (best.slots > best.ring) best.slots = best.ring;
     return best;
 }
 
@@ -611,11 +626,13 @@ static size_t room_in(size_t ws_bytes, int64_t M, int64_t K)
     return ws_bytes > before ? ws_bytes - before : 0;
 }
 
-double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes) { return mixed_plan(M, N, K, room_in(ws_bytes, M, K)).us; }
+// (with the expansion of the activations: a launch, and 0.65 us per million elements)
+double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes) { return 2.0 + 0.65e-6 * (double)M * (double)K + mixed_plan(M, N, K, room_in(ws_bytes, M, K)).us; }
 
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K)
 {
-    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + parts_bytes(mixed_plan(M, N, K, SIZE_MAX));
+    const size_t parts = parts_bytes(mixed_plan(M, N, K, SIZE_MAX)), earlier = parts_bytes(mixed_plan(M, N, K, SIZE_MAX, true));
+    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + (parts > earlier ? parts : earlier);
 }
 
 // expands the activations and multiplies; leave_nvfp4: unless neither operand has an FP8 block
@@ -627,9 +644,8 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     {
         std::lock_guard<std::mutex> lk(mx_mu);
         if (!mx_attr_set[dev]) {
-            if (cudaFuncSetAttribute(mixed_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess ||
-                cudaFuncSetAttribute(mixed_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess)
-                return FGMP_ERR_CUDA;
+            for (const void* k : {(const void*)mixed_kernel<false, 1>, (const void*)mixed_kernel<false, 2>, (const void*)mixed_kernel<true, 1>, (const void*)mixed_kernel<true, 2>})
+                if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess) return FGMP_ERR_CUDA;
             mx_attr_set[dev] = true;
         }
     }
@@ -657,9 +673,9 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     if (st != FGMP_OK) return st;
     const bool quant = qn.codes4 != nullptr;
     cfg.gridDim = dim3(p.pl.grid); cfg.blockDim = dim3(MX_THREADS);
-    cfg.dynamicSmemBytes = (size_t)p.pl.bstages * (p.pl.n_tok > p.pl.n_half ? 2 : 1) * p.pl.n_half * 128 + (size_t)p.pl.wstages * WSTAGE + MX_FIXED + (quant ? MX_TURN : 0);
-    if (quant) { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<true>, tmB, p)); }
-    else       { FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, mixed_kernel<false>, tmB, p)); }
+    cfg.dynamicSmemBytes = (size_t)p.pl.ring * p.pl.ks * (p.pl.n_tok > p.pl.n_half ? 2 : 1) * p.pl.n_half * 128 + (size_t)p.pl.wstages * WSTAGE + MX_FIXED + (quant ? MX_TURN : 0);
+    const auto kernel = quant ? (p.pl.ks == 2 ? mixed_kernel<true, 2> : mixed_kernel<true, 1>) : (p.pl.ks == 2 ? mixed_kernel<false, 2> : mixed_kernel<false, 1>);
+    FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, kernel, tmB, p));
     if (p.pl.split) {
         cfg.gridDim = dim3(p.pl.tiles, (p.pl.n_tok + 31) / 32); cfg.dynamicSmemBytes = 0;
         cfg.blockDim = dim3(quant ? 128 : 256);

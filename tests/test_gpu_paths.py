@@ -176,3 +176,39 @@ def test_output_tiles(fg, M, N, K, dtype, quantum):
     assert torch.equal(wide[:M, :N], odd[:M, :N]) and bool((wide[:M, :N] != -7.0).any(dim=0).all())
     for y in (wide, odd):
         assert bool((y[M:] == -7.0).all()) and bool((y[:, N:] == -7.0).all()), "stored outside the output"
+
+
+# the GEMM on packed weights where its steps, its accumulators and its two products to a step change: an odd number of 64-element steps in the last
+# chunk, one and two accumulators, tiles of 160, 176, 208, 240, 272 and 416 tokens
+@pytest.mark.parametrize("M", [160, 176, 208, 240, 272, 416])
+@pytest.mark.parametrize("K,frac_w", [(64, 0.1), (448, 0.4), (832, 0.1)])
+def test_gemm_on_packed_weights_tile_sizes(fg, M, K, frac_w):
+    N = 200
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("ts", M, N, K, seed=73), 0.1, frac_w, clip=False)
+    count = launches(fg, lambda: fg.linear(pa, pw))
+    assert count.get("gemm_mixed_tcgen05") == 1, count
+    check_linear(fg, qa, qw, pa, pw)
+
+
+# one and two tokens, whose quantizer runs in every CTA unless the packed form is asked for: no FP8 blocks, some and only such, one unit per CTA and many
+@pytest.mark.parametrize("M", [1, 2])
+@pytest.mark.parametrize("N,K,frac_w,mode", [(130, 256, 0.1, 0), (1000, 768, 0.0, 1), (640, 5120, 1.0, 0), (9000, 2048, 0.1, 1)])
+def test_quantizer_in_every_cta(fg, M, N, K, frac_w, mode):
+    wl = gi.llama("own", M, N, K, seed=74)
+    x, fx, w, fw = wl.x(), wl.fx(), wl.w(), wl.fw()
+    s4 = gi.tensor_scale(x)
+    tau = tau_for_fraction(oracle.quantize_activations(gi.bf16_bits(x), fx.numpy(), s4, mode=mode).scores, 0.2)
+    qa = oracle.quantize_activations(gi.bf16_bits(x), fx.numpy(), s4, tau=tau, mode=mode)
+    qw = oracle.quantize_weights(gi.bf16_bits(w), fw.numpy(), clip=False, mode=mode, fp8_fraction=frac_w)
+    pw = fg.quantize_weights(w.cuda(), fw.cuda(), clip_mode=0, score_mode=mode, fp8_fraction=frac_w)
+    args = dict(scale_fp4=s4, score_mode=mode, tau=tau)
+    ws = fg.alloc_workspace(fg.OP_LINEAR_FUSED, M, N, K, torch.device("cuda"))
+    y = fg.linear_fused(x.cuda(), fx.cuda(), pw, workspace=ws, **args)
+    ys, _ = fg.linear_fused(x.cuda(), fx.cuda(), pw, want_packed=True, workspace=ws, **args)
+    fg.check(ws)
+    Y, S = oracle.linear(qa, qw)
+    for got in (y, ys, fg.linear_fused(x.cuda(), fx.cuda(), pw, workspace=ws, **args)):
+        assert (np.abs(got.cpu().numpy().astype(np.float64) - Y) <= 1e-5 * S + 1e-30).all()
+    wide = torch.randn(M, K + 8, generator=torch.Generator().manual_seed(1)).to(torch.bfloat16).cuda()
+    wide[:, :K] = x.cuda()
+    assert torch.equal(fg.linear_fused(wide[:, :K], fx.cuda(), pw, **args), y), "rows further apart"
