@@ -29,12 +29,17 @@
 // Where the activation operand (a "step record" per chunk) comes from:
 //   DEC_FUSED_LP, DEC_FUSED_HP  fused calls (by block score): the CTAs share out the quantizer's work, write the records to
 //                the workspace and stream them from there; the first weight copies are in flight meanwhile.
+//   DEC_OWN1_LP ... DEC_OWN2_HP  fused calls of one or two tokens whose packed form nobody asks for: warps of each CTA quantize what its units
+//                need, unit by unit, straight into the stages.  That is more work in all, and nothing to hand over: 2.7 us lie between the end of the
+//                kernel before and the last shared record, 0.7 more until its copy is in.  11008 x 4096: 1 token 14.4 -> 11.0 us, 2 tokens
+//                16.9 -> 12.2; 28672 x 8192: 33.5 -> 30.0 and 38.7 -> 32.9.  (With 64 threads a token for every unit in turn instead of two units at a
+//                time, two tokens take 14.5 and 48.6: beyond a dozen units that is slower than the shared quantizer.)
 //   DEC_UNPACK   fgmp_linear: made unit by unit in shared memory from the packed activations' records.
 //
-// Warp roles (480 threads): warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, warps 2-9 = a
-// unit's block scales and FP8 blocks into tensor memory (and before that the quantizer, or the step record of the unit), two
-// sets of four warps that take alternate units and own one dense tile each, warps 10-13 = epilogue (one lane quadrant each),
-// warp 14 = step-record producer.
+// Warp roles: warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, from warp 2 on two or three sets of four warps that take
+// the units in turn and put a unit's block scales and FP8 blocks into tensor memory, into a dense tile of their own (the first two sets are the
+// quantizer before that; or each makes the step record of its unit), then four warps of epilogue (one lane quadrant each), then the step-record
+// producer (DEC_OWN: four or eight warps, the quantizer).
 //
 // The roles run different code at the same time, a warp or two per scheduler, so a unit costs what its instructions cost to
 // fetch and issue: what a loop needs once per unit is not unrolled or inlined twice, and a unit passes through few hands
@@ -50,10 +55,9 @@
 
 namespace {
 
-constexpr int DEC_WARPS = 15, DEC_THREADS = 32 * DEC_WARPS;
-constexpr int W_PROD = 0, W_MMA = 1, W_SET = 2, W_EPI = 10, W_STEP = 14;
+constexpr int W_PROD = 0, W_MMA = 1, W_SET = 2;
 constexpr int SET_THREADS = 128;                // one set of FP8 warps
-constexpr int Q_THREADS = 2 * SET_THREADS;      // both sets share out the quantizer's work items
+constexpr int Q_THREADS = 2 * SET_THREADS;      // two sets share out the quantizer's work items
 constexpr int PIECES = 6;                       // base-8 digits of an FP8 activation block
 constexpr uint32_t STG_MASK = REC_BYTES, STG_LIST = STG_MASK + 256;          // the unit's mask, the list of its FP8 blocks
 constexpr uint32_t LIST_CAP = 3712;             // bytes of the list that fit a stage (about 305 blocks); more is read from global
@@ -63,14 +67,25 @@ constexpr uint32_t STG_STEP = STG_LIST + LIST_CAP;                           // 
 constexpr uint32_t AREC_GAP = AREC_AT - AREC_HOT;
 __host__ __device__ inline uint32_t arec_gap(int64_t M) { return M >= 14 ? AREC_GAP : 0u; }
 constexpr int DEC_MAX_STAGES = 6;
-// tensor memory columns: accumulators (two buffers of 112 and of 32); of each set: a dense E4M3 tile of 64, scales (32)
-constexpr uint32_t D4_COL = 0, D8_COL = 224, DENSE_COL = 288, SF_COL = 416;
+// Two sets; three where the quantizer is the CTA's own (the accumulators of two tokens leave the tensor memory for it): 11.2 us instead of 11.3 at one
+// token of 11008 x 4096, 30.6 instead of 31.0 of 28672 x 8192.  For the shared quantizer it is no gain: eight tokens of 28672 x 8192 39.4 instead of
+// 36.1.
+// Tensor memory columns: accumulators (two buffers of each kind); of each set: a dense E4M3 tile of 64, scales (32)
+template <int SETS> struct Dec {
+    static constexpr int W_EPI = W_SET + 4 * SETS, W_STEP = W_EPI + 4;
+    static constexpr uint32_t D4 = SETS == 3 ? 64 : 112, D8 = SETS == 3 ? 16 : 32;
+    static constexpr uint32_t D4_COL = 0, D8_COL = 2 * D4, DENSE_COL = D8_COL + 2 * D8, SF_COL = DENSE_COL + 64 * SETS;
+    static_assert(SF_COL + 32 * SETS <= 512, "tensor memory columns");
+};
 constexpr uint32_t DEC_TMEM_COLS = 512;
 constexpr size_t SMEM_LIMIT = 232448;
 static_assert(STG_STEP % 1024 == 0, "stage layout");
-static_assert(SF_COL + 32 * 2 <= DEC_TMEM_COLS, "tensor memory columns");
 
-enum { DEC_FUSED_LP = 0, DEC_FUSED_HP = 1, DEC_UNPACK = 2 };      // the first two are the fgmp_score_mode of the quantizer
+enum { DEC_FUSED_LP = 0, DEC_FUSED_HP = 1, DEC_UNPACK = 2, DEC_OWN1_LP = 4, DEC_OWN1_HP = 5, DEC_OWN2_LP = 6, DEC_OWN2_HP = 7 };
+// (the lowest bit of the fused ones is the fgmp_score_mode of the quantizer, OWN1 and OWN2 are for one token and for two)
+constexpr int OWN_TURNS = 2;                    // units whose step records are made at a time: 64 threads take about 1 us for a token's, the weights half of that
+constexpr int own_tokens(int src) { return src >= DEC_OWN2_LP ? 2 : src >= DEC_OWN1_LP ? 1 : 0; }
+constexpr int dec_threads(int src, int sets) { return 32 * (W_SET + 4 * sets + 4 + (own_tokens(src) ? 2 * OWN_TURNS * own_tokens(src) : 1)); }
 
 // Step record of a chunk for a batch of M tokens: n4 rows x 128 bytes of E2M1 codes | 2 KiB of block scales in tensor-
 // memory order | n8 rows x 128 bytes of E5M2 values of elements 0..127 | the same of elements 128..255.  Both code tiles
@@ -349,17 +364,19 @@ __device__ __forceinline__ void quantize_item(const DecParams& p, uint32_t c, ui
     }
 }
 
-template <int SRC>
-__global__ void __launch_bounds__(DEC_THREADS, 1)
+template <int SRC, int SETS>
+__global__ void __launch_bounds__(dec_threads(SRC, SETS), 1)
 decode_kernel(const __grid_constant__ DecParams p)
 {
     extern __shared__ uint8_t smem_raw[];
     // 1 KiB aligned; an offset from the array keeps the pointer known to be shared memory (plain ld.shared / st.shared)
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    constexpr bool FUSED = SRC != DEC_UNPACK;
+    constexpr bool FUSED = SRC != DEC_UNPACK, OWN = own_tokens(SRC) != 0, SHARED = FUSED && !OWN;      // SHARED: the CTAs share out the quantizer's work
     constexpr int X = DEC_MAX_STAGES;
+    using D = Dec<SETS>;
+    constexpr int W_EPI = D::W_EPI, W_STEP = D::W_STEP;
     const uint32_t S = p.stages;
-    const uint32_t M = (uint32_t)p.M, n4 = step_n4(M), n8 = step_n8(M), a_bytes = step_bytes(M);
+    const uint32_t M = OWN ? (uint32_t)own_tokens(SRC) : (uint32_t)p.M, n4 = step_n4(M), n8 = step_n8(M), a_bytes = step_bytes(M);
     uint8_t* arecs = smem + S * p.stage_bytes;           // DEC_UNPACK: S packed activation records
     uint64_t* bars = reinterpret_cast<uint64_t*>(arecs + S * p.arec_bytes);
     StageMeta* smeta = reinterpret_cast<StageMeta*>(bars + 4 * X + 4);
@@ -384,7 +401,7 @@ decode_kernel(const __grid_constant__ DecParams p)
     // ------------------------------------------------------------ set-up
     if (warp == W_PROD && lane == 0) {
         for (uint32_t s = 0; s < S; ++s) {
-            mbar_init(wf0 + 8 * s, 1); mbar_init(sf0 + 8 * s, FUSED ? 1 : 4); mbar_init(rd0 + 8 * s, 4); mbar_init(dn0 + 8 * s, 1);
+            mbar_init(wf0 + 8 * s, 1); mbar_init(sf0 + 8 * s, OWN ? 2 * M : SHARED ? 1 : 4); mbar_init(rd0 + 8 * s, 4); mbar_init(dn0 + 8 * s, 1);
         }
         for (int b = 0; b < 2; ++b) { mbar_init(accf0 + 8 * b, 1); mbar_init(acce0 + 8 * b, 4); }
         *abort_flag = 0;
@@ -392,7 +409,7 @@ decode_kernel(const __grid_constant__ DecParams p)
     }
     // The first of the quantizer's work items is asked for right away.  (This kernel may have started before the one
     // before it in the stream has finished; that one lets it start only after its own last claim.)
-    if (FUSED && threadIdx.x == 32 * W_SET) s_misc[1] = atomicInc(p.cw + CW_CLAIM, n_items + G - 1u);
+    if (SHARED && threadIdx.x == 32 * W_SET) s_misc[1] = atomicInc(p.cw + CW_CLAIM, n_items + G - 1u);
     if (warp == W_MMA) tmem_alloc(smem_u32(tmem_slot), DEC_TMEM_COLS);
     if (warp >= W_EPI && warp < W_STEP) digits[threadIdx.x - 32 * W_EPI] = e4m3_digits(min(threadIdx.x - 32u * W_EPI, 126u));
     tc_fence_before();
@@ -461,10 +478,10 @@ decode_kernel(const __grid_constant__ DecParams p)
     } else {
         // Everything before this touches neither the preceding kernel's output nor (but for the claim) the workspace.
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        if (!FUSED) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (!SHARED) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
 
-    if (FUSED && warp >= W_SET && warp < W_EPI) {
+    if (SHARED && warp >= W_SET && warp < W_SET + Q_THREADS / 32) {
         // ------------------------------------------------------------ quantizer
         // Work items are handed out through a counter, so that every item is taken by a CTA that is running: no CTA
         // ever waits for one that has not started.  The counter wraps to zero with the call's last claim.
@@ -479,7 +496,7 @@ decode_kernel(const __grid_constant__ DecParams p)
                 h->fp8_log2_ratio = p.q.ratio; h->n_fp8 = (p.q.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
                 h->error = 0; h->scale_fp8 = p.q.s8; h->fp8_scale_free = 0;
             }
-            quantize_item<SRC>(p, item / quads, item % quads, digits);
+            quantize_item<(SRC & 1)>(p, item / quads, item % quads, digits);
             // The item's stores become visible with the count of finished items: the barrier orders them before the one
             // thread's release.
             quant_bar();
@@ -492,9 +509,34 @@ decode_kernel(const __grid_constant__ DecParams p)
         }
     }
 
-    if (warp == W_STEP) {
+    if (OWN && warp >= W_STEP) {
+        // ------------------------------------------------------------ this CTA's own quantizer: 64 threads, four lanes per block, make what a step
+        // record holds of one token; two units at a time.
+        const uint32_t tq = threadIdx.x - 32u * W_STEP, part = tq >> 6, li = tq & 3u, j = (tq >> 2) & 15u, m = part % M;
+        uint32_t i = part / M, c = (u_begin + i) % C, stage = i, phase = 1;        // (fewer at a time than stages)
+        const uint8_t* row = p.X + (size_t)m * p.ldx * 2 + 32u * j + 8u * li;
+        const float* fish = p.fisher + 16u * j + 4u * li;
+        uint2 x = make_uint2(0u, 0u);
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i < n_units) { x = __ldg(reinterpret_cast<const uint2*>(row + 512u * c)); f = __ldg(reinterpret_cast<const float4*>(fish + 256u * c)); }
+        for (; i < n_units; i += OWN_TURNS) {
+            const BlockQuarter r = quantize_block_quarter<(SRC & 1)>(x, f, p.q);
+            c += OWN_TURNS;
+            while (c >= C) c -= C;
+            if (i + OWN_TURNS < n_units) { x = __ldg(reinterpret_cast<const uint2*>(row + 512u * c)); f = __ldg(reinterpret_cast<const float4*>(fish + 256u * c)); }
+            const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&r.h.x)), vb = __half22float2(*reinterpret_cast<const __half2*>(&r.h.y));
+            const float v[4] = {va.x, va.y, vb.x, vb.y};
+            if (!mbar_wait_warp(dn0 + 8 * stage, phase, abort_flag, p.status, 13)) break;
+            emit_step(smem + stage * p.stage_bytes + STG_STEP, M, n4, n8, m, j, li, r.is8, r.c4, r.sc, r.c8, v, digits);
+            fence_proxy_async();                       // the tensor core reads what ordinary stores wrote
+            __syncwarp();
+            if (lane == 0) mbar_arrive(sf0 + 8 * stage);
+            stage += OWN_TURNS;
+            if (stage >= S) { stage -= S; phase ^= 1u; }
+        }
+    } else if (warp == W_STEP) {
         // ------------------------------------------------------------ step-record producer
-        if (FUSED && lane == 0) {
+        if (SHARED && lane == 0) {
             // every chunk's record is in place once the last work item of the quantizer has been handed in
             bool ok = wait_global_equals(p.cw + CW_QCOUNT, n_items, abort_flag, p.status, 8);
             asm volatile("fence.proxy.async;" ::: "memory");   // records were written with ordinary stores, the bulk copy reads them
@@ -516,7 +558,7 @@ decode_kernel(const __grid_constant__ DecParams p)
         const uint32_t idesc4 = IDESC_NVF4 | ((n4 >> 3) << 17), idesc8 = IDESC_E4M3_E5M2 | ((n8 >> 3) << 17);
         const uint32_t step_lo = (p.stage_bytes >> 4), b8_lo = (n4 * 128u + 2048u) >> 4, b8_half = n8 * 8u;
         const uint32_t w_first = (smem_u32(smem) >> 4) | SW128_LO;
-        uint32_t stage = 0, phase = 0, w4 = w_first, left = C - u_begin % C, accum = 0, acc = 0, acc_phase = 1;
+        uint32_t stage = 0, phase = 0, w4 = w_first, left = C - u_begin % C, accum = 0, acc = 0, acc_phase = 1, set = 0;
         for (uint32_t i = 0; i < n_units; ++i) {
             if (accum == 0) {                          // a tile begins
                 if (!mbar_wait_uniform(acce0 + 8 * acc, acc_phase, abort_flag, p.status, 2)) break;
@@ -525,9 +567,10 @@ decode_kernel(const __grid_constant__ DecParams p)
             if (i == 0 && lane == 0) FGMP_STAMP_ANY(5);
             if (i == n_units - 1 && lane == 0) FGMP_STAMP_ANY(6);
             tc_fence_after();
-            const uint32_t set = i & 1u, a4 = w4 + (STG_STEP >> 4), a8 = a4 + b8_lo;
-            const uint32_t d4 = tmem_base + D4_COL + acc * 112, d8 = tmem_base + D8_COL + acc * 32;
-            const uint32_t sf_t = tmem_base + SF_COL + set * 32, w8 = tmem_base + DENSE_COL + set * 64;
+            const uint32_t a4 = w4 + (STG_STEP >> 4), a8 = a4 + b8_lo;
+            const uint32_t d4 = tmem_base + D::D4_COL + acc * D::D4, d8 = tmem_base + D::D8_COL + acc * D::D8;
+            const uint32_t sf_t = tmem_base + D::SF_COL + set * 32, w8 = tmem_base + D::DENSE_COL + set * 64;
+            set = set == SETS - 1 ? 0u : set + 1u;
             if (elect_one()) {
 #pragma unroll
                 for (int j = 0; j < 4; ++j)
@@ -551,18 +594,18 @@ decode_kernel(const __grid_constant__ DecParams p)
             }
         }
     } else if (warp >= W_SET && warp < W_EPI) {
-        // ------------------------------------------------------------ sets: units set, set + 2, ...: scales and FP8 blocks
+        // ------------------------------------------------------------ sets: units set, set + SETS, ...: scales and FP8 blocks
         // Thread = row of the tile = lane of tensor memory (quadrant warp % 4).
         const uint32_t set = (uint32_t)(warp - W_SET) >> 2, row = 32u * (warp & 3) + lane;
         const uint32_t quadrant = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t dense = quadrant + DENSE_COL + set * 64, sf_t = quadrant + SF_COL + set * 32;
+        const uint32_t dense = quadrant + D::DENSE_COL + set * 64, sf_t = quadrant + D::SF_COL + set * 32;
         uint32_t unscale = 0;                          // 2^-ratio, twice in fp16: back to the E4M3 value of an FP8 element
         if (!FUSED) unscale = (uint32_t)(15 - reinterpret_cast<const fgmp_packed_header*>(p.ablob)->fp8_log2_ratio) * 0x04000400u;
         uint32_t stage = set, phase = 0, done = set, dphase = 0;      // done: stage of the set's last unit
-        for (uint32_t i = set; i < n_units; i += 2) {
+        for (uint32_t i = set; i < n_units; i += SETS) {
             const uint8_t* sb = smem + stage * p.stage_bytes;
-            // (Barriers are waited for by parity, so the stage's unit before this one, the other set's where the number of stages is odd, must be
-            // known to be in.  This set has seen unit i - 4 done, which says so from four stages on.)
+            // (Barriers are waited for by parity, so the stage's unit before this one, another set's where the number of stages is no multiple of that of the
+            // sets, must be known to be in.  This set has seen unit i - 2 SETS done, which says so from twice as many stages as sets on.)
             if (!mbar_wait_warp(wf0 + 8 * stage, phase, abort_flag, p.status, 5)) break;
             if (!FUSED) {
                 // the unit's step record from the packed activation record
@@ -594,10 +637,10 @@ decode_kernel(const __grid_constant__ DecParams p)
                 if (lane == 0) mbar_arrive(sf0 + 8 * stage);
             }
             // the tensor core has read what the set's last unit had in tensor memory
-            if (i >= 2) {
+            if (i >= SETS) {
                 if (!mbar_wait_warp(dn0 + 8 * done, dphase, abort_flag, p.status, 7)) break;
                 tc_fence_after();
-                done += 2;
+                done += SETS;
                 if (done >= S) { done -= S; dphase ^= 1; }
             }
             // Block scales: lane i holds, for MMA step j, the four scale bytes of operand rows i, 32+i, 64+i, 96+i in columns
@@ -654,7 +697,7 @@ decode_kernel(const __grid_constant__ DecParams p)
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(rd0 + 8 * stage);
-            stage += 2;
+            stage += SETS;
             if (stage >= S) { stage -= S; phase ^= 1; }
         }
     }
@@ -688,27 +731,43 @@ decode_kernel(const __grid_constant__ DecParams p)
             uint32_t seen = 0;
             if (!whole && lane == 0) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
             // columns m (NVFP4 blocks), (p + 1) M + m (digits); FP8 weights: m (high), M + m (low)
-            const uint32_t d4 = tmem_base + ((uint32_t)(q * 32) << 16) + D4_COL + accb * 112;
-            const uint32_t d8 = tmem_base + ((uint32_t)(q * 32) << 16) + D8_COL + accb * 32;
+            const uint32_t d4 = tmem_base + ((uint32_t)(q * 32) << 16) + D::D4_COL + accb * D::D4;
+            const uint32_t d8 = tmem_base + ((uint32_t)(q * 32) << 16) + D::D8_COL + accb * D::D8;
             float v[16], t[16];
-            uint32_t r0[16], r1[16], r2[16];
-            // (three loads in flight at a time)
-            tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1); tmem_ld16_async(d8 + M, r2);
-            tmem_wait_ld(r0, r1, r2);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                v[j] = __uint_as_float(r0[j]); t[j] = 0.f;
-                if (has_fp8) v[j] += (__uint_as_float(r1[j]) + __uint_as_float(r2[j])) * rw;     // (else those columns hold nothing)
-            }
-#pragma unroll 1
-            for (uint32_t pc = 1; pc < PIECES; pc += 3) {
-                tmem_ld16_async(d4 + pc * M, r0); tmem_ld16_async(d4 + (pc + 1) * M, r1); tmem_ld16_async(d4 + (pc + 2) * M, r2);
+            uint32_t r0[16], r1[16], r2[16] = {};
+            if (OWN) {
+                // at most 14 and 4 columns: one load of each, the sums in the order of the general form
+                tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1);
                 tmem_wait_ld(r0, r1, r2);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) t[j] += (__uint_as_float(r0[j]) + __uint_as_float(r1[j])) + __uint_as_float(r2[j]);
-            }
+                for (int j = 0; j < 16; ++j) v[j] = 0.f;
 #pragma unroll
-            for (int j = 0; j < 16; ++j) v[j] += t[j] * ra;
+                for (int j = 0; j < own_tokens(SRC); ++j) {
+                    constexpr int T = own_tokens(SRC);
+                    const auto col = [&](int i) { return __uint_as_float(r0[T * i + j]); };
+                    const float high = __uint_as_float(r1[j]), low = __uint_as_float(r1[T + j]);
+                    const float x = has_fp8 ? col(0) + (high + low) * rw : col(0);
+                    v[j] = x + (((col(1) + col(2)) + col(3)) + ((col(4) + col(5)) + col(6))) * ra;
+                }
+            } else {
+                // (three loads in flight at a time)
+                tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1); tmem_ld16_async(d8 + M, r2);
+                tmem_wait_ld(r0, r1, r2);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) {
+                    v[j] = __uint_as_float(r0[j]); t[j] = 0.f;
+                    if (has_fp8) v[j] += (__uint_as_float(r1[j]) + __uint_as_float(r2[j])) * rw;     // (else those columns hold nothing)
+                }
+#pragma unroll 1
+                for (uint32_t pc = 1; pc < PIECES; pc += 3) {
+                    tmem_ld16_async(d4 + pc * M, r0); tmem_ld16_async(d4 + (pc + 1) * M, r1); tmem_ld16_async(d4 + (pc + 2) * M, r2);
+                    tmem_wait_ld(r0, r1, r2);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) t[j] += (__uint_as_float(r0[j]) + __uint_as_float(r1[j])) + __uint_as_float(r2[j]);
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] += t[j] * ra;
+            }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acce0 + 8 * accb);
@@ -783,7 +842,7 @@ decode_kernel(const __grid_constant__ DecParams p)
         const unsigned long long t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
         __syncthreads();
-    } else if (FUSED && threadIdx.x == 0) {
+    } else if (SHARED && threadIdx.x == 0) {
         // the CTA that finishes last takes the count of finished items back, so that the control area is as the next call needs it
         if (atomicInc(p.cw + CW_DONE, G - 1u) == G - 1u)
             asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.cw + CW_QCOUNT), "r"(0u) : "memory");
@@ -817,9 +876,12 @@ fgmp_status set_attrs_once()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
     std::lock_guard<std::mutex> lk(g_dec_mu);
     if (!g_attr_set[dev]) {
-        if (cudaFuncSetAttribute(decode_kernel<DEC_FUSED_LP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess ||
-            cudaFuncSetAttribute(decode_kernel<DEC_FUSED_HP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess ||
-            cudaFuncSetAttribute(decode_kernel<DEC_UNPACK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) != cudaSuccess)
+        bool ok = true;
+        for (const void* k : {(const void*)decode_kernel<DEC_FUSED_LP, 2>, (const void*)decode_kernel<DEC_FUSED_HP, 2>, (const void*)decode_kernel<DEC_OWN1_LP, 3>,
+                              (const void*)decode_kernel<DEC_OWN1_HP, 3>, (const void*)decode_kernel<DEC_OWN2_LP, 3>, (const void*)decode_kernel<DEC_OWN2_HP, 3>,
+                              (const void*)decode_kernel<DEC_UNPACK, 2>})
+            ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) == cudaSuccess;
+        if (!ok)
             return FGMP_ERR_CUDA;
         g_attr_set[dev] = true;
     }
@@ -847,24 +909,25 @@ DecParams base_params(const void* packed_weights, void* Y, int y_is_bf16, int64_
     return p;
 }
 
-template <int SRC>
+template <int SRC, int SETS>
 fgmp_status launch_decode(DecParams p, const DecPlan& d, bool programmatic, cudaStream_t s)
 {
     p.arec_bytes = SRC == DEC_UNPACK ? (p.M <= 8 ? AREC_BYTES - 4096u : AREC_BYTES) - arec_gap(p.M) : 0u;
     p.stage_bytes = (STG_STEP + step_bytes(p.M) + 1023u) & ~1023u;
     constexpr size_t fixed = 1024 /*alignment*/ + 1024 /*barriers, digit table*/;
     const uint32_t fit = (uint32_t)((SMEM_LIMIT - fixed) / (p.stage_bytes + p.arec_bytes));      // 4 (16 tokens) to 7
-    // step records of 16 tokens (see step_bytes); the kernel's sets count on four stages at least
+    // step records of 16 tokens (see step_bytes), of eight; the kernel's sets count on four stages at least, three sets on six
     static_assert(4 * (STG_STEP + 112 * 128 + 2048 + 32 * 256 + AREC_BYTES - AREC_GAP) + fixed <= SMEM_LIMIT && STG_STEP % 1024 == 0, "four stages");
+    static_assert(6 * (STG_STEP + 64 * 128 + 2048 + 16 * 256) + fixed <= SMEM_LIMIT && DEC_MAX_STAGES >= 6, "six stages");
     p.stages = fit < (uint32_t)DEC_MAX_STAGES ? fit : (uint32_t)DEC_MAX_STAGES;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)d.grid); cfg.blockDim = dim3(DEC_THREADS); cfg.stream = s;
+    cfg.gridDim = dim3((unsigned)d.grid); cfg.blockDim = dim3(dec_threads(SRC, SETS)); cfg.stream = s;
     cfg.dynamicSmemBytes = fixed + (size_t)p.stages * (p.stage_bytes + p.arec_bytes);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr; cfg.numAttrs = programmatic ? 1 : 0;
-    FGMP_LAUNCH(FGMP_K_DECODE, s, cudaLaunchKernelEx(&cfg, decode_kernel<SRC>, p));
+    FGMP_LAUNCH(FGMP_K_DECODE, s, cudaLaunchKernelEx(&cfg, decode_kernel<SRC, SETS>, p));
     return fgmp_launch_status();
 }
 
@@ -901,7 +964,7 @@ fgmp_status fgmp_linear_decode(const void* packed_acts, const void* packed_weigh
     fgmp_status st = set_attrs_once();
     if (st != FGMP_OK) return st;
     if (clear_first && cudaMemsetAsync(workspace, 0, 1024 + (size_t)d.tiles * 32, s) != cudaSuccess) return FGMP_ERR_CUDA;
-    return launch_decode<DEC_UNPACK>(p, d, !clear_first, s);
+    return launch_decode<DEC_UNPACK, 2>(p, d, !clear_first, s);
 }
 
 extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const float* fisher_chan,
@@ -946,8 +1009,10 @@ extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const 
         p.q_arec = blob + p.LA.off_arec;
     }
     p.steps = (uint8_t*)workspace + fgmp_align1k(fgmp_ws_decode(M, N, K));
-    return sm == FGMP_SCORE_LP_ERROR ? launch_decode<DEC_FUSED_LP>(p, d, true, (cudaStream_t)cuda_stream)
-                                     : launch_decode<DEC_FUSED_HP>(p, d, true, (cudaStream_t)cuda_stream);
+    const auto launch = [&](auto lp, auto hp) { return (sm == FGMP_SCORE_LP_ERROR ? lp : hp)(p, d, true, (cudaStream_t)cuda_stream); };
+    if (M == 1 && !packed_acts_out) return launch(launch_decode<DEC_OWN1_LP, 3>, launch_decode<DEC_OWN1_HP, 3>);
+    if (M == 2 && !packed_acts_out) return launch(launch_decode<DEC_OWN2_LP, 3>, launch_decode<DEC_OWN2_HP, 3>);
+    return launch(launch_decode<DEC_FUSED_LP, 2>, launch_decode<DEC_FUSED_HP, 2>);
 }
 
 #ifdef FGMP_TIMELINE
