@@ -144,30 +144,6 @@ struct UnitScratch {
         return (m >> j) & 1u ? base[row] + __popc(m & ((1u << j) - 1u)) : 0xffffu;
     }
 };
-
-// Visits every block of one unit of a packed weight tensor, 128 threads per unit, consecutive
-// threads on consecutive blocks of one row: f(row, kb, row in tile, column in chunk, rec, hi) with
-// rec = the unit's record and hi = address of E4M3 codes 8..15 of an FP8 block (codes 0..7 are in its
-// slot), or nullptr if the block is NVFP4.
-template <class F>
-__device__ __forceinline__ void fgmp_for_each_block(const uint8_t* blob, const PackedLayout& L, int64_t unit,
-                                                    UnitScratch& sc, F f)
-{
-    const int64_t tile = unit / L.chunks, c = unit % L.chunks;
-    const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x]);
-    const uint8_t* rec = blob + L.off_rec + (size_t)unit * REC_BYTES;
-    const uint8_t* halves = blob + L.off_ovf + (size_t)reinterpret_cast<const uint32_t*>(blob + L.off_uptr)[unit] * 16 + fgmp_list_halves_offset(cnt);
-    const int j = threadIdx.x & 15;
-#pragma unroll 1
-    for (int i = 0; i < 16; ++i) {
-        const int row = (threadIdx.x >> 4) + 8 * i;
-        const int64_t r = tile * 128 + row, kb = c * 16 + j;
-        if (r >= L.rows || kb >= L.KB) continue;
-        const uint32_t pos = sc.pos(row, j);
-        f(r, kb, row, j, rec, pos != 0xffffu ? halves + (size_t)pos * 8 : (const uint8_t*)nullptr);
-    }
-    __syncthreads();
-}
 #endif
 
 // ---------------------------------------------------------------- conversions

@@ -174,16 +174,38 @@ __global__ void __launch_bounds__(128) unpack_w_kernel(const uint8_t* blob, int6
         const uint16_t* m16 = reinterpret_cast<const uint16_t*>(blob + L.off_mask) + (size_t)blockIdx.x * 128 + threadIdx.x;
         if (r < rows && (c & 1) == 0) mask[r * L.MW + (c >> 1)] = m16[0] | (c + 1 < L.chunks ? (uint32_t)m16[128] << 16 : 0u);
     }
-    fgmp_for_each_block(blob, L, blockIdx.x, sc, [&](int64_t r, int64_t kb, int row, int j, const uint8_t* rec, const uint8_t* hi) {
-        const uint2 slot = *reinterpret_cast<const uint2*>(rec + REC_W4 + fgmp_rec_w4_offset(row, j));
-        if (scales) scales[r * L.KB + kb] = rec[REC_SF + fgmp_rec_sf_offset(row, j)];
-        if (codes4) *reinterpret_cast<uint2*>(codes4 + (r * K) / 2 + kb * 8) = hi ? make_uint2(0u, 0u) : slot;
-        if (codes8) {
-            uint4 c = make_uint4(0, 0, 0, 0);
-            if (hi) { const uint2 h = *reinterpret_cast<const uint2*>(hi); c = make_uint4(slot.x, slot.y, h.x, h.y); }
-            *reinterpret_cast<uint4*>(codes8 + r * K + kb * 16) = c;
+    // eight blocks of the thread in flight, consecutive threads on consecutive blocks of a row (4096 x 4096: 10 us, 16 one at
+    // a time)
+    const int64_t tile = blockIdx.x / L.chunks, c = blockIdx.x % L.chunks;
+    const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[(size_t)blockIdx.x * 128 + threadIdx.x]);
+    const uint8_t* rec = blob + L.off_rec + (size_t)blockIdx.x * REC_BYTES;
+    const uint8_t* halves = blob + L.off_ovf + (size_t)reinterpret_cast<const uint32_t*>(blob + L.off_uptr)[blockIdx.x] * 16 + fgmp_list_halves_offset(cnt);
+    const int j = threadIdx.x & 15;
+    const int64_t kb = c * 16 + j;
+    if (kb >= L.KB) return;
+#pragma unroll 1
+    for (int i0 = 0; i0 < 16; i0 += 8) {
+        uint2 slot[8], hi[8];
+        uint32_t scale[8], is8 = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int row = (threadIdx.x >> 4) + 8 * (i0 + i);
+            const uint32_t pos = sc.pos(row, j);
+            slot[i] = __ldg(reinterpret_cast<const uint2*>(rec + REC_W4 + fgmp_rec_w4_offset(row, j)));
+            scale[i] = __ldg(rec + REC_SF + fgmp_rec_sf_offset(row, j));
+            hi[i] = make_uint2(0u, 0u);
+            if (pos != 0xffffu) { hi[i] = __ldg(reinterpret_cast<const uint2*>(halves + (size_t)pos * 8)); is8 |= 1u << i; }
         }
-    });
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int64_t r = tile * 128 + (threadIdx.x >> 4) + 8 * (i0 + i);
+            if (r >= rows) continue;
+            const bool b8 = (is8 >> i) & 1u;
+            if (scales) scales[r * L.KB + kb] = (uint8_t)scale[i];
+            if (codes4) *reinterpret_cast<uint2*>(codes4 + (r * K) / 2 + kb * 8) = b8 ? make_uint2(0u, 0u) : slot[i];
+            if (codes8) *reinterpret_cast<uint4*>(codes8 + r * K + kb * 16) = b8 ? make_uint4(slot[i].x, slot[i].y, hi[i].x, hi[i].y) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    }
 }
 
 // mean of squares per column of a bf16 matrix; thread per column, rows in order (one fp32 multiply

@@ -9,6 +9,26 @@ namespace {
 
 constexpr int SEL_BINS = 2048;           // bins of a digit of the radix select
 
+// The calls here are chains of small kernels.  Each is launched as a programmatic dependent of the one before it: its blocks come up while
+// that one runs and wait for its end (every block does, so that a kernel's end implies those of all before it).  The last kernel of a packing lets
+// nothing start early, since the GEMMs read packed weights before they wait.  (4096 x 4096 weights and a calibration batch of 512 tokens,
+// eighteen launches: 20 us of 311.)
+__device__ __forceinline__ void chain_begin(bool more = true)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (more) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+void chain_launch(void (*kernel)(P...), int64_t grid, int threads, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid); cfg.blockDim = dim3((unsigned)threads); cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Device-resident state of one packing call (lives at the start of the workspace).
 struct SelectState {
     uint32_t hist[SEL_BINS];
@@ -30,6 +50,7 @@ static_assert(sizeof(SelectState) <= STATE_BYTES, "state section of the workspac
 
 __global__ void state_init_kernel(SelectState* st, float s4_given, unsigned long long k, float tau)
 {
+    chain_begin();
     for (int t = threadIdx.x; t < SEL_BINS; t += blockDim.x) st->hist[t] = 0;
     if (threadIdx.x == 0) {
         st->arrived = 0;
@@ -54,6 +75,7 @@ __device__ __forceinline__ bool last_block(uint32_t* arrived)
 // max |w| and the tensor scale.  A block takes four rows of W at a time: four 16-byte loads per thread in flight.
 __global__ void __launch_bounds__(256) w_amax_kernel(const uint4* W, int64_t ldw8, int64_t N, uint32_t K8, SelectState* st)
 {
+    chain_begin();
     uint32_t m = 0;
     auto take = [&](const uint4& x) {
         const uint32_t w[4] = {x.x, x.y, x.z, x.w};
@@ -134,6 +156,43 @@ __device__ __forceinline__ float clip_error(const float (&v)[16], const float (&
     return j;
 }
 
+__device__ __forceinline__ uint32_t dynamic_scale_of(const uint4* W, int64_t ldw8, int64_t n, int64_t kb, float k6)
+{
+    float v[16];
+    const uint4* wp = W + n * ldw8 + kb * 2;
+    unpack_bf16x16(__ldg(wp), __ldg(wp + 1), v);
+    return block_dynamic_scale(v, k6);
+}
+
+// 256 threads sort what they are given (0..127): index() returns which thread's value is the calling one's in that order
+struct ClipOrder {
+    uint32_t bins[128];
+    uint8_t order[256];
+    __device__ __forceinline__ int index(uint32_t key)
+    {
+        const int t = threadIdx.x;
+        __syncthreads();
+        if (t < 128) bins[t] = 0;
+        __syncthreads();
+        const uint32_t rank = atomicAdd(&bins[key], 1u);
+        __syncthreads();
+        if (t < 32) {
+            uint32_t n[4], sum = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { n[i] = bins[4 * t + i]; sum += n[i]; }
+            uint32_t at = sum;
+            for (int o = 1; o < 32; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, at, o); if (t >= o) at += y; }
+            at -= sum;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) { bins[4 * t + i] = at; at += n[i]; }
+        }
+        __syncthreads();
+        order[bins[key] + rank] = (uint8_t)t;
+        __syncthreads();
+        return order[t];
+    }
+};
+
 // Per block: microscale (dynamic max or Eq. 11 search) and the score under it.
 //
 // The search asks for the scale with the least error among all 126, ties to the dynamic-max scale and then to the smaller
@@ -141,8 +200,9 @@ __device__ __forceinline__ float clip_error(const float (&v)[16], const float (&
 // only grows (every rounding step is monotone), and a sum of non-negative terms is never below one of them, so once such a
 // term alone exceeds the least error found no smaller scale can win.  (Where a sensitivity is negative or NaN the terms are not what
 // this rests on, and all scales are looked at.)  Going up there are few codes left, because the tensor
-// scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left (25 for the longest of a warp): 4096 x 4096 takes 152 us,
-// 172 without packed fp32 instructions, 680 with all 126.
+// scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left, 26 for the longest of a warp, and 20 if the warps of a thread
+// block share its 256 blocks out in the order of their dynamic-max codes, that is of how many there are above: 4096 x 4096 takes 145 us,
+// 152 in the order of the tensor, 172 without packed fp32 instructions, 680 with all 126.
 template <int MODE, bool CLIP>
 __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ldw8, const float* F, int64_t ldf,
                                                       int64_t N, int64_t KB, int ratio, float s8_given, const SelectState* st,
@@ -151,6 +211,8 @@ __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ld
     // scale and its inverse, by code; 127, NaN, is what a block gets whose largest magnitude over a tensor scale of infinity or NaN has
     // no code (weights that are not finite): no scale is better than it
     __shared__ float2 s_d[128];
+    __shared__ ClipOrder clip_order;
+    chain_begin();
     const float s4 = st->s4;
     if (CLIP) {
         if (threadIdx.x < 128) {
@@ -163,7 +225,10 @@ __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ld
     const float s8 = s8_given > 0.f ? s8_given : __fmul_rn(s4, __int_as_float((127 + ratio) << 23));
     const float inv8 = inverse_scale(s8);
     const int64_t B = N * KB;
-    for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < B; b += (int64_t)gridDim.x * blockDim.x) {
+    for (int64_t base = (int64_t)blockIdx.x * 256; base < B; base += (int64_t)gridDim.x * 256) {
+        int64_t b = base + threadIdx.x;
+        if (CLIP) b = base + clip_order.index(b < B ? dynamic_scale_of(W, ldw8, b / KB, b % KB, k6) : 127u);
+        if (b >= B) continue;
         float v[16], f[16];
         load_block(W, ldw8, F, ldf, b / KB, b % KB, v, f);
         uint32_t sc = block_dynamic_scale(v, k6);
@@ -212,7 +277,8 @@ __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ld
 __global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_t B, int pass, SelectState* st)
 {
     __shared__ uint32_t h[SEL_BINS];
-    __shared__ unsigned long long s_sum[512];
+    __shared__ unsigned long long s_warp[16];
+    chain_begin();
     const int bits = pass == 2 ? 10 : 11, shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
     for (int i = threadIdx.x; i < SEL_BINS; i += 512) h[i] = 0;
     __syncthreads();
@@ -235,17 +301,15 @@ __global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_
     unsigned long long sum = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) { own[i] = *reinterpret_cast<volatile uint32_t*>(&st->hist[4 * threadIdx.x + i]); sum += own[i]; }
-    s_sum[threadIdx.x] = sum;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned long long from = sum;                       // sums over the threads t, t + 1, ... : of the warp, then of all
+    for (int o = 1; o < 32; o <<= 1) { const unsigned long long y = __shfl_down_sync(0xffffffffu, from, o); if (lane + o < 32) from += y; }
+    if (lane == 0) s_warp[w] = from;
+    const unsigned long long krem = st->krem;            // (before anybody changes it below)
     __syncthreads();
-    for (int o = 1; o < 512; o <<= 1) {                  // sums over the threads t, t + 1, ...
-        const unsigned long long y = threadIdx.x + o < 512 ? s_sum[threadIdx.x + o] : 0ull;
-        __syncthreads();
-        s_sum[threadIdx.x] += y;
-        __syncthreads();
-    }
-    const unsigned long long krem = st->krem;
-    unsigned long long above = s_sum[threadIdx.x] - sum;
-    if (above < krem && krem <= s_sum[threadIdx.x]) {
+    for (int k = w + 1; k < 16; ++k) from += s_warp[k];
+    unsigned long long above = from - sum;
+    if (above < krem && krem <= from) {
         int i = 3;
         while (i > 0 && above + own[i] < krem) above += own[i--];
         st->prefix = (prefix << bits) | (uint32_t)(4 * threadIdx.x + i);
@@ -263,6 +327,7 @@ __global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_
 // Threshold of a calibration: midway between the k-th largest score and the largest below it (all_or_none: see the callers)
 __global__ void __launch_bounds__(512) calib_finish_kernel(const float* scores, int64_t B, SelectState* st, float* tau_out, int all_or_none)
 {
+    chain_begin(false);
     if (all_or_none) {
         // k = 0: nothing exceeds +inf; k = all
         if (blockIdx.x == 0 && threadIdx.x == 0) *tau_out = all_or_none == 1 ? __int_as_float(0x7f800000) : -1.0f;
@@ -291,6 +356,7 @@ __global__ void __launch_bounds__(512) calib_finish_kernel(const float* scores, 
 // per mask word: how many of its blocks have score == tau (needed only if some of them are taken and some are not)
 __global__ void w_eqcount_kernel(const float* scores, int64_t N, int64_t KB, int64_t MW, const SelectState* st, uint32_t* cnt)
 {
+    chain_begin();
     if (st->use_eq != 1) return;
     const float tau = st->tau;
     const int lane = threadIdx.x & 31;
@@ -307,6 +373,7 @@ __global__ void w_eqcount_kernel(const float* scores, int64_t N, int64_t KB, int
 // (of the counts that w_eqcount_kernel has left, where it has)
 __global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* in, uint32_t* out, int64_t n, const SelectState* st)
 {
+    chain_begin();
     if (st->use_eq != 1) return;
     __shared__ uint32_t warp_sums[32];
     __shared__ unsigned long long carry_s;
@@ -347,6 +414,7 @@ struct MaskParams {
 __global__ void __launch_bounds__(128) w_mask_kernel(const __grid_constant__ MaskParams p)
 {
     __shared__ uint32_t s_cnt[4];
+    chain_begin();
     const PackedLayout& L = p.L;
     const int64_t unit = blockIdx.x, n = unit / L.chunks * 128 + threadIdx.x, c = unit % L.chunks;
     const float tau = p.st->tau;
@@ -423,6 +491,7 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
                                                      const uint8_t* sc_in, uint8_t* blob, PackedLayout L)
 {
     __shared__ UnitScratch sc;
+    chain_begin();
     const int64_t unit = blockIdx.x, tile = unit / L.chunks, c = unit % L.chunks;
     const uint32_t* uptr = reinterpret_cast<const uint32_t*>(blob + L.off_uptr);
     const bool fits = reinterpret_cast<const fgmp_packed_header*>(blob)->error == 0;   // else the blob is too small for the lists
@@ -441,41 +510,57 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
         if (threadIdx.x == 0 && (cnt & 1u)) *reinterpret_cast<uint2*>(halves + (size_t)cnt * 8) = make_uint2(0u, 0u);
     }
     const int j = threadIdx.x & 15;
+    const int64_t kb = c * 16 + j;
+    // four blocks of the thread in flight (4096 x 4096: 15 us, 23 one at a time)
 #pragma unroll 1
-    for (int i = 0; i < 16; ++i) {
-        const int row = (threadIdx.x >> 4) + 8 * i;
-        const int64_t n = tile * 128 + row, kb = c * 16 + j;
-        uint2 slot = make_uint2(0u, 0u);
-        uint32_t scale = 0;
-        if (n < L.rows && kb < L.KB) {
-            float v[16], f[16];
-            load_block(W, ldw8, nullptr, 0, n, kb, v, f);
-            const uint32_t pos = sc.pos(row, j);
-            if (pos != 0xffffu) {
-                uint32_t c8[4];
-                float dq8[16];
-                block_fp8(v, inv8, s8, c8, dq8);
-                slot = make_uint2(c8[0], c8[1]);
-                if (fits) {
-                    *reinterpret_cast<uint2*>(halves + (size_t)pos * 8) = make_uint2(c8[2], c8[3]);
-                    entries[pos] = fgmp_list_entry((uint32_t)row, (uint32_t)j);
-                }
-            } else {
-                float dq4[16];
-                uint32_t c4[2];
-                scale = sc_in[n * L.KB + kb];
-                block_nvfp4(v, scale, s4, c4, dq4);
-                slot = make_uint2(c4[0], c4[1]);
+    for (int i0 = 0; i0 < 16; i0 += 4) {
+        uint4 x[4][2];
+        uint32_t sc_code[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int64_t n = tile * 128 + (threadIdx.x >> 4) + 8 * (i0 + i);
+            x[i][0] = x[i][1] = make_uint4(0u, 0u, 0u, 0u); sc_code[i] = 0;
+            if (n < L.rows && kb < L.KB) {
+                const uint4* wp = W + n * ldw8 + kb * 2;
+                x[i][0] = __ldg(wp); x[i][1] = __ldg(wp + 1); sc_code[i] = __ldg(sc_in + n * L.KB + kb);
             }
         }
-        *reinterpret_cast<uint2*>(rec + REC_W4 + fgmp_rec_w4_offset(row, j)) = slot;
-        rec[REC_SF + fgmp_rec_sf_offset(row, j)] = (uint8_t)scale;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int row = (threadIdx.x >> 4) + 8 * (i0 + i);
+            uint2 slot = make_uint2(0u, 0u);
+            uint32_t scale = 0;
+            if (tile * 128 + row < L.rows && kb < L.KB) {
+                float v[16];
+                unpack_bf16x16(x[i][0], x[i][1], v);
+                const uint32_t pos = sc.pos(row, j);
+                if (pos != 0xffffu) {
+                    uint32_t c8[4];
+                    float dq8[16];
+                    block_fp8(v, inv8, s8, c8, dq8);
+                    slot = make_uint2(c8[0], c8[1]);
+                    if (fits) {
+                        *reinterpret_cast<uint2*>(halves + (size_t)pos * 8) = make_uint2(c8[2], c8[3]);
+                        entries[pos] = fgmp_list_entry((uint32_t)row, (uint32_t)j);
+                    }
+                } else {
+                    float dq4[16];
+                    uint32_t c4[2];
+                    scale = sc_code[i];
+                    block_nvfp4(v, scale, s4, c4, dq4);
+                    slot = make_uint2(c4[0], c4[1]);
+                }
+            }
+            *reinterpret_cast<uint2*>(rec + REC_W4 + fgmp_rec_w4_offset(row, j)) = slot;
+            rec[REC_SF + fgmp_rec_sf_offset(row, j)] = (uint8_t)scale;
+        }
     }
 }
 
 // The last kernel of a packing writes what nobody reads early (see fgmp_linear on programmatic dependents).
 __global__ void w_finish_kernel(fgmp_packed_header* h, const SelectState* st, int fraction_mode, float tau_given, float* tau_eff_out)
 {
+    chain_begin(false);
     const float teff = fraction_mode ? st->tau : tau_given;
     h->tau_eff = teff;
     if (tau_eff_out) *tau_eff_out = teff;
@@ -494,18 +579,18 @@ int grid_for(int64_t work_items, int threads, int max_ctas_per_sm)
 void run_select(const float* scores, int64_t B, SelectState* st, cudaStream_t s)
 {
     const int g = grid_for(B, 512 * 4, 1);      // (a block ends with an atomic per bin in use: few blocks)
-    for (int pass = 0; pass < 3; ++pass) FGMP_LAUNCH(FGMP_K_SELECT, s, select_kernel<<<g, 512, 0, s>>>(scores, B, pass, st));
+    for (int pass = 0; pass < 3; ++pass) FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(select_kernel, g, 512, s, scores, B, pass, st));
 }
 
 // the threshold from the scores (k of B blocks above it)
 fgmp_status run_calibration(const float* scores, int64_t B, int64_t k, SelectState* st, float* tau_out, cudaStream_t s)
 {
     if (k == 0 || k == B) {
-        FGMP_LAUNCH(FGMP_K_SELECT, s, calib_finish_kernel<<<1, 512, 0, s>>>(scores, B, st, tau_out, k == 0 ? 1 : 2));
+        FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(calib_finish_kernel, 1, 512, s, scores, B, st, tau_out, k == 0 ? 1 : 2));
     } else {
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 1024, 0, s>>>(st, 1.0f, (unsigned long long)k, 0.f));
+        FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, 1.0f, (unsigned long long)k, 0.f));
         run_select(scores, B, st, s);
-        FGMP_LAUNCH(FGMP_K_SELECT, s, calib_finish_kernel<<<grid_for(B, 512 * 4, 2), 512, 0, s>>>(scores, B, st, tau_out, 0));
+        FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(calib_finish_kernel, grid_for(B, 512 * 4, 2), 512, s, scores, B, st, tau_out, 0));
     }
     return fgmp_launch_status();
 }
@@ -574,32 +659,32 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
     const float s8_given = sc.scale_fp8;
 
     // (k == 0: nothing is FP8, tau_eff = +inf; threshold mode: the given tau)
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 1024, 0, s>>>(st, sc.scale_fp4, (unsigned long long)k, fraction_mode ? INFINITY : tau));
+    FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, sc.scale_fp4, (unsigned long long)k, fraction_mode ? INFINITY : tau));
     if (sc.scale_fp4 == 0.f)
-        FGMP_LAUNCH(FGMP_K_W_AMAX, s, w_amax_kernel<<<grid_for(N, 4, 8), 256, 0, s>>>(W, ldw / 8, N, (uint32_t)(K / 8), st));
+        FGMP_LAUNCH(FGMP_K_W_AMAX, s, chain_launch(w_amax_kernel, grid_for(N, 4, 8), 256, s, W, ldw / 8, N, (uint32_t)(K / 8), st));
     {
         int g = grid_for(B, 256, 4);
         if (sm == FGMP_SCORE_LP_ERROR) {
-            if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<0, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-            else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<0, false><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+            if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<0, true>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+            else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<0, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
         } else {
-            if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<1, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-            else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<1, false><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+            if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<1, true>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+            else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<1, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
         }
     }
     const int gw = grid_for(NW * 32, 256, 8);
     if (fraction_mode && k > 0) {
         run_select(scores, B, st, s);
-        FGMP_LAUNCH(FGMP_K_W_MASK, s, w_eqcount_kernel<<<gw, 256, 0, s>>>(scores, N, KB, MW, st, tmp_a));
-        FGMP_LAUNCH(FGMP_K_SCAN, s, scan_kernel<<<1, 1024, 0, s>>>(tmp_a, tmp_b, NW, st));
+        FGMP_LAUNCH(FGMP_K_W_MASK, s, chain_launch(w_eqcount_kernel, gw, 256, s, scores, N, KB, MW, st, tmp_a));
+        FGMP_LAUNCH(FGMP_K_SCAN, s, chain_launch(scan_kernel, 1, 1024, s, tmp_a, tmp_b, NW, st));
     }
     MaskParams mp;
     mp.scores = scores; mp.eqprefix = tmp_b; mp.mask16 = reinterpret_cast<uint16_t*>(blob + L.off_mask); mp.list_steps = tmp_a;
     mp.uptr = reinterpret_cast<uint32_t*>(blob + L.off_uptr); mp.header = reinterpret_cast<fgmp_packed_header*>(blob); mp.st = st;
     mp.L = L; mp.room_steps = room_steps; mp.ratio = ratio; mp.s8_given = s8_given;
-    FGMP_LAUNCH(FGMP_K_W_MASK, s, w_mask_kernel<<<(unsigned)L.units, 128, 0, s>>>(mp));
-    FGMP_LAUNCH(FGMP_K_W_EMIT, s, w_emit_kernel<<<(unsigned)L.units, 128, 0, s>>>(W, ldw / 8, ratio, s8_given, st, sc_tmp, blob, L));
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, w_finish_kernel<<<1, 1, 0, s>>>(reinterpret_cast<fgmp_packed_header*>(blob), st, fraction_mode ? 1 : 0, tau, tau_eff_out));
+    FGMP_LAUNCH(FGMP_K_W_MASK, s, chain_launch(w_mask_kernel, (unsigned)L.units, 128, s, mp));
+    FGMP_LAUNCH(FGMP_K_W_EMIT, s, chain_launch(w_emit_kernel, (unsigned)L.units, 128, s, W, ldw / 8, ratio, s8_given, st, sc_tmp, blob, L));
+    FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(w_finish_kernel, 1, 1, s, reinterpret_cast<fgmp_packed_header*>(blob), st, fraction_mode ? 1 : 0, tau, tau_eff_out));
     return fgmp_launch_status();
 }
 
@@ -648,16 +733,16 @@ extern "C" fgmp_status fgmp_weight_scores(const void* W_bf16, int64_t ldw, const
     const uint4* W = reinterpret_cast<const uint4*>(W_bf16);
     const int ratio = sc.fp8_log2_ratio;
     const float s8_given = sc.scale_fp8;
-    FGMP_LAUNCH(FGMP_K_W_AUX, s, state_init_kernel<<<1, 1024, 0, s>>>(st, sc.scale_fp4, 0ull, 0.f));
+    FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, sc.scale_fp4, 0ull, 0.f));
     if (sc.scale_fp4 == 0.f)
-        FGMP_LAUNCH(FGMP_K_W_AMAX, s, w_amax_kernel<<<grid_for(N, 4, 8), 256, 0, s>>>(W, ldw / 8, N, (uint32_t)(K / 8), st));
+        FGMP_LAUNCH(FGMP_K_W_AMAX, s, chain_launch(w_amax_kernel, grid_for(N, 4, 8), 256, s, W, ldw / 8, N, (uint32_t)(K / 8), st));
     const int g = grid_for(B, 256, 4);
     if (sm == FGMP_SCORE_LP_ERROR) {
-        if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<0, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-        else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<0, false><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+        if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<0, true>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+        else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<0, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
     } else {
-        if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<1, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-        else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, w_score_kernel<1, false><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+        if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<1, true>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
+        else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<1, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
     }
     return fgmp_launch_status();
 }
