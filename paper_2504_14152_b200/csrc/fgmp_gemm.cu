@@ -560,10 +560,9 @@ static fgmp_status launch_prefill(const void* packed_acts, const void* packed_we
     fgmp_status st;
     if (nvfp4_first && (st = fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, true, s)) != FGMP_OK) return st;
     // At small and middling batches the weights are dequantized inside the GEMM, once per token tile; with many token tiles a
-    // plane that is expanded once is read faster than that.  Packed weights against planes, whole calls in us, weights 11008 x 4096: 25.4 and
-    // 49.3 at 48 tokens, 31.3 and 49.9 at 203, 47.9 and 70.5 at 400, 84.0 and 88.0 at 777, 102.9 and 89.3 at 1024, 183.1 and 139.6 at 2048;
-    // 4096 x 4096: 44.7 and 40.6 at 1024, 77.8 and 59.7 at 2048.  (Around 1000 tokens planes_us is some 15 to 20 % too high, so that
-    // the line lies a little late: 13 us at 1024 x 11008 x 4096 are the most it costs among these.)
+    // plane that is expanded once is read faster than that.  Packed weights against planes, whole calls in us on weights that alternate:
+    // 44 and 75 at 203 x 13824 x 5120; weights 11008 x 4096: 52 and 76 at 400 tokens, 74 and 95 at 777, 101 and 98 at 1024, 134 and 123 at 1500;
+    // 4096 x 4096: 51.4 and 50.5 at 1024, 56 and 64 at 1200 (two waves of pair tiles), 78 and 68 at 2048.
     // (Behind the all-NVFP4 GEMM: the way of two launches, not three.)
     if (!nvfp4_first && fgmp_mixed_us(M, N, K, ws_bytes) <= planes_us(M, N, K)) {
         st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, qn, leave, !nvfp4_first, s);

@@ -34,8 +34,9 @@ struct ActParams {
 template <int MODE, bool SCORE_ONLY>
 __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
 {
-    // A kernel launched behind this one as a programmatic dependent (the decode-sized GEMM) may
-    // start setting itself up now; it waits for this grid to complete before it reads the result.
+    // Comes up while the kernel before it ends, and waits for that.  Then a kernel launched behind this one as a programmatic dependent may
+    // start setting itself up (and read packed weights: all that came before this grid is done); it waits for this grid before it reads the result.
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (!SCORE_ONLY && blockIdx.x == 0 && threadIdx.x == 0) {
         fgmp_packed_header* h = p.header;
@@ -233,6 +234,18 @@ fgmp_status check_act_args(const void* X, int64_t ldx, const float* fisher, int6
     return FGMP_OK;
 }
 
+template <int MODE, bool SCORE_ONLY>
+void launch_quant(const ActParams& p, cudaStream_t s)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(((int64_t)p.groups * p.MW + QA_THREADS / 32 - 1) / (QA_THREADS / 32)));
+    cfg.blockDim = dim3(QA_THREADS); cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, quant_act_kernel<MODE, SCORE_ONLY>, p);
+}
+
 ActParams make_act_params(const void* X, int64_t ldx, const float* fisher, int64_t M, int64_t K, fgmp_scales sc, float tau)
 {
     ActParams p{};
@@ -277,9 +290,8 @@ extern "C" fgmp_status fgmp_quantize_activations(const void* X_bf16, int64_t ldx
     p.mask = reinterpret_cast<uint32_t*>(blob + L.off_mask); p.codes8 = blob + L.off_codes8;
     p.header = reinterpret_cast<fgmp_packed_header*>(blob);
     if (M <= 16 && !p.free8) p.arec = blob + L.off_arec;     // decode-sized batch: also emit the records of the decode GEMM (tied scales only)
-    const dim3 grid((unsigned)(((int64_t)p.groups * p.MW + QA_THREADS / 32 - 1) / (QA_THREADS / 32)));
-    if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, quant_act_kernel<0, false><<<grid, QA_THREADS, 0, s>>>(p));
-    else                           FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, quant_act_kernel<1, false><<<grid, QA_THREADS, 0, s>>>(p));
+    if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, launch_quant<0, false>(p, s));
+    else                           FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, launch_quant<1, false>(p, s));
     return fgmp_launch_status();
 }
 
@@ -294,9 +306,8 @@ extern "C" fgmp_status fgmp_activation_scores(const void* X_bf16, int64_t ldx, c
     cudaStream_t s = (cudaStream_t)cuda_stream;
     ActParams p = make_act_params(X_bf16, ldx, fisher_chan, M, K, sc, 0.f);
     p.scores = scores;
-    const dim3 grid((unsigned)(((int64_t)p.groups * p.MW + QA_THREADS / 32 - 1) / (QA_THREADS / 32)));
-    if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, quant_act_kernel<0, true><<<grid, QA_THREADS, 0, s>>>(p));
-    else                           FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, quant_act_kernel<1, true><<<grid, QA_THREADS, 0, s>>>(p));
+    if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, launch_quant<0, true>(p, s));
+    else                           FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, launch_quant<1, true>(p, s));
     return fgmp_launch_status();
 }
 
