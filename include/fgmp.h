@@ -262,7 +262,8 @@ fgmp_status fgmp_linear_classes(const void* packed_acts, const void* packed_weig
  * per block, the same single-precision steps in the same order, so codes, scales and masks are those of
  * fgmp_quantize_activations bit for bit), while the first weight records are already on their way, and
  * start multiplying once every chunk has been handed in.  (One or two tokens without packed_acts_out: every thread
- * block quantizes what its own part of the weights is multiplied with, and nothing is handed in.)  Y is what fgmp_linear
+ * block quantizes what its own part of the weights is multiplied with, and nothing is handed in, unless the weights are very
+ * large.)  Y is what fgmp_linear
  * returns for those packed activations, bit for bit.
  *   packed_acts_out (may be NULL): receives the packed activations (size fgmp_acts_bytes(M, K)) for a
  *     caller that wants them (fgmp_unpack, or a later fgmp_linear with other weights); if NULL only the

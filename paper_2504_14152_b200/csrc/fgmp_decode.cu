@@ -33,7 +33,8 @@
 //                need, unit by unit, straight into the stages.  That is more work in all, and nothing to hand over: 2.7 us lie between the end of the
 //                kernel before and the last shared record, 0.7 more until its copy is in.  11008 x 4096: 1 token 14.4 -> 11.0 us, 2 tokens
 //                16.9 -> 12.2; 28672 x 8192: 33.5 -> 30.0 and 38.7 -> 32.9.  (With 64 threads a token for every unit in turn instead of two units at a
-//                time, two tokens take 14.5 and 48.6: beyond a dozen units that is slower than the shared quantizer.)
+//                time, two tokens take 14.5 and 48.6: beyond a dozen units that is slower than the shared quantizer.)  Where a CTA has very many units
+//                the warps that quantize for each of them cost more than the hand-over: see the launch.
 //   DEC_UNPACK   fgmp_linear: made unit by unit in shared memory from the packed activations' records.
 //
 // Warp roles: warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, from warp 2 on two or three sets of four warps that take
@@ -67,9 +68,9 @@ constexpr uint32_t STG_STEP = STG_LIST + LIST_CAP;                           // 
 constexpr uint32_t AREC_GAP = AREC_AT - AREC_HOT;
 __host__ __device__ inline uint32_t arec_gap(int64_t M) { return M >= 14 ? AREC_GAP : 0u; }
 constexpr int DEC_MAX_STAGES = 6;
-// Two sets; three where the quantizer is the CTA's own (the accumulators of two tokens leave the tensor memory for it): 11.2 us instead of 11.3 at one
-// token of 11008 x 4096, 30.6 instead of 31.0 of 28672 x 8192.  For the shared quantizer it is no gain: eight tokens of 28672 x 8192 39.4 instead of
-// 36.1.
+// Two sets; three for one and two tokens without the packed form (their accumulators leave the tensor memory for it): 11.2 us instead of 11.3 at one
+// token of 11008 x 4096, 28.8 and 28.7 of 28672 x 8192; with 20 % FP8 blocks, whose second halves come from global memory, 37 instead of 47.  For more
+// tokens it is no gain: eight of 28672 x 8192 39.4 instead of 36.1.
 // Tensor memory columns: accumulators (two buffers of each kind); of each set: a dense E4M3 tile of 64, scales (32)
 template <int SETS> struct Dec {
     static constexpr int W_EPI = W_SET + 4 * SETS, W_STEP = W_EPI + 4;
@@ -879,7 +880,7 @@ fgmp_status set_attrs_once()
         bool ok = true;
         for (const void* k : {(const void*)decode_kernel<DEC_FUSED_LP, 2>, (const void*)decode_kernel<DEC_FUSED_HP, 2>, (const void*)decode_kernel<DEC_OWN1_LP, 3>,
                               (const void*)decode_kernel<DEC_OWN1_HP, 3>, (const void*)decode_kernel<DEC_OWN2_LP, 3>, (const void*)decode_kernel<DEC_OWN2_HP, 3>,
-                              (const void*)decode_kernel<DEC_UNPACK, 2>})
+                              (const void*)decode_kernel<DEC_FUSED_LP, 3>, (const void*)decode_kernel<DEC_FUSED_HP, 3>, (const void*)decode_kernel<DEC_UNPACK, 2>})
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) == cudaSuccess;
         if (!ok)
             return FGMP_ERR_CUDA;
@@ -1010,8 +1011,15 @@ extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const 
     }
     p.steps = (uint8_t*)workspace + fgmp_align1k(fgmp_ws_decode(M, N, K));
     const auto launch = [&](auto lp, auto hp) { return (sm == FGMP_SCORE_LP_ERROR ? lp : hp)(p, d, true, (cudaStream_t)cuda_stream); };
-    if (M == 1 && !packed_acts_out) return launch(launch_decode<DEC_OWN1_LP, 3>, launch_decode<DEC_OWN1_HP, 3>);
-    if (M == 2 && !packed_acts_out) return launch(launch_decode<DEC_OWN2_LP, 3>, launch_decode<DEC_OWN2_HP, 3>);
+    // One or two tokens: the quantizer in every CTA saves 3 us of hand-over, but costs each unit some issue slots.  Us with it, with the shared one and
+    // three sets, and with two sets, by units per CTA, 10 % FP8 blocks: two tokens 30.4, 32.2, 31.9 at 48, 36.0, 36.6, 36.4 at 54, 51.1, 50.5, 51.8
+    // at 85, 70.1, 66.0, 65.7 at 108, 134, 122, 125 at 217; one token 61.4, 67.0, 66.5 at 108, 88.5, 89.4, 96.4 at 162, 135, 130, 130 at 217.
+    // (Without FP8 blocks two tokens take 42.1, 43.6, 43.5 at 85 and 112, 100, 101 at 217; with 20 % 62.8, 64.8, 81.0 and 166, 164, 197.)
+    if (M <= 2 && !packed_acts_out) {
+        if (d.total > (int64_t)d.grid * (M == 1 ? 200 : 80)) return launch(launch_decode<DEC_FUSED_LP, 3>, launch_decode<DEC_FUSED_HP, 3>);
+        if (M == 1) return launch(launch_decode<DEC_OWN1_LP, 3>, launch_decode<DEC_OWN1_HP, 3>);
+        return launch(launch_decode<DEC_OWN2_LP, 3>, launch_decode<DEC_OWN2_HP, 3>);
+    }
     return launch(launch_decode<DEC_FUSED_LP, 2>, launch_decode<DEC_FUSED_HP, 2>);
 }
 

@@ -212,3 +212,27 @@ def test_quantizer_in_every_cta(fg, M, N, K, frac_w, mode):
     wide = torch.randn(M, K + 8, generator=torch.Generator().manual_seed(1)).to(torch.bfloat16).cuda()
     wide[:, :K] = x.cuda()
     assert torch.equal(fg.linear_fused(wide[:, :K], fx.cuda(), pw, **args), y), "rows further apart"
+
+
+# One or two tokens where the quantizer goes from every CTA to the shared one, by the units of weights that a CTA has: what is shared passes through the
+# workspace.  The same sums either way, and those of the packed tokens.
+@pytest.mark.parametrize("M,units,shared", [(1, 200, False), (1, 201, True), (2, 80, False), (2, 81, True)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_quantizer_of_one_and_two_tokens_by_units_per_cta(fg, M, units, shared, mode):
+    K = 8192
+    N = 128 * (torch.cuda.get_device_properties(0).multi_processor_count * units // (K // 256))
+    w = draw_weights(fg, N, K, 75)
+    g = torch.Generator(device="cuda").manual_seed(units)
+    x, f = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16), torch.rand(K, generator=g, device="cuda") + 0.5
+    s4 = float(x.abs().max()) / 2688.0
+    args = dict(scale_fp4=s4, score_mode=mode, tau=float(fg.calibrate_tau(x, f, scale_fp4=s4, fp8_fraction=0.2, score_mode=mode)))
+    ws = fg.alloc_workspace(fg.OP_LINEAR_FUSED, M, N, K, torch.device("cuda"))
+    records = ws[-(K // 256) * 8192:]                     # (a chunk's record takes at least as much)
+    records.fill_(0x5a)
+    y = fg.linear_fused(x, f, w, workspace=ws, **args)
+    fg.check(ws)
+    assert bool((records != 0x5a).any()) == shared
+    want = fg.linear(fg.quantize_activations(x, f, **args), w)
+    for _ in range(3):
+        assert torch.equal(fg.linear_fused(x, f, w, workspace=ws, **args), want)
+    assert torch.equal(y, want) and torch.equal(fg.linear_fused(x, f, w, want_packed=True, workspace=ws, **args)[0], want)
