@@ -9,7 +9,7 @@ namespace {
 
 constexpr int SEL_BINS = 2048;           // bins of a digit of the radix select
 
-// The calls here are chains of small kernels.  Each (but for the clip search) is launched as a programmatic dependent of the one before it: its blocks come up while
+// The calls here are chains of small kernels.  Each (but see launch_score) is launched as a programmatic dependent of the one before it: its blocks come up while
 // that one runs and wait for its end (every block does, so that a kernel's end implies those of all before it).  The last kernel of a packing lets
 // nothing start early, since the GEMMs read packed weights before they wait.  (4096 x 4096 weights and a calibration batch of 512 tokens,
 // eighteen launches: 20 us of 311.)
@@ -202,9 +202,7 @@ struct ClipOrder {
 // this rests on, and all scales are looked at.)  Going up there are few codes left, because the tensor
 // scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left, 26 for the longest of a warp, and 20 if the warps of a thread
 // block share its 256 blocks out in the order of their dynamic-max codes, that is of how many there are above: 4096 x 4096 takes 145 us,
-// 152 in the order of the tensor, 172 without packed fp32 instructions, 680 with all 126.  No programmatic dependent: its thread blocks would come up where
-// the kernel before it leaves room first, the ones with a round more than the others side by side on a few SMs (scores of 4160 x 1280, 2.2 rounds: 67 us, 56
-// when they start together; of 4096 x 4096 152 and 153).
+// 152 in the order of the tensor, 172 without packed fp32 instructions, 680 with all 126.
 template <int MODE, bool CLIP>
 __global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ldw8, const float* F, int64_t ldf,
                                                       int64_t N, int64_t KB, int ratio, float s8_given, const SelectState* st,
@@ -577,6 +575,25 @@ int grid_for(int64_t work_items, int threads, int max_ctas_per_sm)
     return (int)g;
 }
 
+// Microscales and scores of all blocks.  The clip search is no programmatic dependent where its loop goes round fewer than four times: its thread blocks would come
+// up where the kernel before it leaves room first, and the ones with a round more than the others, the first of the grid, side by side on a few SMs
+// (scores of 4160 x 1280, 2.2 rounds: 67 us, 56 when they start together; 3600 x 2048, 3.04: 74 and 72; 4096 x 4096, 6.9: 152 both ways, a packing 271
+// and 274).
+template <int MODE, bool CLIP, typename... A>
+void launch_score(int64_t B, cudaStream_t s, A... args)
+{
+    const int g = grid_for(B, 256, 4);
+    if (CLIP && B < (int64_t)g * 256 * 4) w_score_kernel<MODE, CLIP><<<g, 256, 0, s>>>(args...);
+    else chain_launch(w_score_kernel<MODE, CLIP>, g, 256, s, args...);
+}
+template <typename... A>
+void run_scores(fgmp_score_mode sm, fgmp_clip_mode cm, int64_t B, cudaStream_t s, A... args)
+{
+    const bool clip = cm == FGMP_CLIP_SW_BRUTE, lp = sm == FGMP_SCORE_LP_ERROR;
+    FGMP_LAUNCH(FGMP_K_W_SCORE, s, lp ? (clip ? launch_score<0, true>(B, s, args...) : launch_score<0, false>(B, s, args...))
+                                      : (clip ? launch_score<1, true>(B, s, args...) : launch_score<1, false>(B, s, args...)));
+}
+
 // three-pass radix select for the k-th largest of scores[0..B)
 void run_select(const float* scores, int64_t B, SelectState* st, cudaStream_t s)
 {
@@ -664,16 +681,7 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
     FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, sc.scale_fp4, (unsigned long long)k, fraction_mode ? INFINITY : tau));
     if (sc.scale_fp4 == 0.f)
         FGMP_LAUNCH(FGMP_K_W_AMAX, s, chain_launch(w_amax_kernel, grid_for(N, 4, 8), 256, s, W, ldw / 8, N, (uint32_t)(K / 8), st));
-    {
-        int g = grid_for(B, 256, 4);
-        if (sm == FGMP_SCORE_LP_ERROR) {
-            if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, (w_score_kernel<0, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores)));
-            else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<0, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-        } else {
-            if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, (w_score_kernel<1, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores)));
-            else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<1, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-        }
-    }
+    run_scores(sm, cm, B, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, (const SelectState*)st, sc_tmp, scores);
     const int gw = grid_for(NW * 32, 256, 8);
     if (fraction_mode && k > 0) {
         run_select(scores, B, st, s);
@@ -738,14 +746,7 @@ extern "C" fgmp_status fgmp_weight_scores(const void* W_bf16, int64_t ldw, const
     FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, sc.scale_fp4, 0ull, 0.f));
     if (sc.scale_fp4 == 0.f)
         FGMP_LAUNCH(FGMP_K_W_AMAX, s, chain_launch(w_amax_kernel, grid_for(N, 4, 8), 256, s, W, ldw / 8, N, (uint32_t)(K / 8), st));
-    const int g = grid_for(B, 256, 4);
-    if (sm == FGMP_SCORE_LP_ERROR) {
-        if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, (w_score_kernel<0, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores)));
-        else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<0, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-    } else {
-        if (cm == FGMP_CLIP_SW_BRUTE) FGMP_LAUNCH(FGMP_K_W_SCORE, s, (w_score_kernel<1, true><<<g, 256, 0, s>>>(W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores)));
-        else                          FGMP_LAUNCH(FGMP_K_W_SCORE, s, chain_launch(w_score_kernel<1, false>, g, 256, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, st, sc_tmp, scores));
-    }
+    run_scores(sm, cm, B, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, (const SelectState*)st, sc_tmp, scores);
     return fgmp_launch_status();
 }
 
