@@ -222,7 +222,7 @@ fgmp_status fgmp_workspace_init(void* workspace, size_t ws_bytes, void* cuda_str
  * applied, accumulated in FP32.  Y is fp32 (y_is_bf16 = 0) or bf16 [M, ldy].  The workspace
  * must have been cleared once with fgmp_workspace_init; one that is sized for a batch of prefill size serves every smaller
  * one of the same layer (with less room than fgmp_workspace_bytes asks for, the work may be cut another way, and the sums
- * taken in another order).  For 1 <= M <= 16, K % 256 == 0 and
+ * taken in another order).  For that it asks for more than the batch itself may use: a smaller batch's partial sums can take more room.  For 1 <= M <= 16, K % 256 == 0 and
  * N <= 258048 the weight-streaming kernel runs, launched as a programmatic dependent of the kernel
  * before it in the stream (its set-up and its first reads of packed_weights overlap that kernel's
  * end; it reads the packed activations and the workspace only after that kernel has completed).  So
@@ -330,6 +330,14 @@ fgmp_status fgmp_linear_static(const void* packed_acts, const void* packed_weigh
  * header does not match the call).  A call of prefill size (M > 16 or K % 256 != 0) starts the status anew, so that
  * it speaks of that call; decode-sized calls leave an earlier error in place. */
 fgmp_status fgmp_check(const void* workspace, void* cuda_stream);
+
+/* ---- parity support: how a call of more than 16 tokens is cut (host only, nothing is launched) ----
+ * For the shape of an fgmp_linear or fgmp_linear_quantize and a workspace of ws_bytes: returns 1 if the call goes through the GEMM on the packed
+ * weights, 0 if through another kernel (operands without FP8 blocks may be taken by the NVFP4 GEMM whatever this says, and rows of Y
+ * that a pitch of its own puts off 16-byte boundaries by the packed weights).  cut, filled in the
+ * first case: tokens of a tile; elements of K that a step of the GEMM takes (64 or 128); accumulators (1 or 2); whether thread blocks share
+ * tiles (1) or each has tiles of its own (0); steps in shared memory; steps in tensor memory. */
+int fgmp_linear_cut(int64_t M, int64_t N, int64_t K, size_t ws_bytes, int32_t cut[6]);
 
 /* ---- parity support: packed -> canonical arrays (device) ----
  * codes4 [rows*K/2] (0 for FP8 blocks), codes8 [rows*K] (0 for FP4 blocks), scales

@@ -537,12 +537,28 @@ static fgmp_status launch_pair_gemm(const GemmParams& p, const uint8_t* planeA, 
     return fgmp_launch_status();
 }
 
-// Modelled time in us of expansion and pair GEMM, beside fgmp_mixed_us: launches and tails, 0.5 us per million elements of either operand, then waves of
-// 256 x 256 tiles over the pairs at 0.32 us per 64 elements of K (13 shapes from 128 to 2048 tokens: within 10 %).
-static double planes_us(int64_t M, int64_t N, int64_t K)
+// Modelled time in us of a call over planes, beside fgmp_mixed_us and fitted with it: 0.574 us per million elements of either operand, then waves of 256 x
+// 256 tiles over the pairs at 0.267 us per 64 elements of K.  A tile's way out takes 4.9 us (with the quantizer in it 10.3, counted to three tenths where
+// a call with it is possible), behind the next tile's products as far as those take that long.  by_element: rows of Y that are not 16-byte aligned leave
+// an element at a time, 40 us a tile in bf16, 24.5 in fp32 (2364 x 8087 x 512, bf16: 233 us, 58 on the packed weights).  Where N says so a caller's
+// pitch may avoid that, but the sums are the same with any pitch; so the line lies where neither rows as they come nor wider ones lose (404 calls).
+static double planes_us(int64_t M, int64_t N, int64_t K, bool by_element)
 {
     const int64_t tiles = ((M + P_BM - 1) / P_BM) * ((N + P_BN - 1) / P_BN), pairs = fgmp_sm_count() / 2;
-    return 8.0 + 0.5e-6 * (double)(M + N) * (double)K + (double)((tiles + pairs - 1) / pairs) * (double)(K / 64) * 0.32;
+    const double more = (double)((tiles + pairs - 1) / pairs - 1), tile = 0.267 * (double)(K / 64), expand = 0.574e-6 * (double)(M + N) * (double)K;
+    if (by_element) return 1.15 * (expand + more * fmax(tile, 8.0) + tile) + 20.0;
+    const bool both = N % 64 == 0;
+    return expand + more * fmax(tile, both ? 6.5 : 4.9) + tile + (both ? 12.7 : 11.0);
+}
+
+// At small and middling batches the weights are dequantized inside the GEMM, once per token tile; with many token tiles a
+// plane that is expanded once is read faster than that.  Packed weights against planes, whole calls in us on weights that alternate:
+// 44 and 75 at 203 x 13824 x 5120; weights 11008 x 4096: 52 and 76 at 400 tokens, 74 and 95 at 777, 96 and 91 at 1024, 134 and 123 at 1500;
+// 4096 x 4096: 51.4 and 50.5 at 1024, 56 and 64 at 1200 (two waves of pair tiles), 78 and 68 at 2048; short rows of weights, whose tiles' way out
+// is not hidden: 63 and 41 at 1220 x 15936 x 768.
+static bool on_packed_weights(int64_t M, int64_t N, int64_t K, size_t ws_bytes, bool aligned_pitch)
+{
+    return fgmp_mixed_us(M, N, K, ws_bytes) <= planes_us(M, N, K, N % 8 != 0 || !aligned_pitch);
 }
 
 // M > 16 or a shape the weight-streaming kernel does not take.  nvfp4: what the caller expects of the operands, see fgmp_linear_expect.
@@ -559,12 +575,8 @@ static fgmp_status launch_prefill(const void* packed_acts, const void* packed_we
     const bool leave = !qn.codes4 && nvfp4 != 0, nvfp4_first = leave && nvfp4 == 1;
     fgmp_status st;
     if (nvfp4_first && (st = fgmp_launch_gemm_nvfp4(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, status, true, s)) != FGMP_OK) return st;
-    // At small and middling batches the weights are dequantized inside the GEMM, once per token tile; with many token tiles a
-    // plane that is expanded once is read faster than that.  Packed weights against planes, whole calls in us on weights that alternate:
-    // 44 and 75 at 203 x 13824 x 5120; weights 11008 x 4096: 52 and 76 at 400 tokens, 74 and 95 at 777, 101 and 98 at 1024, 134 and 123 at 1500;
-    // 4096 x 4096: 51.4 and 50.5 at 1024, 56 and 64 at 1200 (two waves of pair tiles), 78 and 68 at 2048.
     // (Behind the all-NVFP4 GEMM: the way of two launches, not three.)
-    if (!nvfp4_first && fgmp_mixed_us(M, N, K, ws_bytes) <= planes_us(M, N, K)) {
+    if (!nvfp4_first && on_packed_weights(M, N, K, ws_bytes, qn.codes4 || ldy * (y_is_bf16 ? 2 : 4) % 16 == 0)) {
         st = fgmp_linear_mixed(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, qn, leave, !nvfp4_first, s);
     } else {
         uint8_t* planeA = ws + FGMP_WS_CONTROL_BYTES;   // the control area stays as the decode-sized calls need it
@@ -597,6 +609,13 @@ extern "C" fgmp_status fgmp_linear_expect(const void* packed_acts, const void* p
         return fgmp_linear_decode(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, false, s);
     QuantNext off{};
     return launch_prefill(packed_acts, packed_weights, Y, y_is_bf16, ldy, M, N, K, workspace, ws_bytes, off, nvfp4, s);
+}
+
+extern "C" int fgmp_linear_cut(int64_t M, int64_t N, int64_t K, size_t ws_bytes, int32_t cut[6])
+{
+    if (M < 1 || N < 1 || K < 64 || (K % 64) != 0 || !cut || fgmp_decode_supported(M, N, K) || !on_packed_weights(M, N, K, ws_bytes, true)) return 0;
+    fgmp_mixed_cut(M, N, K, ws_bytes, cut);
+    return 1;
 }
 
 extern "C" fgmp_status fgmp_linear(const void* packed_acts, const void* packed_weights,

@@ -51,9 +51,10 @@ fgmp_status fgmp_launch_gemm_nvfp4(const void* packed_acts, const void* packed_w
 fgmp_status fgmp_expand(const void* packed_acts, const void* packed_weights, int64_t M, int64_t N, int64_t K, uint8_t* planeA, uint8_t* planeW,
                         int* status, int cls_a, int cls_w, bool leave_nvfp4, bool first, cudaStream_t s);
 
-// GEMM on the packed weights (fgmp_mixed.cu), and its modelled time in a workspace of that size
+// GEMM on the packed weights (fgmp_mixed.cu), and the modelled time of a call in a workspace of that size
 struct QuantNext;
 double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes);
+void fgmp_mixed_cut(int64_t M, int64_t N, int64_t K, size_t ws_bytes, int32_t* cut);          // see fgmp_linear_cut
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K);
 fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weights, void* Y, int y_is_bf16, int64_t ldy,
                               int64_t M, int64_t N, int64_t K, void* workspace, size_t ws_bytes, const QuantNext& qn, bool leave_nvfp4, bool first, cudaStream_t s);

@@ -548,35 +548,70 @@ __global__ void __launch_bounds__(QUANT ? 128 : 256) mixed_reduce_kernel(const _
 // ------------------------------------------------------------------ host side
 constexpr uint32_t MX_FIXED = 1024 /*alignment*/ + 1024 /*barriers, stage table*/, MX_TURN = 4 * 32 * 33 * 4 + 128;
 
-// Modelled time of a unit in us.  Up to 160 tokens there are two accumulators beside the slots (measured 1.05 up to 96 tokens, 1.15 at 128, 1.22 at
-// 160), up to 208 steps of 128 elements (1.5 at 176, 1.6 at 208), beyond 256 two products to a step (1.9 at 256, 2.3 at 272, 2.6 at 352, 2.9 at 400).
-double unit_us(uint32_t n_tok)
-{
-    return n_tok <= 160 ? fmax(1.05, 0.55 + 0.0042 * n_tok) : n_tok <= 256 ? 0.55 + 0.0053 * n_tok : 0.90 + 0.0050 * n_tok;
-}
-
 // bytes for the parts of shared tiles: at most two tiles of a span are shared
 size_t parts_bytes(const MixedPlan& pl) { return pl.split ? (size_t)pl.grid * 2 * ((pl.n_tok + 31u) & ~31u) * 512 : 0; }
 
+// Modelled time in us of a call that is cut as pl says: launches, the expansion of the activations, the GEMM, the sum over parts.  A fit to every way of
+// cutting 780 random shapes (17 to 8192 tokens, weights of 250 to 28672 rows, 192 to 28672 columns; calls in a row on weights that alternate): the
+// way with the least modelled time, among these and the planes (planes_us), takes 1.02 times the best one's on average, 1.07 at the 95th percentile.  (By a
+// model fitted to 13 shapes before that 1.09 and 1.38; against the form and the model before that one calls now take 0.86 of the time, at
+// most 5 % more within the sizes that it was fitted to.)
+//   - a unit: 0.88 us up to 48 tokens, 1.1 at 160 with two accumulators; 1.27 at 208 with one and steps of 128 elements; 1.45 at 256; 2.3 at 400 with
+//     two products to a step.  In spans 6 and 13 % more.
+//   - the way out of a whole tile, a row of weights to a lane: 6.6 us at 160 tokens.  A second accumulator hides it behind
+//     the next tile's products as far as those take that long, six chunks; with fewer it is what such a call takes (1220 x 15936 x 768: 63 us, on the planes 41).
+//   - the sum over parts: a part after the other, 0.34 us each where a tile has a thread block of its own for its 32 columns (53 x 644 x 8960: one tile of
+//     64 tokens in 26 parts 25 us, of 16 tokens in 7 parts 18)
+//   - launches: the next kernel's thread blocks come up early only where SMs are left that the GEMM does not fill (310 x 448 x 1280: 13.8 us on 140, 10.4
+//     on 100)
+// Where a call with the next layer's quantizer in it is possible its way out counts as well (1.34 us + 0.0403 per token, 3.4 + 0.51 per part), to three tenths: the two
+// calls are cut alike, so that their sums are the same.
+double mixed_us(const MixedPlan& pl, int64_t M, int64_t N, int64_t K)
+{
+    const double n = pl.n_tok, sms = fgmp_sm_count(), left = sms - pl.grid, units = pl.span + (pl.rest ? 1.0 : 0.0);
+    const bool both = N % 64 == 0;
+    const double unit = pl.naccs == 2 ? fmax(0.88, 0.77 + 0.0021 * n) : pl.ks == 2 ? 0.50 + 0.0037 * n : n <= 256 ? 0.475 + 0.0038 * n : 0.495 + 0.0045 * n;
+    const double out = both ? 0.93 + 0.0375 * n : 0.77 + 0.0363 * n;
+    double us = 4.4 + 0.59e-6 * (double)M * (double)K;
+    if ((double)M * (double)K > 6.0 * 8192.0 * left) us += 2.2;
+    if (!pl.split) {
+        const double tile = unit * (double)K / 256.0;
+        return us + (pl.naccs == 2 ? (units - 1.0) * fmax(tile, out) + tile + out : units * (tile + out));
+    }
+    const double inner = fmax(0.0, units / pl.chunks - 1.0) * out, work = (pl.naccs == 2 ? 1.06 : 1.13) * units * unit;
+    const double blocks = pl.tiles * (double)((pl.n_tok + 31) / 32), chain = (1.0 + (double)pl.grid / pl.tiles) * fmax(1.0, 0.75 * blocks / sms);
+    us += pl.naccs == 2 ? fmax(work, inner) + 0.3 : work + inner + 0.5;
+    us += (both ? 2.07 + 0.392 * chain : 1.48 + 0.344 * chain) + 0.012 * n;
+    return blocks > 2.0 * left ? us + 1.4 : us;
+}
+
+// What workspaces are sized by (fgmp_ws_mixed): the figures of an earlier form of the kernel, which cut the work into wider tiles and more often in spans.
+double roomy_us(const MixedPlan& pl)
+{
+    const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / pl.chunks;
+    const double drains = 2 * pl.n_tok + 96 <= MX_TMEM_COLS || tiles < 1.0 ? 1.0 : pl.n_tok <= 256 ? tiles : 2.0 * (tiles + 1.0);
+    return units * (1.08 + 0.0042 * pl.n_tok) + drains * 0.012 * pl.n_tok + (pl.split ? 2.0 + 2.6 * pl.grid * pl.n_tok * 512.0 / 8e6 : 3.0 * tiles);
+}
+
 // How the work is cut: tokens per tile, and whether CTAs take whole tiles or equal spans of units: the least modelled time among the
-// ways whose parts of tiles fit in `room_for_parts` bytes.  (Against every way measured, 13 shapes from 128 to 2048 tokens: the one it takes is the
-// fastest or within 5 % of it.)  `earlier`: by the figures of an earlier form of the kernel, which cut the work into wider tiles.  What callers are
-// asked for as a workspace goes by both, so that it is nowhere less than it was.
-MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts, bool earlier = false)
+// ways whose parts of tiles fit in `room_for_parts` bytes.
+MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts, bool roomy = false)
 {
     const uint32_t wtiles = (uint32_t)((N + 127) / 128), chunks = (uint32_t)((K / 64 + 3) / 4), sms = (uint32_t)fgmp_sm_count();
-    const uint32_t t_min = (uint32_t)((M + MX_MAX_TOK - 1) / MX_MAX_TOK), t_max = 2 * (uint32_t)((M + 255) / 256) + 2;
+    const uint32_t t_min = (uint32_t)((M + MX_MAX_TOK - 1) / MX_MAX_TOK), t_max = 2 * (uint32_t)((M + 255) / 256) + (roomy ? 1 : 8);
     MixedPlan best{};
     best.us = 1e300;
-    for (uint32_t T = t_min; T < t_max && (int64_t)(T - 1) * 16 < M; ++T) {
+    for (uint32_t T = t_min, before = 0; T <= t_max && (int64_t)(T - 1) * 16 < M; ++T) {
         MixedPlan pl{};
         pl.chunks = chunks;
         pl.n_tok = (uint32_t)((M + T - 1) / T + 15) / 16 * 16;
+        if (pl.n_tok == before) continue;
+        before = pl.n_tok;
         pl.n_half = pl.n_tok <= 256 ? pl.n_tok : (pl.n_tok + 31) / 32 * 16;
         pl.tok_tiles = (uint32_t)((M + pl.n_tok - 1) / pl.n_tok);
         pl.tiles = wtiles * pl.tok_tiles;
         pl.ks = pl.n_tok <= 208 ? 2 : 1;
-        pl.naccs = 2 * pl.n_tok + (earlier ? 96 : 96 * pl.ks) <= MX_TMEM_COLS ? 2 : 1;
+        pl.naccs = 2 * pl.n_tok + 96 * pl.ks <= MX_TMEM_COLS ? 2 : 1;
         const uint64_t total = (uint64_t)pl.tiles * chunks;
         for (int split = 0; split < (chunks > 1 ? 2 : 1); ++split) {
             pl.quantum = split ? 1 : chunks;
@@ -587,16 +622,7 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts, boo
             pl.split = split;
             if (split && pl.rest == 0 && pl.span % chunks == 0) continue;
             if (parts_bytes(pl) > room_for_parts) continue;
-            const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / chunks;
-            if (earlier) {
-                const double drains = pl.naccs == 2 || tiles < 1.0 ? 1.0 : pl.n_tok <= 256 ? tiles : 2.0 * (tiles + 1.0);
-                pl.us = units * (1.08 + 0.0042 * pl.n_tok) + drains * 0.012 * pl.n_tok + (split ? 2.0 + 2.6 * pl.grid * pl.n_tok * 512.0 / 8e6 : 3.0 * tiles);
-            } else {
-                // reading an accumulator out hides behind the next tile's products if there are two
-                pl.us = 2.0 + units * unit_us(pl.n_tok) + (pl.naccs == 2 ? 1.0 : split ? 0.7 * (tiles + 1.0) : tiles) * 0.0105 * pl.n_tok;
-                // the second kernel, and what it moves: a partial tile per span or two, written and read
-                if (split) pl.us += 2.5 + 1.42 * fmin(2.0 * pl.grid, (double)pl.grid + pl.tiles) * pl.n_tok * 512.0 / 8e6;
-            }
+            pl.us = roomy ? roomy_us(pl) : mixed_us(pl, M, N, K);
             if (pl.us < best.us) best = pl;
         }
     }
@@ -626,13 +652,21 @@ static size_t room_in(size_t ws_bytes, int64_t M, int64_t K)
     return ws_bytes > before ? ws_bytes - before : 0;
 }
 
-// (with the expansion of the activations: a launch, and 0.65 us per million elements)
-double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes) { return 2.0 + 0.65e-6 * (double)M * (double)K + mixed_plan(M, N, K, room_in(ws_bytes, M, K)).us; }
+double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes) { return mixed_plan(M, N, K, room_in(ws_bytes, M, K)).us; }
 
+void fgmp_mixed_cut(int64_t M, int64_t N, int64_t K, size_t ws_bytes, int32_t* cut)
+{
+    const MixedPlan pl = mixed_plan(M, N, K, room_in(ws_bytes, M, K));
+    const uint32_t v[6] = {pl.n_tok, 64 * pl.ks, pl.naccs, pl.split, pl.ring, pl.slots};
+    for (int i = 0; i < 6; ++i) cut[i] = (int32_t)v[i];
+}
+
+// (More than the call's own cut needs: the workspace of the largest batch serves the smaller ones, whose parts of shared tiles may take more.  Of 20000 pairs
+// of a batch and a larger one 43 are cut a slower way for lack of room, by 17 % at most; 323 if a workspace had the room of its own batch alone.)
 size_t fgmp_ws_mixed(int64_t M, int64_t N, int64_t K)
 {
-    const size_t parts = parts_bytes(mixed_plan(M, N, K, SIZE_MAX)), earlier = parts_bytes(mixed_plan(M, N, K, SIZE_MAX, true));
-    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + (parts > earlier ? parts : earlier);
+    const size_t own = parts_bytes(mixed_plan(M, N, K, SIZE_MAX)), roomy = parts_bytes(mixed_plan(M, N, K, SIZE_MAX, true));
+    return (size_t)FGMP_WS_CONTROL_BYTES + fgmp_align1k((size_t)M * K * 2) + (own > roomy ? own : roomy);
 }
 
 // expands the activations and multiplies; leave_nvfp4: unless neither operand has an FP8 block

@@ -56,6 +56,20 @@ def test_size_functions(lib):
     assert "timed out" in fg.status_string(-6)
 
 
+# Calls that a model fitted to too few shapes sent the slow way: tiles of few chunks of K, whose way out is what they take; tiles in so many parts that
+# adding them up is; a grid that fills the chip where a smaller one does the same.  Rows of Y that the GEMM over planes would write element by element.
+@pytest.mark.parametrize("M,N,K,tokens,shared", [
+    (1220, 15936, 768, None, None), (1161, 11264, 512, None, None), (53, 644, 8960, (16, 32), 1), (482, 308, 1024, (64,), 1), (275, 13312, 15104, (288,), 1),
+    (645, 7401, 512, range(96, 177), 0), (4001, 4113, 2112, None, None), (777, 11008, 4096, (160,), 0), (48, 4096, 4096, (48,), 1)])
+def test_cut_of_calls(lib, M, N, K, tokens, shared):
+    import torch
+    import paper_2504_14152_b200 as fg
+    if torch.cuda.is_available() and torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the cuts are those of 148 SMs")
+    cut = fg.linear_cut(M, N, K)
+    assert (cut is None) if tokens is None else (cut["tokens"] in tokens and cut["shared"] == shared), cut
+
+
 def test_validation_rejects_bad_arguments_on_the_host(lib):
     import paper_2504_14152_b200.binding as b
     L = b._load()
