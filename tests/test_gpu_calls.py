@@ -77,9 +77,9 @@ def test_linear_right_behind_the_quantizing_one(fg, N, K):
 
 # A CTA has more units than the decode kernel has stages (four to six), whose number is odd for some batches:
 # the same sums either way, over and over, with the weights' copies out of L2 and out of HBM.
-@pytest.mark.parametrize("M", [1, 3, 4, 5, 8, 9, 13, 14, 16])
+@pytest.mark.parametrize("M", [1, 2, 3, 4, 5, 8, 9, 13, 14, 16])
 def test_decode_of_packed_tokens_equals_the_fused_step(fg, M):
-    N, K = 8192, 4096
+    N, K = (8192, 4096) if M > 2 else (16384, 4096)       # (one and two tokens: more than twice as many units as stages)
     g = torch.Generator(device="cuda").manual_seed(M)
     x, f = torch.randn(M, K, generator=g, device="cuda").to(torch.bfloat16), torch.rand(K, generator=g, device="cuda") + 0.5
     s4 = float(x.abs().max()) / 2688.0
@@ -94,11 +94,15 @@ def test_decode_of_packed_tokens_equals_the_fused_step(fg, M):
                 assert torch.equal(fg.linear(acts, w), y)
 
 
-# Token tiles of 224 to 384: fewer stages for the tokens than slots for the weights.  Against the GEMM over expanded planes; both sum
-# exact products in fp32 (K = 4096 terms in another order: about 1e-7 of the norm, a stale or early tile is of the order of one).
-@pytest.mark.parametrize("M", [224, 256, 277, 310, 340, 384])
-def test_gemm_on_packed_weights_with_few_token_stages(fg, M):
-    N, K = 11008, 4096
+# Token tiles of 176 to 416: as few stages for the tokens as there are slots for the weights, three to five, each passed through many times.  Against
+# the GEMM over expanded planes; both sum exact products in fp32 (K terms in another order: about 1e-7 of the norm, a stale or early tile is of the order of one).
+@pytest.mark.parametrize("M,N,K,tokens,shared", [
+    (340, 11008, 4096, 176, 1), (208, 18944, 4096, 208, 0), (224, 11008, 4096, 224, 1), (256, 11008, 4096, 256, 1), (672, 7232, 11008, 224, 1), (560, 9819, 3392, 288, 1),
+    (672, 7680, 2752, 336, 1), (1149, 5679, 3840, 384, 0), (830, 6656, 3648, 416, 1)])
+def test_gemm_on_packed_weights_with_few_token_stages(fg, M, N, K, tokens, shared):
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        cut = fg.linear_cut(M, N, K)
+        assert (cut["tokens"], cut["shared"]) == (tokens, shared) and cut["stages"] == cut["slots"] <= 5, cut
     w, acts = draw_weights(fg, N, K, 30), draw_acts(fg, M, K, 31)
     y0, ref = fg.linear(acts, w), fg.linear_classes(acts, w)
     d = (y0 - ref).double()

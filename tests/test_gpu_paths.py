@@ -19,6 +19,14 @@ def launches(fg, call):
     return {name: n for name, (n, _) in fg.profile_end().items()}
 
 
+def cut_of(fg, M, N, K):
+    """(tokens of a tile, whether tiles are shared, accumulators, elements of K per step) of a call on the packed weights"""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the cuts are those of 148 SMs")
+    c = fg.linear_cut(M, N, K)
+    return c and (c["tokens"], c["shared"], c["accumulators"], c["step"])
+
+
 def check_linear(fg, qa, qw, pa, pw, rel=1e-5):
     """fp32 and bf16 output, the latter with a row pitch that rules wide stores out, against the oracle."""
     Y, S = oracle.linear(qa, qw)
@@ -63,10 +71,12 @@ def test_quantizer_behind_split_tiles(fg, M, N, K, mode):
     compare_packed(fg, fg.linear_quantize(pa, pw, f.cuda(), scale_fp4=s4, score_mode=mode, tau=tau), q, tau, "hidden")
 
 
-# a tile of more than 256 tokens (two products on one dequantized operand), the last row of its second half, a ragged weight tile
-@pytest.mark.parametrize("M,N", [(289, 8200), (416, 8256)])
-def test_gemm_on_packed_weights_wide_tiles(fg, M, N):
-    qa, qw, pa, pw = quantize_both(fg, gi.llama("wd", M, N, 5184, seed=68), 0.1, 0.1, clip=False)
+# a tile of more than 256 tokens (two products on one dequantized operand), the last row of its second half, a ragged weight tile; whole tiles and parts,
+# Y and the quantizer
+@pytest.mark.parametrize("M,N,K,tokens,shared", [(830, 5661, 512, 288, 0), (410, 14784, 576, 416, 0), (700, 8007, 2304, 352, 1), (830, 7232, 2816, 416, 1)])
+def test_gemm_on_packed_weights_wide_tiles(fg, M, N, K, tokens, shared):
+    assert cut_of(fg, M, N, K) == (tokens, shared, 1, 64)
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("wd", M, N, K, seed=68), 0.1, 0.1, clip=False)
     y16 = fg.linear(pa, pw, out_dtype=torch.bfloat16)
     count = launches(fg, lambda: fg.linear(pa, pw))
     assert count.get("gemm_mixed_tcgen05") == 1 and "gemm_f16_tcgen05" not in count, count
@@ -178,16 +188,24 @@ def test_output_tiles(fg, M, N, K, dtype, quantum):
         assert bool((y[M:] == -7.0).all()) and bool((y[:, N:] == -7.0).all()), "stored outside the output"
 
 
-# the GEMM on packed weights where its steps, its accumulators and its two products to a step change: an odd number of 64-element steps in the last
-# chunk, one and two accumulators, tiles of 160, 176, 208, 240, 272 and 416 tokens
-@pytest.mark.parametrize("M", [160, 176, 208, 240, 272, 416])
-@pytest.mark.parametrize("K,frac_w", [(64, 0.1), (448, 0.4), (832, 0.1)])
-def test_gemm_on_packed_weights_tile_sizes(fg, M, K, frac_w):
-    N = 200
+# the GEMM on packed weights where its steps and its accumulators change, whole tiles and parts; an odd number of 64-element steps in the last chunk, which
+# is then half of a step or a step of its own, and an even one
+@pytest.mark.parametrize("M,N,K,frac_w,cut", [
+    (150, 9536, 64, 0.1, (160, 0, 2, 128)), (155, 704, 2624, 0.4, (160, 1, 2, 128)), (100, 257, 1088, 0.1, (16, 1, 2, 128)), (176, 9600, 64, 0.1, (176, 0, 1, 128)), (175, 704, 2880, 0.4, (176, 1, 1, 128)),
+    (520, 192, 3456, 0.1, (176, 1, 1, 128)), (207, 9666, 64, 0.4, (208, 0, 1, 128)), (208, 774, 2368, 0.1, (208, 1, 1, 128)), (224, 9983, 64, 0.4, (224, 0, 1, 64)),
+    (447, 576, 2432, 0.1, (224, 1, 1, 64)), (479, 640, 2560, 0.1, (240, 1, 1, 64)), (255, 9580, 256, 0.1, (256, 0, 1, 64)), (256, 806, 2624, 0.4, (256, 1, 1, 64)),
+    (270, 12608, 64, 0.1, (272, 0, 1, 64))])
+def test_gemm_on_packed_weights_tile_sizes(fg, M, N, K, frac_w, cut):
+    assert cut_of(fg, M, N, K) == cut
     qa, qw, pa, pw = quantize_both(fg, gi.llama("ts", M, N, K, seed=73), 0.1, frac_w, clip=False)
     count = launches(fg, lambda: fg.linear(pa, pw))
-    assert count.get("gemm_mixed_tcgen05") == 1, count
+    assert count.get("gemm_mixed_tcgen05") == 1 and ("gemm_reduce" in count) == bool(cut[1]), count
     check_linear(fg, qa, qw, pa, pw)
+    if N % 64 == 0:
+        f, kw = torch.rand(N, generator=torch.Generator().manual_seed(1)).cuda() + 0.5, dict(scale_fp4=1e-2, tau=1e-4)
+        want = fg.quantize_activations(fg.linear(pa, pw, out_dtype=torch.bfloat16), f, **kw)
+        for a, b in zip(fg.unpack(fg.linear_quantize(pa, pw, f, **kw)), fg.unpack(want)):
+            assert torch.equal(a, b)
 
 
 # one and two tokens, whose quantizer runs in every CTA unless the packed form is asked for: no FP8 blocks, some and only such, one unit per CTA and many
@@ -207,8 +225,9 @@ def test_quantizer_in_every_cta(fg, M, N, K, frac_w, mode):
     ys, _ = fg.linear_fused(x.cuda(), fx.cuda(), pw, want_packed=True, workspace=ws, **args)
     fg.check(ws)
     Y, S = oracle.linear(qa, qw)
-    for got in (y, ys, fg.linear_fused(x.cuda(), fx.cuda(), pw, workspace=ws, **args)):
-        assert (np.abs(got.cpu().numpy().astype(np.float64) - Y) <= 1e-5 * S + 1e-30).all()
+    assert (np.abs(y.cpu().numpy().astype(np.float64) - Y) <= 1e-5 * S + 1e-30).all()
+    for got in (ys, fg.linear_fused(x.cuda(), fx.cuda(), pw, workspace=ws, **args), fg.linear(fg.quantize_activations(x.cuda(), fx.cuda(), **args), pw)):
+        assert torch.equal(got.view(torch.int32), y.view(torch.int32)), "bit for bit, whoever quantizes"
     wide = torch.randn(M, K + 8, generator=torch.Generator().manual_seed(1)).to(torch.bfloat16).cuda()
     wide[:, :K] = x.cuda()
     assert torch.equal(fg.linear_fused(wide[:, :K], fx.cuda(), pw, **args), y), "rows further apart"
