@@ -31,10 +31,10 @@
 //                the workspace and stream them from there; the first weight copies are in flight meanwhile.
 //   DEC_OWN1_LP ... DEC_OWN2_HP  fused calls of one or two tokens whose packed form nobody asks for: warps of each CTA quantize what its units
 //                need, unit by unit, straight into the stages.  That is more work in all, and nothing to hand over: 2.7 us lie between the end of the
-//                kernel before and the last shared record, 0.7 more until its copy is in.  11008 x 4096: 1 token 14.4 -> 11.0 us, 2 tokens
-//                16.9 -> 12.2; 28672 x 8192: 33.5 -> 30.0 and 38.7 -> 32.9.  (With 64 threads a token for every unit in turn instead of two units at a
-//                time, two tokens take 14.5 and 48.6: beyond a dozen units that is slower than the shared quantizer.)  Where a CTA has very many units
-//                the warps that quantize for each of them cost more than the hand-over: see the launch.
+//                kernel before and the last shared record, 0.7 more until its copy is in.  In a graph of such calls, 10 % FP8 blocks, shared and own:
+//                11008 x 4096 one token 14.1 and 10.3 us, two 14.1 and 10.8; 28672 x 8192 31.8 and 28.8, 31.7 and 30.4.  (With 64 threads a token
+//                for every unit in turn instead of two units at a time, two tokens took 14.5 and 48.6.)  Where a CTA has very many units the warps that
+//                quantize for each of them cost more than the hand-over: see the launch.
 //   DEC_UNPACK   fgmp_linear: made unit by unit in shared memory from the packed activations' records.
 //
 // Warp roles: warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, from warp 2 on two or three sets of four warps that take
@@ -68,9 +68,9 @@ constexpr uint32_t STG_STEP = STG_LIST + LIST_CAP;                           // 
 constexpr uint32_t AREC_GAP = AREC_AT - AREC_HOT;
 __host__ __device__ inline uint32_t arec_gap(int64_t M) { return M >= 14 ? AREC_GAP : 0u; }
 constexpr int DEC_MAX_STAGES = 6;
-// Two sets; three for one and two tokens without the packed form (their accumulators leave the tensor memory for it): 11.2 us instead of 11.3 at one
-// token of 11008 x 4096, 28.8 and 28.7 of 28672 x 8192; with 20 % FP8 blocks, whose second halves come from global memory, 37 instead of 47.  For more
-// tokens it is no gain: eight of 28672 x 8192 39.4 instead of 36.1.
+// Two sets; three for one and two tokens without the packed form (their accumulators leave the tensor memory for it): 10.35 us instead of 10.47 at one
+// token of 11008 x 4096, 28.8 and 28.7 of 28672 x 8192; with 20 % FP8 blocks, whose second halves come from global memory, 12.3 instead of 13.9 and 36.8
+// instead of 46.7.  For more tokens it is no gain: eight of 28672 x 8192 39.4 instead of 36.1.
 // Tensor memory columns: accumulators (two buffers of each kind); of each set: a dense E4M3 tile of 64, scales (32)
 template <int SETS> struct Dec {
     static constexpr int W_EPI = W_SET + 4 * SETS, W_STEP = W_EPI + 4;

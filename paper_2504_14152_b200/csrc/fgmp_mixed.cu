@@ -8,24 +8,24 @@
 // its 128-row operand from.  What bounds what:
 //   - expanding the weights to a plane first costs 2.7 bytes written and read for every packed byte, which is the whole
 //     call at small batches (4096 x 4096, 48 tokens: 59 us with the plane);
-//   - a 128 x 256 unit of weights takes 1024 clocks of the SIMT pipes at least (256 conversions and 128 multiplies per scheduler, two clocks each),
-//     its MMAs 16 of N/2 clocks for N tokens;
+//   - a 128 x 256 unit of weights takes 256 conversions (half of them of FP8 blocks, under a predicate) and 128 multiplies a scheduler, its MMAs 16 of
+//     N/2 clocks for N tokens;
 //   - the operand from tensor memory leaves shared memory to the token tiles (from shared memory the 64 KiB of a
 //     dequantized unit would be written and read there, 1024 clocks by themselves);
-//   - the issuer and the dequantizing warps share their schedulers, so that a unit costs what its instructions cost to issue: 1380 per scheduler
-//     before, 1200 now.  Hence steps of 128 elements (half as many waits and commits), one wait and one commit for a step's weights and tokens
-//     together, the FP8 blocks' conversions and loads under one predicate with the microscale or the FP8 factor chosen per block, and groups that
-//     pass over units none of whose steps is theirs.  64 x 28672 x 8192 a call: 91 -> 65 us (1.05 us a unit);
+//   - the issuer and the dequantizing warps share their schedulers, so that a unit costs what its instructions cost to issue: 1290 a scheduler at 203
+//     tokens and 1360 at 160, the results' way out included.  Hence steps of 128 elements (half as many waits and commits), one wait and one commit for
+//     a step's weights and tokens together, the FP8 blocks' conversions and loads under one predicate with the microscale or the FP8 factor chosen per
+//     block, and groups that pass over units none of whose steps is theirs.  64 x 28672 x 8192 a call: 91 -> 65 us;
 //   - beyond 160 tokens the token tiles: 12 TB/s come out of L2 then, 45 bytes a clock and SM (64 would be needed at full MMA rate), and a second
-//     accumulator no longer fits beside the slots.  So 160 tokens are the most for the time a unit takes (777 x 11008 x 4096: five tiles of 160 as
-//     whole tiles 60 us, four of 208 in spans 77).
+//     accumulator no longer fits beside the slots.  Up to there a wider tile costs a unit little (777 x 11008 x 4096: five whole tiles of 160 60 us, four
+//     of 208 in spans 77); what is best for a call is in mixed_us.
 // Four groups, CTA pairs that share a token tile, spinning instead of suspended waits and a loop of one elected thread in the issuer were measured
 // and are no faster.
 //
 // Work is (weight tile, token tile, 256-element K chunk) units in that order, split over the CTAs either in
 // equal contiguous spans (stream-K: the partial sums of tiles shared by several CTAs are stored, eight columns of a row at a time, and added
 // up in CTA order by a kernel of their own, which has the whole chip's loads in flight: 43 MB at 203 tokens and 13824 weight
-// rows, 20 us if the CTA that arrives last does it) or in whole tiles, whichever the model in mixed_plan says is faster.
+// rows, 20 us if the CTA that arrives last does it) or in whole tiles, whichever the model in mixed_us says is faster.
 //
 // Warp roles: warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, warp 2 = token-tile producer,
 // warps 3-6 = epilogue, then the dequantization, NG groups of four warps that take the steps in turn.  Every
