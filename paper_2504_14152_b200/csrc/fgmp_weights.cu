@@ -9,7 +9,7 @@ namespace {
 
 constexpr int SEL_BINS = 2048;           // bins of a digit of the radix select
 
-// The calls here are chains of small kernels.  Each (but see launch_score) is launched as a programmatic dependent of the one before it: its blocks come up while
+// The calls here are chains of small kernels.  Each is launched as a programmatic dependent of the one before it: its blocks come up while
 // that one runs and wait for its end (every block does, so that a kernel's end implies those of all before it).  The last kernel of a packing lets
 // nothing start early, since the GEMMs read packed weights before they wait.  (4096 x 4096 weights and a calibration batch of 512 tokens,
 // eighteen launches: 20 us of 311.)
@@ -107,166 +107,229 @@ __global__ void __launch_bounds__(256) w_amax_kernel(const uint4* W, int64_t ldw
         st->s4 = __fdiv_rn(__uint_as_float(*reinterpret_cast<volatile uint32_t*>(&st->amax_bits)), 2688.0f);
 }
 
-__device__ __forceinline__ void load_block(const uint4* W, int64_t ldw8, const float* F, int64_t ldf,
-                                           int64_t n, int64_t kb, float (&v)[16], float (&f)[16])
+__device__ __forceinline__ void load_block(const uint4* wp, const float* fp, float (&v)[16], float (&f)[16])
 {
-    const uint4* wp = W + n * ldw8 + kb * 2;
     unpack_bf16x16(__ldg(wp), __ldg(wp + 1), v);
-    if (F) {
-        const float4* fp = reinterpret_cast<const float4*>(F + n * ldf + kb * 16);
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float4 t = __ldg(fp + i);
-            f[4 * i] = t.x; f[4 * i + 1] = t.y; f[4 * i + 2] = t.z; f[4 * i + 3] = t.w;
-        }
+    for (int i = 0; i < 4; ++i) {
+        const float4 t = __ldg(reinterpret_cast<const float4*>(fp) + i);
+        f[4 * i] = t.x; f[4 * i + 1] = t.y; f[4 * i + 2] = t.z; f[4 * i + 3] = t.w;
     }
 }
 
 // A tensor of zeros has the tensor scale zero: all its codes are zero then, instead of what 0 times infinity rounds to.
 __device__ __forceinline__ float inverse_scale(float s) { return s == 0.f ? 0.f : __fdiv_rn(1.0f, s); }
 
-// two values rounded to E2M1 and back
+// two values rounded to E2M1 and back  (subtracted from as fp16 numbers, which takes the FMA pipe half as long as converting them)
 __device__ __forceinline__ float2 round_e2m1x2(float lo, float hi)
 {
-    uint32_t h2;
-    asm("{\n\t.reg .b8 t;\n\tcvt.rn.satfinite.e2m1x2.f32 t, %1, %2;\n\tcvt.rn.f16x2.e2m1x2 %0, t;\n\t}" : "=r"(h2) : "f"(hi), "f"(lo));
-    return __half22float2(*reinterpret_cast<__half2*>(&h2));
+    float2 q;
+    asm("{\n\t.reg .b8 t;\n\t.reg .b32 h;\n\t.reg .f16 x, y;\n\tcvt.rn.satfinite.e2m1x2.f32 t, %3, %2;\n\tcvt.rn.f16x2.e2m1x2 h, t;\n\tmov.b32 {x, y}, h;\n\t"
+        "sub.rn.f32.f16 %0, x, %4;\n\tsub.rn.f32.f16 %1, y, %4;\n\t}" : "=f"(q.x), "=f"(q.y) : "f"(lo), "f"(hi), "f"(0.f));
+    return q;
 }
 
-// Weighted squared error of a block under microscale d (inv = 1/d), the terms added in element order.  BOUND: clipped = the
-// largest term of an element whose magnitude is not below 6 d, i.e. that is clipped: it only grows with a smaller scale.
-template <bool BOUND>
-__device__ __forceinline__ float clip_error(const float (&v)[16], const float (&f)[16], float2 dd, float& clipped)
+// Weighted squared error of a block under microscale dd.x (dd.y = 1 / dd.x), the terms added in element order
+__device__ __forceinline__ float clip_error(const float (&v)[16], const float (&f)[16], float2 dd)
 {
-    const float d = dd.x, inv = dd.y, d6 = __fmul_rn(6.0f, d);
-    const uint64_t d2 = f32x2_pack(d, d), inv2 = f32x2_pack(inv, inv);
-    float j = 0.f, top = 0.f;
+    const uint64_t d2 = f32x2_pack(dd.x, dd.x), inv2 = f32x2_pack(dd.y, dd.y);
+    float j = 0.f;
 #pragma unroll
     for (int i = 0; i < 16; i += 2) {
         const float2 y = f32x2_unpack(f32x2_mul(f32x2_pack(v[i], v[i + 1]), inv2)), q = round_e2m1x2(y.x, y.y);
         const uint64_t e = f32x2_sub(f32x2_mul(f32x2_pack(q.x, q.y), d2), f32x2_pack(v[i], v[i + 1]));
         const float2 t = f32x2_unpack(f32x2_mul(f32x2_mul(f32x2_pack(f[i], f[i + 1]), e), e));
         j = __fadd_rn(__fadd_rn(j, t.x), t.y);
-        if (BOUND) {
-            top = fmaxf(top, fabsf(v[i]) >= d6 ? t.x : 0.f);
-            top = fmaxf(top, fabsf(v[i + 1]) >= d6 ? t.y : 0.f);
-        }
     }
-    if (BOUND) clipped = top;
     return j;
 }
 
-__device__ __forceinline__ uint32_t dynamic_scale_of(const uint4* W, int64_t ldw8, int64_t n, int64_t kb, float k6)
-{
-    float v[16];
-    const uint4* wp = W + n * ldw8 + kb * 2;
-    unpack_bf16x16(__ldg(wp), __ldg(wp + 1), v);
-    return block_dynamic_scale(v, k6);
-}
+// The clip search (Eq. 11) asks for the scale with the least error among all 126, ties to the dynamic-max scale and then to the smaller code.  It
+// need not look at all of them:
+//   - Twice a scale is never better as long as nothing is clipped: what of its grid {0, 1, 2, 3, 4, 6, 8, 12} x d a value within 6 d can be rounded to is
+//     part of {0, 0.5, 1, 1.5, 2, 3, 4, 6} x d.  In fp32 an element is either rounded to the same number under both, or to 0.5 d or 1.5 d under d, at
+//     most a quarter of d away but for a few 2^-24, and at least that far under 2 d.  So the eight codes above the dynamic-max one (eight codes are an
+//     octave) stand for all larger ones, unless one of them is within CLIP_NEAR of the least error.
+//   - Below the dynamic-max code the largest elements are clipped.  A sum of non-negative terms is never below one of them, so a code can be left out under
+//     which (|v| - 6 d)^2 f of one element alone exceeds an error found so far: that gives the smallest code to look at directly.
+// A warp has a block per lane: nine codes for each, then what is left of all its blocks (2.4 codes a block on average, 7 for the longest: N(0, 1) weights
+// with log-normal sensitivities) is shared out over the lanes.  Blocks that the above does not hold for (sensitivities that are negative or not
+// finite, tensor scales near the ends of fp32, blocks 20000 times smaller than the largest) are searched code by code.
+constexpr float CLIP_NEAR = 1.f - 1.f / 4096, CLIP_TINY = 1.17549435e-38f;      // rounding: below 2^-17 an octave, of which there are 15, and 2^-130 where terms underflow
+constexpr int CLIP_LEAST_CODE = 7;                                               // codes from the next one on are an octave above the one eight below them
 
-// 256 threads sort what they are given (0..127): index() returns which thread's value is the calling one's in that order
-struct ClipOrder {
-    uint32_t bins[128];
-    uint8_t order[256];
-    __device__ __forceinline__ int index(uint32_t key)
-    {
-        const int t = threadIdx.x;
-        __syncthreads();
-        if (t < 128) bins[t] = 0;
-        __syncthreads();
-        const uint32_t rank = atomicAdd(&bins[key], 1u);
-        __syncthreads();
-        if (t < 32) {
-            uint32_t n[4], sum = 0;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { n[i] = bins[4 * t + i]; sum += n[i]; }
-            uint32_t at = sum;
-            for (int o = 1; o < 32; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, at, o); if (t >= o) at += y; }
-            at -= sum;
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { bins[4 * t + i] = at; at += n[i]; }
-        }
-        __syncthreads();
-        order[bins[key] + rank] = (uint8_t)t;
-        __syncthreads();
-        return order[t];
-    }
+struct ClipBest {
+    float j; uint32_t code;
+    // whether code c with error x comes before it
+    __device__ __forceinline__ bool beaten_by(float x, uint32_t c, uint32_t dyn) const { return x < j || (x == j && code != dyn && c < code); }
 };
 
-// Per block: microscale (dynamic max or Eq. 11 search) and the score under it.
-//
-// The search asks for the scale with the least error among all 126, ties to the dynamic-max scale and then to the smaller
-// code.  It need not look at all of them: going down from the dynamic-max code, an element that is clipped has an error that
-// only grows (every rounding step is monotone), and a sum of non-negative terms is never below one of them, so once such a
-// term alone exceeds the least error found no smaller scale can win.  (Where a sensitivity is negative or NaN the terms are not what
-// this rests on, and all scales are looked at.)  Going up there are few codes left, because the tensor
-// scale puts the largest block at code 126.  Of 126 evaluations per block 15 are left, 26 for the longest of a warp, and 20 if the warps of a thread
-// block share its 256 blocks out in the order of their dynamic-max codes, that is of how many there are above: 4096 x 4096 takes 145 us,
-// 152 in the order of the tensor, 172 without packed fp32 instructions, 680 with all 126.
+// code by code from `from` on, without the dynamic-max one
+__device__ __forceinline__ ClipBest clip_scan(const uint4* wp, const float* fp, const float2* s_d, uint32_t dyn, ClipBest best, uint32_t from)
+{
+    asm volatile("" : "+l"(wp), "+l"(fp));                    // (loaded again: the block's registers are others' by now)
+    float v[16], f[16];
+    load_block(wp, fp, v, f);
+#pragma unroll 1
+    for (uint32_t c = from; c <= 126u; ++c) {
+        if (c == dyn) continue;
+        const float x = clip_error(v, f, s_d[c]);
+        if (best.beaten_by(x, c, dyn)) { best.j = x; best.code = c; }
+    }
+    return best;
+}
+
+// The scale code of a lane's block (wp, fp: its values and sensitivities; dyn: its dynamic-max code).  All lanes of a warp call it; `active` ones have a
+// block.  sane: the tensor scale is far from the ends of fp32.  key: 32 words of shared memory of the warp's own.
+__device__ __forceinline__ ClipBest clip_search(const uint4* wp, const float* fp, const float (&v)[16], const float (&f)[16], uint32_t dyn, bool active,
+                                                bool sane, float k6, const float2* s_d, unsigned long long* key)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    ClipBest best{clip_error(v, f, s_d[dyn]), dyn};
+    float least_f = f[0];
+#pragma unroll
+    for (int i = 1; i < 16; i += 2) asm("min.NaN.f32 %0, %0, %1, %2;" : "+f"(least_f) : "f"(f[i]), "f"(f[i < 15 ? i + 1 : i]));
+    const bool ordered = least_f >= 0.f;
+    const float j_dyn = best.j;
+    const bool done = !active || dyn == 127u || (ordered && j_dyn == 0.f);             // (nothing beats no error, and no scale is better than NaN)
+    const bool simple = ordered && sane && dyn >= (uint32_t)CLIP_LEAST_CODE && j_dyn < 1e36f;      // (not where the error is NaN)
+    // the eight codes above
+    float first = __int_as_float(0x7f800000), second = first, third = first;          // the least errors
+    uint32_t at = 0, at2 = 0;
+#pragma unroll 1
+    for (uint32_t k = 1; k <= 8; ++k) {
+        const uint32_t c = dyn + k;
+        if (__all_sync(0xffffffffu, c > 126u)) break;
+        const float x = c <= 126u ? clip_error(v, f, s_d[min(c, 126u)]) : __int_as_float(0x7f800000);
+        third = fminf(third, fmaxf(x, second));
+        if (x < second) { second = x; at2 = c; }
+        if (second < first) { const float y = first; first = second; second = y; const uint32_t z = at; at = at2; at2 = z; }
+    }
+    if (first < best.j) { best.j = first; best.code = at; }
+    const float near = best.j + CLIP_TINY;
+    // what is left: codes below, and those an octave above the best
+    bool scan = false;
+    uint32_t down = 0, octaves = 0, octave = 0, octave2 = 0;
+    if (simple && !done) {
+        float root;
+        asm("sqrt.approx.f32 %0, %1;" : "=f"(root) : "f"(near));
+        root *= 1.f + 1.f / 4096;
+        float lift = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) lift = fmaxf(lift, fabsf(v[i]) * (1.f - 1.f / 65536) - root * rsqrtf(f[i]));
+        // the smallest code with 6 d >= lift
+        uint32_t least = max(f32x2_to_e4m3x2(__fmul_rn(lift, k6), 0.f) & 0x7fu, 1u);
+        if (6.f * s_d[least].x < lift) ++least;
+        down = least < dyn ? dyn - least : 0u;
+        if (best.j > 0.f) {
+            scan = third * CLIP_NEAR <= near;
+            const bool one = first * CLIP_NEAR <= near && at + 8u <= 126u, two = second * CLIP_NEAR <= near && at2 + 8u <= 126u;
+            octaves = (one ? 1u : 0u) + (two ? 1u : 0u);
+            octave = one ? at + 8u : at2 + 8u; octave2 = at2 + 8u;
+        }
+    }
+    const uint32_t mine = down + octaves, what = dyn | (down << 8) | (octave << 16) | (octave2 << 24);
+    uint32_t incl = mine;
+#pragma unroll
+    for (uint32_t o = 1; o < 32; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    key[lane] = ((unsigned long long)__float_as_uint(best.j) << 32) | (best.code == dyn ? 0u : best.code);
+    uint32_t again = 0;                                       // blocks whose best code's octave is no worse to speak of
+    __syncwarp();
+#pragma unroll 1
+    for (uint32_t t = lane; t - lane < total; t += 32) {
+        uint32_t o = 0;                                       // whose item it is
+#pragma unroll
+        for (uint32_t h = 16; h; h >>= 1) if (__shfl_sync(0xffffffffu, incl, o + h - 1u) <= t) o += h;
+        o = min(o, 31u);
+        const uint32_t w = __shfl_sync(0xffffffffu, what, o), i = t - __shfl_sync(0xffffffffu, incl - mine, o), d = w & 0xffu, n = (w >> 8) & 0xffu;
+        const float limit = __shfl_sync(0xffffffffu, best.j, o);
+        const uint4* wo = reinterpret_cast<const uint4*>(__shfl_sync(0xffffffffu, (unsigned long long)wp, o));
+        const float* fo = reinterpret_cast<const float*>(__shfl_sync(0xffffffffu, (unsigned long long)fp, o));
+        bool near_octave = false;
+        if (t < total) {
+            const uint32_t c = i < n ? d - 1u - i : i == n ? (w >> 16) & 0xffu : w >> 24;
+            float vo[16], fo16[16];
+            load_block(wo, fo, vo, fo16);
+            const float x = clip_error(vo, fo16, s_d[c]);
+            if (x <= limit) atomicMin(key + o, ((unsigned long long)__float_as_uint(x) << 32) | c);
+            near_octave = c > d && x * CLIP_NEAR <= limit + CLIP_TINY;
+        }
+        again |= __reduce_or_sync(0xffffffffu, near_octave ? 1u << o : 0u);
+    }
+    __syncwarp();
+    uint32_t from = 1;
+    if (simple) {
+        const unsigned long long k = key[lane];
+        best.j = __uint_as_float((uint32_t)(k >> 32));
+        best.code = (uint32_t)k ? (uint32_t)k : dyn;
+        from = scan || ((again >> lane) & 1u) ? dyn + 9u : 127u;
+    } else {
+        best.j = j_dyn; best.code = dyn;
+    }
+    if (!done && from < 127u) best = clip_scan(wp, fp, s_d, dyn, best, from);
+    __syncwarp();                                             // (the words are the next blocks')
+    return best;
+}
+
+// Per block: microscale (dynamic max or Eq. 11 search) and the score under it.  The search is bound by the FMA and ALU pipes (an evaluation
+// takes 121 clocks of a scheduler that has six warps, 142 with four; nine of them a block and three rounds of shared ones, and 40 % of the instructions are
+// for everything else): 4096 x 4096 weights 85 us, 88 with more registers and four warps a scheduler.  With every lane searching its own block, and one larger code after the other, it took 146 (223 where one weight lies far above the others, 374 where a
+// third of the blocks is zero; now 97 and 77).
+constexpr int SCORE_THREADS = 128, SCORE_BLOCKS = 7;
 template <int MODE, bool CLIP>
-__global__ void __launch_bounds__(256) w_score_kernel(const uint4* W, int64_t ldw8, const float* F, int64_t ldf,
-                                                      int64_t N, int64_t KB, int ratio, float s8_given, const SelectState* st,
-                                                      uint8_t* sc_out, float* scores)
+__global__ void __launch_bounds__(SCORE_THREADS, SCORE_BLOCKS) w_score_kernel(const uint4* W, int64_t ldw8, const float* F, int64_t ldf, uint32_t B, uint32_t KB,
+                                                                             int ratio, float s8_given, const SelectState* st, uint8_t* sc_out, float* scores)
 {
     // scale and its inverse, by code; 127, NaN, is what a block gets whose largest magnitude over a tensor scale of infinity or NaN has
     // no code (weights that are not finite): no scale is better than it
     __shared__ float2 s_d[128];
-    __shared__ ClipOrder clip_order;
+    __shared__ unsigned long long s_key[SCORE_THREADS];
     chain_begin();
     const float s4 = st->s4;
     if (CLIP) {
-        if (threadIdx.x < 128) {
-            const float d = __fmul_rn(e4m3_to_f32(threadIdx.x), s4);
-            s_d[threadIdx.x] = make_float2(d, (d == 0.f) ? 0.f : __fdiv_rn(1.0f, d));
-        }
+        static_assert(SCORE_THREADS == 128, "a code per thread");
+        const float d = __fmul_rn(e4m3_to_f32(threadIdx.x), s4);
+        s_d[threadIdx.x] = make_float2(d, (d == 0.f) ? 0.f : __fdiv_rn(1.0f, d));
         __syncthreads();
     }
     const float k6 = inverse_scale(__fmul_rn(6.0f, s4));
     const float s8 = s8_given > 0.f ? s8_given : __fmul_rn(s4, __int_as_float((127 + ratio) << 23));
     const float inv8 = inverse_scale(s8);
-    const int64_t B = N * KB;
-    for (int64_t base = (int64_t)blockIdx.x * 256; base < B; base += (int64_t)gridDim.x * 256) {
-        int64_t b = base + threadIdx.x;
-        if (CLIP) b = base + clip_order.index(b < B ? dynamic_scale_of(W, ldw8, b / KB, b % KB, k6) : 127u);
-        if (b >= B) continue;
-        float v[16], f[16];
-        load_block(W, ldw8, F, ldf, b / KB, b % KB, v, f);
-        uint32_t sc = block_dynamic_scale(v, k6);
-        if (CLIP) {
-            const int dyn = (int)sc;
-            bool ordered = true;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) ordered &= f[i] >= 0.f;
-            float clipped, best = clip_error<true>(v, f, s_d[dyn], clipped);
-            bool more = !(ordered && clipped > best);
-#pragma unroll 1
-            for (int c = dyn - 1; more && c >= 1; --c) {
-                const float j = clip_error<true>(v, f, s_d[c], clipped);
-                // going down, a tie is a smaller code: it wins unless the dynamic-max code holds the lead
-                if (j < best || (j == best && (int)sc != dyn)) { best = j; sc = (uint32_t)c; }
-                more = !(ordered && clipped > best);
-            }
-#pragma unroll 1
-            for (int c = dyn + 1; c <= 0x7e; ++c) {
-                const float j = clip_error<false>(v, f, s_d[c], clipped);
-                if (j < best) { best = j; sc = (uint32_t)c; }
-            }
+    const uint32_t b = blockIdx.x * (uint32_t)SCORE_THREADS + threadIdx.x;
+    if (!CLIP && b >= B) return;
+    const uint32_t at = min(b, B - 1u), n = at / KB, kb = at - n * KB;
+    const uint4* wp = W + (int64_t)n * ldw8 + kb * 2u;
+    const float* fp = F + (int64_t)n * ldf + kb * 16u;
+    float v[16], f[16];
+    load_block(wp, fp, v, f);
+    uint32_t sc = block_dynamic_scale(v, k6);
+    if (CLIP) {
+        const ClipBest best = clip_search(wp, fp, v, f, sc, b < B, s4 > 1e-18f && s4 < 16.f, k6, s_d, s_key + (threadIdx.x & ~31u));
+        if (b >= B) return;
+        sc = best.code;
+        if (MODE == 0) {                                     // the score is the error itself
+            sc_out[b] = (uint8_t)sc;
+            scores[b] = best.j;
+            return;
         }
-        uint32_t c4[2];
-        float dq4[16];
-        block_nvfp4(v, sc, s4, c4, dq4);
-        float score;
-        if (MODE == 0) {
-            score = weighted_sq_sum(v, dq4, f);
-        } else {
-            uint32_t c8[4];
-            float dq8[16];
-            block_fp8(v, inv8, s8, c8, dq8);
-            score = weighted_sq_sum(dq4, dq8, f);
-        }
-        sc_out[b] = (uint8_t)sc;
-        scores[b] = score;
+        asm volatile("" : "+l"(wp), "+l"(fp));               // (loaded again: the registers were others' meanwhile)
+        load_block(wp, fp, v, f);
     }
+    uint32_t c4[2];
+    float dq4[16];
+    block_nvfp4(v, sc, s4, c4, dq4);
+    float score;
+    if (MODE == 0) {
+        score = weighted_sq_sum(v, dq4, f);
+    } else {
+        uint32_t c8[4];
+        float dq8[16];
+        block_fp8(v, inv8, s8, c8, dq8);
+        score = weighted_sq_sum(dq4, dq8, f);
+    }
+    sc_out[b] = (uint8_t)sc;
+    scores[b] = score;
 }
 
 // ------------------------------------------------------------ radix select (k-th largest)
@@ -575,16 +638,11 @@ int grid_for(int64_t work_items, int threads, int max_ctas_per_sm)
     return (int)g;
 }
 
-// Microscales and scores of all blocks.  The clip search is no programmatic dependent where its loop goes round fewer than four times: its thread blocks would come
-// up where the kernel before it leaves room first, and the ones with a round more than the others, the first of the grid, side by side on a few SMs
-// (scores of 4160 x 1280, 2.2 rounds: 67 us, 56 when they start together; 3600 x 2048, 3.04: 74 and 72; 4096 x 4096, 6.9: 152 both ways, a packing 271
-// and 274).
+// microscales and scores of all blocks
 template <int MODE, bool CLIP, typename... A>
 void launch_score(int64_t B, cudaStream_t s, A... args)
 {
-    const int g = grid_for(B, 256, 4);
-    if (CLIP && B < (int64_t)g * 256 * 4) w_score_kernel<MODE, CLIP><<<g, 256, 0, s>>>(args...);
-    else chain_launch(w_score_kernel<MODE, CLIP>, g, 256, s, args...);
+    chain_launch(w_score_kernel<MODE, CLIP>, (B + SCORE_THREADS - 1) / SCORE_THREADS, SCORE_THREADS, s, args...);
 }
 template <typename... A>
 void run_scores(fgmp_score_mode sm, fgmp_clip_mode cm, int64_t B, cudaStream_t s, A... args)
@@ -681,7 +739,7 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
     FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, sc.scale_fp4, (unsigned long long)k, fraction_mode ? INFINITY : tau));
     if (sc.scale_fp4 == 0.f)
         FGMP_LAUNCH(FGMP_K_W_AMAX, s, chain_launch(w_amax_kernel, grid_for(N, 4, 8), 256, s, W, ldw / 8, N, (uint32_t)(K / 8), st));
-    run_scores(sm, cm, B, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, (const SelectState*)st, sc_tmp, scores);
+    run_scores(sm, cm, B, s, W, ldw / 8, fisher_elem, ldf, (uint32_t)B, (uint32_t)KB, ratio, s8_given, (const SelectState*)st, sc_tmp, scores);
     const int gw = grid_for(NW * 32, 256, 8);
     if (fraction_mode && k > 0) {
         run_select(scores, B, st, s);
@@ -746,7 +804,7 @@ extern "C" fgmp_status fgmp_weight_scores(const void* W_bf16, int64_t ldw, const
     FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, sc.scale_fp4, 0ull, 0.f));
     if (sc.scale_fp4 == 0.f)
         FGMP_LAUNCH(FGMP_K_W_AMAX, s, chain_launch(w_amax_kernel, grid_for(N, 4, 8), 256, s, W, ldw / 8, N, (uint32_t)(K / 8), st));
-    run_scores(sm, cm, B, s, W, ldw / 8, fisher_elem, ldf, N, KB, ratio, s8_given, (const SelectState*)st, sc_tmp, scores);
+    run_scores(sm, cm, B, s, W, ldw / 8, fisher_elem, ldf, (uint32_t)B, (uint32_t)KB, ratio, s8_given, (const SelectState*)st, sc_tmp, scores);
     return fgmp_launch_status();
 }
 

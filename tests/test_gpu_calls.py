@@ -236,6 +236,34 @@ def test_clip_search_with_any_sensitivity(fg):
     compare_packed(fg, fg.quantize_weights(w.cuda(), f.cuda(), clip_mode=1, fp8_fraction=0.0), q, None, "any sign")
 
 
+# The search for the clipping scale looks at few of the 126 codes, by bounds that hold for ordinary blocks; here are ordinary ones and those at the edges
+# of what the bounds rest on: blocks of zeros, with one element, of few values (ties between codes an octave apart), far smaller than the largest
+# (dynamic-max codes up to 7 and just above), sensitivities of zeros, of any size and near the end of fp32.  The scale: derived; the largest blocks clipped
+# at code 126 already; small codes for all blocks; and at either end of fp32.
+@pytest.mark.parametrize("scale", [0.0, 2e-5, 3e-3, 40.0, 1e-20])
+def test_clip_search_at_the_edges_of_its_bounds(fg, scale):
+    N, K = 170, 1088
+    g = torch.Generator().manual_seed(101)
+    w = torch.randn(N, K, generator=g) * 0.02
+    f = torch.exp(1.5 * torch.randn(N, K, generator=g))
+    one = torch.zeros(10, K // 16, 16).scatter_(2, torch.randint(16, (10, K // 16, 1), generator=g), torch.randn(10, K // 16, 1, generator=g))
+    w[:10] = one.reshape(10, K)
+    w[10:20] = 0.02 * torch.randint(-3, 4, (10, K), generator=g)
+    f[12:24] = 1.0
+    w[20:30] = 2.0 ** torch.randint(-9, -3, (10, K), generator=g)
+    w[30:40] *= 1e-5
+    w[40:50] *= torch.exp(-8 * torch.rand(10, K // 16, generator=g)).repeat_interleave(16, 1)
+    w[50:60] = 0.0
+    f[60:70] *= torch.rand(10, K, generator=g) > 0.7
+    f[70:80] = torch.exp(40 * torch.randn(10, K, generator=g)).clamp(max=1e37)
+    f[80:90] *= 1e-37
+    w[90:100] = w[90:100].sign() * 0.0125
+    w[100, 100] = 0.3
+    w = w.to(torch.bfloat16)
+    q = oracle.quantize_weights(gi.bf16_bits(w), f.numpy(), scale_fp4=scale, clip=True, fp8_fraction=0.1)
+    compare_packed(fg, fg.quantize_weights(w.cuda(), f.cuda(), scale_fp4=scale, clip_mode=1, fp8_fraction=0.1), q, None, f"scale {scale}")
+
+
 # A workspace sized for the largest batch serves the smaller ones, among them those whose own size would be larger (the parts of shared
 # tiles take most at middling batches); one byte less than two planes of fp16 is refused.
 @pytest.mark.parametrize("N,K,largest", [(2048, 2048, 1024), (4096, 4096, 817), (1024, 320, 1000)])
