@@ -24,7 +24,7 @@
 //
 // Work is split stream-K style over (128-row tile, 256-element K chunk) units so that all SMs stream the same number of
 // bytes.  Tiles shared by several CTAs are reduced in a fixed order by the CTA that arrives last: results are
-// reproducible bit for bit.
+// reproducible bit for bit.  (For the order of a CTA's units see UnitOrder.)
 //
 // Where the activation operand (a "step record" per chunk) comes from:
 //   DEC_FUSED_LP, DEC_FUSED_HP  fused calls (by block score): the CTAs share out the quantizer's work, write the records to
@@ -154,6 +154,20 @@ __device__ __forceinline__ uint32_t cta_of_unit(const DecParams& p, uint32_t u)
     const uint32_t longer = p.rest * (p.span + 1);
     return u < longer ? u / (p.span + 1) : p.rest + (u - longer) / p.span;
 }
+
+// The units of a CTA in the order in which it takes them: from `begin` on, but the last `front` of them, the part of a tile that the next CTA goes on
+// with, before all others where they are fewer than what the CTA has of the tile before.  Handing in a part's sums and adding them up takes 2.5 to 3.5 us
+// and one set of warps, so that behind a last part of one unit (0.5 us) the part before is still under way: such CTAs were the last to end, by 2 us.  (In a
+// graph, 16 tokens of 11008 x 4096 16.0 -> 14.4 us, one token 10.3 -> 9.8, 28672 x 8192 38.2 -> 37.8 and 28.8 -> 28.6.)
+struct UnitOrder {
+    uint32_t begin, end, front;
+    __device__ __forceinline__ UnitOrder(uint32_t b, uint32_t e, uint32_t C) : begin(b), end(e)
+    {
+        const uint32_t last = e % C, before = min(C, e - b - min(e - b, last));
+        front = last < before ? last : 0u;
+    }
+    __device__ __forceinline__ uint32_t unit(uint32_t i) const { return i < front ? end - front + i : begin + i - front; }
+};
 
 __device__ __forceinline__ void quant_bar() { asm volatile("bar.sync 1, %0;" ::"n"(Q_THREADS) : "memory"); }
 
@@ -365,6 +379,15 @@ __device__ __forceinline__ void quantize_item(const DecParams& p, uint32_t c, ui
     }
 }
 
+// A token's sum of a row from the accumulators: NVFP4 rows and digits (col 0 and 1 .. 6), and of the FP8 weight blocks, where there are any
+template <typename Col>
+__device__ __forceinline__ float token_sum(bool has_fp8, float rw, float ra, const Col& col, uint32_t high, uint32_t low)
+{
+    const auto c = [&](int k) { return __uint_as_float(col(k)); };
+    const float x = has_fp8 ? c(0) + (__uint_as_float(high) + __uint_as_float(low)) * rw : c(0);
+    return x + (((c(1) + c(2)) + c(3)) + ((c(4) + c(5)) + c(6))) * ra;
+}
+
 template <int SRC, int SETS>
 __global__ void __launch_bounds__(dec_threads(SRC, SETS), 1)
 decode_kernel(const __grid_constant__ DecParams p)
@@ -395,6 +418,7 @@ decode_kernel(const __grid_constant__ DecParams p)
     // this CTA's span of (tile, chunk) units
     const uint32_t G = gridDim.x, C = p.chunks;
     const uint32_t u_begin = span_begin(p, blockIdx.x), u_end = span_begin(p, blockIdx.x + 1), n_units = u_end - u_begin;
+    const UnitOrder order(u_begin, u_end, C);
     const uint8_t* lists = p.wblob + p.LW.off_ovf;
     const bool has_fp8 = __ldg(&reinterpret_cast<const fgmp_packed_header*>(p.wblob)->n_fp8) != 0;
     const uint32_t quads = (M + 3u) / 4u, n_items = quads * C;      // the quantizer's work items: (chunk, four tokens)
@@ -439,7 +463,8 @@ decode_kernel(const __grid_constant__ DecParams p)
             bulk_load(dst + AREC_HOT, src + AREC_AT, p.arec_bytes - AREC_HOT, wf0 + 8 * s);
         };
         const uint32_t* uptr = reinterpret_cast<const uint32_t*>(p.wblob + p.LW.off_uptr);
-        uint32_t pf_base = u_begin, pf = 0, stage = 0, phase = 1;
+        uint32_t pf_base = 0, pf = 0, stage = 0, phase = 1;
+        const uint32_t pf_begin = order.front && u_begin + lane <= u_end ? __ldg(uptr + u_begin + lane) : 0u;
         const uint32_t pre = min(S, n_units);
         for (uint32_t i = 0; i <= n_units; ++i) {
             if (i == pre || !ok) {
@@ -448,12 +473,13 @@ decode_kernel(const __grid_constant__ DecParams p)
                 if (!FUSED) {
                     const fgmp_packed_header* ha = reinterpret_cast<const fgmp_packed_header*>(p.ablob);
                     if (ok && !(ha->magic == FGMP_MAGIC && ha->version == FGMP_LAYOUT_VERSION && ha->rows == p.M && ha->K == p.K && ha->kind == 0u && ha->fp8_scale_free == 0)) { ok = 0; bad = 10; }
-                    if (ok && lane < pre) load_arec(lane, u_begin + lane);         // of the stages under way
+                    if (ok && lane < pre) load_arec(lane, order.unit(lane));       // of the stages under way
                 }
                 if (bad && lane == 0) { *abort_flag = 1; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, bad); }
             }
             if (!ok || i == n_units) break;
-            const uint32_t u = u_begin + i;
+            const uint32_t u = order.unit(i);
+            if (i == order.front && i) { pf_base = u; pf = pf_begin; }      // (asked for with the first: their way is as long as a unit takes)
             if (i == 0 || u + 1 - pf_base > 31) {      // next 32 list starts
                 pf_base = u;
                 pf = pf_base + lane <= u_end ? __ldg(uptr + pf_base + lane) : 0u;
@@ -514,7 +540,7 @@ decode_kernel(const __grid_constant__ DecParams p)
         // ------------------------------------------------------------ this CTA's own quantizer: 64 threads, four lanes per block, make what a step
         // record holds of one token; two units at a time.
         const uint32_t tq = threadIdx.x - 32u * W_STEP, part = tq >> 6, li = tq & 3u, j = (tq >> 2) & 15u, m = part % M;
-        uint32_t i = part / M, c = (u_begin + i) % C, stage = i, phase = 1;        // (fewer at a time than stages)
+        uint32_t i = part / M, c = order.unit(i) % C, stage = i, phase = 1;        // (fewer at a time than stages)
         const uint8_t* row = p.X + (size_t)m * p.ldx * 2 + 32u * j + 8u * li;
         const float* fish = p.fisher + 16u * j + 4u * li;
         uint2 x = make_uint2(0u, 0u);
@@ -523,6 +549,7 @@ decode_kernel(const __grid_constant__ DecParams p)
         for (; i < n_units; i += OWN_TURNS) {
             const BlockQuarter r = quantize_block_quarter<(SRC & 1)>(x, f, p.q);
             c += OWN_TURNS;
+            if (i < order.front && i + OWN_TURNS >= order.front) c = u_begin % C + i + OWN_TURNS - order.front;      // (behind the units taken first)
             while (c >= C) c -= C;
             if (i + OWN_TURNS < n_units) { x = __ldg(reinterpret_cast<const uint2*>(row + 512u * c)); f = __ldg(reinterpret_cast<const float4*>(fish + 256u * c)); }
             const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&r.h.x)), vb = __half22float2(*reinterpret_cast<const __half2*>(&r.h.y));
@@ -542,8 +569,9 @@ decode_kernel(const __grid_constant__ DecParams p)
             bool ok = wait_global_equals(p.cw + CW_QCOUNT, n_items, abort_flag, p.status, 8);
             asm volatile("fence.proxy.async;" ::: "memory");   // records were written with ordinary stores, the bulk copy reads them
             FGMP_STAMP_ANY(4);
-            uint32_t stage = 0, phase = 1, c = u_begin % C;
+            uint32_t stage = 0, phase = 1, c = order.unit(0) % C;
             for (uint32_t i = 0; i < n_units && ok; ++i) {
+                if (i == order.front) c = u_begin % C;
                 if (!(ok = mbar_wait(dn0 + 8 * stage, phase, abort_flag, p.status, 13))) break;
                 mbar_expect_tx(sf0 + 8 * stage, a_bytes);
                 bulk_load(smem_u32(smem + stage * p.stage_bytes) + STG_STEP, p.steps + (size_t)c * a_bytes, a_bytes, sf0 + 8 * stage);
@@ -559,7 +587,7 @@ decode_kernel(const __grid_constant__ DecParams p)
         const uint32_t idesc4 = IDESC_NVF4 | ((n4 >> 3) << 17), idesc8 = IDESC_E4M3_E5M2 | ((n8 >> 3) << 17);
         const uint32_t step_lo = (p.stage_bytes >> 4), b8_lo = (n4 * 128u + 2048u) >> 4, b8_half = n8 * 8u;
         const uint32_t w_first = (smem_u32(smem) >> 4) | SW128_LO;
-        uint32_t stage = 0, phase = 0, w4 = w_first, left = C - u_begin % C, accum = 0, acc = 0, acc_phase = 1, set = 0;
+        uint32_t stage = 0, phase = 0, w4 = w_first, left = order.front ? order.front : C - u_begin % C, accum = 0, acc = 0, acc_phase = 1, set = 0;
         for (uint32_t i = 0; i < n_units; ++i) {
             if (accum == 0) {                          // a tile begins
                 if (!mbar_wait_uniform(acce0 + 8 * acc, acc_phase, abort_flag, p.status, 2)) break;
@@ -589,7 +617,7 @@ decode_kernel(const __grid_constant__ DecParams p)
             if (--left == 0 || i + 1 == n_units) {     // the tile (or this CTA's part of it) ends
                 if (elect_one()) umma_commit(accf0 + 8 * acc);
                 __syncwarp();
-                left = C; accum = 0;
+                left = i + 1 == order.front ? C - u_begin % C : C; accum = 0;
                 acc ^= 1u;
                 if (acc == 0) acc_phase ^= 1u;
             }
@@ -711,129 +739,123 @@ decode_kernel(const __grid_constant__ DecParams p)
         // FP8 tensor scale / NVFP4 tensor scale of either operand
         const float rw = __int_as_float((127 + __ldg(&hw->fp8_log2_ratio)) << 23);
         const float ra = FUSED ? p.q.r8 : __int_as_float((127 + ha->fp8_log2_ratio) << 23);
-        const uint32_t row = 32 * q + lane;
-        uint32_t accb = 0, acc_phase = 0, tile = u_begin / C;
-        for (uint32_t u = u_begin; u < u_end; ++tile) {
-            const uint32_t t_begin = tile * C, t_end = t_begin + C;
+        const uint32_t row = 32 * q + lane, octets = OWN ? 1u : (M + 7u) / 8u;
+        // eight tokens' sums of the row, from token 8 o on, to Y
+        const auto emit = [&](const float (&v)[8], uint32_t o, int64_t n) {
+            if (n >= p.N) return;
+            const int64_t at = (int64_t)(8u * o) * p.ldy + n;
+            __nv_bfloat16* yb = reinterpret_cast<__nv_bfloat16*>(p.Ybf) + at;
+            float* yf = p.Y + at;
+#pragma unroll
+            for (uint32_t j = 0; j < (OWN ? (uint32_t)own_tokens(SRC) : 8u); ++j) {
+                if (8u * o + j < M) {
+                    if (p.y_is_bf16) *yb = __float2bfloat16_rn(v[j] * alpha);
+                    else *yf = v[j] * alpha;
+                }
+                yb += p.ldy; yf += p.ldy;
+            }
+        };
+        uint32_t accb = 0, acc_phase = 0;
+        for (uint32_t i = 0; i < n_units;) {
+            const uint32_t u = order.unit(i), tile = u / C, t_begin = tile * C, t_end = t_begin + C, u_stop = min(t_end, u_end);
             const bool whole = u == t_begin && t_end <= u_end;
+            i += u_stop - u;
             uint32_t nseg = 1, slot = 0;
             if (!whole) {                              // (before the wait: the divisions take a while)
                 const uint32_t c_first = cta_of_unit(p, t_begin);
                 nseg = cta_of_unit(p, t_end - 1) - c_first + 1;
                 slot = blockIdx.x - c_first;
             }
-            u = min(t_end, u_end);
+            const int64_t n = (int64_t)tile * 128 + row;
+            float* base = p.partials + ((size_t)tile * p.maxseg * 128 + row) * 16;
             if (!mbar_wait_warp(accf0 + 8 * accb, acc_phase, abort_flag, p.status, 11)) break;
             tc_fence_after();
-            if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(10);
-            // a tile shared with other CTAs: how many of them have handed in their sums already (the answer is
-            // needed only after this CTA's own sums are complete, so the load costs nothing)
+            if (i == n_units && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(10);
+            // a tile shared with other CTAs: how many of them have handed in their sums already (the answer is needed only after this CTA's own sums are
+            // complete; when all others were seen to have arrived, this warp is the last without asking)
             uint32_t* counter = p.counters + tile * 8 + q;
             uint32_t seen = 0;
             if (!whole && lane == 0) asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(counter) : "memory");
             // columns m (NVFP4 blocks), (p + 1) M + m (digits); FP8 weights: m (high), M + m (low)
             const uint32_t d4 = tmem_base + ((uint32_t)(q * 32) << 16) + D::D4_COL + accb * D::D4;
             const uint32_t d8 = tmem_base + ((uint32_t)(q * 32) << 16) + D::D8_COL + accb * D::D8;
-            float v[16], t[16];
-            uint32_t r0[16], r1[16], r2[16] = {};
-            if (OWN) {
-                // at most 14 and 4 columns: one load of each, the sums in the order of the general form
-                tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1);
-                tmem_wait_ld(r0, r1, r2);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] = 0.f;
-#pragma unroll
-                for (int j = 0; j < own_tokens(SRC); ++j) {
-                    constexpr int T = own_tokens(SRC);
-                    const auto col = [&](int i) { return __uint_as_float(r0[T * i + j]); };
-                    const float high = __uint_as_float(r1[j]), low = __uint_as_float(r1[T + j]);
-                    const float x = has_fp8 ? col(0) + (high + low) * rw : col(0);
-                    v[j] = x + (((col(1) + col(2)) + col(3)) + ((col(4) + col(5)) + col(6))) * ra;
-                }
-            } else {
-                // (three loads in flight at a time)
-                tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1); tmem_ld16_async(d8 + M, r2);
-                tmem_wait_ld(r0, r1, r2);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    v[j] = __uint_as_float(r0[j]); t[j] = 0.f;
-                    if (has_fp8) v[j] += (__uint_as_float(r1[j]) + __uint_as_float(r2[j])) * rw;     // (else those columns hold nothing)
-                }
 #pragma unroll 1
-                for (uint32_t pc = 1; pc < PIECES; pc += 3) {
-                    tmem_ld16_async(d4 + pc * M, r0); tmem_ld16_async(d4 + (pc + 1) * M, r1); tmem_ld16_async(d4 + (pc + 2) * M, r2);
+            for (uint32_t o = 0; o < octets; ++o) {
+                float v[8];
+                if constexpr (OWN) {
+                    // at most 14 and 4 columns: one load of each
+                    constexpr int T = own_tokens(SRC);
+                    uint32_t r0[16], r1[16], r2[16] = {};
+                    tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1);
                     tmem_wait_ld(r0, r1, r2);
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) t[j] += (__uint_as_float(r0[j]) + __uint_as_float(r1[j])) + __uint_as_float(r2[j]);
-                }
+                    for (int j = 0; j < 8; ++j) v[j] = 0.f;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) v[j] += t[j] * ra;
+                    for (int j = 0; j < T; ++j) v[j] = token_sum(has_fp8, rw, ra, [&](int k) { return r0[T * k + j]; }, r1[j], r1[T + j]);
+                } else {
+                    uint32_t r[PIECES + 1][8], hi[8], lo[8];
+#pragma unroll
+                    for (uint32_t k = 0; k <= (uint32_t)PIECES; ++k) tmem_ld8_async(d4 + k * M + 8u * o, r[k]);
+                    tmem_ld8_async(d8 + 8u * o, hi); tmem_ld8_async(d8 + M + 8u * o, lo);
+                    tmem_wait_ld8(hi);
+                    tmem_hold8(lo);
+#pragma unroll
+                    for (uint32_t k = 0; k <= (uint32_t)PIECES; ++k) tmem_hold8(r[k]);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = token_sum(has_fp8, rw, ra, [&](int k) { return r[k][j]; }, hi[j], lo[j]);
+                }
+                if (whole) emit(v, o, n);
+                else                                   // this CTA's part (32 bytes per store: whole sectors)
+                    asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                                 ::"l"(base + (size_t)slot * 2048 + 8u * o), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
+                                   "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
+                                   "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])) : "memory");
             }
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(acce0 + 8 * accb);
             accb ^= 1u;
             if (accb == 0) acc_phase ^= 1u;
-            if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(11);
-
-            const int64_t n = (int64_t)tile * 128 + row;
-            bool write_out = whole;
+            if (i == n_units && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(11);
             if (!whole) {
-                // partial tile: publish, and let the warp that arrives last add everything up.  When all the
-                // others were seen to have arrived, this warp is the last without asking and skips the counter.
-                float* base = p.partials + ((size_t)tile * p.maxseg * 128 + row) * 16;
-                float* dst = base + (size_t)slot * 2048;
-                // (32 bytes per store: whole sectors)
-#pragma unroll
-                for (int j = 0; j < 16; j += 8)
-                    if (j < (int)M)
-                        asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                                     ::"l"(dst + j), "r"(__float_as_uint(v[j])), "r"(__float_as_uint(v[j + 1])), "r"(__float_as_uint(v[j + 2])),
-                                       "r"(__float_as_uint(v[j + 3])), "r"(__float_as_uint(v[j + 4])), "r"(__float_as_uint(v[j + 5])),
-                                       "r"(__float_as_uint(v[j + 6])), "r"(__float_as_uint(v[j + 7])) : "memory");
-                // The counter wraps to zero with the last arrival (or is put back by the warp that skipped
-                // it), so the workspace is ready for the next call without being cleared.
+                // The counter wraps to zero with the last arrival (or is put back by the warp that need not ask it), so the workspace is ready for the next
+                // call without being cleared.
                 uint32_t old = __shfl_sync(0xffffffffu, seen, 0);
                 if (old != nseg - 1) {
                     // the warp's stores are ordered before lane 0's release of the counter; its acquire sees the others'
-                    __syncwarp();
                     if (lane == 0)
                         asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;" : "=r"(old) : "l"(counter), "r"(nseg - 1) : "memory");
                     old = __shfl_sync(0xffffffffu, old, 0);
                 } else if (lane == 0) {
                     *counter = 0u;
                 }
-                if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(12);
-                if (old == nseg - 1) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) v[j] = 0.f;
+                if (i == n_units && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(12);
+                if (old == nseg - 1) {                 // this warp is the last: it adds everything up
 #pragma unroll 1
-                    for (uint32_t sgi = 0; sgi < nseg; ++sgi) {       // one sum in slot order
-                        const float* src = base + (size_t)sgi * 2048;
+                    for (uint32_t o = 0; o < octets; ++o) {
+                        float v[8];
 #pragma unroll
-                        for (int j = 0; j < 16; j += 8) {
-                            if (j >= (int)M) break;
-                            uint32_t y8[8];
-                            asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                         : "=r"(y8[0]), "=r"(y8[1]), "=r"(y8[2]), "=r"(y8[3]), "=r"(y8[4]), "=r"(y8[5]), "=r"(y8[6]), "=r"(y8[7])
-                                         : "l"(src + j) : "memory");
+                        for (int j = 0; j < 8; ++j) v[j] = 0.f;
+#pragma unroll 1
+                        for (uint32_t g = 0; g < nseg; g += 2) {       // one sum in slot order, two parts under way at a time
+                            uint32_t y[2][8];
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) v[j + e] += __uint_as_float(y8[e]);
+                            for (uint32_t h = 0; h < 2; ++h)           // (a last one twice)
+                                asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                                             : "=r"(y[h][0]), "=r"(y[h][1]), "=r"(y[h][2]), "=r"(y[h][3]), "=r"(y[h][4]), "=r"(y[h][5]), "=r"(y[h][6]), "=r"(y[h][7])
+                                             : "l"(base + (size_t)min(g + h, nseg - 1u) * 2048 + 8u * o) : "memory");
+#pragma unroll
+                            for (uint32_t h = 0; h < 2; ++h) {
+                                if (g + h >= nseg) break;
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) v[j] += __uint_as_float(y[h][j]);
+                            }
                         }
-                    }
-                    write_out = true;
-                }
-            }
-            if (u == u_end && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(whole ? 7 : 8);    // last segment: sums complete / handed in
-            if (write_out && n < p.N) {
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    if (j < (int)M) {
-                        if (p.y_is_bf16) reinterpret_cast<__nv_bfloat16*>(p.Ybf)[(int64_t)j * p.ldy + n] = __float2bfloat16_rn(v[j] * alpha);
-                        else p.Y[(int64_t)j * p.ldy + n] = v[j] * alpha;
+                        emit(v, o, n);
                     }
                 }
             }
+            if (i == n_units && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(whole ? 7 : 8);    // last segment: sums complete / handed in
         }
     }
 

@@ -93,6 +93,24 @@ def test_gemm_on_packed_weights_wide_tiles(fg, M, N, K, tokens, shared):
         compare_packed(fg, fg.linear_quantize(pa, pw, f.cuda(), scale_fp4=s4, tau=s4 * s4), q, s4 * s4, "hidden")
 
 
+# decode: spans whose last part of a tile is taken before the rest: behind a whole tile, behind a part, beside spans without such a part; a part of one unit
+# and parts of nearly a span; one and two octets of tokens; own and shared quantizer, and packed tokens
+@pytest.mark.parametrize("M,N,K", [(1, 19000, 512), (2, 3968, 2560), (9, 4992, 4096), (5, 2176, 2816), (16, 9500, 1280)])
+def test_decode_takes_short_last_parts_first(fg, M, N, K):
+    wl = gi.llama("front", M, N, K, seed=71)
+    qa, qw, pa, pw = quantize_both(fg, wl, 0.1, 0.1, clip=False)
+    x, fx = wl.x().cuda(), wl.fx().cuda()
+    s4 = qa.scale_fp4
+    Y, S = oracle.linear(qa, qw)
+    tau = tau_for_fraction(oracle.quantize_activations(gi.bf16_bits(wl.x()), wl.fx().numpy(), s4, tau=np.inf).scores, 0.1)
+    for y in (fg.linear(pa, pw), fg.linear_fused(x, fx, pw, scale_fp4=s4, tau=tau)):
+        fg.check(fg.linear.last_workspace)
+        assert (np.abs(y.cpu().numpy().astype(np.float64) - Y) <= 1e-5 * S + 1e-30).all()
+    ws = fg.alloc_workspace(fg.OP_LINEAR_FUSED, M, N, K, torch.device("cuda"))
+    ys = [fg.linear_fused(x, fx, pw, scale_fp4=s4, tau=tau, workspace=ws) for _ in range(20)]
+    assert all(torch.equal(y, ys[0]) for y in ys), "the sum over the parts of a tile has a fixed order"
+
+
 # large batch: both operands expanded to fp16 planes, ragged in every direction
 @pytest.mark.parametrize("frac_a,frac_w", [(0.1, 0.1), (0.0, 1.0)])
 def test_gemm_on_expanded_planes_ragged(fg, frac_a, frac_w):
