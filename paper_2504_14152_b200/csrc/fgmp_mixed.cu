@@ -22,10 +22,10 @@
 // Four groups, CTA pairs that share a token tile, spinning instead of suspended waits and a loop of one elected thread in the issuer were measured
 // and are no faster.
 //
-// Work is (weight tile, token tile, 256-element K chunk) units in that order, split over the CTAs either in
-// equal contiguous spans (stream-K: the partial sums of tiles shared by several CTAs are stored, eight columns of a row at a time, and added
+// Work is (weight tile, token tile, 256-element K chunk) units in that order.  With few tiles each has a cluster of 2 to 8 CTAs, which share its chunks out and
+// add its sums up through one another's shared memory; else it is split over the CTAs either in equal contiguous spans (stream-K: the partial sums of tiles shared by several CTAs are stored, eight columns of a row at a time, and added
 // up in CTA order by a kernel of their own, which has the whole chip's loads in flight: 43 MB at 203 tokens and 13824 weight
-// rows, 20 us if the CTA that arrives last does it) or in whole tiles, whichever the model in mixed_us says is faster.
+// rows, 20 us if the CTA that arrives last does it) or in whole tiles; the model in mixed_us says which is fastest.
 //
 // Warp roles: warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, warp 2 = token-tile producer,
 // warps 3-6 = epilogue, then the dequantization, NG groups of four warps that take the steps in turn.  Every
@@ -60,6 +60,7 @@ struct MixedPlan {
     uint32_t chunks, tiles;              // tiles = wtiles * tok_tiles
     uint32_t grid, span, rest, quantum;  // a CTA's span in quanta of `quantum` units (1, or chunks: whole tiles)
     uint32_t split;                      // 1: some tile is shared by several CTAs, whose parts are added up behind this kernel
+    uint32_t cluster;                    // 0, or the CTAs that share each tile, a cluster that adds its parts up itself (2 to 8)
     uint32_t ks;                         // steps of 64 elements of K that are handed to the MMA issuer at once (1 or 2)
     uint32_t wstages, slots, naccs;
     uint32_t ring;                       // token stages, of ks steps each
@@ -90,7 +91,11 @@ __device__ __forceinline__ void umma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
-__device__ __forceinline__ uint32_t unit_begin(const MixedPlan& pl, uint32_t cta) { return (cta * pl.span + min(cta, pl.rest)) * pl.quantum; }
+__device__ __forceinline__ uint32_t unit_begin(const MixedPlan& pl, uint32_t cta)
+{
+    if (pl.cluster) { const uint32_t tile = cta / pl.cluster; return tile * pl.chunks + (cta - tile * pl.cluster) * pl.chunks / pl.cluster; }
+    return (cta * pl.span + min(cta, pl.rest)) * pl.quantum;
+}
 __device__ __forceinline__ uint32_t cta_of(const MixedPlan& pl, uint32_t u)
 {
     const uint32_t i = u / pl.quantum, longer = pl.rest * (pl.span + 1);
@@ -108,11 +113,11 @@ __device__ __forceinline__ void quantize_row32(const MixedParams& p, int64_t m, 
     if (bits) atomicOr(word, bits << pos);
 }
 
-// One warp's share of a tile's result: 32 token columns from column cc on, lane = weight row n (v: sums in units of alpha)
+// One warp's share of a tile's result: 32 token columns from column cc on, as far as token m_end, lane = weight row n (v: sums in units of alpha)
 template <bool QUANT>
-__device__ __forceinline__ void mixed_emit(const MixedParams& p, const uint32_t (&v)[32], int64_t n, int64_t m0, uint32_t cc, float alpha, int lane, uint32_t* turn)
+__device__ __forceinline__ void mixed_emit(const MixedParams& p, const uint32_t (&v)[32], int64_t n, int64_t m0, int64_t m_end, uint32_t cc, float alpha, int lane,
+                                           uint32_t* turn)
 {
-    const int64_t m_end = min(p.M, m0 + p.pl.n_tok);
     if (QUANT) {
         // turned round in shared memory: lane = token, 32 consecutive values of n = two blocks of the next layer's activations
 #pragma unroll
@@ -154,6 +159,62 @@ __device__ __forceinline__ void add_parts8(const float* src, float* s)
     for (int j = 0; j < 8; ++j) s[j] += __uint_as_float(x[j]);
 }
 
+__device__ __forceinline__ float mixed_alpha(const MixedParams& p, int t_w)
+{
+    return __fmul_rn(__fmul_rn(p.ha->scale_fp4, __ldg(&reinterpret_cast<const fgmp_packed_header*>(p.wblob)->scale_fp4)), __int_as_float((127 + t_w) << 23));
+}
+
+// A cluster that shares a tile: CTA r gets the columns (tokens) r S .. of the sums of all, in parts by CTA, four columns of all rows and then the next four,
+// where the ring of token tiles was.  Each epilogue warp sends its rows to whom they belong, and when all have done so adds up, in CTA order, and
+// emits the columns of its own CTA.
+__device__ __forceinline__ uint32_t cluster_slice(const MixedPlan& pl) { return ((pl.n_tok + pl.cluster - 1u) / pl.cluster + 3u) & ~3u; }
+__device__ __forceinline__ void cluster_send(const MixedPlan& pl, uint32_t acc, uint32_t buf, uint32_t rank, int warp, int lane)
+{
+    const uint32_t S = cluster_slice(pl), row = 32u * ((uint32_t)warp & 3u) + lane, d = acc + ((((uint32_t)warp & 3u) * 32u) << 16);
+    uint32_t owner = 0, at = 0;                          // of the column, and its place there
+#pragma unroll 1
+    for (uint32_t cc = 0; cc < pl.n_tok; cc += 32) {
+        uint32_t v[32];
+        tmem_ld32(d + cc, v);
+#pragma unroll
+        for (uint32_t j = 0; j < 32; j += 4) {
+            if (cc + j < pl.n_tok) {
+                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
+                             ::"r"(cluster_map(buf, owner) + ((rank * S + at) / 4u * 128u + row) * 16u), "r"(v[j]), "r"(v[j + 1]), "r"(v[j + 2]), "r"(v[j + 3]) : "memory");
+                at += 4;
+                if (at == S) { at = 0; ++owner; }
+            }
+        }
+    }
+}
+template <bool QUANT>
+__device__ __forceinline__ void cluster_add(const MixedParams& p, const uint8_t* buf, uint32_t rank, uint32_t tile, int warp, int lane, int t_w, float* extra)
+{
+    const MixedPlan& pl = p.pl;
+    const uint32_t S = cluster_slice(pl), q = (uint32_t)warp & 3u, row = 32u * q + lane;
+    const float alpha = mixed_alpha(p, t_w);
+    uint32_t* turn = reinterpret_cast<uint32_t*>(extra) + q * 32 * 33;
+    const int64_t t0 = (int64_t)(tile % pl.tok_tiles) * pl.n_tok, m0 = t0 + rank * S, n = (int64_t)(tile / pl.tok_tiles) * 128 + row;
+    const int64_t m_end = min(min(p.M, t0 + pl.n_tok), m0 + S);
+#pragma unroll 1
+    for (uint32_t cc = 0; m0 + cc < m_end; cc += 32) {
+        uint32_t v[32];
+#pragma unroll
+        for (uint32_t j = 0; j < 32; j += 4) {
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (cc + j < S) {
+#pragma unroll 1
+                for (uint32_t i = 0; i < pl.cluster; ++i) {
+                    const float4 x = reinterpret_cast<const float4*>(buf)[(i * (S / 4u) + (cc + j) / 4u) * 128u + row];
+                    s.x += x.x; s.y += x.y; s.z += x.z; s.w += x.w;
+                }
+            }
+            v[j] = __float_as_uint(s.x); v[j + 1] = __float_as_uint(s.y); v[j + 2] = __float_as_uint(s.z); v[j + 3] = __float_as_uint(s.w);
+        }
+        mixed_emit<QUANT>(p, v, n, m0, m_end, cc, alpha, lane, turn);
+    }
+}
+
 // Epilogue warps: tensor-memory lane quadrant warp % 4, lane = weight row, column = token
 template <bool QUANT>
 __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tmem_base, int warp, int lane, uint32_t u_begin, uint32_t u_end,
@@ -161,8 +222,7 @@ __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tm
 {
     const MixedPlan& pl = p.pl;
     const uint32_t q = (uint32_t)warp & 3u, C = pl.chunks, NT = pl.n_tok, NP = (NT + 31u) & ~31u, row = 32u * q + lane;   // (NP: columns of a partial tile)
-    const float alpha = __fmul_rn(__fmul_rn(p.ha->scale_fp4, __ldg(&reinterpret_cast<const fgmp_packed_header*>(p.wblob)->scale_fp4)),
-                                  __int_as_float((127 + t_w) << 23));
+    const float alpha = mixed_alpha(p, t_w);
     uint32_t* turn = reinterpret_cast<uint32_t*>(extra) + q * 32 * 33;
     uint32_t acc = 0, acc_phase = 0;
     for (uint32_t u = u_begin; u < u_end;) {
@@ -179,7 +239,7 @@ __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tm
         for (uint32_t cc = 0; cc < NT; cc += 32) {
                 uint32_t v[32];
                 tmem_ld32(d + cc, v);
-                if (whole) mixed_emit<QUANT>(p, v, n, m0, cc, alpha, lane, turn);
+                if (whole) mixed_emit<QUANT>(p, v, n, m0, min(p.M, m0 + NT), cc, alpha, lane, turn);
                 else
 #pragma unroll
                     for (int j = 0; j < 32; j += 8) store_parts8(mine + (cc + j) * 128, v + j);
@@ -288,7 +348,9 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     } else if (may_skip || (warp < W_DEQ && warp != W_MMA)) {
         if (warp == W_TOK && lane == 0) asm volatile("prefetch.tensormap [%0];" ::"l"(&tmB) : "memory");
         asm volatile("griddepcontrol.wait;" ::: "memory");
-        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        // (Clusters: what follows comes up when this grid is done.  Before that its blocks would crowd on the few SMs that are left free: quantizer and call,
+        // 30 x 1664 x 9728, 15.4 us, 18.4 with an early start.)
+        if (!pl.cluster) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
     // (The weights are dequantized before the kernel in front is done, as far as there are slots: only the tokens are its.)
     if (QUANT && blockIdx.x == 0 && threadIdx.x == 32 * W_EPI) {
@@ -455,11 +517,23 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
             if (++stage == WS) { stage = 0; phase ^= 1; }
             if (++c == C) c = 0;
         }
+    } else if (pl.cluster) {
+        mbar_wait_warp(accf0, 0, abort_flag, p.status, 8);       // (this CTA's products are done, and with them its reads of shared memory)
+        tc_fence_after();
     } else {
         mixed_epilogue<QUANT>(p, tmem_base, warp, lane, u_begin, u_end, accf0, acce0, abort_flag, t_w, reinterpret_cast<float*>(extra));
     }
 
     __syncthreads();
+    if (pl.cluster && !skip) {                           // (whatever has gone wrong in a CTA, all of the cluster come here)
+        const uint32_t rank = cluster_ctarank();
+        const bool mine = warp >= W_EPI && warp < W_DEQ;
+        cluster_sync();
+        if (mine) cluster_send(pl, tmem_base, smem_u32(smem), rank, warp, lane);
+        cluster_sync();
+        if (mine) cluster_add<QUANT>(p, smem, rank, blockIdx.x / pl.cluster, warp, lane, t_w, reinterpret_cast<float*>(extra));
+        __syncthreads();
+    }
     if (*abort_flag) {
         // copies may be under way
         const unsigned long long t0 = globaltimer_ns();
@@ -562,16 +636,24 @@ size_t parts_bytes(const MixedPlan& pl) { return pl.split ? (size_t)pl.grid * 2 
 //     the next tile's products as far as those take that long, six chunks; with fewer it is what such a call takes (1220 x 15936 x 768: 63 us, on the planes 41).
 //   - the sum over parts: a part after the other, 0.34 us each where a tile has a thread block of its own for its 32 columns (53 x 644 x 8960: one tile of
 //     64 tokens in 26 parts 25 us, of 16 tokens in 7 parts 18)
+//   - a cluster for each tile: what comes before and behind its units depends on how many SMs it leaves free (fitted to quantizer and call, 136 shapes of up to
+//     1200 tokens, 1400 cuts: off by 4.5 %; calls take 0.893 of the time that the other ways take over these shapes, the best cuts 0.874; three take
+//     2 to 4 % more).  Quantizer and call, 48 x 4096 x 4096, three CTAs a tile: 15.5 us, 18.5 in spans; 30 x 1664 x 9728, eight: 14.5, 21.3; 65 x 2368 x 6080,
+//     four: 16.9, 21.0.
+//     (Layers of fewer than eight weight tiles keep the other ways beyond 96 tokens, although clusters would gain there too, 436 x 256 x 2240 11.4 instead
+//     of 14.0 without the quantizer: they are what the kernel's tile sizes are tested with.)
 //   - launches: the next kernel's thread blocks come up early only where SMs are left that the GEMM does not fill (310 x 448 x 1280: 13.8 us on 140, 10.4
 //     on 100)
 // Where a call with the next layer's quantizer in it is possible its way out counts as well (1.34 us + 0.0403 per token, 3.4 + 0.51 per part), to three tenths: the two
 // calls are cut alike, so that their sums are the same.
-double mixed_us(const MixedPlan& pl, int64_t M, int64_t N, int64_t K)
+double mixed_us(const MixedPlan& pl, int64_t M, int64_t N, int64_t K, double sms)
 {
-    const double n = pl.n_tok, sms = fgmp_sm_count(), left = sms - pl.grid, units = pl.span + (pl.rest ? 1.0 : 0.0);
+    const double n = pl.n_tok, left = sms - pl.grid, units = pl.span + (pl.rest ? 1.0 : 0.0);
     const bool both = N % 64 == 0;
     const double unit = pl.naccs == 2 ? fmax(0.88, 0.77 + 0.0021 * n) : pl.ks == 2 ? 0.50 + 0.0037 * n : n <= 256 ? 0.475 + 0.0038 * n : 0.495 + 0.0045 * n;
     const double out = both ? 0.93 + 0.0375 * n : 0.77 + 0.0363 * n;
+    if (pl.cluster)
+        return 1.02 * (6.0 + 2.47e-6 * (double)M * (double)K + units * (0.767 + 0.0016 * n) + 0.029 * n + 0.02 * fmax(0.0, n - 144.0) + 2.3 * pl.grid / 148.0);
     double us = 4.4 + 0.59e-6 * (double)M * (double)K;
     if ((double)M * (double)K > 6.0 * 8192.0 * left) us += 2.2;
     if (!pl.split) {
@@ -591,6 +673,13 @@ double roomy_us(const MixedPlan& pl)
     const double units = (double)(pl.span + (pl.rest ? 1 : 0)) * pl.quantum, tiles = units / pl.chunks;
     const double drains = 2 * pl.n_tok + 96 <= MX_TMEM_COLS || tiles < 1.0 ? 1.0 : pl.n_tok <= 256 ? tiles : 2.0 * (tiles + 1.0);
     return units * (1.08 + 0.0042 * pl.n_tok) + drains * 0.012 * pl.n_tok + (pl.split ? 2.0 + 2.6 * pl.grid * pl.n_tok * 512.0 / 8e6 : 3.0 * tiles);
+}
+
+// Clusters of c CTAs (2 to 8), each with an SM to itself, that run at once on the 148 SMs of a B200, as cudaOccupancyMaxActiveClusters has them
+uint32_t resident_clusters(uint32_t c, uint32_t sms)
+{
+    static const uint8_t of_148[9] = {0, 0, 74, 45, 33, 26, 22, 15, 15};
+    return (uint32_t)of_148[c] * sms / 148u;
 }
 
 // How the work is cut: tokens per tile, and whether CTAs take whole tiles or equal spans of units: the least modelled time among the
@@ -613,6 +702,13 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts, boo
         pl.ks = pl.n_tok <= 208 ? 2 : 1;
         pl.naccs = 2 * pl.n_tok + 96 * pl.ks <= MX_TMEM_COLS ? 2 : 1;
         const uint64_t total = (uint64_t)pl.tiles * chunks;
+        for (uint32_t c = 2; !roomy && (M <= 96 || wtiles >= 8) && c <= 8 && c <= chunks && pl.n_tok <= 256; ++c) {
+            if (pl.tiles > resident_clusters(c, sms)) break;      // (nor do larger ones fit)
+            MixedPlan cl = pl;
+            cl.cluster = c; cl.naccs = 1; cl.grid = pl.tiles * c; cl.quantum = 1; cl.span = (chunks + c - 1) / c;
+            cl.us = mixed_us(cl, M, N, K, sms);
+            if (cl.us < best.us) best = cl;
+        }
         for (int split = 0; split < (chunks > 1 ? 2 : 1); ++split) {
             pl.quantum = split ? 1 : chunks;
             const uint64_t quanta = total / pl.quantum;
@@ -622,7 +718,7 @@ MixedPlan mixed_plan(int64_t M, int64_t N, int64_t K, size_t room_for_parts, boo
             pl.split = split;
             if (split && pl.rest == 0 && pl.span % chunks == 0) continue;
             if (parts_bytes(pl) > room_for_parts) continue;
-            pl.us = roomy ? roomy_us(pl) : mixed_us(pl, M, N, K);
+            pl.us = roomy ? roomy_us(pl) : mixed_us(pl, M, N, K, sms);
             if (pl.us < best.us) best = pl;
         }
     }
@@ -657,7 +753,7 @@ double fgmp_mixed_us(int64_t M, int64_t N, int64_t K, size_t ws_bytes) { return 
 void fgmp_mixed_cut(int64_t M, int64_t N, int64_t K, size_t ws_bytes, int32_t* cut)
 {
     const MixedPlan pl = mixed_plan(M, N, K, room_in(ws_bytes, M, K));
-    const uint32_t v[6] = {pl.n_tok, 64 * pl.ks, pl.naccs, pl.split, pl.ring, pl.slots};
+    const uint32_t v[6] = {pl.n_tok, 64 * pl.ks, pl.naccs, pl.cluster ? 1u : pl.split, pl.ring, pl.slots};
     for (int i = 0; i < 6; ++i) cut[i] = (int32_t)v[i];
 }
 
@@ -698,11 +794,13 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     CUtensorMap tmB;
     if (!fgmp_map_2d(&tmB, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, plane, M, K, K * 2, p.pl.n_half, 64)) return FGMP_ERR_CUDA;
 
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = p.pl.cluster; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
+    cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = p.pl.cluster ? 2 : 1;
     const fgmp_status st = fgmp_expand(packed_acts, packed_weights, M, N, K, plane, nullptr, p.status, 0, 0, leave_nvfp4, first, s);
     if (st != FGMP_OK) return st;
     const bool quant = qn.codes4 != nullptr;

@@ -93,6 +93,25 @@ def test_gemm_on_packed_weights_wide_tiles(fg, M, N, K, tokens, shared):
         compare_packed(fg, fg.linear_quantize(pa, pw, f.cuda(), scale_fp4=s4, tau=s4 * s4), q, s4 * s4, "hidden")
 
 
+# clusters of 2 to 8 CTAs that share a tile: chunks that do not divide by them, a last chunk of 64 and of 192 elements, slices of tokens that do not divide
+# and empty ones, several token tiles, a ragged weight tile; Y in both types and the next layer's quantizer
+@pytest.mark.parametrize("M,N,K", [(19, 5248, 2112), (43, 640, 9792), (20, 320, 9152), (90, 832, 5632), (269, 1216, 5056), (43, 2435, 12032), (100, 4096, 4096), (33, 1027, 11904)])
+@pytest.mark.parametrize("frac", [0.1, 0.4])
+def test_gemm_on_packed_weights_in_clusters(fg, M, N, K, frac):
+    qa, qw, pa, pw = quantize_both(fg, gi.llama("cl", M, N, K, seed=72), frac, frac, clip=False)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        count = launches(fg, lambda: fg.linear(pa, pw))
+        assert count.get("gemm_mixed_tcgen05") == 1 and "gemm_reduce" not in count and fg.linear_cut(M, N, K)["shared"] == 1, count
+    check_linear(fg, qa, qw, pa, pw)
+    y = fg.linear(pa, pw)
+    assert all(torch.equal(fg.linear(pa, pw), y) for _ in range(10)), "the sum over the parts of a tile has a fixed order"
+    if N % 64 == 0:
+        y16, f = fg.linear(pa, pw, out_dtype=torch.bfloat16), torch.ones(N)
+        s4 = gi.tensor_scale(y16.float().cpu())
+        q = oracle.quantize_activations(gi.bf16_bits(y16.cpu()), f.numpy(), s4, tau=s4 * s4)
+        compare_packed(fg, fg.linear_quantize(pa, pw, f.cuda(), scale_fp4=s4, tau=s4 * s4), q, s4 * s4, "hidden")
+
+
 # decode: spans whose last part of a tile is taken before the rest: behind a whole tile, behind a part, beside spans without such a part; a part of one unit
 # and parts of nearly a span; one and two octets of tokens; own and shared quantizer, and packed tokens
 @pytest.mark.parametrize("M,N,K", [(1, 19000, 512), (2, 3968, 2560), (9, 4992, 4096), (5, 2176, 2816), (16, 9500, 1280)])
