@@ -10,6 +10,7 @@
 #include "fgmp_common.cuh"
 #include "fgmp_host.h"
 #include <cuda_bf16.h>
+#include <atomic>
 
 namespace {
 
@@ -234,16 +235,35 @@ fgmp_status check_act_args(const void* X, int64_t ldx, const float* fisher, int6
     return FGMP_OK;
 }
 
-template <int MODE, bool SCORE_ONLY>
-void launch_quant(const ActParams& p, cudaStream_t s)
+// Shared memory that a small grid asks for, so that an SM holds no more of its thread blocks than it has to: they come up while the kernel before runs, on the
+// SMs that it leaves free, and more of them would crowd there (behind a GEMM on 144 SMs sixty blocks on the other four) instead of waiting for all SMs.
+// Quantizer and linear in a row, 126 x 2304 x 1024: 14.9 us, so 14.0; 328 x 2112 x 768 14.4 and 13.9.  From six blocks an SM on the registers say so.
+int spread_bytes(int64_t blocks)
 {
+    static const int of[] = {0, 120, 80, 60, 48, 40};                // more than 227 KiB over one block more than that
+    const int64_t sms = fgmp_sm_count(), per_sm = (blocks + sms - 1) / sms;
+    return per_sm <= 5 ? of[per_sm] * 1024 : 0;
+}
+
+template <int MODE, bool SCORE_ONLY>
+fgmp_status launch_quant(const ActParams& p, cudaStream_t s)
+{
+    static std::atomic<uint64_t> ready{0};                           // a bit per device
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return FGMP_ERR_CUDA;
+    if (!((ready.load(std::memory_order_acquire) >> dev) & 1u)) {
+        if (cudaFuncSetAttribute(quant_act_kernel<MODE, SCORE_ONLY>, cudaFuncAttributeMaxDynamicSharedMemorySize, spread_bytes(1)) != cudaSuccess) return FGMP_ERR_CUDA;
+        ready.fetch_or(1ull << dev, std::memory_order_release);
+    }
+    const int64_t blocks = ((int64_t)p.groups * p.MW + QA_THREADS / 32 - 1) / (QA_THREADS / 32);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(((int64_t)p.groups * p.MW + QA_THREADS / 32 - 1) / (QA_THREADS / 32)));
+    cfg.gridDim = dim3((unsigned)blocks); cfg.dynamicSmemBytes = (size_t)spread_bytes(blocks);
     cfg.blockDim = dim3(QA_THREADS); cfg.stream = s; cfg.attrs = attr; cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, quant_act_kernel<MODE, SCORE_ONLY>, p);
+    return FGMP_OK;
 }
 
 ActParams make_act_params(const void* X, int64_t ldx, const float* fisher, int64_t M, int64_t K, fgmp_scales sc, float tau)
@@ -290,9 +310,8 @@ extern "C" fgmp_status fgmp_quantize_activations(const void* X_bf16, int64_t ldx
     p.mask = reinterpret_cast<uint32_t*>(blob + L.off_mask); p.codes8 = blob + L.off_codes8;
     p.header = reinterpret_cast<fgmp_packed_header*>(blob);
     if (M <= 16 && !p.free8) p.arec = blob + L.off_arec;     // decode-sized batch: also emit the records of the decode GEMM (tied scales only)
-    if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, launch_quant<0, false>(p, s));
-    else                           FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, launch_quant<1, false>(p, s));
-    return fgmp_launch_status();
+    FGMP_LAUNCH(FGMP_K_ACT_QUANT, s, st = sm == FGMP_SCORE_LP_ERROR ? launch_quant<0, false>(p, s) : launch_quant<1, false>(p, s));
+    return st == FGMP_OK ? fgmp_launch_status() : st;
 }
 
 extern "C" fgmp_status fgmp_activation_scores(const void* X_bf16, int64_t ldx, const float* fisher_chan,
@@ -306,9 +325,8 @@ extern "C" fgmp_status fgmp_activation_scores(const void* X_bf16, int64_t ldx, c
     cudaStream_t s = (cudaStream_t)cuda_stream;
     ActParams p = make_act_params(X_bf16, ldx, fisher_chan, M, K, sc, 0.f);
     p.scores = scores;
-    if (sm == FGMP_SCORE_LP_ERROR) FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, launch_quant<0, true>(p, s));
-    else                           FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, launch_quant<1, true>(p, s));
-    return fgmp_launch_status();
+    FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, st = sm == FGMP_SCORE_LP_ERROR ? launch_quant<0, true>(p, s) : launch_quant<1, true>(p, s));
+    return st == FGMP_OK ? fgmp_launch_status() : st;
 }
 
 extern "C" fgmp_status fgmp_unpack(const void* packed, int64_t rows, int64_t K, uint8_t* codes4, uint8_t* codes8,
