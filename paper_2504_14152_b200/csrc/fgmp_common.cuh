@@ -115,8 +115,8 @@ __host__ __device__ inline uint32_t fgmp_list_entry(uint32_t r, uint32_t j)
 }
 
 #ifdef __CUDACC__
-// Where the FP8 blocks of one unit sit in its list, for 128 threads: thread i brings the 16 mask bits of row i of the
-// tile (0 beyond the last row).
+// Where the FP8 blocks of one unit sit in its list: thread i < 128 brings the 16 mask bits of row i of the tile (0 beyond the last row), further
+// threads of the block only come along.
 struct UnitScratch {
     uint32_t warp[4];
     uint16_t m16[128], base[128];        // mask bits of a row; FP8 blocks of the unit before it
@@ -129,11 +129,13 @@ struct UnitScratch {
         uint32_t incl = own;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
-        if (lane == 31) warp[w] = incl;
+        if (lane == 31 && w < 4) warp[w] = incl;
         __syncthreads();
         const uint32_t c0 = warp[0], c1 = warp[1], c2 = warp[2], c3 = warp[3];
-        m16[threadIdx.x] = (uint16_t)bits;
-        base[threadIdx.x] = (uint16_t)(incl - own + (w > 0 ? c0 : 0u) + (w > 1 ? c1 : 0u) + (w > 2 ? c2 : 0u));
+        if (threadIdx.x < 128) {
+            m16[threadIdx.x] = (uint16_t)bits;
+            base[threadIdx.x] = (uint16_t)(incl - own + (w > 0 ? c0 : 0u) + (w > 1 ? c1 : 0u) + (w > 2 ? c2 : 0u));
+        }
         __syncthreads();
         return c0 + c1 + c2 + c3;
     }

@@ -29,6 +29,9 @@ inline bool fgmp_map_y(CUtensorMap* map, void* Y, int y_is_bf16, int64_t ldy, in
 // workspace sizes of the individual operations
 size_t fgmp_ws_quantize_weights(int64_t N, int64_t K);
 size_t fgmp_ws_calibrate(int64_t M, int64_t K);
+// fgmp_activation_scores, and words that its kernel sets to zero
+fgmp_status fgmp_activation_scores_clear(const void* X_bf16, int64_t ldx, const float* fisher_chan, int64_t M, int64_t K, fgmp_scales sc,
+                                         fgmp_score_mode sm, float* scores, uint32_t* clear, int clear_words, void* cuda_stream);
 size_t fgmp_ws_linear(int64_t M, int64_t N, int64_t K);
 size_t fgmp_ws_linear_least(int64_t M, int64_t N, int64_t K);          // what a call must be given, see fgmp_linear
 size_t fgmp_ws_linear_quantize(int64_t M, int64_t N, int64_t K);

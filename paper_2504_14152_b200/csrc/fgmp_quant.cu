@@ -23,6 +23,7 @@ struct ActParams {
     float s4, k6, s8, inv8, tau;
     uint8_t* codes4; uint8_t* sf; uint32_t* mask; uint8_t* codes8;   // codes8: dense plane
     float* scores;                       // optional (score-only kernel)
+    uint32_t* clear; int clear_words;    // score-only kernel: words that are to be zero when it has ended
     uint8_t* arec;                       // optional per-chunk records for the decode GEMM (M <= 16)
     fgmp_packed_header* header;
     float r8;                            // 2^ratio
@@ -45,6 +46,8 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
         h->fp8_log2_ratio = p.ratio; h->n_fp8 = (p.tau == INFINITY) ? 0 : -1; h->tau_eff = 0.f; h->kind = 0; h->capacity = 0;
         h->error = 0; h->scale_fp8 = p.s8; h->fp8_scale_free = p.free8;
     }
+    if (SCORE_ONLY && blockIdx.x == 0)
+        for (int i = threadIdx.x; i < p.clear_words; i += QA_THREADS) p.clear[i] = 0;
     const uint32_t warp = blockIdx.x * (QA_THREADS / 32) + (threadIdx.x >> 5), MW = (uint32_t)p.MW, group = warp / MW, word = warp - group * MW;
     if (group >= p.groups) return;
     const int64_t kb = (int64_t)word * 32 + (threadIdx.x & 31);
@@ -141,8 +144,7 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
 }
 
 // packed activations -> canonical arrays; one thread per block
-__global__ void unpack_kernel(const uint8_t* blob, int64_t rows, int64_t K,
-                              uint8_t* codes4, uint8_t* codes8, uint8_t* scales, uint32_t* mask)
+__device__ __forceinline__ void unpack_acts(const uint8_t* blob, int64_t rows, int64_t K, uint8_t* codes4, uint8_t* codes8, uint8_t* scales, uint32_t* mask)
 {
     const PackedLayout L = fgmp_layout(rows, K, 0, 0);
     const uint32_t* pmask = reinterpret_cast<const uint32_t*>(blob + L.off_mask);
@@ -165,11 +167,23 @@ __global__ void unpack_kernel(const uint8_t* blob, int64_t rows, int64_t K,
     }
 }
 
-// packed weights -> canonical arrays; one CTA of 128 threads per unit record
-__global__ void __launch_bounds__(128) unpack_w_kernel(const uint8_t* blob, int64_t rows, int64_t K,
-                                                       uint8_t* codes4, uint8_t* codes8, uint8_t* scales, uint32_t* mask)
+__host__ __device__ inline bool unpackable(const fgmp_packed_header& h, int64_t rows, int64_t K)
+{
+    return h.magic == FGMP_MAGIC && h.version == FGMP_LAYOUT_VERSION && h.rows == rows && h.K == K && h.error == 0;
+}
+
+// Packed -> canonical arrays.  The blob says what it is, activations keep planes, weights keep unit records: the kernel looks, so that it need not wait until the
+// host has.  Weights: one CTA of 128 threads per unit record (activations have as many rows to a CTA, more than enough of them to fill the chip).
+__global__ void __launch_bounds__(128) unpack_kernel(const uint8_t* blob, int64_t rows, int64_t K,
+                                                     uint8_t* codes4, uint8_t* codes8, uint8_t* scales, uint32_t* mask)
 {
     __shared__ UnitScratch sc;
+    const fgmp_packed_header& h = *reinterpret_cast<const fgmp_packed_header*>(blob);
+    if (!unpackable(h, rows, K)) return;
+    if (h.kind != 1) {
+        unpack_acts(blob, rows, K, codes4, codes8, scales, mask);
+        return;
+    }
     const PackedLayout L = fgmp_layout(rows, K, 1, 0);
     if (mask) {                                         // canonical order: a row's bits of all chunks, two chunks per word
         const int64_t tile = blockIdx.x / L.chunks, c = blockIdx.x % L.chunks, r = tile * 128 + threadIdx.x;
@@ -208,6 +222,30 @@ __global__ void __launch_bounds__(128) unpack_w_kernel(const uint8_t* blob, int6
             if (codes8) *reinterpret_cast<uint4*>(codes8 + r * K + kb * 16) = b8 ? make_uint4(slot[i].x, slot[i].y, hi[i].x, hi[i].y) : make_uint4(0u, 0u, 0u, 0u);
         }
     }
+}
+
+// Where the host reads a header: pinned memory and an event of the calling thread on the current device, made once and given back when the thread
+// ends (through pageable memory the copy alone takes 8 us longer)
+struct HeaderCopy {
+    fgmp_packed_header* header = nullptr;
+    cudaEvent_t done = nullptr;
+    HeaderCopy() = default;
+    HeaderCopy(const HeaderCopy&) = delete;
+    ~HeaderCopy()
+    {
+        if (done) cudaEventDestroy(done);
+        if (header) cudaFreeHost(header);
+    }
+};
+HeaderCopy* header_copy()
+{
+    static thread_local HeaderCopy of_device[64];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+    HeaderCopy* c = &of_device[dev];
+    if (!c->header && cudaHostAlloc(reinterpret_cast<void**>(&c->header), sizeof(fgmp_packed_header), cudaHostAllocDefault) != cudaSuccess) { c->header = nullptr; return nullptr; }
+    if (!c->done && cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming) != cudaSuccess) { c->done = nullptr; return nullptr; }
+    return c;
 }
 
 // mean of squares per column of a bf16 matrix; thread per column, rows in order (one fp32 multiply
@@ -318,13 +356,19 @@ extern "C" fgmp_status fgmp_activation_scores(const void* X_bf16, int64_t ldx, c
                                               int64_t M, int64_t K, fgmp_scales sc, fgmp_score_mode sm,
                                               float* scores, void* cuda_stream)
 {
+    return fgmp_activation_scores_clear(X_bf16, ldx, fisher_chan, M, K, sc, sm, scores, nullptr, 0, cuda_stream);
+}
+
+fgmp_status fgmp_activation_scores_clear(const void* X_bf16, int64_t ldx, const float* fisher_chan, int64_t M, int64_t K, fgmp_scales sc,
+                                         fgmp_score_mode sm, float* scores, uint32_t* clear, int clear_words, void* cuda_stream)
+{
     fgmp_status st = check_act_args(X_bf16, ldx, fisher_chan, M, K, sc, (int)sm);
     if (st != FGMP_OK) return st;
     if (!scores) return FGMP_ERR_INVALID_ARG;
     if ((st = fgmp_require_sm100()) != FGMP_OK) return st;
     cudaStream_t s = (cudaStream_t)cuda_stream;
     ActParams p = make_act_params(X_bf16, ldx, fisher_chan, M, K, sc, 0.f);
-    p.scores = scores;
+    p.scores = scores; p.clear = clear; p.clear_words = clear_words;
     FGMP_LAUNCH(FGMP_K_ACT_SCORES, s, st = sm == FGMP_SCORE_LP_ERROR ? launch_quant<0, true>(p, s) : launch_quant<1, true>(p, s));
     return st == FGMP_OK ? fgmp_launch_status() : st;
 }
@@ -337,20 +381,15 @@ extern "C" fgmp_status fgmp_unpack(const void* packed, int64_t rows, int64_t K, 
     fgmp_status st;
     if ((st = fgmp_require_sm100()) != FGMP_OK) return st;
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    // the blob says what it is: activations keep planes, weights keep unit records
-    fgmp_packed_header h;
-    if (cudaMemcpyAsync(&h, packed, sizeof(h), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess) return FGMP_ERR_CUDA;
-    if (h.magic != FGMP_MAGIC || h.version != FGMP_LAYOUT_VERSION || h.rows != rows || h.K != K || h.error != 0) return FGMP_ERR_INVALID_ARG;
-    if (h.kind == 1) {
-        const PackedLayout L = fgmp_layout(rows, K, 1, 0);
-        FGMP_LAUNCH(FGMP_K_UNPACK, s, unpack_w_kernel<<<(unsigned)L.units, 128, 0, s>>>((const uint8_t*)packed, rows, K, codes4, codes8, scales, mask));
-    } else {
-        int64_t nblk = rows * (K / 16);
-        int grid = (int)((nblk + 255) / 256 < 148 * 16 ? (nblk + 255) / 256 : 148 * 16);
-        FGMP_LAUNCH(FGMP_K_UNPACK, s, unpack_kernel<<<grid, 256, 0, s>>>((const uint8_t*)packed, rows, K, codes4, codes8, scales, mask));
-    }
-    return fgmp_launch_status();
+    // The host reads the header while the kernel works: what it refuses the kernel has not touched.
+    HeaderCopy* copy = header_copy();
+    if (!copy) return FGMP_ERR_CUDA;
+    if (cudaMemcpyAsync(copy->header, packed, sizeof(fgmp_packed_header), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        cudaEventRecord(copy->done, s) != cudaSuccess) return FGMP_ERR_CUDA;
+    FGMP_LAUNCH(FGMP_K_UNPACK, s, unpack_kernel<<<(unsigned)fgmp_layout(rows, K, 1, 0).units, 128, 0, s>>>((const uint8_t*)packed, rows, K, codes4, codes8, scales, mask));
+    if ((st = fgmp_launch_status()) != FGMP_OK) return st;
+    if (cudaEventSynchronize(copy->done) != cudaSuccess) return FGMP_ERR_CUDA;
+    return unpackable(*copy->header, rows, K) ? FGMP_OK : FGMP_ERR_INVALID_ARG;
 }
 
 extern "C" fgmp_status fgmp_channel_mean_sq(const void* X_bf16, int64_t ldx, int64_t rows, int64_t K,

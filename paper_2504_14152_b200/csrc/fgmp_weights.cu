@@ -41,7 +41,7 @@ struct SelectState {
     uint32_t use_eq;         // 0: none of the blocks equal to tau is taken, 1: the first need_eq of them, 2: all
     unsigned long long need_eq;
     unsigned long long n_fp8;
-    float next_below;        // calibration: largest score strictly below tau
+    uint32_t next_below;     // calibration: largest score of a prefix below the threshold's, as fp32 bits
     uint32_t pad1;
 };
 
@@ -55,7 +55,7 @@ __global__ void state_init_kernel(SelectState* st, float s4_given, unsigned long
     if (threadIdx.x == 0) {
         st->arrived = 0;
         st->amax_bits = 0; st->s4 = s4_given; st->prefix = 0; st->krem = k; st->tau = tau;
-        st->use_eq = 0; st->need_eq = 0; st->n_fp8 = 0; st->next_below = 0.f;
+        st->use_eq = 0; st->need_eq = 0; st->n_fp8 = 0; st->next_below = 0;
     }
 }
 
@@ -337,23 +337,42 @@ __global__ void __launch_bounds__(SCORE_THREADS, SCORE_BLOCKS) w_score_kernel(co
 // the scores each; the last thread block of a pass picks the digit, so that a pass is one launch.  (Four digits of eight bits
 // and a launch for each pick took 200 us for a packing and a calibration, of which the shared counters' conflicts most: the
 // upper eight bits of the scores take a few values only.)
-__global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_t B, int pass, SelectState* st)
+// tau_out, of a calibration (one launch and one pass less than looking for the neighbour behind it; with the state cleared by the kernel that makes the scores
+// a calibration of 512 x 4096 takes 15.8 us, 20.4 before): midway between the k-th largest score and the largest below it.  That is in the last pass's bins, or else the largest that the
+// pass has seen of smaller prefix.
+__global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_t B, int pass, unsigned long long k, SelectState* st, float* tau_out)
 {
-    __shared__ uint32_t h[SEL_BINS];
+    __shared__ uint32_t h[SEL_BINS], s_max[16], s_bin;
     __shared__ unsigned long long s_warp[16];
-    chain_begin();
+    chain_begin(!(pass == 2 && tau_out));
     const int bits = pass == 2 ? 10 : 11, shift = pass == 0 ? 21 : pass == 1 ? 10 : 0;
     for (int i = threadIdx.x; i < SEL_BINS; i += 512) h[i] = 0;
     __syncthreads();
     const uint32_t prefix = st->prefix, low = (1u << bits) - 1u;
     const int64_t stride = (int64_t)gridDim.x * 512;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t below = 0;
     for (int64_t b = (int64_t)blockIdx.x * 512 + threadIdx.x; b < B; b += 4 * stride) {
         uint32_t u[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) u[i] = b + i * stride < B ? __float_as_uint(__ldg(scores + b + i * stride)) : 0u;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < 4; ++i) {
             if (b + i * stride < B && (pass == 0 || (u[i] >> (shift + bits)) == prefix)) atomicAdd(&h[(u[i] >> shift) & low], 1u);
+            if ((u[i] >> 10) < prefix) below = max(below, u[i]);
+        }
+    }
+    const auto block_max = [&](uint32_t x) {                 // for thread 0
+        x = __reduce_max_sync(0xffffffffu, x);
+        __syncthreads();
+        if (lane == 0) s_max[w] = x;
+        __syncthreads();
+        for (int i = 0; threadIdx.x == 0 && i < 16; ++i) x = max(x, s_max[i]);
+        return x;
+    };
+    if (pass == 2 && tau_out) {
+        below = block_max(below);
+        if (threadIdx.x == 0) atomicMax(&st->next_below, below);
     }
     __syncthreads();
     for (int i = threadIdx.x; i < SEL_BINS; i += 512)
@@ -364,11 +383,10 @@ __global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_
     unsigned long long sum = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) { own[i] = *reinterpret_cast<volatile uint32_t*>(&st->hist[4 * threadIdx.x + i]); sum += own[i]; }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     unsigned long long from = sum;                       // sums over the threads t, t + 1, ... : of the warp, then of all
     for (int o = 1; o < 32; o <<= 1) { const unsigned long long y = __shfl_down_sync(0xffffffffu, from, o); if (lane + o < 32) from += y; }
     if (lane == 0) s_warp[w] = from;
-    const unsigned long long krem = st->krem;            // (before anybody changes it below)
+    const unsigned long long krem = pass == 0 ? k : st->krem;      // (before anybody changes it below)
     __syncthreads();
     for (int k = w + 1; k < 16; ++k) from += s_warp[k];
     unsigned long long above = from - sum;
@@ -381,85 +399,64 @@ __global__ void __launch_bounds__(512) select_kernel(const float* scores, int64_
             st->tau = __uint_as_float((prefix << bits) | (uint32_t)(4 * threadIdx.x + i));
             st->need_eq = krem - above;                  // of the blocks equal to tau, take this many
             st->use_eq = krem - above == own[i] ? 2u : 1u;
+            s_bin = (uint32_t)(4 * threadIdx.x + i);
         }
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) st->hist[4 * threadIdx.x + i] = 0;
+    if (pass != 2 || !tau_out) return;
+    __syncthreads();
+    uint32_t next = 0;                                       // the largest bin in use below the threshold's, plus one
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i) if (own[i] && 4 * threadIdx.x + i < s_bin) next = 4 * threadIdx.x + i + 1;
+    next = block_max(next);
+    if (threadIdx.x == 0) {
+        const float tau = __uint_as_float((prefix << bits) | s_bin);
+        uint32_t lower = next ? (prefix << bits) | (next - 1u) : *reinterpret_cast<volatile uint32_t*>(&st->next_below);
+        if (tau != tau) lower = 0;                           // (nothing is below NaN)
+        // if fp32 cannot separate the two, the lower neighbour itself (score > tau still selects the top k)
+        const float y = __uint_as_float(lower), t = __fmul_rn(0.5f, __fadd_rn(tau, y));
+        *tau_out = (t < tau && t >= y) ? t : y;
+    }
 }
 
-// Threshold of a calibration: midway between the k-th largest score and the largest below it (all_or_none: see the callers)
-__global__ void __launch_bounds__(512) calib_finish_kernel(const float* scores, int64_t B, SelectState* st, float* tau_out, int all_or_none)
+// Thresholds that no score decides: k = 0, nothing exceeds +inf; k = all
+__global__ void tau_kernel(float* tau_out, float tau)
 {
     chain_begin(false);
-    if (all_or_none) {
-        // k = 0: nothing exceeds +inf; k = all
-        if (blockIdx.x == 0 && threadIdx.x == 0) *tau_out = all_or_none == 1 ? __int_as_float(0x7f800000) : -1.0f;
-        return;
-    }
-    const float tau = st->tau;
-    uint32_t m = 0;
-    const int64_t stride = (int64_t)gridDim.x * 512;
-    for (int64_t b = (int64_t)blockIdx.x * 512 + threadIdx.x; b < B; b += 4 * stride) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float s = b + i * stride < B ? __ldg(scores + b + i * stride) : 0.f;
-            if (s < tau) m = max(m, __float_as_uint(s));
-        }
-    }
-    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(reinterpret_cast<uint32_t*>(&st->next_below), m);
-    if (last_block(&st->arrived) && threadIdx.x == 0) {
-        // if fp32 cannot separate the two, the lower neighbour itself (score > tau still selects the top k)
-        const float below = *reinterpret_cast<volatile float*>(&st->next_below), t = __fmul_rn(0.5f, __fadd_rn(tau, below));
-        *tau_out = (t < tau && t >= below) ? t : below;
-    }
+    *tau_out = tau;
 }
 
 // ------------------------------------------------------------ mask, prefix sums, emission
-// per mask word: how many of its blocks have score == tau (needed only if some of them are taken and some are not)
-__global__ void w_eqcount_kernel(const float* scores, int64_t N, int64_t KB, int64_t MW, const SelectState* st, uint32_t* cnt)
+// Where some of the blocks with score == tau are taken and some are not: how many there are per mask word, and by the last thread block the
+// exclusive sums of these counts.
+__global__ void __launch_bounds__(1024) w_eqscan_kernel(const float* scores, int64_t N, int64_t KB, int64_t MW, SelectState* st, uint32_t* cnt, uint32_t* out)
 {
     chain_begin();
     if (st->use_eq != 1) return;
     const float tau = st->tau;
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t nw = N * MW;
-    for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw; w += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    for (int64_t w = ((int64_t)blockIdx.x * 1024 + threadIdx.x) >> 5; w < nw; w += (int64_t)gridDim.x * 32) {
         int64_t n = w / MW, kb = (w % MW) * 32 + lane;
         bool eq = kb < KB && scores[n * KB + kb] == tau;
         uint32_t bal = __ballot_sync(0xffffffffu, eq);
         if (lane == 0) cnt[w] = __popc(bal);
     }
-}
-
-// exclusive prefix sum of n uint32 by one CTA of 1024 threads
-// (of the counts that w_eqcount_kernel has left, where it has)
-__global__ void __launch_bounds__(1024) scan_kernel(const uint32_t* in, uint32_t* out, int64_t n, const SelectState* st)
-{
-    chain_begin();
-    if (st->use_eq != 1) return;
+    if (!last_block(&st->arrived)) return;
     __shared__ uint32_t warp_sums[32];
-    __shared__ unsigned long long carry_s;
-    if (threadIdx.x == 0) carry_s = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int64_t base = 0; base < n; base += 1024) {
-        int64_t i = base + threadIdx.x;
-        uint32_t x = i < n ? in[i] : 0;
+    unsigned long long carry = 0;
+    for (int64_t base = 0; base < nw; base += 1024) {
+        const int64_t i = base + threadIdx.x;
+        const uint32_t x = i < nw ? __ldcg(cnt + i) : 0u;
         uint32_t incl = x;
-        for (int o = 1; o < 32; o <<= 1) { uint32_t y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
+        for (int o = 1; o < 32; o <<= 1) { const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o); if (lane >= o) incl += y; }
         if (lane == 31) warp_sums[wid] = incl;
         __syncthreads();
-        if (wid == 0) {
-            uint32_t s = warp_sums[lane], si = s;
-            for (int o = 1; o < 32; o <<= 1) { uint32_t y = __shfl_up_sync(0xffffffffu, si, o); if (lane >= o) si += y; }
-            warp_sums[lane] = si - s;       // exclusive warp offsets
-        }
-        __syncthreads();
-        unsigned long long carry = carry_s;
-        if (i < n) out[i] = (uint32_t)(carry + warp_sums[wid] + incl - x);
-        __syncthreads();
-        if (threadIdx.x == 1023) carry_s = carry + warp_sums[31] + incl;
+        uint32_t before = 0, all = 0;
+        for (int k = 0; k < 32; ++k) { const uint32_t y = warp_sums[k]; before += k < wid ? y : 0u; all += y; }
+        if (i < nw) out[i] = (uint32_t)(carry + before + incl - x);
+        carry += all;
         __syncthreads();
     }
 }
@@ -549,8 +546,10 @@ __global__ void __launch_bounds__(128) w_mask_kernel(const __grid_constant__ Mas
 
 // Writes the record of one unit (codes and microscales of its NVFP4 blocks, the first halves of its FP8
 // blocks, the running counts of FP8 blocks by row) and the list of its FP8 blocks (rows, second halves).  One CTA
-// of 128 threads per unit.
-__global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw8, int ratio, float s8_given, const SelectState* st,
+// of T threads per unit: 128, or 256 where there are few units (a packing of 512 x 1024, 32 units, 40.6 -> 37.9 us, of 3600 x 2048, 232 units, 77.7 -> 75.6; of
+// 4096 x 4096, 512 units, 128.8 and 130.7).
+template <int T>
+__global__ void __launch_bounds__(T) w_emit_kernel(const uint4* W, int64_t ldw8, int ratio, float s8_given, const SelectState* st,
                                                      const uint8_t* sc_in, uint8_t* blob, PackedLayout L)
 {
     __shared__ UnitScratch sc;
@@ -561,7 +560,7 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
     const float s4 = st->s4;
     const float s8 = s8_given > 0.f ? s8_given : __fmul_rn(s4, __int_as_float((127 + ratio) << 23));
     const float inv8 = inverse_scale(s8);
-    const uint32_t cnt = sc.init(reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x]);
+    const uint32_t cnt = sc.init(threadIdx.x < 128 ? reinterpret_cast<const uint16_t*>(blob + L.off_mask)[unit * 128 + threadIdx.x] : 0u);
     uint8_t* rec = blob + L.off_rec + (size_t)unit * REC_BYTES;
     uint8_t* list = blob + L.off_ovf + (size_t)uptr[unit] * 16;
     uint32_t* entries = reinterpret_cast<uint32_t*>(list);
@@ -569,19 +568,19 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
     if (threadIdx.x < 64)                                      // FP8 blocks before every eighth row, then padding
         reinterpret_cast<uint16_t*>(rec + REC_KBSTART)[threadIdx.x] = threadIdx.x < 16 ? sc.base[8 * threadIdx.x] : threadIdx.x == 16 ? (uint16_t)cnt : (uint16_t)0;
     if (fits) {                                                // padding behind the entries and behind the last half
-        for (uint32_t i = cnt + threadIdx.x; i < fgmp_list_halves_offset(cnt) / 4; i += 128) entries[i] = 0;
+        for (uint32_t i = cnt + threadIdx.x; i < fgmp_list_halves_offset(cnt) / 4; i += T) entries[i] = 0;
         if (threadIdx.x == 0 && (cnt & 1u)) *reinterpret_cast<uint2*>(halves + (size_t)cnt * 8) = make_uint2(0u, 0u);
     }
     const int j = threadIdx.x & 15;
     const int64_t kb = c * 16 + j;
     // four blocks of the thread in flight (4096 x 4096: 15 us, 23 one at a time)
 #pragma unroll 1
-    for (int i0 = 0; i0 < 16; i0 += 4) {
+    for (int i0 = 0; i0 < 2048 / T; i0 += 4) {
         uint4 x[4][2];
         uint32_t sc_code[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int64_t n = tile * 128 + (threadIdx.x >> 4) + 8 * (i0 + i);
+            const int64_t n = tile * 128 + (threadIdx.x >> 4) + T / 16 * (i0 + i);
             x[i][0] = x[i][1] = make_uint4(0u, 0u, 0u, 0u); sc_code[i] = 0;
             if (n < L.rows && kb < L.KB) {
                 const uint4* wp = W + n * ldw8 + kb * 2;
@@ -590,7 +589,7 @@ __global__ void __launch_bounds__(128) w_emit_kernel(const uint4* W, int64_t ldw
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int row = (threadIdx.x >> 4) + 8 * (i0 + i);
+            const int row = (threadIdx.x >> 4) + T / 16 * (i0 + i);
             uint2 slot = make_uint2(0u, 0u);
             uint32_t scale = 0;
             if (tile * 128 + row < L.rows && kb < L.KB) {
@@ -652,23 +651,19 @@ void run_scores(fgmp_score_mode sm, fgmp_clip_mode cm, int64_t B, cudaStream_t s
                                       : (clip ? launch_score<1, true>(B, s, args...) : launch_score<1, false>(B, s, args...)));
 }
 
-// three-pass radix select for the k-th largest of scores[0..B)
-void run_select(const float* scores, int64_t B, SelectState* st, cudaStream_t s)
+// three-pass radix select for the k-th largest of scores[0..B); the state is zero but for what the caller needs of it
+void run_select(const float* scores, int64_t B, int64_t k, SelectState* st, float* tau_out, cudaStream_t s)
 {
     const int g = grid_for(B, 512 * 4, 1);      // (a block ends with an atomic per bin in use: few blocks)
-    for (int pass = 0; pass < 3; ++pass) FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(select_kernel, g, 512, s, scores, B, pass, st));
+    for (int pass = 0; pass < 3; ++pass)
+        FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(select_kernel, g, 512, s, scores, B, pass, (unsigned long long)k, st, tau_out));
 }
 
-// the threshold from the scores (k of B blocks above it)
+// the threshold from the scores (k of B blocks above it), the state being zero
 fgmp_status run_calibration(const float* scores, int64_t B, int64_t k, SelectState* st, float* tau_out, cudaStream_t s)
 {
-    if (k == 0 || k == B) {
-        FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(calib_finish_kernel, 1, 512, s, scores, B, st, tau_out, k == 0 ? 1 : 2));
-    } else {
-        FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, 1.0f, (unsigned long long)k, 0.f));
-        run_select(scores, B, st, s);
-        FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(calib_finish_kernel, grid_for(B, 512 * 4, 2), 512, s, scores, B, st, tau_out, 0));
-    }
+    if (k == 0 || k == B) { FGMP_LAUNCH(FGMP_K_SELECT, s, chain_launch(tau_kernel, 1, 1, s, tau_out, k == 0 ? INFINITY : -1.0f)); }
+    else run_select(scores, B, k, st, tau_out, s);
     return fgmp_launch_status();
 }
 
@@ -740,18 +735,17 @@ extern "C" fgmp_status fgmp_quantize_weights(const void* W_bf16, int64_t ldw, co
     if (sc.scale_fp4 == 0.f)
         FGMP_LAUNCH(FGMP_K_W_AMAX, s, chain_launch(w_amax_kernel, grid_for(N, 4, 8), 256, s, W, ldw / 8, N, (uint32_t)(K / 8), st));
     run_scores(sm, cm, B, s, W, ldw / 8, fisher_elem, ldf, (uint32_t)B, (uint32_t)KB, ratio, s8_given, (const SelectState*)st, sc_tmp, scores);
-    const int gw = grid_for(NW * 32, 256, 8);
     if (fraction_mode && k > 0) {
-        run_select(scores, B, st, s);
-        FGMP_LAUNCH(FGMP_K_W_MASK, s, chain_launch(w_eqcount_kernel, gw, 256, s, scores, N, KB, MW, st, tmp_a));
-        FGMP_LAUNCH(FGMP_K_SCAN, s, chain_launch(scan_kernel, 1, 1024, s, tmp_a, tmp_b, NW, st));
+        run_select(scores, B, k, st, nullptr, s);
+        FGMP_LAUNCH(FGMP_K_SCAN, s, chain_launch(w_eqscan_kernel, grid_for(NW * 32, 1024, 2), 1024, s, scores, N, KB, MW, st, tmp_a, tmp_b));
     }
     MaskParams mp;
     mp.scores = scores; mp.eqprefix = tmp_b; mp.mask16 = reinterpret_cast<uint16_t*>(blob + L.off_mask); mp.list_steps = tmp_a;
     mp.uptr = reinterpret_cast<uint32_t*>(blob + L.off_uptr); mp.header = reinterpret_cast<fgmp_packed_header*>(blob); mp.st = st;
     mp.L = L; mp.room_steps = room_steps; mp.ratio = ratio; mp.s8_given = s8_given;
     FGMP_LAUNCH(FGMP_K_W_MASK, s, chain_launch(w_mask_kernel, (unsigned)L.units, 128, s, mp));
-    FGMP_LAUNCH(FGMP_K_W_EMIT, s, chain_launch(w_emit_kernel, (unsigned)L.units, 128, s, W, ldw / 8, ratio, s8_given, st, sc_tmp, blob, L));
+    const auto emit = [&](auto kernel, int threads) { chain_launch(kernel, (unsigned)L.units, threads, s, W, ldw / 8, ratio, s8_given, st, sc_tmp, blob, L); };
+    FGMP_LAUNCH(FGMP_K_W_EMIT, s, L.units <= 2 * fgmp_sm_count() ? emit(w_emit_kernel<256>, 256) : emit(w_emit_kernel<128>, 128));
     FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(w_finish_kernel, 1, 1, s, reinterpret_cast<fgmp_packed_header*>(blob), st, fraction_mode ? 1 : 0, tau, tau_eff_out));
     return fgmp_launch_status();
 }
@@ -771,7 +765,8 @@ extern "C" fgmp_status fgmp_calibrate_tau(const void* X_bf16, int64_t ldx, const
     SelectState* st = reinterpret_cast<SelectState*>(ws);
     float* scores = reinterpret_cast<float*>(ws + STATE_BYTES);
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    fgmp_status stt = fgmp_activation_scores(X_bf16, ldx, fisher_chan, M, K, sc, sm, scores, cuda_stream);
+    fgmp_status stt = fgmp_activation_scores_clear(X_bf16, ldx, fisher_chan, M, K, sc, sm, scores, reinterpret_cast<uint32_t*>(st), sizeof(SelectState) / 4,
+                                                   cuda_stream);
     if (stt != FGMP_OK) return stt;
     int64_t k = (int64_t)floor(fp8_fraction * (double)B + 0.5);
     if (k > B) k = B;
@@ -839,5 +834,6 @@ extern "C" fgmp_status fgmp_global_tau(const float* const* score_arrays, const i
     }
     int64_t k = (int64_t)floor(fp8_fraction * (double)B + 0.5);
     if (k > B) k = B;
+    FGMP_LAUNCH(FGMP_K_W_AUX, s, chain_launch(state_init_kernel, 1, 1024, s, st, 1.0f, 0ull, 0.f));
     return run_calibration(scores, B, k, st, tau_out, s);
 }

@@ -264,6 +264,72 @@ def test_clip_search_at_the_edges_of_its_bounds(fg, scale):
     compare_packed(fg, fg.quantize_weights(w.cuda(), f.cuda(), scale_fp4=scale, clip_mode=1, fp8_fraction=0.1), q, None, f"scale {scale}")
 
 
+# The threshold of a calibration against the sorted scores: the next one below it of its own group of the last pass, of another group, equal to it, none, and
+# apart by one step of fp32; every block, none, and one
+@pytest.mark.parametrize("spread", [0.0, 0.01, 3.0])
+def test_calibration_against_sorted_scores(fg, spread):
+    g = torch.Generator().manual_seed(103)
+    x = (torch.randn(40, 320, generator=g) * torch.exp(spread * torch.randn(40, 1, generator=g))).to(torch.bfloat16)
+    x[8:12] = x[0:4]                                     # equal scores
+    x[30:36] = 0.0
+    x, f = x.cuda(), torch.ones(320, device="cuda")
+    scores = fg.activation_scores(x, f, scale_fp4=1e-3).flatten()
+    order = scores.sort(descending=True).values
+    for k in [0, 1, 2, 50, 333, 650, 679, 680, 681, 799, 800]:
+        tau = fg.calibrate_tau(x, f, scale_fp4=1e-3, fp8_fraction=k / 800)
+        if k in (0, 800):
+            want = torch.tensor(float("inf") if k == 0 else -1.0)
+        else:
+            kth = order[k - 1]
+            lower = order[order < kth]
+            below = lower[0] if lower.numel() else torch.zeros((), device="cuda")
+            mid = 0.5 * (kth + below)
+            want = mid if mid < kth and mid >= below else below
+        assert tau.item() == want.item(), (k, tau.item(), want.item())
+
+
+# More equal scores than are taken: the first of them in row-major order, over more mask words than a thread block has threads
+@pytest.mark.parametrize("N,K,frac", [(600, 2048, 0.3), (129, 320, 0.5), (5000, 576, 0.001)])
+def test_equal_scores_are_taken_in_order(fg, N, K, frac):
+    w, f = torch.full((N, K), 0.02, dtype=torch.bfloat16), torch.ones(N, K)
+    w[3, :64], w[N // 2, 16:32] = 0.05, 0.0
+    q = oracle.quantize_weights(gi.bf16_bits(w), f.numpy(), scale_fp4=3e-4, clip=False, fp8_fraction=frac)
+    compare_packed(fg, fg.quantize_weights(w.cuda(), f.cuda(), scale_fp4=3e-4, clip_mode=0, fp8_fraction=frac), q, None, "equal scores")
+
+
+# What unpacking refuses it leaves alone, whatever kind of tensor it is, and from several threads at once each gets its own answer
+def test_unpacking_refuses_without_touching_and_in_threads(fg):
+    w, a = draw_weights(fg, 300, 320, 104), draw_acts(fg, 30, 320, 105)
+    L = fg.binding._load()
+    for t in (w, a):
+        blob = t.blob.clone()
+        blob[4] += 1                                     # another layout version
+        bad = fg.binding._alloc_aligned(blob.numel(), "cuda").copy_(blob)
+        outs = [torch.full((t.rows * 320,), 7, dtype=torch.uint8, device="cuda") for _ in range(4)]
+        assert L.fgmp_unpack(bad.data_ptr(), t.rows, 320, *[o.data_ptr() for o in outs], torch.cuda.current_stream().cuda_stream) == -1
+        torch.cuda.synchronize()
+        assert all((o == 7).all() for o in outs)
+    want, wrong = [x.clone() for x in fg.unpack(w)], []
+
+    def work(good):
+        with torch.cuda.stream(torch.cuda.Stream()):
+            for _ in range(20):
+                try:
+                    got = fg.unpack(fg.PackedTensor(w.blob, 300 if good else 301, 320, 1))
+                    torch.cuda.current_stream().synchronize()
+                    if not good or any(not torch.equal(x, y) for x, y in zip(got, want)):
+                        wrong.append(good)
+                except fg.FgmpError:
+                    if good:
+                        wrong.append(good)
+
+    torch.cuda.synchronize()
+    threads = [threading.Thread(target=work, args=(i % 2 == 0,)) for i in range(4)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    assert not wrong
+
+
 # A workspace sized for the largest batch serves the smaller ones, among them those whose own size would be larger (the parts of shared
 # tiles take most at middling batches); one byte less than two planes of fp16 is refused.
 @pytest.mark.parametrize("N,K,largest", [(2048, 2048, 1024), (4096, 4096, 817), (1024, 320, 1000)])
