@@ -4,9 +4,9 @@
 // Thread mapping: a warp owns 32 consecutive block columns (one mask word, produced with a ballot) and walks down a few rows, a
 // thread per column, so the 16 per-channel Fisher weights stay in registers; the next row is loaded while one is worked on.
 //
-// Bound by instruction issue from a few hundred rows on (rounding to both formats and back, the score in element order), by the launch
-// below that.  2048 x 5120 takes 10.4 us (2.8 TB/s) and 8192 x 8192 41.5 us; with blocks of 256 columns
-// and one load at a time it was 16.5 and 45 us.  Asking for more resident warps (64 registers) is slower, 13.8 us for the former.
+// Bound by instruction issue from a few hundred rows on (rounding to both formats and back, the score in element order: 250 instructions for 32 blocks), by the
+// launch below that.  Calls in a row on three inputs: 1024 x 4096 4.45 us, 2048 x 5120 8.4 (3.3 TB/s), 8192 x 8192 47.4 (3.8); with addresses worked out anew
+// for every row, and up to eight rows a warp in whatever number of rounds, 5.8, 9.2 and 49.5.  Asking for more resident warps (64 registers) is slower.
 #include "fgmp_common.cuh"
 #include "fgmp_host.h"
 #include <cuda_bf16.h>
@@ -15,6 +15,7 @@
 namespace {
 
 constexpr int QA_THREADS = 128;
+constexpr int QA_RESIDENT = 24;          // warps that an SM holds, by their 80 registers
 
 struct ActParams {
     const uint4* X; int64_t ldx8;        // row stride in 16-byte units
@@ -70,6 +71,13 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
 
     uint4 na = make_uint4(0u, 0u, 0u, 0u), nb = na;
     const uint4* xp = p.X + m0 * p.ldx8 + kb * 2;
+    // (where the row's output goes, moved on from row to row)
+    uint8_t* c4p = p.codes4 + (m0 * p.K) / 2 + kb * 8;
+    uint8_t* c8p = p.codes8 + m0 * p.K + kb * 16;
+    uint32_t* mp = p.mask + m0 * p.MW + word;
+    const uint32_t sf_tile = (uint32_t)(p.K >> 6) * 512u;            // of 128 rows
+    uint8_t* sfp = p.sf + (size_t)(m0 >> 7) * sf_tile + (size_t)(kb >> 2) * 512 + (kb & 3);
+    uint32_t in_tile = (uint32_t)m0 & 127u;
     if (active) { na = __ldcs(xp); nb = __ldcs(xp + 1); }
 #pragma unroll 1
     for (int64_t m = m0; m < m1; ++m) {
@@ -101,7 +109,7 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
                         float dq8[16];
                         block_fp8(v, p.inv8, p.s8, c8, dq8);
                     }
-                    *reinterpret_cast<uint4*>(p.codes8 + m * p.K + kb * 16) = make_uint4(c8[0], c8[1], c8[2], c8[3]);
+                    *reinterpret_cast<uint4*>(c8p) = make_uint4(c8[0], c8[1], c8[2], c8[3]);
                     c4[0] = 0; c4[1] = 0; sc = 0;
                 }
                 if (p.arec) {
@@ -132,13 +140,15 @@ __global__ void __launch_bounds__(QA_THREADS) quant_act_kernel(ActParams p)
                     *reinterpret_cast<uint2*>(rec + AREC_A4 + fgmp_rec_w4_offset((uint32_t)m, j)) = make_uint2(c4[0], c4[1]);
                     rec[AREC_SF + (uint32_t)m * 16 + j] = (uint8_t)sc;
                 }
-                *reinterpret_cast<uint2*>(p.codes4 + (m * p.K) / 2 + kb * 8) = make_uint2(c4[0], c4[1]);
-                p.sf[fgmp_sf_offset(m, kb, p.K)] = (uint8_t)sc;
+                *reinterpret_cast<uint2*>(c4p) = make_uint2(c4[0], c4[1]);
+                sfp[(in_tile & 31u) * 16u + (in_tile >> 5) * 4u] = (uint8_t)sc;
             }
         }
         if (!SCORE_ONLY) {
             const uint32_t bits = __ballot_sync(0xffffffffu, is8);
-            if ((threadIdx.x & 31) == 0) p.mask[m * p.MW + word] = bits;
+            if ((threadIdx.x & 31) == 0) *mp = bits;
+            c4p += p.K >> 1; c8p += p.K; mp += p.MW;
+            if (++in_tile == 128u) { in_tile = 0; sfp += sf_tile; }
         }
     }
 }
@@ -317,10 +327,10 @@ ActParams make_act_params(const void* X, int64_t ldx, const float* fisher, int64
     p.tau = tau;
     p.ratio = sc.fp8_log2_ratio;
     p.r8 = ldexpf(1.0f, sc.fp8_log2_ratio);
-    // rows per warp: one while there are fewer warps than the machine holds (28 per SM), up to eight so that the Fisher weights
-    // are loaded rarely (8192 x 8192: 43 us with up to eight, 46 with four, 53 with two, 70 with one)
-    const int64_t words = M * p.MW, fit = words / ((int64_t)fgmp_sm_count() * 28);
-    p.rows_per_warp = (int)(fit < 1 ? 1 : fit > 8 ? 8 : fit);
+    // Rows per warp: so many that the warps are as many as the chip holds at once, or a whole number of times as many where that would be more than 32.  (1024 x
+    // 4096: two rows for each of 4096 warps, 3552 at once, 5.7 us; three rows 4.45.)
+    const int64_t words = M * p.MW, fit = (int64_t)fgmp_sm_count() * QA_RESIDENT, rounds = (words + 32 * fit - 1) / (32 * fit);
+    p.rows_per_warp = (int)((words + rounds * fit - 1) / (rounds * fit));
     p.groups = (uint32_t)((M + p.rows_per_warp - 1) / p.rows_per_warp);
     return p;
 }
