@@ -91,9 +91,10 @@ __device__ __forceinline__ void umma_f16_ta(uint32_t d_tmem, uint32_t a_tmem, ui
                  "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
+template <bool CL = false>
 __device__ __forceinline__ uint32_t unit_begin(const MixedPlan& pl, uint32_t cta)
 {
-    if (pl.cluster) { const uint32_t tile = cta / pl.cluster; return tile * pl.chunks + (cta - tile * pl.cluster) * pl.chunks / pl.cluster; }
+    if (CL) { const uint32_t tile = cta / pl.cluster; return tile * pl.chunks + (cta - tile * pl.cluster) * pl.chunks / pl.cluster; }
     return (cta * pl.span + min(cta, pl.rest)) * pl.quantum;
 }
 __device__ __forceinline__ uint32_t cta_of(const MixedPlan& pl, uint32_t u)
@@ -251,8 +252,8 @@ __device__ __forceinline__ void mixed_epilogue(const MixedParams& p, uint32_t tm
     }
 }
 
-// QUANT: the next layer's activation quantizer in the epilogue instead of Y.  KS: MixedPlan::ks.
-template <bool QUANT, uint32_t KS>
+// QUANT: the next layer's activation quantizer in the epilogue instead of Y.  KS: MixedPlan::ks.  CL: clusters that share a tile each.
+template <bool QUANT, uint32_t KS, bool CL>
 __global__ void __launch_bounds__(MX_THREADS, 1)
 mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ MixedParams p)
 {
@@ -280,7 +281,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     const uint32_t accf0 = dn0 + 8 * MAX_STEPS, acce0 = accf0 + 16;
     const uint32_t slot_col = pl.naccs * NT;             // tensor memory: accumulators of NT columns, then slots of 32 KS
 
-    const uint32_t u_begin = unit_begin(pl, blockIdx.x), u_end = unit_begin(pl, blockIdx.x + 1);
+    const uint32_t u_begin = unit_begin<CL>(pl, blockIdx.x), u_end = unit_begin<CL>(pl, blockIdx.x + 1);
     // steps (of KS times 64 elements) of a chunk, and of the last one: what of its last step lies beyond K is zeros
     constexpr uint32_t STEPS = 4 / KS;
     const uint32_t last_steps = ((uint32_t)(p.K / 64) - 4u * (C - 1u) + KS - 1u) / KS;
@@ -350,7 +351,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
         asm volatile("griddepcontrol.wait;" ::: "memory");
         // (Clusters: what follows comes up when this grid is done.  Before that its blocks would crowd on the few SMs that are left free: quantizer and call,
         // 30 x 1664 x 9728, 15.4 us, 18.4 with an early start.)
-        if (!pl.cluster) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (!CL) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     }
     // (The weights are dequantized before the kernel in front is done, as far as there are slots: only the tokens are its.)
     if (QUANT && blockIdx.x == 0 && threadIdx.x == 32 * W_EPI) {
@@ -517,7 +518,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
             if (++stage == WS) { stage = 0; phase ^= 1; }
             if (++c == C) c = 0;
         }
-    } else if (pl.cluster) {
+    } else if (CL) {
         mbar_wait_warp(accf0, 0, abort_flag, p.status, 8);       // (this CTA's products are done, and with them its reads of shared memory)
         tc_fence_after();
     } else {
@@ -525,7 +526,7 @@ mixed_kernel(const __grid_constant__ CUtensorMap tmB, const __grid_constant__ Mi
     }
 
     __syncthreads();
-    if (pl.cluster && !skip) {                           // (whatever has gone wrong in a CTA, all of the cluster come here)
+    if (CL && !skip) {                           // (whatever has gone wrong in a CTA, all of the cluster come here)
         const uint32_t rank = cluster_ctarank();
         const bool mine = warp >= W_EPI && warp < W_DEQ;
         cluster_sync();
@@ -774,7 +775,9 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     {
         std::lock_guard<std::mutex> lk(mx_mu);
         if (!mx_attr_set[dev]) {
-            for (const void* k : {(const void*)mixed_kernel<false, 1>, (const void*)mixed_kernel<false, 2>, (const void*)mixed_kernel<true, 1>, (const void*)mixed_kernel<true, 2>})
+            for (const void* k : {(const void*)mixed_kernel<false, 1, false>, (const void*)mixed_kernel<false, 2, false>, (const void*)mixed_kernel<true, 1, false>,
+                                  (const void*)mixed_kernel<true, 2, false>, (const void*)mixed_kernel<false, 1, true>, (const void*)mixed_kernel<false, 2, true>,
+                                  (const void*)mixed_kernel<true, 1, true>, (const void*)mixed_kernel<true, 2, true>})
                 if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MX_SMEM_LIMIT) != cudaSuccess) return FGMP_ERR_CUDA;
             mx_attr_set[dev] = true;
         }
@@ -806,7 +809,9 @@ fgmp_status fgmp_linear_mixed(const void* packed_acts, const void* packed_weight
     const bool quant = qn.codes4 != nullptr;
     cfg.gridDim = dim3(p.pl.grid); cfg.blockDim = dim3(MX_THREADS);
     cfg.dynamicSmemBytes = (size_t)p.pl.ring * p.pl.ks * (p.pl.n_tok > p.pl.n_half ? 2 : 1) * p.pl.n_half * 128 + (size_t)p.pl.wstages * WSTAGE + MX_FIXED + (quant ? MX_TURN : 0);
-    const auto kernel = quant ? (p.pl.ks == 2 ? mixed_kernel<true, 2> : mixed_kernel<true, 1>) : (p.pl.ks == 2 ? mixed_kernel<false, 2> : mixed_kernel<false, 1>);
+    const auto of = [&](auto one, auto two) { return p.pl.ks == 2 ? two : one; };
+    const auto kernel = p.pl.cluster ? (quant ? of(mixed_kernel<true, 1, true>, mixed_kernel<true, 2, true>) : of(mixed_kernel<false, 1, true>, mixed_kernel<false, 2, true>))
+                                     : (quant ? of(mixed_kernel<true, 1, false>, mixed_kernel<true, 2, false>) : of(mixed_kernel<false, 1, false>, mixed_kernel<false, 2, false>));
     FGMP_LAUNCH(FGMP_K_GEMM_MIXED, s, cudaLaunchKernelEx(&cfg, kernel, tmB, p));
     if (p.pl.split) {
         cfg.gridDim = dim3(p.pl.tiles, (p.pl.n_tok + 31) / 32); cfg.dynamicSmemBytes = 0;
