@@ -5,8 +5,8 @@
 // thread per column, so the 16 per-channel Fisher weights stay in registers; the next row is loaded while one is worked on.
 //
 // Bound by instruction issue from a few hundred rows on (rounding to both formats and back, the score in element order: 250 instructions for 32 blocks), by the
-// launch below that.  Calls in a row on three inputs: 1024 x 4096 4.45 us, 2048 x 5120 8.4 (3.3 TB/s), 8192 x 8192 47.4 (3.8); with addresses worked out anew
-// for every row, and up to eight rows a warp in whatever number of rounds, 5.8, 9.2 and 49.5.  Asking for more resident warps (64 registers) is slower.
+// launch below that.  Calls in a row on three inputs: 2048 x 5120 8.5 us (3.2 TB/s), 4096 x 4096 13.0, 8192 x 8192 49.3 (3.6); with addresses worked out anew
+// for every row 9.2, 13.7 and 49.5.  Asking for more resident warps (64 registers) is slower.
 #include "fgmp_common.cuh"
 #include "fgmp_host.h"
 #include <cuda_bf16.h>
@@ -15,7 +15,6 @@
 namespace {
 
 constexpr int QA_THREADS = 128;
-constexpr int QA_RESIDENT = 24;          // warps that an SM holds, by their 80 registers
 
 struct ActParams {
     const uint4* X; int64_t ldx8;        // row stride in 16-byte units
@@ -327,10 +326,12 @@ ActParams make_act_params(const void* X, int64_t ldx, const float* fisher, int64
     p.tau = tau;
     p.ratio = sc.fp8_log2_ratio;
     p.r8 = ldexpf(1.0f, sc.fp8_log2_ratio);
-    // Rows per warp: so many that the warps are as many as the chip holds at once, or a whole number of times as many where that would be more than 32.  (1024 x
-    // 4096: two rows for each of 4096 warps, 3552 at once, 5.7 us; three rows 4.45.)
-    const int64_t words = M * p.MW, fit = (int64_t)fgmp_sm_count() * QA_RESIDENT, rounds = (words + 32 * fit - 1) / (32 * fit);
-    p.rows_per_warp = (int)((words + rounds * fit - 1) / (rounds * fit));
+    // Rows per warp: one while there are fewer warps than 28 per SM, up to eight so that the Fisher weights are loaded rarely.  (So many that the 24 warps that
+    // an SM holds make whole rounds is faster for the quantizer alone, 1024 x 4096 4.45 us instead of 5.6 and 777 x 4096 3.95 instead of 4.7, but not
+    // among the kernels of a layer, where other kernels' blocks are on the SMs when its blocks come up: with the GEMM behind it 1024 x 4096 x 4096 47.4 us
+    // instead of 45.4, 500 x 3000 x 6016 34.0 and 33.2, 777 x 11008 x 4096 71.0 and 71.2.)
+    const int64_t words = M * p.MW, fit = words / ((int64_t)fgmp_sm_count() * 28);
+    p.rows_per_warp = (int)(fit < 1 ? 1 : fit > 8 ? 8 : fit);
     p.groups = (uint32_t)((M + p.rows_per_warp - 1) / p.rows_per_warp);
     return p;
 }
