@@ -29,10 +29,10 @@
 // Where the activation operand (a "step record" per chunk) comes from:
 //   DEC_FUSED_LP, DEC_FUSED_HP  fused calls (by block score): the CTAs share out the quantizer's work, write the records to
 //                the workspace and stream them from there; the first weight copies are in flight meanwhile.
-//   DEC_OWN1_LP ... DEC_OWN2_HP  fused calls of one or two tokens whose packed form nobody asks for: warps of each CTA quantize what its units
+//   DEC_OWN1_LP ... DEC_OWN4_HP  fused calls of one to four tokens whose packed form nobody asks for: warps of each CTA quantize what its units
 //                need, unit by unit, straight into the stages.  That is more work in all, and nothing to hand over: 2.7 us lie between the end of the
 //                kernel before and the last shared record, 0.7 more until its copy is in.  In a graph of such calls, 10 % FP8 blocks, shared and own:
-//                11008 x 4096 one token 14.1 and 10.3 us, two 14.1 and 10.8; 28672 x 8192 31.8 and 28.8, 31.7 and 30.4.  (With 64 threads a token
+//                11008 x 4096 one token 12.6 and 9.9 us, two 12.6 and 10.3, three 12.6 and 10.8; 28672 x 8192 one 31.8 and 28.5, two 31.7 and 30.6.  (With 64 threads a token
 //                for every unit in turn instead of two units at a time, two tokens took 14.5 and 48.6.)  Where a CTA has very many units the warps that
 //                quantize for each of them cost more than the hand-over: see the launch.
 //   DEC_UNPACK   fgmp_linear: made unit by unit in shared memory from the packed activations' records.
@@ -40,7 +40,7 @@
 // Warp roles: warp 0 = weights producer, warp 1 = MMA issuer and owner of the tensor memory, from warp 2 on two or three sets of four warps that take
 // the units in turn and put a unit's block scales and FP8 blocks into tensor memory, into a dense tile of their own (the first two sets are the
 // quantizer before that; or each makes the step record of its unit), then four warps of epilogue (one lane quadrant each), then the step-record
-// producer (DEC_OWN: four or eight warps, the quantizer).
+// producer (DEC_OWN: four warps per token, the quantizer).
 //
 // The roles run different code at the same time, a warp or two per scheduler, so a unit costs what its instructions cost to
 // fetch and issue: what a loop needs once per unit is not unrolled or inlined twice, and a unit passes through few hands
@@ -82,10 +82,11 @@ constexpr uint32_t DEC_TMEM_COLS = 512;
 constexpr size_t SMEM_LIMIT = 232448;
 static_assert(STG_STEP % 1024 == 0, "stage layout");
 
-enum { DEC_FUSED_LP = 0, DEC_FUSED_HP = 1, DEC_UNPACK = 2, DEC_OWN1_LP = 4, DEC_OWN1_HP = 5, DEC_OWN2_LP = 6, DEC_OWN2_HP = 7 };
-// (the lowest bit of the fused ones is the fgmp_score_mode of the quantizer, OWN1 and OWN2 are for one token and for two)
+enum { DEC_FUSED_LP = 0, DEC_FUSED_HP = 1, DEC_UNPACK = 2, DEC_OWN1_LP = 4, DEC_OWN1_HP = 5, DEC_OWN2_LP = 6, DEC_OWN2_HP = 7,
+       DEC_OWN3_LP = 8, DEC_OWN3_HP = 9, DEC_OWN4_LP = 10, DEC_OWN4_HP = 11 };
+// (the lowest bit of the fused ones is the fgmp_score_mode of the quantizer; OWN1 to OWN4 are for that many tokens)
 constexpr int OWN_TURNS = 2;                    // units whose step records are made at a time: 64 threads take about 1 us for a token's, the weights half of that
-constexpr int own_tokens(int src) { return src >= DEC_OWN2_LP ? 2 : src >= DEC_OWN1_LP ? 1 : 0; }
+constexpr int own_tokens(int src) { return src >= DEC_OWN1_LP ? (src - DEC_OWN1_LP) / 2 + 1 : 0; }
 constexpr int dec_threads(int src, int sets) { return 32 * (W_SET + 4 * sets + 4 + (own_tokens(src) ? 2 * OWN_TURNS * own_tokens(src) : 1)); }
 
 // Step record of a chunk for a batch of M tokens: n4 rows x 128 bytes of E2M1 codes | 2 KiB of block scales in tensor-
@@ -379,6 +380,32 @@ __device__ __forceinline__ void quantize_item(const DecParams& p, uint32_t c, ui
     }
 }
 
+// Sums of consecutive tokens of a row to and from a CTA's part of a tile.  Stores are whole sectors of 32 bytes: with 16 bytes for four tokens, three
+// tokens of 4096 x 4096 took 7.9 us instead of 7.5, four of 8192 x 4096 10.3 instead of 10.0.
+__device__ __forceinline__ void store_part(float* dst, const float (&v)[8])
+{
+    asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"l"(dst), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])),
+                   "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])), "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])) : "memory");
+}
+__device__ __forceinline__ void store_part(float* dst, const float (&v)[4])
+{
+    asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %5, %5, %5};"
+                 ::"l"(dst), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3])), "r"(0) : "memory");
+}
+__device__ __forceinline__ void load_part(const float* src, float (&v)[8])
+{
+    uint32_t y[8];
+    asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(y[0]), "=r"(y[1]), "=r"(y[2]), "=r"(y[3]), "=r"(y[4]), "=r"(y[5]), "=r"(y[6]), "=r"(y[7]) : "l"(src) : "memory");
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(y[j]);
+}
+__device__ __forceinline__ void load_part(const float* src, float (&v)[4])
+{
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "l"(src) : "memory");
+}
+
 // A token's sum of a row from the accumulators: NVFP4 rows and digits (col 0 and 1 .. 6), and of the FP8 weight blocks, where there are any
 template <typename Col>
 __device__ __forceinline__ float token_sum(bool has_fp8, float rw, float ra, const Col& col, uint32_t high, uint32_t low)
@@ -395,12 +422,13 @@ decode_kernel(const __grid_constant__ DecParams p)
     extern __shared__ uint8_t smem_raw[];
     // 1 KiB aligned; an offset from the array keeps the pointer known to be shared memory (plain ld.shared / st.shared)
     uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
-    constexpr bool FUSED = SRC != DEC_UNPACK, OWN = own_tokens(SRC) != 0, SHARED = FUSED && !OWN;      // SHARED: the CTAs share out the quantizer's work
+    constexpr int TOKENS = own_tokens(SRC);              // 0: as many as p.M says
+    constexpr bool FUSED = SRC != DEC_UNPACK, OWN = TOKENS != 0, SHARED = FUSED && !OWN;      // SHARED: the CTAs share out the quantizer's work
     constexpr int X = DEC_MAX_STAGES;
     using D = Dec<SETS>;
     constexpr int W_EPI = D::W_EPI, W_STEP = D::W_STEP;
     const uint32_t S = p.stages;
-    const uint32_t M = OWN ? (uint32_t)own_tokens(SRC) : (uint32_t)p.M, n4 = step_n4(M), n8 = step_n8(M), a_bytes = step_bytes(M);
+    const uint32_t M = OWN ? (uint32_t)TOKENS : (uint32_t)p.M, n4 = step_n4(M), n8 = step_n8(M), a_bytes = step_bytes(M);
     uint8_t* arecs = smem + S * p.stage_bytes;           // DEC_UNPACK: S packed activation records
     uint64_t* bars = reinterpret_cast<uint64_t*>(arecs + S * p.arec_bytes);
     StageMeta* smeta = reinterpret_cast<StageMeta*>(bars + 4 * X + 4);
@@ -463,7 +491,7 @@ decode_kernel(const __grid_constant__ DecParams p)
             bulk_load(dst + AREC_HOT, src + AREC_AT, p.arec_bytes - AREC_HOT, wf0 + 8 * s);
         };
         const uint32_t* uptr = reinterpret_cast<const uint32_t*>(p.wblob + p.LW.off_uptr);
-        uint32_t pf_base = 0, pf = 0, stage = 0, phase = 1;
+        uint32_t u = 0, pf_base = 0, pf = 0, refill = 0, stage = 0, phase = 1;
         const uint32_t pf_begin = order.front && u_begin + lane <= u_end ? __ldg(uptr + u_begin + lane) : 0u;
         const uint32_t pre = min(S, n_units);
         for (uint32_t i = 0; i <= n_units; ++i) {
@@ -478,11 +506,11 @@ decode_kernel(const __grid_constant__ DecParams p)
                 if (bad && lane == 0) { *abort_flag = 1; atomicCAS(p.status, 0, (int)FGMP_ERR_INVALID_ARG); atomicExch(p.status + 1, bad); }
             }
             if (!ok || i == n_units) break;
-            const uint32_t u = order.unit(i);
-            if (i == order.front && i) { pf_base = u; pf = pf_begin; }      // (asked for with the first: their way is as long as a unit takes)
-            if (i == 0 || u + 1 - pf_base > 31) {      // next 32 list starts
-                pf_base = u;
-                pf = pf_base + lane <= u_end ? __ldg(uptr + pf_base + lane) : 0u;
+            if (i == refill) {                         // next 32 list starts (one comparison a unit: with the order asked for every time, 2 x 28672 x 8192 took 31.2 us, not 30.6)
+                u = pf_base = order.unit(i);
+                if (i && i == order.front) pf = pf_begin;      // (asked for with the first: their way is as long as a unit takes)
+                else pf = pf_base + lane <= u_end ? __ldg(uptr + pf_base + lane) : 0u;
+                refill = i < order.front ? min(i + 31u, order.front) : i + 31u;
             }
             const uint32_t step0 = __shfl_sync(0xffffffffu, pf, (int)(u - pf_base)), step1 = __shfl_sync(0xffffffffu, pf, (int)(u + 1 - pf_base));
             if (lane == 0) {
@@ -500,6 +528,7 @@ decode_kernel(const __grid_constant__ DecParams p)
                 }
             }
             ok = __shfl_sync(0xffffffffu, ok, 0);
+            ++u;
             if (++stage == S) { stage = 0; phase ^= 1; }
         }
     } else {
@@ -541,6 +570,8 @@ decode_kernel(const __grid_constant__ DecParams p)
         // record holds of one token; two units at a time.
         const uint32_t tq = threadIdx.x - 32u * W_STEP, part = tq >> 6, li = tq & 3u, j = (tq >> 2) & 15u, m = part % M;
         uint32_t i = part / M, c = order.unit(i) % C, stage = i, phase = 1;        // (fewer at a time than stages)
+        // (the units taken first are chunks 0 .. front - 1)
+        uint32_t c_end = i < order.front ? order.front : C, c_jump = i < order.front ? u_begin % C - order.front : 0u - C;
         const uint8_t* row = p.X + (size_t)m * p.ldx * 2 + 32u * j + 8u * li;
         const float* fish = p.fisher + 16u * j + 4u * li;
         uint2 x = make_uint2(0u, 0u);
@@ -549,8 +580,7 @@ decode_kernel(const __grid_constant__ DecParams p)
         for (; i < n_units; i += OWN_TURNS) {
             const BlockQuarter r = quantize_block_quarter<(SRC & 1)>(x, f, p.q);
             c += OWN_TURNS;
-            if (i < order.front && i + OWN_TURNS >= order.front) c = u_begin % C + i + OWN_TURNS - order.front;      // (behind the units taken first)
-            while (c >= C) c -= C;
+            while (c >= c_end) { c += c_jump; c_end = C; c_jump = 0u - C; }
             if (i + OWN_TURNS < n_units) { x = __ldg(reinterpret_cast<const uint2*>(row + 512u * c)); f = __ldg(reinterpret_cast<const float4*>(fish + 256u * c)); }
             const float2 va = __half22float2(*reinterpret_cast<const __half2*>(&r.h.x)), vb = __half22float2(*reinterpret_cast<const __half2*>(&r.h.y));
             const float v[4] = {va.x, va.y, vb.x, vb.y};
@@ -739,16 +769,17 @@ decode_kernel(const __grid_constant__ DecParams p)
         // FP8 tensor scale / NVFP4 tensor scale of either operand
         const float rw = __int_as_float((127 + __ldg(&hw->fp8_log2_ratio)) << 23);
         const float ra = FUSED ? p.q.r8 : __int_as_float((127 + ha->fp8_log2_ratio) << 23);
-        const uint32_t row = 32 * q + lane, octets = OWN ? 1u : (M + 7u) / 8u;
-        // eight tokens' sums of the row, from token 8 o on, to Y
-        const auto emit = [&](const float (&v)[8], uint32_t o, int64_t n) {
+        constexpr uint32_t W = TOKENS > 2 ? 4u : 8u;       // tokens at a time (four: eight take more than 64 registers)
+        const uint32_t row = 32 * q + lane, rounds = (M + W - 1u) / W;
+        // W tokens' sums of the row, from token W o on, to Y
+        const auto emit = [&](const float (&v)[W], uint32_t o, int64_t n) {
             if (n >= p.N) return;
-            const int64_t at = (int64_t)(8u * o) * p.ldy + n;
+            const int64_t at = (int64_t)(W * o) * p.ldy + n;
             __nv_bfloat16* yb = reinterpret_cast<__nv_bfloat16*>(p.Ybf) + at;
             float* yf = p.Y + at;
 #pragma unroll
-            for (uint32_t j = 0; j < (OWN ? (uint32_t)own_tokens(SRC) : 8u); ++j) {
-                if (8u * o + j < M) {
+            for (uint32_t j = 0; j < (OWN ? (uint32_t)TOKENS : W); ++j) {
+                if (W * o + j < M) {
                     if (p.y_is_bf16) *yb = __float2bfloat16_rn(v[j] * alpha);
                     else *yf = v[j] * alpha;
                 }
@@ -780,36 +811,31 @@ decode_kernel(const __grid_constant__ DecParams p)
             const uint32_t d4 = tmem_base + ((uint32_t)(q * 32) << 16) + D::D4_COL + accb * D::D4;
             const uint32_t d8 = tmem_base + ((uint32_t)(q * 32) << 16) + D::D8_COL + accb * D::D8;
 #pragma unroll 1
-            for (uint32_t o = 0; o < octets; ++o) {
-                float v[8];
-                if constexpr (OWN) {
+            for (uint32_t o = 0; o < rounds; ++o) {
+                float v[W];
+                if constexpr (OWN && TOKENS <= 2) {
                     // at most 14 and 4 columns: one load of each
-                    constexpr int T = own_tokens(SRC);
                     uint32_t r0[16], r1[16], r2[16] = {};
                     tmem_ld16_async(d4, r0); tmem_ld16_async(d8, r1);
                     tmem_wait_ld(r0, r1, r2);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = 0.f;
+                    for (uint32_t j = 0; j < W; ++j) v[j] = 0.f;
 #pragma unroll
-                    for (int j = 0; j < T; ++j) v[j] = token_sum(has_fp8, rw, ra, [&](int k) { return r0[T * k + j]; }, r1[j], r1[T + j]);
+                    for (int j = 0; j < TOKENS; ++j) v[j] = token_sum(has_fp8, rw, ra, [&](int k) { return r0[TOKENS * k + j]; }, r1[j], r1[TOKENS + j]);
                 } else {
-                    uint32_t r[PIECES + 1][8], hi[8], lo[8];
+                    uint32_t r[PIECES + 1][W], hi[W], lo[W];
 #pragma unroll
-                    for (uint32_t k = 0; k <= (uint32_t)PIECES; ++k) tmem_ld8_async(d4 + k * M + 8u * o, r[k]);
-                    tmem_ld8_async(d8 + 8u * o, hi); tmem_ld8_async(d8 + M + 8u * o, lo);
-                    tmem_wait_ld8(hi);
-                    tmem_hold8(lo);
+                    for (uint32_t k = 0; k <= (uint32_t)PIECES; ++k) tmem_ld_async(d4 + k * M + W * o, r[k]);
+                    tmem_ld_async(d8 + W * o, hi); tmem_ld_async(d8 + M + W * o, lo);
+                    tmem_wait_ld();
+                    tmem_hold(hi); tmem_hold(lo);
 #pragma unroll
-                    for (uint32_t k = 0; k <= (uint32_t)PIECES; ++k) tmem_hold8(r[k]);
+                    for (uint32_t k = 0; k <= (uint32_t)PIECES; ++k) tmem_hold(r[k]);
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) v[j] = token_sum(has_fp8, rw, ra, [&](int k) { return r[k][j]; }, hi[j], lo[j]);
+                    for (uint32_t j = 0; j < W; ++j) v[j] = token_sum(has_fp8, rw, ra, [&](int k) { return r[k][j]; }, hi[j], lo[j]);
                 }
                 if (whole) emit(v, o, n);
-                else                                   // this CTA's part (32 bytes per store: whole sectors)
-                    asm volatile("st.global.cg.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
-                                 ::"l"(base + (size_t)slot * 2048 + 8u * o), "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-                                   "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-                                   "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])) : "memory");
+                else store_part(base + (size_t)slot * 2048 + W * o, v);         // this CTA's part
             }
             tc_fence_before();
             __syncwarp();
@@ -832,23 +858,20 @@ decode_kernel(const __grid_constant__ DecParams p)
                 if (i == n_units && threadIdx.x == W_EPI * 32) FGMP_STAMP_ANY(12);
                 if (old == nseg - 1) {                 // this warp is the last: it adds everything up
 #pragma unroll 1
-                    for (uint32_t o = 0; o < octets; ++o) {
-                        float v[8];
+                    for (uint32_t o = 0; o < rounds; ++o) {
+                        float v[W];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) v[j] = 0.f;
+                        for (uint32_t j = 0; j < W; ++j) v[j] = 0.f;
 #pragma unroll 1
                         for (uint32_t g = 0; g < nseg; g += 2) {       // one sum in slot order, two parts under way at a time
-                            uint32_t y[2][8];
+                            float y[2][W];
 #pragma unroll
-                            for (uint32_t h = 0; h < 2; ++h)           // (a last one twice)
-                                asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                                             : "=r"(y[h][0]), "=r"(y[h][1]), "=r"(y[h][2]), "=r"(y[h][3]), "=r"(y[h][4]), "=r"(y[h][5]), "=r"(y[h][6]), "=r"(y[h][7])
-                                             : "l"(base + (size_t)min(g + h, nseg - 1u) * 2048 + 8u * o) : "memory");
+                            for (uint32_t h = 0; h < 2; ++h) load_part(base + (size_t)min(g + h, nseg - 1u) * 2048 + W * o, y[h]);      // (a last one twice)
 #pragma unroll
                             for (uint32_t h = 0; h < 2; ++h) {
                                 if (g + h >= nseg) break;
 #pragma unroll
-                                for (int j = 0; j < 8; ++j) v[j] += __uint_as_float(y[h][j]);
+                                for (uint32_t j = 0; j < W; ++j) v[j] += y[h][j];
                             }
                         }
                         emit(v, o, n);
@@ -902,6 +925,8 @@ fgmp_status set_attrs_once()
         bool ok = true;
         for (const void* k : {(const void*)decode_kernel<DEC_FUSED_LP, 2>, (const void*)decode_kernel<DEC_FUSED_HP, 2>, (const void*)decode_kernel<DEC_OWN1_LP, 3>,
                               (const void*)decode_kernel<DEC_OWN1_HP, 3>, (const void*)decode_kernel<DEC_OWN2_LP, 3>, (const void*)decode_kernel<DEC_OWN2_HP, 3>,
+                              (const void*)decode_kernel<DEC_OWN3_LP, 2>, (const void*)decode_kernel<DEC_OWN3_HP, 2>, (const void*)decode_kernel<DEC_OWN4_LP, 2>,
+                              (const void*)decode_kernel<DEC_OWN4_HP, 2>,
                               (const void*)decode_kernel<DEC_FUSED_LP, 3>, (const void*)decode_kernel<DEC_FUSED_HP, 3>, (const void*)decode_kernel<DEC_UNPACK, 2>})
             ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_LIMIT) == cudaSuccess;
         if (!ok)
@@ -1041,6 +1066,16 @@ extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const 
         if (d.total > (int64_t)d.grid * (M == 1 ? 200 : 80)) return launch(launch_decode<DEC_FUSED_LP, 3>, launch_decode<DEC_FUSED_HP, 3>);
         if (M == 1) return launch(launch_decode<DEC_OWN1_LP, 3>, launch_decode<DEC_OWN1_HP, 3>);
         return launch(launch_decode<DEC_OWN2_LP, 3>, launch_decode<DEC_OWN2_HP, 3>);
+    }
+    // Three and four tokens, two sets (twelve and sixteen warps that quantize leave 64 registers to a thread).  Us own and shared, 10 % FP8 blocks, by units
+    // per CTA: three tokens 7.6 and 10.3 at 3.5 (4096 x 4096), 12.3 and 14.1 at 12, 14.6 and 16.1 at 14.6, 18.2 and 18.5 at 21, 18.9 and 19.5 at 24, 21.8
+    // and 21.5 at 28, 34.4 and 32.2 at 48; four 7.9 and 10.3 at 3.5, 10.0 and 11.6 at 7, 12.3 and 13.4 at 10.4, 13.4 and 13.9 at 11.6, 15.3 and 15.2 at 13.8.
+    // (Without FP8 blocks 15.2 and 16.2 at 24 and 11.4 and 12.2 at 11.6, with 20 % 27.2 and 28.9, 17.4 and 18.2.)  More tokens gain where a CTA has a
+    // unit or two alone: eight tokens 6.5 instead of 7.8 at one unit, 8.5 and 8.7 at two, 11.4 and 10.5 at 3.5.
+    const int64_t own_units = M == 3 ? 25 : M == 4 ? 12 : 0;
+    if (!packed_acts_out && d.total <= own_units * d.grid) {
+        if (M == 3) return launch(launch_decode<DEC_OWN3_LP, 2>, launch_decode<DEC_OWN3_HP, 2>);
+        return launch(launch_decode<DEC_OWN4_LP, 2>, launch_decode<DEC_OWN4_HP, 2>);
     }
     return launch(launch_decode<DEC_FUSED_LP, 2>, launch_decode<DEC_FUSED_HP, 2>);
 }

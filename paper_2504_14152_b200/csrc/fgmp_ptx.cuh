@@ -269,21 +269,22 @@ __device__ __forceinline__ void tmem_wait_ld(uint32_t (&a)[16], uint32_t (&b)[16
     asm volatile("" : FGMP_RW16(c) :: "memory");
 }
 
-// eight columns in the same way; tmem_wait_ld8 waits for all loads, and tmem_hold8 names the registers of the others
-__device__ __forceinline__ void tmem_ld8_async(uint32_t taddr, uint32_t (&r)[8])
+// Eight or four columns in the same way; tmem_wait_ld waits for all loads, and tmem_hold names the registers of each
+__device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[8])
 {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]) : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_wait_ld8(uint32_t (&r)[8])
+__device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&r)[4])
 {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]) :: "memory");
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_hold8(uint32_t (&r)[8])
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void tmem_hold(uint32_t (&r)[8])
 {
     asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]) :: "memory");
 }
+__device__ __forceinline__ void tmem_hold(uint32_t (&r)[4]) { asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]) :: "memory"); }
 
 // registers -> TMEM: lane i of the warp writes r[0..15] to columns taddr.col .. +15 of TMEM lane
 // (taddr.lane + i); a warp can only reach the 32 lanes of its quadrant (warp index % 4)

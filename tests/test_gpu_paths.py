@@ -270,6 +270,39 @@ def test_quantizer_in_every_cta(fg, M, N, K, frac_w, mode):
     assert torch.equal(fg.linear_fused(wide[:, :K], fx.cuda(), pw, **args), y), "rows further apart"
 
 
+# three and four tokens: the quantizer in every CTA up to so many units of weights in it (on 148 SMs), shared beyond; one unit, a tile of odd size, no FP8
+# blocks and only such, rows further apart; the same sums whoever quantizes, and the oracle's
+@pytest.mark.parametrize("M,N,K,frac_w,mode,own", [
+    (3, 130, 256, 0.1, 0, True), (4, 130, 256, 0.1, 1, True), (3, 1000, 768, 0.0, 1, True), (4, 640, 5120, 1.0, 0, True), (3, 9000, 2048, 0.1, 1, True),
+    (3, 128 * 37, 25600, 0.1, 0, True), (3, 128 * 74, 13312, 0.1, 1, False), (4, 128 * 74, 6144, 0.1, 1, True), (4, 128 * 148, 3328, 0.1, 0, False)])
+def test_quantizer_of_three_and_four_tokens(fg, M, N, K, frac_w, mode, own):
+    wl = gi.llama("own34", M, 8, K, seed=76)
+    x, fx = wl.x(), wl.fx()
+    s4 = gi.tensor_scale(x)
+    tau = tau_for_fraction(oracle.quantize_activations(gi.bf16_bits(x), fx.numpy(), s4, mode=mode).scores, 0.2)
+    wide = torch.randn(M, K + 8, generator=torch.Generator().manual_seed(1)).to(torch.bfloat16).cuda()
+    wide[:, :K] = x.cuda()
+    x, f, args = wide[:, :K], fx.cuda(), dict(scale_fp4=s4, score_mode=mode, tau=tau)
+    pw = draw_weights(fg, N, K, 77, frac_w)
+    ws = fg.alloc_workspace(fg.OP_LINEAR_FUSED, M, N, K, torch.device("cuda"))
+    records = ws[-(K // 256) * 8192:]                     # (a chunk's record takes at least as much)
+    records.fill_(0x5a)
+    y = fg.linear_fused(x, f, pw, workspace=ws, **args)
+    fg.check(ws)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 148:
+        assert bool((records == 0x5a).all()) == own
+    ys, packed = fg.linear_fused(x, f, pw, want_packed=True, workspace=ws, **args)
+    for got in [ys, fg.linear(packed, pw)] + [fg.linear_fused(x, f, pw, workspace=ws, **args) for _ in range(10)]:
+        assert torch.equal(got.view(torch.int32), y.view(torch.int32)), "bit for bit, whoever quantizes"
+    if N <= 1000:
+        wl = gi.llama("own34", M, N, K, seed=76)
+        qw = oracle.quantize_weights(gi.bf16_bits(wl.w()), wl.fw().numpy(), clip=False, mode=mode, fp8_fraction=frac_w)
+        qa = oracle.quantize_activations(gi.bf16_bits(x.cpu()), fx.numpy(), s4, tau=tau, mode=mode)
+        pw = fg.quantize_weights(wl.w().cuda(), wl.fw().cuda(), clip_mode=0, score_mode=mode, fp8_fraction=frac_w)
+        Y, S = oracle.linear(qa, qw)
+        assert (np.abs(fg.linear_fused(x, f, pw, workspace=ws, **args).cpu().numpy().astype(np.float64) - Y) <= 1e-5 * S + 1e-30).all()
+
+
 # One or two tokens where the quantizer goes from every CTA to the shared one, by the units of weights that a CTA has: what is shared passes through the
 # workspace.  The same sums either way, and those of the packed tokens.
 @pytest.mark.parametrize("M,units,shared", [(1, 200, False), (1, 201, True), (2, 80, False), (2, 81, True)])
