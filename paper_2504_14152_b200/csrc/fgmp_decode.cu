@@ -1067,7 +1067,7 @@ extern "C" fgmp_status fgmp_linear_fused(const void* X_bf16, int64_t ldx, const 
         if (M == 1) return launch(launch_decode<DEC_OWN1_LP, 3>, launch_decode<DEC_OWN1_HP, 3>);
         return launch(launch_decode<DEC_OWN2_LP, 3>, launch_decode<DEC_OWN2_HP, 3>);
     }
-    // Three and four tokens, two sets (twelve and sixteen warps that quantize leave 64 registers to a thread).  Us own and shared, 10 % FP8 blocks, by units
+    // Three and four tokens, two sets (twelve and sixteen warps that quantize leave 72 and 64 registers to a thread).  Us own and shared, 10 % FP8 blocks, by units
     // per CTA: three tokens 7.6 and 10.3 at 3.5 (4096 x 4096), 12.3 and 14.1 at 12, 14.6 and 16.1 at 14.6, 18.2 and 18.5 at 21, 18.9 and 19.5 at 24, 21.8
     // and 21.5 at 28, 34.4 and 32.2 at 48; four 7.9 and 10.3 at 3.5, 10.0 and 11.6 at 7, 12.3 and 13.4 at 10.4, 13.4 and 13.9 at 11.6, 15.3 and 15.2 at 13.8.
     // (Without FP8 blocks 15.2 and 16.2 at 24 and 11.4 and 12.2 at 11.6, with 20 % 27.2 and 28.9, 17.4 and 18.2.)  More tokens gain where a CTA has a
